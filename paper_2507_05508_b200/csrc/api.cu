@@ -1,4 +1,5 @@
 // C ABI of the MLMC compression library: context, argument checks and the launch sequences.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -111,33 +112,56 @@ int normalise_probs(const double* p, int L, double* out) {
 
 int finish(cudaError_t e) { return e == cudaSuccess ? MLMC_OK : MLMC_ERR_CUDA; }
 
-// Thresholds of every live query (sweep 1 + the two masked digit passes for fp32).
-// sweep 1 (leading-digit histogram), and for fp32 sweep 2 (candidates [+ energies]) and the two remaining
-// digit passes over the candidates.
-// brackets (fixed p, fp32): the first sweep also collects the keys of the bins around last call's boundary bins;
+// The selection of a call: thresholds of every query, for adaptive p the probabilities and the draw, the headers.
+// brackets (given p, fp32): the first sweep also collects the keys of the bins around last call's boundary bins;
 // where both boundary bins of a worker's band fall inside, the candidate sweep has nothing left to do.
-void run_selection(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, int L, bool sums,
-                   bool brackets, cudaStream_t s) {
-    brackets = brackets && dtype == MLMC_F32 && !sums && L > 1;
-    launch_reset_selection(ws, dtype, d, M, s);
+void run_selection(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const FinishPlan& plan, bool brackets,
+                   cudaStream_t s) {
     launch_hist1(ws, g, dtype, d, M, ld, brackets, s);
-    launch_resolve1(ws, dtype, M, L, brackets, s);
+    launch_resolve1(ws, dtype, M, plan, brackets, s);
     if (dtype == MLMC_F32) {
-        launch_sums_candidates(ws, g, d, M, ld, L, sums, brackets, s);
-        if (L > 1) {
-            launch_digit_pass(ws, g, d, M, ld, 2, s);
-            launch_resolve23(ws, M, L, 2, s);
-            launch_digit_pass(ws, g, d, M, ld, 3, s);
-            launch_resolve23(ws, M, L, 3, s);
-        }
+        launch_sums_candidates(ws, g, d, M, ld, plan, brackets, s);
+        launch_digit_passes(ws, g, d, M, ld, plan, s);
     }
 }
 
-void run_band_norms(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, int L, cudaStream_t s) {
-    if (dtype == MLMC_BF16)
-        launch_norm_from_hist_bf16(ws, M, L, s);
-    else
-        launch_band_norms_fp32(ws, g, d, M, ld, L, s);
+FinishPlan finish_plan(int64_t d, int L, int nq, bool adaptive, uint64_t seed, uint64_t step, const mlmc_topk_msgs* out) {
+    FinishPlan pl = {};
+    pl.L = L;
+    pl.nq = nq;
+    pl.adaptive = adaptive ? 1 : 0;
+    pl.want_emit = out ? 1 : 0;
+    pl.d = d;
+    pl.seed = seed;
+    pl.step = step;
+    if (out) {
+        pl.out_count = out->count;
+        pl.out_level = out->level;
+        pl.out_p_sel = out->p_sel;
+        pl.capacity = out->capacity;
+    }
+    return pl;
+}
+
+// Adaptive p: every level boundary is a query.
+void select_adaptive(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int64_t* k, int L,
+                     uint64_t seed, uint64_t step, const mlmc_topk_msgs* out, cudaStream_t s) {
+    FinishPlan pl = finish_plan(d, L, L - 1, true, seed, step, out);
+    for (int l = 0; l < L; ++l) pl.k[l] = (uint32_t)k[l];
+    launch_begin_adaptive(ws, dtype, d, M, k, L, s);
+    run_selection(ws, g, dtype, d, M, ld, pl, false, s);
+}
+
+// Given p: the level of every worker is drawn here (it depends on seed, step and worker only), and the two ranks that
+// bound its band are the only queries.
+template <typename Draw>
+void select_drawn(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, int L, bool brackets, uint64_t seed,
+                  uint64_t step, const mlmc_topk_msgs* out, Draw&& draw, cudaStream_t s) {
+    brackets = brackets && dtype == MLMC_F32 && L > 1;
+    DrawnBand bands[kEmitMaxWorkers];
+    for (int m = 0; m < M; ++m) bands[m] = draw(counter_uniform(seed, step, (uint64_t)m));
+    launch_begin_drawn(ws, dtype, d, M, bands, L, brackets, s);
+    run_selection(ws, g, dtype, d, M, ld, finish_plan(d, L, 2, false, seed, step, out), brackets, s);
 }
 
 }  // namespace
@@ -171,13 +195,11 @@ int mlmc_create(mlmc_ctx** out, int device, int64_t d_max, int M_max, int L_max)
     ws.ev_start = ws.ev_stop = nullptr;
     ws.ev_id = nullptr;
     for (int i = 0; i < K_COUNT; ++i) ws.launches_by_id[i] = 0;
-    ws.norm_ctas = ws.sm_count * 4;
     ws.sum_ctas = ws.sm_count * 4;
-    ws.cur_norm_ctas = ws.cur_sum_ctas = 0;
+    ws.cur_sum_ctas = 0;
     // candidate keys: a quarter of the row (boundary bins normally hold a few percent of it); small rows fit whole
     ws.cand_cap = d_max / 4 > (int64_t(1) << 20) ? d_max / 4 : (d_max < (int64_t(1) << 20) ? d_max : (int64_t(1) << 20));
     ws.stat_ctas = ws.sm_count * 4;
-    ws.cur_stat_ctas = 0;
     const int64_t emit_tiles = (d_max + kEmitTile - 1) / kEmitTile;
     const int64_t agg_tiles = (d_max + kAggTile - 1) / kAggTile;
     ws.max_tiles = emit_tiles * M_max;
@@ -187,37 +209,33 @@ int mlmc_create(mlmc_ctx** out, int device, int64_t d_max, int M_max, int L_max)
     const size_t o_werr = pl.take(sizeof(int) * M_max);
     const size_t o_hist1 = pl.take(sizeof(uint32_t) * kBins1 * M_max);
     const size_t o_table1 = pl.take((size_t)kBins1 * M_max);
-    const size_t o_hist2 = pl.take(sizeof(uint32_t) * kMaxQueries * kBins23 * M_max);
+    const size_t o_hist23 = pl.take(sizeof(uint32_t) * kMaxQueries * kBins23 * 2 * M_max);
     const size_t o_map2 = pl.take((size_t)kMaxQueries * kBins23 * M_max);
-    const size_t o_hist3 = pl.take(sizeof(uint32_t) * kMaxQueries * kBins23 * M_max);
+    const size_t o_done = pl.take(sizeof(uint32_t) * M_max);
+    const size_t o_acc = pl.take(sizeof(uint32_t) * M_max);
     const size_t o_queries = pl.take(sizeof(Query) * kMaxQueries * M_max);
-    const size_t o_band = pl.take(sizeof(double) * kMaxLevels * ws.norm_ctas * M_max);
     const size_t o_sum = pl.take(sizeof(double) * kMaxLevels * ws.sum_ctas * M_max);
-    const size_t o_cpart = pl.take(sizeof(unsigned long long) * kMaxLevels * 4 * M_max);
+    const size_t o_cpart = pl.take(sizeof(unsigned long long) * kEnergyCells * 2 * M_max);
     const size_t o_ckeys = pl.take(sizeof(uint32_t) * ws.cand_cap * M_max);
     const size_t o_ccount = pl.take(sizeof(uint32_t) * M_max);
     const size_t o_cover = pl.take(sizeof(int) * M_max);
-    const size_t o_k = pl.take(sizeof(int64_t) * kMaxLevels);
-    const size_t o_pfix = pl.take(sizeof(double) * kMaxLevels);
     const size_t o_pall = pl.take(sizeof(double) * kMaxLevels * M_max);
     const size_t o_dall = pl.take(sizeof(double) * kMaxLevels * M_max);
     const size_t o_u = pl.take(sizeof(double) * M_max);
     const size_t o_emit = pl.take(sizeof(EmitParams) * M_max);
     const size_t o_tdesc = pl.take(sizeof(uint4) * ws.max_tiles);
+    const size_t o_ldesc = pl.take(sizeof(uint4) * emit_counts((int)emit_tiles).total() * M_max);
+    const size_t o_tlist = pl.take(sizeof(uint2) * ws.max_tiles);
+    const size_t o_listn = pl.take(sizeof(uint32_t));
     const size_t o_tmax = pl.take(sizeof(uint32_t) * ws.max_tiles * kEmitGroups);
     const size_t o_groupn = pl.take(sizeof(uint32_t) * M_max);
-    const size_t o_wtiles = pl.take(sizeof(uint32_t) * ws.max_tiles);
-    const size_t o_tilen = pl.take(sizeof(uint32_t) * M_max);
     const size_t o_cfloor = pl.take(sizeof(uint32_t) * M_max);
     const size_t o_aggoff = pl.take(sizeof(uint32_t) * (agg_tiles + 1) * M_max);
     const size_t o_gmax = pl.take(sizeof(uint32_t) * M_max);
     const size_t o_S = pl.take(sizeof(unsigned long long) * kMaxLevels * ws.stat_ctas * M_max);
     const size_t o_blevel = pl.take(sizeof(int32_t) * M_max);
     ws.big_cap = d_max < (int64_t(1) << 20) ? d_max : (int64_t(1) << 20);
-    const size_t o_pbig = pl.take(sizeof(double) * ws.big_cap);
-    const size_t o_cbig = pl.take(sizeof(double) * ws.big_cap);
     ws.rtn_ctas = ws.sm_count * 8;
-    ws.cur_rtn_ctas = 0;
     const size_t o_rtn = pl.take(sizeof(double) * kMaxLevels * ws.rtn_ctas * M_max);
     const size_t o_pbin = pl.take(sizeof(uint32_t) * kMaxLevels * M_max);
     const size_t o_brk = pl.take(sizeof(uint4) * M_max);
@@ -244,34 +262,31 @@ int mlmc_create(mlmc_ctx** out, int device, int64_t d_max, int M_max, int L_max)
     ws.worker_err = reinterpret_cast<int*>(base + o_werr);
     ws.hist1 = reinterpret_cast<uint32_t*>(base + o_hist1);
     ws.table1 = reinterpret_cast<uint8_t*>(base + o_table1);
-    ws.hist2 = reinterpret_cast<uint32_t*>(base + o_hist2);
+    ws.hist2 = ws.hist3 = reinterpret_cast<uint32_t*>(base + o_hist23);
     ws.map2 = reinterpret_cast<uint8_t*>(base + o_map2);
-    ws.hist3 = reinterpret_cast<uint32_t*>(base + o_hist3);
+    ws.done = reinterpret_cast<uint32_t*>(base + o_done);
+    ws.acc_word = reinterpret_cast<uint32_t*>(base + o_acc);
     ws.queries = reinterpret_cast<Query*>(base + o_queries);
-    ws.band_partial = reinterpret_cast<double*>(base + o_band);
     ws.sum_partial = reinterpret_cast<double*>(base + o_sum);
     ws.cand_S = reinterpret_cast<unsigned long long*>(base + o_cpart);
     ws.cand_keys = reinterpret_cast<uint32_t*>(base + o_ckeys);
     ws.cand_count = reinterpret_cast<uint32_t*>(base + o_ccount);
     ws.cand_overflow = reinterpret_cast<int*>(base + o_cover);
-    ws.k_dev = reinterpret_cast<int64_t*>(base + o_k);
-    ws.p_fixed = reinterpret_cast<double*>(base + o_pfix);
     ws.p_all = reinterpret_cast<double*>(base + o_pall);
     ws.delta_all = reinterpret_cast<double*>(base + o_dall);
     ws.u_dev = reinterpret_cast<double*>(base + o_u);
     ws.emit = reinterpret_cast<EmitParams*>(base + o_emit);
     ws.tile_desc = reinterpret_cast<uint4*>(base + o_tdesc);
+    ws.level_desc = reinterpret_cast<uint4*>(base + o_ldesc);
+    ws.tile_list = reinterpret_cast<uint2*>(base + o_tlist);
+    ws.list_n = reinterpret_cast<uint32_t*>(base + o_listn);
     ws.tile_max = reinterpret_cast<uint32_t*>(base + o_tmax);
-    ws.worker_tiles = reinterpret_cast<uint32_t*>(base + o_wtiles);
-    ws.tile_n = reinterpret_cast<uint32_t*>(base + o_tilen);
     ws.group_n = reinterpret_cast<uint32_t*>(base + o_groupn);
     ws.cand_floor = reinterpret_cast<uint32_t*>(base + o_cfloor);
     ws.agg_offsets = reinterpret_cast<uint32_t*>(base + o_aggoff);
     ws.gmax_bits = reinterpret_cast<uint32_t*>(base + o_gmax);
     ws.S_partial = reinterpret_cast<unsigned long long*>(base + o_S);
     ws.bit_level = reinterpret_cast<int32_t*>(base + o_blevel);
-    ws.p_big = reinterpret_cast<double*>(base + o_pbig);
-    ws.cdf_big = reinterpret_cast<double*>(base + o_cbig);
     ws.rtn_partial = reinterpret_cast<double*>(base + o_rtn);
     ws.prev_bin = reinterpret_cast<uint32_t*>(base + o_pbin);
     ws.bracket = reinterpret_cast<uint4*>(base + o_brk);
@@ -322,12 +337,12 @@ int mlmc_get_status(mlmc_ctx* ctx, void* stream) {
 
 int64_t mlmc_launch_count(const mlmc_ctx* ctx) { return ctx ? ctx->ws.launches : 0; }
 
-static const char* const kKernelNames[K_COUNT] = {
-    "draw_fixed", "init_queries", "uniforms", "hist1", "resolve1", "sums_candidates", "cand_pass2", "masked_pass2",
-    "resolve2", "cand_pass3", "masked_pass3", "resolve3", "cand_sums", "norm_sweep", "norm_from_hist_bf16", "probs_draw", "copy_probs", "emit", "agg_offsets",
-    "aggregate_topk", "absmax", "bit_stats", "bit_probs_draw", "bit_pack", "aggregate_bitwise", "tile_list", "band_count", "band_scan", "bit_pack_wide", "reset",
-    "float_draw", "float_pack", "aggregate_floatbits", "rtn_stats", "rtn_probs_draw", "rtn_emit", "aggregate_dense", "stopk_draw", "stopk_params",
-    "sort_count", "sort_scan", "sort_scatter", "segment_norms"};
+static const char* const kKernelNames[] = {
+    "begin", "uniforms", "hist1", "resolve1", "sums_candidates", "cand_pass2", "cand_pass3", "band_header", "copy_probs", "emit",
+    "agg_offsets", "aggregate_topk", "absmax", "bit_stats", "bit_pack", "aggregate_bitwise", "tile_list", "band_count", "bit_pack_wide",
+    "float_pack", "aggregate_floatbits", "rtn_stats", "rtn_emit", "aggregate_dense", "stopk_draw", "sort_count", "sort_scan",
+    "sort_scatter", "segment_norms"};
+static_assert(sizeof(kKernelNames) / sizeof(kKernelNames[0]) == K_COUNT, "a name for every kernel id");
 
 int mlmc_kernel_count(void) { return K_COUNT; }
 
@@ -418,31 +433,22 @@ int mlmc_level_probs(mlmc_ctx* ctx, const void* g, int dtype, int64_t d, int M, 
         if (int rc = normalise_probs(p_host, L, pn)) return rc;
     DeviceGuard guard(ws.device);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    cudaMemsetAsync(ws.worker_err, 0, sizeof(int) * M, s);
-    if (p_host) cudaMemcpyAsync(ws.p_fixed, pn, sizeof(double) * L, cudaMemcpyHostToDevice, s);
+    set_call_size(ws, d, M, dtype == MLMC_BF16 ? 2 : 4);
     const bool need_data = (p_host == nullptr) || (delta_out != nullptr);
-    if (kind == MLMC_TOPK) {
-        cudaMemcpyAsync(ws.k_dev, sched, sizeof(int64_t) * L, cudaMemcpyHostToDevice, s);
-        if (need_data) {
-            launch_init_queries_adaptive(ws, M, L, d, s);
-            run_selection(ws, g, dtype, d, M, ld, L, true, false, s);
-            run_band_norms(ws, g, dtype, d, M, ld, L, s);
-            launch_probs_draw(ws, dtype, M, L, d, true, false, 0, 0, nullptr, s);
-        }
-    } else if (kind == MLMC_BITWISE) {
-        if (need_data) {
-            launch_absmax(ws, g, dtype, d, M, ld, s);
-            launch_bit_stats(ws, g, dtype, d, M, ld, b32, L, s);
-            launch_bit_probs_draw(ws, M, b32, L, true, true, 0, 0, nullptr, s);
-        }
-    } else {
-        if (need_data) {
-            launch_absmax(ws, g, dtype, d, M, ld, s);
-            launch_rtn_stats(ws, g, dtype, d, M, ld, b32, L, s);
-            launch_rtn_probs_draw(ws, M, L, true, true, 0, 0, nullptr, s);
+    if (need_data) {
+        if (kind == MLMC_TOPK) {
+            select_adaptive(ws, g, dtype, d, M, ld, sched, L, 0, 0, nullptr, s);
+        } else if (kind == MLMC_BITWISE) {
+            const DrawPlan plan = bit_draw_plan(ws, b32, L, 0, 0, nullptr);
+            launch_absmax(ws, g, dtype, d, M, ld, plan, nullptr, s);
+            launch_bit_stats(ws, g, dtype, d, M, ld, b32, L, plan, s);
+        } else {
+            const DrawPlan plan = rtn_draw_plan(ws, L, 0, 0, nullptr);
+            launch_absmax(ws, g, dtype, d, M, ld, plan, nullptr, s);
+            launch_rtn_stats(ws, g, dtype, d, M, ld, b32, L, plan, s);
         }
     }
-    launch_copy_probs(ws, M, L, p_host ? ws.p_fixed : nullptr, p_out, delta_out, s);
+    launch_copy_probs(ws, M, L, p_host ? pn : nullptr, p_out, delta_out, s);
     return finish(cudaGetLastError());
 }
 
@@ -459,13 +465,10 @@ int mlmc_compress_topk(mlmc_ctx* ctx, const void* g, int dtype, int64_t d, int M
     Workspace& ws = ctx->ws;
     DeviceGuard guard(ws.device);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    cudaMemsetAsync(ws.worker_err, 0, sizeof(int) * M, s);
-    cudaMemcpyAsync(ws.k_dev, k, sizeof(int64_t) * L, cudaMemcpyHostToDevice, s);
-    const bool adaptive = (p == nullptr);
-    if (adaptive) {
-        launch_init_queries_adaptive(ws, M, L, d, s);
+    set_call_size(ws, d, M, dtype == MLMC_BF16 ? 2 : 4);
+    if (!p) {
+        select_adaptive(ws, g, dtype, d, M, ld, k, L, seed, step, out, s);
     } else {
-        cudaMemcpyAsync(ws.p_fixed, pn, sizeof(double) * L, cudaMemcpyHostToDevice, s);
         // the bins stored by earlier calls belong to one problem: another shape or schedule starts afresh
         bool same = ws.sig_d == d && ws.sig_ld == ld && ws.sig_M == M && ws.sig_L == L && ws.sig_dtype == dtype;
         for (int l = 0; same && l < L; ++l) same = ws.sig_k[l] == k[l];
@@ -474,11 +477,11 @@ int mlmc_compress_topk(mlmc_ctx* ctx, const void* g, int dtype, int64_t d, int M
             ws.sig_d = d; ws.sig_ld = ld; ws.sig_M = M; ws.sig_L = L; ws.sig_dtype = dtype;
             for (int l = 0; l < L; ++l) ws.sig_k[l] = k[l];
         }
-        launch_draw_fixed(ws, M, L, d, seed, step, true, s);  // the draw does not depend on the data: only two thresholds are needed
+        select_drawn(ws, g, dtype, d, M, ld, L, true, seed, step, out, [&](double u) {
+            const int l = draw_from_probs(pn, L, u);
+            return DrawnBand{pn[l], l, l ? (uint32_t)k[l - 1] : 0u, (uint32_t)k[l]};
+        }, s);
     }
-    run_selection(ws, g, dtype, d, M, ld, L, adaptive, !adaptive, s);
-    if (adaptive) run_band_norms(ws, g, dtype, d, M, ld, L, s);
-    launch_probs_draw(ws, dtype, M, L, d, adaptive, true, seed, step, out, s);
     launch_emit(ws, g, dtype, d, M, ld, *out, s);
     return finish(cudaGetLastError());
 }
@@ -496,12 +499,10 @@ int mlmc_compress_bitwise(mlmc_ctx* ctx, const void* g, int dtype, int64_t d, in
     Workspace& ws = ctx->ws;
     DeviceGuard guard(ws.device);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    cudaMemsetAsync(ws.worker_err, 0, sizeof(int) * M, s);
-    const bool adaptive = (p == nullptr);
-    if (!adaptive) cudaMemcpyAsync(ws.p_fixed, pn, sizeof(double) * L, cudaMemcpyHostToDevice, s);
-    launch_absmax(ws, g, dtype, d, M, ld, s);
-    if (adaptive) launch_bit_stats(ws, g, dtype, d, M, ld, b32, L, s);
-    launch_bit_probs_draw(ws, M, b32, L, adaptive, false, seed, step, out, s);
+    set_call_size(ws, d, M, dtype == MLMC_BF16 ? 2 : 4);
+    const DrawPlan plan = bit_draw_plan(ws, b32, L, seed, step, out);
+    launch_absmax(ws, g, dtype, d, M, ld, plan, p ? pn : nullptr, s);
+    if (!p) launch_bit_stats(ws, g, dtype, d, M, ld, b32, L, plan, s);
     launch_bit_pack(ws, g, dtype, d, M, ld, b32, L, *out, s);
     return finish(cudaGetLastError());
 }
@@ -513,6 +514,7 @@ int mlmc_aggregate(mlmc_ctx* ctx, int kind, const void* msgs, const int32_t* b, 
     if (d < 1 || d > ws.d_max || M < 1 || M > ws.M_max) return MLMC_ERR_ARG;
     DeviceGuard guard(ws.device);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    set_call_size(ws, d, M, 4);
     if (kind == MLMC_TOPK) {
         const mlmc_topk_msgs* t = static_cast<const mlmc_topk_msgs*>(msgs);
         if (!t->idx || !t->val || !t->count || !t->level) return MLMC_ERR_ARG;
@@ -556,39 +558,35 @@ int mlmc_compress_stopk(mlmc_ctx* ctx, const void* g, int dtype, int64_t d, int 
                 return MLMC_ERR_NOMEM;
             }
         }
-        cudaMemsetAsync(ws.worker_err, 0, sizeof(int) * M, s);
-        launch_reset_selection(ws, dtype, d, M, s);
+        set_call_size(ws, d, M, dtype == MLMC_BF16 ? 2 : 4);
+        launch_begin_adaptive(ws, dtype, d, M, nullptr, 1, s);
         launch_hist1(ws, g, dtype, d, M, ld, false, s);  // the batch maxima for the emission, and the NaN / Inf check
         for (int m0 = 0; m0 < M; m0 += ws.sort_rows)
             launch_stopk_sorted_rows(ws, g, dtype, d, m0, (M - m0 < ws.sort_rows) ? M - m0 : ws.sort_rows, ld, s_len, L,
                                      seed, step, s);
-        launch_stopk_params(ws, M, s_len, d, out, s);
+        launch_band_header(ws, M, finish_plan(d, 3, 2, false, seed, step, out), s);
         launch_emit(ws, g, dtype, d, M, ld, *out, s);
         return finish(cudaGetLastError());
     }
-    // normalised p and its running sums in ascending l (the draw is min{ l : u < cdf_l }, the last cdf is 1)
-    std::vector<double> pn((size_t)L), cdf((size_t)L);
     double sum = 0.0;
     for (int64_t l = 0; l < L; ++l) {
         if (!(p[l] > 0.0) || !std::isfinite(p[l])) return MLMC_ERR_PROB;
         sum += p[l];
     }
     if (std::fabs(sum - 1.0) > 1e-9) return MLMC_ERR_PROB;
+    // running sums of the normalised p in ascending l: the draw is min{ l : u < cdf_l }, the last cdf is 1
+    std::vector<double> cdf((size_t)L);
     double c = 0.0;
-    for (int64_t l = 0; l < L; ++l) {
-        pn[(size_t)l] = p[l] / sum;
-        c += pn[(size_t)l];
-        cdf[(size_t)l] = (l == L - 1) ? 1.0 : c;
-    }
+    for (int64_t l = 0; l < L; ++l) cdf[(size_t)l] = (c += p[l] / sum);
+    cdf[(size_t)L - 1] = 1.0;
     DeviceGuard guard(ws.device);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    cudaMemsetAsync(ws.worker_err, 0, sizeof(int) * M, s);
-    cudaMemcpyAsync(ws.p_big, pn.data(), sizeof(double) * L, cudaMemcpyHostToDevice, s);
-    cudaMemcpyAsync(ws.cdf_big, cdf.data(), sizeof(double) * L, cudaMemcpyHostToDevice, s);
-    if (cudaStreamSynchronize(s) != cudaSuccess) return MLMC_ERR_CUDA;  // the host arrays go out of scope below
-    launch_stopk_draw(ws, M, L, s_len, d, seed, step, s);
-    run_selection(ws, g, dtype, d, M, ld, 3, false, false, s);  // two queries per worker
-    launch_stopk_params(ws, M, s_len, d, out, s);
+    set_call_size(ws, d, M, dtype == MLMC_BF16 ? 2 : 4);
+    select_drawn(ws, g, dtype, d, M, ld, 3, false, seed, step, out, [&](double u) {
+        const int64_t l = std::upper_bound(cdf.begin(), cdf.end(), u) - cdf.begin();
+        const int64_t hi = s_len * (l + 1);
+        return DrawnBand{p[l] / sum, (int32_t)l, (uint32_t)(s_len * l), (uint32_t)(hi < d ? hi : d)};
+    }, s);
     launch_emit(ws, g, dtype, d, M, ld, *out, s);
     return finish(cudaGetLastError());
 }
@@ -617,9 +615,8 @@ int mlmc_compress_floatbits(mlmc_ctx* ctx, const void* g, int dtype, int64_t d, 
     Workspace& ws = ctx->ws;
     DeviceGuard guard(ws.device);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    cudaMemsetAsync(ws.worker_err, 0, sizeof(int) * M, s);
-    cudaMemcpyAsync(ws.p_fixed, pn, sizeof(double) * L, cudaMemcpyHostToDevice, s);
-    launch_compress_floatbits(ws, g, dtype, d, M, ld, mb, L, seed, step, *out, s);
+    set_call_size(ws, d, M, dtype == MLMC_BF16 ? 2 : 4);
+    launch_compress_floatbits(ws, g, dtype, d, M, ld, mb, L, pn, seed, step, *out, s);
     return finish(cudaGetLastError());
 }
 
@@ -635,6 +632,7 @@ int mlmc_aggregate_floatbits(mlmc_ctx* ctx, const mlmc_float_msgs* msgs, const i
         prev = mb[l];
     }
     DeviceGuard guard(ws.device);
+    set_call_size(ws, d, M, 4);
     launch_aggregate_floatbits(ws, *msgs, mb, L, M, d, out, static_cast<cudaStream_t>(stream));
     return finish(cudaGetLastError());
 }
@@ -652,12 +650,10 @@ int mlmc_compress_rtn(mlmc_ctx* ctx, const void* g, int dtype, int64_t d, int M,
     Workspace& ws = ctx->ws;
     DeviceGuard guard(ws.device);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    cudaMemsetAsync(ws.worker_err, 0, sizeof(int) * M, s);
-    const bool adaptive = (p == nullptr);
-    if (!adaptive) cudaMemcpyAsync(ws.p_fixed, pn, sizeof(double) * L, cudaMemcpyHostToDevice, s);
-    launch_absmax(ws, g, dtype, d, M, ld, s);  // c = max |g|, and the NaN / Inf check
-    if (adaptive) launch_rtn_stats(ws, g, dtype, d, M, ld, r32, L, s);
-    launch_rtn_probs_draw(ws, M, L, adaptive, adaptive, seed, step, out, s);
+    set_call_size(ws, d, M, dtype == MLMC_BF16 ? 2 : 4);
+    const DrawPlan plan = rtn_draw_plan(ws, L, seed, step, out);
+    launch_absmax(ws, g, dtype, d, M, ld, plan, p ? pn : nullptr, s);  // c = max |g|, and the NaN / Inf check
+    if (!p) launch_rtn_stats(ws, g, dtype, d, M, ld, r32, L, plan, s);
     launch_rtn_emit(ws, g, dtype, d, M, ld, r32, L, *out, s);
     return finish(cudaGetLastError());
 }
@@ -667,6 +663,7 @@ int mlmc_aggregate_rtn(mlmc_ctx* ctx, const mlmc_rtn_msgs* msgs, int M, int64_t 
     Workspace& ws = ctx->ws;
     if (d < 1 || d > ws.d_max || M < 1 || M > ws.M_max) return MLMC_ERR_ARG;
     DeviceGuard guard(ws.device);
+    set_call_size(ws, d, M, 4);
     launch_aggregate_dense(ws, msgs->val, msgs->level, M, d, msgs->ldv, out, static_cast<cudaStream_t>(stream));
     return finish(cudaGetLastError());
 }

@@ -51,65 +51,82 @@ struct Quantiser {
     }
 };
 
-// ---- per-worker max |g| as an integer max over magnitude keys; flags NaN / Inf
+// ---- per-worker max |g| as an integer max over magnitude keys; flags NaN / Inf.  With given probabilities (draw != 0)
+// the worker's last block also draws the level and writes the message header.
 template <typename T>
-__global__ void __launch_bounds__(kSweepThreads)
-absmax_kernel(const T* __restrict__ g, int64_t d, int64_t ld, uint32_t* gmax_bits, int* status, int* worker_err) {
+__global__ void __launch_bounds__(kSweepThreads, 3)
+absmax_kernel(const T* __restrict__ g, int64_t d, int64_t ld, uint32_t* gmax_bits, uint32_t* acc, uint32_t* done,
+              DrawPlan pl, ProbList given, int draw, int* status, int* worker_err) {
     using Tr = ElemTraits<T>;
     __shared__ uint32_t sh_max[kSweepThreads / 32];
+    pdl_enter();
     const int m = blockIdx.y;
     const T* row = g + (int64_t)m * ld;
-    int64_t v0, v1;
-    block_vector_range(d, Tr::kVec, blockIdx.x, gridDim.x, &v0, &v1);
     uint32_t mx = 0;
-    // four 16-byte loads per thread are in flight before any is used
+    // Chunks of kBatch vectors per thread, all in flight before any is used, dealt round-robin to the blocks of the worker.
+    // (One contiguous range per block ran between 0.75 and 1.0 of the copy rate, depending on the row length.)
     constexpr int kBatch = 4;
-    const int64_t full_end = min(v1, d / Tr::kVec);  // vectors wholly inside the row
-    int64_t v = v0 + threadIdx.x;
-    for (; v + (int64_t)(kBatch - 1) * blockDim.x < full_end; v += (int64_t)kBatch * blockDim.x) {
+    const int64_t nvec = (d + Tr::kVec - 1) / Tr::kVec, full_end = d / Tr::kVec;  // vectors of the row, and those wholly inside it
+    for (int64_t base = (int64_t)blockIdx.x * kBatch * kSweepThreads; base < nvec; base += (int64_t)gridDim.x * kBatch * kSweepThreads) {
+        const int64_t v = base + threadIdx.x;
+        if (base + kBatch * kSweepThreads > full_end) {  // the row's last chunk
+            for (int64_t u = v; u < nvec; u += kSweepThreads)
+                for_each_in_vector<T>(row, u, d, [&](int64_t, uint32_t bits) { mx = max(mx, Tr::key(bits)); });
+            break;
+        }
         uint4 q[kBatch];
 #pragma unroll
-        for (int j = 0; j < kBatch; ++j) q[j] = __ldg(reinterpret_cast<const uint4*>(row) + v + (int64_t)j * blockDim.x);
+        for (int j = 0; j < kBatch; ++j) q[j] = __ldg(reinterpret_cast<const uint4*>(row) + v + j * kSweepThreads);
 #pragma unroll
         for (int j = 0; j < kBatch; ++j) {
             if constexpr (Tr::kVec == 4) {
                 mx = max(max(mx, q[j].x & 0x7FFFFFFFu), max(q[j].y & 0x7FFFFFFFu, max(q[j].z & 0x7FFFFFFFu, q[j].w & 0x7FFFFFFFu)));
             } else {
-                // both halves at once: the low halves after masking, the high halves shifted down
-                const uint32_t a = max(max(q[j].x & 0x7FFFu, q[j].y & 0x7FFFu), max(q[j].z & 0x7FFFu, q[j].w & 0x7FFFu));
-                const uint32_t b = max(max((q[j].x >> 16) & 0x7FFFu, (q[j].y >> 16) & 0x7FFFu),
-                                       max((q[j].z >> 16) & 0x7FFFu, (q[j].w >> 16) & 0x7FFFu));
-                mx = max(mx, max(a, b));
+                const uint32_t a = __vmaxu2(__vmaxu2(q[j].x & 0x7FFF7FFFu, q[j].y & 0x7FFF7FFFu),
+                                            __vmaxu2(q[j].z & 0x7FFF7FFFu, q[j].w & 0x7FFF7FFFu));
+                mx = max(mx, max(a & 0xFFFFu, a >> 16));
             }
         }
     }
-    for (; v < v1; v += blockDim.x)
-        for_each_in_vector<T>(row, v, d, [&](int64_t, uint32_t bits) { mx = max(mx, Tr::key(bits)); });
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
     if ((threadIdx.x & 31) == 0) sh_max[threadIdx.x >> 5] = mx;
     __syncthreads();
     if (threadIdx.x == 0) {
         for (int w = 1; w < kSweepThreads / 32; ++w) mx = max(mx, sh_max[w]);
-        if (mx >= Tr::kInfKey) {
-            worker_err[m] = MLMC_ERR_NONFINITE;
-            set_status(status, MLMC_ERR_NONFINITE);
+        atomicMax(&acc[m], mx);
+    }
+    if (!last_block(&done[m], gridDim.x) || threadIdx.x != 0) return;
+    mx = __ldcg(&acc[m]);
+    acc[m] = 0u;
+    const uint32_t as_f32 = (Tr::kVec == 8) ? (mx << 16) : mx;
+    gmax_bits[m] = as_f32;
+    if (mx >= Tr::kInfKey) {
+        worker_err[m] = MLMC_ERR_NONFINITE;
+        set_status(status, MLMC_ERR_NONFINITE);
+        void_header(pl, m);
+    } else {
+        worker_err[m] = 0;
+        if (draw) {
+            draw_header(pl, m, given.p, __uint_as_float(as_f32), status, worker_err);
+            if (pl.bit_level[m] >= 0) pl.p_all[m * kMaxLevels + pl.bit_level[m]] = given.p[pl.bit_level[m]];
         }
-        const uint32_t as_f32 = (Tr::kVec == 8) ? (mx << 16) : mx;
-        atomicMax(&gmax_bits[m], as_f32);
     }
 }
 
-// ---- adaptive only: exact field energies S_l = sum_i f_l^2 for every level in one sweep
+// ---- adaptive only: exact field energies S_l = sum_i f_l^2 for every level in one sweep; the worker's last block turns
+// them into probabilities, draws the level and writes the message header.
 // Acc = uint32_t when every field is at most 8 bits wide and a thread sees fewer than 2^16 entries (f^2 < 2^16,
 // so the sum fits 32 bits), else unsigned long long.  Fields come from the prefix codes P_l = q >> (B - b_l):
 // f_l = P_l - (P_{l-1} << w_l), one shift and one multiply-add per level.
 template <typename T, int LMAX, typename Acc>
 __global__ void __launch_bounds__(kSweepThreads)
-bit_stats_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* __restrict__ gmax_bits,
-                 BitSchedule sc, unsigned long long* __restrict__ S_partial, int stat_ctas, const int* worker_err) {
+bit_stats_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* gmax_bits, BitSchedule sc,
+                 unsigned long long* S_partial, int stat_ctas, uint32_t* done, DrawPlan pl, int* status, int* worker_err) {
     using Tr = ElemTraits<T>;
     __shared__ unsigned long long sh_red[kSweepThreads / 32];
+    __shared__ double sh_delta[kMaxLevels], sh_p[kMaxLevels];
+    pdl_enter();
     const int m = blockIdx.y;
     if (worker_err[m]) return;
     const float gmax = __uint_as_float(gmax_bits[m]);
@@ -173,87 +190,24 @@ bit_stats_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t*
         }
         __syncthreads();
     }
-}
-
-__device__ int draw_level_bits(const double* p, int L, double u) {
-    int j_last = -1;
-    for (int j = 0; j < L; ++j)
-        if (p[j] > 0.0) j_last = j;
-    double c = 0.0;
-    for (int j = 0; j < L; ++j) {
-        c += p[j];
-        const double cdf = (j >= j_last) ? 1.0 : c;
-        if (u < cdf) return j;
-    }
-    return 0;
-}
-
-// ---- probabilities, draw and message header of every worker (one warp per worker)
-__global__ void bit_probs_draw_kernel(BitSchedule sc, const uint32_t* gmax_bits, const unsigned long long* S_partial,
-                                      int n_partials, int stat_ctas, const double* p_fixed, int adaptive,
-                                      int need_delta, uint64_t seed, uint64_t step, int M, double* p_all,
-                                      double* delta_all, double* u_dev, int32_t* bit_level, float* out_gmax,
-                                      int32_t* out_level, double* out_p_sel, int w_max, int want_msg, int* status,
-                                      int* worker_err) {
-    const int m = blockIdx.x;
-    const int lane = threadIdx.x;
-    if (m >= M) return;
-    if (worker_err[m]) {
-        if (lane == 0) {
-            bit_level[m] = -1;
-            if (want_msg) {
-                out_level[m] = -1;
-                out_p_sel[m] = 0.0;
-                out_gmax[m] = 0.0f;
-            }
-        }
-        return;
-    }
-    const float gmax = __uint_as_float(gmax_bits[m]);
-    double p[kMaxLevels], delta[kMaxLevels];
-    if (adaptive || need_delta) {
-        for (int l = 0; l < sc.L; ++l) {
-            // exact 128-bit sum of the per-block partials (lanes take every 32nd, integer adds: any order),
-            // rounded once to fp64
-            unsigned __int128 S = 0;
-            for (int c = lane; c < n_partials; c += 32) S += S_partial[((int64_t)m * stat_ctas + c) * kMaxLevels + l];
-            unsigned long long lo = (unsigned long long)S, hi = (unsigned long long)(S >> 64);
+    if (!last_block(&done[m], gridDim.x)) return;
+    // exact 128-bit sums of the per-block partials (integer adds: any order), rounded once to fp64; a warp per level
+    const int lane = threadIdx.x & 31;
+    for (int l = threadIdx.x >> 5; l < sc.L; l += kSweepThreads / 32) {
+        unsigned __int128 S = 0;
+        for (int c = lane; c < (int)gridDim.x; c += 32) S += __ldcg(&S_partial[((int64_t)m * stat_ctas + c) * kMaxLevels + l]);
+        unsigned long long lo = (unsigned long long)S, hi = (unsigned long long)(S >> 64);
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const unsigned long long lo2 = __shfl_xor_sync(0xFFFFFFFFu, lo, o), hi2 = __shfl_xor_sync(0xFFFFFFFFu, hi, o);
-                const unsigned __int128 t = (((unsigned __int128)hi << 64) | lo) + (((unsigned __int128)hi2 << 64) | lo2);
-                lo = (unsigned long long)t;
-                hi = (unsigned long long)(t >> 64);
-            }
-            const double Sd = (double)hi * 0x1.0p64 + (double)lo;
-            delta[l] = (double)gmax * ldexp(1.0, -sc.bits[l]) * sqrt(Sd);
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long lo2 = __shfl_xor_sync(0xFFFFFFFFu, lo, o), hi2 = __shfl_xor_sync(0xFFFFFFFFu, hi, o);
+            const unsigned __int128 t = (((unsigned __int128)hi << 64) | lo) + (((unsigned __int128)hi2 << 64) | lo2);
+            lo = (unsigned long long)t;
+            hi = (unsigned long long)(t >> 64);
         }
+        if (lane == 0) sh_delta[l] = (double)gmax * ldexp(1.0, -sc.bits[l]) * sqrt((double)hi * 0x1.0p64 + (double)lo);
     }
-    if (lane != 0) return;
-    if (adaptive || need_delta)
-        for (int l = 0; l < sc.L; ++l) delta_all[m * kMaxLevels + l] = delta[l];
-    if (adaptive) {
-        double s = 0.0;
-        for (int l = 0; l < sc.L; ++l) s += delta[l];
-        for (int l = 0; l < sc.L; ++l) p[l] = (s > 0.0) ? delta[l] / s : (l == 0 ? 1.0 : 0.0);
-    } else {
-        for (int l = 0; l < sc.L; ++l) p[l] = p_fixed[l];
-    }
-    for (int l = 0; l < sc.L; ++l) p_all[m * kMaxLevels + l] = p[l];
-    const double u = counter_uniform(seed, step, (uint64_t)m);
-    u_dev[m] = u;
-    int level = draw_level_bits(p, sc.L, u);
-    if (want_msg) {
-        if (sc.width[level] > w_max) {
-            worker_err[m] = MLMC_ERR_CAPACITY;
-            set_status(status, MLMC_ERR_CAPACITY);
-            level = -1;
-        }
-        out_level[m] = level;
-        out_p_sel[m] = (level >= 0) ? p[level] : 0.0;
-        out_gmax[m] = gmax;
-    }
-    bit_level[m] = level;
+    __syncthreads();
+    finish_levels(pl, m, sh_delta, sh_p, gmax, status, worker_err);
 }
 
 // ---- pack: every warp turns 1024 consecutive entries into 32 words of each plane.
@@ -264,9 +218,9 @@ __global__ void bit_probs_draw_kernel(BitSchedule sc, const uint32_t* gmax_bits,
 // path's 32 codes per lane would otherwise force on it.
 template <typename T, bool WIDE>
 __global__ void __launch_bounds__(kBitThreads, WIDE ? 2 : 3)
-bit_pack_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* __restrict__ gmax_bits,
-                BitSchedule sc, const int32_t* __restrict__ bit_level, uint32_t* __restrict__ planes, int w_max,
-                int64_t words) {
+bit_pack_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* gmax_bits, BitSchedule sc,
+                const int32_t* bit_level, uint32_t* __restrict__ planes, int w_max, int64_t words) {
+    pdl_enter();
     using Tr = ElemTraits<T>;
     constexpr int kGroup = 1024;
     constexpr int kGroupBytes = kGroup * (int)sizeof(T);
@@ -389,9 +343,9 @@ bit_pack_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* 
 
 // ---- server average of bit-plane messages: thread = one word (32 entries), staged through shared memory
 __global__ void __launch_bounds__(kBitThreads)
-aggregate_bitwise_kernel(const uint32_t* __restrict__ planes, const float* __restrict__ gmax,
-                         const int32_t* __restrict__ level, const double* __restrict__ p_sel, BitSchedule sc,
-                         int w_max, int64_t words, int M, int64_t d, float* __restrict__ out) {
+aggregate_bitwise_kernel(const uint32_t* __restrict__ planes, const float* gmax, const int32_t* level, const double* p_sel,
+                         BitSchedule sc, int w_max, int64_t words, int M, int64_t d, float* __restrict__ out) {
+    pdl_enter();
     __shared__ float sh_out[kBitThreads / 32][32][33];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const float inv_M = 1.0f / (float)M;
@@ -525,42 +479,49 @@ int configure_bit_kernels() {
     return MLMC_OK;
 }
 
-void launch_absmax(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, cudaStream_t s) {
-    cudaMemsetAsync(ws.gmax_bits, 0, (size_t)M * sizeof(uint32_t), s);
-    LaunchScope t(ws, K_ABSMAX, s);
-    if (dtype == MLMC_BF16) {
-        const int nb = bit_blocks(ws, d, 8, M, 8);
-        absmax_kernel<bf16_t><<<dim3(nb, M), kSweepThreads, 0, s>>>(static_cast<const bf16_t*>(g), d, ld, ws.gmax_bits,
-                                                                    ws.status, ws.worker_err);
-    } else {
-        const int nb = bit_blocks(ws, d, 4, M, 8);
-        absmax_kernel<float><<<dim3(nb, M), kSweepThreads, 0, s>>>(static_cast<const float*>(g), d, ld, ws.gmax_bits,
-                                                                   ws.status, ws.worker_err);
+DrawPlan bit_draw_plan(Workspace& ws, const int32_t* b, int L, uint64_t seed, uint64_t step, const mlmc_bit_msgs* out) {
+    DrawPlan pl = {};
+    pl.L = L;
+    for (int l = 0; l < L; ++l) pl.width[l] = b[l] - (l ? b[l - 1] : 0);
+    pl.seed = seed;
+    pl.step = step;
+    pl.bit_level = ws.bit_level;
+    pl.p_all = ws.p_all;
+    pl.delta_all = ws.delta_all;
+    if (out) {
+        pl.w_max = out->w_max;
+        pl.out_scale = out->gmax;
+        pl.out_level = out->level;
+        pl.out_p_sel = out->p_sel;
     }
+    return pl;
+}
+
+void launch_absmax(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const DrawPlan& plan, const double* p,
+                   cudaStream_t s) {
+    const int nb = bit_blocks(ws, d, dtype == MLMC_BF16 ? 8 : 4, M, 8);
+    auto go = [&](auto kernel, auto* row) {
+        launch_kernel(ws, K_ABSMAX, kernel, dim3(nb, M), kSweepThreads, 0, s, row, d, ld, ws.gmax_bits, ws.acc_word, ws.done,
+                      plan, prob_list(p, plan.L), p ? 1 : 0, ws.status, ws.worker_err);
+    };
+    if (dtype == MLMC_BF16) go(absmax_kernel<bf16_t>, static_cast<const bf16_t*>(g));
+    else go(absmax_kernel<float>, static_cast<const float*>(g));
 }
 
 template <typename T, typename Acc>
 static void launch_bit_stats_t(Workspace& ws, const T* g, int64_t d, int M, int64_t ld, const BitSchedule& sc, int nb,
-                               cudaStream_t s) {
-    dim3 grid(nb, M);
-#define MLMC_BIT_STATS(LM)                                                                                          \
-    bit_stats_kernel<T, LM, Acc><<<grid, kSweepThreads, 0, s>>>(g, d, ld, ws.gmax_bits, sc, ws.S_partial, ws.stat_ctas, \
-                                                               ws.worker_err)
-    if (sc.L <= 4) MLMC_BIT_STATS(4);
-    else if (sc.L <= 6) MLMC_BIT_STATS(6);
-    else if (sc.L <= 8) MLMC_BIT_STATS(8);
-    else if (sc.L <= 16) MLMC_BIT_STATS(16);
-    else MLMC_BIT_STATS(23);
-#undef MLMC_BIT_STATS
+                               const DrawPlan& plan, cudaStream_t s) {
+    auto kernel = sc.L <= 4 ? bit_stats_kernel<T, 4, Acc> : sc.L <= 6 ? bit_stats_kernel<T, 6, Acc> : sc.L <= 8 ? bit_stats_kernel<T, 8, Acc>
+                : sc.L <= 16 ? bit_stats_kernel<T, 16, Acc> : bit_stats_kernel<T, 23, Acc>;
+    launch_kernel(ws, K_BIT_STATS, kernel, dim3(nb, M), kSweepThreads, 0, s, g, d, ld, ws.gmax_bits, sc, ws.S_partial,
+                  ws.stat_ctas, ws.done, plan, ws.status, ws.worker_err);
 }
 
 void launch_bit_stats(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* b, int L,
-                      cudaStream_t s) {
+                      const DrawPlan& plan, cudaStream_t s) {
     const BitSchedule sc = make_schedule(b, L);
-    cudaMemsetAsync(ws.S_partial, 0, (size_t)M * ws.stat_ctas * kMaxLevels * sizeof(unsigned long long), s);
     int nb = bit_blocks(ws, d, dtype == MLMC_BF16 ? 8 : 4, M, 4);
     if (nb > ws.stat_ctas) nb = ws.stat_ctas;
-    ws.cur_stat_ctas = nb;
     // 32-bit sums are exact while f^2 < 2^16 and a thread adds fewer than 2^16 of them
     const int vec = dtype == MLMC_BF16 ? 8 : 4;
     const int64_t vec_per_block = ((d + vec - 1) / vec + nb - 1) / nb;
@@ -568,25 +529,13 @@ void launch_bit_stats(Workspace& ws, const void* g, int dtype, int64_t d, int M,
     int w_top = 0;
     for (int l = 0; l < L; ++l) w_top = sc.width[l] > w_top ? sc.width[l] : w_top;
     const bool narrow = w_top <= 8 && per_thread < 65536;
-    LaunchScope t(ws, K_BIT_STATS, s);
     if (dtype == MLMC_BF16) {
-        if (narrow) launch_bit_stats_t<bf16_t, uint32_t>(ws, static_cast<const bf16_t*>(g), d, M, ld, sc, nb, s);
-        else launch_bit_stats_t<bf16_t, unsigned long long>(ws, static_cast<const bf16_t*>(g), d, M, ld, sc, nb, s);
+        if (narrow) launch_bit_stats_t<bf16_t, uint32_t>(ws, static_cast<const bf16_t*>(g), d, M, ld, sc, nb, plan, s);
+        else launch_bit_stats_t<bf16_t, unsigned long long>(ws, static_cast<const bf16_t*>(g), d, M, ld, sc, nb, plan, s);
     } else {
-        if (narrow) launch_bit_stats_t<float, uint32_t>(ws, static_cast<const float*>(g), d, M, ld, sc, nb, s);
-        else launch_bit_stats_t<float, unsigned long long>(ws, static_cast<const float*>(g), d, M, ld, sc, nb, s);
+        if (narrow) launch_bit_stats_t<float, uint32_t>(ws, static_cast<const float*>(g), d, M, ld, sc, nb, plan, s);
+        else launch_bit_stats_t<float, unsigned long long>(ws, static_cast<const float*>(g), d, M, ld, sc, nb, plan, s);
     }
-}
-
-void launch_bit_probs_draw(Workspace& ws, int M, const int32_t* b, int L, bool adaptive, bool need_delta,
-                           uint64_t seed, uint64_t step, const mlmc_bit_msgs* out, cudaStream_t s) {
-    const BitSchedule sc = make_schedule(b, L);
-    LaunchScope t(ws, K_BIT_DRAW, s);
-    bit_probs_draw_kernel<<<M, 32, 0, s>>>(
-        sc, ws.gmax_bits, ws.S_partial, ws.cur_stat_ctas, ws.stat_ctas, ws.p_fixed, adaptive ? 1 : 0, need_delta ? 1 : 0,
-        seed, step, M, ws.p_all, ws.delta_all, ws.u_dev, ws.bit_level, out ? out->gmax : nullptr,
-        out ? out->level : nullptr, out ? out->p_sel : nullptr, out ? out->w_max : 0, out ? 1 : 0, ws.status,
-        ws.worker_err);
 }
 
 template <typename T>
@@ -605,17 +554,15 @@ static void launch_bit_pack_t(Workspace& ws, const T* g, int64_t d, int M, int64
         int64_t nb = ((int64_t)ws.sm_count * 3) / M;  // persistent: three resident blocks per SM, rounded down
         if (nb > by_work) nb = by_work;
         if (nb < 1) nb = 1;
-        LaunchScope t(ws, K_BIT_PACK, s);
-        bit_pack_kernel<T, false><<<dim3((unsigned)nb, M), kBitThreads, smem, s>>>(g, d, ld, ws.gmax_bits, sc, ws.bit_level,
-                                                                                out.planes, out.w_max, words);
+        launch_kernel(ws, K_BIT_PACK, bit_pack_kernel<T, false>, dim3((unsigned)nb, M), kBitThreads, smem, s, g, d, ld,
+                      ws.gmax_bits, sc, ws.bit_level, out.planes, out.w_max, words);
     }
     if (w_top > 8) {  // some level has a wider field
         int64_t nb = ((int64_t)ws.sm_count * 2) / M;  // two resident blocks per SM, rounded down
         if (nb > by_work) nb = by_work;
         if (nb < 1) nb = 1;
-        LaunchScope t(ws, K_BIT_PACK_WIDE, s);
-        bit_pack_kernel<T, true><<<dim3((unsigned)nb, M), kBitThreads, smem, s>>>(g, d, ld, ws.gmax_bits, sc, ws.bit_level,
-                                                                               out.planes, out.w_max, words);
+        launch_kernel(ws, K_BIT_PACK_WIDE, bit_pack_kernel<T, true>, dim3((unsigned)nb, M), kBitThreads, smem, s, g, d, ld,
+                      ws.gmax_bits, sc, ws.bit_level, out.planes, out.w_max, words);
     }
 }
 
@@ -634,15 +581,15 @@ void launch_aggregate_bitwise(Workspace& ws, const mlmc_bit_msgs& msgs, const in
     const int64_t words = (d + 31) / 32;
     int64_t nb = (words + kBitThreads - 1) / kBitThreads;
     // whole waves only: every block does the same number of iterations, so a partial last wave costs a full one
-    int resident = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, aggregate_bitwise_kernel, kBitThreads, 0) != cudaSuccess ||
-        resident < 1)
-        resident = 1;
+    static const int resident = [] {
+        int n = 0;
+        const bool ok = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, aggregate_bitwise_kernel, kBitThreads, 0) == cudaSuccess;
+        return ok && n >= 1 ? n : 1;
+    }();
     const int64_t cap = (int64_t)ws.sm_count * resident * 2;
     if (nb > cap) nb = cap;
-    LaunchScope t(ws, K_AGG_BIT, s);
-    aggregate_bitwise_kernel<<<(unsigned)nb, kBitThreads, 0, s>>>(msgs.planes, msgs.gmax, msgs.level, msgs.p_sel, sc,
-                                                                  msgs.w_max, words, M, d, out);
+    launch_kernel(ws, K_AGG_BIT, aggregate_bitwise_kernel, dim3((unsigned)nb), kBitThreads, 0, s, msgs.planes, msgs.gmax,
+                  msgs.level, msgs.p_sel, sc, msgs.w_max, words, M, d, out);
 }
 
 }  // namespace mlmc

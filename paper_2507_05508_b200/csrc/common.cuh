@@ -23,6 +23,10 @@ constexpr int kEmitTile = 4096;               // 32-bit words per emit tile (1 f
 constexpr int kEmitTileVecs = kEmitTile / 4;  // 16-byte vectors per tile, for both element types
 constexpr int kEmitGroups = kEmitTile / (kEmitRows * 32);  // batches of kEmitRows * 32 words per tile: 8
 constexpr int kEmitGroupVecs = kEmitTileVecs / kEmitGroups;  // 16-byte vectors per batch: 128
+constexpr int kItemTiles = 4;                 // emit tiles per item of the band count: one batch per lane of a warp
+constexpr int kSuperItems = 32;               // items per super-item, super-items per hyper-item: their counts are added up too
+constexpr int kTileBits = 21;                 // of a listed tile: at most 2^20 tiles per worker (d < 2^32)
+constexpr int kEnergyCells = 2 * kMaxLevels;  // (boundary bin, interval) pairs: at most 31 bins, each threshold adds one interval
 constexpr int kAggTile = 4096;                // dense output elements per aggregation tile
 
 // Per-worker selection query: the rank-k element of the total order.
@@ -36,7 +40,8 @@ struct Query {
     uint32_t n;        // #{ key == T }
     uint32_t r;        // how many key == T elements, in index order, are inside Top-k  (k - c)
     uint32_t trivial;  // 1: k == 0 (nothing inside), 2: k >= d (everything inside), 0: live
-    uint32_t pad[3];
+    uint32_t slot2;    // histogram slot of the second digit pass = index of the boundary bin among the distinct ones
+    uint32_t pad[2];
 };
 
 // Emit parameters of one worker, produced by the draw kernel.
@@ -52,12 +57,21 @@ struct EmitParams {
 
 // Kernel identifiers for launch accounting and per-kernel timing.
 enum KernelId {
-    K_DRAW_FIXED = 0, K_INIT_QUERIES, K_UNIFORMS, K_HIST1, K_RESOLVE1, K_SUMS_CAND, K_CAND2, K_MASKED2, K_RESOLVE2, K_CAND3,
-    K_MASKED3, K_RESOLVE3, K_CAND_SUMS, K_NORM_SWEEP, K_NORM_HIST, K_PROBS_DRAW, K_COPY_PROBS, K_EMIT, K_AGG_OFFSETS, K_AGG_TOPK,
-    K_ABSMAX, K_BIT_STATS, K_BIT_DRAW, K_BIT_PACK, K_AGG_BIT, K_TILE_LIST, K_BAND_COUNT, K_BAND_SCAN, K_BIT_PACK_WIDE, K_RESET,
-    K_FLOAT_DRAW, K_FLOAT_PACK, K_AGG_FLOAT, K_RTN_STATS, K_RTN_DRAW, K_RTN_EMIT, K_AGG_DENSE, K_STOPK_DRAW, K_STOPK_PARAMS,
-    K_SORT_COUNT, K_SORT_SCAN, K_SORT_SCATTER, K_SEG_NORMS, K_COUNT
+    K_BEGIN = 0, K_UNIFORMS, K_HIST1, K_RESOLVE1, K_SUMS_CAND, K_CAND2, K_CAND3, K_BAND_HEADER, K_COPY_PROBS, K_EMIT, K_AGG_OFFSETS,
+    K_AGG_TOPK, K_ABSMAX, K_BIT_STATS, K_BIT_PACK, K_AGG_BIT, K_TILE_LIST, K_BAND_COUNT, K_BIT_PACK_WIDE, K_FLOAT_PACK, K_AGG_FLOAT,
+    K_RTN_STATS, K_RTN_EMIT, K_AGG_DENSE, K_STOPK_DRAW, K_SORT_COUNT, K_SORT_SCAN, K_SORT_SCATTER, K_SEG_NORMS, K_COUNT
 };
+
+// Level probabilities handed to a kernel by value.
+struct ProbList {
+    double p[kMaxLevels];
+};
+inline ProbList prob_list(const double* p, int L) {
+    ProbList r = {};
+    if (p)
+        for (int l = 0; l < L; ++l) r.p[l] = p[l];
+    return r;
+}
 
 constexpr int kTimingPool = 2048;  // event pairs kept between two reads
 
@@ -74,44 +88,44 @@ struct Workspace {
     int M_max, L_max;
     int sm_count;
     int64_t launches;
+    bool long_sweeps;            // this call's sweeps are long enough to be launched without overlap (see launch_kernel)
     // device memory
     int* status;                 // sticky status word
     int* worker_err;             // [M] per-worker device error (0 = fine)
     uint32_t* hist1;             // [M][kBins1]  counts, then suffix sums in place
     uint8_t* table1;             // [M][kBins1]  leading-digit bin -> slot of pass 2
-    uint32_t* hist2;             // [M][kMaxQueries][256]
-    uint8_t* map2;               // [M][kMaxQueries][256] (slot2, digit2) -> slot of pass 3
+    uint32_t* hist2;             // [M][kMaxQueries][256], hist3 behind it
+    uint8_t* map2;               // [M][kMaxQueries][256] (slot2, digit2) -> slot of pass 3, or 64 + energy cell
     uint32_t* hist3;             // [M][kMaxQueries][256]
     Query* queries;              // [M][kMaxQueries]
-    double* band_partial;        // [M][norm_ctas][kMaxLevels] per-block open-interval sums (full sweep / bf16)
-    int norm_ctas, cur_norm_ctas;
+    uint32_t* done;              // [M] blocks of a worker that have finished (every kernel that counts leaves it at zero)
     double* sum_partial;         // [M][sum_ctas][kMaxLevels]  sweep 2: energy of the threshold-free bins
     int sum_ctas, cur_sum_ctas;
-    unsigned long long* cand_S;  // [M][kMaxLevels][2 sides][2 halves] integer energy sums of the candidate keys
+    unsigned long long* cand_S;  // [M][kEnergyCells][2 halves] integer energy sums of the boundary-bin keys outside the threshold sub-bins
     uint32_t* cand_keys;         // [M][cand_cap] keys of the boundary-bin elements
     int64_t cand_cap;
     uint32_t* cand_count;        // [M]
     int* cand_overflow;          // [M] 1: the candidates did not fit, full-sweep passes take over
-    int64_t* k_dev;              // [kMaxLevels] schedule
-    double* p_fixed;             // [kMaxLevels] normalised fixed p
     double* p_all;               // [M][kMaxLevels]
     double* delta_all;           // [M][kMaxLevels]
-    double* u_dev;               // [M]
+    double* u_dev;               // [M] (mlmc_read_u)
     EmitParams* emit;            // [M]
-    uint4* tile_desc;            // [M][tiles per worker] per listed tile {C, A, B}: its own counts, then the running totals before it
+    uint4* tile_desc;            // [M][tiles per worker] {C, A, B, tie flag} of every emit tile
+    uint4* level_desc;           // {C, A, B, batches} of every item [M][items], then super-item, then hyper-item
+    uint2* tile_list;            // the tiles of all workers that can hold band entries, in any order: {worker << kTileBits | tile, batch mask}
+    uint32_t* list_n;            // how many
     int64_t max_tiles;
     uint32_t* tile_max;          // [M][tiles per worker][kEmitGroups] largest magnitude key of every batch of every emit tile (sweep 1)
-    uint32_t* worker_tiles;      // [M][tiles per worker] the tiles of a worker that can hold band entries, ascending: tile | batch mask << 24
-    uint32_t* tile_n;            // [M] how many of them
-    uint32_t* group_n;           // [M] how many batches they have to read
+    uint32_t* group_n;           // [M] how many batches the last emission had to read
     int64_t last_emit_tiles;     // tiles per row of the last emission (host side, for mlmc_read_listed_tiles)
     uint32_t* cand_floor;        // [M] smallest key that can be a candidate of sweep 2 (lower edge of the lowest boundary bin)
     uint32_t* agg_offsets;       // [M][agg_tiles_max + 1]
     // bit-wise
     uint32_t* gmax_bits;         // [M]
+    uint32_t* acc_word;          // [M] running maximum (or error flag) of a sweep; its last block leaves it at zero
     unsigned long long* S_partial;  // [M][stat_ctas][kMaxLevels]
-    int stat_ctas, cur_stat_ctas;
-    int32_t* bit_level;          // [M] (mirrors out->level for the pack kernel)
+    int stat_ctas;
+    int32_t* bit_level;          // [M] drawn level of a dense message (-1: void), read by the kernel that writes it
     // fixed-p Top-k: boundary bins of the previous call, per worker and level boundary, reused as brackets
     uint32_t* prev_bin;          // [M][kMaxLevels] leading-digit bin of threshold j at the last call that resolved it (kKeyNone: none)
     uint4* bracket;              // [M] {lo_a, width_a, lo_b, width_b}: bins collected as candidates by the first sweep
@@ -120,15 +134,27 @@ struct Workspace {
     int64_t sig_d, sig_ld;       // host: the problem the stored bins belong to
     int sig_M, sig_L, sig_dtype;
     int64_t sig_k[kMaxLevels];
-    // s-Top-k with more levels than kMaxLevels (fixed p only): normalised p and its running sums
-    double* p_big;               // [big_cap]
-    double* cdf_big;             // [big_cap]
-    int64_t big_cap;
+    // s-Top-k with more levels than kMaxLevels
+    int64_t big_cap;             // most levels
     uint32_t* sort_scratch;      // key buffers, digit tables and segment norms of the radix sort, for sort_rows rows; allocated at first use
     int sort_rows;               // rows that are sorted together
     // RTN: per-block residual energies of every level
     double* rtn_partial;         // [M][rtn_ctas][kMaxLevels]
-    int rtn_ctas, cur_rtn_ctas;
+    int rtn_ctas;
+};
+
+// Level draw and message header of the dense compressors (bit planes, RTN).
+struct DrawPlan {
+    int L;
+    int w_max;                  // planes of the message buffer; width[l] of them are needed (RTN: all 0)
+    int width[kMaxLevels];
+    uint64_t seed, step;
+    int32_t* bit_level;
+    double* p_all;
+    double* delta_all;
+    float* out_scale;           // null: no message (mlmc_level_probs)
+    int32_t* out_level;
+    double* out_p_sel;
 };
 
 // ---------------------------------------------------------------------------------------------
@@ -136,14 +162,38 @@ struct Workspace {
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ void set_status(int* status, int code) { atomicCAS(status, 0, code); }
 
-__device__ __forceinline__ uint64_t splitmix_finalize(uint64_t z) {
+// Every kernel of the library starts with pdl_enter().  The kernels are launched with programmatic stream
+// serialization, so a kernel's blocks may become resident while the kernel before it in the stream is still running;
+// nothing is read or written before the wait, which returns when that kernel has completed and its writes are visible.
+// A chain of short kernels then pays about 1 us per launch instead of 3 to 4.
+__device__ __forceinline__ void pdl_enter() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// True in every thread of the one block of `nblocks` that gets here last: what the other blocks wrote before is
+// visible to it (read with __ldcg).  No block waits for another.  The counter is left at zero for the next kernel.
+__device__ __forceinline__ bool last_block(uint32_t* counter, uint32_t nblocks) {
+    __shared__ bool sh_last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        sh_last = atomicAdd(counter, 1u) == nblocks - 1u;
+        if (sh_last) *counter = 0u;
+        __threadfence();
+    }
+    __syncthreads();
+    return sh_last;
+}
+
+__host__ __device__ __forceinline__ uint64_t splitmix_finalize(uint64_t z) {
     z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
     z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
     return z ^ (z >> 31);
 }
 
 // One uniform in [0,1) per (seed, step, worker): three chained SplitMix64 output rounds.
-__device__ __forceinline__ double counter_uniform(uint64_t seed, uint64_t step, uint64_t worker) {
+__host__ __device__ __forceinline__ double counter_uniform(uint64_t seed, uint64_t step, uint64_t worker) {
     const uint64_t golden = 0x9E3779B97F4A7C15ull;
     uint64_t h = splitmix_finalize(seed + golden);
     h = splitmix_finalize(h + step + golden);
@@ -153,7 +203,7 @@ __device__ __forceinline__ double counter_uniform(uint64_t seed, uint64_t step, 
 
 // cdf in ascending l; the last level with p > 0 and everything after it has cdf 1; l* = min{l : u < cdf_l}
 // ("Sample l ~ p^l", Alg. 2 / Alg. 3).
-__device__ __forceinline__ int draw_from_probs(const double* p, int L, double u) {
+__host__ __device__ __forceinline__ int draw_from_probs(const double* p, int L, double u) {
     int j_last = -1;
     for (int j = 0; j < L; ++j)
         if (p[j] > 0.0) j_last = j;
@@ -164,6 +214,54 @@ __device__ __forceinline__ int draw_from_probs(const double* p, int L, double u)
         if (u < cdf) return j;
     }
     return 0;
+}
+
+// End of the level statistics of one worker, by one thread: the draw and the message header.
+__device__ __forceinline__ void draw_header(const DrawPlan& pl, int m, const double* p, float scale, int* status, int* worker_err) {
+    int level = draw_from_probs(p, pl.L, counter_uniform(pl.seed, pl.step, (uint64_t)m));
+    const double p_sel = p[level];
+    if (pl.out_level) {
+        if (pl.width[level] > pl.w_max) {
+            worker_err[m] = MLMC_ERR_CAPACITY;
+            set_status(status, MLMC_ERR_CAPACITY);
+            level = -1;
+        }
+        pl.out_level[m] = level;
+        pl.out_p_sel[m] = level >= 0 ? p_sel : 0.0;
+        pl.out_scale[m] = scale;
+    }
+    pl.bit_level[m] = level;
+}
+
+__device__ __forceinline__ void void_header(const DrawPlan& pl, int m) {
+    pl.bit_level[m] = -1;
+    if (pl.out_level) {
+        pl.out_level[m] = -1;
+        pl.out_p_sel[m] = 0.0;
+        pl.out_scale[m] = 0.0f;
+    }
+}
+
+// Probabilities from the residual norms sh_delta[L] of one worker (Lemma 3.4), the draw and the header; by the whole block.
+__device__ __forceinline__ void finish_levels(const DrawPlan& pl, int m, const double* sh_delta, double* sh_p, float scale,
+                                              int* status, int* worker_err) {
+    __shared__ double sh_total;
+    if (threadIdx.x == 0) {
+        double s = 0.0;
+        for (int l = 0; l < pl.L; ++l) s += sh_delta[l];
+        sh_total = s;
+    }
+    __syncthreads();
+    if (threadIdx.x < pl.L) {
+        const int l = threadIdx.x;
+        const double s = sh_total;
+        const double p = (s > 0.0) ? sh_delta[l] / s : (l == 0 ? 1.0 : 0.0);
+        sh_p[l] = p;
+        pl.delta_all[m * kMaxLevels + l] = sh_delta[l];
+        pl.p_all[m * kMaxLevels + l] = p;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) draw_header(pl, m, sh_p, scale, status, worker_err);
 }
 
 // Magnitude key: monotone in |g| for finite values.  fp32: 31 bits; bf16: 15 bits.
@@ -251,6 +349,18 @@ inline int emit_tiles_per_worker(int64_t d, int dtype) {
     return (int)((words + kEmitTile - 1) / kEmitTile);
 }
 
+struct EmitCounts {
+    int items, supers, hypers;  // per worker
+    int total() const { return items + supers + hypers; }
+};
+inline EmitCounts emit_counts(int tiles) {
+    EmitCounts n;
+    n.items = (tiles + kItemTiles - 1) / kItemTiles;
+    n.supers = (n.items + kSuperItems - 1) / kSuperItems;
+    n.hypers = (n.supers + kSuperItems - 1) / kSuperItems;
+    return n;
+}
+
 // Brackets one kernel launch: counts it and, when timing is on, records an event pair on the stream.
 struct LaunchScope {
     Workspace& ws;
@@ -270,26 +380,77 @@ struct LaunchScope {
     }
 };
 
+// Kernels that stream the gradients or the messages.
+inline bool is_sweep(int id) {
+    switch (id) {
+        case K_HIST1: case K_SUMS_CAND: case K_BAND_COUNT: case K_EMIT: case K_AGG_TOPK: case K_ABSMAX: case K_BIT_STATS:
+        case K_BIT_PACK: case K_BIT_PACK_WIDE: case K_AGG_BIT: case K_FLOAT_PACK: case K_AGG_FLOAT: case K_RTN_STATS:
+        case K_RTN_EMIT: case K_AGG_DENSE:
+            return true;
+        default:
+            return false;
+    }
+}
+
+// Enqueues one kernel, with programmatic stream serialization (see pdl_enter) unless it is a long sweep.  Blocks that
+// become resident beside the last blocks of the kernel before them inherit its split of L1 and shared memory, and a
+// sweep with a small L1 keeps fewer loads in flight: on 4 GB that cost 5 to 10 % of the sweep (bit-wise step 3.00 ->
+// 3.27 ms, Top-k step 2.33 -> 2.49 ms), where the overlap gains 2 us a launch; the two meet at about 100 MB.
+constexpr int64_t kLongSweepBytes = 100 << 20;
+inline void set_call_size(Workspace& ws, int64_t d, int M, int elem_size) { ws.long_sweeps = d * M * elem_size > kLongSweepBytes; }
+
+template <typename... P, typename... A>
+inline void launch_kernel(Workspace& ws, int id, void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s,
+                          A&&... args) {
+    LaunchScope t(ws, id, s);
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = (ws.long_sweeps && is_sweep(id)) ? 0 : 1;
+    cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // ---------------------------------------------------------------------------------------------
 // launchers (each enqueues on `s` and bumps ws.launches)
 // ---------------------------------------------------------------------------------------------
 // topk_select.cu
 int configure_select_kernels();
-void launch_init_queries_adaptive(Workspace& ws, int M, int L, int64_t d, cudaStream_t s);
-void launch_draw_fixed(Workspace& ws, int M, int L, int64_t d, uint64_t seed, uint64_t step, bool brackets,
-                       cudaStream_t s);
+// One worker of a call whose level is drawn on the host (given p): the level, its probability and the two ranks that
+// bound its band.
+struct DrawnBand {
+    double p;
+    int32_t level;
+    uint32_t k_lo, k_hi;
+};
+void launch_begin_adaptive(Workspace& ws, int dtype, int64_t d, int M, const int64_t* k, int L, cudaStream_t s);
+void launch_begin_drawn(Workspace& ws, int dtype, int64_t d, int M, const DrawnBand* bands, int L, bool brackets, cudaStream_t s);
 void launch_uniforms(Workspace& ws, int M, uint64_t seed, uint64_t step, cudaStream_t s);
-void launch_reset_selection(Workspace& ws, int dtype, int64_t d, int M, cudaStream_t s);
 void launch_hist1(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, bool brackets, cudaStream_t s);
-void launch_resolve1(Workspace& ws, int dtype, int M, int L, bool brackets, cudaStream_t s);
-void launch_sums_candidates(Workspace& ws, const void* g, int64_t d, int M, int64_t ld, int L, bool sums,
-                            bool brackets, cudaStream_t s);
-void launch_digit_pass(Workspace& ws, const void* g, int64_t d, int M, int64_t ld, int pass, cudaStream_t s);
-void launch_resolve23(Workspace& ws, int M, int L, int pass, cudaStream_t s);
-void launch_band_norms_fp32(Workspace& ws, const void* g, int64_t d, int M, int64_t ld, int L, cudaStream_t s);
-void launch_norm_from_hist_bf16(Workspace& ws, int M, int L, cudaStream_t s);
-void launch_probs_draw(Workspace& ws, int dtype, int M, int L, int64_t d, bool adaptive, bool want_emit,
-                       uint64_t seed, uint64_t step, const mlmc_topk_msgs* out, cudaStream_t s);
+// What the last kernel of a selection does with its thresholds.
+struct FinishPlan {
+    int L;              // levels; queries are the L - 1 boundaries (adaptive) or the two of the drawn band
+    int nq;
+    int adaptive;       // energies, probabilities and the draw
+    int want_emit;      // message header and emit parameters
+    int64_t d;
+    uint64_t seed, step;
+    uint32_t k[kMaxLevels];
+    int64_t* out_count;
+    int32_t* out_level;
+    double* out_p_sel;
+    int64_t capacity;
+};
+void launch_resolve1(Workspace& ws, int dtype, int M, const FinishPlan& plan, bool brackets, cudaStream_t s);
+void launch_sums_candidates(Workspace& ws, const void* g, int64_t d, int M, int64_t ld, const FinishPlan& plan, bool brackets,
+                            cudaStream_t s);
+void launch_digit_passes(Workspace& ws, const void* g, int64_t d, int M, int64_t ld, const FinishPlan& plan, cudaStream_t s);
+void launch_band_header(Workspace& ws, int M, const FinishPlan& plan, cudaStream_t s);
 void launch_copy_probs(Workspace& ws, int M, int L, const double* p_fixed, double* p_out, double* delta_out,
                        cudaStream_t s);
 // topk_emit.cu
@@ -299,11 +460,13 @@ void launch_emit(Workspace& ws, const void* g, int dtype, int64_t d, int M, int6
 void launch_aggregate_topk(Workspace& ws, const mlmc_topk_msgs& msgs, int M, int64_t d, float* out, cudaStream_t s);
 // bitwise.cu
 int configure_bit_kernels();
-void launch_absmax(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, cudaStream_t s);
+// Largest magnitude of every worker and the NaN / Inf check; with `p` (given probabilities) also the draw and the header.
+void launch_absmax(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const DrawPlan& plan, const double* p,
+                   cudaStream_t s);
+DrawPlan bit_draw_plan(Workspace& ws, const int32_t* b, int L, uint64_t seed, uint64_t step, const mlmc_bit_msgs* out);
+// Adaptive: field energies of every level, probabilities, draw and header.
 void launch_bit_stats(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* b, int L,
-                      cudaStream_t s);
-void launch_bit_probs_draw(Workspace& ws, int M, const int32_t* b, int L, bool adaptive, bool need_delta,
-                           uint64_t seed, uint64_t step, const mlmc_bit_msgs* out, cudaStream_t s);
+                      const DrawPlan& plan, cudaStream_t s);
 void launch_bit_pack(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* b, int L,
                      const mlmc_bit_msgs& out, cudaStream_t s);
 void launch_aggregate_bitwise(Workspace& ws, const mlmc_bit_msgs& msgs, const int32_t* b, int L, int M, int64_t d,
@@ -311,22 +474,18 @@ void launch_aggregate_bitwise(Workspace& ws, const mlmc_bit_msgs& msgs, const in
 
 // floatbits.cu
 void launch_compress_floatbits(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* mb,
-                               int L, uint64_t seed, uint64_t step, const mlmc_float_msgs& out, cudaStream_t s);
+                               int L, const double* p, uint64_t seed, uint64_t step, const mlmc_float_msgs& out, cudaStream_t s);
 void launch_aggregate_floatbits(Workspace& ws, const mlmc_float_msgs& msgs, const int32_t* mb, int L, int M, int64_t d,
                                 float* out, cudaStream_t s);
 // rtn.cu
+DrawPlan rtn_draw_plan(Workspace& ws, int L, uint64_t seed, uint64_t step, const mlmc_rtn_msgs* out);
+// Adaptive: residual energies of every level, probabilities, draw and header.
 void launch_rtn_stats(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* r, int L,
-                      cudaStream_t s);
-void launch_rtn_probs_draw(Workspace& ws, int M, int L, bool adaptive, bool have_stats, uint64_t seed, uint64_t step,
-                           const mlmc_rtn_msgs* out, cudaStream_t s);
+                      const DrawPlan& plan, cudaStream_t s);
 void launch_rtn_emit(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* r, int L,
                      const mlmc_rtn_msgs& out, cudaStream_t s);
 void launch_aggregate_dense(Workspace& ws, const float* val, const int32_t* level, int M, int64_t d, int64_t ldv,
                             float* out, cudaStream_t s);
-// topk_select.cu: s-Top-k with many levels (fixed p)
-void launch_stopk_draw(Workspace& ws, int M, int64_t L, int64_t s_len, int64_t d, uint64_t seed, uint64_t step,
-                       cudaStream_t s);
-void launch_stopk_params(Workspace& ws, int M, int64_t s_len, int64_t d, const mlmc_topk_msgs* out, cudaStream_t s);
 // stopk_sort.cu: s-Top-k with adaptive p and many segments
 int configure_sort_kernels();
 int stopk_sort_rows(int64_t d_max, int64_t big_cap, int M_max);

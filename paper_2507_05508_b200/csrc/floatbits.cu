@@ -29,38 +29,30 @@ MantissaSchedule make_mantissa_schedule(const int32_t* mb, int L) {
     return sc;
 }
 
-// Level and header of every worker.
-__global__ void float_draw_kernel(const double* __restrict__ p_fixed, MantissaSchedule sc, uint64_t seed, uint64_t step,
-                                  int M, int w_max, double* u_dev, int32_t* bit_level, int32_t* out_level,
-                                  double* out_p_sel, int* status, int* worker_err) {
-    const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= M) return;
-    const double u = counter_uniform(seed, step, (uint64_t)m);
-    u_dev[m] = u;
-    int level = draw_from_probs(p_fixed, sc.L, u);
-    const double p = p_fixed[level];
-    if (sc.hi[level] - sc.lo[level] > w_max) {
-        worker_err[m] = MLMC_ERR_CAPACITY;
-        set_status(status, MLMC_ERR_CAPACITY);
-        level = -1;
-    }
-    bit_level[m] = level;
-    out_level[m] = level;
-    out_p_sel[m] = level >= 0 ? p : 0.0;
-}
-
 // Every warp turns 1024 consecutive entries into 32 words of the sign plane and of each mantissa plane (one warp
 // ballot per row of 32 entries and plane), and into 1024 exponent bytes, which leave through a shared-memory
 // transpose as 32 consecutive bytes per lane.  All 32 rows of a group are requested before the first is used.
+// The draw does not depend on the data: every block makes it itself; the worker's last block writes the header.
 template <typename T>
-__global__ void __launch_bounds__(kFloatThreads)
-float_pack_kernel(const T* __restrict__ g, int64_t d, int64_t ld, MantissaSchedule sc,
-                  const int32_t* __restrict__ bit_level, uint8_t* __restrict__ expo, uint32_t* __restrict__ planes,
-                  int w_max, int64_t words, int32_t* out_level, int* status, int* worker_err) {
+__global__ void __launch_bounds__(kFloatThreads, 3)
+float_pack_kernel(const T* __restrict__ g, int64_t d, int64_t ld, MantissaSchedule sc, ProbList p, uint64_t seed,
+                  uint64_t step, uint8_t* __restrict__ expo, uint32_t* __restrict__ planes, int w_max, int64_t words,
+                  int32_t* out_level, double* out_p_sel, uint32_t* acc, uint32_t* done, int* status) {
     __shared__ __align__(16) uint8_t sh_expo[kFloatThreads / 32][1024];
+    __shared__ int sh_level;
     const int m = blockIdx.y;
-    const int level = bit_level[m];
-    if (level < 0) return;
+    if (threadIdx.x == 0) sh_level = draw_from_probs(p.p, sc.L, counter_uniform(seed, step, (uint64_t)m));
+    __syncthreads();
+    pdl_enter();
+    const int level = sh_level;
+    if (sc.hi[level] - sc.lo[level] > w_max) {  // the field does not fit the message buffer
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            set_status(status, MLMC_ERR_CAPACITY);
+            out_level[m] = -1;
+            out_p_sel[m] = 0.0;
+        }
+        return;
+    }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int lo = sc.lo[level], w = sc.hi[level] - lo;
     const T* row = g + (int64_t)m * ld;
@@ -123,18 +115,21 @@ float_pack_kernel(const T* __restrict__ g, int64_t d, int64_t ld, MantissaSchedu
         }
         __syncwarp();
     }
-    if (bad) {  // NaN or Inf: the worker's message is void
-        worker_err[m] = MLMC_ERR_NONFINITE;
-        set_status(status, MLMC_ERR_NONFINITE);
-        out_level[m] = -1;
-    }
+    if (bad) atomicOr(&acc[m], 1u);
+    if (!last_block(&done[m], gridDim.x) || threadIdx.x != 0) return;
+    const bool any_bad = __ldcg(&acc[m]) != 0u;  // NaN or Inf: the worker's message is void
+    acc[m] = 0u;
+    if (any_bad) set_status(status, MLMC_ERR_NONFINITE);
+    out_level[m] = any_bad ? -1 : level;
+    out_p_sel[m] = p.p[level];
 }
 
 // Server average: thread = one word (32 entries); terms are added in worker order in fp32.
 __global__ void __launch_bounds__(kFloatThreads)
-aggregate_float_kernel(const uint8_t* __restrict__ expo, const uint32_t* __restrict__ planes,
-                       const int32_t* __restrict__ level, const double* __restrict__ p_sel, MantissaSchedule sc,
-                       int w_max, int64_t words, int M, int64_t d, float* __restrict__ out) {
+aggregate_float_kernel(const uint8_t* __restrict__ expo, const uint32_t* __restrict__ planes, const int32_t* level,
+                       const double* p_sel, MantissaSchedule sc, int w_max, int64_t words, int M, int64_t d,
+                       float* __restrict__ out) {
+    pdl_enter();
     __shared__ float sh_out[kFloatThreads / 32][32][33];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const float inv_M = 1.0f / (float)M;
@@ -191,28 +186,21 @@ aggregate_float_kernel(const uint8_t* __restrict__ expo, const uint32_t* __restr
 }  // namespace
 
 void launch_compress_floatbits(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* mb,
-                               int L, uint64_t seed, uint64_t step, const mlmc_float_msgs& out, cudaStream_t s) {
+                               int L, const double* p, uint64_t seed, uint64_t step, const mlmc_float_msgs& out,
+                               cudaStream_t s) {
     const MantissaSchedule sc = make_mantissa_schedule(mb, L);
-    {
-        LaunchScope t(ws, K_FLOAT_DRAW, s);
-        float_draw_kernel<<<(M + 127) / 128, 128, 0, s>>>(ws.p_fixed, sc, seed, step, M, out.w_max, ws.u_dev, ws.bit_level,
-                                                          out.level, out.p_sel, ws.status, ws.worker_err);
-    }
     const int64_t words = (d + 31) / 32;
     const int64_t ngroups = (words + 31) / 32;
     const int64_t by_work = (ngroups + (kFloatThreads / 32) - 1) / (kFloatThreads / 32);
     int64_t nb = ((int64_t)ws.sm_count * 4) / M;  // whole waves of the blocks that fit an SM, rounded down
     if (nb > by_work) nb = by_work;
     if (nb < 1) nb = 1;
-    LaunchScope t(ws, K_FLOAT_PACK, s);
-    if (dtype == MLMC_BF16)
-        float_pack_kernel<bf16_t><<<dim3((unsigned)nb, M), kFloatThreads, 0, s>>>(
-            static_cast<const bf16_t*>(g), d, ld, sc, ws.bit_level, out.expo, out.planes, out.w_max, words, out.level,
-            ws.status, ws.worker_err);
-    else
-        float_pack_kernel<float><<<dim3((unsigned)nb, M), kFloatThreads, 0, s>>>(
-            static_cast<const float*>(g), d, ld, sc, ws.bit_level, out.expo, out.planes, out.w_max, words, out.level,
-            ws.status, ws.worker_err);
+    auto go = [&](auto kernel, auto* row) {
+        launch_kernel(ws, K_FLOAT_PACK, kernel, dim3((unsigned)nb, M), kFloatThreads, 0, s, row, d, ld, sc, prob_list(p, L), seed,
+                      step, out.expo, out.planes, out.w_max, words, out.level, out.p_sel, ws.acc_word, ws.done, ws.status);
+    };
+    if (dtype == MLMC_BF16) go(float_pack_kernel<bf16_t>, static_cast<const bf16_t*>(g));
+    else go(float_pack_kernel<float>, static_cast<const float*>(g));
 }
 
 void launch_aggregate_floatbits(Workspace& ws, const mlmc_float_msgs& msgs, const int32_t* mb, int L, int M, int64_t d,
@@ -222,9 +210,8 @@ void launch_aggregate_floatbits(Workspace& ws, const mlmc_float_msgs& msgs, cons
     int64_t nb = (words + kFloatThreads - 1) / kFloatThreads;
     const int64_t cap = (int64_t)ws.sm_count * 8;
     if (nb > cap) nb = cap;
-    LaunchScope t(ws, K_AGG_FLOAT, s);
-    aggregate_float_kernel<<<(unsigned)nb, kFloatThreads, 0, s>>>(msgs.expo, msgs.planes, msgs.level, msgs.p_sel, sc,
-                                                                  msgs.w_max, words, M, d, out);
+    launch_kernel(ws, K_AGG_FLOAT, aggregate_float_kernel, dim3((unsigned)nb), kFloatThreads, 0, s, msgs.expo, msgs.planes,
+                  msgs.level, msgs.p_sel, sc, msgs.w_max, words, M, d, out);
 }
 
 }  // namespace mlmc

@@ -46,10 +46,12 @@ __device__ __forceinline__ float rtn_value(float v, float c, RtnGrid gq) {
 // Residual energies of every level: partial[m][block][l] = sum over the block's entries of (C^l - C^{l-1})^2.
 template <typename T, int LMAX>
 __global__ void __launch_bounds__(kRtnThreads)
-rtn_stats_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* __restrict__ gmax_bits, RtnSchedule sc,
-                 double* __restrict__ partial, int rtn_ctas, const int* worker_err) {
+rtn_stats_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* gmax_bits, RtnSchedule sc, double* partial,
+                 int rtn_ctas, uint32_t* done, DrawPlan pl, int* status, int* worker_err) {
     using Tr = ElemTraits<T>;
     __shared__ double sh_red[kRtnThreads / 32];
+    __shared__ double sh_delta[kMaxLevels], sh_p[kMaxLevels];
+    pdl_enter();
     const int m = blockIdx.y;
     if (worker_err[m]) return;
     const float c = __uint_as_float(gmax_bits[m]);
@@ -111,57 +113,27 @@ rtn_stats_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t*
         }
         __syncthreads();
     }
-}
-
-// Delta_l, p_l = Delta_l / sum Delta (Lemma 3.4) or the given p, the draw, the message header.
-__global__ void rtn_probs_draw_kernel(int L, const uint32_t* gmax_bits, const double* partial, int n_partials,
-                                      int rtn_ctas, const double* p_fixed, int adaptive, int have_stats, uint64_t seed,
-                                      uint64_t step, int M, double* p_all, double* delta_all, double* u_dev,
-                                      int32_t* bit_level, float* out_c, int32_t* out_level, double* out_p_sel,
-                                      const int* worker_err) {
-    const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= M) return;
-    if (worker_err[m]) {
-        bit_level[m] = -1;
-        if (out_level) {
-            out_level[m] = -1;
-            out_p_sel[m] = 0.0;
-            out_c[m] = 0.0f;
-        }
-        return;
-    }
-    double p[kRtnMaxLevels], s = 0.0;
-    for (int l = 0; l < L; ++l) {
+    if (!last_block(&done[m], gridDim.x)) return;
+    // the per-block partials, a warp per level in a fixed order; then p, the draw and the header
+    const int lane = threadIdx.x & 31;
+    for (int l = threadIdx.x >> 5; l < sc.L; l += kRtnThreads / 32) {
         double e = 0.0;
-        if (have_stats)
-            for (int c = 0; c < n_partials; ++c) e += partial[((int64_t)m * rtn_ctas + c) * kMaxLevels + l];  // block order
-        const double dl = sqrt(e);
-        delta_all[m * kMaxLevels + l] = dl;
-        p[l] = dl;
-        s += dl;
+        for (int b = lane; b < (int)gridDim.x; b += 32) e += __ldcg(&partial[((int64_t)m * rtn_ctas + b) * kMaxLevels + l]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xFFFFFFFFu, e, o);
+        if (lane == 0) sh_delta[l] = sqrt(e);
     }
-    for (int l = 0; l < L; ++l) {
-        p[l] = adaptive ? ((s > 0.0) ? p[l] / s : (l == 0 ? 1.0 : 0.0)) : p_fixed[l];
-        p_all[m * kMaxLevels + l] = p[l];
-    }
-    const double u = counter_uniform(seed, step, (uint64_t)m);
-    u_dev[m] = u;
-    const int level = draw_from_probs(p, L, u);
-    bit_level[m] = level;
-    if (out_level) {
-        out_level[m] = level;
-        out_p_sel[m] = p[level];
-        out_c[m] = __uint_as_float(gmax_bits[m]);
-    }
+    __syncthreads();
+    finish_levels(pl, m, sh_delta, sh_p, c, status, worker_err);
 }
 
 // The dense message of the drawn level: val_i = (C^l - C^{l-1})_i / p_l, rounded to fp32 once.
 template <typename T>
 __global__ void __launch_bounds__(kRtnThreads)
-rtn_emit_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* __restrict__ gmax_bits, RtnSchedule sc,
-                const int32_t* __restrict__ bit_level, const double* __restrict__ p_all, float* __restrict__ val,
-                int64_t ldv) {
+rtn_emit_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* gmax_bits, RtnSchedule sc,
+                const int32_t* bit_level, const double* p_all, float* __restrict__ val, int64_t ldv) {
     using Tr = ElemTraits<T>;
+    pdl_enter();
     const int m = blockIdx.y;
     const int level = bit_level[m];
     if (level < 0) return;
@@ -202,8 +174,9 @@ rtn_emit_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* 
 
 // Server average of dense messages: out[i] = (1/M) sum_m val[m][i] in worker order.
 __global__ void __launch_bounds__(kRtnThreads)
-aggregate_dense_kernel(const float* __restrict__ val, const int32_t* __restrict__ level, int M, int64_t d, int64_t ldv,
+aggregate_dense_kernel(const float* __restrict__ val, const int32_t* level, int M, int64_t d, int64_t ldv,
                        float* __restrict__ out) {
+    pdl_enter();
     const float inv_M = 1.0f / (float)M;
     const bool vec_ok = (ldv % 4 == 0) && (d % 4 == 0);
     if (vec_ok) {
@@ -245,49 +218,47 @@ int rtn_blocks(const Workspace& ws, int64_t d, int vec, int M, int per_sm) {
 
 }  // namespace
 
+DrawPlan rtn_draw_plan(Workspace& ws, int L, uint64_t seed, uint64_t step, const mlmc_rtn_msgs* out) {
+    DrawPlan pl = {};
+    pl.L = L;
+    pl.seed = seed;
+    pl.step = step;
+    pl.bit_level = ws.bit_level;
+    pl.p_all = ws.p_all;
+    pl.delta_all = ws.delta_all;
+    if (out) {
+        pl.out_scale = out->c;
+        pl.out_level = out->level;
+        pl.out_p_sel = out->p_sel;
+    }
+    return pl;
+}
+
 void launch_rtn_stats(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* r, int L,
-                      cudaStream_t s) {
+                      const DrawPlan& plan, cudaStream_t s) {
     const RtnSchedule sc = make_rtn_schedule(r, L);
     int nb = rtn_blocks(ws, d, dtype == MLMC_BF16 ? 8 : 4, M, 8);
     if (nb > ws.rtn_ctas) nb = ws.rtn_ctas;
-    ws.cur_rtn_ctas = nb;
-    dim3 grid(nb, M);
-    LaunchScope t(ws, K_RTN_STATS, s);
-#define MLMC_RTN_STATS(TT, LM)                                                                                      \
-    rtn_stats_kernel<TT, LM><<<grid, kRtnThreads, 0, s>>>(static_cast<const TT*>(g), d, ld, ws.gmax_bits, sc,       \
-                                                         ws.rtn_partial, ws.rtn_ctas, ws.worker_err)
-    if (dtype == MLMC_BF16) {
-        if (L <= 6) MLMC_RTN_STATS(bf16_t, 6);
-        else MLMC_RTN_STATS(bf16_t, kRtnMaxLevels);
-    } else {
-        if (L <= 6) MLMC_RTN_STATS(float, 6);
-        else MLMC_RTN_STATS(float, kRtnMaxLevels);
-    }
-#undef MLMC_RTN_STATS
-}
-
-void launch_rtn_probs_draw(Workspace& ws, int M, int L, bool adaptive, bool have_stats, uint64_t seed, uint64_t step,
-                           const mlmc_rtn_msgs* out, cudaStream_t s) {
-    LaunchScope t(ws, K_RTN_DRAW, s);
-    rtn_probs_draw_kernel<<<(M + 63) / 64, 64, 0, s>>>(L, ws.gmax_bits, ws.rtn_partial, ws.cur_rtn_ctas, ws.rtn_ctas,
-                                                      ws.p_fixed, adaptive ? 1 : 0, have_stats ? 1 : 0, seed, step, M,
-                                                      ws.p_all, ws.delta_all, ws.u_dev, ws.bit_level,
-                                                      out ? out->c : nullptr, out ? out->level : nullptr,
-                                                      out ? out->p_sel : nullptr, ws.worker_err);
+    auto go = [&](auto kernel, auto* row) {
+        launch_kernel(ws, K_RTN_STATS, kernel, dim3(nb, M), kRtnThreads, 0, s, row, d, ld, ws.gmax_bits, sc, ws.rtn_partial,
+                      ws.rtn_ctas, ws.done, plan, ws.status, ws.worker_err);
+    };
+    if (dtype == MLMC_BF16)
+        go(L <= 6 ? rtn_stats_kernel<bf16_t, 6> : rtn_stats_kernel<bf16_t, kRtnMaxLevels>, static_cast<const bf16_t*>(g));
+    else
+        go(L <= 6 ? rtn_stats_kernel<float, 6> : rtn_stats_kernel<float, kRtnMaxLevels>, static_cast<const float*>(g));
 }
 
 void launch_rtn_emit(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* r, int L,
                      const mlmc_rtn_msgs& out, cudaStream_t s) {
     const RtnSchedule sc = make_rtn_schedule(r, L);
     const int nb = rtn_blocks(ws, d, dtype == MLMC_BF16 ? 8 : 4, M, 16);
-    dim3 grid(nb, M);
-    LaunchScope t(ws, K_RTN_EMIT, s);
-    if (dtype == MLMC_BF16)
-        rtn_emit_kernel<bf16_t><<<grid, kRtnThreads, 0, s>>>(static_cast<const bf16_t*>(g), d, ld, ws.gmax_bits, sc,
-                                                            ws.bit_level, ws.p_all, out.val, out.ldv);
-    else
-        rtn_emit_kernel<float><<<grid, kRtnThreads, 0, s>>>(static_cast<const float*>(g), d, ld, ws.gmax_bits, sc,
-                                                           ws.bit_level, ws.p_all, out.val, out.ldv);
+    auto go = [&](auto kernel, auto* row) {
+        launch_kernel(ws, K_RTN_EMIT, kernel, dim3(nb, M), kRtnThreads, 0, s, row, d, ld, ws.gmax_bits, sc, ws.bit_level,
+                      ws.p_all, out.val, out.ldv);
+    };
+    if (dtype == MLMC_BF16) go(rtn_emit_kernel<bf16_t>, static_cast<const bf16_t*>(g));
+    else go(rtn_emit_kernel<float>, static_cast<const float*>(g));
 }
 
 void launch_aggregate_dense(Workspace& ws, const float* val, const int32_t* level, int M, int64_t d, int64_t ldv,
@@ -296,8 +267,7 @@ void launch_aggregate_dense(Workspace& ws, const float* val, const int32_t* leve
     const int64_t cap = (int64_t)ws.sm_count * 16;
     if (nb > cap) nb = cap;
     if (nb < 1) nb = 1;
-    LaunchScope t(ws, K_AGG_DENSE, s);
-    aggregate_dense_kernel<<<(unsigned)nb, kRtnThreads, 0, s>>>(val, level, M, d, ldv, out);
+    launch_kernel(ws, K_AGG_DENSE, aggregate_dense_kernel, dim3((unsigned)nb), kRtnThreads, 0, s, val, level, M, d, ldv, out);
 }
 
 }  // namespace mlmc

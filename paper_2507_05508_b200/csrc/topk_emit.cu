@@ -7,15 +7,20 @@
 //   C = #{ Tb <= key <= Ta },  A = #{ key == Ta },  B = #{ key == Tb }
 // over the elements before it.  The row is cut into tiles of kEmitTile 32-bit words, each of kEmitGroups batches;
 // only the batches whose largest key (recorded by the first selection sweep) reaches Tb can hold band entries,
-// the others are never read.  Four kernels, no waiting between thread blocks:
-//   tile_list   one block per worker: the tiles that hold such a batch, each with the mask of those batches;
-//   band_count  one warp per listed tile: the tile's C, A, B over its masked batches;
-//   band_scan   one block per worker: exclusive running totals over the worker's listed tiles;
-//   band_write  one warp per listed tile: reads the batches again and writes their entries at their final positions.
+// the others are never read.  Three kernels, no waiting between thread blocks:
+//   tile_list   one thread per tile: appends the tiles that hold such a batch, with the mask of those batches, to one list
+//               of all workers' tiles (its order does not matter);
+//   band_count  the warps stride over the list, count C, A, B of every tile and add them to the totals of the item,
+//               super-item and hyper-item the tile lies in;
+//   band_write  the warps stride over the list again: a tile's position is the sum of the counts before it (hyper-items,
+//               super-items, items, tiles: one load per lane each); its entries are written there.
+// How much there is to read differs from worker to worker (their levels differ) and from layer to layer; striding over
+// the list gives every warp the same share.
 //
 // aggregate: the dense mean (1/M) sum_m g~_m (Alg. 2 "Server aggregates") tiled over the index
 // space; because every message is index-sorted, a tile's entries are one contiguous range per
 // worker; they are added into a shared-memory tile in worker order and the tile is written once.
+#include <algorithm>
 #include <atomic>
 
 #include "common.cuh"
@@ -216,256 +221,177 @@ __device__ __forceinline__ uint32_t batch_masks(const uint32_t (&w)[kEmitRows], 
     return flags;
 }
 
-// Flat numbering of the listed tiles of all workers (worker-major).  sh_off[m] = listed tiles of the workers
-// before m; computed by the first warp of every block.
-__device__ __forceinline__ void list_offsets(const uint32_t* __restrict__ tile_n, int M, uint32_t* sh_off) {
-    if (threadIdx.x < 32) {
-        const int lane = threadIdx.x;
-        uint32_t carry = 0;
-        for (int base = 0; base < M; base += 32) {
-            const uint32_t n = (base + lane < M) ? tile_n[base + lane] : 0u;
-            uint32_t incl = n;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-                if (lane >= o) incl += y;
-            }
-            if (base + lane < M) sh_off[base + lane] = carry + incl - n;
-            carry += __shfl_sync(0xFFFFFFFFu, incl, 31);
-        }
-        if (lane == 0) sh_off[M] = carry;
+// Where a tile's counts are added up: {C, A, B, batches} per item, super-item and hyper-item of every worker.
+struct CountLevels {
+    uint4 *items, *supers, *hypers;
+    int n_items, n_supers, n_hypers;  // per worker
+};
+
+// A batch whose largest key is below the lower threshold Tb of the drawn band holds no band entry and no tie of Tb either;
+// it is not read.  List entry: {worker << kTileBits | tile, mask of the batches to read}.
+__global__ void __launch_bounds__(kBandThreads)
+tile_list_kernel(const uint32_t* tile_max, int tiles_per_worker, const EmitParams* emit, uint32_t key_cap, uint4* tiles,
+                 uint2* list, uint32_t* list_n) {
+    pdl_enter();
+    const int m = blockIdx.y, t = blockIdx.x * kBandThreads + threadIdx.x, lane = threadIdx.x & 31;
+    uint4 a = make_uint4(0u, 0u, 0u, 0u), b = a;
+    const bool inside = t < tiles_per_worker;
+    if (inside) {  // the batch maxima of a tile are two 16-byte vectors
+        const uint4* mx = reinterpret_cast<const uint4*>(tile_max) + ((int64_t)m * tiles_per_worker + t) * 2;
+        a = mx[0];
+        b = mx[1];
     }
-    __syncthreads();
-}
-
-// Worker of flat entry f: the last m with sh_off[m] <= f (workers without listed tiles are skipped by the search).
-__device__ __forceinline__ int worker_of(const uint32_t* sh_off, int M, uint32_t f) {
-    int lo = 0, hi = M - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (sh_off[mid] <= f) lo = mid; else hi = mid - 1;
-    }
-    return lo;
-}
-
-// The tiles of every worker that can hold band entries, ascending: a tile whose largest key is below the lower
-// threshold Tb of the drawn band holds none (and no tie of Tb either), so the sweep leaves it out.
-// One block per worker; every warp owns a contiguous range of tiles (a multiple of 32, so that its rows of 32 tiles
-// are coalesced loads), counts its listed tiles, and after one barrier writes them behind those of the warps before.
-constexpr int kListThreads = 1024;
-
-__global__ void __launch_bounds__(kListThreads)
-tile_list_kernel(const uint32_t* __restrict__ tile_max, int tiles_per_worker, const EmitParams* __restrict__ emit,
-                 uint32_t key_cap, uint32_t* __restrict__ worker_tiles, uint32_t* __restrict__ tile_n,
-                 uint32_t* __restrict__ group_n, int* status, int cached) {
-    __shared__ uint32_t sh_warp[kListThreads / 32], sh_grp[kListThreads / 32];
-    extern __shared__ uint8_t sh_mask[];  // [tiles_per_worker] batch masks of the counting pass, when they fit (cached != 0)
-    const int m = blockIdx.x;
     const EmitParams e = emit[m];
-    const bool on = e.enabled && e.level >= 0 && e.expect > 0u;
     const uint32_t Tb = min(e.Tb, key_cap);
-    // the batch maxima of a tile are two 16-byte vectors; a batch below Tb holds no band entry and no tie of Tb
-    const uint4* tmax = reinterpret_cast<const uint4*>(tile_max + (int64_t)m * tiles_per_worker * kEmitGroups);
-    uint32_t* list = worker_tiles + (int64_t)m * tiles_per_worker;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int rows = (tiles_per_worker + kListThreads - 1) / kListThreads;  // rows of 32 tiles per warp
-    const int t0 = warp * rows * 32;
-    auto batch_mask = [&](int t) -> uint32_t {
-        if (t >= tiles_per_worker) return 0u;
-        const uint4 a = __ldg(&tmax[2 * (int64_t)t]), b = __ldg(&tmax[2 * (int64_t)t + 1]);
-        return (a.x >= Tb ? 1u : 0u) | (a.y >= Tb ? 2u : 0u) | (a.z >= Tb ? 4u : 0u) | (a.w >= Tb ? 8u : 0u) |
+    uint32_t mask = 0;
+    if (inside && e.enabled && e.level >= 0 && e.expect > 0u)
+        mask = (a.x >= Tb ? 1u : 0u) | (a.y >= Tb ? 2u : 0u) | (a.z >= Tb ? 4u : 0u) | (a.w >= Tb ? 8u : 0u) |
                (b.x >= Tb ? 16u : 0u) | (b.y >= Tb ? 32u : 0u) | (b.z >= Tb ? 64u : 0u) | (b.w >= Tb ? 128u : 0u);
-    };
-    uint32_t mine = 0, groups = 0;  // listed tiles of this warp (the same in every lane), batches of this lane
-    if (on) {
-#pragma unroll 4
-        for (int r = 0; r < rows; ++r) {
-            const int t = t0 + r * 32 + lane;
-            const uint32_t bm = batch_mask(t);
-            if (cached && t < tiles_per_worker) sh_mask[t] = (uint8_t)bm;  // read back by this same thread below
-            mine += __popc(__ballot_sync(0xFFFFFFFFu, bm != 0u));
-            groups += __popc(bm);
-        }
-    }
-    groups = __reduce_add_sync(0xFFFFFFFFu, groups);
-    if (lane == 0) {
-        sh_warp[warp] = mine;
-        sh_grp[warp] = groups;
-    }
-    __syncthreads();
-    uint32_t before = 0, total = 0, total_groups = 0;
-    for (int w = 0; w < kListThreads / 32; ++w) {
-        const uint32_t x = sh_warp[w];
-        total += x;
-        total_groups += sh_grp[w];
-        if (w < warp) before += x;
-    }
-    if (on && mine) {
-        uint32_t pos = before;
-        const uint32_t lt = (1u << lane) - 1u;
-#pragma unroll 4
-        for (int r = 0; r < rows; ++r) {
-            const int t = t0 + r * 32 + lane;
-            const uint32_t bm = cached ? (t < tiles_per_worker ? (uint32_t)sh_mask[t] : 0u) : batch_mask(t);
-            const uint32_t mk = __ballot_sync(0xFFFFFFFFu, bm != 0u);
-            if (bm) list[pos + __popc(mk & lt)] = (uint32_t)t | (bm << 24);  // tile numbers stay below 2^20
-            pos += __popc(mk);
-        }
-    }
-    if (threadIdx.x == 0) {
-        tile_n[m] = total;
-        group_n[m] = total_groups;
-        if (on && total == 0u) set_status(status, MLMC_ERR_INTERNAL);  // a band with entries lies in some tile
-    }
+    const uint32_t listed = __ballot_sync(0xFFFFFFFFu, mask != 0u);
+    uint32_t base = 0;
+    if (lane == 0 && listed) base = atomicAdd(list_n, (uint32_t)__popc(listed));
+    base = __shfl_sync(0xFFFFFFFFu, base, 0);
+    if (mask) list[base + __popc(listed & ((1u << lane) - 1u))] = make_uint2(((uint32_t)m << kTileBits) | (uint32_t)t, mask);
+    else if (inside) tiles[(int64_t)m * tiles_per_worker + t] = make_uint4(0u, 0u, 0u, 0u);
 }
 
-// Pass 1: C, A, B of every listed tile.  rec[m][j] = {C, A, B, 0} for the j-th listed tile of worker m.
+// Pass 1: tiles[m][t] = {C, A, B, tie flag} of every tile (the tie flag: the tile holds a key equal to a threshold).
+// A warp walks the batches of its tiles as one sequence, the next batch in flight while the current one is counted.
 template <typename T>
 __global__ void __launch_bounds__(kBandThreads)
-band_count_kernel(const T* __restrict__ g, int64_t d, int64_t ld, int tiles_per_worker,
-                  const uint32_t* __restrict__ worker_tiles, const uint32_t* __restrict__ tile_n, int M,
-                  const EmitParams* __restrict__ emit, uint4* __restrict__ rec) {
+band_count_kernel(const T* __restrict__ g, int64_t d, int64_t ld, int tiles_per_worker, int M, const EmitParams* emit,
+                  uint4* tiles, CountLevels lv, const uint2* list, const uint32_t* list_n) {
     using EW = EmitWord<T>;
-    extern __shared__ uint32_t sh_off[];  // [M + 1]
-    list_offsets(tile_n, M, sh_off);
-    const uint32_t total = sh_off[M];
+    extern __shared__ uint2 sh_thr[];  // [M] {Tb, Ta}
+    pdl_enter();
+    for (int m = threadIdx.x; m < M; m += kBandThreads) sh_thr[m] = make_uint2(min(emit[m].Tb, EW::kCap), min(emit[m].Ta, EW::kCap));
+    const uint32_t total = *list_n;
+    __syncthreads();
     const int lane = threadIdx.x & 31;
     const uint32_t warps = gridDim.x * (kBandThreads / 32);
-    for (uint32_t f = blockIdx.x * (kBandThreads / 32) + (threadIdx.x >> 5); f < total; f += warps) {
-        const int m = worker_of(sh_off, M, f);
-        const uint32_t j = f - sh_off[m];
-        const uint32_t entry = worker_tiles[(int64_t)m * tiles_per_worker + j];
-        const int64_t tile = entry & 0xFFFFFFu;
-        uint32_t todo = entry >> 24;  // the batches of the tile that can hold band entries (at least one)
-        const uint32_t Tb = min(__ldg(&emit[m].Tb), EW::kCap), Ta = min(__ldg(&emit[m].Ta), EW::kCap);
-        const T* row = g + (int64_t)m * ld;
-        uint32_t cC = 0, cA = 0, cB = 0;
-        uint32_t cur[kEmitRows], nxt[kEmitRows];
-        load_batch<T>(row, d, tile, __ffs(todo) - 1, lane, cur);
-        todo &= todo - 1u;
+    uint32_t f = blockIdx.x * (kBandThreads / 32) + (threadIdx.x >> 5);
+    if (f >= total) return;
+    uint2 here = list[f], next = make_uint2(0u, 0u);
+    if (f + warps < total) next = list[f + warps];
+    uint32_t todo = here.y, cC = 0, cA = 0, cB = 0, batches = 0;
+    uint32_t cur[kEmitRows], nxt[kEmitRows];
+    auto load = [&](const uint2& e, uint32_t& left, uint32_t (&w)[kEmitRows]) {
+        load_batch<T>(g + (int64_t)(e.x >> kTileBits) * ld, d, e.x & ((1u << kTileBits) - 1u), __ffs(left) - 1, lane, w);
+        left &= left - 1u;
+    };
+    load(here, todo, cur);
 #pragma unroll 1
-        for (bool more = true; more;) {
-            more = todo != 0u;
-            if (more) {  // in flight while this batch is counted
-                load_batch<T>(row, d, tile, __ffs(todo) - 1, lane, nxt);
-                todo &= todo - 1u;
+    for (;;) {
+        const bool last = todo == 0u, more = f + warps < total;  // last batch of the tile; another tile follows
+        uint32_t todo_next = next.y;
+        if (!last) load(here, todo, nxt);
+        else if (more) load(next, todo_next, nxt);
+        const int m = (int)(here.x >> kTileBits);
+        const uint2 thr = sh_thr[m];
+        uint32_t a1, b1;
+        const uint32_t flags = batch_flags<T>(cur, thr.x, thr.y, &a1, &b1);
+        cC += __popc(flags);
+        cA += a1;
+        cB += b1;
+        ++batches;
+        if (last) {
+            const uint32_t totCA = __reduce_add_sync(0xFFFFFFFFu, cC | (cA << 16));  // at most 8192 elements per tile
+            const uint32_t tB = __reduce_add_sync(0xFFFFFFFFu, cB);
+            const uint32_t tC = totCA & 0xFFFFu, tA = totCA >> 16;
+            const int tile = (int)(here.x & ((1u << kTileBits) - 1u));
+            if (lane == 31) tiles[(int64_t)m * tiles_per_worker + tile] = make_uint4(tC, tA, tB, (tA | tB) ? 1u : 0u);
+            if (lane < 12) {  // three levels of four components
+                const int item = tile / kItemTiles, sup = item / kSuperItems, c = lane & 3;
+                uint4* rec = lane < 4 ? lv.items + (int64_t)m * lv.n_items + item
+                           : lane < 8 ? lv.supers + (int64_t)m * lv.n_supers + sup
+                                      : lv.hypers + (int64_t)m * lv.n_hypers + sup / kSuperItems;
+                const uint32_t x = c == 0 ? tC : c == 1 ? tA : c == 2 ? tB : batches;
+                if (x) atomicAdd(reinterpret_cast<uint32_t*>(rec) + c, x);
             }
-            uint32_t a1, b1;
-            const uint32_t flags = batch_flags<T>(cur, Tb, Ta, &a1, &b1);
-            cC += __popc(flags);
-            cA += a1;
-            cB += b1;
-#pragma unroll
-            for (int i = 0; i < kEmitRows; ++i) cur[i] = nxt[i];
+            if (!more) return;
+            cC = cA = cB = batches = 0u;
+            here = next;
+            todo = todo_next;
+            f += warps;
+            if (f + warps < total) next = list[f + warps];
         }
-        const uint32_t totCA = __reduce_add_sync(0xFFFFFFFFu, cC | (cA << 16));  // at most 8192 elements per tile
-        cB = __reduce_add_sync(0xFFFFFFFFu, cB);
-        // the fourth word tells the write pass whether the tile holds a key equal to a threshold at all
-        if (lane == 0)
-            rec[(int64_t)m * tiles_per_worker + j] = make_uint4(totCA & 0xFFFFu, totCA >> 16, cB, ((totCA >> 16) | cB) ? 1u : 0u);
+#pragma unroll
+        for (int i = 0; i < kEmitRows; ++i) cur[i] = nxt[i];
     }
 }
 
-// Pass 2: exclusive running totals over the listed tiles of every worker, in place, and the self-check that the
-// band has exactly k_l - k_{l-1} entries.  One block per worker; every warp owns a contiguous range of the list (a
-// multiple of 32 records, read as coalesced rows), adds it up, and after one barrier scans it row by row from the
-// total of the warps before it.
-__global__ void __launch_bounds__(kListThreads)
-band_scan_kernel(uint4* __restrict__ rec, int tiles_per_worker, const uint32_t* __restrict__ tile_n,
-                 const EmitParams* __restrict__ emit, int* status) {
-    __shared__ uint32_t sh_w[3][kListThreads / 32];
-    const int m = blockIdx.x;
-    const int n = (int)tile_n[m];
-    if (n == 0) return;
-    uint4* r = rec + (int64_t)m * tiles_per_worker;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int rows = (n + kListThreads - 1) / kListThreads;  // rows of 32 records per warp
-    const int t0 = warp * rows * 32;
-    uint32_t sC = 0, sA = 0, sB = 0;
-#pragma unroll 4
-    for (int i = 0; i < rows; ++i) {
-        const int t = t0 + i * 32 + lane;
-        if (t < n) {
-            const uint4 x = r[t];
-            sC += x.x; sA += x.y; sB += x.z;
-        }
-    }
-    sC = __reduce_add_sync(0xFFFFFFFFu, sC);
-    sA = __reduce_add_sync(0xFFFFFFFFu, sA);
-    sB = __reduce_add_sync(0xFFFFFFFFu, sB);
-    if (lane == 0) { sh_w[0][warp] = sC; sh_w[1][warp] = sA; sh_w[2][warp] = sB; }
-    __syncthreads();
-    uint32_t pC = 0, pA = 0, pB = 0, totC = 0, totA = 0, totB = 0;  // running totals before this warp's range
-    for (int w = 0; w < kListThreads / 32; ++w) {
-        const uint32_t xC = sh_w[0][w], xA = sh_w[1][w], xB = sh_w[2][w];
-        totC += xC; totA += xA; totB += xB;
-        if (w < warp) { pC += xC; pA += xA; pB += xB; }
-    }
-    for (int i = 0; i < rows; ++i) {
-        const int t = t0 + i * 32 + lane;
-        if (t0 + i * 32 >= n) break;  // warp-uniform
-        uint4 x = make_uint4(0u, 0u, 0u, 0u);
-        if (t < n) x = r[t];
-        uint32_t iC = x.x, iA = x.y, iB = x.z;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t yC = __shfl_up_sync(0xFFFFFFFFu, iC, o), yA = __shfl_up_sync(0xFFFFFFFFu, iA, o),
-                           yB = __shfl_up_sync(0xFFFFFFFFu, iB, o);
-            if (lane >= o) { iC += yC; iA += yA; iB += yB; }
-        }
-        if (t < n) r[t] = make_uint4(pC + iC - x.x, pA + iA - x.y, pB + iB - x.z, x.w);
-        pC += __shfl_sync(0xFFFFFFFFu, iC, 31);
-        pA += __shfl_sync(0xFFFFFFFFu, iA, 31);
-        pB += __shfl_sync(0xFFFFFFFFu, iB, 31);
-    }
-    if (threadIdx.x == 0) {
-        const EmitParams e = emit[m];
-        if (band_prefix(totC, totA, totB, e.ra, e.rb) != e.expect) set_status(status, MLMC_ERR_INTERNAL);
-    }
-}
-
-// Pass 3: every listed tile is read again and its band entries are written at their final positions.
+// Pass 2: every listed tile is read again and its band entries are written at their final positions.
 // A lane owns 16 consecutive words of a batch, so the order of the lanes is the order of the coordinates: the
 // position of a lane's first entry is the batch's base plus the entries of the lanes before it (one warp scan per
 // batch), and the lane then writes its own entries one after the other.
 template <typename T>
 __global__ void __launch_bounds__(kBandThreads, 4)
-band_write_kernel(const T* __restrict__ g, int64_t d, int64_t ld, int tiles_per_worker,
-                  const uint32_t* __restrict__ worker_tiles, const uint32_t* __restrict__ tile_n, int M,
-                  const EmitParams* __restrict__ emit, const uint4* __restrict__ rec,
-                  uint32_t* __restrict__ idx_out, float* __restrict__ val_out, int64_t capacity) {
+band_write_kernel(const T* __restrict__ g, int64_t d, int64_t ld, int tiles_per_worker, int M, const EmitParams* emit,
+                  const uint4* tiles, CountLevels lv, const uint2* list, const uint32_t* list_n,
+                  uint32_t* __restrict__ idx_out, float* __restrict__ val_out, int64_t capacity, uint32_t* group_n,
+                  int* status) {
     using EW = EmitWord<T>;
     constexpr int S = EW::S;
     static_assert(kEmitRows == 16, "a lane owns four 16-byte chunks of a batch");
     // every warp stages its batches in a ring of three shared-memory slots: two copies are in flight while a
     // batch is ranked, and the words of a batch can be addressed by a run-time index
-    extern __shared__ __align__(16) uint32_t sh_dyn[];  // [warps][3][kBatchWords] ring, then sh_off[M + 1]
-    uint32_t* sh_off = sh_dyn + (kBandThreads / 32) * kWriteSlots * kBatchWords;
-    list_offsets(tile_n, M, sh_off);
-    const uint32_t total = sh_off[M];
+    extern __shared__ __align__(16) uint32_t sh_dyn[];  // [warps][3][kBatchWords]
+    pdl_enter();
     const int lane = threadIdx.x & 31;
+    const int warps = gridDim.x * (kBandThreads / 32), gw = blockIdx.x * (kBandThreads / 32) + (threadIdx.x >> 5);
+    // the band of every worker has exactly k_l - k_{l-1} entries, and they lie in some batch
+    for (int m = gw; m < M; m += warps) {
+        uint4 x = make_uint4(0u, 0u, 0u, 0u);
+        for (int i = lane; i < lv.n_hypers; i += 32) {
+            const uint4 y = lv.hypers[(int64_t)m * lv.n_hypers + i];
+            x.x += y.x; x.y += y.y; x.z += y.z; x.w += y.w;
+        }
+        x.x = __reduce_add_sync(0xFFFFFFFFu, x.x);
+        x.y = __reduce_add_sync(0xFFFFFFFFu, x.y);
+        x.z = __reduce_add_sync(0xFFFFFFFFu, x.z);
+        x.w = __reduce_add_sync(0xFFFFFFFFu, x.w);
+        if (lane == 0) {
+            const EmitParams e = emit[m];
+            group_n[m] = x.w;
+            if (e.enabled && e.level >= 0 && e.expect > 0u && (x.w == 0u || band_prefix(x.x, x.y, x.z, e.ra, e.rb) != e.expect))
+                set_status(status, MLMC_ERR_INTERNAL);
+        }
+    }
+    const uint32_t total = *list_n;
     uint32_t* ring = sh_dyn + (threadIdx.x >> 5) * kWriteSlots * kBatchWords;
     // where this lane's words sit in a slot: word r at own + (r ^ own_xor), i.e. chunk q at swz(4 * lane + q)
     const int own = lane * kEmitRows, own_xor = ((lane >> 1) & 3) << 2;
-    const uint32_t warps = gridDim.x * (kBandThreads / 32);
-    for (uint32_t f = blockIdx.x * (kBandThreads / 32) + (threadIdx.x >> 5); f < total; f += warps) {
-        const int m = worker_of(sh_off, M, f);
-        const uint32_t j = f - sh_off[m];
-        const uint32_t entry = worker_tiles[(int64_t)m * tiles_per_worker + j];
-        const int64_t tile = entry & 0xFFFFFFu;
+    uint2 next = gw < (int)total ? list[gw] : make_uint2(0u, 0u);
+    for (uint32_t f = gw; f < total; f += warps) {
+        const uint2 entry = next;
+        if (f + warps < total) next = list[f + warps];
+        const int m = (int)(entry.x >> kTileBits);
+        const int64_t tile = entry.x & ((1u << kTileBits) - 1u);
         const EmitParams ep = emit[m];
+        const uint32_t flags = tiles[(int64_t)m * tiles_per_worker + tile].w;
+        uint4 before = make_uint4(0u, 0u, 0u, 0u);  // counts before this tile
+        {
+            const int item = (int)tile / kItemTiles, sup = item / kSuperItems, hyp = sup / kSuperItems;
+            auto add = [&](const uint4& x) { before.x += x.x; before.y += x.y; before.z += x.z; };
+            if (lane < (int)tile % kItemTiles) add(tiles[(int64_t)m * tiles_per_worker + item * kItemTiles + lane]);
+            if (lane < item % kSuperItems) add(lv.items[(int64_t)m * lv.n_items + sup * kSuperItems + lane]);
+            if (lane < sup % kSuperItems) add(lv.supers[(int64_t)m * lv.n_supers + hyp * kSuperItems + lane]);
+            for (int i = lane; i < hyp; i += 32) add(lv.hypers[(int64_t)m * lv.n_hypers + i]);
+            before.x = __reduce_add_sync(0xFFFFFFFFu, before.x);
+            before.y = __reduce_add_sync(0xFFFFFFFFu, before.y);
+            before.z = __reduce_add_sync(0xFFFFFFFFu, before.z);
+        }
         const uint32_t Tb = min(ep.Tb, EW::kCap), Ta = min(ep.Ta, EW::kCap);
         const uint32_t W = Ta - Tb;
         const float inv_p = (float)ep.inv_p;
         const T* row = g + (int64_t)m * ld;
         uint32_t* idx_w = idx_out + (int64_t)m * capacity;
         float* val_w = val_out + (int64_t)m * capacity;
-        const uint4 pre = __ldg(&rec[(int64_t)m * tiles_per_worker + j]);
-        uint32_t rC = pre.x, rA = pre.y, rB = pre.z;  // running totals before the current batch
-        const bool tile_ties = pre.w != 0u;           // found by the count pass
+        uint32_t rC = before.x, rA = before.y, rB = before.z;  // running totals before the current batch
+        const bool tile_ties = flags != 0u;           // found by the count pass
         // Only the batches of the tile that can hold band entries are read (mask from the listing): `todo` walks them
         // for processing, `ahead` two batches further for the copies.
-        uint32_t todo = entry >> 24, ahead = todo;
+        uint32_t todo = entry.y, ahead = todo;
         __syncwarp();  // the previous tile's last batches have been read by every lane
         copy_batch_async<T>(row, d, tile, __ffs(ahead) - 1, lane, ring);
         ahead &= ahead - 1u;
@@ -575,9 +501,9 @@ band_write_kernel(const T* __restrict__ g, int64_t d, int64_t ld, int tiles_per_
 }
 
 // offsets[m][t] = first message entry of worker m whose index is >= t * kAggTile  (t = 0..ntiles)
-__global__ void agg_offsets_kernel(const uint32_t* __restrict__ idx, const int64_t* __restrict__ count,
-                                   const int32_t* __restrict__ level, int64_t capacity, int M, int ntiles,
-                                   uint32_t* __restrict__ offsets) {
+__global__ void agg_offsets_kernel(const uint32_t* idx, const int64_t* count, const int32_t* level, int64_t capacity, int M,
+                                   int ntiles, uint32_t* offsets) {
+    pdl_enter();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (int64_t)M * (ntiles + 1)) return;
     const int m = (int)(i / (ntiles + 1)), t = (int)(i % (ntiles + 1));
@@ -595,7 +521,8 @@ __global__ void agg_offsets_kernel(const uint32_t* __restrict__ idx, const int64
 // M is at most kEmitMaxWorkers: the offsets of all workers for one tile are fetched together.
 __global__ void __launch_bounds__(256)
 aggregate_topk_kernel(const uint32_t* __restrict__ idx, const float* __restrict__ val, int64_t capacity, int M,
-                      int64_t d, int ntiles, const uint32_t* __restrict__ offsets, float* __restrict__ out) {
+                      int64_t d, int ntiles, const uint32_t* offsets, float* __restrict__ out) {
+    pdl_enter();
     __shared__ __align__(16) float acc[kAggTile];
     extern __shared__ uint32_t sh_off[];  // [2 M]: first and one-past-last message entry of every worker in this tile
     const float inv_M = 1.0f / (float)M;
@@ -643,7 +570,8 @@ constexpr int kAggWarps = kAggTile / kAggSub;
 
 __global__ void __launch_bounds__(kAggWarps * 32)
 aggregate_topk_warps_kernel(const uint32_t* __restrict__ idx, const float* __restrict__ val, int64_t capacity, int M,
-                            int64_t d, int ntiles, const uint32_t* __restrict__ offsets, float* __restrict__ out) {
+                            int64_t d, int ntiles, const uint32_t* offsets, float* __restrict__ out) {
+    pdl_enter();
     __shared__ __align__(16) float acc_all[kAggTile];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float* acc = acc_all + warp * kAggSub;
@@ -704,80 +632,59 @@ aggregate_topk_warps_kernel(const uint32_t* __restrict__ idx, const float* __res
 
 }  // namespace
 
-int configure_emit_kernels() {  // the write pass: 48 KB ring + the list offsets of up to kEmitMaxWorkers workers
-    const int smem = (kBandThreads / 32) * kWriteSlots * kBatchWords * (int)sizeof(uint32_t) +
-                     (kEmitMaxWorkers + 1) * (int)sizeof(uint32_t);
-    if (cudaFuncSetAttribute(tile_list_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024) != cudaSuccess ||
-        cudaFuncSetAttribute(band_write_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+int configure_emit_kernels() {
+    const int smem = (kBandThreads / 32) * kWriteSlots * kBatchWords * (int)sizeof(uint32_t);
+    if (cudaFuncSetAttribute(band_write_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
         cudaFuncSetAttribute(band_write_kernel<bf16_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
         return MLMC_ERR_CUDA;
     return MLMC_OK;
 }
 
+namespace {
+
+template <typename T>
+void launch_emit_t(Workspace& ws, const T* g, int dtype, int64_t d, int M, int64_t ld, const mlmc_topk_msgs& out,
+                   cudaStream_t s) {
+    const int tpw = emit_tiles_per_worker(d, dtype);
+    const EmitCounts n = emit_counts(tpw);
+    const CountLevels lv = {ws.level_desc, ws.level_desc + (int64_t)M * n.items, ws.level_desc + (int64_t)M * (n.items + n.supers),
+                            n.items, n.supers, n.hypers};
+    const int wpb = kBandThreads / 32;
+    const size_t smem_w = (size_t)wpb * kWriteSlots * kBatchWords * sizeof(uint32_t);
+    ws.last_emit_tiles = tpw;
+    launch_kernel(ws, K_TILE_LIST, tile_list_kernel, dim3((tpw + kBandThreads - 1) / kBandThreads, M), kBandThreads, 0, s,
+                  ws.tile_max, tpw, ws.emit, EmitWord<T>::kCap, ws.tile_desc, ws.tile_list, ws.list_n);
+    // two whole waves: the warps stride over the list, so a partial last wave costs a full one
+    static const int resident = [] {
+        int n = 0;
+        const bool ok = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, band_count_kernel<T>, kBandThreads, 256) == cudaSuccess;
+        return ok && n >= 1 ? n : 1;
+    }();
+    const int64_t by_work = ((int64_t)tpw * M + wpb - 1) / wpb;
+    auto blocks = [&](int per_sm) { return (unsigned)std::min<int64_t>(by_work, (int64_t)ws.sm_count * per_sm * 2); };
+    launch_kernel(ws, K_BAND_COUNT, band_count_kernel<T>, dim3(blocks(resident)), kBandThreads, (size_t)M * sizeof(uint2), s, g, d,
+                  ld, tpw, M, ws.emit, ws.tile_desc, lv, ws.tile_list, ws.list_n);
+    launch_kernel(ws, K_EMIT, band_write_kernel<T>, dim3(blocks(4)), kBandThreads, smem_w, s, g, d, ld, tpw, M, ws.emit,
+                  ws.tile_desc, lv, ws.tile_list, ws.list_n, out.idx, out.val, out.capacity, ws.group_n, ws.status);
+}
+
+}  // namespace
+
 void launch_emit(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const mlmc_topk_msgs& out,
                  cudaStream_t s) {
-    const int tpw = emit_tiles_per_worker(d, dtype);
-    const int64_t most = (int64_t)tpw * M;  // listed tiles at most
-    ws.last_emit_tiles = tpw;
-    {
-        LaunchScope t(ws, K_TILE_LIST, s);
-        const int cached = tpw <= 96 * 1024;  // one byte per tile in shared memory
-        tile_list_kernel<<<M, kListThreads, cached ? (size_t)tpw : 0, s>>>(
-            ws.tile_max, tpw, ws.emit, dtype == MLMC_BF16 ? 0x7F80u : 0x7F800000u, ws.worker_tiles, ws.tile_n, ws.group_n,
-            ws.status, cached);
-    }
-    const int wpb = kBandThreads / 32;
-    const size_t smem = (size_t)(M + 1) * sizeof(uint32_t);
-    const size_t smem_w = smem + (size_t)(kBandThreads / 32) * kWriteSlots * kBatchWords * sizeof(uint32_t);
-    // grids of two whole waves: the warps take tiles with a grid stride, so a partial last wave costs a full one
-    auto two_waves = [&](const void* kernel, size_t dyn_smem) -> int64_t {
-        int resident = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, kernel, kBandThreads, dyn_smem) != cudaSuccess || resident < 1)
-            resident = 1;
-        int64_t grid = (int64_t)ws.sm_count * resident * 2;
-        const int64_t by_work = (most + wpb - 1) / wpb;
-        return grid < by_work ? grid : by_work;
-    };
-    const bool bf = dtype == MLMC_BF16;
-    const int64_t grid = two_waves(bf ? (const void*)band_count_kernel<bf16_t> : (const void*)band_count_kernel<float>, smem);
-    const int64_t grid_w = two_waves(bf ? (const void*)band_write_kernel<bf16_t> : (const void*)band_write_kernel<float>, smem_w);
-    {
-        LaunchScope t(ws, K_BAND_COUNT, s);
-        if (dtype == MLMC_BF16)
-            band_count_kernel<bf16_t><<<(unsigned)grid, kBandThreads, smem, s>>>(
-                static_cast<const bf16_t*>(g), d, ld, tpw, ws.worker_tiles, ws.tile_n, M, ws.emit, ws.tile_desc);
-        else
-            band_count_kernel<float><<<(unsigned)grid, kBandThreads, smem, s>>>(
-                static_cast<const float*>(g), d, ld, tpw, ws.worker_tiles, ws.tile_n, M, ws.emit, ws.tile_desc);
-    }
-    {
-        LaunchScope t(ws, K_BAND_SCAN, s);
-        band_scan_kernel<<<M, kListThreads, 0, s>>>(ws.tile_desc, tpw, ws.tile_n, ws.emit, ws.status);
-    }
-    LaunchScope t(ws, K_EMIT, s);
-    if (dtype == MLMC_BF16)
-        band_write_kernel<bf16_t><<<(unsigned)grid_w, kBandThreads, smem_w, s>>>(
-            static_cast<const bf16_t*>(g), d, ld, tpw, ws.worker_tiles, ws.tile_n, M, ws.emit, ws.tile_desc, out.idx,
-            out.val, out.capacity);
-    else
-        band_write_kernel<float><<<(unsigned)grid_w, kBandThreads, smem_w, s>>>(
-            static_cast<const float*>(g), d, ld, tpw, ws.worker_tiles, ws.tile_n, M, ws.emit, ws.tile_desc, out.idx,
-            out.val, out.capacity);
+    if (dtype == MLMC_BF16) launch_emit_t(ws, static_cast<const bf16_t*>(g), dtype, d, M, ld, out, s);
+    else launch_emit_t(ws, static_cast<const float*>(g), dtype, d, M, ld, out, s);
 }
 
 void launch_aggregate_topk(Workspace& ws, const mlmc_topk_msgs& msgs, int M, int64_t d, float* out, cudaStream_t s) {
     const int ntiles = (int)((d + kAggTile - 1) / kAggTile);
     const int64_t n_off = (int64_t)M * (ntiles + 1);
-    {
-        LaunchScope t(ws, K_AGG_OFFSETS, s);
-        agg_offsets_kernel<<<(unsigned)((n_off + 255) / 256), 256, 0, s>>>(msgs.idx, msgs.count, msgs.level,
-                                                                           msgs.capacity, M, ntiles, ws.agg_offsets);
-    }
+    launch_kernel(ws, K_AGG_OFFSETS, agg_offsets_kernel, dim3((unsigned)((n_off + 255) / 256)), 256, 0, s, msgs.idx, msgs.count,
+                  msgs.level, msgs.capacity, M, ntiles, ws.agg_offsets);
     int grid = ws.sm_count * 8;
     if (grid > ntiles) grid = ntiles;
-    LaunchScope t(ws, K_AGG_TOPK, s);
-    aggregate_topk_warps_kernel<<<grid, kAggWarps * 32, 0, s>>>(msgs.idx, msgs.val, msgs.capacity, M, d, ntiles,
-                                                                ws.agg_offsets, out);
+    launch_kernel(ws, K_AGG_TOPK, aggregate_topk_warps_kernel, dim3(grid), kAggWarps * 32, 0, s, msgs.idx, msgs.val,
+                  msgs.capacity, M, d, ntiles, ws.agg_offsets, out);
 }
 
 }  // namespace mlmc
