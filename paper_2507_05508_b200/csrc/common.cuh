@@ -473,6 +473,7 @@ void launch_aggregate_bitwise(Workspace& ws, const mlmc_bit_msgs& msgs, const in
                               float* out, cudaStream_t s);
 
 // floatbits.cu
+int configure_float_kernels();
 void launch_compress_floatbits(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* mb,
                                int L, const double* p, uint64_t seed, uint64_t step, const mlmc_float_msgs& out, cudaStream_t s);
 void launch_aggregate_floatbits(Workspace& ws, const mlmc_float_msgs& msgs, const int32_t* mb, int L, int M, int64_t d,

@@ -29,16 +29,80 @@ MantissaSchedule make_mantissa_schedule(const int32_t* mb, int L) {
     return sc;
 }
 
-// Every warp turns 1024 consecutive entries into 32 words of the sign plane and of each mantissa plane (one warp
-// ballot per row of 32 entries and plane), and into 1024 exponent bytes, which leave through a shared-memory
-// transpose as 32 consecutive bytes per lane.  All 32 rows of a group are requested before the first is used.
+// 32 x 32 bit transpose: on return bit t of x[b] is bit b of the former x[t].
+__device__ __forceinline__ void transpose_bits(uint32_t (&x)[32]) {
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        const uint32_t a = x[k], b = x[k + 16];
+        x[k] = __byte_perm(a, b, 0x5410);
+        x[k + 16] = __byte_perm(a, b, 0x7632);
+    }
+#pragma unroll
+    for (int k = 0; k < 32; ++k) {
+        if (k & 8) continue;
+        const uint32_t a = x[k], b = x[k + 8];
+        x[k] = __byte_perm(a, b, 0x6240);
+        x[k + 8] = __byte_perm(a, b, 0x7351);
+    }
+#pragma unroll
+    for (int j = 4; j > 0; j >>= 1) {
+        const uint32_t mask = j == 4 ? 0x0F0F0F0Fu : j == 2 ? 0x33333333u : 0x55555555u;
+#pragma unroll
+        for (int k = 0; k < 32; ++k) {
+            if (k & j) continue;
+            const uint32_t t = ((x[k] >> j) ^ x[k + j]) & mask;
+            x[k + j] ^= t;
+            x[k] ^= t << j;
+        }
+    }
+}
+
+// Bits 0..15 of x to the even bit positions.
+__device__ __forceinline__ uint32_t spread_bits(uint32_t x) {
+    x = (x | (x << 8)) & 0x00FF00FFu;
+    x = (x | (x << 4)) & 0x0F0F0F0Fu;
+    x = (x | (x << 2)) & 0x33333333u;
+    return (x | (x << 1)) & 0x55555555u;
+}
+
+// Word of bit `bit` of a lane's 32 entries.  fp32: one funnel shift collects the top bit of each (shifted) entry.
+// bf16: the words hold two entries; the bits of the low and the high halves are collected apart and interleaved.
+template <typename T>
+__device__ __forceinline__ uint32_t plane_word(const uint32_t* x, int bit) {
+    uint32_t w = 0;
+    if constexpr (sizeof(T) == 4) {
+#pragma unroll
+        for (int t = 31; t >= 0; --t) w = __funnelshift_l(x[t] << (31 - bit), w, 1);
+        return w;
+    } else {
+        uint32_t h = 0;  // bit = position in the 16-bit encoding
+#pragma unroll
+        for (int t = 15; t >= 0; --t) {
+            h = __funnelshift_l(x[t] << (15 - bit), h, 1);
+            w = __funnelshift_l(x[t] << (31 - bit), w, 1);
+        }
+        return spread_bits(w) | (spread_bits(h) << 1);
+    }
+}
+
+// A warp turns 1024 consecutive entries into 32 words of the sign plane and of each mantissa plane and into 1024 exponent
+// bytes.  A lane owns 32 consecutive entries, so every word is collected in the lane's own registers (2 instructions
+// per entry and plane; from 6 planes on one bit transpose for all of them is cheaper).  The entries come through a
+// ring of two shared-memory slots per warp filled by 16-byte asynchronous copies; the 16-byte chunks of a lane are
+// XOR-ed with its number so that the lanes' reads fall into different banks.
 // The draw does not depend on the data: every block makes it itself; the worker's last block writes the header.
+// Bound by HBM (reads 4 or 2 bytes, writes 1 byte and 1 + w bits per entry).  Ballots over rows of 32 entries took 1.14 ms
+// for 8 x 124M fp32 entries (0.72 of the copy rate).
 template <typename T>
 __global__ void __launch_bounds__(kFloatThreads, 3)
 float_pack_kernel(const T* __restrict__ g, int64_t d, int64_t ld, MantissaSchedule sc, ProbList p, uint64_t seed,
                   uint64_t step, uint8_t* __restrict__ expo, uint32_t* __restrict__ planes, int w_max, int64_t words,
                   int32_t* out_level, double* out_p_sel, uint32_t* acc, uint32_t* done, int* status) {
-    __shared__ __align__(16) uint8_t sh_expo[kFloatThreads / 32][1024];
+    constexpr int kWords = 32 * (int)sizeof(T) / 4;   // 32-bit words of a lane's entries
+    constexpr int kChunks = kWords / 4;               // 16-byte chunks
+    constexpr int kSlot = 32 * kWords;                // words per slot
+    constexpr int kMantBits = sizeof(T) == 4 ? 23 : 7;
+    extern __shared__ __align__(16) uint32_t sh_ring[];  // [warps][2][kSlot]
     __shared__ int sh_level;
     const int m = blockIdx.y;
     if (threadIdx.x == 0) sh_level = draw_from_probs(p.p, sc.L, counter_uniform(seed, step, (uint64_t)m));
@@ -58,64 +122,100 @@ float_pack_kernel(const T* __restrict__ g, int64_t d, int64_t ld, MantissaSchedu
     const T* row = g + (int64_t)m * ld;
     uint32_t* out = planes + (int64_t)m * (1 + w_max) * words;
     uint8_t* ex = expo + (int64_t)m * words * 32;
+    uint32_t* ring = sh_ring + warp * 2 * kSlot;
     const int64_t ngroups = (words + 31) / 32;
     const int64_t stride = (int64_t)gridDim.x * (kFloatThreads / 32);
-    bool bad = false;
-    for (int64_t grp = (int64_t)blockIdx.x * (kFloatThreads / 32) + warp; grp < ngroups; grp += stride) {
-        const int64_t e0 = grp * 1024;
-        uint32_t x[32];  // fp32 encodings of this lane's entry of every row (entries past d read as +0)
-        if (e0 + 1024 <= d) {
+    // chunk c of lane l is kept at chunk position c ^ (l mod kChunks) (bf16: l / 2, a lane's chunks are 64 bytes)
+    auto place = [&](int l, int c) { return l * kWords + ((c ^ ((kChunks == 8 ? l : l >> 1) & (kChunks - 1))) << 2); };
+    auto fetch = [&](int64_t grp, uint32_t* slot) {
+        if (grp < ngroups) {
+            const int64_t e0 = grp * 1024;
+            if (e0 + 1024 <= d) {
+                const uint4* src = reinterpret_cast<const uint4*>(row + e0);
 #pragma unroll
-            for (int s = 0; s < 32; ++s) {
-                if constexpr (sizeof(T) == 4)
-                    x[s] = __ldg(reinterpret_cast<const uint32_t*>(row) + e0 + s * 32 + lane);
-                else
-                    x[s] = (uint32_t)__ldg(reinterpret_cast<const uint16_t*>(row) + e0 + s * 32 + lane) << 16;
-            }
-        } else {
-#pragma unroll
-            for (int s = 0; s < 32; ++s) {
-                const int64_t i = e0 + s * 32 + lane;
-                x[s] = 0u;
-                if (i < d) {
-                    if constexpr (sizeof(T) == 4)
-                        x[s] = reinterpret_cast<const uint32_t*>(row)[i];
-                    else
-                        x[s] = (uint32_t)reinterpret_cast<const uint16_t*>(row)[i] << 16;
+                for (int j = 0; j < kChunks; ++j) {
+                    const int i = j * 32 + lane;  // chunk of the group
+                    cp_async_16(slot + place(i / kChunks, i % kChunks), src + i);
+                }
+            } else {  // ragged last group: entries past d read as +0
+                for (int i = lane; i < kSlot; i += 32) {
+                    uint32_t v = 0u;
+                    if constexpr (sizeof(T) == 4) {
+                        if (e0 + i < d) v = reinterpret_cast<const uint32_t*>(row)[e0 + i];
+                    } else {
+                        const uint16_t* h = reinterpret_cast<const uint16_t*>(row) + e0;
+                        if (e0 + 2 * i < d) v = h[2 * i];
+                        if (e0 + 2 * i + 1 < d) v |= (uint32_t)h[2 * i + 1] << 16;
+                    }
+                    slot[place(i / kWords, (i % kWords) / 4) + (i & 3)] = v;
                 }
             }
         }
+        cp_async_commit();
+    };
+    const bool wide_store = (reinterpret_cast<uintptr_t>(expo) & 31) == 0;
+    uint32_t top = 0;  // largest exponent field seen, at the top of the word
+    int64_t grp = (int64_t)blockIdx.x * (kFloatThreads / 32) + warp;
+    fetch(grp, ring);
+    for (int it = 0; grp < ngroups; grp += stride, ++it) {
+        fetch(grp + stride, ring + ((it + 1) & 1) * kSlot);
+        cp_async_wait<1>();
+        __syncwarp();
+        const uint32_t* slot = ring + (it & 1) * kSlot;
+        uint32_t x[32];
+#pragma unroll
+        for (int c = 0; c < kChunks; ++c) {
+            const uint4 q = *reinterpret_cast<const uint4*>(slot + place(lane, c));
+            x[4 * c] = q.x; x[4 * c + 1] = q.y; x[4 * c + 2] = q.z; x[4 * c + 3] = q.w;
+        }
+        __syncwarp();  // the slot has been read by every lane: the copy after next may land in it
         const int64_t word = grp * 32 + lane;
-        uint32_t sign_w = 0;
+        const bool live = word < words;
+        uint32_t e[8];  // the lane's exponent bytes
+        if constexpr (sizeof(T) == 4) {
 #pragma unroll
-        for (int s = 0; s < 32; ++s) {
-            const uint32_t bs = __ballot_sync(0xFFFFFFFFu, (int)x[s] < 0);
-            if (lane == s) sign_w = bs;
-            const uint32_t E = (x[s] >> 23) & 0xFFu;
-            bad |= E == 0xFFu;
-            sh_expo[warp][s * 32 + lane] = (uint8_t)E;
-        }
-        if (word < words) out[word] = sign_w;
-        for (int j = 1; j <= w; ++j) {
-            const int bit = 23 - (lo + j);  // mantissa digit lo + j of the fp32 encoding
-            uint32_t mine = 0;
-#pragma unroll
-            for (int s = 0; s < 32; ++s) {
-                const uint32_t b = __ballot_sync(0xFFFFFFFFu, (x[s] >> bit) & 1u);
-                if (lane == s) mine = b;
+            for (int q = 0; q < 8; ++q) {
+                const uint32_t a = x[4 * q] << 1, b = x[4 * q + 1] << 1, c = x[4 * q + 2] << 1, f = x[4 * q + 3] << 1;
+                top = max(top, max(max(a, b), max(c, f)));
+                e[q] = __byte_perm(__byte_perm(a, b, 0x0073), __byte_perm(c, f, 0x0073), 0x5410);
             }
-            if (word < words) out[(int64_t)j * words + word] = mine;
+        } else {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const uint32_t a = x[2 * q] << 1, b = x[2 * q + 1] << 1;  // a bit of the low half reaches bit 16: not part of a field
+                e[q] = __byte_perm(a, b, 0x7531);
+                top = max(top, max(max(a, a << 16), max(b, b << 16)));
+            }
         }
-        __syncwarp();
-        if (word < words) {  // the 32 exponent bytes of word `word`: rows are contiguous in the shared-memory matrix
-            const uint4 a = reinterpret_cast<const uint4*>(&sh_expo[warp][lane * 32])[0];
-            const uint4 b = reinterpret_cast<const uint4*>(&sh_expo[warp][lane * 32])[1];
-            reinterpret_cast<uint4*>(ex + word * 32)[0] = a;
-            reinterpret_cast<uint4*>(ex + word * 32)[1] = b;
+        if (live) {
+            uint8_t* dst = ex + word * 32;
+            if (wide_store) {
+                asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(e[0]), "r"(e[1]), "r"(e[2]),
+                             "r"(e[3]), "r"(e[4]), "r"(e[5]), "r"(e[6]), "r"(e[7])
+                             : "memory");
+            } else {
+                reinterpret_cast<uint4*>(dst)[0] = make_uint4(e[0], e[1], e[2], e[3]);
+                reinterpret_cast<uint4*>(dst)[1] = make_uint4(e[4], e[5], e[6], e[7]);
+            }
         }
-        __syncwarp();
+        const uint32_t sign_w = plane_word<T>(x, sizeof(T) == 4 ? 31 : 15);
+        if (live) out[word] = sign_w;
+        if (sizeof(T) == 2 || w < 6) {
+            for (int j = 1; j <= w; ++j) {  // mantissa digit lo + j
+                const uint32_t pw = plane_word<T>(x, kMantBits - (lo + j));
+                if (live) out[(int64_t)j * words + word] = pw;
+            }
+        } else {
+            transpose_bits(x);
+#pragma unroll
+            for (int bit = 22; bit >= 0; --bit) {
+                const int j = kMantBits - bit - lo;
+                if (live && j >= 1 && j <= w) out[(int64_t)j * words + word] = x[bit];
+            }
+        }
     }
-    if (bad) atomicOr(&acc[m], 1u);
+    cp_async_wait<0>();
+    if (top >= 0xFF000000u) atomicOr(&acc[m], 1u);
     if (!last_block(&done[m], gridDim.x) || threadIdx.x != 0) return;
     const bool any_bad = __ldcg(&acc[m]) != 0u;  // NaN or Inf: the worker's message is void
     acc[m] = 0u;
@@ -125,48 +225,91 @@ float_pack_kernel(const T* __restrict__ g, int64_t d, int64_t ld, MantissaSchedu
 }
 
 // Server average: thread = one word (32 entries); terms are added in worker order in fp32.
-__global__ void __launch_bounds__(kFloatThreads)
+// A term is +-2^(E - 127) (1 + f 2^-mb_l / p): the power of two times a multiplier, added by one fused multiply-add (the
+// product with a power of two is exact, so this is the sum of the rounded term).  An exponent field 0 has no leading one
+// and the scale of exponent field 1; a word that holds one takes the general form.
+// Bound by issue: 8 to 14 instructions per entry and worker; the general form for every entry took 0.88 ms for 8 x 124M.
+__global__ void __launch_bounds__(kFloatThreads, 2)
 aggregate_float_kernel(const uint8_t* __restrict__ expo, const uint32_t* __restrict__ planes, const int32_t* level,
                        const double* p_sel, MantissaSchedule sc, int w_max, int64_t words, int M, int64_t d,
                        float* __restrict__ out) {
-    pdl_enter();
     __shared__ float sh_out[kFloatThreads / 32][32][33];
+    __shared__ float sh_c[kFloatThreads];   // 2^-mb_l / p_l of the next workers
+    __shared__ int sh_lv[kFloatThreads];
+    pdl_enter();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const float inv_M = 1.0f / (float)M;
     const int64_t nblk = (words + kFloatThreads - 1) / kFloatThreads;
     for (int64_t blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
         const int64_t word = blk * kFloatThreads + threadIdx.x;
+        const int64_t at = word < words ? word : words - 1;  // lanes past the end repeat the last word
         float acc[32];
 #pragma unroll
         for (int t = 0; t < 32; ++t) acc[t] = 0.0f;
-        if (word < words) {
-            for (int m = 0; m < M; ++m) {  // fixed worker order
-                const int lv = level[m];
+        for (int m0 = 0; m0 < M; m0 += kFloatThreads) {
+            const int nm = min(M - m0, kFloatThreads);
+            if (m0 > 0 || blk == blockIdx.x || M > kFloatThreads) {
+                __syncthreads();
+                if (threadIdx.x < nm) {
+                    const int lv = level[m0 + threadIdx.x];
+                    sh_lv[threadIdx.x] = lv;
+                    sh_c[threadIdx.x] = lv >= 0 ? (float)(ldexp(1.0, -sc.hi[lv]) / p_sel[m0 + threadIdx.x]) : 0.0f;
+                }
+                __syncthreads();
+            }
+            // exponents, signs and the first plane of the next worker are in flight while this one's are added
+            uint4 ea_n, eb_n;
+            uint32_t sgn_n, pw_n;
+            auto preload = [&](int i) {
+                if (i >= nm || sh_lv[i] < 0) return;
+                const uint32_t* pm = planes + (int64_t)(m0 + i) * (1 + w_max) * words + at;
+                const uint4* em = reinterpret_cast<const uint4*>(expo + ((int64_t)(m0 + i) * words + at) * 32);
+                ea_n = __ldg(em);
+                eb_n = __ldg(em + 1);
+                sgn_n = __ldg(pm);
+                pw_n = __ldg(pm + words);
+            };
+            preload(0);
+            for (int i = 0; i < nm; ++i) {  // fixed worker order
+                const uint4 ea = ea_n, eb = eb_n;
+                const uint32_t sgn = sgn_n, pw1 = pw_n;
+                const int lv = sh_lv[i];
+                preload(i + 1);
                 if (lv < 0) continue;
                 const int w = sc.hi[lv] - sc.lo[lv];
-                const float c = (float)(ldexp(1.0, -sc.hi[lv]) / p_sel[m]);  // 2^-mb_l / p_l
-                const uint32_t* pm = planes + (int64_t)m * (1 + w_max) * words;
-                const uint8_t* em = expo + ((int64_t)m * words + word) * 32;
-                const uint32_t sgn = pm[word];
-                const uint4 ea = reinterpret_cast<const uint4*>(em)[0], eb = reinterpret_cast<const uint4*>(em)[1];
-                const uint32_t eb4[8] = {ea.x, ea.y, ea.z, ea.w, eb.x, eb.y, eb.z, eb.w};
-                uint32_t f[32];
+                const float c = sh_c[i];
+                const uint32_t e4[8] = {ea.x, ea.y, ea.z, ea.w, eb.x, eb.y, eb.z, eb.w};
+                uint32_t zero = 0;  // some exponent byte is 0
 #pragma unroll
-                for (int t = 0; t < 32; ++t) f[t] = 0u;
-                for (int j = 1; j <= w; ++j) {
-                    const uint32_t pw = pm[(int64_t)j * words + word];
+                for (int q = 0; q < 8; ++q) zero |= (e4[q] - 0x01010101u) & ~e4[q] & 0x80808080u;
+                if (zero == 0u && w == 1) {
+                    const uint32_t m1 = __float_as_uint(1.0f + c);
 #pragma unroll
-                    for (int t = 0; t < 32; ++t) f[t] = (f[t] << 1) | ((pw >> t) & 1u);
-                }
+                    for (int t = 0; t < 32; ++t) {
+                        const float base = __uint_as_float((t & 3) == 3 ? ((e4[t >> 2] >> 1) & 0x7F800000u)
+                                                                        : ((e4[t >> 2] << (23 - 8 * (t & 3))) & 0x7F800000u));
+                        const uint32_t mag = (pw1 & (1u << t)) ? m1 : 0x3F800000u;
+                        acc[t] = fmaf(base, __uint_as_float(mag ^ ((sgn << (31 - t)) & 0x80000000u)), acc[t]);
+                    }
+                } else {
+                    uint32_t f[32];
 #pragma unroll
-                for (int t = 0; t < 32; ++t) {
-                    const uint32_t E = (eb4[t >> 2] >> (8 * (t & 3))) & 0xFFu;
-                    // exponent field 0: no leading one, and the scale of exponent field 1
-                    const float base = __uint_as_float(E << 23);                   // 2^(E - 127), or 0
-                    const float scale = __uint_as_float(max(E, 1u) << 23);         // 2^(max(E, 1) - 127)
-                    const float ff = __uint_as_float(0x4B000000u | f[t]) - 8388608.0f;  // exact integer-to-float
-                    const float v = fmaf(ff * c, scale, base);  // the power of two last: ff c is a normal number
-                    acc[t] += __uint_as_float(__float_as_uint(v) ^ (((sgn >> t) & 1u) << 31));
+                    for (int t = 0; t < 32; ++t) f[t] = (pw1 >> t) & 1u;
+                    const uint32_t* pm = planes + (int64_t)(m0 + i) * (1 + w_max) * words + at;
+                    for (int j = 2; j <= w; ++j) {
+                        const uint32_t pw = __ldg(pm + (int64_t)j * words);
+#pragma unroll
+                        for (int t = 0; t < 32; ++t) f[t] = (f[t] << 1) | ((pw >> t) & 1u);
+                    }
+#pragma unroll
+                    for (int t = 0; t < 32; ++t) {
+                        const uint32_t E = (e4[t >> 2] >> (8 * (t & 3))) & 0xFFu;
+                        const float base = __uint_as_float(E << 23);                   // 2^(E - 127), or 0
+                        const float scale = __uint_as_float(max(E, 1u) << 23);         // 2^(max(E, 1) - 127)
+                        const float ff = __uint_as_float(0x4B000000u | f[t]) - 8388608.0f;  // exact integer-to-float
+                        const float v = fmaf(ff * c, scale, base);  // the power of two last: ff c is a normal number
+                        acc[t] += __uint_as_float(__float_as_uint(v) ^ ((sgn << (31 - t)) & 0x80000000u));
+                    }
                 }
             }
         }
@@ -183,7 +326,15 @@ aggregate_float_kernel(const uint8_t* __restrict__ expo, const uint32_t* __restr
     }
 }
 
+size_t float_pack_smem(size_t elem) { return (kFloatThreads / 32) * 2 * 1024 * elem; }
+
 }  // namespace
+
+int configure_float_kernels() {
+    const bool ok = cudaFuncSetAttribute(float_pack_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)float_pack_smem(4)) == cudaSuccess;
+    return ok ? MLMC_OK : MLMC_ERR_CUDA;
+}
 
 void launch_compress_floatbits(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* mb,
                                int L, const double* p, uint64_t seed, uint64_t step, const mlmc_float_msgs& out,
@@ -192,11 +343,11 @@ void launch_compress_floatbits(Workspace& ws, const void* g, int dtype, int64_t 
     const int64_t words = (d + 31) / 32;
     const int64_t ngroups = (words + 31) / 32;
     const int64_t by_work = (ngroups + (kFloatThreads / 32) - 1) / (kFloatThreads / 32);
-    int64_t nb = ((int64_t)ws.sm_count * 4) / M;  // whole waves of the blocks that fit an SM, rounded down
+    int64_t nb = ((int64_t)ws.sm_count * 3) / M;  // persistent: three resident blocks per SM, rounded down
     if (nb > by_work) nb = by_work;
     if (nb < 1) nb = 1;
     auto go = [&](auto kernel, auto* row) {
-        launch_kernel(ws, K_FLOAT_PACK, kernel, dim3((unsigned)nb, M), kFloatThreads, 0, s, row, d, ld, sc, prob_list(p, L), seed,
+        launch_kernel(ws, K_FLOAT_PACK, kernel, dim3((unsigned)nb, M), kFloatThreads, float_pack_smem(sizeof(*row)), s, row, d, ld, sc, prob_list(p, L), seed,
                       step, out.expo, out.planes, out.w_max, words, out.level, out.p_sel, ws.acc_word, ws.done, ws.status);
     };
     if (dtype == MLMC_BF16) go(float_pack_kernel<bf16_t>, static_cast<const bf16_t*>(g));
