@@ -177,7 +177,7 @@ int mlmc_create(mlmc_ctx** out, int device, int64_t d_max, int M_max, int L_max)
     cudaDeviceProp prop;
     if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) return MLMC_ERR_CUDA;
     if (configure_select_kernels() != MLMC_OK || configure_emit_kernels() != MLMC_OK ||
-        configure_bit_kernels() != MLMC_OK || configure_float_kernels() != MLMC_OK || configure_sort_kernels() != MLMC_OK)
+        configure_bit_kernels() != MLMC_OK || configure_float_kernels() != MLMC_OK || configure_segment_kernels() != MLMC_OK)
         return MLMC_ERR_CUDA;
 
     mlmc_ctx* ctx = new (std::nothrow) mlmc_ctx();
@@ -241,8 +241,9 @@ int mlmc_create(mlmc_ctx** out, int device, int64_t d_max, int M_max, int L_max)
     const size_t o_brk = pl.take(sizeof(uint4) * M_max);
     const size_t o_bhit = pl.take(sizeof(int) * M_max);
     const size_t o_bstat = pl.take(sizeof(unsigned long long) * 4);
-    ws.sort_scratch = nullptr;
-    ws.sort_rows = 0;
+    ws.seg_scratch = nullptr;
+    ws.seg_rows = 0;
+    ws.seg_cap = 0;
     ws.sig_d = ws.sig_ld = -1;
     ws.sig_M = ws.sig_L = ws.sig_dtype = -1;
 
@@ -315,7 +316,7 @@ int mlmc_destroy(mlmc_ctx* ctx) {
         delete[] ctx->ws.ev_stop;
         delete[] ctx->ws.ev_id;
     }
-    if (ctx->ws.sort_scratch) cudaFree(ctx->ws.sort_scratch);
+    if (ctx->ws.seg_scratch) cudaFree(ctx->ws.seg_scratch);
     const cudaError_t e = cudaFree(ctx->slab);
     delete ctx;
     return finish(e);
@@ -340,8 +341,8 @@ int64_t mlmc_launch_count(const mlmc_ctx* ctx) { return ctx ? ctx->ws.launches :
 static const char* const kKernelNames[] = {
     "begin", "uniforms", "hist1", "resolve1", "sums_candidates", "cand_pass2", "cand_pass3", "band_header", "copy_probs", "emit",
     "agg_offsets", "aggregate_topk", "absmax", "bit_stats", "bit_pack", "aggregate_bitwise", "tile_list", "band_count", "bit_pack_wide",
-    "float_pack", "aggregate_floatbits", "rtn_stats", "rtn_emit", "aggregate_dense", "stopk_draw", "sort_count", "sort_scan",
-    "sort_scatter", "segment_norms"};
+    "float_pack", "aggregate_floatbits", "rtn_stats", "rtn_emit", "aggregate_dense", "segment_resolve",
+    "segment_sweep", "segment_buckets", "segment_norms", "segment_draw"};
 static_assert(sizeof(kKernelNames) / sizeof(kKernelNames[0]) == K_COUNT, "a name for every kernel id");
 
 int mlmc_kernel_count(void) { return K_COUNT; }
@@ -546,24 +547,14 @@ int mlmc_compress_stopk(mlmc_ctx* ctx, const void* g, int dtype, int64_t d, int 
     Workspace& ws = ctx->ws;
     if (L > ws.big_cap) return MLMC_ERR_ARG;
     if (!p) {
-        // Adaptive p with many segments (Lemma 3.4 needs the norm of every segment): the rows are sorted, several
-        // at a time, in scratch memory that the context allocates at the first such call.
+        // Adaptive p with many segments: Lemma 3.4 needs the norm of every segment
         DeviceGuard guard(ws.device);
         cudaStream_t s = static_cast<cudaStream_t>(stream);
-        if (!ws.sort_scratch) {
-            ws.sort_rows = stopk_sort_rows(ws.d_max, ws.big_cap, ws.M_max);
-            if (cudaMalloc(&ws.sort_scratch, stopk_sort_scratch_bytes(ws.d_max, ws.big_cap, ws.M_max)) != cudaSuccess) {
-                cudaGetLastError();
-                ws.sort_scratch = nullptr;
-                return MLMC_ERR_NOMEM;
-            }
-        }
+        if (int rc = reserve_segments(ws, L)) return rc;
         set_call_size(ws, d, M, dtype == MLMC_BF16 ? 2 : 4);
         launch_begin_adaptive(ws, dtype, d, M, nullptr, 1, s);
-        launch_hist1(ws, g, dtype, d, M, ld, false, s);  // the batch maxima for the emission, and the NaN / Inf check
-        for (int m0 = 0; m0 < M; m0 += ws.sort_rows)
-            launch_stopk_sorted_rows(ws, g, dtype, d, m0, (M - m0 < ws.sort_rows) ? M - m0 : ws.sort_rows, ld, s_len, L,
-                                     seed, step, s);
+        launch_hist1(ws, g, dtype, d, M, ld, false, s);
+        launch_segments(ws, g, dtype, d, M, ld, s_len, L, seed, step, s);
         launch_band_header(ws, M, finish_plan(d, 3, 2, false, seed, step, out), s);
         launch_emit(ws, g, dtype, d, M, ld, *out, s);
         return finish(cudaGetLastError());

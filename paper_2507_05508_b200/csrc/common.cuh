@@ -59,7 +59,7 @@ struct EmitParams {
 enum KernelId {
     K_BEGIN = 0, K_UNIFORMS, K_HIST1, K_RESOLVE1, K_SUMS_CAND, K_CAND2, K_CAND3, K_BAND_HEADER, K_COPY_PROBS, K_EMIT, K_AGG_OFFSETS,
     K_AGG_TOPK, K_ABSMAX, K_BIT_STATS, K_BIT_PACK, K_AGG_BIT, K_TILE_LIST, K_BAND_COUNT, K_BIT_PACK_WIDE, K_FLOAT_PACK, K_AGG_FLOAT,
-    K_RTN_STATS, K_RTN_EMIT, K_AGG_DENSE, K_STOPK_DRAW, K_SORT_COUNT, K_SORT_SCAN, K_SORT_SCATTER, K_SEG_NORMS, K_COUNT
+    K_RTN_STATS, K_RTN_EMIT, K_AGG_DENSE, K_SEG_RESOLVE, K_SEG_SWEEP, K_SEG_BUCKETS, K_SEG_NORMS, K_SEG_DRAW, K_COUNT
 };
 
 // Level probabilities handed to a kernel by value.
@@ -136,8 +136,9 @@ struct Workspace {
     int64_t sig_k[kMaxLevels];
     // s-Top-k with more levels than kMaxLevels
     int64_t big_cap;             // most levels
-    uint32_t* sort_scratch;      // key buffers, digit tables and segment norms of the radix sort, for sort_rows rows; allocated at first use
-    int sort_rows;               // rows that are sorted together
+    void* seg_scratch;           // buffers of the segment norms (stopk_segments.cu) for seg_rows rows and seg_cap segments; allocated at first use
+    int seg_rows;
+    int64_t seg_cap;
     // RTN: per-block residual energies of every level
     double* rtn_partial;         // [M][rtn_ctas][kMaxLevels]
     int rtn_ctas;
@@ -161,6 +162,29 @@ struct DrawPlan {
 // device helpers
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ void set_status(int* status, int code) { atomicCAS(status, 0, code); }
+
+// Adds the three 16-bit limbs of x (below 2^48) to the shared-memory words at addr, addr + STRIDE and addr + 2 STRIDE bytes.
+// (Under a predicate each of the three becomes a branch: 33 instead of 22 instructions per entry.)
+template <uint32_t STRIDE>
+__device__ __forceinline__ void shared_add_limbs(uint32_t addr, uint64_t x) {
+    asm volatile("red.shared.add.u32 [%0], %1;\n\tred.shared.add.u32 [%0 + %4], %2;\n\tred.shared.add.u32 [%0 + %5], %3;" ::"r"(addr),
+                 "r"((uint32_t)x & 0xFFFFu), "r"(__byte_perm((uint32_t)x, 0u, 0x4432)), "r"((uint32_t)(x >> 32)), "n"(STRIDE),
+                 "n"(2 * STRIDE)
+                 : "memory");
+}
+
+// Stores x at the shared-memory address `at` and moves on by STEP bytes, where `flag` is negative; no branch.
+template <uint32_t STEP>
+__device__ __forceinline__ void shared_push_if_negative(int flag, uint32_t& at, uint32_t x) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.lt.s32 p, %1, 0;\n\t@p st.shared.u32 [%0], %2;\n\t@p add.u32 %0, %0, %3;\n\t}"
+                 : "+r"(at) : "r"(flag), "r"(x), "n"(STEP) : "memory");
+}
+
+// mant^2 of an fp32 entry (the implicit bit included, below the normal range none): the entry is mant 2^(max(e,1) - 150).
+__device__ __forceinline__ uint64_t mantissa_squared(uint32_t bits) {
+    const uint32_t mant = min(bits & 0x7FFFFFFFu, (bits & 0x7FFFFFu) | 0x800000u);  // the key itself where it lies below 2^23
+    return (uint64_t)mant * mant;
+}
 
 // Every kernel of the library starts with pdl_enter().  The kernels are launched with programmatic stream
 // serialization, so a kernel's blocks may become resident while the kernel before it in the stream is still running;
@@ -385,7 +409,7 @@ inline bool is_sweep(int id) {
     switch (id) {
         case K_HIST1: case K_SUMS_CAND: case K_BAND_COUNT: case K_EMIT: case K_AGG_TOPK: case K_ABSMAX: case K_BIT_STATS:
         case K_BIT_PACK: case K_BIT_PACK_WIDE: case K_AGG_BIT: case K_FLOAT_PACK: case K_AGG_FLOAT: case K_RTN_STATS:
-        case K_RTN_EMIT: case K_AGG_DENSE:
+        case K_RTN_EMIT: case K_AGG_DENSE: case K_SEG_SWEEP:
             return true;
         default:
             return false;
@@ -487,11 +511,10 @@ void launch_rtn_emit(Workspace& ws, const void* g, int dtype, int64_t d, int M, 
                      const mlmc_rtn_msgs& out, cudaStream_t s);
 void launch_aggregate_dense(Workspace& ws, const float* val, const int32_t* level, int M, int64_t d, int64_t ldv,
                             float* out, cudaStream_t s);
-// stopk_sort.cu: s-Top-k with adaptive p and many segments
-int configure_sort_kernels();
-int stopk_sort_rows(int64_t d_max, int64_t big_cap, int M_max);
-size_t stopk_sort_scratch_bytes(int64_t d_max, int64_t big_cap, int M_max);
-void launch_stopk_sorted_rows(Workspace& ws, const void* g, int dtype, int64_t d, int m0, int rows, int64_t ld,
-                              int64_t s_len, int64_t L, uint64_t seed, uint64_t step, cudaStream_t s);
+// stopk_segments.cu: s-Top-k with adaptive p and many segments
+int configure_segment_kernels();
+int reserve_segments(Workspace& ws, int64_t L);
+void launch_segments(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, int64_t s_len, int64_t L,
+                     uint64_t seed, uint64_t step, cudaStream_t s);
 
 }  // namespace mlmc

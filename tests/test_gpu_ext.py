@@ -341,3 +341,34 @@ def test_stopk_exponential_decay_closed_forms(B, ora, ctx):
         assert np.allclose(p_out[m].cpu().numpy(), np.sqrt(delta2) / np.sqrt(delta2).sum(), rtol=2e-6)
         assert dl.sum() ** 2 - float(np.sum(g_np[m].astype(np.float64) ** 2)) == pytest.approx(exact_var, rel=1e-4)
     check_stopk(B, ora, ctx, g, s, None, 2, 0)
+
+
+@pytest.mark.parametrize("case", ["one_bin", "ties_few_values", "many_cells", "groups", "tail"])
+def test_stopk_adaptive_segment_norms_edges(B, ora, ctx, case):
+    """The segment norms where they can go wrong: all keys in one histogram bin (hundreds of boundaries in one bucket, all of
+    its sub-bins), a few distinct values (boundaries that share a threshold), more cells than the sweep keeps in shared
+    memory, rows taken in several groups, and rows of one sweep trip more or less a few entries."""
+    rng = np.random.default_rng(61)
+    if case == "one_bin":
+        g_np = rng.uniform(1.0, 1.0078, (2, 60_001)).astype(np.float32)
+        for s in (100, 1500):
+            check_stopk(B, ora, ctx, to_dev(g_np), s, None, 3, s)
+    elif case == "ties_few_values":
+        g_np = rng.choice(np.array([0.5, -0.5, 0.5000001, 3.0, 0.0], dtype=np.float32), (2, 90_001), p=[0.3, 0.3, 0.29, 0.01, 0.1])
+        for s in (1000, 2500):
+            check_stopk(B, ora, ctx, to_dev(g_np), s, None, 4, s)
+    elif case == "many_cells":
+        g_np = (rng.choice([-1.0, 1.0], (1, 400_000)) * 2.0 ** rng.uniform(-120, 120, (1, 400_000))).astype(np.float32)
+        check_stopk(B, ora, ctx, to_dev(g_np), 50, None, 5, 0)                     # L = 8000: thousands of bins without a boundary
+    elif case == "groups":
+        g = to_dev((rng.standard_normal((3, 50_003)) * 10.0 ** rng.uniform(-3, 0, (3, 50_003))).astype(np.float32))
+        big = B.mlmc_create(0, 130_000_000, 3, 32)                                 # the scratch memory holds two such rows
+        try:
+            for step in range(2):
+                check_stopk(B, ora, big, g, 601, None, 7, step, expect_excluded=1)
+        finally:
+            B.mlmc_destroy(big)
+    else:
+        for d in (8191, 8192, 8195, 24_576):
+            g_np = (rng.standard_normal((2, d)) * 10.0 ** rng.uniform(-2, 0, (2, d))).astype(np.float32)
+            check_stopk(B, ora, ctx, to_dev(g_np), d // 40, None, 8, d, expect_excluded=1)
