@@ -3,8 +3,8 @@
 //   C^l(v) = clip(delta^l round(v / delta^l), -c, c),  delta^l = 2c / (2^{r_l} - 1),  c = max_i |v_i|;
 // the top level is the identity (Def. 3.1) and C^{-1} = 0.  The residual C^l - C^{l-1} is dense and has no band or
 // bit-plane structure, so the adaptive probabilities (Lemma 3.4, Alg. 3) need ||C^l - C^{l-1}|| of every level from
-// one sweep: every thread keeps one fp64 accumulator per level in registers (every entry contributes to every
-// level, so no accumulator has to be selected).  Then the draw, and a sweep that writes the dense message.
+// one sweep: every thread keeps one fp64 accumulator per level in registers.  Then the draw, and a sweep that writes the
+// dense message.
 //
 // The rounding decides an integer, so its arithmetic is fixed (the same on the host checker): with
 // inv = fl32((2^r - 1) / (2c)) and delta = fl32(2c / (2^r - 1)), t = fl32(v inv), k = t rounded to nearest, ties to
@@ -43,59 +43,153 @@ __device__ __forceinline__ float rtn_value(float v, float c, RtnGrid gq) {
     return fminf(fmaxf(__fmul_rn(k, gq.delta), -c), c);
 }
 
+// What the statistics need to know of a level: its grid, the largest magnitude that rounds to 0 and the largest one that
+// the clipping cannot touch (both as bits of a magnitude, so that they compare as integers).
+struct RtnLevel {
+    float inv, delta;
+    int zero_upto, free_upto;  // -1: none
+};
+
+__device__ RtnLevel rtn_level(float c, int r) {
+    const RtnGrid gq = rtn_grid(c, r);
+    RtnLevel v;
+    v.inv = gq.inv;
+    v.delta = gq.delta;
+    // t = fl32(m inv) does not fall as m grows, and t <= 1/2 rounds to 0 (ties to even)
+    v.zero_upto = v.free_upto = -1;
+    if (!(gq.inv <= 3.0e38f)) return v;  // c below the normal range: 1 / delta overflows, and 0 inv is not a number
+    uint32_t z = min(__float_as_uint(0.5f / gq.inv), 0x7F7FFFFFu);
+    while (z > 0u && __fmul_rn(__uint_as_float(z), gq.inv) > 0.5f) --z;
+    while (z < 0x7F7FFFFFu && __fmul_rn(__uint_as_float(z + 1u), gq.inv) <= 0.5f) ++z;
+    v.zero_upto = (int)z;
+    const float f = c - gq.delta;  // |k delta| <= |v| + delta / 2 (1 + 2^-20)
+    if (f > 0.0f) v.free_upto = __float_as_int(f);
+    return v;
+}
+
 // Residual energies of every level: partial[m][block][l] = sum over the block's entries of (C^l - C^{l-1})^2.
+// A warp takes the entries level by level, kRtnHeld per lane.  The levels whose grid is so coarse that the largest of the
+// warp's entries rounds to 0 contribute nothing and are skipped: the clipping value is the row's largest magnitude, and
+// in a gradient with per-layer scales most entries are small beside it.  The first level that is left has C^{l-1} = 0, so
+// its residual is its value.  The differences and sums are fp64 (a difference of two fp32 values is exact); what bounds the
+// kernel where nothing is skipped is the conversion of one fp32 value to fp64 per entry and level (16 per clock and SM).
+// 8 x 124M fp32 entries, L = 5: 2.29 ms with every entry taken through every level.
+constexpr int kRtnHeld = 8;
+
 template <typename T, int LMAX>
-__global__ void __launch_bounds__(kRtnThreads)
+__global__ void __launch_bounds__(kRtnThreads, LMAX <= 6 ? 3 : 2)
 rtn_stats_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* gmax_bits, RtnSchedule sc, double* partial,
                  int rtn_ctas, uint32_t* done, DrawPlan pl, int* status, int* worker_err) {
     using Tr = ElemTraits<T>;
     __shared__ double sh_red[kRtnThreads / 32];
     __shared__ double sh_delta[kMaxLevels], sh_p[kMaxLevels];
+    __shared__ RtnLevel sh_lv[kRtnMaxLevels];
     pdl_enter();
     const int m = blockIdx.y;
     if (worker_err[m]) return;
     const float c = __uint_as_float(gmax_bits[m]);
+    if (threadIdx.x < sc.L - 1) sh_lv[threadIdx.x] = rtn_level(c > 0.0f ? c : 1.0f, sc.r[threadIdx.x]);
+    __syncthreads();
     double acc[LMAX];
-    RtnGrid grid[LMAX];
 #pragma unroll
-    for (int l = 0; l < LMAX; ++l) {
-        acc[l] = 0.0;
-        grid[l] = rtn_grid(c > 0.0f ? c : 1.0f, (l < sc.L - 1) ? sc.r[l] : 1);
-    }
-    if (c > 0.0f) {
-        const T* row = g + (int64_t)m * ld;
-        int64_t v0, v1;
-        block_vector_range(d, Tr::kVec, blockIdx.x, gridDim.x, &v0, &v1);
-        auto take = [&](uint32_t bits) {
-            const float v = Tr::value(bits);
-            double prev = 0.0;  // C^{l-1}
+    for (int l = 0; l < LMAX; ++l) acc[l] = 0.0;
+    auto take = [&](const float (&v)[kRtnHeld]) {
+        int mx = 0;
 #pragma unroll
-            for (int l = 0; l < LMAX; ++l) {
-                // levels past the identity repeat it: their residual is v - v = 0
-                const double cur = (l < sc.L - 1) ? (double)rtn_value(v, c, grid[l]) : (double)v;
-                const double res = cur - prev;
-                acc[l] = fma(res, res, acc[l]);
-                prev = cur;
+        for (int e = 0; e < kRtnHeld; ++e) mx = max(mx, __float_as_int(v[e]) & 0x7FFFFFFF);
+        mx = __reduce_max_sync(0xFFFFFFFFu, mx);
+        double prev[kRtnHeld];  // C^{l-1}
+        bool first = true;      // C^{l-1} = 0 for every entry of the warp (warp-uniform)
+#pragma unroll
+        for (int l = 0; l < LMAX; ++l) {
+            if (l > sc.L - 1) break;
+            if (l == sc.L - 1) {  // the identity
+#pragma unroll
+                for (int e = 0; e < kRtnHeld; ++e) {
+                    const double res = first ? (double)v[e] : (double)v[e] - prev[e];
+                    acc[l] = fma(res, res, acc[l]);
+                }
+                break;
             }
-        };
-        constexpr int kBatch = 2;
-        const int64_t full_end = min(v1, d / Tr::kVec);
-        int64_t v = v0 + threadIdx.x;
-        for (; v + (int64_t)(kBatch - 1) * blockDim.x < full_end; v += (int64_t)kBatch * blockDim.x) {
-            uint4 qv[kBatch];
+            const RtnLevel lv = sh_lv[l];
+            if (mx <= lv.zero_upto) continue;  // the grids get finer: once a level is not skipped, none after it is
+            float x[kRtnHeld];
 #pragma unroll
-            for (int j = 0; j < kBatch; ++j) qv[j] = __ldg(reinterpret_cast<const uint4*>(row) + v + (int64_t)j * blockDim.x);
+            for (int e = 0; e < kRtnHeld; ++e) {
+                const float k = __fadd_rn(__fadd_rn(__fmul_rn(v[e], lv.inv), 12582912.0f), -12582912.0f);
+                x[e] = __fmul_rn(k, lv.delta);
+            }
+            if (mx > lv.free_upto) {
 #pragma unroll
-            for (int j = 0; j < kBatch; ++j) {
-                if constexpr (Tr::kVec == 4) {
-                    take(qv[j].x); take(qv[j].y); take(qv[j].z); take(qv[j].w);
-                } else {
-                    take(qv[j].x & 0xFFFFu); take(qv[j].x >> 16); take(qv[j].y & 0xFFFFu); take(qv[j].y >> 16);
-                    take(qv[j].z & 0xFFFFu); take(qv[j].z >> 16); take(qv[j].w & 0xFFFFu); take(qv[j].w >> 16);
+                for (int e = 0; e < kRtnHeld; ++e) x[e] = fminf(fmaxf(x[e], -c), c);
+            }
+            if (first) {
+#pragma unroll
+                for (int e = 0; e < kRtnHeld; ++e) {
+                    prev[e] = (double)x[e];
+                    acc[l] = fma(prev[e], prev[e], acc[l]);
+                }
+                first = false;
+            } else {
+#pragma unroll
+                for (int e = 0; e < kRtnHeld; ++e) {
+                    const double cur = (double)x[e], res = cur - prev[e];
+                    acc[l] = fma(res, res, acc[l]);
+                    prev[e] = cur;
                 }
             }
         }
-        for (; v < v1; v += blockDim.x) for_each_in_vector<T>(row, v, d, [&](int64_t, uint32_t bits) { take(bits); });
+    };
+    if (c > 0.0f) {
+        const T* row = g + (int64_t)m * ld;
+        constexpr int kVecs = kRtnHeld / Tr::kVec;  // 16-byte vectors per lane and trip; the next trip's are in flight
+        constexpr int kTrip = kRtnThreads * kVecs;
+        const int64_t full_end = d / Tr::kVec;
+        const int64_t trips = full_end / kTrip;
+        auto expand = [&](const uint4 (&q)[kVecs], float (&v)[kRtnHeld]) {
+#pragma unroll
+            for (int j = 0; j < kVecs; ++j) {
+                const uint32_t w[4] = {q[j].x, q[j].y, q[j].z, q[j].w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    if constexpr (Tr::kVec == 4) {
+                        v[4 * j + i] = __uint_as_float(w[i]);
+                    } else {
+                        v[8 * j + 2 * i] = __uint_as_float(w[i] << 16);
+                        v[8 * j + 2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
+                    }
+                }
+            }
+        };
+        uint4 nxt[kVecs];
+        auto load = [&](int64_t trip) {
+            if (trip >= trips) return;
+#pragma unroll
+            for (int j = 0; j < kVecs; ++j)
+                nxt[j] = __ldg(reinterpret_cast<const uint4*>(row) + trip * kTrip + j * kRtnThreads + threadIdx.x);
+        };
+        load(blockIdx.x);
+        for (int64_t trip = blockIdx.x; trip < trips; trip += gridDim.x) {
+            float v[kRtnHeld];
+            expand(nxt, v);
+            load(trip + gridDim.x);
+            take(v);
+        }
+        if (blockIdx.x == gridDim.x - 1) {  // the rest of the row, fewer than kTrip + 1 vectors, one by one
+            for (int64_t i = trips * kTrip * Tr::kVec + threadIdx.x; i < d; i += kRtnThreads) {
+                float v;
+                if constexpr (Tr::kVec == 4) v = reinterpret_cast<const float*>(row)[i];
+                else v = __uint_as_float((uint32_t)reinterpret_cast<const uint16_t*>(row)[i] << 16);
+                double prev = 0.0;
+#pragma unroll
+                for (int l = 0; l < LMAX; ++l) {
+                    if (l > sc.L - 1) break;
+                    const double cur = (l < sc.L - 1) ? (double)rtn_value(v, c, {sh_lv[l].inv, sh_lv[l].delta}) : (double)v;
+                    acc[l] = fma(cur - prev, cur - prev, acc[l]);
+                    prev = cur;
+                }
+            }
+        }
     }
     // fixed-order reduction: shuffle tree per warp, then the warp sums in warp order
 #pragma unroll
@@ -237,7 +331,7 @@ DrawPlan rtn_draw_plan(Workspace& ws, int L, uint64_t seed, uint64_t step, const
 void launch_rtn_stats(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* r, int L,
                       const DrawPlan& plan, cudaStream_t s) {
     const RtnSchedule sc = make_rtn_schedule(r, L);
-    int nb = rtn_blocks(ws, d, dtype == MLMC_BF16 ? 8 : 4, M, 8);
+    int nb = rtn_blocks(ws, d, dtype == MLMC_BF16 ? 8 : 4, M, L <= 6 ? 6 : 4);  // two waves of the resident blocks
     if (nb > ws.rtn_ctas) nb = ws.rtn_ctas;
     auto go = [&](auto kernel, auto* row) {
         launch_kernel(ws, K_RTN_STATS, kernel, dim3(nb, M), kRtnThreads, 0, s, row, d, ld, ws.gmax_bits, sc, ws.rtn_partial,
