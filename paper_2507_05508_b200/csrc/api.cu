@@ -143,14 +143,22 @@ FinishPlan finish_plan(int64_t d, int L, int nq, bool adaptive, uint64_t seed, u
     return pl;
 }
 
-// Adaptive p: every level boundary is a query.
+// Adaptive p: every level boundary is a query.  Rows that a cluster's shared memory holds (2.8 MB) take one launch.
 void select_adaptive(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int64_t* k, int L,
                      uint64_t seed, uint64_t step, const mlmc_topk_msgs* out, cudaStream_t s) {
     FinishPlan pl = finish_plan(d, L, L - 1, true, seed, step, out);
     for (int l = 0; l < L; ++l) pl.k[l] = (uint32_t)k[l];
+    if (cluster_blocks(ws, dtype, d, M) > 0) {
+        launch_cluster_topk(ws, g, dtype, d, M, ld, pl, nullptr, out, s);
+        return;
+    }
     launch_begin_adaptive(ws, dtype, d, M, k, L, s);
     run_selection(ws, g, dtype, d, M, ld, pl, false, s);
+    if (out) launch_emit(ws, g, dtype, d, M, ld, *out, s);
 }
+
+// Longer rows use last call's boundary bins as brackets instead.
+constexpr int64_t kClusterDrawnBytes = 1 << 20;
 
 // Given p: the level of every worker is drawn here (it depends on seed, step and worker only), and the two ranks that
 // bound its band are the only queries.
@@ -160,8 +168,14 @@ void select_drawn(Workspace& ws, const void* g, int dtype, int64_t d, int M, int
     brackets = brackets && dtype == MLMC_F32 && L > 1;
     DrawnBand bands[kEmitMaxWorkers];
     for (int m = 0; m < M; ++m) bands[m] = draw(counter_uniform(seed, step, (uint64_t)m));
+    const FinishPlan pl = finish_plan(d, L, 2, false, seed, step, out);
+    if (d * (dtype == MLMC_BF16 ? 2 : 4) <= kClusterDrawnBytes && cluster_blocks(ws, dtype, d, M) > 0) {
+        launch_cluster_topk(ws, g, dtype, d, M, ld, pl, bands, out, s);
+        return;
+    }
     launch_begin_drawn(ws, dtype, d, M, bands, L, brackets, s);
-    run_selection(ws, g, dtype, d, M, ld, finish_plan(d, L, 2, false, seed, step, out), brackets, s);
+    run_selection(ws, g, dtype, d, M, ld, pl, brackets, s);
+    launch_emit(ws, g, dtype, d, M, ld, *out, s);
 }
 
 }  // namespace
@@ -183,6 +197,10 @@ int mlmc_create(mlmc_ctx** out, int device, int64_t d_max, int M_max, int L_max)
     mlmc_ctx* ctx = new (std::nothrow) mlmc_ctx();
     if (!ctx) return MLMC_ERR_NOMEM;
     Workspace& ws = ctx->ws;
+    if (configure_cluster_kernels(ws) != MLMC_OK) {
+        delete ctx;
+        return MLMC_ERR_CUDA;
+    }
     ws.device = device;
     ws.d_max = d_max;
     ws.M_max = M_max;
@@ -342,7 +360,7 @@ static const char* const kKernelNames[] = {
     "begin", "uniforms", "hist1", "resolve1", "sums_candidates", "cand_pass2", "cand_pass3", "band_header", "copy_probs", "emit",
     "agg_offsets", "aggregate_topk", "absmax", "bit_stats", "bit_pack", "aggregate_bitwise", "tile_list", "band_count", "bit_pack_wide",
     "float_pack", "aggregate_floatbits", "rtn_stats", "rtn_emit", "aggregate_dense", "segment_resolve",
-    "segment_sweep", "segment_buckets", "segment_norms", "segment_draw"};
+    "segment_sweep", "segment_buckets", "segment_norms", "segment_draw", "cluster_topk"};
 static_assert(sizeof(kKernelNames) / sizeof(kKernelNames[0]) == K_COUNT, "a name for every kernel id");
 
 int mlmc_kernel_count(void) { return K_COUNT; }
@@ -483,7 +501,6 @@ int mlmc_compress_topk(mlmc_ctx* ctx, const void* g, int dtype, int64_t d, int M
             return DrawnBand{pn[l], l, l ? (uint32_t)k[l - 1] : 0u, (uint32_t)k[l]};
         }, s);
     }
-    launch_emit(ws, g, dtype, d, M, ld, *out, s);
     return finish(cudaGetLastError());
 }
 
@@ -578,7 +595,6 @@ int mlmc_compress_stopk(mlmc_ctx* ctx, const void* g, int dtype, int64_t d, int 
         const int64_t hi = s_len * (l + 1);
         return DrawnBand{p[l] / sum, (int32_t)l, (uint32_t)(s_len * l), (uint32_t)(hi < d ? hi : d)};
     }, s);
-    launch_emit(ws, g, dtype, d, M, ld, *out, s);
     return finish(cudaGetLastError());
 }
 

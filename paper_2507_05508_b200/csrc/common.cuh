@@ -59,7 +59,7 @@ struct EmitParams {
 enum KernelId {
     K_BEGIN = 0, K_UNIFORMS, K_HIST1, K_RESOLVE1, K_SUMS_CAND, K_CAND2, K_CAND3, K_BAND_HEADER, K_COPY_PROBS, K_EMIT, K_AGG_OFFSETS,
     K_AGG_TOPK, K_ABSMAX, K_BIT_STATS, K_BIT_PACK, K_AGG_BIT, K_TILE_LIST, K_BAND_COUNT, K_BIT_PACK_WIDE, K_FLOAT_PACK, K_AGG_FLOAT,
-    K_RTN_STATS, K_RTN_EMIT, K_AGG_DENSE, K_SEG_RESOLVE, K_SEG_SWEEP, K_SEG_BUCKETS, K_SEG_NORMS, K_SEG_DRAW, K_COUNT
+    K_RTN_STATS, K_RTN_EMIT, K_AGG_DENSE, K_SEG_RESOLVE, K_SEG_SWEEP, K_SEG_BUCKETS, K_SEG_NORMS, K_SEG_DRAW, K_CLUSTER_TOPK, K_COUNT
 };
 
 // Level probabilities handed to a kernel by value.
@@ -88,6 +88,7 @@ struct Workspace {
     int M_max, L_max;
     int sm_count;
     int64_t launches;
+    int cluster_most;            // largest thread-block cluster of the short-row kernels (0: none)
     bool long_sweeps;            // this call's sweeps are long enough to be launched without overlap (see launch_kernel)
     // device memory
     int* status;                 // sticky status word
@@ -424,20 +425,34 @@ constexpr int64_t kLongSweepBytes = 100 << 20;
 inline void set_call_size(Workspace& ws, int64_t d, int M, int elem_size) { ws.long_sweeps = d * M * elem_size > kLongSweepBytes; }
 
 template <typename... P, typename... A>
-inline void launch_kernel(Workspace& ws, int id, void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s,
-                          A&&... args) {
+inline void launch_kernel_cluster(Workspace& ws, int id, int cluster, void (*kernel)(P...), dim3 grid, int threads, size_t smem,
+                                  cudaStream_t s, A&&... args) {
     LaunchScope t(ws, id, s);
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[2];
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cfg.attrs = &attr;
-    cfg.numAttrs = (ws.long_sweeps && is_sweep(id)) ? 0 : 1;
+    cfg.attrs = attr;
+    if (cluster > 1) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+        attr[cfg.numAttrs].val.clusterDim.x = (unsigned)cluster;
+        attr[cfg.numAttrs].val.clusterDim.y = attr[cfg.numAttrs].val.clusterDim.z = 1;
+        ++cfg.numAttrs;
+    }
+    if (!(ws.long_sweeps && is_sweep(id))) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[cfg.numAttrs].val.programmaticStreamSerializationAllowed = 1;
+        ++cfg.numAttrs;
+    }
     cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
+template <typename... P, typename... A>
+inline void launch_kernel(Workspace& ws, int id, void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s,
+                          A&&... args) {
+    launch_kernel_cluster(ws, id, 1, kernel, grid, threads, smem, s, args...);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -511,6 +526,11 @@ void launch_rtn_emit(Workspace& ws, const void* g, int dtype, int64_t d, int M, 
                      const mlmc_rtn_msgs& out, cudaStream_t s);
 void launch_aggregate_dense(Workspace& ws, const float* val, const int32_t* level, int M, int64_t d, int64_t ldv,
                             float* out, cudaStream_t s);
+// topk_cluster.cu: Top-k messages of short rows in one launch
+int configure_cluster_kernels(Workspace& ws);
+int cluster_blocks(const Workspace& ws, int dtype, int64_t d, int M);
+void launch_cluster_topk(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const FinishPlan& plan,
+                         const DrawnBand* bands, const mlmc_topk_msgs* out, cudaStream_t s);
 // stopk_segments.cu: s-Top-k with adaptive p and many segments
 int configure_segment_kernels();
 int reserve_segments(Workspace& ws, int64_t L);

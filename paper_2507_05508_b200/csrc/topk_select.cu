@@ -14,7 +14,7 @@
 //
 // Launches of a selection: begin, hist1, resolve1 and, for fp32, sums_candidates and two digit passes.  The step that
 // needs the whole result of a kernel runs in the block of each worker that finishes last.
-#include "common.cuh"
+#include "topk_finish.cuh"
 
 namespace mlmc {
 
@@ -44,20 +44,6 @@ __device__ __forceinline__ void clear_all(const ZeroList& z) {
     }
 }
 
-__device__ __forceinline__ Query make_query(uint32_t k, int64_t d) {
-    Query q = {};
-    q.k = k;
-    q.slot = kNoSlot;
-    q.trivial = (k == 0u) ? 1u : ((int64_t)k >= d ? 2u : 0u);
-    if (q.trivial == 1u) {
-        q.T = kKeyNone;
-    } else if (q.trivial == 2u) {
-        q.T = 0u;
-        q.r = 0xFFFFFFFFu;
-    }
-    return q;
-}
-
 struct RankList {
     uint32_t k[kMaxQueries];
     int nq;
@@ -72,12 +58,6 @@ begin_adaptive_kernel(ZeroList z, RankList ranks, Query* queries, int64_t d, int
         if (j < ranks.nq) queries[i] = make_query(ranks.k[j], d);
     }
 }
-
-// CAP workers fit the parameter list (24 KB of parameters at 1024 workers).
-template <int CAP>
-struct DrawnList {
-    DrawnBand band[CAP];
-};
 
 template <int CAP>
 __global__ void __launch_bounds__(512)
@@ -270,98 +250,6 @@ hist1_kernel(const T* __restrict__ g, int64_t d, int64_t ld, uint32_t* __restric
 }
 
 // -------------------------------------------------------------------------------------------
-// message headers, probabilities and the draw
-// -------------------------------------------------------------------------------------------
-// Header and emit parameters of one worker whose band (k_lo, k_hi] lies between the thresholds of two queries
-// (null: no threshold on that side).  One thread.
-__device__ void fill_emit(const FinishPlan& pl, int m, int level, double p_sel, const Query* q_lo, const Query* q_hi,
-                          uint32_t k_lo, uint32_t k_hi, EmitParams* emit, int* status, int* worker_err) {
-    EmitParams e = {};
-    e.level = level;
-    e.Ta = q_lo ? q_lo->T : kKeyNone;
-    e.ra = q_lo ? q_lo->r : 0u;
-    e.Tb = q_hi ? q_hi->T : 0u;
-    e.rb = q_hi ? q_hi->r : 0xFFFFFFFFu;
-    e.inv_p = (p_sel > 0.0) ? 1.0 / p_sel : 0.0;
-    e.expect = k_hi - k_lo;
-    e.enabled = 1;
-    if ((int64_t)e.expect > pl.capacity) {
-        e.enabled = 0;
-        worker_err[m] = MLMC_ERR_CAPACITY;
-        set_status(status, MLMC_ERR_CAPACITY);
-    }
-    emit[m] = e;
-    pl.out_count[m] = e.enabled ? (int64_t)e.expect : 0;
-    pl.out_level[m] = e.enabled ? level : -1;
-    pl.out_p_sel[m] = p_sel;
-}
-
-__device__ void fail_worker(const FinishPlan& pl, int m, EmitParams* emit) {
-    if (!pl.want_emit) return;
-    EmitParams e = {};
-    e.level = -1;
-    emit[m] = e;
-    pl.out_count[m] = 0;
-    pl.out_level[m] = -1;
-    pl.out_p_sel[m] = 0.0;
-}
-
-// The end of a selection, by one block per worker.  q: the worker's queries (in shared memory, complete).
-// Adaptive: E[l] = energy of the entries strictly between two thresholds (shared memory); the energy of the threshold
-// keys K is added from their counts, |ranks of K  intersect  (k_{l-1}, k_l]| * val(K)^2; Delta_l = sqrt(E_l);
-// p_l = Delta_l / sum Delta (Lemma 3.4); the level draw.  Then the header of the drawn band.
-__device__ void finish_selection(const FinishPlan& pl, int m, int is_bf16, const Query* q, double* E, double* p_all,
-                                 double* delta_all, EmitParams* emit, int* status, int* worker_err) {
-    __shared__ double sh_p[kMaxLevels];
-    __shared__ double sh_sum;
-    const int L = pl.L;
-    if (pl.adaptive) {
-        const int l = threadIdx.x;
-        if (l < L) {
-            double x2 = E[l];
-            const int64_t lo = l ? (int64_t)pl.k[l - 1] : 0, hi = (int64_t)pl.k[l];
-            uint32_t prev_T = kKeyNone;
-            for (int j = 0; j < L - 1; ++j) {
-                if (q[j].trivial) continue;
-                const uint32_t T = q[j].T;
-                if (T == prev_T) continue;  // thresholds descend: the same key as the query before is counted once
-                prev_T = T;
-                const int64_t c0 = q[j].c, c1 = c0 + (int64_t)q[j].n;
-                const int64_t ov = min(c1, hi) - max(c0, lo);
-                if (ov > 0) {
-                    const double x = (double)__uint_as_float(is_bf16 ? (T << 16) : T);
-                    x2 = fma((double)ov, x * x, x2);
-                }
-            }
-            E[l] = sqrt(x2);
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double s = 0.0;
-            for (int i = 0; i < L; ++i) s += E[i];
-            sh_sum = s;
-        }
-        __syncthreads();
-        if (l < L) {
-            const double s = sh_sum;
-            const double p = (s > 0.0) ? E[l] / s : (l == 0 ? 1.0 : 0.0);
-            sh_p[l] = p;
-            p_all[m * kMaxLevels + l] = p;
-            delta_all[m * kMaxLevels + l] = E[l];
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x != 0 || !pl.want_emit) return;
-    if (pl.adaptive) {
-        const int level = draw_from_probs(sh_p, L, counter_uniform(pl.seed, pl.step, (uint64_t)m));
-        fill_emit(pl, m, level, sh_p[level], level ? &q[level - 1] : nullptr, level < L - 1 ? &q[level] : nullptr,
-                  level ? pl.k[level - 1] : 0u, pl.k[level], emit, status, worker_err);
-    } else {
-        fill_emit(pl, m, emit[m].level, p_all[m * kMaxLevels], &q[0], &q[1], q[0].k, q[1].k, emit, status, worker_err);
-    }
-}
-
-// -------------------------------------------------------------------------------------------
 // after sweep 1: every live query descends into its bin
 // -------------------------------------------------------------------------------------------
 // One block per worker; thread t owns the 32 bins from 32 t.  One scan over the 1024 sums, then the thread whose bins
@@ -383,7 +271,7 @@ resolve1_kernel(const uint32_t* hist1, Query* queries, uint8_t* table1, uint32_t
     const int m = blockIdx.x, nq = pl.nq;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (worker_err[m]) {
-        if (is_bf16 && threadIdx.x == 0) fail_worker(pl, m, emit);
+        if (is_bf16 && threadIdx.x == 0) fail_worker(pl, m, &emit[m]);
         return;
     }
     constexpr int per = kBins1 / kResolveThreads;
@@ -470,7 +358,7 @@ resolve1_kernel(const uint32_t* hist1, Query* queries, uint8_t* table1, uint32_t
             }
             __syncthreads();
         }
-        finish_selection(pl, m, 1, sh_q, sh_E, p_all, delta_all, emit, status, worker_err);
+        finish_selection(pl, m, 1, sh_q, sh_E, p_all, delta_all, emit[m].level, p_all[m * kMaxLevels], &emit[m], status, worker_err);
         return;
     }
     // slots of the second digit pass: live queries in the same bin share one (bins descend with j)
@@ -745,7 +633,7 @@ digit_pass_kernel(const float* __restrict__ g, int64_t d, int64_t ld, const uint
     const int m = blockIdx.y, nq = pl.nq;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (worker_err[m]) {
-        if (PASS == 3 && blockIdx.x == 0 && threadIdx.x == 0) fail_worker(pl, m, emit);
+        if (PASS == 3 && blockIdx.x == 0 && threadIdx.x == 0) fail_worker(pl, m, &emit[m]);
         return;
     }
     uint32_t* sh_hist = sh_digit;
@@ -961,7 +849,7 @@ digit_pass_kernel(const float* __restrict__ g, int64_t d, int64_t ld, const uint
         }
         __syncthreads();
     }
-    finish_selection(pl, m, 0, sh_q, sh_E, p_all, delta_all, emit, status, worker_err);
+    finish_selection(pl, m, 0, sh_q, sh_E, p_all, delta_all, emit[m].level, p_all[m * kMaxLevels], &emit[m], status, worker_err);
 }
 
 __global__ void copy_probs_kernel(const double* p_all, const double* delta_all, ProbList p_fixed, int fixed, int M, int L,
@@ -982,11 +870,11 @@ __global__ void band_header_kernel(FinishPlan pl, const Query* queries, const do
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
     if (m >= M) return;
     if (worker_err[m]) {
-        fail_worker(pl, m, emit);
+        fail_worker(pl, m, &emit[m]);
         return;
     }
     const Query* q = queries + m * kMaxQueries;
-    fill_emit(pl, m, emit[m].level, p_all[m * kMaxLevels], &q[0], &q[1], q[0].k, q[1].k, emit, status, worker_err);
+    fill_emit(pl, m, emit[m].level, p_all[m * kMaxLevels], &q[0], &q[1], q[0].k, q[1].k, &emit[m], status, worker_err);
 }
 
 int blocks_per_worker(const Workspace& ws, int64_t d, int vec, int threads, int M, int waves) {
