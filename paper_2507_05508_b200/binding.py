@@ -98,8 +98,15 @@ def lib() -> C.CDLL:
     return _lib
 
 
+# The handle of the current stream without building a torch.cuda.Stream object (1.5 us a call).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    if _raw_stream is None or _raw_device is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_raw_device())
 
 
 def _dtype_code(g: torch.Tensor) -> int:
@@ -115,10 +122,21 @@ def _check(rc: int, where: str) -> None:
         raise MlmcError(rc, where)
 
 
+_host_arrays = {}     # (ctype, values) -> C array: a program hands over the same few schedules and probabilities step after step
+_HOST_ARRAYS_MOST = 64
+
+
 def _host_array(ctype, values: Optional[Sequence]):
+    """The values as a C array (read only for the library), kept for the next call with equal values."""
     if values is None:
         return None
-    return (ctype * len(values))(*values)
+    key = (ctype, tuple(values))
+    a = _host_arrays.get(key)
+    if a is None:
+        if len(_host_arrays) >= _HOST_ARRAYS_MOST:
+            _host_arrays.clear()
+        a = _host_arrays[key] = (ctype * len(key[1]))(*key[1])
+    return a
 
 
 def mlmc_create(device: int, d_max: int, M_max: int, L_max: int) -> C.c_void_p:
@@ -188,8 +206,8 @@ def _g_args(g: torch.Tensor):
 def mlmc_level_probs(ctx, g: torch.Tensor, kind: int, sched: Sequence[int], p: Optional[Sequence[float]],
                      p_out: torch.Tensor, delta_out: Optional[torch.Tensor]) -> None:
     ptr, dt, d, M, ld = _g_args(g)
-    sch = _host_array(C.c_int64, list(sched))
-    ph = _host_array(C.c_double, None if p is None else list(p))
+    sch = _host_array(C.c_int64, sched)
+    ph = _host_array(C.c_double, p)
     L = len(sched) + (1 if kind == MLMC_RTN else 0)      # the RTN schedule lists the widths below the identity level
     _check(lib().mlmc_level_probs(ctx, ptr, dt, d, M, ld, kind, sch, L, ph, p_out.data_ptr(),
                                   None if delta_out is None else delta_out.data_ptr(), _stream()), "mlmc_level_probs")
@@ -198,8 +216,8 @@ def mlmc_level_probs(ctx, g: torch.Tensor, kind: int, sched: Sequence[int], p: O
 def mlmc_compress_topk(ctx, g: torch.Tensor, k: Sequence[int], p: Optional[Sequence[float]], seed: int, step: int,
                        out: "TopkBuffers") -> None:
     ptr, dt, d, M, ld = _g_args(g)
-    kh = _host_array(C.c_int64, list(k))
-    ph = _host_array(C.c_double, None if p is None else list(p))
+    kh = _host_array(C.c_int64, k)
+    ph = _host_array(C.c_double, p)
     _check(lib().mlmc_compress_topk(ctx, ptr, dt, d, M, ld, kh, len(k), ph, seed, step, C.byref(out.struct),
                                     _stream()), "mlmc_compress_topk")
 
@@ -207,15 +225,15 @@ def mlmc_compress_topk(ctx, g: torch.Tensor, k: Sequence[int], p: Optional[Seque
 def mlmc_compress_bitwise(ctx, g: torch.Tensor, b: Sequence[int], p: Optional[Sequence[float]], seed: int, step: int,
                           out: "BitBuffers") -> None:
     ptr, dt, d, M, ld = _g_args(g)
-    bh = _host_array(C.c_int32, list(b))
-    ph = _host_array(C.c_double, None if p is None else list(p))
+    bh = _host_array(C.c_int32, b)
+    ph = _host_array(C.c_double, p)
     _check(lib().mlmc_compress_bitwise(ctx, ptr, dt, d, M, ld, bh, len(b), ph, seed, step, C.byref(out.struct),
                                        _stream()), "mlmc_compress_bitwise")
 
 
 def mlmc_aggregate(ctx, kind: int, msgs, b: Optional[Sequence[int]], M: int, d: int, out: torch.Tensor) -> None:
     assert out.is_cuda and out.dtype == torch.float32 and out.is_contiguous() and out.numel() >= d
-    bh = _host_array(C.c_int32, None if b is None else list(b))
+    bh = _host_array(C.c_int32, b)
     _check(lib().mlmc_aggregate(ctx, kind, C.byref(msgs.struct), bh, 0 if b is None else len(b), M, d,
                                 out.data_ptr(), _stream()), "mlmc_aggregate")
 
@@ -230,7 +248,7 @@ def mlmc_aggregate_topk_noalloc(msgs: "TopkBuffers", M: int, d: int, out: torch.
 def mlmc_compress_stopk(ctx, g: torch.Tensor, s: int, p: Optional[Sequence[float]], seed: int, step: int,
                         out: "TopkBuffers") -> None:
     ptr, dt, d, M, ld = _g_args(g)
-    ph = None if p is None else (C.c_double * len(p)).from_buffer_copy(memoryview(_as_f64(p)))
+    ph = _host_array(C.c_double, p) if p is None or len(p) <= 4096 else (C.c_double * len(p)).from_buffer_copy(memoryview(_as_f64(p)))
     _check(lib().mlmc_compress_stopk(ctx, ptr, dt, d, M, ld, s, ph, seed, step, C.byref(out.struct), _stream()),
            "mlmc_compress_stopk")
 
@@ -243,15 +261,15 @@ def _as_f64(p):
 def mlmc_compress_floatbits(ctx, g: torch.Tensor, mb: Sequence[int], p: Optional[Sequence[float]], seed: int, step: int,
                             out: "FloatBuffers") -> None:
     ptr, dt, d, M, ld = _g_args(g)
-    mh = _host_array(C.c_int32, list(mb))
-    ph = _host_array(C.c_double, None if p is None else list(p))
+    mh = _host_array(C.c_int32, mb)
+    ph = _host_array(C.c_double, p)
     _check(lib().mlmc_compress_floatbits(ctx, ptr, dt, d, M, ld, mh, len(mb), ph, seed, step, C.byref(out.struct),
                                          _stream()), "mlmc_compress_floatbits")
 
 
 def mlmc_aggregate_floatbits(ctx, msgs: "FloatBuffers", mb: Sequence[int], M: int, d: int, out: torch.Tensor) -> None:
     assert out.is_cuda and out.dtype == torch.float32 and out.is_contiguous() and out.numel() >= d
-    mh = _host_array(C.c_int32, list(mb))
+    mh = _host_array(C.c_int32, mb)
     _check(lib().mlmc_aggregate_floatbits(ctx, C.byref(msgs.struct), mh, len(mb), M, d, out.data_ptr(), _stream()),
            "mlmc_aggregate_floatbits")
 
@@ -260,8 +278,8 @@ def mlmc_compress_rtn(ctx, g: torch.Tensor, r: Sequence[int], p: Optional[Sequen
                       out: "RtnBuffers") -> None:
     """r: the L - 1 round-to-nearest widths; level L - 1 is the identity."""
     ptr, dt, d, M, ld = _g_args(g)
-    rh = _host_array(C.c_int32, list(r)) if len(r) else None
-    ph = _host_array(C.c_double, None if p is None else list(p))
+    rh = _host_array(C.c_int32, r) if len(r) else None
+    ph = _host_array(C.c_double, p)
     _check(lib().mlmc_compress_rtn(ctx, ptr, dt, d, M, ld, rh, len(r) + 1, ph, seed, step, C.byref(out.struct),
                                    _stream()), "mlmc_compress_rtn")
 
