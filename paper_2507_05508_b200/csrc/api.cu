@@ -31,7 +31,8 @@ struct DeviceGuard {
     int prev = -1;
     bool ok = true;
     explicit DeviceGuard(int dev) {
-        ok = cudaGetDevice(&prev) == cudaSuccess && cudaSetDevice(dev) == cudaSuccess;
+        ok = cudaGetDevice(&prev) == cudaSuccess && (prev == dev || cudaSetDevice(dev) == cudaSuccess);
+        if (prev == dev) prev = -1;  // nothing to put back
     }
     ~DeviceGuard() {
         if (prev >= 0) cudaSetDevice(prev);

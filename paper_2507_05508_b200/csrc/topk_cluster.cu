@@ -14,6 +14,8 @@
 //   4. the band: counts per batch, exchanged between the blocks, then every batch is written at its final position.
 #include <cooperative_groups.h>
 
+#include <type_traits>
+
 #include "topk_band.cuh"
 #include "topk_finish.cuh"
 
@@ -30,17 +32,20 @@ constexpr int kClBins = 1 << kClDigit1;
 constexpr int kClHistWords = 8192;               // 16384 16-bit counts, or the energy cells
 constexpr int kClBatches = 86;                   // batches per block at most: 172 KB of the row,
 constexpr int kClBatchesBf16 = 63;               // for bf16 as many as a 16-bit count takes
-constexpr int kClCells = 32 + 256;               // interval + (254 - exponent field)
-constexpr int kClCopies = 8;                     // copies of a cell's limbs
-static_assert(kClCells * 3 * kClCopies <= kClHistWords, "the cells take the place of the histogram");
+constexpr int kClCells = 32 + 256;               // interval + (largest exponent - exponent)
+constexpr int kClCopiesLow = 8;                  // copies of a cell's limbs: 32 where the cells are few enough, else 8
+static_assert(kClCells * 3 * kClCopiesLow <= kClHistWords, "the cells take the place of the histogram");
 static_assert(kClBatches * kBatchWords < 65536 && kClBatchesBf16 * kBatchWords * 2 < 65536, "16-bit counts, and 16-bit limbs added at most 65535 times");
 
 struct ClusterShared {
     Query q[kMaxQueries];
     uint32_t first[kMaxQueries], slots;          // first query of a boundary bin (slot), number of slots
+    int bin[kMaxQueries];                        // leading-digit bin of a query; kClBins above, -1 below every bin
+    uint32_t listed, low_bin;                    // keys of the boundary bins; lowest bin with a key
     double E[kMaxLevels];
     EmitParams emit;
-    uint32_t total[kClMost], top[kClMost];       // per block: keys in its bins / its largest key
+    uint32_t top[kClMost];                       // per block: its largest key
+    uint16_t part[kClMost][kClMost];             // [block][range of bins]: the block's keys in the range
     uint4 counts[kClMost];                       // per block: {C, A, B, batches}
     uint32_t warp[32];
     uint32_t batch_max[kClBatches];
@@ -72,6 +77,10 @@ cluster_topk_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int nq = pl.nq;
     for (int i = t; i < kClHistWords; i += kClThreads) sh_hist[i] = 0u;
+    if (t == 0) {
+        sh.listed = 0u;
+        sh.low_bin = kClBins;
+    }
     if (t < nq) sh.q[t] = make_query(pl.adaptive ? pl.k[t] : (t ? drawn.band[m].k_hi : drawn.band[m].k_lo), d);
     pdl_enter();
 
@@ -115,6 +124,19 @@ cluster_topk_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid
     __syncthreads();
     my_top = __reduce_max_sync(0xFFFFFFFFu, sh.warp[lane]);
     if (t < CL) cluster.map_shared_rank(sh.top, t)[rank] = my_top;
+    const int own = kClBins / CL;  // bins of the first digit that a block resolves, two per word
+    if (warp < CL) {  // warp r: how many of this block's keys lie in the range of block r
+        uint32_t n = 0, low = kClBins;
+        for (int i = lane; i < own / 2; i += 32) {
+            const uint32_t x = sh_hist[warp * (own / 2) + i];
+            n += (x & 0xFFFFu) + (x >> 16);
+            if (x) low = min(low, (uint32_t)(warp * own + 2 * i));
+        }
+        n = __reduce_add_sync(0xFFFFFFFFu, n);
+        low = __reduce_min_sync(0xFFFFFFFFu, low);
+        if (lane < CL) cluster.map_shared_rank(&sh.part[0][0], lane)[rank * kClMost + warp] = (uint16_t)n;
+        if (lane == 0 && low < kClBins) atomicMin(&sh.low_bin, low);
+    }
     cluster.sync();
     uint32_t top = 0;
     for (int r = 0; r < CL; ++r) top = max(top, sh.top[r]);
@@ -132,41 +154,60 @@ cluster_topk_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid
         return;
     }
 
-    // ---- 2. first digit: this block takes the bins [rank, rank + 1) * kClBins / CL
+    // ---- 2. first digit: this block takes the bins [rank, rank + 1) * own
     if (nq > 0) {
-        const int own = kClBins / CL;  // 512 or 1024 bins, two per word
-        uint32_t c0 = 0, c1 = 0;
-        const int word = (rank * own) / 2 + t;
-        if (t < own / 2) {
-#pragma unroll 8
-            for (int r = 0; r < CL; ++r) {
-                const uint32_t x = cluster.map_shared_rank(sh_hist, r)[word];
-                c0 += x & 0xFFFFu;
-                c1 += x >> 16;
+        // a thread owns `span` consecutive words of the block's range (more than one only in small clusters)
+        constexpr int kMostWords = kClBins / 2 / kClThreads;
+        const int span = max(1, own / 2 / kClThreads), word = (rank * own) / 2 + t * span;
+        uint32_t c[2 * kMostWords] = {}, above = 0, sum = 0;
+        if (t * span < own / 2) {
+            if (span == 1) {
+                uint32_t x[kClMost];
+#pragma unroll
+                for (int r = 0; r < kClMost; ++r) x[r] = (r < CL) ? cluster.map_shared_rank(sh_hist, r)[word] : 0u;
+#pragma unroll
+                for (int r = 0; r < kClMost; ++r) {
+                    c[0] += x[r] & 0xFFFFu;
+                    c[1] += x[r] >> 16;
+                }
+            } else {
+                for (int r = 0; r < CL; ++r)
+#pragma unroll
+                    for (int i = 0; i < kMostWords; ++i) {
+                        const uint32_t x = i < span ? cluster.map_shared_rank(sh_hist, r)[word + i] : 0u;
+                        c[2 * i] += x & 0xFFFFu;
+                        c[2 * i + 1] += x >> 16;
+                    }
             }
         }
-        // keys of the block's bins above this thread's: suffix sums (threads past own / 2 hold none)
-        const uint32_t sum = c0 + c1;
+#pragma unroll
+        for (int i = 0; i < 2 * kMostWords; ++i) sum += c[i];
+        // keys in the ranges above this block's, then in the block's bins above this thread's
+        for (int i = lane; i < CL * kClMost; i += 32) above += (i % kClMost > rank && i % kClMost < CL) ? sh.part[i / kClMost][i % kClMost] : 0u;
+        above = __reduce_add_sync(0xFFFFFFFFu, above);
         uint32_t suffix = sum;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const uint32_t y = __shfl_down_sync(0xFFFFFFFFu, suffix, o);
             if (lane + o < 32) suffix += y;
         }
+        __syncthreads();  // sh.warp has been read
         if (lane == 0) sh.warp[warp] = suffix;
         __syncthreads();
-        const uint32_t w = sh.warp[lane];
-        uint32_t above = suffix - sum + __reduce_add_sync(0xFFFFFFFFu, lane > warp ? w : 0u);
-        const uint32_t mine = __reduce_add_sync(0xFFFFFFFFu, w);
-        if (t < CL) cluster.map_shared_rank(sh.total, t)[rank] = mine;
-        cluster.sync();
-        for (int r = rank + 1; r < CL; ++r) above += sh.total[r];
-        if (t < own / 2) {
+        above += suffix - sum + __reduce_add_sync(0xFFFFFFFFu, lane > warp ? sh.warp[lane] : 0u);
+        if (sum) {
             for (int j = 0; j < nq; ++j) {
                 const uint32_t k = sh.q[j].k;
-                if (sh.q[j].trivial == 0u && above < k && k <= above + sum) {  // this thread's bins hold rank k
-                    const bool upper = k <= above + c1;
-                    const uint32_t bin = (uint32_t)(2 * word + (upper ? 1 : 0)), ab = upper ? above : above + c1;
+                if (above < k && k <= above + sum && sh.q[j].trivial == 0u) {  // this thread's bins hold rank k
+                    uint32_t bin = 0, ab = 0, run = above;
+#pragma unroll
+                    for (int i = 2 * kMostWords - 1; i >= 0; --i) {  // the last bin that is entered holds the rank
+                        if (run < k) {
+                            bin = (uint32_t)(2 * word + i);
+                            ab = run;
+                        }
+                        run += c[i];
+                    }
                     for (int r = 0; r < CL; ++r) {
                         Query& q = cluster.map_shared_rank(sh.q, r)[j];
                         q.prefix = bin << kShift1;
@@ -177,49 +218,53 @@ cluster_topk_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid
         }
         cluster.sync();
     }
-    // codes of the bins: 64 + slot where a boundary lies in the bin, else the number of boundaries above it
-    if (t < kMaxQueries) {
-        const int j = t;
-        uint32_t slot = 0, prev = kKeyNone;
-        bool is_first = false;
-        if (j < nq) {
-            for (int i = 0; i <= j; ++i) {
-                if (sh.q[i].trivial) continue;
-                const bool next = prev == kKeyNone || sh.q[i].prefix != prev;
-                if (next && prev != kKeyNone) ++slot;
-                if (i == j) is_first = next;
-                prev = sh.q[i].prefix;
-            }
-            if (!sh.q[j].trivial) {
-                sh.q[j].slot2 = slot;
-                if (is_first) sh.first[slot] = (uint32_t)j;
-            }
+    // The live queries are contiguous (k = 0 before them, k >= d after them) and their prefixes descend: queries with the
+    // same prefix share a histogram slot, numbered by the first of them.  By warp 0, a query per lane.
+    auto number_slots = [&](bool first_digit) {
+        const bool live = lane < nq && sh.q[lane].trivial == 0u;
+        const uint32_t prefix = live ? sh.q[lane].prefix : kKeyNone, prev = __shfl_up_sync(0xFFFFFFFFu, prefix, 1);
+        const bool is_first = live && (lane == 0 || prefix != prev);
+        const uint32_t firsts = __ballot_sync(0xFFFFFFFFu, is_first);
+        const uint32_t slot = (uint32_t)__popc(firsts & ((2u << lane) - 1u)) - 1u;
+        if (live) sh.q[lane].slot = slot;
+        if (first_digit) {
+            if (live) sh.q[lane].slot2 = slot;
+            if (is_first) sh.first[slot] = (uint32_t)lane;
+            if (lane < nq) sh.bin[lane] = live ? (int)(prefix >> kShift1) : (sh.q[lane].trivial == 2u ? -1 : kClBins);
+            if (lane == 0) sh.slots = (uint32_t)__popc(firsts);
         }
-        const uint32_t firsts = __ballot_sync(0xFFFFFFFFu, j < nq && is_first);
-        if (j == 0) sh.slots = (uint32_t)__popc(firsts);
-    }
+    };
+    if (warp == 0) number_slots(true);
     for (int i = t; i < kClHistWords; i += kClThreads) sh_hist[i] = 0u;
     __syncthreads();
     {
+        // codes of the bins: 64 + slot where a boundary lies in the bin, else the number of boundaries above it
         constexpr int per = kClBins / kClThreads;  // 8 consecutive bins per thread
-        int j = 0;
-        auto bin_of = [&](int i) -> int {
-            const Query& q = sh.q[i];
-            return q.trivial == 0u ? (int)(q.prefix >> kShift1) : (q.trivial == 2u ? -1 : kClBins);
-        };
-        uint32_t codes[2] = {0u, 0u};
+        const int hi_bin = t * per + per - 1;
+        int j = 0, n = nq;                         // the first query whose bin is not above the thread's
+        while (n > 0) {
+            const int half = n >> 1;
+            if (sh.bin[j + half] > hi_bin) { j += half + 1; n -= half + 1; } else n = half;
+        }
+        uint32_t codes[2];
+        if (j == nq || sh.bin[j] < t * per) {
+            codes[0] = codes[1] = (uint32_t)j * 0x01010101u;
+        } else {
+            codes[0] = codes[1] = 0u;
 #pragma unroll
-        for (int i = per - 1; i >= 0; --i) {
-            const int b = t * per + i;
-            while (j < nq && bin_of(j) > b) ++j;
-            const uint32_t code = (j < nq && bin_of(j) == b) ? 64u + sh.q[j].slot2 : (uint32_t)j;
-            codes[i >> 2] |= code << (8 * (i & 3));
+            for (int i = per - 1; i >= 0; --i) {
+                const int b = t * per + i;
+                while (j < nq && sh.bin[j] > b) ++j;
+                const uint32_t code = (j < nq && sh.bin[j] == b) ? 64u + sh.q[j].slot2 : (uint32_t)j;
+                codes[i >> 2] |= code << (8 * (i & 3));
+            }
         }
         reinterpret_cast<uint2*>(sh_tab)[t] = make_uint2(codes[0], codes[1]);
     }
     __syncthreads();
     const int words4 = nb * kBatchWords / 4;
-    // every key of the block's words; the padding past the row's end has keys above every finite one
+    // every key of the block's words (place: its element number in shared memory); the padding past the row's end has
+    // keys above every finite one
     auto for_each_key = [&](auto&& f) {
         for (int i = t; i < words4; i += kClThreads) {
             const uint4 q = *reinterpret_cast<const uint4*>(sh_row + i * 4);
@@ -227,156 +272,204 @@ cluster_topk_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid
 #pragma unroll
             for (int c = 0; c < 4; ++c)
 #pragma unroll
-                for (int s = 0; s < EW::S; ++s) f(EW::key(x[c], s));
+                for (int s = 0; s < EW::S; ++s) f(EW::key(x[c], s), (uint32_t)((i * 4 + c) * EW::S + s));
         }
     };
-    // one more digit of every query: count_bits bits at `shift`, counted per slot.  Every CL-th query is this block's.
-    auto descend = [&](int shift, int bits, bool last) {
+    // The places of the keys in boundary bins are listed by the first pass over them, behind the counts (two digits of at
+    // most `slots` slots), as far as they fit; otherwise the passes after it look at every key again.
+    const uint32_t hist_words = (sh.slots << kBits2) / 2 > (uint32_t)(nq << kShift2) / 2 ? (sh.slots << kBits2) / 2 : (uint32_t)(nq << kShift2) / 2;
+    uint16_t* sh_list = reinterpret_cast<uint16_t*>(sh_hist + ((hist_words + 3u) & ~3u));
+    const uint32_t list_cap = 2u * (kClHistWords - ((hist_words + 3u) & ~3u));
+    auto key_at = [&](uint32_t place) -> uint32_t { return EW::key(sh_row[place / EW::S], place % EW::S); };
+    auto for_each_boundary_key = [&](auto&& f) {
+        const uint32_t n = sh.listed;
+        if (n <= list_cap) {
+            for (uint32_t i = t; i < n; i += kClThreads) f(key_at(sh_list[i]));
+        } else {
+            for_each_key([&](uint32_t key, uint32_t) {
+                if (sh_tab[key >> kShift1] >= 64u) f(key);
+            });
+        }
+    };
+    // One more digit of every query: `bits` bits at `shift`, counted per slot.  Warp w of block r takes query r + w CL: a
+    // lane adds up its share of the slot's counts over the blocks, the warp finds the digit and tells every block.
+    auto descend = [&](auto bits_tag, int shift, bool last) {
+        constexpr int bits = decltype(bits_tag)::value;
+        constexpr int words = (1 << bits) / 2 < 32 ? (1 << bits) / 2 : 32;  // lanes with counts
+        constexpr int per = (1 << bits) / 2 / words;                       // words per lane: 8 (9 bits) or 1 (2 bits)
         cluster.sync();  // every block's counts are complete
-        const int nwords = (1 << bits) / 2 > 0 ? (1 << bits) / 2 : 1;
-        for (int j = rank; j < nq; j += CL) {
-            if (sh.q[j].trivial) continue;  // block-uniform
-            const uint32_t base = (sh.q[j].slot << bits) / 2;
-            uint32_t c0 = 0, c1 = 0;
-            if (t < nwords) {
-#pragma unroll 8
+        const int j = rank + warp * CL;
+        if (j < nq && sh.q[j].trivial == 0u) {
+            const int base = (int)(sh.q[j].slot << bits) / 2 + (words - 1 - lane) * per;  // lane 0 owns the largest digits
+            uint32_t c[2 * per] = {}, sum = 0;
+            if (lane < words) {
                 for (int r = 0; r < CL; ++r) {
-                    const uint32_t x = cluster.map_shared_rank(sh_hist, r)[base + t];
-                    c0 += x & 0xFFFFu;
-                    c1 += x >> 16;
+                    const uint32_t* src = cluster.map_shared_rank(sh_hist, r) + base;
+                    if constexpr (per == 8) {
+                        const uint4 a = reinterpret_cast<const uint4*>(src)[0], b = reinterpret_cast<const uint4*>(src)[1];
+                        const uint32_t x[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            c[2 * i] += x[i] & 0xFFFFu;
+                            c[2 * i + 1] += x[i] >> 16;
+                        }
+                    } else {
+                        c[0] += src[0] & 0xFFFFu;
+                        c[1] += src[0] >> 16;
+                    }
                 }
             }
-            const uint32_t sum = c0 + c1;
-            uint32_t suffix = sum;
+#pragma unroll
+            for (int i = 0; i < 2 * per; ++i) sum += c[i];
+            uint32_t upto = sum;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_down_sync(0xFFFFFFFFu, suffix, o);
-                if (lane + o < 32) suffix += y;
+                const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, upto, o);
+                if (lane >= o) upto += y;
             }
-            __syncthreads();
-            if (lane == 0) sh.warp[warp] = suffix;
-            __syncthreads();
-            const uint32_t w = sh.warp[lane];
-            const uint32_t above = suffix - sum + __reduce_add_sync(0xFFFFFFFFu, lane > warp ? w : 0u);
             const uint32_t rem = sh.q[j].rem;
-            __syncthreads();  // read by everyone before the owner rewrites it
-            if (t < nwords && above < rem && rem <= above + sum) {
-                const bool upper = rem <= above + c1;
-                const uint32_t digit = (uint32_t)(2 * t + (upper ? 1 : 0)), left = rem - (upper ? above : above + c1);
-                const uint32_t prefix = sh.q[j].prefix | (digit << shift), n = upper ? c1 : c0;
-                for (int r = 0; r < CL; ++r) {
-                    Query& q = cluster.map_shared_rank(sh.q, r)[j];
-                    q.prefix = prefix;
-                    q.rem = left;
-                    if (last) {
-                        q.T = prefix;
-                        q.r = left;
-                        q.n = n;
-                        q.c = q.k - left;
-                    }
+            uint32_t run = upto - sum, digit = 0, left = 0, n = 0;
+            const bool mine = run < rem && rem <= upto;
+#pragma unroll
+            for (int i = 2 * per - 1; i >= 0; --i) {
+                if (run < rem) {  // the last digit that is entered holds the rank
+                    digit = (uint32_t)((words - 1 - lane) * per * 2 + i);
+                    left = rem - run;
+                    n = c[i];
+                }
+                run += c[i];
+            }
+            const int from = __ffs(__ballot_sync(0xFFFFFFFFu, mine)) - 1;
+            digit = __shfl_sync(0xFFFFFFFFu, digit, from);
+            left = __shfl_sync(0xFFFFFFFFu, left, from);
+            n = __shfl_sync(0xFFFFFFFFu, n, from);
+            const uint32_t prefix = sh.q[j].prefix | (digit << shift), k = sh.q[j].k;
+            __syncwarp();
+            if (lane < CL) {
+                Query& q = cluster.map_shared_rank(sh.q, lane)[j];
+                q.prefix = prefix;
+                q.rem = left;
+                if (last) {
+                    q.T = prefix;
+                    q.r = left;
+                    q.n = n;
+                    q.c = k - left;
                 }
             }
         }
         cluster.sync();
     };
+    auto count = [&](uint32_t i) { atomicAdd(&sh_hist[i >> 1], 1u << ((i & 1u) * 16u)); };
     if (nq > 0) {
-        if (t < nq) sh.q[t].slot = sh.q[t].slot2;
-        for_each_key([&](uint32_t key) {
+        for_each_key([&](uint32_t key, uint32_t place) {
             const uint32_t code = sh_tab[key >> kShift1];
             if (code >= 64u) {
-                const uint32_t i = ((code - 64u) << kBits2) | ((key >> kShift2) & ((1u << kBits2) - 1u));
-                atomicAdd(&sh_hist[i >> 1], 1u << ((i & 1u) * 16u));
+                count(((code - 64u) << kBits2) | ((key >> kShift2) & ((1u << kBits2) - 1u)));
+                const uint32_t at = atomicAdd(&sh.listed, 1u);
+                if (at < list_cap) sh_list[at] = (uint16_t)place;
             }
         });
-        descend(kShift2, kBits2, kShift2 == 0);
+        descend(std::integral_constant<int, kBits2>(), kShift2, kShift2 == 0);
         if constexpr (kShift2 > 0) {
-            if (t < nq && !sh.q[t].trivial) {  // queries with the same prefix share a slot (prefixes descend)
-                uint32_t slot = 0, prev = kKeyNone;
-                for (int i = 0; i <= t; ++i) {
-                    if (sh.q[i].trivial) continue;
-                    if (prev != kKeyNone && sh.q[i].prefix != prev) ++slot;
-                    prev = sh.q[i].prefix;
-                }
-                sh.q[t].slot = slot;
-            }
-            for (int i = t; i < kClHistWords; i += kClThreads) sh_hist[i] = 0u;
+            if (warp == 0) number_slots(false);
+            for (uint32_t i = t; i < hist_words; i += kClThreads) sh_hist[i] = 0u;
             __syncthreads();
-            for_each_key([&](uint32_t key) {
-                const uint32_t code = sh_tab[key >> kShift1];
-                if (code >= 64u) {
-                    const uint32_t s = code - 64u;
-                    for (int j = (int)sh.first[s]; j < nq && !sh.q[j].trivial && sh.q[j].slot2 == s; ++j) {
-                        if ((sh.q[j].prefix >> kShift2) == (key >> kShift2)) {
-                            const uint32_t i = (sh.q[j].slot << kShift2) | (key & ((1u << kShift2) - 1u));
-                            atomicAdd(&sh_hist[i >> 1], 1u << ((i & 1u) * 16u));
-                            break;
-                        }
+            for_each_boundary_key([&](uint32_t key) {
+                const uint32_t s = sh_tab[key >> kShift1] - 64u;
+                for (int j = (int)sh.first[s]; j < nq && sh.q[j].trivial == 0u && sh.q[j].slot2 == s; ++j) {
+                    if ((sh.q[j].prefix >> kShift2) == (key >> kShift2)) {
+                        count((sh.q[j].slot << kShift2) | (key & ((1u << kShift2) - 1u)));
+                        break;
                     }
                 }
             });
-            descend(0, kShift2, true);
+            descend(std::integral_constant<int, (kShift2 > 0 ? kShift2 : 2)>(), 0, true);
         }
     }
 
     // ---- 3. energies of the open intervals
     if (pl.adaptive) {
+        // A cell is (interval, exponent), numbered interval + (largest exponent - exponent): neither falls as the keys fall.
+        auto exponent = [&](uint32_t key) -> int { return (int)((Tr::kVec == 4 ? key : key << 16) >> 23); };
+        const int top_e = exponent(top);
+        const int span = nq + 1 + top_e - exponent(min(sh.low_bin, (uint32_t)kClBins - 1u) << kShift1);  // cells of this block
+        const bool many = span * 3 * 32 > kClHistWords;
+        const int copies = many ? kClCopiesLow : 32, copy = lane & (copies - 1);
+        // the keys of the boundary bins first, while their list is intact: their cells wait in a register each
         __syncthreads();
-        for (int i = t; i < kClCells * 3 * kClCopies; i += kClThreads) sh_hist[i] = 0u;
+        const uint32_t nlist = sh.listed;
+        const bool by_list = nq > 0 && nlist <= list_cap && nlist <= 8u * kClThreads;
+        uint32_t held[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) held[i] = (by_list && (uint32_t)(t + i * kClThreads) < nlist) ? sh_list[t + i * kClThreads] : 0xFFFFFFFFu;
         __syncthreads();
-        const uint32_t copy = lane & (kClCopies - 1);
-        const uint32_t top_e = 254u;
-        for_each_key([&](uint32_t key) {
-            uint32_t interval = sh_tab[key >> kShift1];
-            if (interval >= 64u) {
-                const uint32_t s = interval - 64u;
-                int j = (int)sh.first[s];
-                while (j < nq && sh.q[j].T > key) ++j;  // thresholds descend; a query with k = d has T = 0
-                if (j < nq && sh.q[j].T == key && sh.q[j].trivial == 0u) return;  // a threshold key: added from its count
-                interval = (uint32_t)j;
-            }
-            if (key >= Tr::kInfKey || key == 0u) return;  // padding; zeros add nothing
+        for (int i = t; i < kClHistWords; i += kClThreads) sh_hist[i] = 0u;
+        __syncthreads();
+        auto add = [&](uint32_t interval, uint32_t key) {
             const uint32_t bits = Tr::kVec == 4 ? key : key << 16;
             const uint64_t m2 = mantissa_squared(bits);
-            uint32_t* a = sh_hist + (interval + top_e - (bits >> 23)) * (3 * kClCopies) + copy;
+            uint32_t* a = sh_hist + (interval + top_e - (bits >> 23)) * (3 * copies) + copy;
             atomicAdd(a, (uint32_t)m2 & 0xFFFFu);
-            atomicAdd(a + kClCopies, (uint32_t)(m2 >> 16) & 0xFFFFu);
-            atomicAdd(a + 2 * kClCopies, (uint32_t)(m2 >> 32));
+            atomicAdd(a + copies, (uint32_t)(m2 >> 16) & 0xFFFFu);
+            atomicAdd(a + 2 * copies, (uint32_t)(m2 >> 32));
+        };
+        auto add_boundary = [&](uint32_t key) {
+            int j = (int)sh.first[sh_tab[key >> kShift1] - 64u];
+            while (j < nq && sh.q[j].T > key) ++j;  // thresholds descend; a query with k >= d has T = 0
+            if (j < nq && sh.q[j].T == key && sh.q[j].trivial == 0u) return;  // a threshold key: added from its count
+            add((uint32_t)j, key);
+        };
+        for_each_key([&](uint32_t key, uint32_t) {
+            const uint32_t code = sh_tab[key >> kShift1];
+            if (key >= Tr::kInfKey || key == 0u) return;  // padding; zeros add nothing
+            if (code < 64u) add(code, key);
+            else if (!by_list) add_boundary(key);
         });
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (held[i] != 0xFFFFFFFFu) {
+                const uint32_t key = key_at(held[i]);
+                if (key != 0u) add_boundary(key);
+            }
         __syncthreads();
         unsigned long long* sh_sum = reinterpret_cast<unsigned long long*>(sh_tab);  // [kClCells][2]: the codes are not needed any more
         static_assert(kClCells * 16 <= kClBins, "the sums take the place of the codes");
         if (t < kClCells) {
             unsigned long long lo = 0, hi = 0;
-            const uint32_t* a = sh_hist + t * (3 * kClCopies);
-#pragma unroll
-            for (int r = 0; r < kClCopies; ++r) {
-                lo += (unsigned long long)a[r] + ((unsigned long long)a[kClCopies + r] << 16);
-                hi += a[2 * kClCopies + r];
+            if (many || t < span) {
+                const uint32_t* a = sh_hist + t * (3 * copies);
+                for (int r = 0; r < copies; ++r) {
+                    const int c = (r + t) & (copies - 1);  // neighbours start in different banks
+                    lo += (unsigned long long)a[c] + ((unsigned long long)a[copies + c] << 16);
+                    hi += a[2 * copies + c];
+                }
             }
             sh_sum[2 * t] = lo;
             sh_sum[2 * t + 1] = hi;
         }
         cluster.sync();
         double* sh_cell = reinterpret_cast<double*>(sh_hist);  // [kClCells]: sum of mant^2 over the row
-        if (t < kClCells) {
-            unsigned long long lo = 0, hi = 0;
-#pragma unroll 4
-            for (int r = 0; r < CL; ++r) {
-                const unsigned long long* o = cluster.map_shared_rank(sh_sum, r);
-                lo += o[2 * t];
-                hi += o[2 * t + 1];
-            }
-            const unsigned __int128 tot = ((unsigned __int128)hi << 32) + lo;
-            sh_cell[t] = (double)(unsigned long long)(tot >> 64) * 0x1.0p64 + (double)(unsigned long long)tot;
+        if (t < 2 * kClCells) {  // thread 2 c + h adds half h of cell c over the blocks
+            unsigned long long x[kClMost], sum = 0;
+#pragma unroll
+            for (int r = 0; r < kClMost; ++r) x[r] = (r < CL) ? cluster.map_shared_rank(sh_sum, r)[t] : 0ull;
+#pragma unroll
+            for (int r = 0; r < kClMost; ++r) sum += x[r];
+            const unsigned long long hi = __shfl_down_sync(0xFFFFFFFFu, sum, 1);
+            const unsigned __int128 tot = ((unsigned __int128)hi << 32) + sum;
+            if ((t & 1) == 0) sh_cell[t >> 1] = (double)(unsigned long long)(tot >> 64) * 0x1.0p64 + (double)(unsigned long long)tot;
         }
+        static_assert(2 * kClCells % 32 == 0 && 2 * kClCells <= kClThreads, "whole warps");
         __syncthreads();
         // interval l, one warp each: the exponents between those of its two thresholds, in a fixed order
         for (int l = warp; l < pl.L; l += kClThreads / 32) {
             const uint32_t T_up = l ? sh.q[l - 1].T : kKeyNone, T_dn = l < nq ? sh.q[l].T : 0u;
-            auto exponent = [&](uint32_t key) -> int { return (int)((Tr::kVec == 4 ? key : key << 16) >> 23); };
-            const int e_hi = T_up == kKeyNone ? 254 : exponent(T_up), e_lo = T_dn == kKeyNone ? 255 : exponent(T_dn);
+            const int e_hi = T_up == kKeyNone ? top_e : exponent(T_up), e_lo = T_dn == kKeyNone ? 255 : exponent(T_dn);
             double e = 0.0;
-            for (int x = e_hi - lane; x >= e_lo; x -= 32) e += ldexp(sh_cell[l + 254 - x], 2 * ((x ? x : 1) - 150));
+            for (int x = e_hi - lane; x >= e_lo; x -= 32) {
+                const double c = sh_cell[l + top_e - x];
+                if (c != 0.0) e += ldexp(c, 2 * ((x ? x : 1) - 150));
+            }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xFFFFFFFFu, e, o);
             if (lane == 0) sh.E[l] = e;
@@ -499,8 +592,10 @@ int configure_cluster_kernels(Workspace& ws) {
 int cluster_blocks(const Workspace& ws, int dtype, int64_t d, int M) {
     const int batches = emit_tiles_per_worker(d, dtype) * kEmitGroups;
     if (M > 32 || ws.cluster_most == 0) return 0;
-    int cl = 8;
-    if (batches > 8 * 32 && ws.cluster_most >= 16) cl = 16;  // more than 64 KB per block: twice the blocks
+    // The smallest cluster whose blocks have at most 32 batches (64 KB, 16 words per thread), and no more workers than fit
+    // the GPU at a time: a barrier and an exchange between more blocks take longer than the work that they share out.
+    int cl = 1;
+    while (cl < ws.cluster_most && (batches + cl - 1) / cl > 32) cl *= 2;
     return (batches + cl - 1) / cl <= (dtype == MLMC_BF16 ? kClBatchesBf16 : kClBatches) ? cl : 0;
 }
 

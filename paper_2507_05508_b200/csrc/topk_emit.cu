@@ -353,6 +353,48 @@ aggregate_topk_warps_kernel(const uint32_t* __restrict__ idx, const float* __res
     }
 }
 
+// The same average in one launch for short vectors: a block finds the edges of its warps' coordinates in every message
+// by itself (binary searches over whole messages, one edge of one worker per thread).
+__global__ void __launch_bounds__(kAggWarps * 32)
+aggregate_topk_direct_kernel(const uint32_t* __restrict__ idx, const float* __restrict__ val, const int64_t* count,
+                             const int32_t* level, int64_t capacity, int M, int64_t d, float* __restrict__ out) {
+    constexpr int kEdges = kAggWarps + 1;
+    __shared__ __align__(16) float acc_all[kAggTile];
+    extern __shared__ uint32_t sh_edge[];  // [M][kEdges]
+    pdl_enter();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint64_t tile0 = (uint64_t)blockIdx.x * kAggTile;
+    for (int i = threadIdx.x; i < M * kEdges; i += kAggWarps * 32) {
+        const int m = i / kEdges;
+        const uint64_t target = tile0 + (uint64_t)(i % kEdges) * kAggSub;
+        const uint32_t* a = idx + (int64_t)m * capacity;
+        uint32_t lo = 0, hi = level[m] < 0 ? 0u : (uint32_t)count[m];
+        while (lo < hi) {
+            const uint32_t mid = lo + ((hi - lo) >> 1);
+            if ((uint64_t)__ldg(&a[mid]) < target) lo = mid + 1; else hi = mid;
+        }
+        sh_edge[i] = lo;
+    }
+    float* acc = acc_all + warp * kAggSub;
+    const float inv_M = 1.0f / (float)M;
+#pragma unroll
+    for (int i = 0; i < kAggSub / 128; ++i) reinterpret_cast<float4*>(acc)[i * 32 + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+    __syncthreads();
+    const int64_t base = (int64_t)tile0 + (int64_t)warp * kAggSub;
+    for (int m = 0; m < M; ++m) {  // fixed worker order: reproducible fp32 sums
+        const uint32_t b0 = sh_edge[m * kEdges + warp], b1 = sh_edge[m * kEdges + warp + 1];
+        const uint32_t* a = idx + (int64_t)m * capacity;
+        const float* v = val + (int64_t)m * capacity;
+        for (uint32_t j = b0 + lane; j < b1; j += 32) {
+            const uint32_t off = __ldg(&a[j]) - (uint32_t)base;  // indices are unique within a worker
+            if (off < (uint32_t)kAggSub) acc[off] += __ldg(&v[j]);
+        }
+        __syncwarp();
+    }
+    for (int i = lane; i < kAggSub; i += 32)
+        if (base + i < d) out[base + i] = acc[i] * inv_M;
+}
+
 }  // namespace
 
 int configure_emit_kernels() {
@@ -401,6 +443,12 @@ void launch_emit(Workspace& ws, const void* g, int dtype, int64_t d, int M, int6
 
 void launch_aggregate_topk(Workspace& ws, const mlmc_topk_msgs& msgs, int M, int64_t d, float* out, cudaStream_t s) {
     const int ntiles = (int)((d + kAggTile - 1) / kAggTile);
+    if (M <= 32 && ntiles <= ws.sm_count * 4) {  // half a wave of blocks: one launch instead of two, a few us of searches
+        launch_kernel(ws, K_AGG_TOPK, aggregate_topk_direct_kernel, dim3(ntiles), kAggWarps * 32,
+                      (size_t)M * (kAggWarps + 1) * sizeof(uint32_t), s, msgs.idx, msgs.val, msgs.count, msgs.level, msgs.capacity, M, d,
+                      out);
+        return;
+    }
     const int64_t n_off = (int64_t)M * (ntiles + 1);
     launch_kernel(ws, K_AGG_OFFSETS, agg_offsets_kernel, dim3((unsigned)((n_off + 255) / 256)), 256, 0, s, msgs.idx, msgs.count,
                   msgs.level, msgs.capacity, M, ntiles, ws.agg_offsets);

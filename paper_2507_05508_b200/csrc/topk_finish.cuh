@@ -62,56 +62,56 @@ __device__ void fail_worker(const FinishPlan& pl, int m, EmitParams* out) {
 
 // The end of a selection, by one block per worker.  q: the worker's queries (in shared memory, complete).
 // Adaptive: E[l] = energy of the entries strictly between two thresholds (shared memory); the energy of the threshold
-// keys K is added from their counts, |ranks of K  intersect  (k_{l-1}, k_l]| * val(K)^2; Delta_l = sqrt(E_l);
-// p_l = Delta_l / sum Delta (Lemma 3.4); the level draw.  Then the header of the drawn band; `level` and `p_sel` are the
-// level drawn on the host and its probability where p is given.
-__device__ void finish_selection(const FinishPlan& pl, int m, int is_bf16, const Query* q, double* E, double* p_all,
+// keys is added from their counts: of the keys equal to T_{l-1} the n - r past rank k_{l-1}, of those equal to T_l the first
+// r; Delta_l = sqrt(E_l); p_l = Delta_l / sum Delta (Lemma 3.4); the level draw.  Then the header of the drawn band;
+// `level` and `p_sel` are the level drawn on the host and its probability where p is given.  A level per lane of warp 0.
+__device__ void finish_selection(const FinishPlan& pl, int m, int is_bf16, const Query* q, const double* E, double* p_all,
                                  double* delta_all, int level, double p_sel, EmitParams* out, int* status, int* worker_err) {
-    __shared__ double sh_p[kMaxLevels];
-    __shared__ double sh_sum;
-    const int L = pl.L;
+    if (threadIdx.x >= 32) return;
+    const int L = pl.L, l = threadIdx.x;
     if (pl.adaptive) {
-        const int l = threadIdx.x;
+        double delta = 0.0;
         if (l < L) {
-            double x2 = E[l];
-            const int64_t lo = l ? (int64_t)pl.k[l - 1] : 0, hi = (int64_t)pl.k[l];
-            uint32_t prev_T = kKeyNone;
-            for (int j = 0; j < L - 1; ++j) {
-                if (q[j].trivial) continue;
-                const uint32_t T = q[j].T;
-                if (T == prev_T) continue;  // thresholds descend: the same key as the query before is counted once
-                prev_T = T;
-                const int64_t c0 = q[j].c, c1 = c0 + (int64_t)q[j].n;
-                const int64_t ov = min(c1, hi) - max(c0, lo);
-                if (ov > 0) {
-                    const double x = (double)__uint_as_float(is_bf16 ? (T << 16) : T);
-                    x2 = fma((double)ov, x * x, x2);
-                }
+            const Query* up = (l > 0 && q[l - 1].trivial == 0u) ? &q[l - 1] : nullptr;
+            const Query* dn = (l < L - 1 && q[l].trivial == 0u) ? &q[l] : nullptr;
+            auto square = [&](uint32_t T) -> double {
+                const double x = (double)__uint_as_float(is_bf16 ? (T << 16) : T);
+                return x * x;
+            };
+            double e = E[l];
+            if (up && dn && up->T == dn->T) {
+                e = fma((double)(pl.k[l] - pl.k[l - 1]), square(dn->T), e);  // the whole band is ties
+            } else {
+                if (up) e = fma((double)(up->n - up->r), square(up->T), e);
+                if (dn) e = fma((double)dn->r, square(dn->T), e);
             }
-            E[l] = sqrt(x2);
+            delta = sqrt(e);
         }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double s = 0.0;
-            for (int i = 0; i < L; ++i) s += E[i];
-            sh_sum = s;
-        }
-        __syncthreads();
+        double total = delta;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xFFFFFFFFu, total, o);
+        const double p = (total > 0.0) ? delta / total : (l == 0 ? 1.0 : 0.0);
         if (l < L) {
-            const double s = sh_sum;
-            const double p = (s > 0.0) ? E[l] / s : (l == 0 ? 1.0 : 0.0);
-            sh_p[l] = p;
             p_all[m * kMaxLevels + l] = p;
-            delta_all[m * kMaxLevels + l] = E[l];
+            delta_all[m * kMaxLevels + l] = delta;
         }
-        __syncthreads();
-    }
-    if (threadIdx.x != 0 || !pl.want_emit) return;
-    if (pl.adaptive) {
-        level = draw_from_probs(sh_p, L, counter_uniform(pl.seed, pl.step, (uint64_t)m));
-        fill_emit(pl, m, level, sh_p[level], level ? &q[level - 1] : nullptr, level < L - 1 ? &q[level] : nullptr,
-                  level ? pl.k[level - 1] : 0u, pl.k[level], out, status, worker_err);
-    } else {
+        if (!pl.want_emit) return;
+        // l* = min{ l : u < cdf_l }; the last level with p > 0 has cdf 1
+        double cdf = p;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const double y = __shfl_up_sync(0xFFFFFFFFu, cdf, o);
+            if (l >= o) cdf += y;
+        }
+        const double u = counter_uniform(pl.seed, pl.step, (uint64_t)m);
+        const uint32_t positive = __ballot_sync(0xFFFFFFFFu, p > 0.0);  // never empty
+        const uint32_t below = __ballot_sync(0xFFFFFFFFu, p > 0.0 && u < cdf);
+        level = below ? __ffs(below) - 1 : 31 - __clz((int)positive);
+        p_sel = __shfl_sync(0xFFFFFFFFu, p, level);
+        if (l == 0)
+            fill_emit(pl, m, level, p_sel, level ? &q[level - 1] : nullptr, level < L - 1 ? &q[level] : nullptr,
+                      level ? pl.k[level - 1] : 0u, pl.k[level], out, status, worker_err);
+    } else if (l == 0 && pl.want_emit) {
         fill_emit(pl, m, level, p_sel, &q[0], &q[1], q[0].k, q[1].k, out, status, worker_err);
     }
 }
