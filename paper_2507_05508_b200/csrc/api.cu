@@ -359,7 +359,7 @@ int64_t mlmc_launch_count(const mlmc_ctx* ctx) { return ctx ? ctx->ws.launches :
 
 static const char* const kKernelNames[] = {
     "begin", "uniforms", "hist1", "resolve1", "sums_candidates", "cand_pass2", "cand_pass3", "band_header", "copy_probs", "emit",
-    "agg_offsets", "aggregate_topk", "absmax", "bit_stats", "bit_pack", "aggregate_bitwise", "tile_list", "band_count", "bit_pack_wide",
+    "agg_offsets", "aggregate_topk", "absmax", "bit_stats", "bit_pack", "aggregate_bitwise", "tile_list", "band_count",
     "float_pack", "aggregate_floatbits", "rtn_stats", "rtn_emit", "aggregate_dense", "segment_resolve",
     "segment_sweep", "segment_buckets", "segment_norms", "segment_draw", "cluster_topk"};
 static_assert(sizeof(kKernelNames) / sizeof(kKernelNames[0]) == K_COUNT, "a name for every kernel id");

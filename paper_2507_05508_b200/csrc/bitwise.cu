@@ -7,7 +7,7 @@
 //   f_l = (q >> (B - b_l)) & (2^{w_l} - 1),  w_l = b_l - b_{l-1},  worth  sign f_l 2^{-b_l} gmax,
 // sent as one sign plane and w_l magnitude planes.  Adaptive probabilities (Lemma 3.4) use the exact
 // integer field energies S_l = sum_i f_l^2:  Delta_l = gmax 2^{-b_l} sqrt(S_l).
-#include "common.cuh"
+#include "bitplanes.cuh"
 
 namespace mlmc {
 
@@ -24,32 +24,40 @@ struct BitSchedule {
     int bits[kMaxLevels];       // b_l
 };
 
-// The code q = min(trunc(fl32(|g| / gmax) * 2^B), 2^B - 1) with the IEEE-rounded fp32 quotient, for a fixed
-// divisor.  The quotient is formed in fp64 as |g| * (1 / gmax) and rounded to fp32 once: a quotient of two
-// 24-bit significands is never closer than 2^-49 (relative) to the midpoint of two fp32 numbers, the fp64
-// product is within 2^-52 of it, so this rounding is the same as that of the fp32 division.
+// The code of an entry at b bits, min(trunc(e 2^b), 2^b - 1) with the IEEE-rounded fp32 quotient e = fl32(|g| / gmax).  (The
+// top bits of a longer code are the shorter code: both truncate the same e.)
+// The divisor is fixed, so the quotient comes from its correctly rounded reciprocal by two correction steps (Markstein,
+// "Computation of elementary functions on the IBM RISC System/6000 processor", 1990: with the reciprocal correctly rounded
+// and a quotient within one ulp, one step of remainder and correction rounds like the division).  The truncation is the
+// addition of 2^23 with rounding toward zero.  Seven fp32 operations; the fp64 product and conversions used before took
+// two slots of the conversion unit.  The remainders must not underflow and the reciprocal must be normal; outside
+// 2^-60 <= gmax <= 2^100 the entry is divided.
 struct Quantiser {
-    double inv_scaled;  // fl64(1 / gmax) * 2^B
-    uint32_t qmax;      // 2^B - 1
-    bool widen_by_bits;  // gmax >= 2^-100: an fp32 operand below the normal range cannot reach q = 1, so its
-                         // fp64 image may be built from the bit pattern as if it were normal
-    __device__ __forceinline__ Quantiser(float g, int B) {
-        inv_scaled = g > 0.0f ? ldexp(1.0 / (double)g, B) : 0.0;
-        qmax = (1u << B) - 1u;
-        widen_by_bits = g >= 0x1.0p-100f;
+    float gmax, inv;
+    bool steps;
+    __device__ __forceinline__ explicit Quantiser(float g) {
+        gmax = g > 0.0f ? g : 1.0f;
+        inv = __frcp_rn(gmax);
+        steps = gmax >= 0x1.0p-60f && gmax <= 0x1.0p100f;
     }
-    __device__ __forceinline__ uint32_t code(uint32_t mag_bits /* sign bit cleared */) const {
-        double x;
-        if (widen_by_bits)
-            x = __hiloint2double((int)((mag_bits >> 3) + 0x38000000u), (int)(mag_bits << 29));
-        else
-            x = (double)__uint_as_float(mag_bits);
-        // fl32(|g| / gmax) * 2^B in one rounding: scaling by a power of two commutes with both roundings (a
-        // quotient so small that its fp32 image would be subnormal has the code 0 either way)
-        const float scaled = (float)(x * inv_scaled);
-        return min(__float2uint_rz(scaled), qmax);  // truncation: the lower bits are discarded
+    __device__ __forceinline__ uint32_t code(float mag /* |g| */, float scale /* 2^b, b <= 23 */) const {
+        float e;
+        if (steps) {
+            e = __fmul_rn(mag, inv);
+            e = __fmaf_rn(__fmaf_rn(-e, gmax, mag), inv, e);
+            e = __fmaf_rn(__fmaf_rn(-e, gmax, mag), inv, e);
+        } else {
+            e = __fdiv_rn(mag, gmax);
+        }
+        // e = 1 has no b-bit fraction: the largest e below it has the code 2^b - 1
+        return __float_as_uint(__fmaf_rz(fminf(e, 0x1.fffffep-1f), scale, 8388608.0f)) - 0x4B000000u;
     }
 };
+
+// An entry below gmax 2^-b (1 - 2^-20) has fl32(|g| / gmax) < 2^-b: its code at b bits is 0.
+__device__ __forceinline__ int zero_code_below(float gmax, int b) {
+    return gmax > 0.0f ? __float_as_int(gmax * ldexpf(1.0f - 0x1.0p-20f, -b)) : 0x7FFFFFFF;
+}
 
 // ---- per-worker max |g| as an integer max over magnitude keys; flags NaN / Inf.  With given probabilities (draw != 0)
 // the worker's last block also draws the level and writes the message header.
@@ -119,8 +127,59 @@ absmax_kernel(const T* __restrict__ g, int64_t d, int64_t ld, uint32_t* gmax_bit
 // Acc = uint32_t when every field is at most 8 bits wide and a thread sees fewer than 2^16 entries (f^2 < 2^16,
 // so the sum fits 32 bits), else unsigned long long.  Fields come from the prefix codes P_l = q >> (B - b_l):
 // f_l = P_l - (P_{l-1} << w_l), one shift and one multiply-add per level.
+// A warp takes its entries level by level, kBitHeld per lane, from the first level at which the largest of them has a code
+// above 0 (the coarse levels of a gradient with per-layer scales are nearly all zero).  8 x 124M fp32 entries, six levels:
+// 1.0 ms with every entry taken through every level and the fp64 quotient (issue and the conversion unit).
+constexpr int kBitHeld = 8;
+
 template <typename T, int LMAX, typename Acc>
-__global__ void __launch_bounds__(kSweepThreads)
+__device__ __forceinline__ void take_fields(const float (&v)[kBitHeld], const Quantiser& qz, float scale, const int (&zero_below)[LMAX],
+                                            const BitSchedule& sc, Acc (&acc)[LMAX]) {
+    int mx = 0;
+#pragma unroll
+    for (int e = 0; e < kBitHeld; ++e) mx = max(mx, __float_as_int(v[e]) & 0x7FFFFFFF);
+    mx = __reduce_max_sync(0xFFFFFFFFu, mx);
+    if (mx < zero_below[LMAX - 1]) return;  // the thresholds fall with the level; those past L repeat the last
+    uint32_t q[kBitHeld], prev[kBitHeld];
+#pragma unroll
+    for (int e = 0; e < kBitHeld; ++e) {
+        q[e] = qz.code(fabsf(v[e]), scale);
+        prev[e] = 0u;
+    }
+#pragma unroll
+    for (int l = 0; l < LMAX; ++l) {
+        if (l >= sc.L) break;
+        if (mx < zero_below[l]) continue;
+        const int shift = sc.shift[l];
+        const uint32_t neg_pow = 0u - (1u << sc.width[l]);
+#pragma unroll
+        for (int e = 0; e < kBitHeld; ++e) {
+            const uint32_t P = q[e] >> shift, f = prev[e] * neg_pow + P;
+            acc[l] += (Acc)f * f;
+            prev[e] = P;
+        }
+    }
+}
+
+template <typename T>
+__device__ __forceinline__ void expand_vectors(const uint4* q, float (&v)[kBitHeld]) {  // kBitHeld entries
+#pragma unroll
+    for (int j = 0; j < kBitHeld / ElemTraits<T>::kVec; ++j) {
+        const uint32_t w[4] = {q[j].x, q[j].y, q[j].z, q[j].w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if constexpr (ElemTraits<T>::kVec == 4) {
+                v[4 * j + i] = __uint_as_float(w[i]);
+            } else {
+                v[8 * j + 2 * i] = __uint_as_float(w[i] << 16);
+                v[8 * j + 2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
+            }
+        }
+    }
+}
+
+template <typename T, int LMAX, typename Acc>
+__global__ void __launch_bounds__(kSweepThreads, LMAX <= 8 ? 2 : 1)
 bit_stats_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* gmax_bits, BitSchedule sc,
                  unsigned long long* S_partial, int stat_ctas, uint32_t* done, DrawPlan pl, int* status, int* worker_err) {
     using Tr = ElemTraits<T>;
@@ -130,50 +189,49 @@ bit_stats_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t*
     const int m = blockIdx.y;
     if (worker_err[m]) return;
     const float gmax = __uint_as_float(gmax_bits[m]);
-    const Quantiser qz(gmax, sc.B);
+    const Quantiser qz(gmax);
+    const float scale = (float)(1u << sc.B);
     Acc acc[LMAX];
-    int sh[LMAX];
-    uint32_t neg_pow[LMAX];
+    int zero_below[LMAX];
 #pragma unroll
-    for (int l = 0; l < LMAX; ++l) {  // the schedule in registers; levels past L get shift 0 and width 0: their field is q - q = 0
+    for (int l = 0; l < LMAX; ++l) {
         acc[l] = 0;
-        sh[l] = (l < sc.L) ? sc.shift[l] : 0;
-        neg_pow[l] = 0u - (1u << ((l < sc.L) ? sc.width[l] : 0));
+        zero_below[l] = zero_code_below(gmax, sc.bits[min(l, sc.L - 1)]);
     }
     if (gmax > 0.0f) {
         const T* row = g + (int64_t)m * ld;
-        int64_t v0, v1;
-        block_vector_range(d, Tr::kVec, blockIdx.x, gridDim.x, &v0, &v1);
-        auto take = [&](uint32_t bits) {
-            const uint32_t q = qz.code(__float_as_uint(Tr::value(bits)) & 0x7FFFFFFFu);
-            uint32_t prev = 0;  // P_{l-1}
+        constexpr int kVecs = kBitHeld / Tr::kVec;  // 16-byte vectors per lane and trip; the next trip's are in flight
+        constexpr int kTrip = kSweepThreads * kVecs;
+        const int64_t trips = d / Tr::kVec / kTrip;
+        uint4 nxt[kVecs];
+        auto load = [&](int64_t trip) {
+            if (trip >= trips) return;
 #pragma unroll
-            for (int l = 0; l < LMAX; ++l) {
-                const uint32_t P = q >> sh[l];
-                const uint32_t f = prev * neg_pow[l] + P;
-                acc[l] += (Acc)f * f;
-                prev = P;
-            }
+            for (int j = 0; j < kVecs; ++j)
+                nxt[j] = __ldg(reinterpret_cast<const uint4*>(row) + trip * kTrip + j * kSweepThreads + threadIdx.x);
         };
-        // two 16-byte loads per thread are in flight before either is used
-        constexpr int kBatch = 2;
-        const int64_t full_end = min(v1, d / Tr::kVec);  // vectors wholly inside the row
-        int64_t v = v0 + threadIdx.x;
-        for (; v + (int64_t)(kBatch - 1) * blockDim.x < full_end; v += (int64_t)kBatch * blockDim.x) {
-            uint4 qv[kBatch];
+        load(blockIdx.x);
+        for (int64_t trip = blockIdx.x; trip < trips; trip += gridDim.x) {
+            float v[kBitHeld];
+            expand_vectors<T>(nxt, v);
+            load(trip + gridDim.x);
+            take_fields<T, LMAX, Acc>(v, qz, scale, zero_below, sc, acc);
+        }
+        if (blockIdx.x == gridDim.x - 1) {  // the rest of the row; entries past it read as 0, which adds nothing
+            for (int64_t i0 = trips * kTrip * Tr::kVec; i0 < d; i0 += (int64_t)kSweepThreads * kBitHeld) {
+                float v[kBitHeld];
 #pragma unroll
-            for (int j = 0; j < kBatch; ++j) qv[j] = __ldg(reinterpret_cast<const uint4*>(row) + v + (int64_t)j * blockDim.x);
-#pragma unroll
-            for (int j = 0; j < kBatch; ++j) {
-                if constexpr (Tr::kVec == 4) {
-                    take(qv[j].x); take(qv[j].y); take(qv[j].z); take(qv[j].w);
-                } else {
-                    take(qv[j].x & 0xFFFFu); take(qv[j].x >> 16); take(qv[j].y & 0xFFFFu); take(qv[j].y >> 16);
-                    take(qv[j].z & 0xFFFFu); take(qv[j].z >> 16); take(qv[j].w & 0xFFFFu); take(qv[j].w >> 16);
+                for (int e = 0; e < kBitHeld; ++e) {
+                    const int64_t i = i0 + e * kSweepThreads + threadIdx.x;
+                    v[e] = 0.0f;
+                    if (i < d) {
+                        if constexpr (Tr::kVec == 4) v[e] = reinterpret_cast<const float*>(row)[i];
+                        else v[e] = __uint_as_float((uint32_t)reinterpret_cast<const uint16_t*>(row)[i] << 16);
+                    }
                 }
+                take_fields<T, LMAX, Acc>(v, qz, scale, zero_below, sc, acc);
             }
         }
-        for (; v < v1; v += blockDim.x) for_each_in_vector<T>(row, v, d, [&](int64_t, uint32_t bits) { take(bits); });
     }
 #pragma unroll
     for (int l = 0; l < LMAX; ++l) {
@@ -210,132 +268,91 @@ bit_stats_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t*
     finish_levels(pl, m, sh_delta, sh_p, gmax, status, worker_err);
 }
 
-// ---- pack: every warp turns 1024 consecutive entries into 32 words of each plane.
-// The entries of a group are staged in a two-slot shared-memory ring private to the warp: the next group's
-// copy (cp.async) is in flight while the current group is coded and packed.
-// WIDE = false serves the workers whose drawn level has a field of at most 8 bits, WIDE = true the others (each
-// instance leaves the other's workers alone): the narrow path keeps no per-row state in registers, which the wide
-// path's 32 codes per lane would otherwise force on it.
-template <typename T, bool WIDE>
-__global__ void __launch_bounds__(kBitThreads, WIDE ? 2 : 3)
+// ---- pack: a warp turns 1024 consecutive entries into 32 words of each plane, a lane owning 32 consecutive entries (one
+// word per plane).  The entries come through a ring of two shared-memory slots per warp: the next group's copy is in
+// flight while the current group is coded.  A plane's word is collected by one shift and one funnel shift per entry, from
+// 6 planes on by one bit transpose for all of them.  A group whose largest entry has the code 0 at the drawn level's bits is
+// not coded: its magnitude planes are zero.
+// Bound by HBM.  Rows of 32 entries across the lanes with a ballot each took 1.04 ms for 8 x 124M fp32 entries.
+template <typename T>
+__device__ __forceinline__ void pack_group(const uint32_t* slot, const Quantiser& qz, float scale, int zero_below, int w, int64_t word,
+                                           int64_t words, uint32_t* __restrict__ out) {
+    const int lane = threadIdx.x & 31;
+    const bool live = word < words;
+    float x[32];
+#pragma unroll
+    for (int c = 0; c < kGroupChunks<T>; ++c) {
+        const uint4 q = *reinterpret_cast<const uint4*>(slot + group_place<T>(lane, c));
+        const uint32_t u[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if constexpr (sizeof(T) == 4) {
+                x[4 * c + i] = __uint_as_float(u[i]);
+            } else {
+                x[8 * c + 2 * i] = __uint_as_float(u[i] << 16);
+                x[8 * c + 2 * i + 1] = __uint_as_float(u[i] & 0xFFFF0000u);
+            }
+        }
+    }
+    uint32_t sign_w = 0;
+    float mx = 0.0f;
+#pragma unroll
+    for (int t = 31; t >= 0; --t) {
+        sign_w = __funnelshift_l(__float_as_uint(x[t]), sign_w, 1);
+        mx = fmaxf(mx, fabsf(x[t]));
+    }
+    if (live) out[word] = sign_w;
+    if (!__any_sync(0xFFFFFFFFu, __float_as_int(mx) >= zero_below)) {
+        if (live)
+            for (int j = 1; j <= w; ++j) out[(int64_t)j * words + word] = 0u;
+        return;
+    }
+    uint32_t q[32];
+#pragma unroll
+    for (int t = 0; t < 32; ++t) q[t] = qz.code(fabsf(x[t]), scale);
+    if (w < 6) {
+        for (int j = 1; j <= w; ++j) {
+            const int up = 31 - (w - j);
+            uint32_t pw = 0;
+#pragma unroll
+            for (int t = 31; t >= 0; --t) pw = __funnelshift_l(q[t] << up, pw, 1);
+            if (live) out[(int64_t)j * words + word] = pw;
+        }
+    } else {
+        transpose_bits(q);
+#pragma unroll
+        for (int bit = 22; bit >= 0; --bit)
+            if (live && bit < w) out[(int64_t)(w - bit) * words + word] = q[bit];
+    }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kBitThreads, 3)
 bit_pack_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* gmax_bits, BitSchedule sc,
                 const int32_t* bit_level, uint32_t* __restrict__ planes, int w_max, int64_t words) {
+    extern __shared__ __align__(16) uint32_t sh_ring[];  // [warps][2][kGroupSlot]
     pdl_enter();
-    using Tr = ElemTraits<T>;
-    constexpr int kGroup = 1024;
-    constexpr int kGroupBytes = kGroup * (int)sizeof(T);
-    extern __shared__ __align__(16) uint8_t sh_pack[];  // [warps][2][kGroupBytes], then [warps][1024] field bytes
     const int m = blockIdx.y;
     const int level = bit_level[m];
     if (level < 0) return;
-    if ((sc.width[level] > 8) != WIDE) return;  // the other instance's worker
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int warps_per_block = kBitThreads / 32;
-    const int64_t ngroups = (words + 31) / 32;  // groups of 32 words = 1024 entries
+    const int64_t ngroups = (words + 31) / 32;
     const float gmax = __uint_as_float(gmax_bits[m]);
-    const Quantiser qz(gmax, sc.B);
-    const int shift = sc.shift[level];
-    const uint32_t mask = sc.mask[level];
-    const int w = sc.width[level];
+    const Quantiser qz(gmax);
+    const int w = sc.width[level], bits = sc.bits[level];
+    const int zero_below = zero_code_below(gmax, bits);
+    const float scale = (float)(1u << bits);
     const T* row = g + (int64_t)m * ld;
     uint32_t* out = planes + (int64_t)m * (1 + w_max) * words;
-    uint8_t* ring = sh_pack + warp * 2 * kGroupBytes;
-    uint8_t* bytes = sh_pack + warps_per_block * 2 * kGroupBytes + warp * 1024;  // 32 rows x 32 field bytes
-    auto fetch = [&](int64_t grp, int stage) {  // one commit per call
-        if (grp < ngroups) {
-            const int64_t e0 = grp * kGroup;
-            uint8_t* dst = ring + stage * kGroupBytes;
-            if (e0 + kGroup <= d) {
-                const uint8_t* src = reinterpret_cast<const uint8_t*>(row + e0);
-#pragma unroll
-                for (int c = lane; c < kGroupBytes / 16; c += 32) cp_async_16(dst + c * 16, src + c * 16);
-            } else {  // ragged last group: entries past d read as +0
-                for (int i = lane; i < kGroup; i += 32) {
-                    if constexpr (Tr::kVec == 4)
-                        reinterpret_cast<uint32_t*>(dst)[i] = (e0 + i < d) ? reinterpret_cast<const uint32_t*>(row)[e0 + i] : 0u;
-                    else
-                        reinterpret_cast<uint16_t*>(dst)[i] = (e0 + i < d) ? reinterpret_cast<const uint16_t*>(row)[e0 + i] : (uint16_t)0;
-                }
-            }
-        }
-        cp_async_commit();
-    };
-    const int64_t stride = (int64_t)gridDim.x * warps_per_block;
-    int64_t grp = (int64_t)blockIdx.x * warps_per_block + warp;
-    // An entry below gmax 2^-b_l (1 - 2^-20) has fl32(|g| / gmax) < 2^-b_l, so its top b_l code bits and with them
-    // the field of level l are zero.  A row of 32 entries that are all below that bound is not coded at all: in
-    // a gradient with per-layer scales and a few outliers this is most rows of the high levels.
-    const uint32_t zero_below = (gmax > 0.0f) ? __float_as_uint(gmax * ldexpf(1.0f - 0x1.0p-20f, -sc.bits[level])) : 0x7FFFFFFFu;
-    fetch(grp, 0);
+    uint32_t* ring = sh_ring + warp * 2 * kGroupSlot<T>;
+    const int64_t stride = (int64_t)gridDim.x * (kBitThreads / 32);
+    int64_t grp = (int64_t)blockIdx.x * (kBitThreads / 32) + warp;
+    fetch_group<T>(row, d, grp, ngroups, ring);
     for (int it = 0; grp < ngroups; grp += stride, ++it) {
-        fetch(grp + stride, (it + 1) & 1);
+        fetch_group<T>(row, d, grp + stride, ngroups, ring + ((it + 1) & 1) * kGroupSlot<T>);
         cp_async_wait<1>();  // this group has landed (the next one may still be in flight)
         __syncwarp();
-        const uint8_t* buf = ring + (it & 1) * kGroupBytes;
-        const int64_t word = grp * 32 + lane;
-        auto entry_bits = [&](int s) -> uint32_t {
-            uint32_t bits;
-            if constexpr (Tr::kVec == 4)
-                bits = reinterpret_cast<const uint32_t*>(buf)[s * 32 + lane];
-            else
-                bits = reinterpret_cast<const uint16_t*>(buf)[s * 32 + lane];
-            return __float_as_uint(Tr::value(bits));
-        };
-        if constexpr (!WIDE) {
-            // Fields of at most 8 bits go through a byte matrix in shared memory: lane L writes the field of each of
-            // its 32 rows, then lane r gathers bit b of the 32 bytes of row r, four bytes per multiply
-            // (((x >> b) & 0x01010101) * 0x01020408 puts the four bits side by side in bits 24..27).  This costs
-            // a quarter of one ballot per row and plane.  The sign plane takes one ballot per row.
-            uint32_t sign_w = 0;
-            bool coded = false;  // warp-uniform: some row of the group was coded
-#pragma unroll
-            for (int s = 0; s < 32; ++s) {
-                const uint32_t xb = entry_bits(s);
-                const uint32_t bs = __ballot_sync(0xFFFFFFFFu, (int)xb < 0);
-                if (lane == s) sign_w = bs;
-                uint32_t f = 0;
-                if (__any_sync(0xFFFFFFFFu, (xb & 0x7FFFFFFFu) >= zero_below)) {
-                    f = (qz.code(xb & 0x7FFFFFFFu) >> shift) & mask;
-                    coded = true;
-                }
-                bytes[s * 32 + lane] = (uint8_t)f;
-            }
-            __syncwarp();
-            if (word < words) out[word] = sign_w;
-            if (coded) {
-                const uint4 lo = reinterpret_cast<const uint4*>(bytes + lane * 32)[0];
-                const uint4 hi = reinterpret_cast<const uint4*>(bytes + lane * 32)[1];
-                const uint32_t x[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
-                for (int j = 1; j <= w; ++j) {
-                    const int bit = w - j;
-                    uint32_t pw = 0;
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) pw |= ((((x[c] >> bit) & 0x01010101u) * 0x01020408u) >> 24 & 0xFu) << (4 * c);
-                    if (word < words) out[(int64_t)j * words + word] = pw;
-                }
-            } else if (word < words) {  // every field of the group is zero
-                for (int j = 1; j <= w; ++j) out[(int64_t)j * words + word] = 0u;
-            }
-        } else {
-            uint32_t code[32];  // bit 31 = sign, low bits = field
-#pragma unroll
-            for (int s = 0; s < 32; ++s) {
-                const uint32_t xb = entry_bits(s);
-                code[s] = xb & 0x80000000u;
-                if (__any_sync(0xFFFFFFFFu, (xb & 0x7FFFFFFFu) >= zero_below))
-                    code[s] |= (qz.code(xb & 0x7FFFFFFFu) >> shift) & mask;
-            }
-            for (int j = 0; j <= w; ++j) {
-                const int bit = (j == 0) ? 31 : (w - j);
-                uint32_t mine = 0;
-#pragma unroll
-                for (int s = 0; s < 32; ++s) {
-                    const uint32_t b = __ballot_sync(0xFFFFFFFFu, (code[s] >> bit) & 1u);
-                    if (lane == s) mine = b;
-                }
-                if (word < words) out[(int64_t)j * words + word] = mine;
-            }
-        }
+        pack_group<T>(ring + (it & 1) * kGroupSlot<T>, qz, scale, zero_below, w, grp * 32 + lane, words, out);
         __syncwarp();  // everyone is done with this slot before the copy after next lands in it
     }
     cp_async_wait<0>();
@@ -387,32 +404,35 @@ aggregate_bitwise_kernel(const uint32_t* __restrict__ planes, const float* gmax,
                         acc[t] += __uint_as_float((ub & on) ^ (((sgn >> t) & 1u) << 31));
                     }
                 }
-            } else if (w <= 8) {
-                // fields of at most 8 bits: each plane word is spread into the 32 field bytes, four bits per
-                // multiply ((nibble * 0x00204081) & 0x01010101 puts bit i of the nibble at bit 0 of byte i)
+            } else if (w <= 8 && fabsf(unit) < 0x1p100f) {
+                // fields of at most 8 bits: one bit transpose of 8 x 8 blocks turns the plane words (bit k of every field
+                // in word k) into field bytes, four entries per word; a byte below the bits of 2^23 is 2^23 + f, and
+                // (2^23 + f) unit - 2^23 unit is f unit rounded once
                 const uint32_t* pm = planes + (int64_t)m * (1 + w_max) * words;
-                uint32_t pw[8], any = pw1;
-                pw[0] = pw1;
+                uint32_t fb[8], any = pw1;
 #pragma unroll
-                for (int j = 2; j <= 8; ++j) {
-                    pw[j - 1] = (j <= w && word < words) ? pm[(int64_t)j * words + word] : 0u;
-                    any |= pw[j - 1];
+                for (int k = 0; k < 8; ++k) {  // bit k of the fields: plane w - k
+                    fb[k] = (k == w - 1) ? pw1 : (k < w && word < words) ? pm[(int64_t)(w - k) * words + word] : 0u;
+                    any |= fb[k];
                 }
                 if (any != 0u) {
-                    uint32_t fb[8] = {};
 #pragma unroll
-                    for (int j = 1; j <= 8; ++j) {
-                        if (j <= w) {
+                    for (int j = 4; j > 0; j >>= 1) {
+                        const uint32_t mask = j == 4 ? 0x0F0F0F0Fu : j == 2 ? 0x33333333u : 0x55555555u;
 #pragma unroll
-                            for (int c = 0; c < 8; ++c)
-                                fb[c] |= ((((pw[j - 1] >> (4 * c)) & 0xFu) * 0x00204081u) & 0x01010101u) << (w - j);
+                        for (int k = 0; k < 8; ++k) {
+                            if (k & j) continue;
+                            const uint32_t x = ((fb[k] >> j) ^ fb[k + j]) & mask;
+                            fb[k + j] ^= x;
+                            fb[k] ^= x << j;
                         }
                     }
+                    const float offset = -8388608.0f * unit;
 #pragma unroll
                     for (int t = 0; t < 32; ++t) {
-                        const uint32_t f = (fb[t >> 2] >> (8 * (t & 3))) & 0xFFu;
-                        const float ff = __uint_as_float(0x4B000000u | f) - 8388608.0f;  // exact integer-to-float through 2^23
-                        acc[t] += __uint_as_float(__float_as_uint(ff * unit) ^ (((sgn >> t) & 1u) << 31));
+                        const float ff = __uint_as_float(__byte_perm(fb[t & 7], 0x4B000000u, 0x7650u + (uint32_t)(t >> 3)));
+                        const float v = fmaf(ff, unit, offset);
+                        acc[t] += __uint_as_float(__float_as_uint(v) ^ ((sgn << (31 - t)) & 0x80000000u));
                     }
                 }
             } else {
@@ -469,14 +489,14 @@ int bit_blocks(const Workspace& ws, int64_t d, int vec, int M, int waves) {
     return (int)(nb < 1 ? 1 : nb);
 }
 
+size_t bit_pack_smem(size_t elem) { return (kBitThreads / 32) * 2 * 1024 * elem; }
+
 }  // namespace
 
 int configure_bit_kernels() {
-    const int smem = (kBitThreads / 32) * (2 * 1024 * 4 + 1024);
-    if (cudaFuncSetAttribute(bit_pack_kernel<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-        cudaFuncSetAttribute(bit_pack_kernel<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
-        return MLMC_ERR_CUDA;
-    return MLMC_OK;
+    const bool ok = cudaFuncSetAttribute(bit_pack_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)bit_pack_smem(4)) == cudaSuccess;
+    return ok ? MLMC_OK : MLMC_ERR_CUDA;
 }
 
 DrawPlan bit_draw_plan(Workspace& ws, const int32_t* b, int L, uint64_t seed, uint64_t step, const mlmc_bit_msgs* out) {
@@ -523,9 +543,8 @@ void launch_bit_stats(Workspace& ws, const void* g, int dtype, int64_t d, int M,
     int nb = bit_blocks(ws, d, dtype == MLMC_BF16 ? 8 : 4, M, 4);
     if (nb > ws.stat_ctas) nb = ws.stat_ctas;
     // 32-bit sums are exact while f^2 < 2^16 and a thread adds fewer than 2^16 of them
-    const int vec = dtype == MLMC_BF16 ? 8 : 4;
-    const int64_t vec_per_block = ((d + vec - 1) / vec + nb - 1) / nb;
-    const int64_t per_thread = ((vec_per_block + kSweepThreads - 1) / kSweepThreads + 1) * vec;
+    const int64_t trips = d / (kSweepThreads * kBitHeld);
+    const int64_t per_thread = ((trips + nb - 1) / nb + 2) * kBitHeld;
     int w_top = 0;
     for (int l = 0; l < L; ++l) w_top = sc.width[l] > w_top ? sc.width[l] : w_top;
     const bool narrow = w_top <= 8 && per_thread < 65536;
@@ -544,26 +563,11 @@ static void launch_bit_pack_t(Workspace& ws, const T* g, int64_t d, int M, int64
     const int64_t words = (d + 31) / 32;
     const int64_t ngroups = (words + 31) / 32;
     const int64_t by_work = (ngroups + (kBitThreads / 32) - 1) / (kBitThreads / 32);
-    const size_t smem = (kBitThreads / 32) * (2 * 1024 * sizeof(T) + 1024);
-    int w_top = 0, w_low = 64;
-    for (int l = 0; l < sc.L; ++l) {
-        w_top = sc.width[l] > w_top ? sc.width[l] : w_top;
-        w_low = sc.width[l] < w_low ? sc.width[l] : w_low;
-    }
-    if (w_low <= 8) {  // some level has a field of at most 8 bits
-        int64_t nb = ((int64_t)ws.sm_count * 3) / M;  // persistent: three resident blocks per SM, rounded down
-        if (nb > by_work) nb = by_work;
-        if (nb < 1) nb = 1;
-        launch_kernel(ws, K_BIT_PACK, bit_pack_kernel<T, false>, dim3((unsigned)nb, M), kBitThreads, smem, s, g, d, ld,
-                      ws.gmax_bits, sc, ws.bit_level, out.planes, out.w_max, words);
-    }
-    if (w_top > 8) {  // some level has a wider field
-        int64_t nb = ((int64_t)ws.sm_count * 2) / M;  // two resident blocks per SM, rounded down
-        if (nb > by_work) nb = by_work;
-        if (nb < 1) nb = 1;
-        launch_kernel(ws, K_BIT_PACK_WIDE, bit_pack_kernel<T, true>, dim3((unsigned)nb, M), kBitThreads, smem, s, g, d, ld,
-                      ws.gmax_bits, sc, ws.bit_level, out.planes, out.w_max, words);
-    }
+    int64_t nb = ((int64_t)ws.sm_count * 3) / M;  // persistent: three resident blocks per SM, rounded down
+    if (nb > by_work) nb = by_work;
+    if (nb < 1) nb = 1;
+    launch_kernel(ws, K_BIT_PACK, bit_pack_kernel<T>, dim3((unsigned)nb, M), kBitThreads, bit_pack_smem(sizeof(T)), s, g, d, ld,
+                  ws.gmax_bits, sc, ws.bit_level, out.planes, out.w_max, words);
 }
 
 void launch_bit_pack(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* b, int L,

@@ -58,7 +58,7 @@ struct EmitParams {
 // Kernel identifiers for launch accounting and per-kernel timing.
 enum KernelId {
     K_BEGIN = 0, K_UNIFORMS, K_HIST1, K_RESOLVE1, K_SUMS_CAND, K_CAND2, K_CAND3, K_BAND_HEADER, K_COPY_PROBS, K_EMIT, K_AGG_OFFSETS,
-    K_AGG_TOPK, K_ABSMAX, K_BIT_STATS, K_BIT_PACK, K_AGG_BIT, K_TILE_LIST, K_BAND_COUNT, K_BIT_PACK_WIDE, K_FLOAT_PACK, K_AGG_FLOAT,
+    K_AGG_TOPK, K_ABSMAX, K_BIT_STATS, K_BIT_PACK, K_AGG_BIT, K_TILE_LIST, K_BAND_COUNT, K_FLOAT_PACK, K_AGG_FLOAT,
     K_RTN_STATS, K_RTN_EMIT, K_AGG_DENSE, K_SEG_RESOLVE, K_SEG_SWEEP, K_SEG_BUCKETS, K_SEG_NORMS, K_SEG_DRAW, K_CLUSTER_TOPK, K_COUNT
 };
 
@@ -409,7 +409,7 @@ struct LaunchScope {
 inline bool is_sweep(int id) {
     switch (id) {
         case K_HIST1: case K_SUMS_CAND: case K_BAND_COUNT: case K_EMIT: case K_AGG_TOPK: case K_ABSMAX: case K_BIT_STATS:
-        case K_BIT_PACK: case K_BIT_PACK_WIDE: case K_AGG_BIT: case K_FLOAT_PACK: case K_AGG_FLOAT: case K_RTN_STATS:
+        case K_BIT_PACK: case K_AGG_BIT: case K_FLOAT_PACK: case K_AGG_FLOAT: case K_RTN_STATS:
         case K_RTN_EMIT: case K_AGG_DENSE: case K_SEG_SWEEP:
             return true;
         default:

@@ -5,7 +5,7 @@
 // and exponent are sent with every message (App. B counts 1 + exponent + 1 bits per entry), and they are the base
 // g^0 = sign 2^(E - bias) of the estimate g^0 + (1/p^l)(C^l - C^{l-1}).  The level draw does not depend on the data
 // (App. B's lemma gives fixed probabilities), so one sweep over the gradient writes the whole message.
-#include "common.cuh"
+#include "bitplanes.cuh"
 
 namespace mlmc {
 
@@ -27,34 +27,6 @@ MantissaSchedule make_mantissa_schedule(const int32_t* mb, int L) {
         sc.hi[l] = mb[l];
     }
     return sc;
-}
-
-// 32 x 32 bit transpose: on return bit t of x[b] is bit b of the former x[t].
-__device__ __forceinline__ void transpose_bits(uint32_t (&x)[32]) {
-#pragma unroll
-    for (int k = 0; k < 16; ++k) {
-        const uint32_t a = x[k], b = x[k + 16];
-        x[k] = __byte_perm(a, b, 0x5410);
-        x[k + 16] = __byte_perm(a, b, 0x7632);
-    }
-#pragma unroll
-    for (int k = 0; k < 32; ++k) {
-        if (k & 8) continue;
-        const uint32_t a = x[k], b = x[k + 8];
-        x[k] = __byte_perm(a, b, 0x6240);
-        x[k + 8] = __byte_perm(a, b, 0x7351);
-    }
-#pragma unroll
-    for (int j = 4; j > 0; j >>= 1) {
-        const uint32_t mask = j == 4 ? 0x0F0F0F0Fu : j == 2 ? 0x33333333u : 0x55555555u;
-#pragma unroll
-        for (int k = 0; k < 32; ++k) {
-            if (k & j) continue;
-            const uint32_t t = ((x[k] >> j) ^ x[k + j]) & mask;
-            x[k + j] ^= t;
-            x[k] ^= t << j;
-        }
-    }
 }
 
 // Bits 0..15 of x to the even bit positions.
@@ -98,9 +70,8 @@ __global__ void __launch_bounds__(kFloatThreads, 3)
 float_pack_kernel(const T* __restrict__ g, int64_t d, int64_t ld, MantissaSchedule sc, ProbList p, uint64_t seed,
                   uint64_t step, uint8_t* __restrict__ expo, uint32_t* __restrict__ planes, int w_max, int64_t words,
                   int32_t* out_level, double* out_p_sel, uint32_t* acc, uint32_t* done, int* status) {
-    constexpr int kWords = 32 * (int)sizeof(T) / 4;   // 32-bit words of a lane's entries
-    constexpr int kChunks = kWords / 4;               // 16-byte chunks
-    constexpr int kSlot = 32 * kWords;                // words per slot
+    constexpr int kChunks = kGroupChunks<T>;
+    constexpr int kSlot = kGroupSlot<T>;
     constexpr int kMantBits = sizeof(T) == 4 ? 23 : 7;
     extern __shared__ __align__(16) uint32_t sh_ring[];  // [warps][2][kSlot]
     __shared__ int sh_level;
@@ -125,34 +96,7 @@ float_pack_kernel(const T* __restrict__ g, int64_t d, int64_t ld, MantissaSchedu
     uint32_t* ring = sh_ring + warp * 2 * kSlot;
     const int64_t ngroups = (words + 31) / 32;
     const int64_t stride = (int64_t)gridDim.x * (kFloatThreads / 32);
-    // chunk c of lane l is kept at chunk position c ^ (l mod kChunks) (bf16: l / 2, a lane's chunks are 64 bytes)
-    auto place = [&](int l, int c) { return l * kWords + ((c ^ ((kChunks == 8 ? l : l >> 1) & (kChunks - 1))) << 2); };
-    auto fetch = [&](int64_t grp, uint32_t* slot) {
-        if (grp < ngroups) {
-            const int64_t e0 = grp * 1024;
-            if (e0 + 1024 <= d) {
-                const uint4* src = reinterpret_cast<const uint4*>(row + e0);
-#pragma unroll
-                for (int j = 0; j < kChunks; ++j) {
-                    const int i = j * 32 + lane;  // chunk of the group
-                    cp_async_16(slot + place(i / kChunks, i % kChunks), src + i);
-                }
-            } else {  // ragged last group: entries past d read as +0
-                for (int i = lane; i < kSlot; i += 32) {
-                    uint32_t v = 0u;
-                    if constexpr (sizeof(T) == 4) {
-                        if (e0 + i < d) v = reinterpret_cast<const uint32_t*>(row)[e0 + i];
-                    } else {
-                        const uint16_t* h = reinterpret_cast<const uint16_t*>(row) + e0;
-                        if (e0 + 2 * i < d) v = h[2 * i];
-                        if (e0 + 2 * i + 1 < d) v |= (uint32_t)h[2 * i + 1] << 16;
-                    }
-                    slot[place(i / kWords, (i % kWords) / 4) + (i & 3)] = v;
-                }
-            }
-        }
-        cp_async_commit();
-    };
+    auto fetch = [&](int64_t grp, uint32_t* slot) { fetch_group<T>(row, d, grp, ngroups, slot); };
     const bool wide_store = (reinterpret_cast<uintptr_t>(expo) & 31) == 0;
     uint32_t top = 0;  // largest exponent field seen, at the top of the word
     int64_t grp = (int64_t)blockIdx.x * (kFloatThreads / 32) + warp;
@@ -165,7 +109,7 @@ float_pack_kernel(const T* __restrict__ g, int64_t d, int64_t ld, MantissaSchedu
         uint32_t x[32];
 #pragma unroll
         for (int c = 0; c < kChunks; ++c) {
-            const uint4 q = *reinterpret_cast<const uint4*>(slot + place(lane, c));
+            const uint4 q = *reinterpret_cast<const uint4*>(slot + group_place<T>(lane, c));
             x[4 * c] = q.x; x[4 * c + 1] = q.y; x[4 * c + 2] = q.z; x[4 * c + 3] = q.w;
         }
         __syncwarp();  // the slot has been read by every lane: the copy after next may land in it
