@@ -64,7 +64,7 @@ __device__ __forceinline__ int zero_code_below(float gmax, int b) {
 template <typename T>
 __global__ void __launch_bounds__(kSweepThreads, 3)
 absmax_kernel(const T* __restrict__ g, int64_t d, int64_t ld, uint32_t* gmax_bits, uint32_t* acc, uint32_t* done,
-              DrawPlan pl, ProbList given, int draw, int* status, int* worker_err) {
+              const __grid_constant__ DrawPlan pl, const __grid_constant__ DrawnLevels drawn, int draw, int* status, int* worker_err) {
     using Tr = ElemTraits<T>;
     __shared__ uint32_t sh_max[kSweepThreads / 32];
     pdl_enter();
@@ -115,10 +115,7 @@ absmax_kernel(const T* __restrict__ g, int64_t d, int64_t ld, uint32_t* gmax_bit
         void_header(pl, m);
     } else {
         worker_err[m] = 0;
-        if (draw) {
-            draw_header(pl, m, given.p, __uint_as_float(as_f32), status, worker_err);
-            if (pl.bit_level[m] >= 0) pl.p_all[m * kMaxLevels + pl.bit_level[m]] = given.p[pl.bit_level[m]];
-        }
+        if (draw) write_header(pl, m, drawn.level[m], drawn.p[drawn.level[m]], __uint_as_float(as_f32), status, worker_err);
     }
 }
 
@@ -183,8 +180,8 @@ __global__ void __launch_bounds__(kSweepThreads, LMAX <= 8 ? 2 : 1)
 bit_stats_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* gmax_bits, BitSchedule sc,
                  unsigned long long* S_partial, int stat_ctas, uint32_t* done, DrawPlan pl, int* status, int* worker_err) {
     using Tr = ElemTraits<T>;
-    __shared__ unsigned long long sh_red[kSweepThreads / 32];
-    __shared__ double sh_delta[kMaxLevels], sh_p[kMaxLevels];
+    __shared__ unsigned long long sh_red[LMAX][kSweepThreads / 32];
+    __shared__ double sh_delta[kMaxLevels];
     pdl_enter();
     const int m = blockIdx.y;
     if (worker_err[m]) return;
@@ -239,14 +236,14 @@ bit_stats_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t*
         unsigned long long x = (unsigned long long)acc[l];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xFFFFFFFFu, x, o);
-        if ((threadIdx.x & 31) == 0) sh_red[threadIdx.x >> 5] = x;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            unsigned long long s = 0;
-            for (int w = 0; w < kSweepThreads / 32; ++w) s += sh_red[w];
-            S_partial[((int64_t)m * stat_ctas + blockIdx.x) * kMaxLevels + l] = s;
-        }
-        __syncthreads();
+        if ((threadIdx.x & 31) == 0) sh_red[l][threadIdx.x >> 5] = x;
+    }
+    __syncthreads();
+    if (threadIdx.x < sc.L) {
+        unsigned long long s = 0;
+#pragma unroll
+        for (int w = 0; w < kSweepThreads / 32; ++w) s += sh_red[threadIdx.x][w];
+        S_partial[((int64_t)m * stat_ctas + blockIdx.x) * kMaxLevels + threadIdx.x] = s;
     }
     if (!last_block(&done[m], gridDim.x)) return;
     // exact 128-bit sums of the per-block partials (integer adds: any order), rounded once to fp64; a warp per level
@@ -265,7 +262,7 @@ bit_stats_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t*
         if (lane == 0) sh_delta[l] = (double)gmax * ldexp(1.0, -sc.bits[l]) * sqrt((double)hi * 0x1.0p64 + (double)lo);
     }
     __syncthreads();
-    finish_levels(pl, m, sh_delta, sh_p, gmax, status, worker_err);
+    finish_levels(pl, m, sh_delta, gmax, status, worker_err);
 }
 
 // ---- pack: a warp turns 1024 consecutive entries into 32 words of each plane, a lane owning 32 consecutive entries (one
@@ -519,10 +516,11 @@ DrawPlan bit_draw_plan(Workspace& ws, const int32_t* b, int L, uint64_t seed, ui
 
 void launch_absmax(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const DrawPlan& plan, const double* p,
                    cudaStream_t s) {
+    const DrawnLevels drawn = draw_levels(p, plan.L, plan.seed, plan.step, M);
     const int nb = bit_blocks(ws, d, dtype == MLMC_BF16 ? 8 : 4, M, 8);
     auto go = [&](auto kernel, auto* row) {
         launch_kernel(ws, K_ABSMAX, kernel, dim3(nb, M), kSweepThreads, 0, s, row, d, ld, ws.gmax_bits, ws.acc_word, ws.done,
-                      plan, prob_list(p, plan.L), p ? 1 : 0, ws.status, ws.worker_err);
+                      plan, drawn, p ? 1 : 0, ws.status, ws.worker_err);
     };
     if (dtype == MLMC_BF16) go(absmax_kernel<bf16_t>, static_cast<const bf16_t*>(g));
     else go(absmax_kernel<float>, static_cast<const float*>(g));

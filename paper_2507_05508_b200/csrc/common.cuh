@@ -73,6 +73,12 @@ inline ProbList prob_list(const double* p, int L) {
     return r;
 }
 
+// The levels of a call with given probabilities: they depend on seed, step and worker only, so the host draws them.
+struct DrawnLevels {
+    double p[kMaxLevels];
+    uint8_t level[kEmitMaxWorkers];
+};
+
 constexpr int kTimingPool = 2048;  // event pairs kept between two reads
 
 struct Workspace {
@@ -241,10 +247,9 @@ __host__ __device__ __forceinline__ int draw_from_probs(const double* p, int L, 
     return 0;
 }
 
-// End of the level statistics of one worker, by one thread: the draw and the message header.
-__device__ __forceinline__ void draw_header(const DrawPlan& pl, int m, const double* p, float scale, int* status, int* worker_err) {
-    int level = draw_from_probs(p, pl.L, counter_uniform(pl.seed, pl.step, (uint64_t)m));
-    const double p_sel = p[level];
+// Header of one worker's dense message, by one thread.
+__device__ __forceinline__ void write_header(const DrawPlan& pl, int m, int level, double p_sel, float scale, int* status,
+                                             int* worker_err) {
     if (pl.out_level) {
         if (pl.width[level] > pl.w_max) {
             worker_err[m] = MLMC_ERR_CAPACITY;
@@ -256,6 +261,7 @@ __device__ __forceinline__ void draw_header(const DrawPlan& pl, int m, const dou
         pl.out_scale[m] = scale;
     }
     pl.bit_level[m] = level;
+    if (level >= 0) pl.p_all[m * kMaxLevels + level] = p_sel;
 }
 
 __device__ __forceinline__ void void_header(const DrawPlan& pl, int m) {
@@ -267,26 +273,48 @@ __device__ __forceinline__ void void_header(const DrawPlan& pl, int m) {
     }
 }
 
-// Probabilities from the residual norms sh_delta[L] of one worker (Lemma 3.4), the draw and the header; by the whole block.
-__device__ __forceinline__ void finish_levels(const DrawPlan& pl, int m, const double* sh_delta, double* sh_p, float scale,
-                                              int* status, int* worker_err) {
-    __shared__ double sh_total;
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int l = 0; l < pl.L; ++l) s += sh_delta[l];
-        sh_total = s;
+// p_l = delta_l / sum delta (Lemma 3.4; all weight on level 0 where every delta is 0) and the draw l* = min{ l : u < cdf_l },
+// by one warp, a level per lane (delta = 0 past the last level).  The last level with p > 0 has cdf 1.
+__device__ __forceinline__ int warp_draw(double delta, double u, double* p_out) {
+    const int l = threadIdx.x & 31;
+    double total = delta;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xFFFFFFFFu, total, o);
+    const double p = (total > 0.0) ? delta / total : (l == 0 ? 1.0 : 0.0);
+    double cdf = p;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const double y = __shfl_up_sync(0xFFFFFFFFu, cdf, o);
+        if (l >= o) cdf += y;
     }
-    __syncthreads();
-    if (threadIdx.x < pl.L) {
-        const int l = threadIdx.x;
-        const double s = sh_total;
-        const double p = (s > 0.0) ? sh_delta[l] / s : (l == 0 ? 1.0 : 0.0);
-        sh_p[l] = p;
-        pl.delta_all[m * kMaxLevels + l] = sh_delta[l];
+    const uint32_t positive = __ballot_sync(0xFFFFFFFFu, p > 0.0);  // never empty
+    const uint32_t below = __ballot_sync(0xFFFFFFFFu, p > 0.0 && u < cdf);
+    *p_out = p;
+    return below ? __ffs(below) - 1 : 31 - __clz((int)positive);
+}
+
+// Probabilities from the residual norms sh_delta[L] of one worker, the draw and the header; by warp 0 of the block.
+__device__ __forceinline__ void finish_levels(const DrawPlan& pl, int m, const double* sh_delta, float scale, int* status,
+                                              int* worker_err) {
+    if (threadIdx.x >= 32) return;
+    const int l = threadIdx.x;
+    const double delta = l < pl.L ? sh_delta[l] : 0.0;
+    double p;
+    const int level = warp_draw(delta, counter_uniform(pl.seed, pl.step, (uint64_t)m), &p);
+    if (l < pl.L) {
+        pl.delta_all[m * kMaxLevels + l] = delta;
         pl.p_all[m * kMaxLevels + l] = p;
     }
-    __syncthreads();
-    if (threadIdx.x == 0) draw_header(pl, m, sh_p, scale, status, worker_err);
+    const double p_sel = __shfl_sync(0xFFFFFFFFu, p, level);
+    if (l == 0) write_header(pl, m, level, p_sel, scale, status, worker_err);
+}
+
+inline DrawnLevels draw_levels(const double* p, int L, uint64_t seed, uint64_t step, int M) {
+    DrawnLevels r = {};
+    if (!p) return r;
+    for (int l = 0; l < L; ++l) r.p[l] = p[l];
+    for (int m = 0; m < M; ++m) r.level[m] = (uint8_t)draw_from_probs(p, L, counter_uniform(seed, step, (uint64_t)m));
+    return r;
 }
 
 // Magnitude key: monotone in |g| for finite values.  fp32: 31 bits; bf16: 15 bits.

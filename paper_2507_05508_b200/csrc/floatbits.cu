@@ -62,24 +62,21 @@ __device__ __forceinline__ uint32_t plane_word(const uint32_t* x, int bit) {
 // per entry and plane; from 6 planes on one bit transpose for all of them is cheaper).  The entries come through a
 // ring of two shared-memory slots per warp filled by 16-byte asynchronous copies; the 16-byte chunks of a lane are
 // XOR-ed with its number so that the lanes' reads fall into different banks.
-// The draw does not depend on the data: every block makes it itself; the worker's last block writes the header.
+// The draw does not depend on the data (it is the host's); the worker's last block writes the header.
 // Bound by HBM (reads 4 or 2 bytes, writes 1 byte and 1 + w bits per entry).  Ballots over rows of 32 entries took 1.14 ms
 // for 8 x 124M fp32 entries (0.72 of the copy rate).
 template <typename T>
 __global__ void __launch_bounds__(kFloatThreads, 3)
-float_pack_kernel(const T* __restrict__ g, int64_t d, int64_t ld, MantissaSchedule sc, ProbList p, uint64_t seed,
-                  uint64_t step, uint8_t* __restrict__ expo, uint32_t* __restrict__ planes, int w_max, int64_t words,
+float_pack_kernel(const T* __restrict__ g, int64_t d, int64_t ld, MantissaSchedule sc, const __grid_constant__ DrawnLevels drawn,
+                  uint8_t* __restrict__ expo, uint32_t* __restrict__ planes, int w_max, int64_t words,
                   int32_t* out_level, double* out_p_sel, uint32_t* acc, uint32_t* done, int* status) {
     constexpr int kChunks = kGroupChunks<T>;
     constexpr int kSlot = kGroupSlot<T>;
     constexpr int kMantBits = sizeof(T) == 4 ? 23 : 7;
     extern __shared__ __align__(16) uint32_t sh_ring[];  // [warps][2][kSlot]
-    __shared__ int sh_level;
     const int m = blockIdx.y;
-    if (threadIdx.x == 0) sh_level = draw_from_probs(p.p, sc.L, counter_uniform(seed, step, (uint64_t)m));
-    __syncthreads();
+    const int level = drawn.level[m];
     pdl_enter();
-    const int level = sh_level;
     if (sc.hi[level] - sc.lo[level] > w_max) {  // the field does not fit the message buffer
         if (blockIdx.x == 0 && threadIdx.x == 0) {
             set_status(status, MLMC_ERR_CAPACITY);
@@ -165,7 +162,7 @@ float_pack_kernel(const T* __restrict__ g, int64_t d, int64_t ld, MantissaSchedu
     acc[m] = 0u;
     if (any_bad) set_status(status, MLMC_ERR_NONFINITE);
     out_level[m] = any_bad ? -1 : level;
-    out_p_sel[m] = p.p[level];
+    out_p_sel[m] = drawn.p[level];
 }
 
 // Server average: thread = one word (32 entries); terms are added in worker order in fp32.
@@ -290,9 +287,9 @@ void launch_compress_floatbits(Workspace& ws, const void* g, int dtype, int64_t 
     int64_t nb = ((int64_t)ws.sm_count * 3) / M;  // persistent: three resident blocks per SM, rounded down
     if (nb > by_work) nb = by_work;
     if (nb < 1) nb = 1;
+    const DrawnLevels drawn = draw_levels(p, L, seed, step, M);
     auto go = [&](auto kernel, auto* row) {
-        launch_kernel(ws, K_FLOAT_PACK, kernel, dim3((unsigned)nb, M), kFloatThreads, float_pack_smem(sizeof(*row)), s, row, d, ld, sc, prob_list(p, L), seed,
-                      step, out.expo, out.planes, out.w_max, words, out.level, out.p_sel, ws.acc_word, ws.done, ws.status);
+        launch_kernel(ws, K_FLOAT_PACK, kernel, dim3((unsigned)nb, M), kFloatThreads, float_pack_smem(sizeof(*row)), s, row, d, ld, sc, drawn, out.expo, out.planes, out.w_max, words, out.level, out.p_sel, ws.acc_word, ws.done, ws.status);
     };
     if (dtype == MLMC_BF16) go(float_pack_kernel<bf16_t>, static_cast<const bf16_t*>(g));
     else go(float_pack_kernel<float>, static_cast<const float*>(g));

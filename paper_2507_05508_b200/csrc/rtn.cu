@@ -81,8 +81,8 @@ __global__ void __launch_bounds__(kRtnThreads, LMAX <= 6 ? 3 : 2)
 rtn_stats_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* gmax_bits, RtnSchedule sc, double* partial,
                  int rtn_ctas, uint32_t* done, DrawPlan pl, int* status, int* worker_err) {
     using Tr = ElemTraits<T>;
-    __shared__ double sh_red[kRtnThreads / 32];
-    __shared__ double sh_delta[kMaxLevels], sh_p[kMaxLevels];
+    __shared__ double sh_red[LMAX][kRtnThreads / 32];
+    __shared__ double sh_delta[kMaxLevels];
     __shared__ RtnLevel sh_lv[kRtnMaxLevels];
     pdl_enter();
     const int m = blockIdx.y;
@@ -198,14 +198,14 @@ rtn_stats_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t*
         double x = acc[l];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xFFFFFFFFu, x, o);
-        if ((threadIdx.x & 31) == 0) sh_red[threadIdx.x >> 5] = x;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double s = 0.0;
-            for (int w = 0; w < kRtnThreads / 32; ++w) s += sh_red[w];
-            partial[((int64_t)m * rtn_ctas + blockIdx.x) * kMaxLevels + l] = s;
-        }
-        __syncthreads();
+        if ((threadIdx.x & 31) == 0) sh_red[l][threadIdx.x >> 5] = x;
+    }
+    __syncthreads();
+    if (threadIdx.x < sc.L) {
+        double s = 0.0;
+#pragma unroll
+        for (int w = 0; w < kRtnThreads / 32; ++w) s += sh_red[threadIdx.x][w];
+        partial[((int64_t)m * rtn_ctas + blockIdx.x) * kMaxLevels + threadIdx.x] = s;
     }
     if (!last_block(&done[m], gridDim.x)) return;
     // the per-block partials, a warp per level in a fixed order; then p, the draw and the header
@@ -218,7 +218,7 @@ rtn_stats_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t*
         if (lane == 0) sh_delta[l] = sqrt(e);
     }
     __syncthreads();
-    finish_levels(pl, m, sh_delta, sh_p, c, status, worker_err);
+    finish_levels(pl, m, sh_delta, c, status, worker_err);
 }
 
 // The dense message of the drawn level: val_i = (C^l - C^{l-1})_i / p_l, rounded to fp32 once.

@@ -87,26 +87,13 @@ __device__ void finish_selection(const FinishPlan& pl, int m, int is_bf16, const
             }
             delta = sqrt(e);
         }
-        double total = delta;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xFFFFFFFFu, total, o);
-        const double p = (total > 0.0) ? delta / total : (l == 0 ? 1.0 : 0.0);
+        double p;
+        level = warp_draw(delta, counter_uniform(pl.seed, pl.step, (uint64_t)m), &p);
         if (l < L) {
             p_all[m * kMaxLevels + l] = p;
             delta_all[m * kMaxLevels + l] = delta;
         }
         if (!pl.want_emit) return;
-        // l* = min{ l : u < cdf_l }; the last level with p > 0 has cdf 1
-        double cdf = p;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const double y = __shfl_up_sync(0xFFFFFFFFu, cdf, o);
-            if (l >= o) cdf += y;
-        }
-        const double u = counter_uniform(pl.seed, pl.step, (uint64_t)m);
-        const uint32_t positive = __ballot_sync(0xFFFFFFFFu, p > 0.0);  // never empty
-        const uint32_t below = __ballot_sync(0xFFFFFFFFu, p > 0.0 && u < cdf);
-        level = below ? __ffs(below) - 1 : 31 - __clz((int)positive);
         p_sel = __shfl_sync(0xFFFFFFFFu, p, level);
         if (l == 0)
             fill_emit(pl, m, level, p_sel, level ? &q[level - 1] : nullptr, level < L - 1 ? &q[level] : nullptr,
