@@ -14,6 +14,8 @@
 //
 // Launches of a selection: begin, hist1, resolve1 and, for fp32, sums_candidates and two digit passes.  The step that
 // needs the whole result of a kernel runs in the block of each worker that finishes last.
+#include <algorithm>
+
 #include "topk_finish.cuh"
 
 namespace mlmc {
@@ -23,6 +25,7 @@ namespace {
 constexpr int kHistThreads = 1024;
 constexpr int kResolveThreads = 1024;
 constexpr int kDigitThreads = 512;
+constexpr int kBatchKeys = kEmitGroupVecs * 4;  // fp32 entries of a batch of the emit tiles
 
 // -------------------------------------------------------------------------------------------
 // begin: everything a selection accumulates into is cleared, and the queries are set up
@@ -439,166 +442,196 @@ resolve1_kernel(const uint32_t* hist1, Query* queries, uint8_t* table1, uint32_t
 // sweep 2 (fp32): per-interval energy of the bins that hold no threshold, and compaction of the keys
 // of the bins that do ("candidates": a few percent of the data) for the remaining digit passes
 // -------------------------------------------------------------------------------------------
-constexpr int kS2Threads = 512;
-constexpr int kS2Vecs = 2;                                   // 16-byte vectors per thread per round
-constexpr int kS2Round = kS2Threads * kS2Vecs * 4;            // elements per round
-constexpr int kStageSlack = 1024;                             // candidates that may wait for the next flush
-constexpr int kStage = kS2Round + kStageSlack;                // staged candidate keys per block
+// A warp takes one batch of the emit tiles at a time (four 16-byte vectors per lane, the next batch's vectors in flight) and
+// nothing is exchanged between warps before the end: the energies are added up per thread (fp64, a column of shared memory per
+// interval and thread), the candidates go to the warp's own stage.
+//   table: bin -> code.  code < 64: the bin lies wholly inside open interval `code` (between two thresholds); any other bin may
+//   hold a threshold and its keys are candidates.  The copy in shared memory has the sign bit set there, above the number of a
+//   column that nobody reads, so that an entry costs no branch.
+//   Below the lowest boundary bin there is one interval, and no candidate.  That is half of the entries or more, and in a
+//   gradient with per-layer scales whole batches: a batch whose largest key (recorded by the first sweep) lies below is added
+//   to a register without a look-up, and so is a row of 32 vectors (4 entries per lane) of any other batch whose keys do.
+//   In the rest, keys below share one word of the table, which leaves the banks to the others.
+// Without energies (given p) only the batches that reach the lowest boundary bin are read at all.
+// Bound by the shared-memory pipe where entries are looked up (90 % of its rate: a look-up of 2.6 wavefronts on average, load
+// and store of the column two each), else by DRAM.  With blocks that exchange their candidates at a barrier per tile, and
+// every entry looked up: 1.23 ms for 8 x 124M keys and 15 levels (now 1.08), 77 us for 16 x 11.7M and given p (now 23).
+constexpr int kS2Threads = 1024;      // 512 where the columns of 1024 threads do not fit (many levels)
+constexpr int kS2Stage = 383;         // keys per warp stage (half a batch adds at most 256), and one word for their number
+constexpr int kS2SmemMost = 227 * 1024;
 
-// table: bin -> code.  code < 64: the bin lies wholly inside open interval `code` (between two thresholds);
-// code >= 64: the bin may hold a threshold, its keys are compacted into the candidate buffer.
-// SUMS: per-interval energy of the threshold-free bins (adaptive p).  Loads are double-buffered in registers:
-// the next round's 16-byte vectors are in flight while the current round is processed.
 template <bool SUMS>
-__global__ void __launch_bounds__(kS2Threads, 2)
+__global__ void __launch_bounds__(kS2Threads, 1)
 sums_candidates_kernel(const float* __restrict__ g, int64_t d, int64_t ld, const uint8_t* table, int L,
                        double* __restrict__ sum_partial, int sum_ctas,
                        uint32_t* __restrict__ cand_keys, int64_t cand_cap, uint32_t* cand_count, int* cand_overflow,
                        const int* worker_err, const uint32_t* tile_max,
                        int tiles_per_worker, const uint32_t* cand_floor, const int* bracket_hit) {
     extern __shared__ __align__(16) uint8_t sh_raw[];
-    uint8_t* sh_table = sh_raw;                                                   // [32768]
-    uint32_t* sh_stage = reinterpret_cast<uint32_t*>(sh_raw + kBins1);            // [kStage]
-    double* sh_acc = reinterpret_cast<double*>(sh_raw + kBins1 + kStage * 4);     // [L][kS2Threads]  (SUMS)
-    __shared__ uint32_t sh_n;
-    __shared__ uint32_t sh_base;
+    const int threads = blockDim.x, warps = threads / 32, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint8_t* sh_table = sh_raw;                                                                      // [kBins1]
+    uint32_t* wcount = reinterpret_cast<uint32_t*>(sh_raw + kBins1) + warp * (kS2Stage + 1);         // [warps][1 + kS2Stage]
+    uint32_t* wstage = wcount + 1;
+    double* column = reinterpret_cast<double*>(sh_raw + kBins1 + warps * (kS2Stage + 1) * 4);        // [L + 1][threads]  (SUMS)
+    double* mine = column + threadIdx.x;
     pdl_enter();
     const int m = blockIdx.y;
     if (worker_err[m]) return;
     if (!SUMS && bracket_hit && bracket_hit[m]) return;  // the first sweep collected every boundary-bin key already
+    const uint32_t floor_key = cand_floor[m];
+    const uint32_t below = floor_key ? floor_key - 1u : 0u;  // every key below the floor is looked up here
     {
         const uint4* src = reinterpret_cast<const uint4*>(table + (int64_t)m * kBins1);
         uint4* dst = reinterpret_cast<uint4*>(sh_table);
-        for (int i = threadIdx.x; i < kBins1 / 16; i += kS2Threads) dst[i] = src[i];
+        const uint32_t unread = 0x80u | (uint32_t)L;
+        auto place = [&](uint32_t w) {  // four codes
+            const uint32_t boundary = __vcmpgeu4(w, 0x40404040u);
+            return (w & ~boundary) | (boundary & (unread * 0x01010101u));
+        };
+        for (int i = threadIdx.x; i < kBins1 / 16; i += threads) {
+            const uint4 x = src[i];
+            dst[i] = make_uint4(place(x.x), place(x.y), place(x.z), place(x.w));
+        }
         if (SUMS)
-            for (int i = threadIdx.x; i < L * kS2Threads; i += kS2Threads) sh_acc[i] = 0.0;
-        if (threadIdx.x == 0) sh_n = 0;
+            for (int l = 0; l <= L; ++l) mine[l * threads] = 0.0;
+        if (lane == 0) *wcount = 0u;
     }
     __syncthreads();
     const float* row = g + (int64_t)m * ld;
     uint32_t* cand = cand_keys + (int64_t)m * cand_cap;
-    // A round is one emit tile (kEmitTileVecs vectors); block b takes rounds b, b + gridDim.x, ...  Without
-    // energies (fixed p) only the candidates matter: a tile whose largest key lies below the lowest boundary bin
-    // holds none and is not read.  Such tiles cluster (whole layers lie below the thresholds), so the rounds are
-    // dealt out round-robin rather than in contiguous ranges.
-    static_assert(kS2Threads * kS2Vecs == kEmitTileVecs, "one round of the sweep is one emit tile");
-    const int64_t v1 = (d + 3) / 4;                                  // vectors of the row
-    const int64_t v0 = min((int64_t)blockIdx.x * kEmitTileVecs, v1);  // this block's first round
-    const int64_t vstep = (int64_t)gridDim.x * kEmitTileVecs;
-    const int64_t full_end = d / 4;  // vectors wholly inside the row
-    // which of the block's rounds hold a candidate, looked up once (rounds past the flag array are swept anyway)
-    constexpr int kWantFlags = 2048;
-    __shared__ uint8_t sh_want[kWantFlags];
-    if (!SUMS) {
-        const uint32_t floor_key = cand_floor[m];
-        const uint4* tmax = reinterpret_cast<const uint4*>(tile_max + ((int64_t)m * tiles_per_worker + blockIdx.x) * kEmitGroups);
-        const int64_t nrounds = (v1 - v0 + vstep - 1) / vstep;
-        static_assert(kEmitGroups == 8, "a tile's batch maxima are two 16-byte vectors");
-        for (int r = threadIdx.x; r < kWantFlags && r < nrounds; r += kS2Threads) {
-            const uint4 a = tmax[(int64_t)r * gridDim.x * 2], b = tmax[(int64_t)r * gridDim.x * 2 + 1];
-            sh_want[r] = max(max(max(a.x, a.y), max(a.z, a.w)), max(max(b.x, b.y), max(b.z, b.w))) >= floor_key;
+    const uint32_t* tmax = tile_max + (int64_t)m * tiles_per_worker * kEmitGroups;
+
+    auto flush = [&]() {  // called by the whole warp, after a __syncwarp
+        const uint32_t n = *wcount;
+        uint32_t base = 0;
+        if (lane == 0 && n) base = atomicAdd(&cand_count[m], n);
+        base = __shfl_sync(0xFFFFFFFFu, base, 0);
+        if ((int64_t)base + n <= cand_cap) {
+            for (uint32_t i = lane; i < n; i += 32) cand[base + i] = wstage[i];
+        } else if (lane == 0) {
+            cand_overflow[m] = 1;  // too many keys share the boundary bins: the full-sweep passes take over
         }
-        __syncthreads();
-    }
-    auto wanted = [&](int64_t vb) -> bool {  // block-uniform
-        if (SUMS) return true;
-        const int64_t r = (vb - v0) / vstep;
-        return vb < v1 && (r >= kWantFlags || sh_want[r]);
+        __syncwarp();
+        if (lane == 0) *wcount = 0u;
+        __syncwarp();
+    };
+    double low[2] = {0.0, 0.0};  // energy of the entries below the floor that were not looked up
+    auto add_low = [&](const uint4& q) {
+        const double x0 = (double)__uint_as_float(q.x), x1 = (double)__uint_as_float(q.y), x2 = (double)__uint_as_float(q.z),
+                     x3 = (double)__uint_as_float(q.w);
+        low[0] = fma(x0, x0, low[0]);
+        low[1] = fma(x1, x1, low[1]);
+        low[0] = fma(x2, x2, low[0]);
+        low[1] = fma(x3, x3, low[1]);
+    };
+    auto look_up = [&](uint32_t bits) -> int {  // negative: a candidate
+        return (int)reinterpret_cast<const int8_t*>(sh_table)[max(bits & 0x7FFFFFFFu, below) >> 16];
+    };
+    auto add = [&](uint32_t bits, int code) {
+        double* a = mine + (code & 63) * threads;
+        const double x = (double)__uint_as_float(bits);
+        *a = fma(x, x, *a);
+    };
+    auto look = [&](const uint4& q) -> uint32_t {  // one vector; the mask of its candidates
+        const int c0 = look_up(q.x), c1 = look_up(q.y), c2 = look_up(q.z), c3 = look_up(q.w);
+        if (SUMS) {
+            add(q.x, c0);
+            add(q.y, c1);
+            add(q.z, c2);
+            add(q.w, c3);
+        }
+        return (c0 < 0 ? 1u : 0u) | (c1 < 0 ? 2u : 0u) | (c2 < 0 ? 4u : 0u) | (c3 < 0 ? 8u : 0u);
+    };
+    auto reaches = [&](const uint4& q) -> bool {  // warp-uniform
+        const uint32_t k = max(max(q.x & 0x7FFFFFFFu, q.y & 0x7FFFFFFFu), max(q.z & 0x7FFFFFFFu, q.w & 0x7FFFFFFFu));
+        return __any_sync(0xFFFFFFFFu, k >= floor_key);
     };
 
-    auto flush = [&]() {  // called by all threads
-        const uint32_t n = sh_n;
-        if (threadIdx.x == 0 && n) sh_base = atomicAdd(&cand_count[m], n);
-        __syncthreads();
-        if (n) {
-            const uint32_t base = sh_base;
-            if ((int64_t)base + n <= cand_cap) {
-                for (uint32_t i = threadIdx.x; i < n; i += kS2Threads) cand[base + i] = sh_stage[i];
-            } else if (threadIdx.x == 0) {
-                cand_overflow[m] = 1;  // too many keys share the boundary bins: the full-sweep passes take over
-            }
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) sh_n = 0;
-        __syncthreads();
-    };
-    // One element: its energy goes to the interval's accumulator; a key of a boundary bin only sets its bit in `cm`,
-    // and the thread stages all its candidates of the round together (one counter update and one divergent region
-    // per thread and round instead of one per candidate).
-    auto take = [&](uint32_t bits, uint32_t bit, uint32_t& cm) {
-        const uint32_t key = bits & 0x7FFFFFFFu;
-        const uint32_t code = sh_table[key >> 16];
-        if (code < 64u) {
-            if (SUMS) {
-                const double x = (double)__uint_as_float(key);
-                double* a = &sh_acc[code * kS2Threads + threadIdx.x];
-                *a = fma(x, x, *a);
-            }
-        } else {
-            cm |= bit;
-        }
-    };
-    auto load_round = [&](int64_t vb, uint4 (&q)[kS2Vecs]) {
+    auto take = [&](const uint4 (&q)[4], bool high) {  // one batch
+        if (SUMS && !high) {
 #pragma unroll
-        for (int j = 0; j < kS2Vecs; ++j) {
-            const int64_t v = vb + j * kS2Threads + threadIdx.x;
-            if (v < full_end) q[j] = __ldg(reinterpret_cast<const uint4*>(row) + v);
+            for (int j = 0; j < 4; ++j) add_low(q[j]);
+            return;
+        }
+#pragma unroll
+        for (int h = 0; h < 4; h += 2) {
+            uint32_t cm = 0;  // bit 4 j + e: element e of vector h + j is a candidate
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                if (reaches(q[h + j])) cm |= look(q[h + j]) << (4 * j);
+                else if (SUMS) add_low(q[h + j]);
+            }
+            if (!__any_sync(0xFFFFFFFFu, cm != 0u)) continue;
+            if (cm) {  // few lanes have one, and rarely two
+                uint32_t pos = atomicAdd(wcount, (uint32_t)__popc(cm));
+                do {
+                    const int at = __ffs(cm) - 1;
+                    cm &= cm - 1u;
+                    const uint4& lo = q[h];
+                    const uint4& hi = q[h + 1];
+                    const uint32_t x = (at & 4) ? hi.x : lo.x, y = (at & 4) ? hi.y : lo.y, z = (at & 4) ? hi.z : lo.z,
+                                   w = (at & 4) ? hi.w : lo.w;
+                    const uint32_t xz = (at & 2) ? z : x, yw = (at & 2) ? w : y;
+                    wstage[pos++] = ((at & 1) ? yw : xz) & 0x7FFFFFFFu;
+                } while (cm);
+            }
+            __syncwarp();
+            if (*wcount > (uint32_t)(kS2Stage - 256)) flush();  // every lane reads the same number
+            __syncwarp();
         }
     };
 
-    uint4 cur[kS2Vecs], nxt[kS2Vecs];
-    bool want_cur = wanted(v0);
-    if (want_cur) load_round(v0, cur);
-    for (int64_t vb = v0; vb < v1; vb += vstep) {
-        const bool want_nxt = wanted(vb + vstep);
-        if (want_nxt) load_round(vb + vstep, nxt);
-        if (!SUMS && !want_cur) {  // nothing to do in this round: no barrier either (block-uniform)
-            want_cur = want_nxt;
+    // Batches are dealt round-robin to the warps of all blocks of the worker: which batches are costly differs from layer to
+    // layer.  A lane looks at the largest key of one of the warp's next 32 batches.
+    const int nbatch = (int)((d + kBatchKeys - 1) / kBatchKeys), stride = gridDim.x * warps;
+    auto load = [&](int b, uint4 (&q)[4]) {
+        if ((int64_t)(b + 1) * kBatchKeys > d) return;  // the row's ragged end
 #pragma unroll
-            for (int j = 0; j < kS2Vecs; ++j) cur[j] = nxt[j];
-            continue;
-        }
-        uint32_t cm = 0;  // bit 4 j + e: element e of vector j is a candidate
+        for (int j = 0; j < 4; ++j) q[j] = __ldg(reinterpret_cast<const uint4*>(row) + (int64_t)b * kEmitGroupVecs + j * 32 + lane);
+    };
+    for (int64_t base = blockIdx.x * warps + warp; base < nbatch; base += (int64_t)32 * stride) {
+        const int64_t own = base + (int64_t)lane * stride;
+        const uint32_t high = __ballot_sync(0xFFFFFFFFu, own < nbatch && tmax[min(own, (int64_t)nbatch - 1)] >= floor_key);
+        uint32_t todo = SUMS ? __ballot_sync(0xFFFFFFFFu, own < nbatch) : high;
+        if (!todo) continue;
+        uint4 cur[4], nxt[4];
+        load((int)base + (__ffs(todo) - 1) * stride, nxt);
+        while (todo) {
+            const int i = __ffs(todo) - 1, b = (int)base + i * stride;
+            todo &= todo - 1u;
 #pragma unroll
-        for (int j = 0; j < kS2Vecs; ++j) {
-            const int64_t v = vb + j * kS2Threads + threadIdx.x;
-            if (v < full_end) {
-                take(cur[j].x, 1u << (4 * j), cm); take(cur[j].y, 2u << (4 * j), cm);
-                take(cur[j].z, 4u << (4 * j), cm); take(cur[j].w, 8u << (4 * j), cm);
-            } else if (v < v1) {  // ragged tail of the row: staged one by one
-                for (int64_t i = v * 4; i < d; ++i) {
-                    uint32_t one = 0;
-                    const uint32_t bits = reinterpret_cast<const uint32_t*>(row)[i];
-                    take(bits, 1u, one);
-                    if (one) sh_stage[atomicAdd(&sh_n, 1u)] = bits & 0x7FFFFFFFu;
+            for (int j = 0; j < 4; ++j) cur[j] = nxt[j];
+            if (todo) load((int)base + (__ffs(todo) - 1) * stride, nxt);
+            if ((int64_t)(b + 1) * kBatchKeys > d) {
+                for (int64_t at = (int64_t)b * kBatchKeys; at < d; at += 32) {
+                    int code = 0;
+                    uint32_t bits = 0;
+                    if (at + lane < d) {
+                        bits = reinterpret_cast<const uint32_t*>(row)[at + lane];
+                        code = look_up(bits);
+                        if (SUMS) add(bits, code);
+                    }
+                    if (code < 0) wstage[atomicAdd(wcount, 1u)] = bits & 0x7FFFFFFFu;
+                    __syncwarp();
+                    if (*wcount > (uint32_t)(kS2Stage - 256)) flush();  // every lane reads the same number
+                    __syncwarp();
                 }
+                continue;
             }
+            take(cur, (high >> i) & 1u);
         }
-        if (cm) {
-            uint32_t pos = atomicAdd(&sh_n, (uint32_t)__popc(cm));
-#pragma unroll
-            for (int j = 0; j < kS2Vecs; ++j) {
-                if (cm & (1u << (4 * j))) sh_stage[pos++] = cur[j].x & 0x7FFFFFFFu;
-                if (cm & (2u << (4 * j))) sh_stage[pos++] = cur[j].y & 0x7FFFFFFFu;
-                if (cm & (4u << (4 * j))) sh_stage[pos++] = cur[j].z & 0x7FFFFFFFu;
-                if (cm & (8u << (4 * j))) sh_stage[pos++] = cur[j].w & 0x7FFFFFFFu;
-            }
-        }
-        __syncthreads();
-        if (sh_n > (uint32_t)kStageSlack) flush();  // uniform: sh_n is read after the barrier; a round adds at most kS2Round
-        want_cur = want_nxt;
-#pragma unroll
-        for (int j = 0; j < kS2Vecs; ++j) cur[j] = nxt[j];
     }
+    __syncwarp();
     flush();
     if (SUMS) {
-        for (int l = 0; l < L; ++l) {  // fixed-order tree: reproducible sums
-            double* a = sh_acc + l * kS2Threads;
-            for (int s = kS2Threads >> 1; s > 0; s >>= 1) {
-                if (threadIdx.x < s) a[threadIdx.x] += a[threadIdx.x + s];
-                __syncthreads();
-            }
-            if (threadIdx.x == 0) sum_partial[((int64_t)m * sum_ctas + blockIdx.x) * kMaxLevels + l] = a[0];
+        mine[(look_up(0u) & 63) * threads] += low[0] + low[1];
+        __syncthreads();
+        for (int l = warp; l < L; l += warps) {  // in a fixed order
+            double e = 0.0;
+            for (int i = lane; i < threads; i += 32) e += column[l * threads + i];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xFFFFFFFFu, e, o);
+            if (lane == 0) sum_partial[((int64_t)m * sum_ctas + blockIdx.x) * kMaxLevels + l] = e;
         }
     }
 }
@@ -886,8 +919,8 @@ int blocks_per_worker(const Workspace& ws, int64_t d, int vec, int threads, int 
     return (int)(nb < 1 ? 1 : nb);
 }
 
-size_t s2_smem(int L, bool sums) {
-    return kBins1 + (size_t)kStage * 4 + (sums ? (size_t)L * kS2Threads * sizeof(double) : 0);
+size_t s2_smem(int L, bool sums, int threads) {
+    return kBins1 + (size_t)(threads / 32) * (kS2Stage + 1) * 4 + (sums ? (size_t)(L + 1) * threads * sizeof(double) : 0);
 }
 
 size_t digit_smem(int nq, bool cells) {
@@ -977,12 +1010,12 @@ void launch_resolve1(Workspace& ws, int dtype, int M, const FinishPlan& plan, bo
 void launch_sums_candidates(Workspace& ws, const void* g, int64_t d, int M, int64_t ld, const FinishPlan& plan, bool brackets,
                             cudaStream_t s) {
     const bool sums = plan.adaptive != 0;
-    int nb = blocks_per_worker(ws, d, 4, kS2Threads, M, sums ? 2 : 8);  // without the accumulators four blocks fit an SM
-    if (nb > ws.sum_ctas) nb = ws.sum_ctas;
+    const int threads = sums && s2_smem(plan.L, sums, kS2Threads) > (size_t)kS2SmemMost ? kS2Threads / 2 : kS2Threads;
+    const int nb = std::min(blocks_per_worker(ws, d, 4, threads, M, 1), ws.sum_ctas);
     ws.cur_sum_ctas = nb;
-    launch_kernel(ws, K_SUMS_CAND, sums ? sums_candidates_kernel<true> : sums_candidates_kernel<false>, dim3(nb, M), kS2Threads,
-                  s2_smem(plan.L, sums), s, static_cast<const float*>(g), d, ld, ws.table1, plan.L, ws.sum_partial, ws.sum_ctas,
-                  ws.cand_keys, ws.cand_cap, ws.cand_count, ws.cand_overflow, ws.worker_err, ws.tile_max,
+    launch_kernel(ws, K_SUMS_CAND, sums ? sums_candidates_kernel<true> : sums_candidates_kernel<false>, dim3(nb, M), threads,
+                  s2_smem(plan.L, sums, threads), s, static_cast<const float*>(g), d, ld, ws.table1, plan.L, ws.sum_partial,
+                  ws.sum_ctas, ws.cand_keys, ws.cand_cap, ws.cand_count, ws.cand_overflow, ws.worker_err, ws.tile_max,
                   emit_tiles_per_worker(d, MLMC_F32), ws.cand_floor, brackets ? ws.bracket_hit : nullptr);
 }
 
@@ -1021,13 +1054,13 @@ void launch_copy_probs(Workspace& ws, int M, int L, const double* p_fixed, doubl
 int configure_select_kernels() {
     const int hist = (int)(kBins1 * sizeof(uint32_t));
     const int stage = (int)((kHistThreads / 32) * (kWarpStage + 1) * sizeof(uint32_t));
-    const int s2 = (int)s2_smem(kMaxLevels, true), digits = (int)digit_smem(kMaxQueries, true);
+    const int digits = (int)digit_smem(kMaxQueries, true);
     auto set = [](auto kernel, int bytes) {
         return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess;
     };
     const bool ok = set(hist1_kernel<float, false>, hist) && set(hist1_kernel<float, true>, hist + stage) &&
-                    set(hist1_kernel<bf16_t, false>, hist) && set(sums_candidates_kernel<true>, s2) &&
-                    set(sums_candidates_kernel<false>, s2) && set(digit_pass_kernel<2, true>, digits) &&
+                    set(hist1_kernel<bf16_t, false>, hist) && set(sums_candidates_kernel<true>, kS2SmemMost) &&
+                    set(sums_candidates_kernel<false>, (int)s2_smem(0, false, kS2Threads)) && set(digit_pass_kernel<2, true>, digits) &&
                     set(digit_pass_kernel<2, false>, digits) && set(digit_pass_kernel<3, true>, digits) &&
                     set(digit_pass_kernel<3, false>, digits);
     return ok ? MLMC_OK : MLMC_ERR_CUDA;
