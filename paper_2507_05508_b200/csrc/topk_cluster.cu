@@ -542,6 +542,9 @@ cluster_topk_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid
     if (!on) return;
     uint32_t* idx_w = idx_out + (int64_t)m * pl.capacity;
     float* val_w = val_out + (int64_t)m * pl.capacity;
+    // the offsets of a batch's entries take the place of the histogram (fp32: 1 KB per warp; those of bf16 do not fit)
+    uint16_t* stage = EW::S == 1 ? reinterpret_cast<uint16_t*>(sh_hist + warp * (kClHistWords / 32)) : nullptr;
+    static_assert(kBatchWords * 2 <= kClHistWords / 32 * 4, "a batch's offsets fit");
     for (int b = warp; b < nb; b += 32) {
         if (sh.batch_c[b] == 0) continue;
         uint32_t pc = 0, pa = 0, pb = 0;  // counts of the block's batches before this one
@@ -550,7 +553,8 @@ cluster_topk_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid
         pa = __reduce_add_sync(0xFFFFFFFFu, pa);
         pb = __reduce_add_sync(0xFFFFFFFFu, pb);
         uint3 run = make_uint3(before.x + pc, before.y + pa, before.z + pb);
-        emit_batch<T>(sh_row + b * kBatchWords, band, (sh.batch_a[b] | sh.batch_b[b]) != 0, (uint32_t)((b0 + b) * kBatchWords * EW::S), run,
+        __syncwarp();  // the stage has been read
+        emit_batch<T>(sh_row + b * kBatchWords, stage, band, (sh.batch_a[b] | sh.batch_b[b]) != 0, (uint32_t)((b0 + b) * kBatchWords * EW::S), run,
                       idx_w, val_w, pl.capacity);
     }
 }

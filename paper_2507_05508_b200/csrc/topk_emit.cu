@@ -30,7 +30,11 @@ namespace mlmc {
 namespace {
 
 constexpr int kBandThreads = 256;               // 8 warps per block, one tile per warp at a time
-constexpr int kWriteSlots = 3;                  // shared-memory batches per warp of the write pass
+constexpr int kWriteSlots = 3;                  // shared-memory batches per warp of the write pass,
+constexpr int kWriteBlocks = 3;                 // and blocks per SM
+// words of shared memory per warp of the write pass: the batches and the offsets of one batch's entries
+template <typename T>
+constexpr int kWriteWords = kWriteSlots * kEmitRows * 32 + kEmitRows * 32 * EmitWord<T>::S / 2;
 
 // Where a tile's counts are added up: {C, A, B, batches} per item, super-item and hyper-item of every worker.
 struct CountLevels {
@@ -133,7 +137,7 @@ band_count_kernel(const T* __restrict__ g, int64_t d, int64_t ld, int tiles_per_
 
 // Pass 2: every listed tile is read again and its band entries are written at their final positions.
 template <typename T>
-__global__ void __launch_bounds__(kBandThreads, 4)
+__global__ void __launch_bounds__(kBandThreads, kWriteBlocks)
 band_write_kernel(const T* __restrict__ g, int64_t d, int64_t ld, int tiles_per_worker, int M, const EmitParams* emit,
                   const uint4* tiles, CountLevels lv, const uint2* list, const uint32_t* list_n,
                   uint32_t* __restrict__ idx_out, float* __restrict__ val_out, int64_t capacity, uint32_t* group_n,
@@ -142,7 +146,7 @@ band_write_kernel(const T* __restrict__ g, int64_t d, int64_t ld, int tiles_per_
     constexpr int S = EW::S;
     // every warp stages its batches in a ring of three shared-memory slots: two copies are in flight while a
     // batch is ranked, and the words of a batch can be addressed by a run-time index
-    extern __shared__ __align__(16) uint32_t sh_dyn[];  // [warps][3][kBatchWords]
+    extern __shared__ __align__(16) uint32_t sh_dyn[];  // [warps][kWriteWords]
     pdl_enter();
     const int lane = threadIdx.x & 31;
     const int warps = gridDim.x * (kBandThreads / 32), gw = blockIdx.x * (kBandThreads / 32) + (threadIdx.x >> 5);
@@ -165,7 +169,8 @@ band_write_kernel(const T* __restrict__ g, int64_t d, int64_t ld, int tiles_per_
         }
     }
     const uint32_t total = *list_n;
-    uint32_t* ring = sh_dyn + (threadIdx.x >> 5) * kWriteSlots * kBatchWords;
+    uint32_t* ring = sh_dyn + (threadIdx.x >> 5) * kWriteWords<T>;
+    uint16_t* stage = reinterpret_cast<uint16_t*>(ring + kWriteSlots * kBatchWords);
     uint2 next = gw < (int)total ? list[gw] : make_uint2(0u, 0u);
     for (uint32_t f = gw; f < total; f += warps) {
         const uint2 entry = next;
@@ -217,7 +222,7 @@ band_write_kernel(const T* __restrict__ g, int64_t d, int64_t ld, int tiles_per_
             cp_async_wait<2>();  // this batch has landed
             __syncwarp();
             const uint32_t e0 = (uint32_t)((tile * kEmitTile + (int64_t)b * kBatchWords) * S);
-            emit_batch<T>(ring + (it % kWriteSlots) * kBatchWords, band, tile_ties, e0, run, idx_w, val_w, capacity);
+            emit_batch<T>(ring + (it % kWriteSlots) * kBatchWords, stage, band, tile_ties, e0, run, idx_w, val_w, capacity);
         }
     }
     cp_async_wait<0>();
@@ -288,8 +293,12 @@ aggregate_topk_kernel(const uint32_t* __restrict__ idx, const float* __restrict_
 // coordinate is the same as in the kernel above, so the two give identical results).  Lane l finds, for worker
 // m0 + l, where the warp's coordinates begin and end inside that worker's slice of the tile (two binary searches in
 // an index-sorted slice); the warp then walks the workers one after the other.
+// Bound by the latency of the entries while a worker's were added before the next one's were asked for (205 us for 32 x
+// 25.6M coordinates, 84 us for 3 x 22.6M dense ones); with the next chunk in flight 143 and 45 us.  Chunks of 64 entries:
+// 128 cost registers and blocks per SM (137 -> 151 us on the sparse messages of 8 x 124M coordinates, with 64: 127).
 constexpr int kAggSub = 512;
 constexpr int kAggWarps = kAggTile / kAggSub;
+constexpr int kChunk = 2;
 
 __global__ void __launch_bounds__(kAggWarps * 32)
 aggregate_topk_warps_kernel(const uint32_t* __restrict__ idx, const float* __restrict__ val, int64_t capacity, int M,
@@ -323,18 +332,45 @@ aggregate_topk_warps_kernel(const uint32_t* __restrict__ idx, const float* __res
                     s0 = (warp == 0) ? o0 : first_at_least((uint64_t)base);
                     s1 = (warp == kAggWarps - 1) ? o1 : first_at_least((uint64_t)base + kAggSub);
                 }
-                const int nm = min(32, M - m0);
-                for (int mm = 0; mm < nm; ++mm) {  // fixed worker order: reproducible fp32 sums
-                    const uint32_t b0 = __shfl_sync(0xFFFFFFFFu, s0, mm), b1 = __shfl_sync(0xFFFFFFFFu, s1, mm);
-                    if (b1 > b0) {  // warp-uniform
-                        const uint32_t* a = idx + (int64_t)(m0 + mm) * capacity;
-                        const float* v = val + (int64_t)(m0 + mm) * capacity;
-                        for (uint32_t j = b0 + lane; j < b1; j += 32) {
-                            const uint32_t off = __ldg(&a[j]) - (uint32_t)base;  // indices are unique within a worker
-                            if (off < (uint32_t)kAggSub) acc[off] += __ldg(&v[j]);  // an unsorted message cannot reach outside
-                        }
-                        __syncwarp();
+                // The entries in chunks of 32 kChunk, worker by worker (fixed order: reproducible fp32 sums); the next chunk is
+                // in flight while one is added.  A chunk's missing entries lie outside the warp's coordinates.
+                uint32_t live = __ballot_sync(0xFFFFFFFFu, s1 > s0);
+                uint32_t at = 0, end = 0, off[kChunk];
+                float v[kChunk];
+                const uint32_t* a = idx;
+                const float* x = val;
+                auto fetch = [&](uint32_t (&o)[kChunk], float (&y)[kChunk]) -> bool {  // the next chunk, if there is one
+                    if (at >= end) {
+                        if (!live) return false;
+                        const int mm = __ffs(live) - 1;
+                        live &= live - 1u;
+                        at = __shfl_sync(0xFFFFFFFFu, s0, mm);
+                        end = __shfl_sync(0xFFFFFFFFu, s1, mm);
+                        a = idx + (int64_t)(m0 + mm) * capacity;
+                        x = val + (int64_t)(m0 + mm) * capacity;
                     }
+#pragma unroll
+                    for (int k = 0; k < kChunk; ++k) {
+                        const uint32_t j = k * 32 + lane;
+                        o[k] = j < end - at ? __ldg(&a[at + j]) : (uint32_t)base - 1u;
+                        y[k] = j < end - at ? __ldg(&x[at + j]) : 0.0f;
+                    }
+                    at += min((uint32_t)kChunk * 32u, end - at);
+                    return true;
+                };
+                bool more = fetch(off, v);
+                while (more) {
+                    uint32_t off_n[kChunk];
+                    float v_n[kChunk];
+                    more = fetch(off_n, v_n);
+#pragma unroll
+                    for (int k = 0; k < kChunk; ++k) {
+                        const uint32_t o = off[k] - (uint32_t)base;      // indices are unique within a worker
+                        if (o < (uint32_t)kAggSub) acc[o] += v[k];       // an unsorted message cannot reach outside
+                        off[k] = off_n[k];
+                        v[k] = v_n[k];
+                    }
+                    __syncwarp();
                 }
             }
         }
@@ -398,11 +434,12 @@ aggregate_topk_direct_kernel(const uint32_t* __restrict__ idx, const float* __re
 }  // namespace
 
 int configure_emit_kernels() {
-    const int smem = (kBandThreads / 32) * kWriteSlots * kBatchWords * (int)sizeof(uint32_t);
-    if (cudaFuncSetAttribute(band_write_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-        cudaFuncSetAttribute(band_write_kernel<bf16_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
-        return MLMC_ERR_CUDA;
-    return MLMC_OK;
+    auto set = [](auto kernel, int words) {
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (kBandThreads / 32) * words * (int)sizeof(uint32_t)) == cudaSuccess;
+    };
+    return set(band_write_kernel<float>, kWriteWords<float>) && set(band_write_kernel<bf16_t>, kWriteWords<bf16_t>) ? MLMC_OK
+                                                                                                                   : MLMC_ERR_CUDA;
 }
 
 namespace {
@@ -415,7 +452,7 @@ void launch_emit_t(Workspace& ws, const T* g, int dtype, int64_t d, int M, int64
     const CountLevels lv = {ws.level_desc, ws.level_desc + (int64_t)M * n.items, ws.level_desc + (int64_t)M * (n.items + n.supers),
                             n.items, n.supers, n.hypers};
     const int wpb = kBandThreads / 32;
-    const size_t smem_w = (size_t)wpb * kWriteSlots * kBatchWords * sizeof(uint32_t);
+    const size_t smem_w = (size_t)wpb * kWriteWords<T> * sizeof(uint32_t);
     ws.last_emit_tiles = tpw;
     launch_kernel(ws, K_TILE_LIST, tile_list_kernel, dim3((tpw + kBandThreads - 1) / kBandThreads, M), kBandThreads, 0, s,
                   ws.tile_max, tpw, ws.emit, EmitWord<T>::kCap, ws.tile_desc, ws.tile_list, ws.list_n);
@@ -429,7 +466,7 @@ void launch_emit_t(Workspace& ws, const T* g, int dtype, int64_t d, int M, int64
     auto blocks = [&](int per_sm) { return (unsigned)std::min<int64_t>(by_work, (int64_t)ws.sm_count * per_sm * 2); };
     launch_kernel(ws, K_BAND_COUNT, band_count_kernel<T>, dim3(blocks(resident)), kBandThreads, (size_t)M * sizeof(uint2), s, g, d,
                   ld, tpw, M, ws.emit, ws.tile_desc, lv, ws.tile_list, ws.list_n);
-    launch_kernel(ws, K_EMIT, band_write_kernel<T>, dim3(blocks(4)), kBandThreads, smem_w, s, g, d, ld, tpw, M, ws.emit,
+    launch_kernel(ws, K_EMIT, band_write_kernel<T>, dim3(blocks(kWriteBlocks)), kBandThreads, smem_w, s, g, d, ld, tpw, M, ws.emit,
                   ws.tile_desc, lv, ws.tile_list, ws.list_n, out.idx, out.val, out.capacity, ws.group_n, ws.status);
 }
 
@@ -452,8 +489,12 @@ void launch_aggregate_topk(Workspace& ws, const mlmc_topk_msgs& msgs, int M, int
     const int64_t n_off = (int64_t)M * (ntiles + 1);
     launch_kernel(ws, K_AGG_OFFSETS, agg_offsets_kernel, dim3((unsigned)((n_off + 255) / 256)), 256, 0, s, msgs.idx, msgs.count,
                   msgs.level, msgs.capacity, M, ntiles, ws.agg_offsets);
-    int grid = ws.sm_count * 8;
-    if (grid > ntiles) grid = ntiles;
+    static const int resident = [] {
+        int n = 0;
+        const bool ok = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, aggregate_topk_warps_kernel, kAggWarps * 32, 0) == cudaSuccess;
+        return ok && n >= 1 ? n : 1;
+    }();
+    const int grid = std::min(ntiles, ws.sm_count * resident);
     launch_kernel(ws, K_AGG_TOPK, aggregate_topk_warps_kernel, dim3(grid), kAggWarps * 32, 0, s, msgs.idx, msgs.val,
                   msgs.capacity, M, d, ntiles, ws.agg_offsets, out);
 }
