@@ -108,7 +108,16 @@ __global__ void uniforms_kernel(double* u_dev, int M, uint64_t seed, uint64_t st
 // brackets is not tested (in a gradient with per-layer scales that is most batches).  Every warp stages its keys in a
 // private shared-memory buffer and moves the buffer to the candidate list when it fills up (one global counter update
 // per move).
-constexpr int kWarpStage = 767;  // keys per warp stage (a warp adds at most 512 per trip), plus one word for its count: 96 KB per block
+// The stage is small so that the block leaves an L1 cache to the streamed vectors (with 96 KB of stages beside the 128 KB of
+// counts the sweep of 16 x 11.7M keys took 170 us instead of 146).
+constexpr int kWarpStage = 319;  // keys per warp stage (half a batch adds at most 256), plus one word for its count: 40 KB per block
+
+// The key of element `at` of two vectors.
+__device__ __forceinline__ uint32_t nth_key(const uint4& lo, const uint4& hi, int at) {
+    const uint32_t x = (at & 4) ? hi.x : lo.x, y = (at & 4) ? hi.y : lo.y, z = (at & 4) ? hi.z : lo.z, w = (at & 4) ? hi.w : lo.w;
+    const uint32_t xz = (at & 2) ? z : x, yw = (at & 2) ? w : y;
+    return ((at & 1) ? yw : xz) & 0x7FFFFFFFu;
+}
 
 template <typename T, bool BR>
 __global__ void __launch_bounds__(kHistThreads, 1)
@@ -196,26 +205,25 @@ hist1_kernel(const T* __restrict__ g, int64_t d, int64_t ld, uint32_t* __restric
             wm = __reduce_max_sync(0xFFFFFFFFu, vm);
             if constexpr (BR) {
                 if (wm >= lo_min) {  // warp-uniform
-                    uint32_t cm = 0;  // bit 4 j + e: element e of vector j lies in a bracket
 #pragma unroll
-                    for (int j = 0; j < kBatch; ++j) {
-                        cm |= in_bracket(q[j].x) ? (1u << (4 * j)) : 0u;
-                        cm |= in_bracket(q[j].y) ? (2u << (4 * j)) : 0u;
-                        cm |= in_bracket(q[j].z) ? (4u << (4 * j)) : 0u;
-                        cm |= in_bracket(q[j].w) ? (8u << (4 * j)) : 0u;
-                    }
-                    if (cm) {  // this lane's keys go to the warp's stage at a position taken from the warp's counter
-                        uint32_t pos = atomicAdd(wcount, (uint32_t)__popc(cm));
+                    for (int h = 0; h < kBatch; h += 2) {
+                        uint32_t cm = 0;  // bit 4 j + e: element e of vector h + j lies in a bracket
 #pragma unroll
-                        for (int j = 0; j < kBatch; ++j) {
-                            if (cm & (1u << (4 * j))) wstage[pos++] = q[j].x & 0x7FFFFFFFu;
-                            if (cm & (2u << (4 * j))) wstage[pos++] = q[j].y & 0x7FFFFFFFu;
-                            if (cm & (4u << (4 * j))) wstage[pos++] = q[j].z & 0x7FFFFFFFu;
-                            if (cm & (8u << (4 * j))) wstage[pos++] = q[j].w & 0x7FFFFFFFu;
+                        for (int j = 0; j < 2; ++j) {
+                            cm |= in_bracket(q[h + j].x) ? (1u << (4 * j)) : 0u;
+                            cm |= in_bracket(q[h + j].y) ? (2u << (4 * j)) : 0u;
+                            cm |= in_bracket(q[h + j].z) ? (4u << (4 * j)) : 0u;
+                            cm |= in_bracket(q[h + j].w) ? (8u << (4 * j)) : 0u;
                         }
+                        if (!__any_sync(0xFFFFFFFFu, cm != 0u)) continue;
+                        if (cm) {  // this lane's keys go to the warp's stage at a position taken from the warp's counter
+                            uint32_t pos = atomicAdd(wcount, (uint32_t)__popc(cm));
+                            for (; cm; cm &= cm - 1u) wstage[pos++] = nth_key(q[h], q[h + 1], __ffs(cm) - 1);
+                        }
+                        __syncwarp();
+                        if (*wcount > (uint32_t)(kWarpStage - 256)) flush_stage();  // room for another half
+                        __syncwarp();
                     }
-                    __syncwarp();
-                    if (*wcount > (uint32_t)(kWarpStage - 32 * 4 * kBatch)) flush_stage();  // room for one more trip
                 }
             }
         } else {  // the row's end, vector by vector; batches past it have the largest key 0
@@ -564,16 +572,7 @@ sums_candidates_kernel(const float* __restrict__ g, int64_t d, int64_t ld, const
             if (!__any_sync(0xFFFFFFFFu, cm != 0u)) continue;
             if (cm) {  // few lanes have one, and rarely two
                 uint32_t pos = atomicAdd(wcount, (uint32_t)__popc(cm));
-                do {
-                    const int at = __ffs(cm) - 1;
-                    cm &= cm - 1u;
-                    const uint4& lo = q[h];
-                    const uint4& hi = q[h + 1];
-                    const uint32_t x = (at & 4) ? hi.x : lo.x, y = (at & 4) ? hi.y : lo.y, z = (at & 4) ? hi.z : lo.z,
-                                   w = (at & 4) ? hi.w : lo.w;
-                    const uint32_t xz = (at & 2) ? z : x, yw = (at & 2) ? w : y;
-                    wstage[pos++] = ((at & 1) ? yw : xz) & 0x7FFFFFFFu;
-                } while (cm);
+                for (; cm; cm &= cm - 1u) wstage[pos++] = nth_key(q[h], q[h + 1], __ffs(cm) - 1);
             }
             __syncwarp();
             if (*wcount > (uint32_t)(kS2Stage - 256)) flush();  // every lane reads the same number
@@ -984,7 +983,10 @@ void launch_uniforms(Workspace& ws, int M, uint64_t seed, uint64_t step, cudaStr
 void launch_hist1(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, bool brackets, cudaStream_t s) {
     const int tpw = emit_tiles_per_worker(d, dtype);
     size_t smem = kBins1 * sizeof(uint32_t);
-    const int nb = blocks_per_worker(ws, d, dtype == MLMC_BF16 ? 8 : 4, kHistThreads, M, 2);
+    // One wave of blocks (every block clears and flushes a whole histogram: two waves cost 2 % at 16 x 11.7M keys), unless
+    // whole blocks per worker leave more than 5 % of the SMs idle (32 workers: 456 against 401 us for 26M bf16 keys each).
+    const int waves = ws.sm_count / M * M * 20 < ws.sm_count * 19 ? 2 : 1;
+    const int nb = blocks_per_worker(ws, d, dtype == MLMC_BF16 ? 8 : 4, kHistThreads, M, waves);
     auto go = [&](auto kernel, auto* row) {
         launch_kernel(ws, K_HIST1, kernel, dim3(nb, M), kHistThreads, smem, s, row, d, ld, ws.hist1, ws.tile_max, tpw,
                       ws.status, ws.worker_err, ws.bracket, ws.cand_keys, ws.cand_cap, ws.cand_count, ws.cand_overflow);
