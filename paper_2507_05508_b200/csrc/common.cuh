@@ -180,11 +180,10 @@ __device__ __forceinline__ void shared_add_limbs(uint32_t addr, uint64_t x) {
                  : "memory");
 }
 
-// Stores x at the shared-memory address `at` and moves on by STEP bytes, where `flag` is negative; no branch.
-template <uint32_t STEP>
-__device__ __forceinline__ void shared_push_if_negative(int flag, uint32_t& at, uint32_t x) {
+// Stores x at the shared-memory address `at` and moves on by `step` bytes, where `flag` is negative; no branch.
+__device__ __forceinline__ void shared_push_if_negative(int flag, uint32_t& at, uint32_t x, uint32_t step) {
     asm volatile("{\n\t.reg .pred p;\n\tsetp.lt.s32 p, %1, 0;\n\t@p st.shared.u32 [%0], %2;\n\t@p add.u32 %0, %0, %3;\n\t}"
-                 : "+r"(at) : "r"(flag), "r"(x), "n"(STEP) : "memory");
+                 : "+r"(at) : "r"(flag), "r"(x), "r"(step) : "memory");
 }
 
 // mant^2 of an fp32 entry (the implicit bit included, below the normal range none): the entry is mant 2^(max(e,1) - 150).

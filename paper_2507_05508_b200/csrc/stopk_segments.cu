@@ -349,7 +349,7 @@ segment_sweep_kernel(const float* __restrict__ g, int64_t d, int64_t ld, int m0,
 #pragma unroll
         for (int e = 0; e < kTripVecs * 4; ++e) {
             take(x[e], code[e]);
-            shared_push_if_negative<4>(code[e], at, x[e]);
+            shared_push_if_negative(code[e], at, x[e], 4u);
         }
         // a buffer without room for another trip?  (every thread gets the same answer)
         const bool full = __syncthreads_or(fill > (uint32_t)(kWarpBuffer - 32 * kTripVecs * 4));

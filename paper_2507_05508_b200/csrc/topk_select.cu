@@ -452,78 +452,98 @@ resolve1_kernel(const uint32_t* hist1, Query* queries, uint8_t* table1, uint32_t
 // -------------------------------------------------------------------------------------------
 // A warp takes one batch of the emit tiles at a time (four 16-byte vectors per lane, the next batch's vectors in flight) and
 // nothing is exchanged between warps before the end: the energies are added up per thread (fp64, a column of shared memory per
-// interval and thread), the candidates go to the warp's own stage.
-//   table: bin -> code.  code < 64: the bin lies wholly inside open interval `code` (between two thresholds); any other bin may
-//   hold a threshold and its keys are candidates.  The copy in shared memory has the sign bit set there, above the number of a
-//   column that nobody reads, so that an entry costs no branch.
-//   Below the lowest boundary bin there is one interval, and no candidate.  That is half of the entries or more, and in a
-//   gradient with per-layer scales whole batches: a batch whose largest key (recorded by the first sweep) lies below is added
-//   to a register without a look-up, and so is a row of 32 vectors (4 entries per lane) of any other batch whose keys do.
-//   In the rest, keys below share one word of the table, which leaves the banks to the others.
+// interval and thread), the candidates wait in slots of the thread's own, and a warp moves them on when a lane's fill up.
+//   groups: 16 consecutive bins share a word {which of them hold a threshold (high half), boundary bins above the 16 (low
+//   half)}: the interval of a key is the latter plus the bits at or above its bin.  The gradient's magnitudes in a warp fall
+//   into a few dozen of the 2048 words, most of them in different banks; looked up bin by bin the banks collide three times.
+//   A candidate's energy goes to a column that nobody reads, so that an entry costs no branch.
+//   Below the lowest boundary bin there is one interval and no candidate: a batch whose largest key (recorded by the first
+//   sweep) lies below is added to a register without a look-up.  In a gradient with per-layer scales those are whole layers.
 // Without energies (given p) only the batches that reach the lowest boundary bin are read at all.
-// Bound by the shared-memory pipe where entries are looked up (90 % of its rate: a look-up of 2.6 wavefronts on average, load
-// and store of the column two each), else by DRAM.  With blocks that exchange their candidates at a barrier per tile, and
-// every entry looked up: 1.23 ms for 8 x 124M keys and 15 levels (now 1.08), 77 us for 16 x 11.7M and given p (now 23).
+// The columns bound the kernel (load and store, two shared-memory wavefronts each, of about 6 per warp and entry), with the
+// arithmetic pipe close behind; where no batch is looked up, DRAM does.
 constexpr int kS2Threads = 1024;      // 512 where the columns of 1024 threads do not fit (many levels)
-constexpr int kS2Stage = 383;         // keys per warp stage (half a batch adds at most 256), and one word for their number
-constexpr int kS2SmemMost = 227 * 1024;
+constexpr int kS2Slots = 8;           // candidates per thread; a vector adds at most 4
+constexpr int kS2Groups = kBins1 / 16;
+constexpr int kS2SmemMost = 226 * 1024;  // beside the static arrays
 
 template <bool SUMS>
 __global__ void __launch_bounds__(kS2Threads, 1)
-sums_candidates_kernel(const float* __restrict__ g, int64_t d, int64_t ld, const uint8_t* table, int L,
+sums_candidates_kernel(const float* __restrict__ g, int64_t d, int64_t ld, const uint8_t* table, const Query* queries, int nq, int L,
                        double* __restrict__ sum_partial, int sum_ctas,
                        uint32_t* __restrict__ cand_keys, int64_t cand_cap, uint32_t* cand_count, int* cand_overflow,
                        const int* worker_err, const uint32_t* tile_max,
                        int tiles_per_worker, const uint32_t* cand_floor, const int* bracket_hit) {
     extern __shared__ __align__(16) uint8_t sh_raw[];
+    __shared__ uint8_t sh_above[kMaxLevels + 1];   // boundary bins above a bin of code j
+    __shared__ uint8_t sh_code[kMaxLevels + 1];    // interval (number of thresholds above) with so many boundary bins above it
     const int threads = blockDim.x, warps = threads / 32, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint8_t* sh_table = sh_raw;                                                                      // [kBins1]
-    uint32_t* wcount = reinterpret_cast<uint32_t*>(sh_raw + kBins1) + warp * (kS2Stage + 1);         // [warps][1 + kS2Stage]
-    uint32_t* wstage = wcount + 1;
-    double* column = reinterpret_cast<double*>(sh_raw + kBins1 + warps * (kS2Stage + 1) * 4);        // [L + 1][threads]  (SUMS)
+    uint32_t* sh_group = reinterpret_cast<uint32_t*>(sh_raw);                                        // [kS2Groups]
+    uint32_t* slots = sh_group + kS2Groups + threadIdx.x;                                            // [kS2Slots][threads]
+    double* column = reinterpret_cast<double*>(sh_group + kS2Groups + kS2Slots * threads);           // [L + 1][threads]  (SUMS)
     double* mine = column + threadIdx.x;
     pdl_enter();
     const int m = blockIdx.y;
     if (worker_err[m]) return;
     if (!SUMS && bracket_hit && bracket_hit[m]) return;  // the first sweep collected every boundary-bin key already
     const uint32_t floor_key = cand_floor[m];
-    const uint32_t below = floor_key ? floor_key - 1u : 0u;  // every key below the floor is looked up here
-    {
-        const uint4* src = reinterpret_cast<const uint4*>(table + (int64_t)m * kBins1);
-        uint4* dst = reinterpret_cast<uint4*>(sh_table);
-        const uint32_t unread = 0x80u | (uint32_t)L;
-        auto place = [&](uint32_t w) {  // four codes
-            const uint32_t boundary = __vcmpgeu4(w, 0x40404040u);
-            return (w & ~boundary) | (boundary & (unread * 0x01010101u));
-        };
-        for (int i = threadIdx.x; i < kBins1 / 16; i += threads) {
-            const uint4 x = src[i];
-            dst[i] = make_uint4(place(x.x), place(x.y), place(x.z), place(x.w));
+    if (warp == 0) {  // queries share boundary bins: the live ones are contiguous, their slots ascend
+        const Query q = queries[m * kMaxQueries + min(lane, nq > 0 ? nq - 1 : 0)];
+        const bool live = lane < nq && q.trivial == 0u;
+        const uint32_t slot = live ? q.slot : kNoSlot, next = __shfl_down_sync(0xFFFFFFFFu, slot, 1);
+        const uint32_t none = __ballot_sync(0xFFFFFFFFu, lane < nq && q.trivial == 1u);  // k = 0: thresholds above every bin
+        if (lane == 0) {
+            sh_above[0] = 0;
+            sh_code[0] = (uint8_t)__popc(none);
         }
-        if (SUMS)
-            for (int l = 0; l <= L; ++l) mine[l * threads] = 0.0;
-        if (lane == 0) *wcount = 0u;
+        if (live) {
+            sh_above[lane + 1] = (uint8_t)(slot + 1u);
+            if (lane == 31 || next != slot) sh_code[slot + 1u] = (uint8_t)(lane + 1);
+        } else if (lane < nq) {
+            sh_above[lane + 1] = 0;
+        }
+    }
+    if (SUMS)
+        for (int l = 0; l <= L; ++l) mine[l * threads] = 0.0;
+    __syncthreads();
+    for (int i = threadIdx.x; i < kS2Groups; i += threads) {
+        const uint4 x = reinterpret_cast<const uint4*>(table + (int64_t)m * kBins1)[i];
+        auto boundary = [](uint32_t w) {  // bit i: code i of the four is 64 or more
+            const uint32_t c = __vcmpgeu4(w, 0x40404040u);
+            return (c & 1u) | ((c >> 7) & 2u) | ((c >> 14) & 4u) | ((c >> 21) & 8u);
+        };
+        const uint32_t mask = boundary(x.x) | boundary(x.y) << 4 | boundary(x.z) << 8 | boundary(x.w) << 12, top = x.w >> 24;
+        sh_group[i] = mask << 16 | (top >= 64u ? top - 64u : sh_above[top]);
     }
     __syncthreads();
     const float* row = g + (int64_t)m * ld;
     uint32_t* cand = cand_keys + (int64_t)m * cand_cap;
     const uint32_t* tmax = tile_max + (int64_t)m * tiles_per_worker * kEmitGroups;
 
-    auto flush = [&]() {  // called by the whole warp, after a __syncwarp
-        const uint32_t n = *wcount;
+    const uint32_t slots0 = (uint32_t)__cvta_generic_to_shared(slots), step = (uint32_t)threads * 4u;
+    uint32_t at = slots0;
+    auto flush = [&]() {  // called by the whole warp
+        const uint32_t n = (at - slots0) / step;
+        uint32_t upto = n;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, upto, o);
+            if (lane >= o) upto += y;
+        }
+        const uint32_t total = __shfl_sync(0xFFFFFFFFu, upto, 31);
+        if (total == 0u) return;
         uint32_t base = 0;
-        if (lane == 0 && n) base = atomicAdd(&cand_count[m], n);
+        if (lane == 0) base = atomicAdd(&cand_count[m], total);
         base = __shfl_sync(0xFFFFFFFFu, base, 0);
-        if ((int64_t)base + n <= cand_cap) {
-            for (uint32_t i = lane; i < n; i += 32) cand[base + i] = wstage[i];
+        if ((int64_t)base + total <= cand_cap) {
+            uint32_t* to = cand + base + (upto - n);
+            for (uint32_t i = 0; i < n; ++i) to[i] = slots[i * threads] & 0x7FFFFFFFu;
         } else if (lane == 0) {
             cand_overflow[m] = 1;  // too many keys share the boundary bins: the full-sweep passes take over
         }
-        __syncwarp();
-        if (lane == 0) *wcount = 0u;
-        __syncwarp();
+        at = slots0;
     };
-    double low[2] = {0.0, 0.0};  // energy of the entries below the floor that were not looked up
+    double low[2] = {0.0, 0.0};  // energy of the batches below the floor
     auto add_low = [&](const uint4& q) {
         const double x0 = (double)__uint_as_float(q.x), x1 = (double)__uint_as_float(q.y), x2 = (double)__uint_as_float(q.z),
                      x3 = (double)__uint_as_float(q.w);
@@ -532,53 +552,21 @@ sums_candidates_kernel(const float* __restrict__ g, int64_t d, int64_t ld, const
         low[0] = fma(x2, x2, low[0]);
         low[1] = fma(x3, x3, low[1]);
     };
-    auto look_up = [&](uint32_t bits) -> int {  // negative: a candidate
-        return (int)reinterpret_cast<const int8_t*>(sh_table)[max(bits & 0x7FFFFFFFu, below) >> 16];
+    auto look_up = [&](uint32_t bits) -> uint32_t {  // byte offset of the group's word: four times key bits 30..20
+        return *reinterpret_cast<const uint32_t*>(sh_raw + ((bits >> 18) & 0x1FFCu));
     };
-    auto add = [&](uint32_t bits, int code) {
-        double* a = mine + (code & 63) * threads;
-        const double x = (double)__uint_as_float(bits);
-        *a = fma(x, x, *a);
-    };
-    auto look = [&](const uint4& q) -> uint32_t {  // one vector; the mask of its candidates
-        const int c0 = look_up(q.x), c1 = look_up(q.y), c2 = look_up(q.z), c3 = look_up(q.w);
+    auto take = [&](uint32_t bits, uint32_t group) -> uint32_t {  // bit 0: a candidate
+        const uint32_t u = __funnelshift_r(group, 0u, (bits >> 16) | 16u);  // the boundary bins from the key's own upwards
         if (SUMS) {
-            add(q.x, c0);
-            add(q.y, c1);
-            add(q.z, c2);
-            add(q.w, c3);
+            const uint32_t n = (u & 1u) ? (uint32_t)L : (group & 0xFFFFu) + (uint32_t)__popc(u);
+            double* a = mine + n * (uint32_t)threads;
+            const double x = (double)__uint_as_float(bits);
+            *a = fma(x, x, *a);
         }
-        return (c0 < 0 ? 1u : 0u) | (c1 < 0 ? 2u : 0u) | (c2 < 0 ? 4u : 0u) | (c3 < 0 ? 8u : 0u);
+        return u;
     };
-    auto reaches = [&](const uint4& q) -> bool {  // warp-uniform
-        const uint32_t k = max(max(q.x & 0x7FFFFFFFu, q.y & 0x7FFFFFFFu), max(q.z & 0x7FFFFFFFu, q.w & 0x7FFFFFFFu));
-        return __any_sync(0xFFFFFFFFu, k >= floor_key);
-    };
-
-    auto take = [&](const uint4 (&q)[4], bool high) {  // one batch
-        if (SUMS && !high) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) add_low(q[j]);
-            return;
-        }
-#pragma unroll
-        for (int h = 0; h < 4; h += 2) {
-            uint32_t cm = 0;  // bit 4 j + e: element e of vector h + j is a candidate
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                if (reaches(q[h + j])) cm |= look(q[h + j]) << (4 * j);
-                else if (SUMS) add_low(q[h + j]);
-            }
-            if (!__any_sync(0xFFFFFFFFu, cm != 0u)) continue;
-            if (cm) {  // few lanes have one, and rarely two
-                uint32_t pos = atomicAdd(wcount, (uint32_t)__popc(cm));
-                for (; cm; cm &= cm - 1u) wstage[pos++] = nth_key(q[h], q[h + 1], __ffs(cm) - 1);
-            }
-            __syncwarp();
-            if (*wcount > (uint32_t)(kS2Stage - 256)) flush();  // every lane reads the same number
-            __syncwarp();
-        }
-    };
+    auto set_aside = [&](uint32_t u, uint32_t bits) { shared_push_if_negative((int)(u << 31), at, bits, step); };
+    auto full = [&]() -> bool { return __any_sync(0xFFFFFFFFu, at > slots0 + (kS2Slots - 4) * step); };
 
     // Batches are dealt round-robin to the warps of all blocks of the worker: which batches are costly differs from layer to
     // layer.  A lane looks at the largest key of one of the warp's next 32 batches.
@@ -602,35 +590,46 @@ sums_candidates_kernel(const float* __restrict__ g, int64_t d, int64_t ld, const
             for (int j = 0; j < 4; ++j) cur[j] = nxt[j];
             if (todo) load((int)base + (__ffs(todo) - 1) * stride, nxt);
             if ((int64_t)(b + 1) * kBatchKeys > d) {
-                for (int64_t at = (int64_t)b * kBatchKeys; at < d; at += 32) {
-                    int code = 0;
-                    uint32_t bits = 0;
-                    if (at + lane < d) {
-                        bits = reinterpret_cast<const uint32_t*>(row)[at + lane];
-                        code = look_up(bits);
-                        if (SUMS) add(bits, code);
+                for (int64_t e = (int64_t)b * kBatchKeys + lane; e - lane < d; e += 32) {
+                    if (e < d) {
+                        const uint32_t bits = reinterpret_cast<const uint32_t*>(row)[e];
+                        set_aside(take(bits, look_up(bits)), bits);
                     }
-                    if (code < 0) wstage[atomicAdd(wcount, 1u)] = bits & 0x7FFFFFFFu;
                     __syncwarp();
-                    if (*wcount > (uint32_t)(kS2Stage - 256)) flush();  // every lane reads the same number
-                    __syncwarp();
+                    if (full()) flush();
                 }
-                continue;
+            } else if (SUMS && !((high >> i) & 1u)) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) add_low(cur[j]);
+            } else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const uint32_t g0 = look_up(cur[j].x), g1 = look_up(cur[j].y), g2 = look_up(cur[j].z), g3 = look_up(cur[j].w);
+                    const uint32_t u0 = take(cur[j].x, g0), u1 = take(cur[j].y, g1), u2 = take(cur[j].z, g2), u3 = take(cur[j].w, g3);
+                    if (__any_sync(0xFFFFFFFFu, ((u0 | u1 | u2 | u3) & 1u) != 0u)) {  // a store takes its turn even if no lane has one
+                        set_aside(u0, cur[j].x);
+                        set_aside(u1, cur[j].y);
+                        set_aside(u2, cur[j].z);
+                        set_aside(u3, cur[j].w);
+                        if (full()) flush();
+                    }
+                }
             }
-            take(cur, (high >> i) & 1u);
         }
     }
     __syncwarp();
     flush();
     if (SUMS) {
-        mine[(look_up(0u) & 63) * threads] += low[0] + low[1];
+        const uint32_t lowest = sh_group[0], last = (lowest & 0xFFFFu) + (uint32_t)__popc(lowest >> 16);  // the interval below all
+        mine[last * threads] += low[0] + low[1];
+        if (threadIdx.x < L) sum_partial[((int64_t)m * sum_ctas + blockIdx.x) * kMaxLevels + threadIdx.x] = 0.0;
         __syncthreads();
-        for (int l = warp; l < L; l += warps) {  // in a fixed order
+        for (uint32_t c = warp; c <= last; c += warps) {  // in a fixed order
             double e = 0.0;
-            for (int i = lane; i < threads; i += 32) e += column[l * threads + i];
+            for (int i = lane; i < threads; i += 32) e += column[c * threads + i];
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xFFFFFFFFu, e, o);
-            if (lane == 0) sum_partial[((int64_t)m * sum_ctas + blockIdx.x) * kMaxLevels + l] = e;
+            if (lane == 0) sum_partial[((int64_t)m * sum_ctas + blockIdx.x) * kMaxLevels + sh_code[c]] = e;
         }
     }
 }
@@ -919,7 +918,7 @@ int blocks_per_worker(const Workspace& ws, int64_t d, int vec, int threads, int 
 }
 
 size_t s2_smem(int L, bool sums, int threads) {
-    return kBins1 + (size_t)(threads / 32) * (kS2Stage + 1) * 4 + (sums ? (size_t)(L + 1) * threads * sizeof(double) : 0);
+    return (size_t)(kS2Groups + kS2Slots * threads) * 4 + (sums ? (size_t)(L + 1) * threads * sizeof(double) : 0);
 }
 
 size_t digit_smem(int nq, bool cells) {
@@ -1016,8 +1015,8 @@ void launch_sums_candidates(Workspace& ws, const void* g, int64_t d, int M, int6
     const int nb = std::min(blocks_per_worker(ws, d, 4, threads, M, 1), ws.sum_ctas);
     ws.cur_sum_ctas = nb;
     launch_kernel(ws, K_SUMS_CAND, sums ? sums_candidates_kernel<true> : sums_candidates_kernel<false>, dim3(nb, M), threads,
-                  s2_smem(plan.L, sums, threads), s, static_cast<const float*>(g), d, ld, ws.table1, plan.L, ws.sum_partial,
-                  ws.sum_ctas, ws.cand_keys, ws.cand_cap, ws.cand_count, ws.cand_overflow, ws.worker_err, ws.tile_max,
+                  s2_smem(plan.L, sums, threads), s, static_cast<const float*>(g), d, ld, ws.table1, ws.queries,
+                  plan.nq, plan.L, ws.sum_partial, ws.sum_ctas, ws.cand_keys, ws.cand_cap, ws.cand_count, ws.cand_overflow, ws.worker_err, ws.tile_max,
                   emit_tiles_per_worker(d, MLMC_F32), ws.cand_floor, brackets ? ws.bracket_hit : nullptr);
 }
 
