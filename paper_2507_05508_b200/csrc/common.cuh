@@ -386,6 +386,43 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
+// A block's threads stream the 16-byte vectors of `src`, VECS per thread and trip: trips first, first + step, ... below `end`.
+// Three trips are in flight while one is used; a thread copies and reads only its own vectors, so there is no barrier.
+// ring: [4][VECS][THREADS] vectors of shared memory.  (The loop is not unrolled over the slots: the bodies are long, and
+// four copies of one miss the instruction cache.)
+template <int VECS, int THREADS, typename F>
+__device__ __forceinline__ void stream_trips(const uint4* __restrict__ src, int64_t first, int64_t step, int64_t end, uint4* ring, F&& f) {
+    if (first >= end) return;
+    uint4* mine = ring + threadIdx.x;
+    const uint4* from = src + first * (VECS * THREADS) + threadIdx.x;
+    const int64_t ahead = step * (VECS * THREADS);
+    int left = (int)((end - first + step - 1) / step), unasked = left;  // trips to use, trips to ask for
+    auto fetch = [&](int at) {
+        if (unasked > 0) {
+#pragma unroll
+            for (int j = 0; j < VECS; ++j) cp_async_16(mine + at + j * THREADS, from + j * THREADS);
+            from += ahead;
+            --unasked;
+        }
+        cp_async_commit();
+    };
+#pragma unroll
+    for (int i = 0; i < 3; ++i) fetch(i * VECS * THREADS);
+    int at = 0, to = 3 * VECS * THREADS;  // slot in use, slot to fill
+#pragma unroll 1
+    do {
+        fetch(to);
+        cp_async_wait<3>();
+        uint4 q[VECS];
+#pragma unroll
+        for (int j = 0; j < VECS; ++j) q[j] = mine[at + j * THREADS];
+        f(q);
+        to = at;
+        at = at + VECS * THREADS < 4 * VECS * THREADS ? at + VECS * THREADS : 0;
+    } while (--left);
+    cp_async_wait<0>();
+}
+
 // Contiguous range of 16-byte vectors handled by block `bx` of `nb` blocks over a row of d elements.
 __device__ __forceinline__ void block_vector_range(int64_t d, int vec, int bx, int nb, int64_t* v0, int64_t* v1) {
     const int64_t nvec = (d + vec - 1) / vec;
@@ -411,6 +448,14 @@ inline EmitCounts emit_counts(int tiles) {
     n.supers = (n.items + kSuperItems - 1) / kSuperItems;
     n.hypers = (n.supers + kSuperItems - 1) / kSuperItems;
     return n;
+}
+
+// Resident blocks per SM, at least 1.
+template <typename K>
+int resident_blocks(K kernel, int threads, size_t smem) {
+    int n = 0;
+    const bool ok = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, smem) == cudaSuccess;
+    return ok && n >= 1 ? n : 1;
 }
 
 // Brackets one kernel launch: counts it and, when timing is on, records an event pair on the stream.

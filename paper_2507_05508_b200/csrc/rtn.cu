@@ -9,6 +9,9 @@
 // The rounding decides an integer, so its arithmetic is fixed (the same on the host checker): with
 // inv = fl32((2^r - 1) / (2c)) and delta = fl32(2c / (2^r - 1)), t = fl32(v inv), k = t rounded to nearest, ties to
 // even, C = clip(fl32(k delta), -c, c).  Residuals, norms and the scaling by 1/p are fp64.
+#include <algorithm>
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace mlmc {
@@ -73,14 +76,16 @@ __device__ RtnLevel rtn_level(float c, int r) {
 // in a gradient with per-layer scales most entries are small beside it.  The first level that is left has C^{l-1} = 0, so
 // its residual is its value.  The differences and sums are fp64 (a difference of two fp32 values is exact); what bounds the
 // kernel where nothing is skipped is the conversion of one fp32 value to fp64 per entry and level (16 per clock and SM).
-// 8 x 124M fp32 entries, L = 5: 2.29 ms with every entry taken through every level.
+// 8 x 124M fp32 entries, L = 5: 2.29 ms with every entry taken through every level; 1.02 with one trip in flight and one and
+// a half waves of blocks, now 0.87.
 constexpr int kRtnHeld = 8;
 
 template <typename T, int LMAX>
-__global__ void __launch_bounds__(kRtnThreads, LMAX <= 6 ? 3 : 2)
-rtn_stats_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* gmax_bits, RtnSchedule sc, double* partial,
-                 int rtn_ctas, uint32_t* done, DrawPlan pl, int* status, int* worker_err) {
+__global__ void __launch_bounds__(kRtnThreads, LMAX <= 6 ? 4 : 3)
+rtn_stats_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* gmax_bits, const __grid_constant__ RtnSchedule sc, double* partial,
+                 int rtn_ctas, uint32_t* done, const __grid_constant__ DrawPlan pl, int* status, int* worker_err) {
     using Tr = ElemTraits<T>;
+    extern __shared__ __align__(16) uint4 sh_vectors[];  // [4][vectors per trip][kRtnThreads]
     __shared__ double sh_red[LMAX][kRtnThreads / 32];
     __shared__ double sh_delta[kMaxLevels];
     __shared__ RtnLevel sh_lv[kRtnMaxLevels];
@@ -142,7 +147,7 @@ rtn_stats_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t*
     };
     if (c > 0.0f) {
         const T* row = g + (int64_t)m * ld;
-        constexpr int kVecs = kRtnHeld / Tr::kVec;  // 16-byte vectors per lane and trip; the next trip's are in flight
+        constexpr int kVecs = kRtnHeld / Tr::kVec;  // 16-byte vectors per lane and trip
         constexpr int kTrip = kRtnThreads * kVecs;
         const int64_t full_end = d / Tr::kVec;
         const int64_t trips = full_end / kTrip;
@@ -161,20 +166,11 @@ rtn_stats_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t*
                 }
             }
         };
-        uint4 nxt[kVecs];
-        auto load = [&](int64_t trip) {
-            if (trip >= trips) return;
-#pragma unroll
-            for (int j = 0; j < kVecs; ++j)
-                nxt[j] = __ldg(reinterpret_cast<const uint4*>(row) + trip * kTrip + j * kRtnThreads + threadIdx.x);
-        };
-        load(blockIdx.x);
-        for (int64_t trip = blockIdx.x; trip < trips; trip += gridDim.x) {
+        stream_trips<kVecs, kRtnThreads>(reinterpret_cast<const uint4*>(row), blockIdx.x, gridDim.x, trips, sh_vectors, [&](const uint4 (&q)[kVecs]) {
             float v[kRtnHeld];
-            expand(nxt, v);
-            load(trip + gridDim.x);
+            expand(q, v);
             take(v);
-        }
+        });
         if (blockIdx.x == gridDim.x - 1) {  // the rest of the row, fewer than kTrip + 1 vectors, one by one
             for (int64_t i = trips * kTrip * Tr::kVec + threadIdx.x; i < d; i += kRtnThreads) {
                 float v;
@@ -328,19 +324,29 @@ DrawPlan rtn_draw_plan(Workspace& ws, int L, uint64_t seed, uint64_t step, const
     return pl;
 }
 
+namespace {
+template <typename T, int LMAX>
+void launch_rtn_stats_t(Workspace& ws, const T* g, int64_t d, int M, int64_t ld, const RtnSchedule& sc, const DrawPlan& plan,
+                        cudaStream_t s) {
+    constexpr size_t smem = (size_t)4 * kRtnThreads * kRtnHeld * sizeof(T);
+    static const int resident = resident_blocks(rtn_stats_kernel<T, LMAX>, kRtnThreads, smem);
+    // whole waves (a partial last one costs a full one), four of them: how much a block skips differs (one: 910 us, two: 897,
+    // four: 866 for 8 x 124M entries)
+    const int nb = std::min(rtn_blocks(ws, d, ElemTraits<T>::kVec, M, 4 * resident), ws.rtn_ctas);
+    launch_kernel(ws, K_RTN_STATS, rtn_stats_kernel<T, LMAX>, dim3(nb, M), kRtnThreads, smem, s, g, d, ld, ws.gmax_bits, sc,
+                  ws.rtn_partial, ws.rtn_ctas, ws.done, plan, ws.status, ws.worker_err);
+}
+}  // namespace
+
 void launch_rtn_stats(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* r, int L,
                       const DrawPlan& plan, cudaStream_t s) {
     const RtnSchedule sc = make_rtn_schedule(r, L);
-    int nb = rtn_blocks(ws, d, dtype == MLMC_BF16 ? 8 : 4, M, L <= 6 ? 6 : 4);  // two waves of the resident blocks
-    if (nb > ws.rtn_ctas) nb = ws.rtn_ctas;
-    auto go = [&](auto kernel, auto* row) {
-        launch_kernel(ws, K_RTN_STATS, kernel, dim3(nb, M), kRtnThreads, 0, s, row, d, ld, ws.gmax_bits, sc, ws.rtn_partial,
-                      ws.rtn_ctas, ws.done, plan, ws.status, ws.worker_err);
+    auto go = [&](auto* row) {
+        if (L <= 6) launch_rtn_stats_t<std::remove_const_t<std::remove_pointer_t<decltype(row)>>, 6>(ws, row, d, M, ld, sc, plan, s);
+        else launch_rtn_stats_t<std::remove_const_t<std::remove_pointer_t<decltype(row)>>, kRtnMaxLevels>(ws, row, d, M, ld, sc, plan, s);
     };
-    if (dtype == MLMC_BF16)
-        go(L <= 6 ? rtn_stats_kernel<bf16_t, 6> : rtn_stats_kernel<bf16_t, kRtnMaxLevels>, static_cast<const bf16_t*>(g));
-    else
-        go(L <= 6 ? rtn_stats_kernel<float, 6> : rtn_stats_kernel<float, kRtnMaxLevels>, static_cast<const float*>(g));
+    if (dtype == MLMC_BF16) go(static_cast<const bf16_t*>(g));
+    else go(static_cast<const float*>(g));
 }
 
 void launch_rtn_emit(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* r, int L,
