@@ -192,13 +192,14 @@ int mlmc_create(mlmc_ctx** out, int device, int64_t d_max, int M_max, int L_max)
     cudaDeviceProp prop;
     if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) return MLMC_ERR_CUDA;
     if (configure_select_kernels() != MLMC_OK || configure_emit_kernels() != MLMC_OK ||
-        configure_bit_kernels() != MLMC_OK || configure_float_kernels() != MLMC_OK || configure_segment_kernels() != MLMC_OK)
+        configure_float_kernels() != MLMC_OK || configure_segment_kernels() != MLMC_OK)
         return MLMC_ERR_CUDA;
 
     mlmc_ctx* ctx = new (std::nothrow) mlmc_ctx();
     if (!ctx) return MLMC_ERR_NOMEM;
     Workspace& ws = ctx->ws;
-    if (configure_cluster_kernels(ws) != MLMC_OK) {
+    for (int& n : ws.dense_fit) n = M_max;
+    if (configure_cluster_kernels(ws) != MLMC_OK || configure_bit_kernels(ws) != MLMC_OK || configure_rtn_kernels(ws) != MLMC_OK) {
         delete ctx;
         return MLMC_ERR_CUDA;
     }
@@ -361,7 +362,7 @@ static const char* const kKernelNames[] = {
     "begin", "uniforms", "hist1", "resolve1", "sums_candidates", "cand_pass2", "cand_pass3", "band_header", "copy_probs", "emit",
     "agg_offsets", "aggregate_topk", "absmax", "bit_stats", "bit_pack", "aggregate_bitwise", "tile_list", "band_count",
     "float_pack", "aggregate_floatbits", "rtn_stats", "rtn_emit", "aggregate_dense", "segment_resolve",
-    "segment_sweep", "segment_buckets", "segment_norms", "segment_draw", "cluster_topk"};
+    "segment_sweep", "segment_buckets", "segment_norms", "segment_draw", "cluster_topk", "cluster_bitwise", "cluster_rtn"};
 static_assert(sizeof(kKernelNames) / sizeof(kKernelNames[0]) == K_COUNT, "a name for every kernel id");
 
 int mlmc_kernel_count(void) { return K_COUNT; }
@@ -520,6 +521,7 @@ int mlmc_compress_bitwise(mlmc_ctx* ctx, const void* g, int dtype, int64_t d, in
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     set_call_size(ws, d, M, dtype == MLMC_BF16 ? 2 : 4);
     const DrawPlan plan = bit_draw_plan(ws, b32, L, seed, step, out);
+    if (launch_bit_cluster(ws, g, dtype, d, M, ld, b32, L, plan, p ? pn : nullptr, *out, s)) return finish(cudaGetLastError());
     launch_absmax(ws, g, dtype, d, M, ld, plan, p ? pn : nullptr, s);
     if (!p) launch_bit_stats(ws, g, dtype, d, M, ld, b32, L, plan, s);
     launch_bit_pack(ws, g, dtype, d, M, ld, b32, L, *out, s);
@@ -660,6 +662,7 @@ int mlmc_compress_rtn(mlmc_ctx* ctx, const void* g, int dtype, int64_t d, int M,
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     set_call_size(ws, d, M, dtype == MLMC_BF16 ? 2 : 4);
     const DrawPlan plan = rtn_draw_plan(ws, L, seed, step, out);
+    if (launch_rtn_cluster(ws, g, dtype, d, M, ld, r32, L, plan, p ? pn : nullptr, *out, s)) return finish(cudaGetLastError());
     launch_absmax(ws, g, dtype, d, M, ld, plan, p ? pn : nullptr, s);  // c = max |g|, and the NaN / Inf check
     if (!p) launch_rtn_stats(ws, g, dtype, d, M, ld, r32, L, plan, s);
     launch_rtn_emit(ws, g, dtype, d, M, ld, r32, L, *out, s);

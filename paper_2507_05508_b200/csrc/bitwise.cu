@@ -7,7 +7,7 @@
 //   f_l = (q >> (B - b_l)) & (2^{w_l} - 1),  w_l = b_l - b_{l-1},  worth  sign f_l 2^{-b_l} gmax,
 // sent as one sign plane and w_l magnitude planes.  Adaptive probabilities (Lemma 3.4) use the exact
 // integer field energies S_l = sum_i f_l^2:  Delta_l = gmax 2^{-b_l} sqrt(S_l).
-#include "bitplanes.cuh"
+#include "dense_cluster.cuh"
 
 namespace mlmc {
 
@@ -34,30 +34,36 @@ struct BitSchedule {
 // "Computation of elementary functions on the IBM RISC System/6000 processor", 1990: with the reciprocal correctly rounded
 // and a quotient within one ulp, one step of remainder and correction rounds like the division).  The truncation is the
 // addition of 2^23 with rounding toward zero.  Seven fp32 operations; the fp64 product and conversions used before took
-// two slots of the conversion unit.  The remainders must not underflow and the reciprocal must be normal; outside
-// 2^-60 <= gmax <= 2^100 the entry is divided.
+// two slots of the conversion unit.  The remainders must not underflow and the reciprocal must be normal: where gmax lies
+// outside [2^-60, 2^100], numerator and divisor are moved by a power of two.  (That is exact, except for numerators whose
+// quotient lies far below 2^-23: their code is 0 either way.)
 struct Quantiser {
-    float gmax, inv;
-    bool steps;
+    float gmax, inv, move;
     __device__ __forceinline__ explicit Quantiser(float g) {
         gmax = g > 0.0f ? g : 1.0f;
+        move = gmax < 0x1.0p-60f ? 0x1.0p100f : gmax > 0x1.0p100f ? 0x1.0p-64f : 1.0f;
+        gmax *= move;
         inv = __frcp_rn(gmax);
-        steps = gmax >= 0x1.0p-60f && gmax <= 0x1.0p100f;
     }
-    // the code in the low 23 bits, the bits of 2^23 above
-    __device__ __forceinline__ uint32_t code_bits(float mag /* |g| */, float scale /* 2^b, b <= 23 */) const {
-        float e;
-        if (steps) {
-            e = __fmul_rn(mag, inv);
-            e = __fmaf_rn(__fmaf_rn(-e, gmax, mag), inv, e);
-            e = __fmaf_rn(__fmaf_rn(-e, gmax, mag), inv, e);
-        } else {
-            e = __fdiv_rn(mag, gmax);
+    // The codes of N entries at b bits (scale 2^b, b <= 23): in the low 23 bits, the bits of 2^23 above.
+    template <int N>
+    __device__ __forceinline__ void codes(const float (&v)[N], float scale, uint32_t (&q)[N]) const {
+        float x[N];
+#pragma unroll
+        for (int i = 0; i < N; ++i) x[i] = fabsf(v[i]);
+        if (move != 1.0f) {
+#pragma unroll
+            for (int i = 0; i < N; ++i) x[i] *= move;
         }
-        // e = 1 has no b-bit fraction: the largest e below it has the code 2^b - 1
-        return __float_as_uint(__fmaf_rz(fminf(e, 0x1.fffffep-1f), scale, 8388608.0f));
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            float e = __fmul_rn(x[i], inv);
+            e = __fmaf_rn(__fmaf_rn(-e, gmax, x[i]), inv, e);
+            e = __fmaf_rn(__fmaf_rn(-e, gmax, x[i]), inv, e);
+            // e = 1 has no b-bit fraction: the largest e below it has the code 2^b - 1
+            q[i] = __float_as_uint(__fmaf_rz(fminf(e, 0x1.fffffep-1f), scale, 8388608.0f));
+        }
     }
-    __device__ __forceinline__ uint32_t code(float mag, float scale) const { return code_bits(mag, scale) - 0x4B000000u; }
 };
 
 // An entry below gmax 2^-b (1 - 2^-20) has fl32(|g| / gmax) < 2^-b: its code at b bits is 0.
@@ -148,8 +154,7 @@ __device__ __forceinline__ void take_fields(const float (&v)[kBitHeld], const Qu
     if constexpr (sizeof(Acc) == 4) {
         uint32_t q[kBitHeld], w[kBitHeld / 4];
         int run = -1;
-#pragma unroll
-        for (int e = 0; e < kBitHeld; ++e) q[e] = qz.code_bits(fabsf(v[e]), scale);
+        qz.codes(v, scale, q);
 #pragma unroll
         for (int l = 0; l < LMAX; ++l) {
             if (l >= sc.L) break;
@@ -169,9 +174,10 @@ __device__ __forceinline__ void take_fields(const float (&v)[kBitHeld], const Qu
         }
     } else {
         uint32_t q[kBitHeld], prev[kBitHeld];
+        qz.codes(v, scale, q);
 #pragma unroll
         for (int e = 0; e < kBitHeld; ++e) {
-            q[e] = qz.code(fabsf(v[e]), scale);
+            q[e] -= 0x4B000000u;
             prev[e] = 0u;
         }
 #pragma unroll
@@ -337,8 +343,7 @@ __device__ __forceinline__ void pack_group(const uint32_t* slot, const Quantiser
         return;
     }
     uint32_t q[32];
-#pragma unroll
-    for (int t = 0; t < 32; ++t) q[t] = qz.code(fabsf(x[t]), scale);
+    qz.codes(x, scale, q);  // the bits above a field leave with the shifts, or are planes that are not written
     if (w < 6) {
         for (int j = 1; j <= w; ++j) {
             const int up = 31 - (w - j);
@@ -385,6 +390,74 @@ bit_pack_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* 
         __syncwarp();  // everyone is done with this slot before the copy after next lands in it
     }
     cp_async_wait<0>();
+}
+
+// ---- short rows: all of the above in one launch (dense_cluster.cuh).  Fields of at most 8 bits, at most kDenseLevels levels.
+// 6 x 400,003 bf16 entries, six levels, adaptive: 24 us for the three kernels above, 16 for this one.
+constexpr int kBitDenseWarps = 32;
+
+template <typename T>
+__global__ void __launch_bounds__(kBitDenseWarps * 32, 1)
+bit_cluster_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid_constant__ BitSchedule sc,
+                   const __grid_constant__ DrawPlan pl, const __grid_constant__ DrawnLevels drawn, int adaptive, int per_block,
+                   uint32_t* __restrict__ planes, int w_max, int64_t words, int* status, int* worker_err) {
+    using Tr = ElemTraits<T>;
+    extern __shared__ __align__(16) uint32_t sh_slots[];
+    __shared__ DenseShared<kBitDenseWarps, unsigned long long> sh;
+    __shared__ int sh_below[kDenseLevels];
+    cg::cluster_group cluster = cg::this_cluster();
+    pdl_enter();
+    const int rank = (int)cluster.block_rank(), m = blockIdx.x / (int)cluster.num_blocks();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t ngroups = (words + 31) / 32, g0 = (int64_t)rank * per_block;
+    const int n = (int)max((int64_t)0, min((int64_t)per_block, ngroups - g0));
+    const uint32_t top = dense_load<T>(cluster, g + (int64_t)m * ld, d, g0, n, sh_slots, sh);
+    const bool bad = top >= Tr::kInfKey, first = rank == 0;
+    if (first && threadIdx.x == 0) {
+        worker_err[m] = bad ? MLMC_ERR_NONFINITE : 0;
+        if (bad) {
+            set_status(status, MLMC_ERR_NONFINITE);
+            void_header(pl, m);
+        }
+    }
+    if (bad) return;  // the same in every block
+    const float gmax = __uint_as_float(Tr::kVec == 8 ? top << 16 : top);
+    const Quantiser qz(gmax);
+    double delta = 0.0;
+    if (adaptive) {
+        if (threadIdx.x < kDenseLevels) sh_below[threadIdx.x] = zero_code_below(gmax, sc.bits[min((int)threadIdx.x, sc.L - 1)]);
+        __syncthreads();
+        uint32_t acc[kDenseLevels];
+        int zero_below[kDenseLevels];
+#pragma unroll
+        for (int l = 0; l < kDenseLevels; ++l) {
+            acc[l] = 0u;
+            zero_below[l] = sh_below[l];
+        }
+        if (gmax > 0.0f) {
+            constexpr int kVecs = kBitHeld / Tr::kVec;  // a warp takes a quarter of a group
+#pragma unroll 1
+            for (int u = warp; u < 4 * n; u += kBitDenseWarps) {
+                const uint4* x = reinterpret_cast<const uint4*>(sh_slots + (u >> 2) * kGroupSlot<T>) + (u & 3) * kVecs * 32 + lane;
+                uint4 q[kVecs];
+#pragma unroll
+                for (int j = 0; j < kVecs; ++j) q[j] = x[j * 32];
+                float v[kBitHeld];
+                expand_vectors<T>(q, v);
+                take_fields<T, kDenseLevels, uint32_t>(v, qz, (float)(1u << sc.B), zero_below, sc, acc);
+            }
+        }
+        const unsigned long long S = dense_sums(cluster, acc, sh);
+        if (threadIdx.x < sc.L) delta = (double)gmax * ldexp(1.0, -sc.bits[threadIdx.x]) * sqrt((double)S);
+    }
+    double p;
+    const int level = dense_level(pl, drawn, adaptive, m, first, delta, gmax, sh, &p, status, worker_err);
+    if (sc.width[level] > w_max) return;  // reported with the header
+    const float scale = (float)(1u << sc.bits[level]);
+    const int zero_below = zero_code_below(gmax, sc.bits[level]);
+    uint32_t* out = planes + (int64_t)m * (1 + w_max) * words;
+    for (int i = warp; i < n; i += kBitDenseWarps)
+        pack_group<T>(sh_slots + i * kGroupSlot<T>, qz, scale, zero_below, sc.width[level], (g0 + i) * 32 + lane, words, out);
 }
 
 // ---- server average of bit-plane messages: thread = one word (32 entries), staged through shared memory
@@ -530,8 +603,9 @@ size_t bit_pack_smem(size_t elem) { return (kBitThreads / 32) * 2 * 1024 * elem;
 
 }  // namespace
 
-int configure_bit_kernels() {
-    const bool ok = cudaFuncSetAttribute(bit_pack_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+int configure_bit_kernels(Workspace& ws) {
+    const bool ok = configure_dense_cluster(bit_cluster_kernel<float>, kBitDenseWarps * 32, ws) && configure_dense_cluster(bit_cluster_kernel<bf16_t>, kBitDenseWarps * 32, ws) &&
+                    cudaFuncSetAttribute(bit_pack_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)bit_pack_smem(4)) == cudaSuccess;
     return ok ? MLMC_OK : MLMC_ERR_CUDA;
 }
@@ -593,6 +667,26 @@ void launch_bit_stats(Workspace& ws, const void* g, int dtype, int64_t d, int M,
         if (narrow) launch_bit_stats_t<float, uint32_t>(ws, static_cast<const float*>(g), d, M, ld, sc, nb, plan, s);
         else launch_bit_stats_t<float, unsigned long long>(ws, static_cast<const float*>(g), d, M, ld, sc, nb, plan, s);
     }
+}
+
+// The whole message of short rows in one launch; false: the row is not for it.
+bool launch_bit_cluster(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* b, int L,
+                        const DrawPlan& plan, const double* p, const mlmc_bit_msgs& out, cudaStream_t s) {
+    const BitSchedule sc = make_schedule(b, L);
+    int w_top = 0;
+    for (int l = 0; l < L; ++l) w_top = std::max(w_top, sc.width[l]);
+    const int cl = dense_cluster_blocks(ws, d, M);
+    if (cl == 0 || (!p && (L > kDenseLevels || w_top > 8))) return false;
+    const DrawnLevels drawn = draw_levels(p, L, plan.seed, plan.step, M);
+    const int64_t words = (d + 31) / 32;
+    const int per = (int)(((words + 31) / 32 + cl - 1) / cl);
+    auto go = [&](auto kernel, auto* row, size_t elem) {
+        launch_kernel_cluster(ws, K_BIT_CLUSTER, cl, kernel, dim3(M * cl), kBitDenseWarps * 32, per * 1024 * elem, s, row, d, ld, sc, plan,
+                              drawn, p ? 0 : 1, per, out.planes, out.w_max, words, ws.status, ws.worker_err);
+    };
+    if (dtype == MLMC_BF16) go(bit_cluster_kernel<bf16_t>, static_cast<const bf16_t*>(g), 2);
+    else go(bit_cluster_kernel<float>, static_cast<const float*>(g), 4);
+    return true;
 }
 
 template <typename T>

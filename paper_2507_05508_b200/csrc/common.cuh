@@ -59,7 +59,8 @@ struct EmitParams {
 enum KernelId {
     K_BEGIN = 0, K_UNIFORMS, K_HIST1, K_RESOLVE1, K_SUMS_CAND, K_CAND2, K_CAND3, K_BAND_HEADER, K_COPY_PROBS, K_EMIT, K_AGG_OFFSETS,
     K_AGG_TOPK, K_ABSMAX, K_BIT_STATS, K_BIT_PACK, K_AGG_BIT, K_TILE_LIST, K_BAND_COUNT, K_FLOAT_PACK, K_AGG_FLOAT,
-    K_RTN_STATS, K_RTN_EMIT, K_AGG_DENSE, K_SEG_RESOLVE, K_SEG_SWEEP, K_SEG_BUCKETS, K_SEG_NORMS, K_SEG_DRAW, K_CLUSTER_TOPK, K_COUNT
+    K_RTN_STATS, K_RTN_EMIT, K_AGG_DENSE, K_SEG_RESOLVE, K_SEG_SWEEP, K_SEG_BUCKETS, K_SEG_NORMS, K_SEG_DRAW, K_CLUSTER_TOPK,
+    K_BIT_CLUSTER, K_RTN_CLUSTER, K_COUNT
 };
 
 // Level probabilities handed to a kernel by value.
@@ -95,6 +96,7 @@ struct Workspace {
     int sm_count;
     int64_t launches;
     int cluster_most;            // largest thread-block cluster of the short-row kernels (0: none)
+    int dense_fit[5];            // clusters of 1, 2, .. 16 blocks of the short-row dense kernels that run at a time
     bool long_sweeps;            // this call's sweeps are long enough to be launched without overlap (see launch_kernel)
     // device memory
     int* status;                 // sticky status word
@@ -570,7 +572,7 @@ void launch_emit(Workspace& ws, const void* g, int dtype, int64_t d, int M, int6
                  cudaStream_t s);
 void launch_aggregate_topk(Workspace& ws, const mlmc_topk_msgs& msgs, int M, int64_t d, float* out, cudaStream_t s);
 // bitwise.cu
-int configure_bit_kernels();
+int configure_bit_kernels(Workspace& ws);
 // Largest magnitude of every worker and the NaN / Inf check; with `p` (given probabilities) also the draw and the header.
 void launch_absmax(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const DrawPlan& plan, const double* p,
                    cudaStream_t s);
@@ -578,6 +580,8 @@ DrawPlan bit_draw_plan(Workspace& ws, const int32_t* b, int L, uint64_t seed, ui
 // Adaptive: field energies of every level, probabilities, draw and header.
 void launch_bit_stats(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* b, int L,
                       const DrawPlan& plan, cudaStream_t s);
+bool launch_bit_cluster(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* b, int L,
+                        const DrawPlan& plan, const double* p, const mlmc_bit_msgs& out, cudaStream_t s);
 void launch_bit_pack(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* b, int L,
                      const mlmc_bit_msgs& out, cudaStream_t s);
 void launch_aggregate_bitwise(Workspace& ws, const mlmc_bit_msgs& msgs, const int32_t* b, int L, int M, int64_t d,
@@ -594,6 +598,9 @@ DrawPlan rtn_draw_plan(Workspace& ws, int L, uint64_t seed, uint64_t step, const
 // Adaptive: residual energies of every level, probabilities, draw and header.
 void launch_rtn_stats(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* r, int L,
                       const DrawPlan& plan, cudaStream_t s);
+int configure_rtn_kernels(Workspace& ws);
+bool launch_rtn_cluster(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* r, int L,
+                        const DrawPlan& plan, const double* p, const mlmc_rtn_msgs& out, cudaStream_t s);
 void launch_rtn_emit(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* r, int L,
                      const mlmc_rtn_msgs& out, cudaStream_t s);
 void launch_aggregate_dense(Workspace& ws, const float* val, const int32_t* level, int M, int64_t d, int64_t ldv,

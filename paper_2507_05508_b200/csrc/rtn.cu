@@ -12,7 +12,7 @@
 #include <algorithm>
 #include <type_traits>
 
-#include "common.cuh"
+#include "dense_cluster.cuh"
 
 namespace mlmc {
 
@@ -80,6 +80,96 @@ __device__ RtnLevel rtn_level(float c, int r) {
 // a half waves of blocks, now 0.87.
 constexpr int kRtnHeld = 8;
 
+template <typename T>
+__device__ __forceinline__ void rtn_expand(const uint4* q, float (&v)[kRtnHeld]) {
+#pragma unroll
+    for (int j = 0; j < kRtnHeld / ElemTraits<T>::kVec; ++j) {
+        const uint32_t w[4] = {q[j].x, q[j].y, q[j].z, q[j].w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if constexpr (ElemTraits<T>::kVec == 4) {
+                v[4 * j + i] = __uint_as_float(w[i]);
+            } else {
+                v[8 * j + 2 * i] = __uint_as_float(w[i] << 16);
+                v[8 * j + 2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
+            }
+        }
+    }
+}
+
+// One trip of a warp: kRtnHeld entries per lane.
+template <int LMAX>
+__device__ __forceinline__ void take_levels(const float (&v)[kRtnHeld], float c, const RtnLevel* levels, int L, double (&acc)[LMAX]) {
+    int mx = 0;
+#pragma unroll
+    for (int e = 0; e < kRtnHeld; ++e) mx = max(mx, __float_as_int(v[e]) & 0x7FFFFFFF);
+    mx = __reduce_max_sync(0xFFFFFFFFu, mx);
+    double prev[kRtnHeld];  // C^{l-1}
+    bool first = true;      // C^{l-1} = 0 for every entry of the warp (warp-uniform)
+#pragma unroll
+    for (int l = 0; l < LMAX; ++l) {
+        if (l > L - 1) break;
+        if (l == L - 1) {  // the identity
+            if (first) {
+#pragma unroll
+                for (int e = 0; e < kRtnHeld; ++e) prev[e] = 0.0;
+            }
+            double odd = 0.0;  // two chains of additions
+#pragma unroll
+            for (int e = 0; e < kRtnHeld; ++e) {
+                const double res = (double)v[e] - prev[e];
+                if (e & 1) odd = fma(res, res, odd);
+                else acc[l] = fma(res, res, acc[l]);
+            }
+            acc[l] += odd;
+            break;
+        }
+        const RtnLevel lv = levels[l];
+        if (mx <= lv.zero_upto) continue;  // the grids get finer: once a level is not skipped, none after it is
+        float x[kRtnHeld];
+#pragma unroll
+        for (int e = 0; e < kRtnHeld; ++e) {
+            const float k = __fadd_rn(__fadd_rn(__fmul_rn(v[e], lv.inv), 12582912.0f), -12582912.0f);
+            x[e] = __fmul_rn(k, lv.delta);
+        }
+        if (mx > lv.free_upto) {
+#pragma unroll
+            for (int e = 0; e < kRtnHeld; ++e) x[e] = fminf(fmaxf(x[e], -c), c);
+        }
+        double odd = 0.0;
+        if (first) {
+#pragma unroll
+            for (int e = 0; e < kRtnHeld; ++e) {
+                prev[e] = (double)x[e];
+                if (e & 1) odd = fma(prev[e], prev[e], odd);
+                else acc[l] = fma(prev[e], prev[e], acc[l]);
+            }
+            first = false;
+        } else {
+#pragma unroll
+            for (int e = 0; e < kRtnHeld; ++e) {
+                const double cur = (double)x[e], res = cur - prev[e];
+                if (e & 1) odd = fma(res, res, odd);
+                else acc[l] = fma(res, res, acc[l]);
+                prev[e] = cur;
+            }
+        }
+        acc[l] += odd;
+    }
+}
+
+template <int LMAX>
+__device__ __forceinline__ void take_entry(float v, float c, const RtnLevel* levels, int L, double (&acc)[LMAX]) {
+    double prev = 0.0;
+#pragma unroll
+    for (int l = 0; l < LMAX; ++l) {
+        if (l > L - 1) break;
+        const double cur = (l < L - 1) ? (double)rtn_value(v, c, {levels[l].inv, levels[l].delta}) : (double)v;
+        acc[l] = fma(cur - prev, cur - prev, acc[l]);
+        prev = cur;
+    }
+}
+
 template <typename T, int LMAX>
 __global__ void __launch_bounds__(kRtnThreads, LMAX <= 6 ? 4 : 3)
 rtn_stats_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* gmax_bits, const __grid_constant__ RtnSchedule sc, double* partial,
@@ -98,92 +188,23 @@ rtn_stats_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t*
     double acc[LMAX];
 #pragma unroll
     for (int l = 0; l < LMAX; ++l) acc[l] = 0.0;
-    auto take = [&](const float (&v)[kRtnHeld]) {
-        int mx = 0;
-#pragma unroll
-        for (int e = 0; e < kRtnHeld; ++e) mx = max(mx, __float_as_int(v[e]) & 0x7FFFFFFF);
-        mx = __reduce_max_sync(0xFFFFFFFFu, mx);
-        double prev[kRtnHeld];  // C^{l-1}
-        bool first = true;      // C^{l-1} = 0 for every entry of the warp (warp-uniform)
-#pragma unroll
-        for (int l = 0; l < LMAX; ++l) {
-            if (l > sc.L - 1) break;
-            if (l == sc.L - 1) {  // the identity
-#pragma unroll
-                for (int e = 0; e < kRtnHeld; ++e) {
-                    const double res = first ? (double)v[e] : (double)v[e] - prev[e];
-                    acc[l] = fma(res, res, acc[l]);
-                }
-                break;
-            }
-            const RtnLevel lv = sh_lv[l];
-            if (mx <= lv.zero_upto) continue;  // the grids get finer: once a level is not skipped, none after it is
-            float x[kRtnHeld];
-#pragma unroll
-            for (int e = 0; e < kRtnHeld; ++e) {
-                const float k = __fadd_rn(__fadd_rn(__fmul_rn(v[e], lv.inv), 12582912.0f), -12582912.0f);
-                x[e] = __fmul_rn(k, lv.delta);
-            }
-            if (mx > lv.free_upto) {
-#pragma unroll
-                for (int e = 0; e < kRtnHeld; ++e) x[e] = fminf(fmaxf(x[e], -c), c);
-            }
-            if (first) {
-#pragma unroll
-                for (int e = 0; e < kRtnHeld; ++e) {
-                    prev[e] = (double)x[e];
-                    acc[l] = fma(prev[e], prev[e], acc[l]);
-                }
-                first = false;
-            } else {
-#pragma unroll
-                for (int e = 0; e < kRtnHeld; ++e) {
-                    const double cur = (double)x[e], res = cur - prev[e];
-                    acc[l] = fma(res, res, acc[l]);
-                    prev[e] = cur;
-                }
-            }
-        }
-    };
     if (c > 0.0f) {
         const T* row = g + (int64_t)m * ld;
         constexpr int kVecs = kRtnHeld / Tr::kVec;  // 16-byte vectors per lane and trip
         constexpr int kTrip = kRtnThreads * kVecs;
         const int64_t full_end = d / Tr::kVec;
         const int64_t trips = full_end / kTrip;
-        auto expand = [&](const uint4 (&q)[kVecs], float (&v)[kRtnHeld]) {
-#pragma unroll
-            for (int j = 0; j < kVecs; ++j) {
-                const uint32_t w[4] = {q[j].x, q[j].y, q[j].z, q[j].w};
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    if constexpr (Tr::kVec == 4) {
-                        v[4 * j + i] = __uint_as_float(w[i]);
-                    } else {
-                        v[8 * j + 2 * i] = __uint_as_float(w[i] << 16);
-                        v[8 * j + 2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
-                    }
-                }
-            }
-        };
         stream_trips<kVecs, kRtnThreads>(reinterpret_cast<const uint4*>(row), blockIdx.x, gridDim.x, trips, sh_vectors, [&](const uint4 (&q)[kVecs]) {
             float v[kRtnHeld];
-            expand(q, v);
-            take(v);
+            rtn_expand<T>(q, v);
+            take_levels<LMAX>(v, c, sh_lv, sc.L, acc);
         });
         if (blockIdx.x == gridDim.x - 1) {  // the rest of the row, fewer than kTrip + 1 vectors, one by one
             for (int64_t i = trips * kTrip * Tr::kVec + threadIdx.x; i < d; i += kRtnThreads) {
                 float v;
                 if constexpr (Tr::kVec == 4) v = reinterpret_cast<const float*>(row)[i];
                 else v = __uint_as_float((uint32_t)reinterpret_cast<const uint16_t*>(row)[i] << 16);
-                double prev = 0.0;
-#pragma unroll
-                for (int l = 0; l < LMAX; ++l) {
-                    if (l > sc.L - 1) break;
-                    const double cur = (l < sc.L - 1) ? (double)rtn_value(v, c, {sh_lv[l].inv, sh_lv[l].delta}) : (double)v;
-                    acc[l] = fma(cur - prev, cur - prev, acc[l]);
-                    prev = cur;
-                }
+                take_entry<LMAX>(v, c, sh_lv, sc.L, acc);
             }
         }
     }
@@ -217,6 +238,37 @@ rtn_stats_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t*
     finish_levels(pl, m, sh_delta, c, status, worker_err);
 }
 
+// val_i of the drawn level's message.
+template <typename T>
+struct Residual {
+    double inv_p;
+    float c;
+    bool top, first;
+    RtnGrid hi, lo;
+    __device__ __forceinline__ Residual(float c_, const RtnSchedule& sc, int level, double p)
+        : inv_p(p > 0.0 ? 1.0 / p : 0.0), c(c_), top(level == sc.L - 1), first(level == 0) {
+        hi = rtn_grid(c > 0.0f ? c : 1.0f, top ? 1 : sc.r[level]);
+        lo = rtn_grid(c > 0.0f ? c : 1.0f, first ? 1 : sc.r[level - 1]);
+    }
+    __device__ __forceinline__ float operator()(uint32_t bits) const {
+        const float v = ElemTraits<T>::value(bits);
+        if (!(c > 0.0f)) return 0.0f;
+        const double h = top ? (double)v : (double)rtn_value(v, c, hi);
+        const double l = first ? 0.0 : (double)rtn_value(v, c, lo);
+        return (float)((h - l) * inv_p);
+    }
+    __device__ __forceinline__ void vector(const uint4& q, float* __restrict__ out) const {  // a vector's entries, out 16-byte aligned
+        if constexpr (sizeof(T) == 4) {
+            reinterpret_cast<float4*>(out)[0] = make_float4((*this)(q.x), (*this)(q.y), (*this)(q.z), (*this)(q.w));
+        } else {
+            reinterpret_cast<float4*>(out)[0] =
+                make_float4((*this)(q.x & 0xFFFFu), (*this)(q.x >> 16), (*this)(q.y & 0xFFFFu), (*this)(q.y >> 16));
+            reinterpret_cast<float4*>(out)[1] =
+                make_float4((*this)(q.z & 0xFFFFu), (*this)(q.z >> 16), (*this)(q.w & 0xFFFFu), (*this)(q.w >> 16));
+        }
+    }
+};
+
 // The dense message of the drawn level: val_i = (C^l - C^{l-1})_i / p_l, rounded to fp32 once.
 template <typename T>
 __global__ void __launch_bounds__(kRtnThreads)
@@ -228,36 +280,112 @@ rtn_emit_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* 
     const int level = bit_level[m];
     if (level < 0) return;
     const float c = __uint_as_float(gmax_bits[m]);
-    const double p = p_all[m * kMaxLevels + level];
-    const double inv_p = p > 0.0 ? 1.0 / p : 0.0;
-    const bool top = level == sc.L - 1, first = level == 0;
-    const RtnGrid g_hi = rtn_grid(c > 0.0f ? c : 1.0f, top ? 1 : sc.r[level]);
-    const RtnGrid g_lo = rtn_grid(c > 0.0f ? c : 1.0f, first ? 1 : sc.r[level - 1]);
+    const Residual<T> residual(c, sc, level, p_all[m * kMaxLevels + level]);
     const T* row = g + (int64_t)m * ld;
     float* out = val + (int64_t)m * ldv;
-    auto residual = [&](uint32_t bits) -> float {
-        const float v = Tr::value(bits);
-        if (!(c > 0.0f)) return 0.0f;
-        const double hi = top ? (double)v : (double)rtn_value(v, c, g_hi);
-        const double lo = first ? 0.0 : (double)rtn_value(v, c, g_lo);
-        return (float)((hi - lo) * inv_p);
-    };
-    const int64_t nvec = (d + Tr::kVec - 1) / Tr::kVec;
-    const bool vec_ok = (ldv % 4 == 0);
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < nvec; v += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t base = v * Tr::kVec;
-        if (base + Tr::kVec <= d && vec_ok) {
-            const uint4 q = __ldg(reinterpret_cast<const uint4*>(row) + v);
-            if constexpr (Tr::kVec == 4) {
-                reinterpret_cast<float4*>(out + base)[0] = make_float4(residual(q.x), residual(q.y), residual(q.z), residual(q.w));
-            } else {
-                reinterpret_cast<float4*>(out + base)[0] =
-                    make_float4(residual(q.x & 0xFFFFu), residual(q.x >> 16), residual(q.y & 0xFFFFu), residual(q.y >> 16));
-                reinterpret_cast<float4*>(out + base)[1] =
-                    make_float4(residual(q.z & 0xFFFFu), residual(q.z >> 16), residual(q.w & 0xFFFFu), residual(q.w >> 16));
-            }
+    // Chunks of kBatch vectors per thread, all in flight before the first is used.
+    constexpr int kBatch = 4;
+    const int64_t nvec = (d + Tr::kVec - 1) / Tr::kVec, full_end = (ldv % 4 == 0) ? d / Tr::kVec : 0;
+    for (int64_t base = (int64_t)blockIdx.x * kBatch * kRtnThreads; base < nvec; base += (int64_t)gridDim.x * kBatch * kRtnThreads) {
+        const int64_t v = base + threadIdx.x;
+        if (base + kBatch * kRtnThreads <= full_end) {
+            uint4 q[kBatch];
+#pragma unroll
+            for (int j = 0; j < kBatch; ++j) q[j] = __ldg(reinterpret_cast<const uint4*>(row) + v + j * kRtnThreads);
+#pragma unroll
+            for (int j = 0; j < kBatch; ++j) residual.vector(q[j], out + (v + j * kRtnThreads) * Tr::kVec);
         } else {
-            for_each_in_vector<T>(row, v, d, [&](int64_t i, uint32_t bits) { out[i] = residual(bits); });
+            for (int64_t u = v; u < min(nvec, base + kBatch * kRtnThreads); u += kRtnThreads) {
+                if (u < full_end) residual.vector(__ldg(reinterpret_cast<const uint4*>(row) + u), out + u * Tr::kVec);
+                else for_each_in_vector<T>(row, u, d, [&](int64_t i, uint32_t bits) { out[i] = residual(bits); });
+            }
+        }
+    }
+}
+
+// Short rows: all of the above in one launch (dense_cluster.cuh); with adaptive probabilities at most kRtnDenseLevels levels.
+// 4 x 50,000 bf16 entries, adaptive: 20.5 us for the three kernels above, 15.5 for this one.
+constexpr int kRtnDenseLevels = 6;
+constexpr int kRtnDenseWarps = 16;  // the fp64 statistics need the registers
+
+template <typename T>
+__global__ void __launch_bounds__(kRtnDenseWarps * 32, 1)
+rtn_cluster_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid_constant__ RtnSchedule sc,
+                   const __grid_constant__ DrawPlan pl, const __grid_constant__ DrawnLevels drawn, int adaptive, int per_block,
+                   float* __restrict__ val, int64_t ldv, int* status, int* worker_err) {
+    using Tr = ElemTraits<T>;
+    extern __shared__ __align__(16) uint32_t sh_slots[];
+    __shared__ DenseShared<kRtnDenseWarps, double> sh;
+    __shared__ RtnLevel sh_lv[kRtnDenseLevels];
+    cg::cluster_group cluster = cg::this_cluster();
+    pdl_enter();
+    const int rank = (int)cluster.block_rank(), m = blockIdx.x / (int)cluster.num_blocks();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t g0 = (int64_t)rank * per_block;
+    const int n = (int)max((int64_t)0, min((int64_t)per_block, (d + 1023) / 1024 - g0));
+    const uint32_t top = dense_load<T>(cluster, g + (int64_t)m * ld, d, g0, n, sh_slots, sh);
+    const bool bad = top >= Tr::kInfKey, first = rank == 0;
+    if (first && threadIdx.x == 0) {
+        worker_err[m] = bad ? MLMC_ERR_NONFINITE : 0;
+        if (bad) {
+            set_status(status, MLMC_ERR_NONFINITE);
+            void_header(pl, m);
+        }
+    }
+    if (bad) return;  // the same in every block
+    const float c = __uint_as_float(Tr::kVec == 8 ? top << 16 : top);
+    auto entry = [&](int i, int e) -> uint32_t {  // entry e of group i
+        const uint32_t w = sh_slots[i * kGroupSlot<T> + group_place<T>(e / 32, (e % 32) / Tr::kVec) + (e % Tr::kVec) * (int)sizeof(T) / 4];
+        return sizeof(T) == 4 ? w : (e & 1) ? w >> 16 : w & 0xFFFFu;
+    };
+    double delta = 0.0;
+    if (adaptive) {
+        if (threadIdx.x < sc.L - 1) sh_lv[threadIdx.x] = rtn_level(c > 0.0f ? c : 1.0f, sc.r[threadIdx.x]);
+        __syncthreads();
+        double acc[kRtnDenseLevels];
+#pragma unroll
+        for (int l = 0; l < kRtnDenseLevels; ++l) acc[l] = 0.0;
+        if (c > 0.0f) {
+            constexpr int kVecs = kRtnHeld / Tr::kVec;  // a warp takes a quarter of a group
+#pragma unroll 1
+            for (int u = warp; u < 4 * n; u += kRtnDenseWarps) {
+                const int64_t e0 = (g0 + (u >> 2)) * 1024;
+                if (e0 + 1024 <= d) {
+                    const uint4* x = reinterpret_cast<const uint4*>(sh_slots + (u >> 2) * kGroupSlot<T>) + (u & 3) * kVecs * 32 + lane;
+                    uint4 q[kVecs];
+#pragma unroll
+                    for (int j = 0; j < kVecs; ++j) q[j] = x[j * 32];
+                    float v[kRtnHeld];
+                    rtn_expand<T>(q, v);
+                    take_levels<kRtnDenseLevels>(v, c, sh_lv, sc.L, acc);
+                } else {  // entries past the row's end are not entries
+                    for (int e = (u & 3) * 256 + lane; e < (u & 3) * 256 + 256 && e0 + e < d; e += 32)
+                        take_entry<kRtnDenseLevels>(Tr::value(entry(u >> 2, e)), c, sh_lv, sc.L, acc);
+                }
+            }
+        }
+        double all[kDenseLevels];
+#pragma unroll
+        for (int l = 0; l < kDenseLevels; ++l) all[l] = l < kRtnDenseLevels ? acc[min(l, kRtnDenseLevels - 1)] : 0.0;
+        delta = sqrt(dense_sums(cluster, all, sh));
+        if (threadIdx.x >= sc.L) delta = 0.0;
+    }
+    double p;
+    const int level = dense_level(pl, drawn, adaptive, m, first, delta, c, sh, &p, status, worker_err);
+    const Residual<T> residual(c, sc, level, p);
+    float* out = val + (int64_t)m * ldv;
+    const bool vec_ok = (ldv % 4 == 0);
+    for (int u = warp; u < 4 * n; u += kRtnDenseWarps) {  // a quarter of a group
+        const int i = u >> 2;
+        const int64_t e0 = (g0 + i) * 1024;
+        if (e0 + 1024 <= d && vec_ok) {
+            constexpr int kQuarter = kGroupChunks<T> * 8;
+#pragma unroll
+            for (int k = (u & 3) * kQuarter + lane, j = 0; j < kQuarter / 32; ++j, k += 32)
+                residual.vector(*reinterpret_cast<const uint4*>(sh_slots + i * kGroupSlot<T> + group_place<T>(k / kGroupChunks<T>, k % kGroupChunks<T>)),
+                                out + e0 + k * Tr::kVec);
+        } else {
+            for (int e = (u & 3) * 256 + lane; e < (u & 3) * 256 + 256 && e0 + e < d; e += 32) out[e0 + e] = residual(entry(i, e));
         }
     }
 }
@@ -268,26 +396,22 @@ aggregate_dense_kernel(const float* __restrict__ val, const int32_t* level, int 
                        float* __restrict__ out) {
     pdl_enter();
     const float inv_M = 1.0f / (float)M;
-    const bool vec_ok = (ldv % 4 == 0) && (d % 4 == 0);
-    if (vec_ok) {
-        const int64_t n4 = d / 4;
-        for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n4; v += (int64_t)gridDim.x * blockDim.x) {
-            float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-            for (int m = 0; m < M; ++m) {
-                if (level[m] < 0) continue;
-                const float4 x = __ldg(reinterpret_cast<const float4*>(val + (int64_t)m * ldv) + v);
-                a.x += x.x; a.y += x.y; a.z += x.z; a.w += x.w;
-            }
-            a.x *= inv_M; a.y *= inv_M; a.z *= inv_M; a.w *= inv_M;
-            reinterpret_cast<float4*>(out)[v] = a;
+    const int64_t n4 = (ldv % 4 == 0 && reinterpret_cast<uintptr_t>(out) % 16 == 0) ? d / 4 : 0;
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n4; v += (int64_t)gridDim.x * blockDim.x) {
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int m = 0; m < M; ++m) {
+            if (level[m] < 0) continue;
+            const float4 x = __ldg(reinterpret_cast<const float4*>(val + (int64_t)m * ldv) + v);
+            a.x += x.x; a.y += x.y; a.z += x.z; a.w += x.w;
         }
-    } else {
-        for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < d; i += (int64_t)gridDim.x * blockDim.x) {
-            float a = 0.f;
-            for (int m = 0; m < M; ++m)
-                if (level[m] >= 0) a += val[(int64_t)m * ldv + i];
-            out[i] = a * inv_M;
-        }
+        a.x *= inv_M; a.y *= inv_M; a.z *= inv_M; a.w *= inv_M;
+        reinterpret_cast<float4*>(out)[v] = a;
+    }
+    for (int64_t i = n4 * 4 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < d; i += (int64_t)gridDim.x * blockDim.x) {
+        float a = 0.f;
+        for (int m = 0; m < M; ++m)
+            if (level[m] >= 0) a += val[(int64_t)m * ldv + i];
+        out[i] = a * inv_M;
     }
 }
 
@@ -347,6 +471,27 @@ void launch_rtn_stats(Workspace& ws, const void* g, int dtype, int64_t d, int M,
     };
     if (dtype == MLMC_BF16) go(static_cast<const bf16_t*>(g));
     else go(static_cast<const float*>(g));
+}
+
+// The whole message of short rows in one launch; false: the row is not for it.
+bool launch_rtn_cluster(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* r, int L,
+                        const DrawPlan& plan, const double* p, const mlmc_rtn_msgs& out, cudaStream_t s) {
+    const int cl = dense_cluster_blocks(ws, d, M);
+    if (cl == 0 || (!p && L > kRtnDenseLevels)) return false;
+    const RtnSchedule sc = make_rtn_schedule(r, L);
+    const DrawnLevels drawn = draw_levels(p, L, plan.seed, plan.step, M);
+    const int per = (int)(((d + 1023) / 1024 + cl - 1) / cl);
+    auto go = [&](auto kernel, auto* row, size_t elem) {
+        launch_kernel_cluster(ws, K_RTN_CLUSTER, cl, kernel, dim3(M * cl), kRtnDenseWarps * 32, per * 1024 * elem, s, row, d, ld, sc, plan,
+                              drawn, p ? 0 : 1, per, out.val, out.ldv, ws.status, ws.worker_err);
+    };
+    if (dtype == MLMC_BF16) go(rtn_cluster_kernel<bf16_t>, static_cast<const bf16_t*>(g), 2);
+    else go(rtn_cluster_kernel<float>, static_cast<const float*>(g), 4);
+    return true;
+}
+
+int configure_rtn_kernels(Workspace& ws) {
+    return configure_dense_cluster(rtn_cluster_kernel<float>, kRtnDenseWarps * 32, ws) && configure_dense_cluster(rtn_cluster_kernel<bf16_t>, kRtnDenseWarps * 32, ws) ? MLMC_OK : MLMC_ERR_CUDA;
 }
 
 void launch_rtn_emit(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* r, int L,

@@ -82,6 +82,7 @@ cluster_topk_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid
         sh.low_bin = kClBins;
     }
     if (t < nq) sh.q[t] = make_query(pl.adaptive ? pl.k[t] : (t ? drawn.band[m].k_hi : drawn.band[m].k_lo), d);
+    cluster.barrier_arrive();
     pdl_enter();
 
     // ---- 1. the block's batches (512 words each) into shared memory, chunks in the swizzled order of the emission
@@ -123,6 +124,7 @@ cluster_topk_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid
     if (lane == 0) sh.warp[warp] = my_top;
     __syncthreads();
     my_top = __reduce_max_sync(0xFFFFFFFFu, sh.warp[lane]);
+    cluster.barrier_wait();  // every block of the cluster runs: its shared memory can be written
     if (t < CL) cluster.map_shared_rank(sh.top, t)[rank] = my_top;
     const int own = kClBins / CL;  // bins of the first digit that a block resolves, two per word
     if (warp < CL) {  // warp r: how many of this block's keys lie in the range of block r
