@@ -1,4 +1,5 @@
 // C ABI of the MLMC compression library: context, argument checks and the launch sequences.
+#include <mutex>
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -179,6 +180,32 @@ void select_drawn(Workspace& ws, const void* g, int dtype, int64_t d, int M, int
     launch_emit(ws, g, dtype, d, M, ld, *out, s);
 }
 
+// Shared-memory limits of the kernels and the clusters that fit, set and asked for once per device in the life of the
+// process (a create after the first takes milliseconds less).
+bool configure_kernels(int device, KernelLimits* out) {
+    constexpr int kMostDevices = 64;
+    static std::mutex lock;
+    static bool known[kMostDevices];
+    static KernelLimits limits[kMostDevices];
+    std::lock_guard<std::mutex> hold(lock);
+    const bool keep = device < kMostDevices;
+    if (keep && known[device]) {
+        *out = limits[device];
+        return true;
+    }
+    KernelLimits l = {};
+    if (configure_select_kernels() != MLMC_OK || configure_emit_kernels() != MLMC_OK || configure_float_kernels() != MLMC_OK ||
+        configure_segment_kernels() != MLMC_OK || configure_rtn_kernels() != MLMC_OK || configure_cluster_kernels(&l) != MLMC_OK ||
+        configure_bit_kernels(&l) != MLMC_OK)
+        return false;
+    if (keep) {
+        limits[device] = l;
+        known[device] = true;
+    }
+    *out = l;
+    return true;
+}
+
 }  // namespace
 
 extern "C" {
@@ -189,25 +216,20 @@ int mlmc_create(mlmc_ctx** out, int device, int64_t d_max, int M_max, int L_max)
         return MLMC_ERR_ARG;
     DeviceGuard guard(device);
     if (!guard.ok) return MLMC_ERR_CUDA;
-    cudaDeviceProp prop;
-    if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) return MLMC_ERR_CUDA;
-    if (configure_select_kernels() != MLMC_OK || configure_emit_kernels() != MLMC_OK ||
-        configure_float_kernels() != MLMC_OK || configure_segment_kernels() != MLMC_OK)
-        return MLMC_ERR_CUDA;
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return MLMC_ERR_CUDA;
+    KernelLimits limits;
+    if (!configure_kernels(device, &limits)) return MLMC_ERR_CUDA;
 
     mlmc_ctx* ctx = new (std::nothrow) mlmc_ctx();
     if (!ctx) return MLMC_ERR_NOMEM;
     Workspace& ws = ctx->ws;
-    for (int& n : ws.dense_fit) n = M_max;
-    if (configure_cluster_kernels(ws) != MLMC_OK || configure_bit_kernels(ws) != MLMC_OK || configure_rtn_kernels(ws) != MLMC_OK) {
-        delete ctx;
-        return MLMC_ERR_CUDA;
-    }
+    ws.limits = limits;
     ws.device = device;
     ws.d_max = d_max;
     ws.M_max = M_max;
     ws.L_max = L_max;
-    ws.sm_count = prop.multiProcessorCount;
+    ws.sm_count = sms;
     ws.launches = 0;
     ws.timing = false;
     ws.last_emit_tiles = 0;

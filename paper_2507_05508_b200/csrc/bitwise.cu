@@ -603,10 +603,11 @@ size_t bit_pack_smem(size_t elem) { return (kBitThreads / 32) * 2 * 1024 * elem;
 
 }  // namespace
 
-int configure_bit_kernels(Workspace& ws) {
-    const bool ok = configure_dense_cluster(bit_cluster_kernel<float>, kBitDenseWarps * 32, ws) && configure_dense_cluster(bit_cluster_kernel<bf16_t>, kBitDenseWarps * 32, ws) &&
+int configure_bit_kernels(KernelLimits* limits) {
+    const bool ok = configure_dense_cluster(bit_cluster_kernel<float>) && configure_dense_cluster(bit_cluster_kernel<bf16_t>) &&
                     cudaFuncSetAttribute(bit_pack_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)bit_pack_smem(4)) == cudaSuccess;
+    dense_cluster_fit(bit_cluster_kernel<float>, kBitDenseWarps * 32, limits);
     return ok ? MLMC_OK : MLMC_ERR_CUDA;
 }
 

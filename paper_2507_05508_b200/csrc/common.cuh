@@ -82,6 +82,12 @@ struct DrawnLevels {
 
 constexpr int kTimingPool = 2048;  // event pairs kept between two reads
 
+// What the device can place.
+struct KernelLimits {
+    int cluster_most;            // largest thread-block cluster of the short-row Top-k kernel (0: none)
+    int dense_fit[5];            // clusters of 1, 2, .. 16 blocks of the short-row dense kernels that run at a time
+};
+
 struct Workspace {
     // per-kernel timing (off by default): one CUDA event pair around every kernel launch
     bool timing;
@@ -95,8 +101,7 @@ struct Workspace {
     int M_max, L_max;
     int sm_count;
     int64_t launches;
-    int cluster_most;            // largest thread-block cluster of the short-row kernels (0: none)
-    int dense_fit[5];            // clusters of 1, 2, .. 16 blocks of the short-row dense kernels that run at a time
+    KernelLimits limits;
     bool long_sweeps;            // this call's sweeps are long enough to be launched without overlap (see launch_kernel)
     // device memory
     int* status;                 // sticky status word
@@ -572,7 +577,7 @@ void launch_emit(Workspace& ws, const void* g, int dtype, int64_t d, int M, int6
                  cudaStream_t s);
 void launch_aggregate_topk(Workspace& ws, const mlmc_topk_msgs& msgs, int M, int64_t d, float* out, cudaStream_t s);
 // bitwise.cu
-int configure_bit_kernels(Workspace& ws);
+int configure_bit_kernels(KernelLimits* limits);
 // Largest magnitude of every worker and the NaN / Inf check; with `p` (given probabilities) also the draw and the header.
 void launch_absmax(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const DrawPlan& plan, const double* p,
                    cudaStream_t s);
@@ -598,7 +603,7 @@ DrawPlan rtn_draw_plan(Workspace& ws, int L, uint64_t seed, uint64_t step, const
 // Adaptive: residual energies of every level, probabilities, draw and header.
 void launch_rtn_stats(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* r, int L,
                       const DrawPlan& plan, cudaStream_t s);
-int configure_rtn_kernels(Workspace& ws);
+int configure_rtn_kernels();
 bool launch_rtn_cluster(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* r, int L,
                         const DrawPlan& plan, const double* p, const mlmc_rtn_msgs& out, cudaStream_t s);
 void launch_rtn_emit(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* r, int L,
@@ -606,7 +611,7 @@ void launch_rtn_emit(Workspace& ws, const void* g, int dtype, int64_t d, int M, 
 void launch_aggregate_dense(Workspace& ws, const float* val, const int32_t* level, int M, int64_t d, int64_t ldv,
                             float* out, cudaStream_t s);
 // topk_cluster.cu: Top-k messages of short rows in one launch
-int configure_cluster_kernels(Workspace& ws);
+int configure_cluster_kernels(KernelLimits* limits);
 int cluster_blocks(const Workspace& ws, int dtype, int64_t d, int M);
 void launch_cluster_topk(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const FinishPlan& plan,
                          const DrawnBand* bands, const mlmc_topk_msgs* out, cudaStream_t s);

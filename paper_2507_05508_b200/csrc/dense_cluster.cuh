@@ -39,7 +39,7 @@ inline int dense_cluster_blocks(const Workspace& ws, int64_t d, int M) {
     const int64_t groups = (d + 1023) / 1024;
     int best = 0;
     for (int i = 0; i < 5; ++i) {
-        if (M > ws.dense_fit[i]) break;
+        if (M > ws.limits.dense_fit[i]) break;
         best = 1 << i;
         if (groups <= (int64_t)kDenseSpread << i) break;
     }
@@ -160,11 +160,15 @@ __device__ __forceinline__ int dense_level(const DrawPlan& pl, const DrawnLevels
 }
 
 template <typename K>
-bool configure_dense_cluster(K kernel, int threads, Workspace& ws) {
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDenseBytes) != cudaSuccess ||
-        cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
-        return false;
-    for (int i = 0; i < 5; ++i) {  // clusters of 2^i blocks that run at a time
+bool configure_dense_cluster(K kernel) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDenseBytes) == cudaSuccess &&
+           cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+}
+
+// Clusters of 2^i blocks that run at a time (a block takes an SM).
+template <typename K>
+void dense_cluster_fit(K kernel, int threads, KernelLimits* limits) {
+    for (int i = 0; i < 5; ++i) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(1 << i);
         cfg.blockDim = dim3(threads);
@@ -180,9 +184,8 @@ bool configure_dense_cluster(K kernel, int threads, Workspace& ws) {
             cudaGetLastError();
             n = 0;
         }
-        ws.dense_fit[i] = std::min(ws.dense_fit[i], n);
+        limits->dense_fit[i] = n;
     }
-    return true;
 }
 
 }  // namespace

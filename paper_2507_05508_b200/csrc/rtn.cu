@@ -490,8 +490,8 @@ bool launch_rtn_cluster(Workspace& ws, const void* g, int dtype, int64_t d, int 
     return true;
 }
 
-int configure_rtn_kernels(Workspace& ws) {
-    return configure_dense_cluster(rtn_cluster_kernel<float>, kRtnDenseWarps * 32, ws) && configure_dense_cluster(rtn_cluster_kernel<bf16_t>, kRtnDenseWarps * 32, ws) ? MLMC_OK : MLMC_ERR_CUDA;
+int configure_rtn_kernels() {
+    return configure_dense_cluster(rtn_cluster_kernel<float>) && configure_dense_cluster(rtn_cluster_kernel<bf16_t>) ? MLMC_OK : MLMC_ERR_CUDA;
 }
 
 void launch_rtn_emit(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* r, int L,

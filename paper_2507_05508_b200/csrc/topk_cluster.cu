@@ -565,8 +565,8 @@ size_t cluster_smem(int per_block) { return kClFixedSmem + (size_t)per_block * k
 
 }  // namespace
 
-int configure_cluster_kernels(Workspace& ws) {
-    ws.cluster_most = 0;
+int configure_cluster_kernels(KernelLimits* limits) {
+    limits->cluster_most = 0;
     auto set = [&](auto kernel) {
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cluster_smem(kClBatches)) != cudaSuccess) return false;
         return cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
@@ -586,7 +586,7 @@ int configure_cluster_kernels(Workspace& ws) {
         cfg.numAttrs = 1;
         int n = 0;
         if (cudaOccupancyMaxActiveClusters(&n, cluster_topk_kernel<float>, &cfg) == cudaSuccess && n >= 1) {
-            ws.cluster_most = cl;
+            limits->cluster_most = cl;
             break;
         }
         cudaGetLastError();
@@ -597,11 +597,11 @@ int configure_cluster_kernels(Workspace& ws) {
 // Blocks per cluster for this call, 0: the row is too long (or the workers too many) for it.
 int cluster_blocks(const Workspace& ws, int dtype, int64_t d, int M) {
     const int batches = emit_tiles_per_worker(d, dtype) * kEmitGroups;
-    if (M > 32 || ws.cluster_most == 0) return 0;
+    if (M > 32 || ws.limits.cluster_most == 0) return 0;
     // The smallest cluster whose blocks have at most 32 batches (64 KB, 16 words per thread), and no more workers than fit
     // the GPU at a time: a barrier and an exchange between more blocks take longer than the work that they share out.
     int cl = 1;
-    while (cl < ws.cluster_most && (batches + cl - 1) / cl > 32) cl *= 2;
+    while (cl < ws.limits.cluster_most && (batches + cl - 1) / cl > 32) cl *= 2;
     return (batches + cl - 1) / cl <= (dtype == MLMC_BF16 ? kClBatchesBf16 : kClBatches) ? cl : 0;
 }
 

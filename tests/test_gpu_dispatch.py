@@ -1,0 +1,143 @@
+"""The lengths at which the library changes its kernels, and the edges of their tiles, against the CPU oracle.
+
+Every case runs compress and aggregate through the C ABI and compares messages and averages (the checks of the parity tests).
+"""
+import numpy as np
+import pytest
+import torch
+
+from paper_2507_05508_b200 import workloads as wl
+from test_gpu_ext import check_floatbits, check_rtn
+from test_gpu_parity import check_bitwise, check_topk, padded, to_dev
+
+pytestmark = pytest.mark.gpu
+
+BITS = [1, 2, 4, 8, 16, 23]
+
+
+@pytest.fixture(scope="module")
+def B():
+    from paper_2507_05508_b200 import binding
+    binding.lib()
+    return binding
+
+
+@pytest.fixture(scope="module")
+def ctx(B):
+    c = B.mlmc_create(0, 2_500_000, 20, 32)
+    yield c
+    B.mlmc_destroy(c)
+
+
+def layered(d, M, dtype="f32", seed=5):
+    """Heavy-tailed rows with a few layers of different scale."""
+    rng = np.random.default_rng(seed)
+    scale = np.repeat(10.0 ** rng.uniform(-4, -1, 7), -(-d // 7))[:d]
+    g = torch.from_numpy((rng.standard_t(3, (M, d)) * scale).astype(np.float32)).cuda()
+    return padded(g.to(torch.bfloat16) if dtype == "bf16" else g, 8)
+
+
+def geometric(L):
+    return list(wl.geometric_probs(L))
+
+
+def doubling(d, first):
+    k = []
+    while first < d:
+        k.append(first)
+        first *= 2
+    return k + [d]
+
+
+# one block or two; the longest row of a cluster with given p and with adaptive p, fp32 and bf16; one entry more
+@pytest.mark.parametrize("dtype,d,M,adaptive", [
+    ("f32", 511, 2, True), ("f32", 16_384, 3, True), ("f32", 16_385, 3, True), ("f32", 262_144, 2, False), ("f32", 262_145, 2, False),
+    ("f32", 704_512, 1, True), ("f32", 704_513, 1, True), ("bf16", 32_769, 2, True), ("bf16", 524_289, 1, False),
+    ("bf16", 1_032_192, 1, True), ("bf16", 1_032_193, 1, True)])
+def test_topk_row_lengths(B, ora, ctx, dtype, d, M, adaptive):
+    k = doubling(d, max(1, d // 500))
+    check_topk(B, ora, ctx, layered(d, M, dtype), k, None if adaptive else geometric(len(k)), 3, 1, expect_excluded=1)
+
+
+# the average in one launch (up to four tiles per SM) and in two
+@pytest.mark.parametrize("d,M", [(4_096, 20), (4_097, 1), (2_424_832, 2), (2_424_833, 2)])
+def test_topk_average_lengths(B, ora, ctx, d, M):
+    k = [d // 3, d]
+    check_topk(B, ora, ctx, layered(d, M), k, [0.5, 0.5], 1, 2)
+
+
+# bands from a few entries per batch of 512 words to whole batches, on both sides of the staged emission, with and without ties
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("share", [0.02, 0.12, 0.125, 0.5, 1.0])
+def test_dense_and_sparse_bands(B, ora, ctx, dtype, share):
+    d = 530_001
+    lo = int(d * (1 - share) / 2)
+    k = [lo, lo + max(1, int(d * share)), d] if share < 1.0 else [0, d]
+    p = [1e-9] * len(k)
+    p[1] = 1.0 - 1e-9 * (len(k) - 1)
+    g = layered(d, 2, dtype)
+    check_topk(B, ora, ctx, g, k, p, 4, 0)
+    rng = np.random.default_rng(8)
+    ties = torch.from_numpy(rng.choice(np.array([0.5, -0.5, 0.25, 3.0, 0.1], dtype=np.float32), (2, d))).cuda()
+    check_topk(B, ora, ctx, padded(ties.to(g.dtype), 8), k, p, 4, 1)
+
+
+# thresholds that share a leading-digit bin, trivial ranks, and so many levels that the second sweep takes smaller blocks
+@pytest.mark.parametrize("case", ["shared_bins", "trivial_ranks", "many_levels"])
+def test_second_sweep_intervals(B, ora, ctx, case):
+    d = 720_003
+    if case == "shared_bins":
+        g = to_dev((1.0 + 0.02 * np.random.default_rng(1).random((1, d))).astype(np.float32))
+        k = [int(d * f) for f in (0.1, 0.2, 0.21, 0.5, 0.9, 0.99)] + [d]
+    elif case == "trivial_ranks":
+        g, k = layered(d, 1), [0, 0, 7, 7, d // 2, d, d]
+    else:
+        g, k = layered(d, 1), sorted({int(d * (i + 1) / 32) for i in range(31)}) + [d]
+    check_topk(B, ora, ctx, g, k, None, 2, 3, expect_excluded=1)
+
+
+# a group of 1024 entries, a group per warp, the longest row of a cluster, and one entry more
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("d,M", [(1, 1), (1_023, 3), (1_025, 20), (16_384, 2), (16_385, 2), (458_752, 1), (458_753, 1)])
+def test_dense_row_lengths(B, ora, ctx, dtype, d, M):
+    g = layered(d, M, dtype)
+    for p in (None, geometric(6)):
+        check_bitwise(B, ora, ctx, g, BITS, p, 7, 1)
+    for p in (None, geometric(5)):
+        check_rtn(B, ora, ctx, g, [2, 4, 8, 16], p, 7, 1)
+
+
+# schedules outside the one-launch kernels: a field above 8 bits, more levels
+@pytest.mark.parametrize("b", [[9, 23], [2, 9, 12, 20], list(range(1, 11)), [3, 11, 19]])
+def test_bitwise_schedules_of_a_short_row(B, ora, ctx, b):
+    g = layered(5_003, 3)
+    check_bitwise(B, ora, ctx, g, b, None, 9, 0)
+    check_bitwise(B, ora, ctx, g, b, geometric(len(b)), 9, 0)
+
+
+# the divisor of the bit-wise quotient at both ends of fp32 and around the limits between which it is used as it is
+@pytest.mark.parametrize("top", [2.0 ** -100, 0.999 * 2.0 ** -60, 2.0 ** -60, 1.0, 2.0 ** 100, 1.001 * 2.0 ** 100, 3.4e38])
+@pytest.mark.parametrize("d", [4_001, 460_001])
+def test_bitwise_scales(B, ora, ctx, top, d):
+    rng = np.random.default_rng(2)
+    g = rng.uniform(-1, 1, (1, d)) * np.exp(-rng.uniform(0, 12, (1, d)))
+    g[0, 0] = 1.0
+    g = to_dev((g * top).astype(np.float32))
+    check_bitwise(B, ora, ctx, g, BITS, None, 1, 0)
+    check_bitwise(B, ora, ctx, g, [23], [1.0], 1, 0)
+
+
+# planes one by one and by bit transposes, ragged words, groups of zeros
+@pytest.mark.parametrize("mb", [[1, 2, 4, 8, 16, 23], [5, 11, 23], [23]])
+@pytest.mark.parametrize("d", [31, 33, 1_024, 70_001])
+def test_floatbits_lengths(B, ora, ctx, mb, d):
+    g = layered(d, 2)
+    g[:, d // 3:d // 2] = 0.0
+    check_floatbits(B, ora, ctx, g, mb, geometric(len(mb)), 6, 0)
+
+
+# statistics of long rows: trips of the ring and what is left of them, few and many levels
+@pytest.mark.parametrize("r", [[2, 4, 8, 16], list(range(1, 17))])
+@pytest.mark.parametrize("d", [460_800, 460_801, 1_000_003])
+def test_rtn_long_rows(B, ora, ctx, r, d):
+    check_rtn(B, ora, ctx, layered(d, 1), r, None, 3, 0)
