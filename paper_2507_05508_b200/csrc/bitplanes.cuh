@@ -79,5 +79,66 @@ __device__ __forceinline__ void transpose_bits(uint32_t (&x)[32]) {
     }
 }
 
+// ---- averages of plane messages: a thread adds up one word (32 entries) of every worker's planes, worker after worker.  Its
+// words come through a ring of kAvgSlots shared-memory slots, thread by thread: the next three workers' are in flight.  (In
+// registers there was room for one worker and one plane of it: 20 KB in flight per SM, half of what HBM needs.)
+constexpr int kAvgThreads = 256;
+constexpr int kAvgSlots = 4;
+constexpr int kAvgStage = 32 * 33;   // words of a warp's output rows; they take the place of its ring
+constexpr int kAvgPlanes = 8;       // magnitude planes in the ring; the fields of wider levels are read as they are used
+
+__device__ __forceinline__ void cp_async_4(void* smem_dst, const void* gmem_src) {
+    const uint32_t s = (uint32_t)__cvta_generic_to_shared(smem_dst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gmem_src) : "memory");
+}
+
+// fb[k] holds bit k of 32 fields of at most 8 bits; afterwards byte t >> 3 of fb[t & 7] is the field of entry t.
+__device__ __forceinline__ void fields_to_bytes(uint32_t (&fb)[8]) {
+#pragma unroll
+    for (int j = 4; j > 0; j >>= 1) {
+        const uint32_t mask = j == 4 ? 0x0F0F0F0Fu : j == 2 ? 0x33333333u : 0x55555555u;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            if (k & j) continue;
+            const uint32_t x = ((fb[k] >> j) ^ fb[k + j]) & mask;
+            fb[k + j] ^= x;
+            fb[k] ^= x << j;
+        }
+    }
+}
+
+// f unit for the field f of entry t, rounded once: a byte below the bits of 2^23 is 2^23 + f, and offset = -2^23 unit.
+__device__ __forceinline__ float field_times(const uint32_t (&fb)[8], int t, float unit, float offset) {
+    return fmaf(__uint_as_float(__byte_perm(fb[t & 7], 0x4B000000u, 0x7650u + (uint32_t)(t >> 3))), unit, offset);
+}
+
+// Fields of any width, plane by plane.
+__device__ __forceinline__ void gather_fields(const uint32_t* __restrict__ plane1, int64_t words, int w, uint32_t (&f)[32]) {
+#pragma unroll
+    for (int t = 0; t < 32; ++t) f[t] = 0u;
+    for (int j = 0; j < w; ++j) {
+        const uint32_t pw = __ldg(plane1 + (int64_t)j * words);
+#pragma unroll
+        for (int t = 0; t < 32; ++t) f[t] = (f[t] << 1) | ((pw >> t) & 1u);
+    }
+}
+
+// The 32 sums of every lane of a warp, whose words are word0 + lane, leave as rows of 128 bytes.  stage: 32 x 33 words.
+__device__ __forceinline__ void store_words(uint32_t* stage_words, const float (&acc)[32], float factor, int64_t word0, int64_t d,
+                                            float* __restrict__ out) {
+    float (*stage)[33] = reinterpret_cast<float (*)[33]>(stage_words);
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+#pragma unroll
+    for (int t = 0; t < 32; ++t) stage[lane][t] = acc[t] * factor;
+    __syncwarp();
+#pragma unroll 4
+    for (int r = 0; r < 32; ++r) {
+        const int64_t i = (word0 + r) * 32 + lane;
+        if (i < d) out[i] = stage[r][lane];
+    }
+    __syncwarp();
+}
+
 }  // namespace
 }  // namespace mlmc

@@ -460,114 +460,89 @@ bit_cluster_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid_
         pack_group<T>(sh_slots + i * kGroupSlot<T>, qz, scale, zero_below, sc.width[level], (g0 + i) * 32 + lane, words, out);
 }
 
-// ---- server average of bit-plane messages: thread = one word (32 entries), staged through shared memory
-__global__ void __launch_bounds__(kBitThreads)
+// ---- server average of bit-plane messages.  8 x 124M entries, six levels: 372 us with one worker in flight, now 250.
+constexpr int kAvgBitRows = 1 + kAvgPlanes;
+constexpr int kAvgBitWords = kAvgSlots * kAvgBitRows * 32 > kAvgStage ? kAvgSlots * kAvgBitRows * 32 : kAvgStage;  // per warp
+constexpr size_t kAvgBitSmem = (size_t)kAvgBitWords * (kAvgThreads / 32) * 4;
+
+__global__ void __launch_bounds__(kAvgThreads)
 aggregate_bitwise_kernel(const uint32_t* __restrict__ planes, const float* gmax, const int32_t* level, const double* p_sel,
-                         BitSchedule sc, int w_max, int64_t words, int M, int64_t d, float* __restrict__ out) {
+                         const __grid_constant__ BitSchedule sc, int w_max, int64_t words, int M, int64_t d, float* __restrict__ out) {
+    extern __shared__ __align__(16) uint32_t sh_ring[];  // [warps][kAvgSlots][kAvgBitRows][32], units and levels
+    float* sh_unit = reinterpret_cast<float*>(sh_ring + kAvgThreads / 32 * kAvgBitWords);  // value of one unit of the field: 2^{-b_l} gmax / p_l
+    int* sh_level = reinterpret_cast<int*>(sh_unit + M);
     pdl_enter();
-    __shared__ float sh_out[kBitThreads / 32][32][33];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t* ring = sh_ring + warp * kAvgBitWords;
     const float inv_M = 1.0f / (float)M;
-    const int64_t nblk = (words + kBitThreads - 1) / kBitThreads;
+    const int64_t nblk = (words + kAvgThreads - 1) / kAvgThreads;
     for (int64_t blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
-        const int64_t word = blk * kBitThreads + threadIdx.x;
+        const int64_t word = blk * kAvgThreads + threadIdx.x, at = min(word, words - 1);  // lanes past the end repeat the last word
         float acc[32];
 #pragma unroll
         for (int t = 0; t < 32; ++t) acc[t] = 0.0f;
-        // the sign word and the first magnitude plane of the next worker are loaded before this worker's are used
-        uint32_t sgn_n = 0, pw1_n = 0;
-        auto preload = [&](int mm) {
-            if (mm < M && level[mm] >= 0 && word < words) {
-                const uint32_t* pm = planes + (int64_t)mm * (1 + w_max) * words;
-                sgn_n = pm[word];
-                pw1_n = pm[words + word];
-            } else {
-                sgn_n = 0;
-                pw1_n = 0;
+        auto fetch = [&](int m) {  // the sign word to row 0, bit k of the fields (plane w - k) to row 1 + k
+            const int lv = m < M ? __ldg(&level[m]) : -1;
+            if (lv >= 0) {
+                const int w = sc.width[lv];
+                const uint32_t* from = planes + (int64_t)m * (1 + w_max) * words + at;
+                uint32_t* to = ring + (m & (kAvgSlots - 1)) * kAvgBitRows * 32 + lane;
+                cp_async_4(to, from);
+                if (w <= kAvgPlanes)
+                    for (int k = 0; k < w; ++k) cp_async_4(to + (1 + k) * 32, from + (int64_t)(w - k) * words);
             }
+            cp_async_commit();
         };
-        preload(0);
+#pragma unroll
+        for (int m = 0; m < kAvgSlots - 1; ++m) fetch(m);
+        if (blk == blockIdx.x) {  // while the first words are on their way
+            for (int m = threadIdx.x; m < M; m += kAvgThreads) {
+                const int lv = level[m];
+                sh_level[m] = lv;
+                sh_unit[m] = lv >= 0 ? (float)(ldexp((double)gmax[m], -sc.bits[lv]) / p_sel[m]) : 0.0f;
+            }
+            __syncthreads();
+        }
         for (int m = 0; m < M; ++m) {  // fixed worker order
-            const int lv = level[m];
-            const uint32_t sgn = sgn_n, pw1 = pw1_n;
-            preload(m + 1);
+            fetch(m + kAvgSlots - 1);
+            cp_async_wait<kAvgSlots - 1>();
+            const int lv = sh_level[m];
             if (lv < 0) continue;
             const int w = sc.width[lv];
-            // value of one unit of the field: 2^{-b_l} gmax / p_l
-            const float unit = (float)(ldexp((double)gmax[m], -sc.bits[lv]) / p_sel[m]);
-            // A word whose fields are all zero adds +-0 to every entry, which changes nothing: it is skipped.  The
-            // high levels of a heavy-tailed gradient are almost all zero, so whole warps skip.
-            if (w == 1) {  // the paper's case: one information bit and one sign bit per entry
-                if (pw1 != 0u) {
-                    const uint32_t ub = __float_as_uint(unit);
+            const float unit = sh_unit[m];
+            const uint32_t* from = ring + (m & (kAvgSlots - 1)) * kAvgBitRows * 32 + lane;
+            const uint32_t sgn = from[0];
+            if (w <= kAvgPlanes && fabsf(unit) < 0x1p100f) {
+                uint32_t fb[8], any = 0u;
 #pragma unroll
-                    for (int t = 0; t < 32; ++t) {
-                        const uint32_t on = 0u - ((pw1 >> t) & 1u);
-                        acc[t] += __uint_as_float((ub & on) ^ (((sgn >> t) & 1u) << 31));
-                    }
-                }
-            } else if (w <= 8 && fabsf(unit) < 0x1p100f) {
-                // fields of at most 8 bits: one bit transpose of 8 x 8 blocks turns the plane words (bit k of every field
-                // in word k) into field bytes, four entries per word; a byte below the bits of 2^23 is 2^23 + f, and
-                // (2^23 + f) unit - 2^23 unit is f unit rounded once
-                const uint32_t* pm = planes + (int64_t)m * (1 + w_max) * words;
-                uint32_t fb[8], any = pw1;
-#pragma unroll
-                for (int k = 0; k < 8; ++k) {  // bit k of the fields: plane w - k
-                    fb[k] = (k == w - 1) ? pw1 : (k < w && word < words) ? pm[(int64_t)(w - k) * words + word] : 0u;
+                for (int k = 0; k < 8; ++k) {
+                    fb[k] = k < w ? from[(1 + k) * 32] : 0u;
                     any |= fb[k];
                 }
+                // A word whose fields are all zero adds +-0 to every entry, which changes nothing.  The high levels of a
+                // heavy-tailed gradient are almost all zero, so whole warps skip.
                 if (any != 0u) {
-#pragma unroll
-                    for (int j = 4; j > 0; j >>= 1) {
-                        const uint32_t mask = j == 4 ? 0x0F0F0F0Fu : j == 2 ? 0x33333333u : 0x55555555u;
-#pragma unroll
-                        for (int k = 0; k < 8; ++k) {
-                            if (k & j) continue;
-                            const uint32_t x = ((fb[k] >> j) ^ fb[k + j]) & mask;
-                            fb[k + j] ^= x;
-                            fb[k] ^= x << j;
-                        }
-                    }
+                    fields_to_bytes(fb);
                     const float offset = -8388608.0f * unit;
 #pragma unroll
-                    for (int t = 0; t < 32; ++t) {
-                        const float ff = __uint_as_float(__byte_perm(fb[t & 7], 0x4B000000u, 0x7650u + (uint32_t)(t >> 3)));
-                        const float v = fmaf(ff, unit, offset);
-                        acc[t] += __uint_as_float(__float_as_uint(v) ^ ((sgn << (31 - t)) & 0x80000000u));
-                    }
+                    for (int t = 0; t < 32; ++t)
+                        acc[t] += __uint_as_float(__float_as_uint(field_times(fb, t, unit, offset)) ^ ((sgn << (31 - t)) & 0x80000000u));
                 }
             } else {
-                const uint32_t* pm = planes + (int64_t)m * (1 + w_max) * words;
                 uint32_t f[32];
-#pragma unroll
-                for (int t = 0; t < 32; ++t) f[t] = (pw1 >> t) & 1u;
-                for (int j = 2; j <= w; ++j) {
-                    const uint32_t pw = (word < words) ? pm[(int64_t)j * words + word] : 0u;
-#pragma unroll
-                    for (int t = 0; t < 32; ++t) f[t] = (f[t] << 1) | ((pw >> t) & 1u);
-                }
+                gather_fields(planes + ((int64_t)m * (1 + w_max) + 1) * words + at, words, w, f);
 #pragma unroll
                 for (int t = 0; t < 32; ++t) {
-                    // f < 2^23: exact integer-to-float through the 2^23 offset, without the conversion unit
-                    const float ff = __uint_as_float(0x4B000000u | f[t]) - 8388608.0f;
-                    acc[t] += __uint_as_float(__float_as_uint(ff * unit) ^ (((sgn >> t) & 1u) << 31));
+                    const float ff = __uint_as_float(0x4B000000u | f[t]) - 8388608.0f;  // f < 2^23: exact
+                    acc[t] += __uint_as_float(__float_as_uint(ff * unit) ^ ((sgn << (31 - t)) & 0x80000000u));
                 }
             }
         }
-        // transpose through shared memory so that the 32 floats of a word leave as one 128-byte row
-#pragma unroll
-        for (int t = 0; t < 32; ++t) sh_out[warp][lane][t] = acc[t] * inv_M;
-        __syncwarp();
-        const int64_t wbase = blk * kBitThreads + warp * 32;
-#pragma unroll 4
-        for (int r = 0; r < 32; ++r) {
-            const int64_t i = (wbase + r) * 32 + lane;
-            if (i < d) out[i] = sh_out[warp][r][lane];
-        }
-        __syncwarp();
+        cp_async_wait<0>();
+        store_words(ring, acc, inv_M, blk * kAvgThreads + warp * 32, d, out);
     }
 }
+
 
 BitSchedule make_schedule(const int32_t* b, int L) {
     BitSchedule sc = {};
@@ -604,7 +579,9 @@ size_t bit_pack_smem(size_t elem) { return (kBitThreads / 32) * 2 * 1024 * elem;
 }  // namespace
 
 int configure_bit_kernels(KernelLimits* limits) {
-    const bool ok = configure_dense_cluster(bit_cluster_kernel<float>) && configure_dense_cluster(bit_cluster_kernel<bf16_t>) &&
+    const bool ok = cudaFuncSetAttribute(aggregate_bitwise_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)kAvgBitSmem + kEmitMaxWorkers * 8) == cudaSuccess &&
+                    configure_dense_cluster(bit_cluster_kernel<float>) && configure_dense_cluster(bit_cluster_kernel<bf16_t>) &&
                     cudaFuncSetAttribute(bit_pack_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)bit_pack_smem(4)) == cudaSuccess;
     dense_cluster_fit(bit_cluster_kernel<float>, kBitDenseWarps * 32, limits);
@@ -716,12 +693,11 @@ void launch_aggregate_bitwise(Workspace& ws, const mlmc_bit_msgs& msgs, const in
                               float* out, cudaStream_t s) {
     const BitSchedule sc = make_schedule(b, L);
     const int64_t words = (d + 31) / 32;
-    int64_t nb = (words + kBitThreads - 1) / kBitThreads;
+    const size_t smem = kAvgBitSmem + (size_t)M * 8;
     // whole waves only: every block does the same number of iterations, so a partial last wave costs a full one
-    static const int resident = resident_blocks(aggregate_bitwise_kernel, kBitThreads, 0);
-    const int64_t cap = (int64_t)ws.sm_count * resident * 2;
-    if (nb > cap) nb = cap;
-    launch_kernel(ws, K_AGG_BIT, aggregate_bitwise_kernel, dim3((unsigned)nb), kBitThreads, 0, s, msgs.planes, msgs.gmax,
+    static const int resident = resident_blocks(aggregate_bitwise_kernel, kAvgThreads, kAvgBitSmem + 64);
+    const int64_t nb = std::min((words + kAvgThreads - 1) / kAvgThreads, (int64_t)ws.sm_count * resident * 2);
+    launch_kernel(ws, K_AGG_BIT, aggregate_bitwise_kernel, dim3((unsigned)nb), kAvgThreads, smem, s, msgs.planes, msgs.gmax,
                   msgs.level, msgs.p_sel, sc, msgs.w_max, words, M, d, out);
 }
 

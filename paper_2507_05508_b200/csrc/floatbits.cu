@@ -5,6 +5,8 @@
 // and exponent are sent with every message (App. B counts 1 + exponent + 1 bits per entry), and they are the base
 // g^0 = sign 2^(E - bias) of the estimate g^0 + (1/p^l)(C^l - C^{l-1}).  The level draw does not depend on the data
 // (App. B's lemma gives fixed probabilities), so one sweep over the gradient writes the whole message.
+#include <algorithm>
+
 #include "bitplanes.cuh"
 
 namespace mlmc {
@@ -169,101 +171,110 @@ float_pack_kernel(const T* __restrict__ g, int64_t d, int64_t ld, MantissaSchedu
 // A term is +-2^(E - 127) (1 + f 2^-mb_l / p): the power of two times a multiplier, added by one fused multiply-add (the
 // product with a power of two is exact, so this is the sum of the rounded term).  An exponent field 0 has no leading one
 // and the scale of exponent field 1; a word that holds one takes the general form.
-// Bound by issue: 8 to 14 instructions per entry and worker; the general form for every entry took 0.88 ms for 8 x 124M.
-__global__ void __launch_bounds__(kFloatThreads, 2)
+// Bound by issue: 8 to 12 instructions per entry and worker.  8 x 124M entries: 0.88 ms with the general form for every entry,
+// 0.55 with one worker in flight and fields wider than a bit gathered bit by bit, now 0.48 (10M x 8, wider fields: 161 -> 74 us).
+constexpr int kAvgFloatRows = 8 + 1 + kAvgPlanes;  // words of a thread: 32 exponents, signs, planes
+constexpr int kAvgFloatWords = kAvgSlots * kAvgFloatRows * 32 > kAvgStage ? kAvgSlots * kAvgFloatRows * 32 : kAvgStage;  // per warp
+constexpr size_t kAvgFloatSmem = (size_t)kAvgFloatWords * (kAvgThreads / 32) * 4;
+
+__global__ void __launch_bounds__(kAvgThreads)
 aggregate_float_kernel(const uint8_t* __restrict__ expo, const uint32_t* __restrict__ planes, const int32_t* level,
-                       const double* p_sel, MantissaSchedule sc, int w_max, int64_t words, int M, int64_t d,
+                       const double* p_sel, const __grid_constant__ MantissaSchedule sc, int w_max, int64_t words, int M, int64_t d,
                        float* __restrict__ out) {
-    __shared__ float sh_out[kFloatThreads / 32][32][33];
-    __shared__ float sh_c[kFloatThreads];   // 2^-mb_l / p_l of the next workers
-    __shared__ int sh_lv[kFloatThreads];
+    // [warps][kAvgSlots][32 x two vectors of exponents, then rows of signs and planes][32], units and levels
+    extern __shared__ __align__(16) uint32_t sh_ring[];
+    float* sh_unit = reinterpret_cast<float*>(sh_ring + kAvgThreads / 32 * kAvgFloatWords);  // 2^-mb_l / p_l
+    int* sh_level = reinterpret_cast<int*>(sh_unit + M);
     pdl_enter();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t* ring = sh_ring + warp * kAvgFloatWords;
     const float inv_M = 1.0f / (float)M;
-    const int64_t nblk = (words + kFloatThreads - 1) / kFloatThreads;
+    const int64_t nblk = (words + kAvgThreads - 1) / kAvgThreads;
     for (int64_t blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
-        const int64_t word = blk * kFloatThreads + threadIdx.x;
-        const int64_t at = word < words ? word : words - 1;  // lanes past the end repeat the last word
+        const int64_t word = blk * kAvgThreads + threadIdx.x, at = min(word, words - 1);  // lanes past the end repeat the last word
         float acc[32];
 #pragma unroll
         for (int t = 0; t < 32; ++t) acc[t] = 0.0f;
-        for (int m0 = 0; m0 < M; m0 += kFloatThreads) {
-            const int nm = min(M - m0, kFloatThreads);
-            if (m0 > 0 || blk == blockIdx.x || M > kFloatThreads) {
-                __syncthreads();
-                if (threadIdx.x < nm) {
-                    const int lv = level[m0 + threadIdx.x];
-                    sh_lv[threadIdx.x] = lv;
-                    sh_c[threadIdx.x] = lv >= 0 ? (float)(ldexp(1.0, -sc.hi[lv]) / p_sel[m0 + threadIdx.x]) : 0.0f;
-                }
-                __syncthreads();
-            }
-            // exponents, signs and the first plane of the next worker are in flight while this one's are added
-            uint4 ea_n, eb_n;
-            uint32_t sgn_n, pw_n;
-            auto preload = [&](int i) {
-                if (i >= nm || sh_lv[i] < 0) return;
-                const uint32_t* pm = planes + (int64_t)(m0 + i) * (1 + w_max) * words + at;
-                const uint4* em = reinterpret_cast<const uint4*>(expo + ((int64_t)(m0 + i) * words + at) * 32);
-                ea_n = __ldg(em);
-                eb_n = __ldg(em + 1);
-                sgn_n = __ldg(pm);
-                pw_n = __ldg(pm + words);
-            };
-            preload(0);
-            for (int i = 0; i < nm; ++i) {  // fixed worker order
-                const uint4 ea = ea_n, eb = eb_n;
-                const uint32_t sgn = sgn_n, pw1 = pw_n;
-                const int lv = sh_lv[i];
-                preload(i + 1);
-                if (lv < 0) continue;
+        auto slot = [&](int m) { return ring + (m & (kAvgSlots - 1)) * kAvgFloatRows * 32; };
+        auto fetch = [&](int m) {  // the sign word to row 0, bit k of the fields (plane w - k) to row 1 + k
+            const int lv = m < M ? __ldg(&level[m]) : -1;
+            if (lv >= 0) {
                 const int w = sc.hi[lv] - sc.lo[lv];
-                const float c = sh_c[i];
-                const uint32_t e4[8] = {ea.x, ea.y, ea.z, ea.w, eb.x, eb.y, eb.z, eb.w};
-                uint32_t zero = 0;  // some exponent byte is 0
+                const uint32_t* from = planes + (int64_t)m * (1 + w_max) * words + at;
+                const uint8_t* e = expo + ((int64_t)m * words + at) * 32;
+                uint32_t* to = slot(m);
+                cp_async_16(to + lane * 4, e);
+                cp_async_16(to + (32 + lane) * 4, e + 16);
+                to += 8 * 32 + lane;
+                cp_async_4(to, from);
+                if (w <= kAvgPlanes)
+                    for (int k = 0; k < w; ++k) cp_async_4(to + (1 + k) * 32, from + (int64_t)(w - k) * words);
+            }
+            cp_async_commit();
+        };
 #pragma unroll
-                for (int q = 0; q < 8; ++q) zero |= (e4[q] - 0x01010101u) & ~e4[q] & 0x80808080u;
-                if (zero == 0u && w == 1) {
-                    const uint32_t m1 = __float_as_uint(1.0f + c);
+        for (int m = 0; m < kAvgSlots - 1; ++m) fetch(m);
+        if (blk == blockIdx.x) {  // while the first words are on their way
+            for (int m = threadIdx.x; m < M; m += kAvgThreads) {
+                const int lv = level[m];
+                sh_level[m] = lv;
+                sh_unit[m] = lv >= 0 ? (float)(ldexp(1.0, -sc.hi[lv]) / p_sel[m]) : 0.0f;
+            }
+            __syncthreads();
+        }
+        for (int m = 0; m < M; ++m) {  // fixed worker order
+            fetch(m + kAvgSlots - 1);
+            cp_async_wait<kAvgSlots - 1>();
+            const int lv = sh_level[m];
+            if (lv < 0) continue;
+            const int w = sc.hi[lv] - sc.lo[lv];
+            const float c = sh_unit[m];
+            const uint32_t* from = slot(m);
+            const uint4 ea = reinterpret_cast<const uint4*>(from)[lane], eb = reinterpret_cast<const uint4*>(from)[32 + lane];
+            from += 8 * 32 + lane;
+            const uint32_t sgn = from[0];
+            const uint32_t e4[8] = {ea.x, ea.y, ea.z, ea.w, eb.x, eb.y, eb.z, eb.w};
+            uint32_t zero = 0;  // some exponent byte is 0
 #pragma unroll
-                    for (int t = 0; t < 32; ++t) {
-                        const float base = __uint_as_float((t & 3) == 3 ? ((e4[t >> 2] >> 1) & 0x7F800000u)
-                                                                        : ((e4[t >> 2] << (23 - 8 * (t & 3))) & 0x7F800000u));
-                        const uint32_t mag = (pw1 & (1u << t)) ? m1 : 0x3F800000u;
-                        acc[t] = fmaf(base, __uint_as_float(mag ^ ((sgn << (31 - t)) & 0x80000000u)), acc[t]);
-                    }
-                } else {
-                    uint32_t f[32];
+            for (int q = 0; q < 8; ++q) zero |= (e4[q] - 0x01010101u) & ~e4[q] & 0x80808080u;
+            // 2^(E - 127) of entry t
+            auto base = [&](int t) {
+                return __uint_as_float((t & 3) == 3 ? ((e4[t >> 2] >> 1) & 0x7F800000u) : ((e4[t >> 2] << (23 - 8 * (t & 3))) & 0x7F800000u));
+            };
+            if (zero == 0u && w == 1) {
+                const uint32_t pw1 = from[32], m1 = __float_as_uint(1.0f + c);
 #pragma unroll
-                    for (int t = 0; t < 32; ++t) f[t] = (pw1 >> t) & 1u;
-                    const uint32_t* pm = planes + (int64_t)(m0 + i) * (1 + w_max) * words + at;
-                    for (int j = 2; j <= w; ++j) {
-                        const uint32_t pw = __ldg(pm + (int64_t)j * words);
+                for (int t = 0; t < 32; ++t) {
+                    const uint32_t mag = (pw1 & (1u << t)) ? m1 : 0x3F800000u;
+                    acc[t] = fmaf(base(t), __uint_as_float(mag ^ ((sgn << (31 - t)) & 0x80000000u)), acc[t]);
+                }
+            } else if (zero == 0u && w <= kAvgPlanes && c < 0x1p100f) {
+                uint32_t fb[8];
 #pragma unroll
-                        for (int t = 0; t < 32; ++t) f[t] = (f[t] << 1) | ((pw >> t) & 1u);
-                    }
+                for (int k = 0; k < 8; ++k) fb[k] = k < w ? from[(1 + k) * 32] : 0u;
+                fields_to_bytes(fb);
+                const float offset = -8388608.0f * c;
 #pragma unroll
-                    for (int t = 0; t < 32; ++t) {
-                        const uint32_t E = (e4[t >> 2] >> (8 * (t & 3))) & 0xFFu;
-                        const float base = __uint_as_float(E << 23);                   // 2^(E - 127), or 0
-                        const float scale = __uint_as_float(max(E, 1u) << 23);         // 2^(max(E, 1) - 127)
-                        const float ff = __uint_as_float(0x4B000000u | f[t]) - 8388608.0f;  // exact integer-to-float
-                        const float v = fmaf(ff * c, scale, base);  // the power of two last: ff c is a normal number
-                        acc[t] += __uint_as_float(__float_as_uint(v) ^ ((sgn << (31 - t)) & 0x80000000u));
-                    }
+                for (int t = 0; t < 32; ++t) {  // (1 + f c) 2^(E - 127): the power of two is exact
+                    const uint32_t mag = __float_as_uint(1.0f + field_times(fb, t, c, offset));
+                    acc[t] = fmaf(base(t), __uint_as_float(mag ^ ((sgn << (31 - t)) & 0x80000000u)), acc[t]);
+                }
+            } else {
+                uint32_t f[32];
+                gather_fields(planes + ((int64_t)m * (1 + w_max) + 1) * words + at, words, w, f);
+#pragma unroll
+                for (int t = 0; t < 32; ++t) {
+                    const uint32_t E = (e4[t >> 2] >> (8 * (t & 3))) & 0xFFu;
+                    const float low = __uint_as_float(E << 23);                    // 2^(E - 127), or 0
+                    const float scale = __uint_as_float(max(E, 1u) << 23);         // 2^(max(E, 1) - 127)
+                    const float ff = __uint_as_float(0x4B000000u | f[t]) - 8388608.0f;  // exact integer-to-float
+                    const float v = fmaf(ff * c, scale, low);  // the power of two last: ff c is a normal number
+                    acc[t] += __uint_as_float(__float_as_uint(v) ^ ((sgn << (31 - t)) & 0x80000000u));
                 }
             }
         }
-#pragma unroll
-        for (int t = 0; t < 32; ++t) sh_out[warp][lane][t] = acc[t] * inv_M;
-        __syncwarp();
-        const int64_t wbase = blk * kFloatThreads + warp * 32;
-#pragma unroll 4
-        for (int r = 0; r < 32; ++r) {
-            const int64_t i = (wbase + r) * 32 + lane;
-            if (i < d) out[i] = sh_out[warp][r][lane];
-        }
-        __syncwarp();
+        cp_async_wait<0>();
+        store_words(ring, acc, inv_M, blk * kAvgThreads + warp * 32, d, out);
     }
 }
 
@@ -272,7 +283,9 @@ size_t float_pack_smem(size_t elem) { return (kFloatThreads / 32) * 2 * 1024 * e
 }  // namespace
 
 int configure_float_kernels() {
-    const bool ok = cudaFuncSetAttribute(float_pack_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    const bool ok = cudaFuncSetAttribute(aggregate_float_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)kAvgFloatSmem + kEmitMaxWorkers * 8) == cudaSuccess &&
+                    cudaFuncSetAttribute(float_pack_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)float_pack_smem(4)) == cudaSuccess;
     return ok ? MLMC_OK : MLMC_ERR_CUDA;
 }
@@ -299,10 +312,10 @@ void launch_aggregate_floatbits(Workspace& ws, const mlmc_float_msgs& msgs, cons
                                 float* out, cudaStream_t s) {
     const MantissaSchedule sc = make_mantissa_schedule(mb, L);
     const int64_t words = (d + 31) / 32;
-    int64_t nb = (words + kFloatThreads - 1) / kFloatThreads;
-    const int64_t cap = (int64_t)ws.sm_count * 8;
-    if (nb > cap) nb = cap;
-    launch_kernel(ws, K_AGG_FLOAT, aggregate_float_kernel, dim3((unsigned)nb), kFloatThreads, 0, s, msgs.expo, msgs.planes,
+    const size_t smem = kAvgFloatSmem + (size_t)M * 8;
+    static const int resident = resident_blocks(aggregate_float_kernel, kAvgThreads, kAvgFloatSmem + 64);
+    const int64_t nb = std::min((words + kAvgThreads - 1) / kAvgThreads, (int64_t)ws.sm_count * resident * 2);
+    launch_kernel(ws, K_AGG_FLOAT, aggregate_float_kernel, dim3((unsigned)nb), kAvgThreads, smem, s, msgs.expo, msgs.planes,
                   msgs.level, msgs.p_sel, sc, msgs.w_max, words, M, d, out);
 }
 
