@@ -23,9 +23,9 @@ struct BitSchedule {
     int width[kMaxLevels];      // w_l
     int bits[kMaxLevels];       // b_l
     // levels of at most 8 bits in runs of at most 8 bits together
-    int run_shift[kMaxLevels];  // B - the b of the run's last level
-    int in_run[kMaxLevels];     // the last level's b - b_l
-    uint32_t mask4[kMaxLevels]; // 2^{w_l} - 1 in every byte
+    uint32_t run_up[kMaxLevels];  // moves the run to the top byte of the code: 2^(24 - B + b of its last level)
+    int in_run[kMaxLevels];       // the last level's b - b_l: where the field sits in the byte
+    uint32_t mask4[kMaxLevels];   // the field's bits, in every byte
 };
 
 // The code of an entry at b bits, min(trunc(e 2^b), 2^b - 1) with the IEEE-rounded fp32 quotient e = fl32(|g| / gmax).  (The
@@ -48,18 +48,23 @@ struct Quantiser {
     // The codes of N entries at b bits (scale 2^b, b <= 23): in the low 23 bits, the bits of 2^23 above.
     template <int N>
     __device__ __forceinline__ void codes(const float (&v)[N], float scale, uint32_t (&q)[N]) const {
-        float x[N];
-#pragma unroll
-        for (int i = 0; i < N; ++i) x[i] = fabsf(v[i]);
         if (move != 1.0f) {
+            float x[N];
 #pragma unroll
-            for (int i = 0; i < N; ++i) x[i] *= move;
+            for (int i = 0; i < N; ++i) x[i] = v[i] * move;
+            quotients(x, scale, q);
+        } else {
+            quotients(v, scale, q);
         }
+    }
+    template <int N>
+    __device__ __forceinline__ void quotients(const float (&v)[N], float scale, uint32_t (&q)[N]) const {
 #pragma unroll
         for (int i = 0; i < N; ++i) {
-            float e = __fmul_rn(x[i], inv);
-            e = __fmaf_rn(__fmaf_rn(-e, gmax, x[i]), inv, e);
-            e = __fmaf_rn(__fmaf_rn(-e, gmax, x[i]), inv, e);
+            const float x = fabsf(v[i]);
+            float e = __fmul_rn(x, inv);
+            e = __fmaf_rn(__fmaf_rn(-e, gmax, x), inv, e);
+            e = __fmaf_rn(__fmaf_rn(-e, gmax, x), inv, e);
             // e = 1 has no b-bit fraction: the largest e below it has the code 2^b - 1
             q[i] = __float_as_uint(__fmaf_rz(fminf(e, 0x1.fffffep-1f), scale, 8388608.0f));
         }
@@ -139,36 +144,37 @@ absmax_kernel(const T* __restrict__ g, int64_t d, int64_t ld, uint32_t* gmax_bit
 // A warp takes its entries level by level, kBitHeld per lane, from the first level at which the largest of them has a code
 // above 0 (the coarse levels of a gradient with per-layer scales are nearly all zero).  Fields of at most 8 bits are summed
 // four entries per instruction: levels that share a byte (1, 1, 2 and 4 bits, say) are packed into words of four entries
-// once, then a level is a shift, a mask and a byte product.  The instructions bound the kernel.  8 x 124M fp32 entries, six
-// levels: 1.0 ms with every entry taken through every level and the fp64 quotient, 0.82 field by field, now 0.76 (bf16 codes of 36M x 16: 0.55 -> 0.41).
+// once, then a level is a mask and a byte product.  Shifts are multiplications where they can be: the shifter and the logic
+// share a pipe of half the rate, which bound the kernel.  8 x 124M fp32 entries, six
+// levels: 1.0 ms with every entry taken through every level and the fp64 quotient, 0.82 field by field, now 0.73 (bf16 codes of 36M x 16: 0.55 -> 0.37).
 constexpr int kBitHeld = 8;
 
 template <typename T, int LMAX, typename Acc>
 __device__ __forceinline__ void take_fields(const float (&v)[kBitHeld], const Quantiser& qz, float scale, const int (&zero_below)[LMAX],
                                             const BitSchedule& sc, Acc (&acc)[LMAX]) {
-    int mx = 0;
+    float top = 0.0f;
 #pragma unroll
-    for (int e = 0; e < kBitHeld; ++e) mx = max(mx, __float_as_int(v[e]) & 0x7FFFFFFF);
-    mx = __reduce_max_sync(0xFFFFFFFFu, mx);
+    for (int e = 0; e < kBitHeld; ++e) top = fmaxf(top, fabsf(v[e]));
+    const int mx = __reduce_max_sync(0xFFFFFFFFu, __float_as_int(top));
     if (mx < zero_below[LMAX - 1]) return;  // the thresholds fall with the level; those past L repeat the last
     if constexpr (sizeof(Acc) == 4) {
         uint32_t q[kBitHeld], w[kBitHeld / 4];
-        int run = -1;
+        uint32_t run = 0u;
         qz.codes(v, scale, q);
 #pragma unroll
         for (int l = 0; l < LMAX; ++l) {
             if (l >= sc.L) break;
             if (mx < zero_below[l]) continue;
-            if (sc.run_shift[l] != run) {  // the byte of the run of every entry, four per word
-                run = sc.run_shift[l];
+            if (sc.run_up[l] != run) {  // the byte of the run of every entry, four per word
+                run = sc.run_up[l];
 #pragma unroll
                 for (int e = 0; e < kBitHeld; e += 4)
-                    w[e / 4] = __byte_perm(__byte_perm(q[e] >> run, q[e + 1] >> run, 0x0040),
-                                           __byte_perm(q[e + 2] >> run, q[e + 3] >> run, 0x0040), 0x5410);
+                    w[e / 4] = __byte_perm(__byte_perm(q[e] * run, q[e + 1] * run, 0x0073),
+                                           __byte_perm(q[e + 2] * run, q[e + 3] * run, 0x0073), 0x5410);
             }
 #pragma unroll
-            for (int e = 0; e < kBitHeld / 4; ++e) {
-                const uint32_t f = (w[e] >> sc.in_run[l]) & sc.mask4[l];
+            for (int e = 0; e < kBitHeld / 4; ++e) {  // the field stays where it is: its square counts 2^(2 in_run)
+                const uint32_t f = w[e] & sc.mask4[l];
                 acc[l] = __dp4a(f, f, acc[l]);
             }
         }
@@ -271,7 +277,7 @@ bit_stats_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t*
 #pragma unroll
     for (int l = 0; l < LMAX; ++l) {
         if (l >= sc.L) break;
-        unsigned long long x = (unsigned long long)acc[l];
+        unsigned long long x = (unsigned long long)(sizeof(Acc) == 4 ? acc[l] >> (2 * sc.in_run[l]) : acc[l]);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xFFFFFFFFu, x, o);
         if ((threadIdx.x & 31) == 0) sh_red[l][threadIdx.x >> 5] = x;
@@ -447,6 +453,8 @@ bit_cluster_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid_
                 take_fields<T, kDenseLevels, uint32_t>(v, qz, (float)(1u << sc.B), zero_below, sc, acc);
             }
         }
+#pragma unroll
+        for (int l = 0; l < kDenseLevels; ++l) acc[l] >>= 2 * sc.in_run[l];
         const unsigned long long S = dense_sums(cluster, acc, sh);
         if (threadIdx.x < sc.L) delta = (double)gmax * ldexp(1.0, -sc.bits[threadIdx.x]) * sqrt((double)S);
     }
@@ -554,13 +562,13 @@ BitSchedule make_schedule(const int32_t* b, int L) {
         sc.width[l] = w;
         sc.shift[l] = sc.B - b[l];
         sc.mask[l] = (w >= 32) ? 0xFFFFFFFFu : ((1u << w) - 1u);
-        sc.mask4[l] = (sc.mask[l] & 0xFFu) * 0x01010101u;
     }
     for (int l = 0, end; l < L; l = end) {
         for (end = l + 1; end < L && b[end] - (l ? b[l - 1] : 0) <= 8;) ++end;
         for (int i = l; i < end; ++i) {
-            sc.run_shift[i] = sc.B - b[end - 1];
+            sc.run_up[i] = 1u << (24 - sc.B + b[end - 1]);
             sc.in_run[i] = b[end - 1] - b[i];
+            sc.mask4[i] = ((sc.mask[i] << sc.in_run[i]) & 0xFFu) * 0x01010101u;
         }
     }
     return sc;
