@@ -284,8 +284,7 @@ int mlmc_create(mlmc_ctx** out, int device, int64_t d_max, int M_max, int L_max)
     const size_t o_bhit = pl.take(sizeof(int) * M_max);
     const size_t o_bstat = pl.take(sizeof(unsigned long long) * 4);
     ws.seg_scratch = nullptr;
-    ws.seg_rows = 0;
-    ws.seg_cap = 0;
+    ws.seg_bytes = 0;
     ws.sig_d = ws.sig_ld = -1;
     ws.sig_M = ws.sig_L = ws.sig_dtype = -1;
 
@@ -592,7 +591,7 @@ int mlmc_compress_stopk(mlmc_ctx* ctx, const void* g, int dtype, int64_t d, int 
         // Adaptive p with many segments: Lemma 3.4 needs the norm of every segment
         DeviceGuard guard(ws.device);
         cudaStream_t s = static_cast<cudaStream_t>(stream);
-        if (int rc = reserve_segments(ws, L)) return rc;
+        if (int rc = reserve_segments(ws)) return rc;
         set_call_size(ws, d, M, dtype == MLMC_BF16 ? 2 : 4);
         launch_begin_adaptive(ws, dtype, d, M, nullptr, 1, s);
         launch_hist1(ws, g, dtype, d, M, ld, false, s);

@@ -150,9 +150,8 @@ struct Workspace {
     int64_t sig_k[kMaxLevels];
     // s-Top-k with more levels than kMaxLevels
     int64_t big_cap;             // most levels
-    void* seg_scratch;           // buffers of the segment norms (stopk_segments.cu) for seg_rows rows and seg_cap segments; allocated at first use
-    int seg_rows;
-    int64_t seg_cap;
+    void* seg_scratch;           // buffers of the segment norms (stopk_segments.cu), allocated at first use
+    size_t seg_bytes;
     // RTN: per-block residual energies of every level
     double* rtn_partial;         // [M][rtn_ctas][kMaxLevels]
     int rtn_ctas;
@@ -617,7 +616,7 @@ void launch_cluster_topk(Workspace& ws, const void* g, int dtype, int64_t d, int
                          const DrawnBand* bands, const mlmc_topk_msgs* out, cudaStream_t s);
 // stopk_segments.cu: s-Top-k with adaptive p and many segments
 int configure_segment_kernels();
-int reserve_segments(Workspace& ws, int64_t L);
+int reserve_segments(Workspace& ws);
 void launch_segments(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, int64_t s_len, int64_t L,
                      uint64_t seed, uint64_t step, cudaStream_t s);
 

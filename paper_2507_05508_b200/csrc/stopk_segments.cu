@@ -52,7 +52,7 @@ struct RowHead {
 
 // Scratch memory of the rows that are taken together, by row strides.
 struct SegScratch {
-    uint32_t* keys;          // [rows][d_max]       keys of the buckets
+    uint32_t* keys;          // [rows][d]           keys of the buckets
     uint16_t* table;         // [rows][kBins1]      bin -> cell, or 0x8000 | bucket
     Bucket* bucket;          // [rows][kBins1]
     Wide* bucket_sum;        // [rows][kBins1]      energy of a bucket
@@ -766,10 +766,10 @@ struct SegPlanner {
     }
 };
 
-size_t plan_scratch(char* base, int rows, int64_t d_max, int64_t seg_cap, SegScratch* sc) {
+size_t plan_scratch(char* base, int rows, int64_t d, int64_t seg_cap, SegScratch* sc) {
     SegPlanner pl{base};
     const size_t r = (size_t)rows;
-    sc->keys = pl.take<uint32_t>(r * d_max);
+    sc->keys = pl.take<uint32_t>(r * d);
     sc->table = pl.take<uint16_t>(r * kBins1);
     sc->bucket = pl.take<Bucket>(r * kBins1);
     sc->bucket_sum = pl.take<Wide>(r * kBins1);
@@ -781,7 +781,7 @@ size_t plan_scratch(char* base, int rows, int64_t d_max, int64_t seg_cap, SegScr
     sc->prefix = pl.take<Wide>(r * seg_cap);
     sc->delta = pl.take<double>(r * seg_cap);
     sc->head = pl.take<RowHead>(r);
-    sc->key_stride = d_max;
+    sc->key_stride = d;
     sc->seg_cap = seg_cap;
     return pl.off + 256;
 }
@@ -795,22 +795,22 @@ int configure_segment_kernels() {
     return ok ? MLMC_OK : MLMC_ERR_CUDA;
 }
 
-// Scratch memory for L segments per row: as many rows together as fit in the budget (at least one, at most M_max).
-// Taken at the first call, and again when a later call has more segments than it was taken for.
-int reserve_segments(Workspace& ws, int64_t L) {
-    if (ws.seg_scratch && L <= ws.seg_cap) return MLMC_OK;
-    if (ws.seg_scratch) cudaFree(ws.seg_scratch);
-    ws.seg_scratch = nullptr;
-    const int64_t cap = std::min(ws.big_cap, std::max(L, (int64_t)4096));
+// Scratch memory, taken at the first call and kept as it is until the context is destroyed: room for as many rows of d_max
+// keys and 4096 segments as fit in the budget (at most M_max), and in any case for one row with the most segments.  How many
+// rows a call takes together follows from its own d and L.  (It never moves, so that a captured graph keeps valid addresses and
+// no later call has to allocate.)
+int reserve_segments(Workspace& ws) {
+    if (ws.seg_scratch) return MLMC_OK;
     SegScratch sc;
-    const size_t one = plan_scratch(nullptr, 1, ws.d_max, cap, &sc);
-    ws.seg_rows = (int)std::min<int64_t>(ws.M_max, std::max<int64_t>(1, (int64_t)(kSegScratchBudget / one)));
-    if (cudaMalloc(&ws.seg_scratch, plan_scratch(nullptr, ws.seg_rows, ws.d_max, cap, &sc)) != cudaSuccess) {
+    const int64_t few = std::min(ws.big_cap, (int64_t)4096);
+    const int64_t rows = std::max<int64_t>(1, (int64_t)(kSegScratchBudget / plan_scratch(nullptr, 1, ws.d_max, few, &sc)));
+    ws.seg_bytes = std::max(plan_scratch(nullptr, (int)std::min<int64_t>(ws.M_max, rows), ws.d_max, few, &sc),
+                            plan_scratch(nullptr, 1, ws.d_max, ws.big_cap, &sc));
+    if (cudaMalloc(&ws.seg_scratch, ws.seg_bytes) != cudaSuccess) {
         cudaGetLastError();
         ws.seg_scratch = nullptr;
         return MLMC_ERR_NOMEM;
     }
-    ws.seg_cap = cap;
     return MLMC_OK;
 }
 
@@ -818,10 +818,12 @@ int reserve_segments(Workspace& ws, int64_t L) {
 void launch_segments(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, int64_t s_len, int64_t L,
                      uint64_t seed, uint64_t step, cudaStream_t s) {
     SegScratch sc;
-    plan_scratch(static_cast<char*>(ws.seg_scratch), ws.seg_rows, ws.d_max, ws.seg_cap, &sc);
+    int together = (int)std::min<size_t>((size_t)M, ws.seg_bytes / plan_scratch(nullptr, 1, d, L, &sc));  // at least 1
+    while (together < M && plan_scratch(nullptr, together + 1, d, L, &sc) <= ws.seg_bytes) ++together;
+    plan_scratch(static_cast<char*>(ws.seg_scratch), together, d, L, &sc);
     const uint32_t sl = (uint32_t)s_len, nl = (uint32_t)L, du = (uint32_t)d;
-    for (int m0 = 0; m0 < M; m0 += ws.seg_rows) {
-        const int rows = std::min(ws.seg_rows, M - m0);
+    for (int m0 = 0; m0 < M; m0 += together) {
+        const int rows = std::min(together, M - m0);
         auto resolve = [&](auto kernel) {
             launch_kernel(ws, K_SEG_RESOLVE, kernel, dim3(rows), kSegThreads, 0, s, ws.hist1, m0, sl, nl, sc, ws.worker_err);
         };

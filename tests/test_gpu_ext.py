@@ -372,3 +372,32 @@ def test_stopk_adaptive_segment_norms_edges(B, ora, ctx, case):
         for d in (8191, 8192, 8195, 24_576):
             g_np = (rng.standard_normal((2, d)) * 10.0 ** rng.uniform(-2, 0, (2, d))).astype(np.float32)
             check_stopk(B, ora, ctx, to_dev(g_np), d // 40, None, 8, d, expect_excluded=1)
+
+
+def test_stopk_adaptive_scratch_stays_where_it_is(B, ora):
+    """The scratch memory of the segment norms is taken once: a call captured in a graph may have more segments than any call
+    before it, and a replay still holds after later calls with many more."""
+    rng = np.random.default_rng(62)
+    d = 60_001
+    c = B.mlmc_create(0, d, 2, 32)
+    try:
+        first = to_dev(rng.standard_normal((2, d)).astype(np.float32))
+        check_stopk(B, ora, c, first, d // 40, None, 9, 0, expect_excluded=1)      # takes the scratch memory
+        g = to_dev(rng.standard_normal((2, d)).astype(np.float32))
+        graphs = []
+        for s in (1000, 9):                                                        # 61 and 6667 segments
+            ref, out = B.TopkBuffers(2, s), B.TopkBuffers(2, s)
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph):
+                B.mlmc_compress_stopk(c, g, s, None, 9, 1, out)
+            graphs.append((graph, s, ref, out))
+        check_stopk(B, ora, c, first, 1, None, 9, 2, expect_excluded=1)            # 60,001 segments
+        for graph, s, ref, out in graphs:
+            B.mlmc_compress_stopk(c, g, s, None, 9, 1, ref)
+            graph.replay()
+            assert B.mlmc_get_status(c) == B.MLMC_OK
+            assert torch.equal(out.level, ref.level) and torch.equal(out.p_sel, ref.p_sel) and torch.equal(out.count, ref.count)
+            for m, n in enumerate(ref.count.tolist()):
+                assert torch.equal(out.idx[m, :n], ref.idx[m, :n]) and torch.equal(out.val[m, :n], ref.val[m, :n])
+    finally:
+        B.mlmc_destroy(c)
