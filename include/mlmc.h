@@ -169,7 +169,7 @@ int mlmc_compress_floatbits(mlmc_ctx* ctx, const void* g, int dtype, int64_t d, 
                             const int32_t* mb, int L, const double* p, uint64_t seed, uint64_t step,
                             const mlmc_float_msgs* out, void* stream);
 
-/* Server average of floating-point messages into dense out[d] (fp32, worker order 0..M-1). */
+/* Server average of floating-point messages into dense out[d] (fp32, worker order 0..M-1).  expo must be 16-byte aligned. */
 int mlmc_aggregate_floatbits(mlmc_ctx* ctx, const mlmc_float_msgs* msgs, const int32_t* mb, int L, int M, int64_t d,
                              float* out, void* stream);
 

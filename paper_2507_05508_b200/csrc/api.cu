@@ -654,6 +654,7 @@ int mlmc_compress_floatbits(mlmc_ctx* ctx, const void* g, int dtype, int64_t d, 
 int mlmc_aggregate_floatbits(mlmc_ctx* ctx, const mlmc_float_msgs* msgs, const int32_t* mb, int L, int M, int64_t d,
                              float* out, void* stream) {
     if (!ctx || !msgs || !out || !msgs->expo || !msgs->planes || !msgs->level || !msgs->p_sel) return MLMC_ERR_ARG;
+    if (reinterpret_cast<uintptr_t>(msgs->expo) % 16 != 0) return MLMC_ERR_ARG;  // read 16 bytes at a time
     Workspace& ws = ctx->ws;
     if (d < 1 || d > ws.d_max || M < 1 || M > ws.M_max || L < 1 || L > kMaxLevels) return MLMC_ERR_ARG;
     if (!mb) return MLMC_ERR_ARG;

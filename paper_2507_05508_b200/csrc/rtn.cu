@@ -396,7 +396,8 @@ aggregate_dense_kernel(const float* __restrict__ val, const int32_t* level, int 
                        float* __restrict__ out) {
     pdl_enter();
     const float inv_M = 1.0f / (float)M;
-    const int64_t n4 = (ldv % 4 == 0 && reinterpret_cast<uintptr_t>(out) % 16 == 0) ? d / 4 : 0;
+    const bool aligned = ldv % 4 == 0 && ((reinterpret_cast<uintptr_t>(val) | reinterpret_cast<uintptr_t>(out)) & 15) == 0;
+    const int64_t n4 = aligned ? d / 4 : 0;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n4; v += (int64_t)gridDim.x * blockDim.x) {
         float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
         for (int m = 0; m < M; ++m) {

@@ -273,7 +273,7 @@ aggregate_topk_kernel(const uint32_t* __restrict__ idx, const float* __restrict_
                 __syncthreads();
             }
         }
-        if (base + kAggTile <= d && (d & 3) == 0) {
+        if (base + kAggTile <= d && reinterpret_cast<uintptr_t>(out) % 16 == 0) {
             for (int i = threadIdx.x; i < kAggTile / 4; i += blockDim.x) {
                 float4 x = reinterpret_cast<const float4*>(acc)[i];
                 x.x *= inv_M; x.y *= inv_M; x.z *= inv_M; x.w *= inv_M;
@@ -374,7 +374,7 @@ aggregate_topk_warps_kernel(const uint32_t* __restrict__ idx, const float* __res
                 }
             }
         }
-        if (base + kAggSub <= d && (d & 3) == 0) {
+        if (base + kAggSub <= d && reinterpret_cast<uintptr_t>(out) % 16 == 0) {
 #pragma unroll
             for (int i = 0; i < kAggSub / 128; ++i) {
                 float4 x = reinterpret_cast<const float4*>(acc)[i * 32 + lane];

@@ -141,3 +141,38 @@ def test_floatbits_lengths(B, ora, ctx, mb, d):
 @pytest.mark.parametrize("d", [460_800, 460_801, 1_000_003])
 def test_rtn_long_rows(B, ora, ctx, r, d):
     check_rtn(B, ora, ctx, layered(d, 1), r, None, 3, 0)
+
+
+# buffers that start at any element: the averages take vectors only where the addresses allow it
+@pytest.mark.parametrize("d", [8_192, 2_424_836])
+def test_averages_into_unaligned_buffers(B, ctx, d):
+    M, k = 2, [d // 50, d]
+    g = layered(d, M)
+    plain = torch.empty(d, dtype=torch.float32, device="cuda")
+    shifted = torch.full((d + 8,), float("nan"), dtype=torch.float32, device="cuda")
+    for off in (1, 2, 3):
+        msgs = B.TopkBuffers(M, d)
+        B.mlmc_compress_topk(ctx, g, k, [0.5, 0.5], 3, off, msgs)
+        for average in (lambda out: B.mlmc_aggregate(ctx, B.MLMC_TOPK, msgs, None, M, d, out),
+                        lambda out: B.mlmc_aggregate_topk_noalloc(msgs, M, d, out)):
+            average(plain)
+            average(shifted[off:off + d])
+            assert torch.equal(plain, shifted[off:off + d])
+        rtn, moved = B.RtnBuffers(M, d), B.RtnBuffers(M, d)
+        B.mlmc_compress_rtn(ctx, g, [2, 4], [0.3, 0.3, 0.4], 3, off, rtn)
+        room = torch.zeros(M * rtn.ldv + 8, dtype=torch.float32, device="cuda")
+        val = room[off:off + M * rtn.ldv]
+        val.copy_(rtn.val.flatten())
+        moved.level.copy_(rtn.level)
+        moved.struct.val = val.data_ptr()
+        B.mlmc_aggregate_rtn(ctx, rtn, M, d, plain)
+        for msg in (rtn, moved):
+            for out in (torch.empty(d, dtype=torch.float32, device="cuda"), shifted[off:off + d]):
+                B.mlmc_aggregate_rtn(ctx, msg, M, d, out)
+                assert torch.equal(plain, out)
+    assert B.mlmc_get_status(ctx) == B.MLMC_OK
+    floats = B.FloatBuffers(M, d, 23)
+    floats.struct.expo += 4
+    with pytest.raises(B.MlmcError) as e:
+        B.mlmc_aggregate_floatbits(ctx, floats, [23], M, d, plain)
+    assert e.value.code == B.MLMC_ERR_ARG
