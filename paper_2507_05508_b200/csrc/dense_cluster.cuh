@@ -139,7 +139,7 @@ __device__ __forceinline__ int dense_level(const DrawPlan& pl, const DrawnLevels
     if (adaptive) {
         if (threadIdx.x < 32) {
             double p;
-            const int drawn_level = warp_draw(delta, counter_uniform(pl.seed, pl.step, (uint64_t)m), &p);
+            const int drawn_level = warp_draw(delta, pl.L, counter_uniform(pl.seed, pl.step, (uint64_t)m), &p);
             if (first && lane < pl.L) {
                 pl.delta_all[m * kMaxLevels + lane] = delta;
                 pl.p_all[m * kMaxLevels + lane] = p;

@@ -88,7 +88,7 @@ __device__ void finish_selection(const FinishPlan& pl, int m, int is_bf16, const
             delta = sqrt(e);
         }
         double p;
-        level = warp_draw(delta, counter_uniform(pl.seed, pl.step, (uint64_t)m), &p);
+        level = warp_draw(delta, L, counter_uniform(pl.seed, pl.step, (uint64_t)m), &p);
         if (l < L) {
             p_all[m * kMaxLevels + l] = p;
             delta_all[m * kMaxLevels + l] = delta;

@@ -176,3 +176,52 @@ def test_averages_into_unaligned_buffers(B, ctx, d):
     with pytest.raises(B.MlmcError) as e:
         B.mlmc_aggregate_floatbits(ctx, floats, [23], M, d, plain)
     assert e.value.code == B.MLMC_ERR_ARG
+
+
+# p_l = Delta_l / sum Delta and the running sums of the draw go over the levels in ascending order, on every path: the results
+# follow bit for bit from the norms
+@pytest.mark.parametrize("kind,d,M", [("topk", 9_001, 16), ("topk", 9_001, 40), ("topk", 1_100_001, 12), ("bitwise", 9_001, 16),
+                                      ("bitwise", 500_001, 12), ("rtn", 9_001, 16), ("rtn", 500_001, 12)])
+def test_probabilities_and_draw_follow_from_the_norms(B, kind, d, M):
+    g = layered(d, M)
+    sched = {"topk": doubling(d, 1 + d // 3000)[:30], "bitwise": BITS, "rtn": [2, 4, 8, 16]}[kind]
+    if kind == "topk":
+        sched[-1] = d
+    L = len(sched) + (kind == "rtn")
+    # the norms of both calls are exact integer sums but for RTN, where a short row's message and its norms by themselves come
+    # from different kernels: d additions in fp64, in another order
+    tol = d * 2.0 ** -53 if kind == "rtn" else 0.0
+    c = B.mlmc_create(0, d, M, 32)
+    try:
+        p_out = torch.zeros((M, L), dtype=torch.float64, device="cuda")
+        delta = torch.zeros((M, L), dtype=torch.float64, device="cuda")
+        code = {"topk": B.MLMC_TOPK, "bitwise": B.MLMC_BITWISE, "rtn": B.MLMC_RTN}[kind]
+        B.mlmc_level_probs(c, g, code, sched, None, p_out, delta)
+        p_out, delta = p_out.cpu().numpy(), delta.cpu().numpy()
+        for m in range(M):
+            total = 0.0
+            for x in delta[m].tolist():
+                total += x
+            assert (p_out[m] == delta[m] / total).all()
+        for step in range(6):
+            u = B.mlmc_read_u(c, 5, step, M)
+            if kind == "topk":
+                out = B.TopkBuffers(M, wl.max_band(sched))
+                B.mlmc_compress_topk(c, g, sched, None, 5, step, out)
+            elif kind == "bitwise":
+                out = B.BitBuffers(M, d, 8)
+                B.mlmc_compress_bitwise(c, g, sched, None, 5, step, out)
+            else:
+                out = B.RtnBuffers(M, d)
+                B.mlmc_compress_rtn(c, g, sched, None, 5, step, out)
+            assert B.mlmc_get_status(c) == B.MLMC_OK
+            levels, p_sel = out.level.tolist(), out.p_sel.tolist()
+            for m in range(M):
+                cdf, last = 0.0, max(l for l in range(L) if p_out[m, l] > 0)
+                for l in range(L):
+                    cdf += p_out[m, l]
+                    if u[m] < cdf or l == last:
+                        break
+                assert levels[m] == l and abs(p_sel[m] - p_out[m, l]) <= tol * p_out[m, l]
+    finally:
+        B.mlmc_destroy(c)
