@@ -1,5 +1,4 @@
 // C ABI of the MLMC compression library: context, argument checks and the launch sequences.
-#include <mutex>
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -180,30 +179,12 @@ void select_drawn(Workspace& ws, const void* g, int dtype, int64_t d, int M, int
     launch_emit(ws, g, dtype, d, M, ld, *out, s);
 }
 
-// Shared-memory limits of the kernels and the clusters that fit, set and asked for once per device in the life of the
-// process (a create after the first takes milliseconds less).
-bool configure_kernels(int device, KernelLimits* out) {
-    constexpr int kMostDevices = 64;
-    static std::mutex lock;
-    static bool known[kMostDevices];
-    static KernelLimits limits[kMostDevices];
-    std::lock_guard<std::mutex> hold(lock);
-    const bool keep = device < kMostDevices;
-    if (keep && known[device]) {
-        *out = limits[device];
-        return true;
-    }
-    KernelLimits l = {};
-    if (configure_select_kernels() != MLMC_OK || configure_emit_kernels() != MLMC_OK || configure_float_kernels() != MLMC_OK ||
-        configure_segment_kernels() != MLMC_OK || configure_rtn_kernels() != MLMC_OK || configure_cluster_kernels(&l) != MLMC_OK ||
-        configure_bit_kernels(&l) != MLMC_OK)
-        return false;
-    if (keep) {
-        limits[device] = l;
-        known[device] = true;
-    }
-    *out = l;
-    return true;
+// Shared-memory limits of the kernels, and what the device can place.  Both belong to the current CUDA context (a device
+// reset starts a new one), so every create sets and asks.
+bool configure_kernels(KernelLimits* limits) {
+    return configure_select_kernels() == MLMC_OK && configure_emit_kernels(limits) == MLMC_OK && configure_float_kernels(limits) == MLMC_OK &&
+           configure_segment_kernels() == MLMC_OK && configure_rtn_kernels(limits) == MLMC_OK && configure_cluster_kernels(limits) == MLMC_OK &&
+           configure_bit_kernels(limits) == MLMC_OK;
 }
 
 }  // namespace
@@ -218,8 +199,8 @@ int mlmc_create(mlmc_ctx** out, int device, int64_t d_max, int M_max, int L_max)
     if (!guard.ok) return MLMC_ERR_CUDA;
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return MLMC_ERR_CUDA;
-    KernelLimits limits;
-    if (!configure_kernels(device, &limits)) return MLMC_ERR_CUDA;
+    KernelLimits limits = {};
+    if (!configure_kernels(&limits)) return MLMC_ERR_CUDA;
 
     mlmc_ctx* ctx = new (std::nothrow) mlmc_ctx();
     if (!ctx) return MLMC_ERR_NOMEM;

@@ -593,6 +593,7 @@ int configure_bit_kernels(KernelLimits* limits) {
                     cudaFuncSetAttribute(bit_pack_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)bit_pack_smem(4)) == cudaSuccess;
     dense_cluster_fit(bit_cluster_kernel<float>, kBitDenseWarps * 32, limits);
+    limits->aggregate_bitwise = resident_blocks(aggregate_bitwise_kernel, kAvgThreads, kAvgBitSmem + 64);
     return ok ? MLMC_OK : MLMC_ERR_CUDA;
 }
 
@@ -703,8 +704,7 @@ void launch_aggregate_bitwise(Workspace& ws, const mlmc_bit_msgs& msgs, const in
     const int64_t words = (d + 31) / 32;
     const size_t smem = kAvgBitSmem + (size_t)M * 8;
     // whole waves only: every block does the same number of iterations, so a partial last wave costs a full one
-    static const int resident = resident_blocks(aggregate_bitwise_kernel, kAvgThreads, kAvgBitSmem + 64);
-    const int64_t nb = std::min((words + kAvgThreads - 1) / kAvgThreads, (int64_t)ws.sm_count * resident * 2);
+    const int64_t nb = std::min((words + kAvgThreads - 1) / kAvgThreads, (int64_t)ws.sm_count * ws.limits.aggregate_bitwise * 2);
     launch_kernel(ws, K_AGG_BIT, aggregate_bitwise_kernel, dim3((unsigned)nb), kAvgThreads, smem, s, msgs.planes, msgs.gmax,
                   msgs.level, msgs.p_sel, sc, msgs.w_max, words, M, d, out);
 }

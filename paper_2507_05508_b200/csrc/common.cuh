@@ -86,6 +86,10 @@ constexpr int kTimingPool = 2048;  // event pairs kept between two reads
 struct KernelLimits {
     int cluster_most;            // largest thread-block cluster of the short-row Top-k kernel (0: none)
     int dense_fit[5];            // clusters of 1, 2, .. 16 blocks of the short-row dense kernels that run at a time
+    // blocks per SM
+    int band_count[2];           // fp32, bf16
+    int aggregate_topk, aggregate_bitwise, aggregate_float;
+    int rtn_stats[2][2];         // fp32, bf16; few levels, many
 };
 
 struct Workspace {
@@ -573,7 +577,7 @@ void launch_band_header(Workspace& ws, int M, const FinishPlan& plan, cudaStream
 void launch_copy_probs(Workspace& ws, int M, int L, const double* p_fixed, double* p_out, double* delta_out,
                        cudaStream_t s);
 // topk_emit.cu
-int configure_emit_kernels();
+int configure_emit_kernels(KernelLimits* limits);
 void launch_emit(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const mlmc_topk_msgs& out,
                  cudaStream_t s);
 void launch_aggregate_topk(Workspace& ws, const mlmc_topk_msgs& msgs, int M, int64_t d, float* out, cudaStream_t s);
@@ -594,7 +598,7 @@ void launch_aggregate_bitwise(Workspace& ws, const mlmc_bit_msgs& msgs, const in
                               float* out, cudaStream_t s);
 
 // floatbits.cu
-int configure_float_kernels();
+int configure_float_kernels(KernelLimits* limits);
 void launch_compress_floatbits(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* mb,
                                int L, const double* p, uint64_t seed, uint64_t step, const mlmc_float_msgs& out, cudaStream_t s);
 void launch_aggregate_floatbits(Workspace& ws, const mlmc_float_msgs& msgs, const int32_t* mb, int L, int M, int64_t d,
@@ -604,7 +608,7 @@ DrawPlan rtn_draw_plan(Workspace& ws, int L, uint64_t seed, uint64_t step, const
 // Adaptive: residual energies of every level, probabilities, draw and header.
 void launch_rtn_stats(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* r, int L,
                       const DrawPlan& plan, cudaStream_t s);
-int configure_rtn_kernels();
+int configure_rtn_kernels(KernelLimits* limits);
 bool launch_rtn_cluster(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* r, int L,
                         const DrawPlan& plan, const double* p, const mlmc_rtn_msgs& out, cudaStream_t s);
 void launch_rtn_emit(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* r, int L,

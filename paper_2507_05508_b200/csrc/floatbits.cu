@@ -282,11 +282,12 @@ size_t float_pack_smem(size_t elem) { return (kFloatThreads / 32) * 2 * 1024 * e
 
 }  // namespace
 
-int configure_float_kernels() {
+int configure_float_kernels(KernelLimits* limits) {
     const bool ok = cudaFuncSetAttribute(aggregate_float_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)kAvgFloatSmem + kEmitMaxWorkers * 8) == cudaSuccess &&
                     cudaFuncSetAttribute(float_pack_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)float_pack_smem(4)) == cudaSuccess;
+    limits->aggregate_float = resident_blocks(aggregate_float_kernel, kAvgThreads, kAvgFloatSmem + 64);
     return ok ? MLMC_OK : MLMC_ERR_CUDA;
 }
 
@@ -313,8 +314,7 @@ void launch_aggregate_floatbits(Workspace& ws, const mlmc_float_msgs& msgs, cons
     const MantissaSchedule sc = make_mantissa_schedule(mb, L);
     const int64_t words = (d + 31) / 32;
     const size_t smem = kAvgFloatSmem + (size_t)M * 8;
-    static const int resident = resident_blocks(aggregate_float_kernel, kAvgThreads, kAvgFloatSmem + 64);
-    const int64_t nb = std::min((words + kAvgThreads - 1) / kAvgThreads, (int64_t)ws.sm_count * resident * 2);
+    const int64_t nb = std::min((words + kAvgThreads - 1) / kAvgThreads, (int64_t)ws.sm_count * ws.limits.aggregate_float * 2);
     launch_kernel(ws, K_AGG_FLOAT, aggregate_float_kernel, dim3((unsigned)nb), kAvgThreads, smem, s, msgs.expo, msgs.planes,
                   msgs.level, msgs.p_sel, sc, msgs.w_max, words, M, d, out);
 }

@@ -450,11 +450,13 @@ DrawPlan rtn_draw_plan(Workspace& ws, int L, uint64_t seed, uint64_t step, const
 }
 
 namespace {
+size_t rtn_stats_smem(size_t elem) { return (size_t)4 * kRtnThreads * kRtnHeld * elem; }
+
 template <typename T, int LMAX>
 void launch_rtn_stats_t(Workspace& ws, const T* g, int64_t d, int M, int64_t ld, const RtnSchedule& sc, const DrawPlan& plan,
                         cudaStream_t s) {
-    constexpr size_t smem = (size_t)4 * kRtnThreads * kRtnHeld * sizeof(T);
-    static const int resident = resident_blocks(rtn_stats_kernel<T, LMAX>, kRtnThreads, smem);
+    const size_t smem = rtn_stats_smem(sizeof(T));
+    const int resident = ws.limits.rtn_stats[sizeof(T) == 2][LMAX == kRtnMaxLevels];
     // whole waves (a partial last one costs a full one), four of them: how much a block skips differs (one: 910 us, two: 897,
     // four: 866 for 8 x 124M entries)
     const int nb = std::min(rtn_blocks(ws, d, ElemTraits<T>::kVec, M, 4 * resident), ws.rtn_ctas);
@@ -491,8 +493,13 @@ bool launch_rtn_cluster(Workspace& ws, const void* g, int dtype, int64_t d, int 
     return true;
 }
 
-int configure_rtn_kernels() {
-    return configure_dense_cluster(rtn_cluster_kernel<float>) && configure_dense_cluster(rtn_cluster_kernel<bf16_t>) ? MLMC_OK : MLMC_ERR_CUDA;
+int configure_rtn_kernels(KernelLimits* limits) {
+    if (!configure_dense_cluster(rtn_cluster_kernel<float>) || !configure_dense_cluster(rtn_cluster_kernel<bf16_t>)) return MLMC_ERR_CUDA;
+    limits->rtn_stats[0][0] = resident_blocks(rtn_stats_kernel<float, 6>, kRtnThreads, rtn_stats_smem(4));
+    limits->rtn_stats[0][1] = resident_blocks(rtn_stats_kernel<float, kRtnMaxLevels>, kRtnThreads, rtn_stats_smem(4));
+    limits->rtn_stats[1][0] = resident_blocks(rtn_stats_kernel<bf16_t, 6>, kRtnThreads, rtn_stats_smem(2));
+    limits->rtn_stats[1][1] = resident_blocks(rtn_stats_kernel<bf16_t, kRtnMaxLevels>, kRtnThreads, rtn_stats_smem(2));
+    return MLMC_OK;
 }
 
 void launch_rtn_emit(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* r, int L,

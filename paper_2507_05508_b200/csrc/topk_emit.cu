@@ -433,13 +433,16 @@ aggregate_topk_direct_kernel(const uint32_t* __restrict__ idx, const float* __re
 
 }  // namespace
 
-int configure_emit_kernels() {
+int configure_emit_kernels(KernelLimits* limits) {
     auto set = [](auto kernel, int words) {
         return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (kBandThreads / 32) * words * (int)sizeof(uint32_t)) == cudaSuccess;
     };
-    return set(band_write_kernel<float>, kWriteWords<float>) && set(band_write_kernel<bf16_t>, kWriteWords<bf16_t>) ? MLMC_OK
-                                                                                                                   : MLMC_ERR_CUDA;
+    if (!set(band_write_kernel<float>, kWriteWords<float>) || !set(band_write_kernel<bf16_t>, kWriteWords<bf16_t>)) return MLMC_ERR_CUDA;
+    limits->band_count[0] = resident_blocks(band_count_kernel<float>, kBandThreads, 256);
+    limits->band_count[1] = resident_blocks(band_count_kernel<bf16_t>, kBandThreads, 256);
+    limits->aggregate_topk = resident_blocks(aggregate_topk_warps_kernel, kAggWarps * 32, 0);
+    return MLMC_OK;
 }
 
 namespace {
@@ -457,7 +460,7 @@ void launch_emit_t(Workspace& ws, const T* g, int dtype, int64_t d, int M, int64
     launch_kernel(ws, K_TILE_LIST, tile_list_kernel, dim3((tpw + kBandThreads - 1) / kBandThreads, M), kBandThreads, 0, s,
                   ws.tile_max, tpw, ws.emit, EmitWord<T>::kCap, ws.tile_desc, ws.tile_list, ws.list_n);
     // two whole waves: the warps stride over the list, so a partial last wave costs a full one
-    static const int resident = resident_blocks(band_count_kernel<T>, kBandThreads, 256);
+    const int resident = ws.limits.band_count[dtype == MLMC_BF16];
     const int64_t by_work = ((int64_t)tpw * M + wpb - 1) / wpb;
     auto blocks = [&](int per_sm) { return (unsigned)std::min<int64_t>(by_work, (int64_t)ws.sm_count * per_sm * 2); };
     launch_kernel(ws, K_BAND_COUNT, band_count_kernel<T>, dim3(blocks(resident)), kBandThreads, (size_t)M * sizeof(uint2), s, g, d,
@@ -485,8 +488,7 @@ void launch_aggregate_topk(Workspace& ws, const mlmc_topk_msgs& msgs, int M, int
     const int64_t n_off = (int64_t)M * (ntiles + 1);
     launch_kernel(ws, K_AGG_OFFSETS, agg_offsets_kernel, dim3((unsigned)((n_off + 255) / 256)), 256, 0, s, msgs.idx, msgs.count,
                   msgs.level, msgs.capacity, M, ntiles, ws.agg_offsets);
-    static const int resident = resident_blocks(aggregate_topk_warps_kernel, kAggWarps * 32, 0);
-    const int grid = std::min(ntiles, ws.sm_count * resident);
+    const int grid = std::min(ntiles, ws.sm_count * ws.limits.aggregate_topk);
     launch_kernel(ws, K_AGG_TOPK, aggregate_topk_warps_kernel, dim3(grid), kAggWarps * 32, 0, s, msgs.idx, msgs.val,
                   msgs.capacity, M, d, ntiles, ws.agg_offsets, out);
 }

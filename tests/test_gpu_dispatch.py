@@ -225,3 +225,53 @@ def test_probabilities_and_draw_follow_from_the_norms(B, kind, d, M):
                 assert levels[m] == l and abs(p_sel[m] - p_out[m, l]) <= tol * p_out[m, l]
     finally:
         B.mlmc_destroy(c)
+
+
+RESET = """
+import ctypes, sys
+import numpy as np
+sys.path.insert(0, sys.argv[1])
+from paper_2507_05508_b200 import binding as B
+import oracle
+rt = ctypes.CDLL("libcudart.so.12")
+vp, sz = ctypes.c_void_p, ctypes.c_size_t
+rt.cudaMalloc.argtypes, rt.cudaMemcpy.argtypes = [vp, sz], [vp, vp, sz, ctypes.c_int]
+M, d, k = 2, 40_000, [100, 5000, 40_000]
+g = np.random.default_rng(1).standard_normal((M, d)).astype(np.float32)
+
+def device(n):
+    p = vp()
+    assert rt.cudaMalloc(ctypes.byref(p), n) == 0
+    return p.value
+
+for step in range(2):                      # the second round runs in a new CUDA context of the same process
+    ctx = B.mlmc_create(0, d, M, 32)
+    at = device(g.nbytes)
+    assert rt.cudaMemcpy(at, g.ctypes.data, g.nbytes, 1) == 0
+    fields = [device(M * d * 4), device(M * d * 4), device(M * 8), device(M * 4), device(M * 8)]
+    msgs = B.mlmc_topk_msgs(*fields, d)
+    sched = (ctypes.c_int64 * 3)(*k)
+    assert B.lib().mlmc_compress_topk(ctx, at, B.MLMC_F32, d, M, d, sched, 3, None, 1, step, ctypes.byref(msgs), None) == 0
+    assert B.lib().mlmc_get_status(ctx, None) == 0
+    level = np.zeros(M, np.int32)
+    idx = np.zeros((M, d), np.uint32)
+    assert rt.cudaMemcpy(level.ctypes.data, fields[3], level.nbytes, 2) == 0
+    assert rt.cudaMemcpy(idx.ctypes.data, fields[0], idx.nbytes, 2) == 0
+    for m in range(M):
+        o = oracle.topk(g[m], k, p=None, seed=1, step=step, worker=m)
+        assert level[m] == o.level and np.array_equal(idx[m, :o.idx.size], o.idx)
+    B.mlmc_destroy(ctx)
+    assert rt.cudaDeviceReset() == 0
+print("both contexts agree with the oracle")
+"""
+
+
+def test_create_after_a_device_reset(ora):
+    """Kernel attributes belong to the CUDA context: a context created after cudaDeviceReset (which ends the process's own
+    context only) works as the first one did."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", RESET, root], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "both contexts agree" in r.stdout, r.stdout + r.stderr
