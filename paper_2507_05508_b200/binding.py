@@ -10,6 +10,7 @@ import ctypes as C
 import os
 from typing import Optional, Sequence
 
+import numpy as np
 import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
@@ -124,12 +125,25 @@ def _check(rc: int, where: str) -> None:
 
 _host_arrays = {}     # (ctype, values) -> C array: a program hands over the same few schedules and probabilities step after step
 _HOST_ARRAYS_MOST = 64
+_HOST_ARRAY_LONGEST = 64      # (1000 numbers: 31 us to look up, 21 us to convert)
+
+
+_PLAIN = {True: frozenset((float, np.float64)), False: frozenset((int, np.int64, np.int32))}
+
+
+def _plain(ctype, values) -> bool:
+    """Only numbers that the C array takes, and takes alike where they compare equal (1.0 and 1 do, and c_int64 refuses one)."""
+    return type(values) in (list, tuple) and len(values) <= _HOST_ARRAY_LONGEST and \
+        _PLAIN[ctype is C.c_double].issuperset(map(type, values))
 
 
 def _host_array(ctype, values: Optional[Sequence]):
-    """The values as a C array (read only for the library), kept for the next call with equal values."""
+    """The values as a C array (read only for the library); one of plain numbers is kept for the next call with equal values."""
     if values is None:
         return None
+    if not _plain(ctype, values):
+        values = list(values)
+        return (ctype * len(values))(*values)
     key = (ctype, tuple(values))
     a = _host_arrays.get(key)
     if a is None:
@@ -248,7 +262,8 @@ def mlmc_aggregate_topk_noalloc(msgs: "TopkBuffers", M: int, d: int, out: torch.
 def mlmc_compress_stopk(ctx, g: torch.Tensor, s: int, p: Optional[Sequence[float]], seed: int, step: int,
                         out: "TopkBuffers") -> None:
     ptr, dt, d, M, ld = _g_args(g)
-    ph = _host_array(C.c_double, p) if p is None or len(p) <= 4096 else (C.c_double * len(p)).from_buffer_copy(memoryview(_as_f64(p)))
+    ph = None if p is None else _host_array(C.c_double, p) if _plain(C.c_double, p) else \
+        (C.c_double * len(p)).from_buffer_copy(memoryview(_as_f64(p)))
     _check(lib().mlmc_compress_stopk(ctx, ptr, dt, d, M, ld, s, ph, seed, step, C.byref(out.struct), _stream()),
            "mlmc_compress_stopk")
 

@@ -64,3 +64,29 @@ def test_generators_are_seeded_and_structured():
     w4 = wl.shrink(wl.C4, 10_000, 2)
     g4 = wl.gradients(w4, 0)
     assert g4.dtype.is_floating_point and g4.element_size() == 2 and wl.as_numpy_bits(g4).dtype == np.uint16
+
+
+def test_host_arrays_take_and_refuse_what_ctypes_does():
+    """Arrays are kept for equal plain numbers only: what ctypes takes or refuses does not depend on the calls before."""
+    from paper_2507_05508_b200 import binding as B
+    first = B._host_array(ctypes.c_int64, [1, 2])
+    assert list(first) == [1, 2] and B._host_array(ctypes.c_int64, (1, 2)) is first
+    for values in ([1.0, 2.0], [1, 2.0], ["1", "2"]):
+        try:
+            B._host_array(ctypes.c_int64, values)
+            assert False, values
+        except TypeError:
+            pass
+    assert list(B._host_array(ctypes.c_int64, np.array([1, 2]))) == [1, 2]
+    assert list(B._host_array(ctypes.c_double, [np.array(0.25), np.array(0.75)])) == [0.25, 0.75]      # not hashable
+    assert list(B._host_array(ctypes.c_double, (x / 4 for x in (1, 3)))) == [0.25, 0.75]
+    assert list(B._host_array(ctypes.c_double, [1])) == [1.0] and B._host_array(ctypes.c_double, None) is None
+    values = [0.5, 0.5]
+    kept = B._host_array(ctypes.c_double, values)
+    values[0] = 0.25
+    assert list(kept) == [0.5, 0.5] and list(B._host_array(ctypes.c_double, values)) == [0.25, 0.5]
+    for i in range(3 * B._HOST_ARRAYS_MOST):                 # bounded
+        B._host_array(ctypes.c_int32, [i])
+    assert len(B._host_arrays) <= B._HOST_ARRAYS_MOST
+    assert B._host_array(ctypes.c_double, [0.0] * (B._HOST_ARRAY_LONGEST + 1)) is not \
+        B._host_array(ctypes.c_double, [0.0] * (B._HOST_ARRAY_LONGEST + 1))
