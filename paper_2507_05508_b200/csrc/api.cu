@@ -183,7 +183,7 @@ void select_drawn(Workspace& ws, const void* g, int dtype, int64_t d, int M, int
 // reset starts a new one), so every create sets and asks.
 bool configure_kernels(KernelLimits* limits) {
     return configure_select_kernels() == MLMC_OK && configure_emit_kernels(limits) == MLMC_OK && configure_float_kernels(limits) == MLMC_OK &&
-           configure_segment_kernels() == MLMC_OK && configure_rtn_kernels(limits) == MLMC_OK && configure_cluster_kernels(limits) == MLMC_OK &&
+           configure_segment_kernels(limits) == MLMC_OK && configure_rtn_kernels(limits) == MLMC_OK && configure_cluster_kernels(limits) == MLMC_OK &&
            configure_bit_kernels(limits) == MLMC_OK;
 }
 
@@ -364,7 +364,7 @@ static const char* const kKernelNames[] = {
     "begin", "uniforms", "hist1", "resolve1", "sums_candidates", "cand_pass2", "cand_pass3", "band_header", "copy_probs", "emit",
     "agg_offsets", "aggregate_topk", "absmax", "bit_stats", "bit_pack", "aggregate_bitwise", "tile_list", "band_count",
     "float_pack", "aggregate_floatbits", "rtn_stats", "rtn_emit", "aggregate_dense", "segment_resolve",
-    "segment_sweep", "segment_buckets", "segment_norms", "segment_draw", "cluster_topk", "cluster_bitwise", "cluster_rtn"};
+    "segment_sweep", "segment_buckets", "segment_norms", "segment_draw", "cluster_topk", "cluster_bitwise", "cluster_rtn", "sort_rows"};
 static_assert(sizeof(kKernelNames) / sizeof(kKernelNames[0]) == K_COUNT, "a name for every kernel id");
 
 int mlmc_kernel_count(void) { return K_COUNT; }

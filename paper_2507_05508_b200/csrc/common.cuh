@@ -60,7 +60,7 @@ enum KernelId {
     K_BEGIN = 0, K_UNIFORMS, K_HIST1, K_RESOLVE1, K_SUMS_CAND, K_CAND2, K_CAND3, K_BAND_HEADER, K_COPY_PROBS, K_EMIT, K_AGG_OFFSETS,
     K_AGG_TOPK, K_ABSMAX, K_BIT_STATS, K_BIT_PACK, K_AGG_BIT, K_TILE_LIST, K_BAND_COUNT, K_FLOAT_PACK, K_AGG_FLOAT,
     K_RTN_STATS, K_RTN_EMIT, K_AGG_DENSE, K_SEG_RESOLVE, K_SEG_SWEEP, K_SEG_BUCKETS, K_SEG_NORMS, K_SEG_DRAW, K_CLUSTER_TOPK,
-    K_BIT_CLUSTER, K_RTN_CLUSTER, K_COUNT
+    K_BIT_CLUSTER, K_RTN_CLUSTER, K_SORT_ROWS, K_COUNT
 };
 
 // Level probabilities handed to a kernel by value.
@@ -90,6 +90,7 @@ struct KernelLimits {
     int band_count[2];           // fp32, bf16
     int aggregate_topk, aggregate_bitwise, aggregate_float;
     int rtn_stats[2][2];         // fp32, bf16; few levels, many
+    int sort_rows;
 };
 
 struct Workspace {
@@ -539,6 +540,23 @@ inline void launch_kernel(Workspace& ws, int id, void (*kernel)(P...), dim3 grid
     launch_kernel_cluster(ws, id, 1, kernel, grid, threads, smem, s, args...);
 }
 
+// Enqueues one kernel whose blocks all run at a time (they meet at grid barriers).
+template <typename... P, typename... A>
+inline void launch_kernel_grid(Workspace& ws, int id, void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, A&&... args) {
+    LaunchScope t(ws, id, s);
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeCooperative;
+    attr.val.cooperative = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // ---------------------------------------------------------------------------------------------
 // launchers (each enqueues on `s` and bumps ws.launches)
 // ---------------------------------------------------------------------------------------------
@@ -621,7 +639,7 @@ int cluster_blocks(const Workspace& ws, int dtype, int64_t d, int M);
 void launch_cluster_topk(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const FinishPlan& plan,
                          const DrawnBand* bands, const mlmc_topk_msgs* out, cudaStream_t s);
 // stopk_segments.cu: s-Top-k with adaptive p and many segments
-int configure_segment_kernels();
+int configure_segment_kernels(KernelLimits* limits);
 int reserve_segments(Workspace& ws);
 void launch_segments(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, int64_t s_len, int64_t L,
                      uint64_t seed, uint64_t step, cudaStream_t s);

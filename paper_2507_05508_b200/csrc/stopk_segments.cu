@@ -11,10 +11,11 @@
 //   bf16: a bin is one key; the segment energies and the thresholds follow from the histogram alone.
 // Then p, the draw and the two thresholds of the drawn segment; the band is emitted like every other Top-k message.
 // Rows are taken together while their scratch memory fits in a fixed budget.
-// A radix sort of the rows (four passes of count and scatter) took 4.5 ms for 16 rows of 11.7M keys and L = 100.
+// A row whose buckets would hold most of its keys, or one of them a large share, is sorted instead (stopk_sort.cu): a bucket is
+// the work of one block, and ties and zeros meet in one.
 #include <algorithm>
 
-#include "common.cuh"
+#include "stopk_sort.cuh"
 
 namespace mlmc {
 
@@ -23,7 +24,17 @@ namespace {
 constexpr int kSegThreads = 1024;
 constexpr int kBucketThreads = 256;
 constexpr int kMaxCells = kBins1;                            // (segment, exponent) pairs of bins without a boundary
-constexpr size_t kSegScratchBudget = size_t(1) << 30;
+constexpr size_t kSegScratchBudget = size_t(1) << 31;
+
+// A row is sorted (stopk_sort.cu) where too many of its keys lie in buckets, or more than 1/32 of them in one bucket; not where that
+// is fewer than kFewKeys keys in all, or kFewEqual in one bucket: the passes of a sort take that long at least.
+//   Moving a key to its bucket costs more the more blocks of a row meet at the buckets' counters: 45 us per 10^6 keys with 4 rows in
+//   flight, 27 with 16, where a sort takes 25 per 10^6 keys of the row.  So the share from which on a row is sorted is 9/16 with
+//   up to 8 rows and 13/16 with more.  Normal entries, 11.7M x 4, buckets against sort: share 0.53 1412 and 1410 us, 0.66 1732
+//   and 1408; 11.7M x 16: 0.75 3364 and 5003, 0.89 4708 and 5001; 2M x 16: 0.75 1018 and 1091, 0.89 1163 and 1020.
+//   A bucket is the work of one block: 10^6 keys of different values 0.2 ms, equal ones 1.9 ms.
+constexpr uint32_t kFewKeys = 1u << 18, kFewEqual = 1u << 14;
+uint32_t sort_from(uint32_t d, int rows) { return std::max(kFewKeys, d / 16 * (rows <= 8 ? 9 : 13)); }
 
 // One boundary bin of a row.
 struct Bucket {
@@ -45,11 +56,6 @@ __device__ __forceinline__ double wide_to_double(unsigned __int128 x) {
 // mant^2 units of a bin with biased exponent ex, as a power of two
 __device__ __forceinline__ double energy_unit(double x, int ex) { return ldexp(x, 2 * ((ex ? ex : 1) - 150)); }
 
-struct RowHead {
-    uint32_t buckets, cells;
-    uint32_t pad[2];
-};
-
 // Scratch memory of the rows that are taken together, by row strides.
 struct SegScratch {
     uint32_t* keys;          // [rows][d]           keys of the buckets
@@ -64,6 +70,7 @@ struct SegScratch {
     Wide* prefix;            // [rows][seg_cap]     energy of the keys of its bucket inside boundary j
     double* delta;           // [rows][seg_cap]     norm of segment l
     RowHead* head;           // [rows]
+    SortBuffers sort;        // of the rows that are sorted; the first buffer is `keys`
     int64_t key_stride, seg_cap;
 };
 
@@ -102,14 +109,18 @@ struct Boundaries {
 
 // Which bins hold a boundary.  One block per row; thread t owns the 32 bins from 32 (1023 - t), so that the order of
 // the threads is the order of falling keys.  Boundary j is rank s (j + 1), j < L - 1.
+// sort_all, sort_one: with more keys than that in buckets, or in one of them, the row is sorted.
 // bf16: only the running counts are needed: hist[b] becomes #{key >= b}.
 template <bool BF16>
 __global__ void __launch_bounds__(kSegThreads, 1)
-segment_resolve_kernel(uint32_t* hist1, int m0, uint32_t s_len, uint32_t L, SegScratch sc, const int* worker_err) {
-    __shared__ uint32_t sh_warp[32];
+segment_resolve_kernel(uint32_t* hist1, int m0, uint32_t sort_all, uint32_t sort_one, uint32_t s_len, uint32_t L, SegScratch sc, const int* worker_err) {
+    __shared__ uint32_t sh_warp[32], sh_most[32];
     pdl_enter();
     const int row = blockIdx.x, m = m0 + row;
-    if (worker_err[m]) return;
+    if (worker_err[m]) {
+        if (threadIdx.x == 0) sc.head[row].sorted = 0u;
+        return;
+    }
     const int group = kSegThreads - 1 - (int)threadIdx.x;
     uint4* src = reinterpret_cast<uint4*>(hist1 + (int64_t)m * kBins1 + group * 32);
     uint32_t cnt[32];
@@ -135,7 +146,7 @@ segment_resolve_kernel(uint32_t* hist1, int m0, uint32_t s_len, uint32_t L, SegS
     // first pass over the bins: how many buckets, cells and collected keys this thread has.  A cell is the bins of one
     // segment without a boundary and of one exponent: the four threads of an exponent carry it on.
     const uint32_t top = L - 1;  // boundaries
-    uint32_t nb = 0, nc = 0, nk = 0, carry = 0xFFFFFFFFu;
+    uint32_t nb = 0, nc = 0, nk = 0, most = 0, carry = 0xFFFFFFFFu;
     {
         uint32_t last = 0xFFFFFFFFu, first = 0xFFFFFFFFu;
         Boundaries at(above, s_len, top);
@@ -146,6 +157,7 @@ segment_resolve_kernel(uint32_t* hist1, int m0, uint32_t s_len, uint32_t L, SegS
             if (at.advance(cnt[i])) {
                 ++nb;
                 nk += cnt[i];
+                most = max(most, cnt[i]);
             } else if (lo != last) {
                 ++nc;
                 if (last == 0xFFFFFFFFu) first = lo;
@@ -159,10 +171,15 @@ segment_resolve_kernel(uint32_t* hist1, int m0, uint32_t s_len, uint32_t L, SegS
         }
         if (carry != 0xFFFFFFFFu && carry == first) --nc;
     }
+    most = __reduce_max_sync(0xFFFFFFFFu, most);
+    if ((threadIdx.x & 31) == 0) sh_most[threadIdx.x >> 5] = most;  // read after the barriers of the scans
     uint32_t all_b, all_c, all_k;
     uint32_t b = block_exclusive_sum(nb, sh_warp, &all_b), c = block_exclusive_sum(nc, sh_warp, &all_c),
              k = block_exclusive_sum(nk, sh_warp, &all_k);
-    if (threadIdx.x == 0) sc.head[row] = {all_b, all_c, {0u, 0u}};
+    most = __reduce_max_sync(0xFFFFFFFFu, sh_most[threadIdx.x & 31]);
+    const bool sorted = all_k > sort_all || most > sort_one;
+    if (threadIdx.x == 0) sc.head[row] = {all_b, all_c, sorted ? 1u : 0u, 0u};
+    if (sorted) return;
     unsigned long long* cell = sc.cell + (int64_t)row * kMaxCells * 2;
     for (uint32_t i = threadIdx.x; i < all_c * 2; i += kSegThreads) cell[i] = 0ull;
     uint16_t* table = sc.table + (int64_t)row * kBins1 + group * 32;
@@ -235,6 +252,7 @@ segment_sweep_kernel(const float* __restrict__ g, int64_t d, int64_t ld, int m0,
     const int row = blockIdx.y, m = m0 + row;
     if (worker_err[m]) return;
     const RowHead head = sc.head[row];
+    if (head.sorted) return;
     const int lane = threadIdx.x & 31;
     const uint32_t cells = head.cells;
     int copies_log = 5;
@@ -425,7 +443,7 @@ bucket_kernel(int m0, uint32_t s_len, SegScratch sc, const int* worker_err) {
     __shared__ uint32_t sh_marked;
     pdl_enter();
     const int row = blockIdx.y;
-    if (worker_err[m0 + row]) return;
+    if (worker_err[m0 + row] || sc.head[row].sorted) return;  // (so a bucket has at most 2^27 keys)
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const uint32_t buckets = sc.head[row].buckets;
     for (uint32_t bi = blockIdx.x; bi < buckets; bi += gridDim.x) {
@@ -606,7 +624,7 @@ segment_norm_kernel(const uint32_t* hist1 /* bf16: #{key >= b} */, int m0, uint3
     pdl_enter();
     const int row = blockIdx.y, m = m0 + row, lane = threadIdx.x & 31;
     const uint32_t l = blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (l >= L || worker_err[m]) return;
+    if (l >= L || worker_err[m] || (!BF16 && sc.head[row].sorted)) return;
     double e = 0.0;
     if constexpr (BF16) {
         const uint32_t* S = hist1 + (int64_t)m * kBins1;
@@ -745,6 +763,16 @@ segment_draw_kernel(const uint32_t* hist1, int m0, uint32_t d, uint32_t s_len, u
             }
             q.T = (uint32_t)lo;
             q.r = k - (lo == kBins1 - 1 ? 0u : S[lo + 1]);
+        } else if (sc.head[row].sorted) {
+            const uint32_t* keys = sc.sort.b + (int64_t)row * sc.sort.stride;
+            const uint32_t at = keys[k - 1u];
+            uint32_t lo = 0, hi = k - 1u;  // the first place of that key
+            while (lo < hi) {
+                const uint32_t mid = lo + (hi - lo) / 2;
+                if (keys[mid] < at) lo = mid + 1; else hi = mid;
+            }
+            q.T = kSortFlip - at;
+            q.r = k - lo;
         } else {
             const uint2 b = sc.bound[(int64_t)row * sc.seg_cap + k / s_len - 1u];
             q.T = b.x;
@@ -781,6 +809,12 @@ size_t plan_scratch(char* base, int rows, int64_t d, int64_t seg_cap, SegScratch
     sc->prefix = pl.take<Wide>(r * seg_cap);
     sc->delta = pl.take<double>(r * seg_cap);
     sc->head = pl.take<RowHead>(r);
+    const size_t tiles = (size_t)sort_tiles(d);
+    sc->sort.a = sc->keys;
+    sc->sort.b = pl.take<uint32_t>(r * d);
+    sc->sort.table = pl.take<uint32_t>(r * 256 * tiles);
+    sc->sort.totals = pl.take<uint32_t>(r * 256);
+    sc->sort.stride = d;
     sc->key_stride = d;
     sc->seg_cap = seg_cap;
     return pl.off + 256;
@@ -788,11 +822,11 @@ size_t plan_scratch(char* base, int rows, int64_t d, int64_t seg_cap, SegScratch
 
 }  // namespace
 
-int configure_segment_kernels() {
+int configure_segment_kernels(KernelLimits* limits) {
     const bool ok =
         cudaFuncSetAttribute(segment_sweep_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSegSweepSmem) == cudaSuccess &&
         cudaFuncSetAttribute(segment_sweep_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSegSweepSmem) == cudaSuccess;
-    return ok ? MLMC_OK : MLMC_ERR_CUDA;
+    return ok ? configure_sort_kernels(limits) : MLMC_ERR_CUDA;
 }
 
 // Scratch memory, taken at the first call and kept as it is until the context is destroyed: room for as many rows of d_max
@@ -825,7 +859,8 @@ void launch_segments(Workspace& ws, const void* g, int dtype, int64_t d, int M, 
     for (int m0 = 0; m0 < M; m0 += together) {
         const int rows = std::min(together, M - m0);
         auto resolve = [&](auto kernel) {
-            launch_kernel(ws, K_SEG_RESOLVE, kernel, dim3(rows), kSegThreads, 0, s, ws.hist1, m0, sl, nl, sc, ws.worker_err);
+            launch_kernel(ws, K_SEG_RESOLVE, kernel, dim3(rows), kSegThreads, 0, s, ws.hist1, m0, sort_from(du, rows),
+                          std::max(kFewEqual, du / 32), sl, nl, sc, ws.worker_err);
         };
         auto norms = [&](auto norm, auto draw) {
             launch_kernel(ws, K_SEG_NORMS, norm, dim3((nl + 7) / 8, rows), 256, 0, s, ws.hist1, m0, du, sl, nl, sc, ws.worker_err);
@@ -842,6 +877,8 @@ void launch_segments(Workspace& ws, const void* g, int dtype, int64_t d, int M, 
         const int nb = (int)std::max<int64_t>(1, std::min<int64_t>(by_work, ws.sm_count / rows));
         launch_kernel(ws, K_SEG_SWEEP, L + 255 > kCellWords ? segment_sweep_kernel<true> : segment_sweep_kernel<false>, dim3(nb, rows), kSegThreads, kSegSweepSmem, s,
                       static_cast<const float*>(g), d, ld, m0, sc, ws.worker_err);
+        if (d > kFewEqual)  // shorter rows are never sorted
+            launch_sorted_rows(ws, static_cast<const float*>(g) + (int64_t)m0 * ld, d, rows, ld, sc.head, sc.sort, sl, nl, sc.delta, sc.seg_cap, s);
         // a block per bucket while there are few; at most as many buckets as boundaries
         const int most = (int)std::min<int64_t>(L - 1, kBins1);
         const int blocks = std::max(1, std::min(most, ws.sm_count * 16 / rows));

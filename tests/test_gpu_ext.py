@@ -401,3 +401,50 @@ def test_stopk_adaptive_scratch_stays_where_it_is(B, ora):
                 assert torch.equal(out.idx[m, :n], ref.idx[m, :n]) and torch.equal(out.val[m, :n], ref.val[m, :n])
     finally:
         B.mlmc_destroy(c)
+
+
+@pytest.mark.parametrize("s", [40, 1023, 1024, 20_011])
+@pytest.mark.parametrize("case", ["mixed", "spread", "one_tile"])
+def test_stopk_adaptive_sorted_rows(B, ora, ctx, case, s):
+    """Rows that are sorted, beside rows that are not: mostly zeros, one magnitude, a few magnitudes, and entries spread over more
+    bins with a boundary than without."""
+    rng = np.random.default_rng(63)
+    d = {"mixed": 200_003, "spread": 700_001, "one_tile": 40_960}[case]
+    normal = rng.standard_normal((4, d))
+    g_np = normal * 10.0 ** rng.uniform(-4, 0, (4, d))
+    if case == "spread":
+        g_np[:2] = normal[:2]                                                      # 1001 boundaries: nearly every occupied bin
+    else:
+        g_np[0] = normal[0] * (rng.random(d) < 0.05)
+        g_np[1] = np.where(rng.random(d) < 0.5, 0.01, -0.01)
+        g_np[3] = np.round(normal[3] * 4) / 8
+    for step in range(2):
+        check_stopk(B, ora, ctx, to_dev(g_np.astype(np.float32)), s, None, 12, step, expect_excluded=1)
+
+
+def test_stopk_adaptive_rows_in_groups_and_a_void_row(B, ora):
+    """More rows than the scratch memory holds with so many segments; then a row with an Inf among sorted ones."""
+    rng = np.random.default_rng(64)
+    d, M = 40_003, 7
+    g_np = (rng.standard_normal((M, d)) * 10.0 ** rng.uniform(-3, 0, (M, d))).astype(np.float32)
+    g_np[::2] *= rng.random((4, d)) < 0.1
+    c = B.mlmc_create(0, d, M, 32)
+    try:
+        check_stopk(B, ora, c, to_dev(g_np), 1, None, 13, 0, expect_excluded=2)
+        check_stopk(B, ora, c, to_dev(g_np), 100, None, 13, 1, expect_excluded=1)
+        bad = g_np.copy()
+        bad[2, 77] = np.inf
+        out = B.TopkBuffers(M, 100)
+        B.mlmc_compress_stopk(c, to_dev(bad), 100, None, 13, 1, out)
+        assert B.mlmc_get_status(c) == B.MLMC_ERR_NONFINITE
+        ref = B.TopkBuffers(M, 100)
+        B.mlmc_compress_stopk(c, to_dev(g_np), 100, None, 13, 1, ref)
+        assert B.mlmc_get_status(c) == B.MLMC_OK
+        for m in range(M):
+            if m == 2:
+                assert int(out.level[m]) == -1 and int(out.count[m]) == 0
+            else:
+                n = int(ref.count[m])
+                assert int(out.level[m]) == int(ref.level[m]) and torch.equal(out.idx[m, :n], ref.idx[m, :n])
+    finally:
+        B.mlmc_destroy(c)
