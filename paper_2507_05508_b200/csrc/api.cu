@@ -144,7 +144,7 @@ FinishPlan finish_plan(int64_t d, int L, int nq, bool adaptive, uint64_t seed, u
     return pl;
 }
 
-// Adaptive p: every level boundary is a query.  Rows that a cluster's shared memory holds (2.8 MB) take one launch.
+// Adaptive p: every level boundary is a query.  Rows that a cluster's shared memory holds (at most 2.9 MB) take one launch.
 void select_adaptive(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int64_t* k, int L,
                      uint64_t seed, uint64_t step, const mlmc_topk_msgs* out, cudaStream_t s) {
     FinishPlan pl = finish_plan(d, L, L - 1, true, seed, step, out);

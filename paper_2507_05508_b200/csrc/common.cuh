@@ -84,8 +84,9 @@ constexpr int kTimingPool = 2048;  // event pairs kept between two reads
 
 // What the device can place.
 struct KernelLimits {
-    int cluster_most;            // largest thread-block cluster of the short-row Top-k kernel (0: none)
-    int dense_fit[5];            // clusters of 1, 2, .. 16 blocks of the short-row dense kernels that run at a time
+    // clusters of 1, 2, .. 16 blocks that run at a time
+    int topk_fit[5];             // of the short-row Top-k kernel
+    int dense_fit[5];            // of the short-row dense kernels
     // blocks per SM
     int band_count[2];           // fp32, bf16
     int aggregate_topk, aggregate_bitwise, aggregate_float;

@@ -30,12 +30,12 @@ constexpr int kClMost = 16;                      // blocks per cluster (8 is the
 constexpr int kClDigit1 = 13;
 constexpr int kClBins = 1 << kClDigit1;
 constexpr int kClHistWords = 8192;               // 16384 16-bit counts, or the energy cells
-constexpr int kClBatches = 86;                   // batches per block at most: 172 KB of the row,
-constexpr int kClBatchesBf16 = 63;               // for bf16 as many as a 16-bit count takes
+constexpr int kClBatches = 91;                   // batches per block at most: as much of the row (182 KB) as shared memory holds
+constexpr int kClEasy = 32;                      // batches per block from which on the cluster grows (64 KB, 16 words per thread)
 constexpr int kClCells = 32 + 256;               // interval + (largest exponent - exponent)
 constexpr int kClCopiesLow = 8;                  // copies of a cell's limbs: 32 where the cells are few enough, else 8
 static_assert(kClCells * 3 * kClCopiesLow <= kClHistWords, "the cells take the place of the histogram");
-static_assert(kClBatches * kBatchWords < 65536 && kClBatchesBf16 * kBatchWords * 2 < 65536, "16-bit counts, and 16-bit limbs added at most 65535 times");
+static_assert(kClBatches * kBatchWords < 65536 && kClEasy * kBatchWords * 2 < 65536, "16-bit counts, and 16-bit limbs added at most 65535 times");
 
 struct ClusterShared {
     Query q[kMaxQueries];
@@ -53,6 +53,9 @@ struct ClusterShared {
 };
 
 constexpr size_t kClFixedSmem = kClHistWords * 4 + kClBins;  // histogram, bin codes; then the row
+constexpr size_t kClSharedMost = 227 * 1024;
+static_assert(kClFixedSmem + kClBatches * kBatchWords * 4 + sizeof(ClusterShared) + 64 <= kClSharedMost &&
+              kClFixedSmem + (kClBatches + 1) * kBatchWords * 4 + sizeof(ClusterShared) > kClSharedMost, "the most that fits");
 
 template <typename T>
 __global__ void __launch_bounds__(kClThreads, 1)
@@ -566,43 +569,54 @@ size_t cluster_smem(int per_block) { return kClFixedSmem + (size_t)per_block * k
 }  // namespace
 
 int configure_cluster_kernels(KernelLimits* limits) {
-    limits->cluster_most = 0;
     auto set = [&](auto kernel) {
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cluster_smem(kClBatches)) != cudaSuccess) return false;
         return cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
     };
     if (!set(cluster_topk_kernel<float>) || !set(cluster_topk_kernel<bf16_t>)) return MLMC_ERR_CUDA;
-    // the largest cluster that the device can place with the largest blocks
-    for (int cl : {16, 8}) {
+    // clusters of 2^i blocks that run at a time (a block takes an SM)
+    for (int i = 0; i < 5; ++i) {
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(cl);
+        cfg.gridDim = dim3(1 << i);
         cfg.blockDim = dim3(kClThreads);
         cfg.dynamicSmemBytes = cluster_smem(kClBatches);
         cudaLaunchAttribute attr;
         attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = cl;
+        attr.val.clusterDim.x = 1 << i;
         attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
         cfg.attrs = &attr;
         cfg.numAttrs = 1;
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, cluster_topk_kernel<float>, &cfg) == cudaSuccess && n >= 1) {
-            limits->cluster_most = cl;
-            break;
+        if (cudaOccupancyMaxActiveClusters(&n, cluster_topk_kernel<float>, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            n = 0;
         }
-        cudaGetLastError();
+        limits->topk_fit[i] = n;
     }
     return MLMC_OK;
 }
 
-// Blocks per cluster for this call, 0: the row is too long (or the workers too many) for it.
+// Blocks per cluster for this call, 0: the row is too long, or the workers are too many, for the cluster to be the faster way.
+// The smallest cluster whose blocks have at most kClEasy batches: a barrier and an exchange between more blocks take longer
+// than the work that they share out.  Clusters that do not fit the GPU at a time run one after the other, where the launch
+// chain has the whole GPU: two waves are worth it for fp32 rows whose blocks are not stretched beyond kClEasy batches, three never.
+// bf16 rows (whose chain needs one sweep) only in one wave and not stretched.  us per call, cluster / chain, layered rows:
+//   fp32, adaptive     131k x 12 33 / 77, x 16 (two waves) 61 / 77, x 32 (three) 93 / 90; 262k x 8 (two) 75 / 75, x 16 (three)
+//                      112 / 83; 700k x 4 58 / 78, x 8 (two, stretched) 105 / 89, x 32 258 / 134
+//   fp32, given p      262k x 4 24 / 54, x 8 (two) 46 / 55, x 16 (three) 68 / 60
+//   bf16, adaptive     262k x 12 50 / 56, x 16 (two) 68 / 58; 500k x 4 46 / 51; 700k x 4 (stretched) 59 / 53, x 32 236 / 85
+//   bf16, given p      500k x 4 22 / 36, x 8 (two) 40 / 36, x 32 99 / 55
 int cluster_blocks(const Workspace& ws, int dtype, int64_t d, int M) {
-    const int batches = emit_tiles_per_worker(d, dtype) * kEmitGroups;
-    if (M > 32 || ws.limits.cluster_most == 0) return 0;
-    // The smallest cluster whose blocks have at most 32 batches (64 KB, 16 words per thread), and no more workers than fit
-    // the GPU at a time: a barrier and an exchange between more blocks take longer than the work that they share out.
-    int cl = 1;
-    while (cl < ws.limits.cluster_most && (batches + cl - 1) / cl > 32) cl *= 2;
-    return (batches + cl - 1) / cl <= (dtype == MLMC_BF16 ? kClBatchesBf16 : kClBatches) ? cl : 0;
+    const int64_t batches = (int64_t)emit_tiles_per_worker(d, dtype) * kEmitGroups;
+    if (M > 32) return 0;
+    int i = 0;
+    while (i < 4 && ws.limits.topk_fit[i + 1] > 0 && batches > (int64_t)kClEasy << i) ++i;
+    const int fit = ws.limits.topk_fit[i];
+    if (fit == 0) return 0;
+    const int64_t per = (batches + (1 << i) - 1) >> i;
+    const int waves = (M + fit - 1) / fit;
+    const int64_t most = dtype == MLMC_BF16 ? (waves == 1 ? kClEasy : 0) : waves == 1 ? kClBatches : waves == 2 ? kClEasy : 0;
+    return per <= most ? 1 << i : 0;
 }
 
 void launch_cluster_topk(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const FinishPlan& plan,

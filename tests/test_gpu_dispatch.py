@@ -275,3 +275,12 @@ def test_create_after_a_device_reset(ora):
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     r = subprocess.run([sys.executable, "-c", RESET, root], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and "both contexts agree" in r.stdout, r.stdout + r.stderr
+
+
+# what a cluster holds and one entry more; as many workers as fit the GPU at a time in one, two and three waves
+@pytest.mark.parametrize("dtype,d,M,adaptive", [
+    ("f32", 745_472, 1, True), ("f32", 745_473, 1, True), ("bf16", 524_288, 1, True), ("bf16", 524_289, 1, True), ("bf16", 65_536, 20, True),
+    ("f32", 131_072, 14, True), ("f32", 131_072, 20, True), ("f32", 262_144, 7, True), ("f32", 262_144, 13, False), ("f32", 262_144, 20, False)])
+def test_topk_cluster_waves(B, ora, ctx, dtype, d, M, adaptive):
+    k = doubling(d, max(1, d // 500))
+    check_topk(B, ora, ctx, layered(d, M, dtype), k, None if adaptive else geometric(len(k)), 3, 1, expect_excluded=1)
