@@ -141,7 +141,7 @@ hist1_kernel(const T* __restrict__ g, int64_t d, int64_t ld, uint32_t* __restric
         if (br.z != 0xFFFFFFFFu) { lo_b = br.z << 16; span_b = ((br.w + 1u) << 16) - 1u; }
         if (lane == 0) *wcount = 0u;
     }
-    const uint32_t lo_min = min(lo_a, lo_b);
+    uint32_t lo_min = min(lo_a, lo_b);  // no key reaches it once the list is full: the warp collects no more
     auto in_bracket = [&](uint32_t bits) -> bool {
         const uint32_t key = bits & 0x7FFFFFFFu;
         return (key - lo_a) <= span_a || (key - lo_b) <= span_b;  // an empty bracket: key - lo wraps to key + 1 > 0
@@ -155,8 +155,9 @@ hist1_kernel(const T* __restrict__ g, int64_t d, int64_t ld, uint32_t* __restric
             if ((int64_t)base + wfill <= cand_cap) {
                 uint32_t* dst = cand_keys + (int64_t)m * cand_cap + base;
                 for (uint32_t i = lane; i < wfill; i += 32) dst[i] = wstage[i];
-            } else if (lane == 0) {
-                cand_overflow[m] = 1;
+            } else {
+                if (lane == 0) cand_overflow[m] = 1;
+                lo_min = 0xFFFFFFFFu;
             }
             __syncwarp();
             if (lane == 0) *wcount = 0u;
@@ -522,6 +523,7 @@ sums_candidates_kernel(const float* __restrict__ g, int64_t d, int64_t ld, const
 
     const uint32_t slots0 = (uint32_t)__cvta_generic_to_shared(slots), step = (uint32_t)threads * 4u;
     uint32_t at = slots0;
+    bool over = false;  // the list is full (warp-uniform)
     auto flush = [&]() {  // called by the whole warp
         const uint32_t n = (at - slots0) / step;
         uint32_t upto = n;
@@ -538,8 +540,9 @@ sums_candidates_kernel(const float* __restrict__ g, int64_t d, int64_t ld, const
         if ((int64_t)base + total <= cand_cap) {
             uint32_t* to = cand + base + (upto - n);
             for (uint32_t i = 0; i < n; ++i) to[i] = slots[i * threads] & 0x7FFFFFFFu;
-        } else if (lane == 0) {
-            cand_overflow[m] = 1;  // too many keys share the boundary bins: the full-sweep passes take over
+        } else {
+            over = true;
+            if (lane == 0) cand_overflow[m] = 1;  // too many keys share the boundary bins: the full-sweep passes take over
         }
         at = slots0;
     };
@@ -602,6 +605,7 @@ sums_candidates_kernel(const float* __restrict__ g, int64_t d, int64_t ld, const
 #pragma unroll
                 for (int j = 0; j < 4; ++j) add_low(cur[j]);
             } else {
+                if (!SUMS && over) return;  // nothing is left to do (a warp's own barriers only from here on)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const uint32_t g0 = look_up(cur[j].x), g1 = look_up(cur[j].y), g2 = look_up(cur[j].z), g3 = look_up(cur[j].w);
