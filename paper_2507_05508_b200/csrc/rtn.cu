@@ -390,7 +390,10 @@ rtn_cluster_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid_
     }
 }
 
-// Server average of dense messages: out[i] = (1/M) sum_m val[m][i] in worker order.
+// Server average of dense messages: out[i] = (1/M) sum_m val[m][i] in worker order, four workers' entries in flight.  (With one
+// and its level before it, 200 workers of 3000 entries took 34 us, 64 of 200,000 12.8.)
+constexpr int kAvgTogether = 4;
+
 __global__ void __launch_bounds__(kRtnThreads)
 aggregate_dense_kernel(const float* __restrict__ val, const int32_t* level, int M, int64_t d, int64_t ldv,
                        float* __restrict__ out) {
@@ -400,10 +403,19 @@ aggregate_dense_kernel(const float* __restrict__ val, const int32_t* level, int 
     const int64_t n4 = aligned ? d / 4 : 0;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n4; v += (int64_t)gridDim.x * blockDim.x) {
         float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int m = 0; m < M; ++m) {
-            if (level[m] < 0) continue;
-            const float4 x = __ldg(reinterpret_cast<const float4*>(val + (int64_t)m * ldv) + v);
-            a.x += x.x; a.y += x.y; a.z += x.z; a.w += x.w;
+        for (int m0 = 0; m0 < M; m0 += kAvgTogether) {
+            float4 x[kAvgTogether];
+            bool on[kAvgTogether];
+#pragma unroll
+            for (int j = 0; j < kAvgTogether; ++j) on[j] = m0 + j < M && level[m0 + j] >= 0;
+#pragma unroll
+            for (int j = 0; j < kAvgTogether; ++j)
+                if (on[j]) x[j] = __ldg(reinterpret_cast<const float4*>(val + (int64_t)(m0 + j) * ldv) + v);
+#pragma unroll
+            for (int j = 0; j < kAvgTogether; ++j)
+                if (on[j]) {
+                    a.x += x[j].x; a.y += x[j].y; a.z += x[j].z; a.w += x[j].w;
+                }
         }
         a.x *= inv_M; a.y *= inv_M; a.z *= inv_M; a.w *= inv_M;
         reinterpret_cast<float4*>(out)[v] = a;
