@@ -385,8 +385,8 @@ bit_pack_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* 
     const T* row = g + (int64_t)m * ld;
     uint32_t* out = planes + (int64_t)m * (1 + w_max) * words;
     uint32_t* ring = sh_ring + warp * 2 * kGroupSlot<T>;
-    const int64_t stride = (int64_t)gridDim.x * (kBitThreads / 32);
-    int64_t grp = (int64_t)blockIdx.x * (kBitThreads / 32) + warp;
+    const int64_t stride = (int64_t)gridDim.x * (blockDim.x / 32);
+    int64_t grp = (int64_t)blockIdx.x * (blockDim.x / 32) + warp;
     fetch_group<T>(row, d, grp, ngroups, ring);
     for (int it = 0; grp < ngroups; grp += stride, ++it) {
         fetch_group<T>(row, d, grp + stride, ngroups, ring + ((it + 1) & 1) * kGroupSlot<T>);
@@ -582,7 +582,7 @@ int bit_blocks(const Workspace& ws, int64_t d, int vec, int M, int waves) {
     return (int)(nb < 1 ? 1 : nb);
 }
 
-size_t bit_pack_smem(size_t elem) { return (kBitThreads / 32) * 2 * 1024 * elem; }
+size_t bit_pack_smem(size_t elem, int warps) { return (size_t)warps * 2 * 1024 * elem; }
 
 }  // namespace
 
@@ -591,7 +591,7 @@ int configure_bit_kernels(KernelLimits* limits) {
                                          (int)kAvgBitSmem + kEmitMaxWorkers * 8) == cudaSuccess &&
                     configure_dense_cluster(bit_cluster_kernel<float>) && configure_dense_cluster(bit_cluster_kernel<bf16_t>) &&
                     cudaFuncSetAttribute(bit_pack_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)bit_pack_smem(4)) == cudaSuccess;
+                                         (int)bit_pack_smem(4, kBitThreads / 32)) == cudaSuccess;
     dense_cluster_fit(bit_cluster_kernel<float>, kBitDenseWarps * 32, limits);
     limits->aggregate_bitwise = resident_blocks(aggregate_bitwise_kernel, kAvgThreads, kAvgBitSmem + 64);
     return ok ? MLMC_OK : MLMC_ERR_CUDA;
@@ -681,11 +681,12 @@ static void launch_bit_pack_t(Workspace& ws, const T* g, int64_t d, int M, int64
                               const mlmc_bit_msgs& out, cudaStream_t s) {
     const int64_t words = (d + 31) / 32;
     const int64_t ngroups = (words + 31) / 32;
-    const int64_t by_work = (ngroups + (kBitThreads / 32) - 1) / (kBitThreads / 32);
+    const int warps = (int)std::min<int64_t>(ngroups, kBitThreads / 32);  // of short rows as many blocks as possible fit an SM
+    const int64_t by_work = (ngroups + warps - 1) / warps;
     int64_t nb = ((int64_t)ws.sm_count * 3) / M;  // persistent: three resident blocks per SM, rounded down
     if (nb > by_work) nb = by_work;
     if (nb < 1) nb = 1;
-    launch_kernel(ws, K_BIT_PACK, bit_pack_kernel<T>, dim3((unsigned)nb, M), kBitThreads, bit_pack_smem(sizeof(T)), s, g, d, ld,
+    launch_kernel(ws, K_BIT_PACK, bit_pack_kernel<T>, dim3((unsigned)nb, M), warps * 32, bit_pack_smem(sizeof(T), warps), s, g, d, ld,
                   ws.gmax_bits, sc, ws.bit_level, out.planes, out.w_max, words);
 }
 

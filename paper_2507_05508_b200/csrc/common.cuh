@@ -218,6 +218,7 @@ __device__ __forceinline__ void pdl_enter() {
 __device__ __forceinline__ bool last_block(uint32_t* counter, uint32_t nblocks) {
     __shared__ bool sh_last;
     __syncthreads();
+    if (nblocks == 1u) return true;
     if (threadIdx.x == 0) {
         __threadfence();
         sh_last = atomicAdd(counter, 1u) == nblocks - 1u;

@@ -94,11 +94,11 @@ float_pack_kernel(const T* __restrict__ g, int64_t d, int64_t ld, MantissaSchedu
     uint8_t* ex = expo + (int64_t)m * words * 32;
     uint32_t* ring = sh_ring + warp * 2 * kSlot;
     const int64_t ngroups = (words + 31) / 32;
-    const int64_t stride = (int64_t)gridDim.x * (kFloatThreads / 32);
+    const int64_t stride = (int64_t)gridDim.x * (blockDim.x / 32);
     auto fetch = [&](int64_t grp, uint32_t* slot) { fetch_group<T>(row, d, grp, ngroups, slot); };
     const bool wide_store = (reinterpret_cast<uintptr_t>(expo) & 31) == 0;
     uint32_t top = 0;  // largest exponent field seen, at the top of the word
-    int64_t grp = (int64_t)blockIdx.x * (kFloatThreads / 32) + warp;
+    int64_t grp = (int64_t)blockIdx.x * (blockDim.x / 32) + warp;
     fetch(grp, ring);
     for (int it = 0; grp < ngroups; grp += stride, ++it) {
         fetch(grp + stride, ring + ((it + 1) & 1) * kSlot);
@@ -278,7 +278,7 @@ aggregate_float_kernel(const uint8_t* __restrict__ expo, const uint32_t* __restr
     }
 }
 
-size_t float_pack_smem(size_t elem) { return (kFloatThreads / 32) * 2 * 1024 * elem; }
+size_t float_pack_smem(size_t elem, int warps) { return (size_t)warps * 2 * 1024 * elem; }
 
 }  // namespace
 
@@ -286,7 +286,7 @@ int configure_float_kernels(KernelLimits* limits) {
     const bool ok = cudaFuncSetAttribute(aggregate_float_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)kAvgFloatSmem + kEmitMaxWorkers * 8) == cudaSuccess &&
                     cudaFuncSetAttribute(float_pack_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)float_pack_smem(4)) == cudaSuccess;
+                                         (int)float_pack_smem(4, kFloatThreads / 32)) == cudaSuccess;
     limits->aggregate_float = resident_blocks(aggregate_float_kernel, kAvgThreads, kAvgFloatSmem + 64);
     return ok ? MLMC_OK : MLMC_ERR_CUDA;
 }
@@ -297,13 +297,14 @@ void launch_compress_floatbits(Workspace& ws, const void* g, int dtype, int64_t 
     const MantissaSchedule sc = make_mantissa_schedule(mb, L);
     const int64_t words = (d + 31) / 32;
     const int64_t ngroups = (words + 31) / 32;
-    const int64_t by_work = (ngroups + (kFloatThreads / 32) - 1) / (kFloatThreads / 32);
+    const int warps = (int)std::min<int64_t>(ngroups, kFloatThreads / 32);  // of short rows as many blocks as possible fit an SM
+    const int64_t by_work = (ngroups + warps - 1) / warps;
     int64_t nb = ((int64_t)ws.sm_count * 3) / M;  // persistent: three resident blocks per SM, rounded down
     if (nb > by_work) nb = by_work;
     if (nb < 1) nb = 1;
     const DrawnLevels drawn = draw_levels(p, L, seed, step, M);
     auto go = [&](auto kernel, auto* row) {
-        launch_kernel(ws, K_FLOAT_PACK, kernel, dim3((unsigned)nb, M), kFloatThreads, float_pack_smem(sizeof(*row)), s, row, d, ld, sc, drawn, out.expo, out.planes, out.w_max, words, out.level, out.p_sel, ws.acc_word, ws.done, ws.status);
+        launch_kernel(ws, K_FLOAT_PACK, kernel, dim3((unsigned)nb, M), warps * 32, float_pack_smem(sizeof(*row), warps), s, row, d, ld, sc, drawn, out.expo, out.planes, out.w_max, words, out.level, out.p_sel, ws.acc_word, ws.done, ws.status);
     };
     if (dtype == MLMC_BF16) go(float_pack_kernel<bf16_t>, static_cast<const bf16_t*>(g));
     else go(float_pack_kernel<float>, static_cast<const float*>(g));
