@@ -112,14 +112,21 @@ __device__ __forceinline__ float field_times(const uint32_t (&fb)[8], int t, flo
     return fmaf(__uint_as_float(__byte_perm(fb[t & 7], 0x4B000000u, 0x7650u + (uint32_t)(t >> 3))), unit, offset);
 }
 
-// Fields of any width, plane by plane.
+// Fields of any width, plane by plane, the words of AHEAD planes in flight.
+template <int AHEAD>
 __device__ __forceinline__ void gather_fields(const uint32_t* __restrict__ plane1, int64_t words, int w, uint32_t (&f)[32]) {
 #pragma unroll
     for (int t = 0; t < 32; ++t) f[t] = 0u;
-    for (int j = 0; j < w; ++j) {
-        const uint32_t pw = __ldg(plane1 + (int64_t)j * words);
+    for (int j0 = 0; j0 < w; j0 += AHEAD) {
+        uint32_t pw[AHEAD];
 #pragma unroll
-        for (int t = 0; t < 32; ++t) f[t] = (f[t] << 1) | ((pw >> t) & 1u);
+        for (int j = 0; j < AHEAD; ++j) pw[j] = j0 + j < w ? __ldg(plane1 + (int64_t)(j0 + j) * words) : 0u;
+#pragma unroll
+        for (int j = 0; j < AHEAD; ++j) {
+            if (j0 + j >= w) break;
+#pragma unroll
+            for (int t = 0; t < 32; ++t) f[t] = (f[t] << 1) | ((pw[j] >> t) & 1u);
+        }
     }
 }
 

@@ -538,7 +538,7 @@ aggregate_bitwise_kernel(const uint32_t* __restrict__ planes, const float* gmax,
                 }
             } else {
                 uint32_t f[32];
-                gather_fields(planes + ((int64_t)m * (1 + w_max) + 1) * words + at, words, w, f);
+                gather_fields<1>(planes + ((int64_t)m * (1 + w_max) + 1) * words + at, words, w, f);
 #pragma unroll
                 for (int t = 0; t < 32; ++t) {
                     const float ff = __uint_as_float(0x4B000000u | f[t]) - 8388608.0f;  // f < 2^23: exact

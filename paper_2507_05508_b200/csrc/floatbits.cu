@@ -261,7 +261,7 @@ aggregate_float_kernel(const uint8_t* __restrict__ expo, const uint32_t* __restr
                 }
             } else {
                 uint32_t f[32];
-                gather_fields(planes + ((int64_t)m * (1 + w_max) + 1) * words + at, words, w, f);
+                gather_fields<4>(planes + ((int64_t)m * (1 + w_max) + 1) * words + at, words, w, f);
 #pragma unroll
                 for (int t = 0; t < 32; ++t) {
                     const uint32_t E = (e4[t >> 2] >> (8 * (t & 3))) & 0xFFu;
