@@ -1,4 +1,5 @@
 // C ABI of the MLMC compression library: context, argument checks and the launch sequences.
+#include <mutex>
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -6,7 +7,7 @@
 #include <new>
 #include <vector>
 
-#include "common.cuh"
+#include "stopk_sort.cuh"
 
 using namespace mlmc;
 
@@ -179,12 +180,36 @@ void select_drawn(Workspace& ws, const void* g, int dtype, int64_t d, int M, int
     launch_emit(ws, g, dtype, d, M, ld, *out, s);
 }
 
-// Shared-memory limits of the kernels, and what the device can place.  Both belong to the current CUDA context (a device
-// reset starts a new one), so every create sets and asks.
-bool configure_kernels(KernelLimits* limits) {
-    return configure_select_kernels() == MLMC_OK && configure_emit_kernels(limits) == MLMC_OK && configure_float_kernels(limits) == MLMC_OK &&
-           configure_segment_kernels(limits) == MLMC_OK && configure_rtn_kernels(limits) == MLMC_OK && configure_cluster_kernels(limits) == MLMC_OK &&
-           configure_bit_kernels(limits) == MLMC_OK;
+// The kernels' shared-memory limits and cluster attributes belong to the current CUDA context (a device reset starts a new one),
+// so every create sets them.  What the device can place is asked for once per device: the queries take a millisecond.
+bool configure_kernels(int device, KernelLimits* out) {
+    if (configure_select_kernels() != MLMC_OK || configure_emit_kernels() != MLMC_OK || configure_float_kernels() != MLMC_OK ||
+        configure_segment_kernels() != MLMC_OK || configure_sort_kernels() != MLMC_OK || configure_rtn_kernels() != MLMC_OK ||
+        configure_cluster_kernels() != MLMC_OK || configure_bit_kernels() != MLMC_OK)
+        return false;
+    constexpr int kMostDevices = 64;
+    static std::mutex lock;
+    static bool known[kMostDevices];
+    static KernelLimits limits[kMostDevices];
+    std::lock_guard<std::mutex> hold(lock);
+    const bool keep = device < kMostDevices;
+    if (keep && known[device]) {
+        *out = limits[device];
+        return true;
+    }
+    KernelLimits l = {};
+    emit_limits(&l);
+    float_limits(&l);
+    sort_limits(&l);
+    rtn_limits(&l);
+    cluster_limits(&l);
+    bit_limits(&l);
+    if (keep) {
+        limits[device] = l;
+        known[device] = true;
+    }
+    *out = l;
+    return true;
 }
 
 }  // namespace
@@ -199,8 +224,8 @@ int mlmc_create(mlmc_ctx** out, int device, int64_t d_max, int M_max, int L_max)
     if (!guard.ok) return MLMC_ERR_CUDA;
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return MLMC_ERR_CUDA;
-    KernelLimits limits = {};
-    if (!configure_kernels(&limits)) return MLMC_ERR_CUDA;
+    KernelLimits limits;
+    if (!configure_kernels(device, &limits)) return MLMC_ERR_CUDA;
 
     mlmc_ctx* ctx = new (std::nothrow) mlmc_ctx();
     if (!ctx) return MLMC_ERR_NOMEM;

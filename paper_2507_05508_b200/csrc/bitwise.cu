@@ -586,15 +586,18 @@ size_t bit_pack_smem(size_t elem, int warps) { return (size_t)warps * 2 * 1024 *
 
 }  // namespace
 
-int configure_bit_kernels(KernelLimits* limits) {
+int configure_bit_kernels() {
     const bool ok = cudaFuncSetAttribute(aggregate_bitwise_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)kAvgBitSmem + kEmitMaxWorkers * 8) == cudaSuccess &&
                     configure_dense_cluster(bit_cluster_kernel<float>) && configure_dense_cluster(bit_cluster_kernel<bf16_t>) &&
                     cudaFuncSetAttribute(bit_pack_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)bit_pack_smem(4, kBitThreads / 32)) == cudaSuccess;
-    dense_cluster_fit(bit_cluster_kernel<float>, kBitDenseWarps * 32, limits);
-    limits->aggregate_bitwise = resident_blocks(aggregate_bitwise_kernel, kAvgThreads, kAvgBitSmem + 64);
     return ok ? MLMC_OK : MLMC_ERR_CUDA;
+}
+
+void bit_limits(KernelLimits* limits) {
+    clusters_that_fit(bit_cluster_kernel<float>, kBitDenseWarps * 32, kDenseBytes, limits->dense_fit);
+    limits->aggregate_bitwise = resident_blocks(aggregate_bitwise_kernel, kAvgThreads, kAvgBitSmem + 64);
 }
 
 DrawPlan bit_draw_plan(Workspace& ws, const int32_t* b, int L, uint64_t seed, uint64_t step, const mlmc_bit_msgs* out) {

@@ -473,6 +473,28 @@ int resident_blocks(K kernel, int threads, size_t smem) {
     return ok && n >= 1 ? n : 1;
 }
 
+// Clusters of 2^i blocks that run at a time (a block takes an SM).
+template <typename K>
+void clusters_that_fit(K kernel, int threads, size_t smem, int (&fit)[5]) {
+    for (int i = 0; i < 5; ++i) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(1 << i);
+        cfg.blockDim = dim3(threads);
+        cfg.dynamicSmemBytes = smem;
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = 1 << i;
+        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        fit[i] = 0;
+        if (cudaOccupancyMaxActiveClusters(&fit[i], kernel, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            fit[i] = 0;
+        }
+    }
+}
+
 // Brackets one kernel launch: counts it and, when timing is on, records an event pair on the stream.
 struct LaunchScope {
     Workspace& ws;
@@ -597,12 +619,14 @@ void launch_band_header(Workspace& ws, int M, const FinishPlan& plan, cudaStream
 void launch_copy_probs(Workspace& ws, int M, int L, const double* p_fixed, double* p_out, double* delta_out,
                        cudaStream_t s);
 // topk_emit.cu
-int configure_emit_kernels(KernelLimits* limits);
+int configure_emit_kernels();
+void emit_limits(KernelLimits* limits);
 void launch_emit(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const mlmc_topk_msgs& out,
                  cudaStream_t s);
 void launch_aggregate_topk(Workspace& ws, const mlmc_topk_msgs& msgs, int M, int64_t d, float* out, cudaStream_t s);
 // bitwise.cu
-int configure_bit_kernels(KernelLimits* limits);
+int configure_bit_kernels();
+void bit_limits(KernelLimits* limits);
 // Largest magnitude of every worker and the NaN / Inf check; with `p` (given probabilities) also the draw and the header.
 void launch_absmax(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const DrawPlan& plan, const double* p,
                    cudaStream_t s);
@@ -618,7 +642,8 @@ void launch_aggregate_bitwise(Workspace& ws, const mlmc_bit_msgs& msgs, const in
                               float* out, cudaStream_t s);
 
 // floatbits.cu
-int configure_float_kernels(KernelLimits* limits);
+int configure_float_kernels();
+void float_limits(KernelLimits* limits);
 void launch_compress_floatbits(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* mb,
                                int L, const double* p, uint64_t seed, uint64_t step, const mlmc_float_msgs& out, cudaStream_t s);
 void launch_aggregate_floatbits(Workspace& ws, const mlmc_float_msgs& msgs, const int32_t* mb, int L, int M, int64_t d,
@@ -628,7 +653,8 @@ DrawPlan rtn_draw_plan(Workspace& ws, int L, uint64_t seed, uint64_t step, const
 // Adaptive: residual energies of every level, probabilities, draw and header.
 void launch_rtn_stats(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* r, int L,
                       const DrawPlan& plan, cudaStream_t s);
-int configure_rtn_kernels(KernelLimits* limits);
+int configure_rtn_kernels();
+void rtn_limits(KernelLimits* limits);
 bool launch_rtn_cluster(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* r, int L,
                         const DrawPlan& plan, const double* p, const mlmc_rtn_msgs& out, cudaStream_t s);
 void launch_rtn_emit(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* r, int L,
@@ -636,12 +662,13 @@ void launch_rtn_emit(Workspace& ws, const void* g, int dtype, int64_t d, int M, 
 void launch_aggregate_dense(Workspace& ws, const float* val, const int32_t* level, int M, int64_t d, int64_t ldv,
                             float* out, cudaStream_t s);
 // topk_cluster.cu: Top-k messages of short rows in one launch
-int configure_cluster_kernels(KernelLimits* limits);
+int configure_cluster_kernels();
+void cluster_limits(KernelLimits* limits);
 int cluster_blocks(const Workspace& ws, int dtype, int64_t d, int M);
 void launch_cluster_topk(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const FinishPlan& plan,
                          const DrawnBand* bands, const mlmc_topk_msgs* out, cudaStream_t s);
 // stopk_segments.cu: s-Top-k with adaptive p and many segments
-int configure_segment_kernels(KernelLimits* limits);
+int configure_segment_kernels();
 int reserve_segments(Workspace& ws);
 void launch_segments(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, int64_t s_len, int64_t L,
                      uint64_t seed, uint64_t step, cudaStream_t s);

@@ -165,28 +165,5 @@ bool configure_dense_cluster(K kernel) {
            cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
 }
 
-// Clusters of 2^i blocks that run at a time (a block takes an SM).
-template <typename K>
-void dense_cluster_fit(K kernel, int threads, KernelLimits* limits) {
-    for (int i = 0; i < 5; ++i) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(1 << i);
-        cfg.blockDim = dim3(threads);
-        cfg.dynamicSmemBytes = kDenseBytes;
-        cudaLaunchAttribute attr;
-        attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = 1 << i;
-        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-        cfg.attrs = &attr;
-        cfg.numAttrs = 1;
-        int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
-            cudaGetLastError();
-            n = 0;
-        }
-        limits->dense_fit[i] = n;
-    }
-}
-
 }  // namespace
 }  // namespace mlmc

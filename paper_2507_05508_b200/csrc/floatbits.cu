@@ -282,14 +282,15 @@ size_t float_pack_smem(size_t elem, int warps) { return (size_t)warps * 2 * 1024
 
 }  // namespace
 
-int configure_float_kernels(KernelLimits* limits) {
+int configure_float_kernels() {
     const bool ok = cudaFuncSetAttribute(aggregate_float_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)kAvgFloatSmem + kEmitMaxWorkers * 8) == cudaSuccess &&
                     cudaFuncSetAttribute(float_pack_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)float_pack_smem(4, kFloatThreads / 32)) == cudaSuccess;
-    limits->aggregate_float = resident_blocks(aggregate_float_kernel, kAvgThreads, kAvgFloatSmem + 64);
     return ok ? MLMC_OK : MLMC_ERR_CUDA;
 }
+
+void float_limits(KernelLimits* limits) { limits->aggregate_float = resident_blocks(aggregate_float_kernel, kAvgThreads, kAvgFloatSmem + 64); }
 
 void launch_compress_floatbits(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* mb,
                                int L, const double* p, uint64_t seed, uint64_t step, const mlmc_float_msgs& out,

@@ -505,13 +505,15 @@ bool launch_rtn_cluster(Workspace& ws, const void* g, int dtype, int64_t d, int 
     return true;
 }
 
-int configure_rtn_kernels(KernelLimits* limits) {
-    if (!configure_dense_cluster(rtn_cluster_kernel<float>) || !configure_dense_cluster(rtn_cluster_kernel<bf16_t>)) return MLMC_ERR_CUDA;
+int configure_rtn_kernels() {
+    return configure_dense_cluster(rtn_cluster_kernel<float>) && configure_dense_cluster(rtn_cluster_kernel<bf16_t>) ? MLMC_OK : MLMC_ERR_CUDA;
+}
+
+void rtn_limits(KernelLimits* limits) {
     limits->rtn_stats[0][0] = resident_blocks(rtn_stats_kernel<float, 6>, kRtnThreads, rtn_stats_smem(4));
     limits->rtn_stats[0][1] = resident_blocks(rtn_stats_kernel<float, kRtnMaxLevels>, kRtnThreads, rtn_stats_smem(4));
     limits->rtn_stats[1][0] = resident_blocks(rtn_stats_kernel<bf16_t, 6>, kRtnThreads, rtn_stats_smem(2));
     limits->rtn_stats[1][1] = resident_blocks(rtn_stats_kernel<bf16_t, kRtnMaxLevels>, kRtnThreads, rtn_stats_smem(2));
-    return MLMC_OK;
 }
 
 void launch_rtn_emit(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* r, int L,

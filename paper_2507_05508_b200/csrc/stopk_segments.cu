@@ -822,11 +822,11 @@ size_t plan_scratch(char* base, int rows, int64_t d, int64_t seg_cap, SegScratch
 
 }  // namespace
 
-int configure_segment_kernels(KernelLimits* limits) {
+int configure_segment_kernels() {
     const bool ok =
         cudaFuncSetAttribute(segment_sweep_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSegSweepSmem) == cudaSuccess &&
         cudaFuncSetAttribute(segment_sweep_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSegSweepSmem) == cudaSuccess;
-    return ok ? configure_sort_kernels(limits) : MLMC_ERR_CUDA;
+    return ok ? MLMC_OK : MLMC_ERR_CUDA;
 }
 
 // Scratch memory, taken at the first call and kept as it is until the context is destroyed: room for as many rows of d_max

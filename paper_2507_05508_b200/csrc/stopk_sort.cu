@@ -346,18 +346,19 @@ sort_rows_kernel(const uint32_t* g, int64_t d, int64_t ld, int rows, const RowHe
 
 }  // namespace
 
-int configure_sort_kernels(KernelLimits* limits) {  // the tile and the tables pass 48 KB
-    const int bytes = (int)(kSortSmemWords * sizeof(uint32_t));
-    if (cudaFuncSetAttribute(sort_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return MLMC_ERR_CUDA;
-    limits->sort_rows = resident_blocks(sort_rows_kernel, kSortThreads, bytes);
-    return MLMC_OK;
+constexpr size_t kSortSmem = kSortSmemWords * sizeof(uint32_t);  // the tile and the tables pass 48 KB
+
+int configure_sort_kernels() {
+    return cudaFuncSetAttribute(sort_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSortSmem) == cudaSuccess ? MLMC_OK : MLMC_ERR_CUDA;
 }
+
+void sort_limits(KernelLimits* limits) { limits->sort_rows = resident_blocks(sort_rows_kernel, kSortThreads, kSortSmem); }
 
 void launch_sorted_rows(Workspace& ws, const float* g, int64_t d, int rows, int64_t ld, const RowHead* head, const SortBuffers& buf,
                         uint32_t s_len, uint32_t L, double* delta, int64_t seg_cap, cudaStream_t s) {
     const int tiles = (int)sort_tiles(d);
     const int blocks = (int)std::min<int64_t>((int64_t)tiles * rows, (int64_t)ws.sm_count * ws.limits.sort_rows);  // all of them run at a time
-    launch_kernel_grid(ws, K_SORT_ROWS, sort_rows_kernel, dim3((unsigned)blocks), kSortThreads, kSortSmemWords * sizeof(uint32_t), s,
+    launch_kernel_grid(ws, K_SORT_ROWS, sort_rows_kernel, dim3((unsigned)blocks), kSortThreads, kSortSmem, s,
                        reinterpret_cast<const uint32_t*>(g), d, ld, rows, head, buf, tiles, s_len, L, delta, seg_cap);
 }
 

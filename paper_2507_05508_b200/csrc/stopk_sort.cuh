@@ -25,7 +25,8 @@ struct SortBuffers {
     int64_t stride;
 };
 
-int configure_sort_kernels(KernelLimits* limits);
+int configure_sort_kernels();
+void sort_limits(KernelLimits* limits);
 // Sorts the rows with head.sorted and writes the norms of their segments to delta[rows][seg_cap].
 void launch_sorted_rows(Workspace& ws, const float* g, int64_t d, int rows, int64_t ld, const RowHead* head, const SortBuffers& buf,
                         uint32_t s_len, uint32_t L, double* delta, int64_t seg_cap, cudaStream_t s);

@@ -568,33 +568,15 @@ size_t cluster_smem(int per_block) { return kClFixedSmem + (size_t)per_block * k
 
 }  // namespace
 
-int configure_cluster_kernels(KernelLimits* limits) {
+int configure_cluster_kernels() {
     auto set = [&](auto kernel) {
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cluster_smem(kClBatches)) != cudaSuccess) return false;
         return cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
     };
-    if (!set(cluster_topk_kernel<float>) || !set(cluster_topk_kernel<bf16_t>)) return MLMC_ERR_CUDA;
-    // clusters of 2^i blocks that run at a time (a block takes an SM)
-    for (int i = 0; i < 5; ++i) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(1 << i);
-        cfg.blockDim = dim3(kClThreads);
-        cfg.dynamicSmemBytes = cluster_smem(kClBatches);
-        cudaLaunchAttribute attr;
-        attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = 1 << i;
-        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-        cfg.attrs = &attr;
-        cfg.numAttrs = 1;
-        int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, cluster_topk_kernel<float>, &cfg) != cudaSuccess) {
-            cudaGetLastError();
-            n = 0;
-        }
-        limits->topk_fit[i] = n;
-    }
-    return MLMC_OK;
+    return set(cluster_topk_kernel<float>) && set(cluster_topk_kernel<bf16_t>) ? MLMC_OK : MLMC_ERR_CUDA;
 }
+
+void cluster_limits(KernelLimits* limits) { clusters_that_fit(cluster_topk_kernel<float>, kClThreads, cluster_smem(kClBatches), limits->topk_fit); }
 
 // Blocks per cluster for this call, 0: the row is too long, or the workers are too many, for the cluster to be the faster way.
 // The smallest cluster whose blocks have at most kClEasy batches: a barrier and an exchange between more blocks take longer

@@ -433,16 +433,19 @@ aggregate_topk_direct_kernel(const uint32_t* __restrict__ idx, const float* __re
 
 }  // namespace
 
-int configure_emit_kernels(KernelLimits* limits) {
+int configure_emit_kernels() {
     auto set = [](auto kernel, int words) {
         return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (kBandThreads / 32) * words * (int)sizeof(uint32_t)) == cudaSuccess;
     };
-    if (!set(band_write_kernel<float>, kWriteWords<float>) || !set(band_write_kernel<bf16_t>, kWriteWords<bf16_t>)) return MLMC_ERR_CUDA;
+    return set(band_write_kernel<float>, kWriteWords<float>) && set(band_write_kernel<bf16_t>, kWriteWords<bf16_t>) ? MLMC_OK
+                                                                                                                   : MLMC_ERR_CUDA;
+}
+
+void emit_limits(KernelLimits* limits) {
     limits->band_count[0] = resident_blocks(band_count_kernel<float>, kBandThreads, 256);
     limits->band_count[1] = resident_blocks(band_count_kernel<bf16_t>, kBandThreads, 256);
     limits->aggregate_topk = resident_blocks(aggregate_topk_warps_kernel, kAggWarps * 32, 0);
-    return MLMC_OK;
 }
 
 namespace {
