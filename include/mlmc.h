@@ -138,10 +138,10 @@ int mlmc_aggregate(mlmc_ctx* ctx, int kind, const void* msgs, const int32_t* b, 
  * segments and a given p the level is drawn before the data is read and only the two thresholds of its segment are
  * selected.  With more segments and adaptive p every segment norm is needed: one sweep for a histogram of the leading
  * key digits and, for fp32, one more that adds up the energies of the bins without a segment boundary and collects the
- * keys of the others; rows with too many of those are sorted instead.  As many rows are taken together as fit in 2 GiB of
- * scratch memory (about 8.2 d + 40 L bytes and 3 MB per row; in any case there is room for one row of d_max entries with the most
- * segments), which the first such call on a context takes with one cudaMalloc (MLMC_ERR_NOMEM if it fails; kept until
- * mlmc_destroy): make that call before capturing one.
+ * keys of the others; rows with too many of those are sorted instead.  As many rows are taken together as fit in 1 GiB of
+ * scratch memory (about 4 d + 40 L bytes and 3 MB per row, and 4 max(2^25, d) for the sort; in any case there is room for one row of
+ * d_max entries with the most segments), which the first such call on a context takes with one cudaMalloc
+ * (MLMC_ERR_NOMEM if it fails; kept until mlmc_destroy): make that call before capturing one.
  * Returns MLMC_ERR_ARG when L exceeds the limit. */
 int mlmc_compress_stopk(mlmc_ctx* ctx, const void* g, int dtype, int64_t d, int M, int64_t ld, int64_t s,
                         const double* p, uint64_t seed, uint64_t step, const mlmc_topk_msgs* out, void* stream);

@@ -24,7 +24,7 @@ namespace {
 constexpr int kSegThreads = 1024;
 constexpr int kBucketThreads = 256;
 constexpr int kMaxCells = kBins1;                            // (segment, exponent) pairs of bins without a boundary
-constexpr size_t kSegScratchBudget = size_t(1) << 31;
+constexpr size_t kSegScratchBudget = size_t(1) << 30;
 
 // A row is sorted (stopk_sort.cu) where too many of its keys lie in buckets, or more than 1/32 of them in one bucket; not where that
 // is fewer than kFewKeys keys in all, or kFewEqual in one bucket: the passes of a sort take that long at least.
@@ -764,7 +764,7 @@ segment_draw_kernel(const uint32_t* hist1, int m0, uint32_t d, uint32_t s_len, u
             q.T = (uint32_t)lo;
             q.r = k - (lo == kBins1 - 1 ? 0u : S[lo + 1]);
         } else if (sc.head[row].sorted) {
-            const uint32_t* keys = sc.sort.b + (int64_t)row * sc.sort.stride;
+            const uint32_t* keys = sc.sort.a + (int64_t)row * sc.sort.stride;
             const uint32_t at = keys[k - 1u];
             uint32_t lo = 0, hi = k - 1u;  // the first place of that key
             while (lo < hi) {
@@ -809,15 +809,28 @@ size_t plan_scratch(char* base, int rows, int64_t d, int64_t seg_cap, SegScratch
     sc->prefix = pl.take<Wide>(r * seg_cap);
     sc->delta = pl.take<double>(r * seg_cap);
     sc->head = pl.take<RowHead>(r);
-    const size_t tiles = (size_t)sort_tiles(d);
+    const size_t tiles = (size_t)sort_tiles(d), slots = (size_t)sort_slots(d, rows);
     sc->sort.a = sc->keys;
-    sc->sort.b = pl.take<uint32_t>(r * d);
-    sc->sort.table = pl.take<uint32_t>(r * 256 * tiles);
-    sc->sort.totals = pl.take<uint32_t>(r * 256);
+    sc->sort.b = pl.take<uint32_t>(slots * d);
+    sc->sort.table = pl.take<uint32_t>(slots * 256 * tiles);
+    sc->sort.totals = pl.take<uint32_t>(slots * 256);
     sc->sort.stride = d;
+    sc->sort.slots = (int)slots;
     sc->key_stride = d;
     sc->seg_cap = seg_cap;
     return pl.off + 256;
+}
+
+// Rows whose scratch memory fits in so many bytes, at least one.
+int rows_within(size_t bytes, int most, int64_t d, int64_t L) {
+    SegScratch sc;
+    int lo = 1, hi = most;
+    while (lo < hi) {
+        const int mid = lo + (hi - lo + 1) / 2;
+        if (plan_scratch(nullptr, mid, d, L, &sc) <= bytes) lo = mid;
+        else hi = mid - 1;
+    }
+    return lo;
 }
 
 }  // namespace
@@ -837,8 +850,7 @@ int reserve_segments(Workspace& ws) {
     if (ws.seg_scratch) return MLMC_OK;
     SegScratch sc;
     const int64_t few = std::min(ws.big_cap, (int64_t)4096);
-    const int64_t rows = std::max<int64_t>(1, (int64_t)(kSegScratchBudget / plan_scratch(nullptr, 1, ws.d_max, few, &sc)));
-    ws.seg_bytes = std::max(plan_scratch(nullptr, (int)std::min<int64_t>(ws.M_max, rows), ws.d_max, few, &sc),
+    ws.seg_bytes = std::max(plan_scratch(nullptr, rows_within(kSegScratchBudget, ws.M_max, ws.d_max, few), ws.d_max, few, &sc),
                             plan_scratch(nullptr, 1, ws.d_max, ws.big_cap, &sc));
     if (cudaMalloc(&ws.seg_scratch, ws.seg_bytes) != cudaSuccess) {
         cudaGetLastError();
@@ -852,8 +864,7 @@ int reserve_segments(Workspace& ws) {
 void launch_segments(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, int64_t s_len, int64_t L,
                      uint64_t seed, uint64_t step, cudaStream_t s) {
     SegScratch sc;
-    int together = (int)std::min<size_t>((size_t)M, ws.seg_bytes / plan_scratch(nullptr, 1, d, L, &sc));  // at least 1
-    while (together < M && plan_scratch(nullptr, together + 1, d, L, &sc) <= ws.seg_bytes) ++together;
+    const int together = rows_within(ws.seg_bytes, M, d, L);
     plan_scratch(static_cast<char*>(ws.seg_scratch), together, d, L, &sc);
     const uint32_t sl = (uint32_t)s_len, nl = (uint32_t)L, du = (uint32_t)d;
     for (int m0 = 0; m0 < M; m0 += together) {

@@ -8,7 +8,7 @@
 // stride over the tiles of the rows to be sorted.  (As 13 launches it cost 17 us on calls without such a row, now 3.)
 // The steps are bound by latency: a scatter takes 210 us for 4 x 11.7M keys, a count 30; the loads of a tile go out together, while
 // the tile before is written (one by one behind the test for the row's end a count took 137).
-// 11.7M x 4, L = 100, 95 % zeros: 28.6 ms in buckets, 1.68 sorted; 16 rows with 30 % zeros: 9.0 and 5.1 ms.
+// 11.7M x 4, L = 100, 95 % zeros: 28.6 ms in buckets, 1.72 sorted; 16 rows with 30 % zeros, three of them at a time: 8.7 and 5.6 ms.
 #include <algorithm>
 
 #include <cooperative_groups.h>
@@ -49,15 +49,16 @@ struct PassInput {
     const uint32_t* rows;
     int64_t stride;
     uint32_t flip;                                           // kSortFlip for the gradient, else 0
+    bool by_slot;
     __device__ __forceinline__ uint32_t key(uint32_t x) const { return (x ^ flip) & (flip ? kSortFlip : 0xFFFFFFFFu); }
 };
 
 constexpr int kSortSmemWords = kSortTile + 3 * kSortWarps * 256;  // the ordered tile, the warp tables, two mask tables
 
 // The keys of a tile, kSortItems per thread; each warp owns kWarpKeys consecutive ones.
-__device__ __forceinline__ void load_tile(const PassInput& in, int row, int tile, int64_t n, uint32_t (&key)[kSortItems]) {
+__device__ __forceinline__ void load_tile(const PassInput& in, int slot, int row, int tile, int64_t n, uint32_t (&key)[kSortItems]) {
     const int64_t w0 = (int64_t)tile * kSortTile + (int64_t)(threadIdx.x >> 5) * kWarpKeys + (threadIdx.x & 31);
-    const uint32_t* src = in.rows + (int64_t)row * in.stride + w0;
+    const uint32_t* src = in.rows + (int64_t)(in.by_slot ? slot : row) * in.stride + w0;
     if ((int64_t)(tile + 1) * kSortTile <= n) {
 #pragma unroll
         for (int j = 0; j < kSortItems; ++j) key[j] = __ldcg(src + j * 32);
@@ -67,8 +68,8 @@ __device__ __forceinline__ void load_tile(const PassInput& in, int row, int tile
     }
 }
 
-// table[digit][tile] of a row = keys of the tile with that digit.
-__device__ __forceinline__ void count_tile(const PassInput& in, const uint32_t (&key)[kSortItems], int row, int tile, int64_t n, int shift, uint32_t* table, int tiles,
+// table[digit][tile] of a slot = keys of the tile with that digit.
+__device__ __forceinline__ void count_tile(const PassInput& in, const uint32_t (&key)[kSortItems], int slot, int tile, int64_t n, int shift, uint32_t* table, int tiles,
                                            uint32_t* sh_hist /* [warp][256] */) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t w0 = (int64_t)tile * kSortTile + (int64_t)warp * kWarpKeys + lane;
@@ -82,12 +83,12 @@ __device__ __forceinline__ void count_tile(const PassInput& in, const uint32_t (
         uint32_t tot = 0;
 #pragma unroll
         for (int w = 0; w < kSortWarps; ++w) tot += sh_hist[w * 256 + threadIdx.x];
-        table[((int64_t)row * 256 + threadIdx.x) * tiles + tile] = tot;
+        table[((int64_t)slot * 256 + threadIdx.x) * tiles + tile] = tot;
     }
     __syncthreads();
 }
 
-// Exclusive scan, in place, of the tile counts of one digit of one row, by a warp; the digit's total goes to totals[row][digit].
+// Exclusive scan, in place, of the tile counts of one digit of one row, by a warp; the digit's total goes to totals[slot][digit].
 // The scatter adds the totals of the digits below.
 __device__ __forceinline__ void scan_digit(uint32_t* entries, int tiles, uint32_t* total) {
     const int lane = threadIdx.x & 31;
@@ -128,7 +129,7 @@ __device__ __forceinline__ void scan_digit(uint32_t* entries, int tiles, uint32_
 // clearing of the step before).
 // The next tile's keys are asked for (load_next) when this tile's have left their registers.
 template <typename F>
-__device__ __forceinline__ void scatter_tile(const PassInput& in, uint32_t (&key)[kSortItems], F&& load_next, int row, int tile, uint32_t* out, int64_t out_stride,
+__device__ __forceinline__ void scatter_tile(const PassInput& in, uint32_t (&key)[kSortItems], F&& load_next, int slot, int tile, uint32_t* out_row,
                                              int64_t n, int shift, const uint32_t* tables, const uint32_t* totals, int tiles, uint32_t* sh_dyn) {
     uint32_t* sh_key = sh_dyn;                            // [kSortTile]
     uint32_t* sh_hist = sh_dyn + kSortTile;               // [warp][256]
@@ -175,7 +176,7 @@ __device__ __forceinline__ void scatter_tile(const PassInput& in, uint32_t (&key
         if (threadIdx.x < 256) {
 #pragma unroll
             for (int w = 0; w < kSortWarps; ++w) total += sh_hist[w * 256 + threadIdx.x];
-            gtotal = totals[row * 256 + threadIdx.x];
+            gtotal = __ldcg(&totals[slot * 256 + threadIdx.x]);
         }
         uint32_t incl = total, gincl = gtotal;
 #pragma unroll
@@ -198,7 +199,7 @@ __device__ __forceinline__ void scatter_tile(const PassInput& in, uint32_t (&key
                 start += sh_wsum[w];
                 gstart += sh_gsum[w];
             }
-            sh_shift[threadIdx.x] = gstart + tables[((int64_t)row * 256 + threadIdx.x) * tiles + tile] - start;
+            sh_shift[threadIdx.x] = gstart + __ldcg(&tables[((int64_t)slot * 256 + threadIdx.x) * tiles + tile]) - start;
             uint32_t run = start;
 #pragma unroll
             for (int w = 0; w < kSortWarps; ++w) {
@@ -219,7 +220,6 @@ __device__ __forceinline__ void scatter_tile(const PassInput& in, uint32_t (&key
     __syncthreads();
     load_next();
     const int tile_n = (int)((n - tile0 < (int64_t)kSortTile) ? (n - tile0) : (int64_t)kSortTile);
-    uint32_t* out_row = out + (int64_t)row * out_stride;
 #pragma unroll
     for (int j = 0; j < kSortItems; ++j) {
         const int pos = j * kSortThreads + threadIdx.x;
@@ -267,13 +267,14 @@ sort_rows_kernel(const uint32_t* g, int64_t d, int64_t ld, int rows, const RowHe
     extern __shared__ __align__(16) uint32_t sh_dyn[];
     __shared__ uint16_t sh_list[kEmitMaxWorkers];
     pdl_enter();
-    const int n_rows = list_rows(head, rows, sh_list);
-    if (n_rows == 0) return;
+    const int listed = list_rows(head, rows, sh_list);
+    if (listed == 0) return;
     cg::grid_group grid = cg::this_grid();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // the block's tiles: every gridDim.x-th of all rows to be sorted
+    const uint32_t warps = gridDim.x * kSortWarps, first = blockIdx.x * kSortWarps + warp;
+    // the block's tiles: every gridDim.x-th of all rows that are sorted at a time
     struct Place {
-        int i, tile;   // the i-th of those rows
+        int i, tile;   // the slot of the row
     };
     auto settle = [&](Place at) -> Place {
         while (at.tile >= tiles) {
@@ -283,64 +284,67 @@ sort_rows_kernel(const uint32_t* g, int64_t d, int64_t ld, int rows, const RowHe
         return at;
     };
     const Place start = settle({0, (int)blockIdx.x});
-    PassInput in = {g, ld, kSortFlip};
 #pragma unroll 1
-    for (int p = 0; p < 4; ++p) {  // 31-bit keys: from the gradient to a, to b, to a, to b
-        const int shift = 8 * p;
-        uint32_t* dst = (p & 1) ? buf.b : buf.a;
-        uint32_t key[kSortItems], next[kSortItems];
-        auto load = [&](const Place& at, uint32_t (&k)[kSortItems]) {
-            if (at.i < n_rows) load_tile(in, sh_list[at.i], at.tile, d, k);
-        };
-        load(start, key);
+    for (int r0 = 0; r0 < listed; r0 += buf.slots) {
+        const int n_rows = min(buf.slots, listed - r0);
+        const uint16_t* list = sh_list + r0;
+        PassInput in = {g, ld, kSortFlip, false};
 #pragma unroll 1
-        for (Place at = start; at.i < n_rows;) {
-            const Place then = settle({at.i, at.tile + (int)gridDim.x});
-            load(then, next);
-            count_tile(in, key, sh_list[at.i], at.tile, d, shift, buf.table, tiles, sh_dyn);
+        for (int p = 0; p < 4; ++p) {  // 31-bit keys: from the gradient to b, to a, to b, to a
+            const int shift = 8 * p;
+            uint32_t key[kSortItems], next[kSortItems];
+            auto load = [&](const Place& at, uint32_t (&k)[kSortItems]) {
+                if (at.i < n_rows) load_tile(in, at.i, list[at.i], at.tile, d, k);
+            };
+            load(start, key);
+#pragma unroll 1
+            for (Place at = start; at.i < n_rows;) {
+                const Place then = settle({at.i, at.tile + (int)gridDim.x});
+                load(then, next);
+                count_tile(in, key, at.i, at.tile, d, shift, buf.table, tiles, sh_dyn);
 #pragma unroll
-            for (int j = 0; j < kSortItems; ++j) key[j] = next[j];
-            at = then;
-        }
-        grid.sync();
-        for (int i = (int)blockIdx.x * kSortWarps + warp; i < n_rows * 256; i += (int)gridDim.x * kSortWarps) {
-            const int entry = sh_list[i >> 8] * 256 + (i & 255);
-            scan_digit(buf.table + (int64_t)entry * tiles, tiles, &buf.totals[entry]);
-        }
-        grid.sync();
-        load(start, key);
+                for (int j = 0; j < kSortItems; ++j) key[j] = next[j];
+                at = then;
+            }
+            grid.sync();
+            for (uint32_t i = first; i < (uint32_t)n_rows * 256u; i += warps) scan_digit(buf.table + (int64_t)i * tiles, tiles, &buf.totals[i]);
+            grid.sync();
+            load(start, key);
 #pragma unroll 1
-        for (Place at = start; at.i < n_rows;) {
-            const Place then = settle({at.i, at.tile + (int)gridDim.x});
-            scatter_tile(in, key, [&]() { load(then, key); }, sh_list[at.i], at.tile, dst, buf.stride, d, shift, buf.table, buf.totals, tiles, sh_dyn);
-            at = then;
+            for (Place at = start; at.i < n_rows;) {
+                const Place then = settle({at.i, at.tile + (int)gridDim.x});
+                uint32_t* out_row = (p & 1) ? buf.a + (int64_t)list[at.i] * buf.stride : buf.b + (int64_t)at.i * buf.stride;
+                scatter_tile(in, key, [&]() { load(then, key); }, at.i, at.tile, out_row, d, shift, buf.table, buf.totals, tiles, sh_dyn);
+                at = then;
+            }
+            grid.sync();
+            in = {(p & 1) ? buf.a : buf.b, buf.stride, 0u, (p & 1) == 0};
         }
-        grid.sync();
-        in = {dst, buf.stride, 0u};
-    }
-    const uint32_t cps = (s_len + kNormChunk - 1) / kNormChunk, warps = gridDim.x * kSortWarps, first = blockIdx.x * kSortWarps + warp;
-    const int64_t items = (int64_t)L * cps;
-    double* partial = reinterpret_cast<double*>(buf.table);
-    for (int i = 0; i < n_rows; ++i) {
-        const uint32_t* keys = in.rows + (int64_t)sh_list[i] * in.stride;
-        for (int64_t at = first; at < items; at += warps) {
-            const int64_t l = at / cps, begin = l * s_len + (at - l * cps) * kNormChunk;
-            const int64_t end = min(min(begin + kNormChunk, (l + 1) * (int64_t)s_len), d);
-            const double e = segment_energy(keys, begin, end);
-            if (lane == 0) {
-                if (cps == 1) delta[(int64_t)sh_list[i] * seg_cap + l] = sqrt(e);
-                else partial[(int64_t)sh_list[i] * 128 * tiles + at] = e;
+        const uint32_t cps = (s_len + kNormChunk - 1) / kNormChunk;
+        const int64_t items = (int64_t)L * cps;
+        double* partial = reinterpret_cast<double*>(buf.table);
+        for (int i = 0; i < n_rows; ++i) {
+            const uint32_t* keys = buf.a + (int64_t)list[i] * buf.stride;
+            for (int64_t at = first; at < items; at += warps) {
+                const int64_t l = at / cps, begin = l * s_len + (at - l * cps) * kNormChunk;
+                const int64_t end = min(min(begin + kNormChunk, (l + 1) * (int64_t)s_len), d);
+                const double e = segment_energy(keys, begin, end);
+                if (lane == 0) {
+                    if (cps == 1) delta[(int64_t)list[i] * seg_cap + l] = sqrt(e);
+                    else partial[(int64_t)i * 128 * tiles + at] = e;
+                }
             }
         }
-    }
-    if (cps == 1) return;
-    grid.sync();
-    for (int64_t at = (int64_t)first * 32 + lane; at < (int64_t)n_rows * L; at += (int64_t)warps * 32) {
-        const int row = sh_list[at / L];
-        const double* part = partial + (int64_t)row * 128 * tiles + (at % L) * cps;
-        double e = 0.0;
-        for (uint32_t c = 0; c < cps; ++c) e += __ldcg(part + c);
-        delta[(int64_t)row * seg_cap + at % L] = sqrt(e);
+        if (cps == 1) continue;  // the next rows' counts do not touch what is read here
+        grid.sync();
+        for (int64_t at = (int64_t)first * 32 + lane; at < (int64_t)n_rows * L; at += (int64_t)warps * 32) {
+            const int i = (int)(at / L);
+            const double* part = partial + (int64_t)i * 128 * tiles + (at % L) * cps;
+            double e = 0.0;
+            for (uint32_t c = 0; c < cps; ++c) e += __ldcg(part + c);
+            delta[(int64_t)list[i] * seg_cap + at % L] = sqrt(e);
+        }
+        grid.sync();  // the sums have been read: the table takes the next rows' counts
     }
 }
 
@@ -357,7 +361,7 @@ void sort_limits(KernelLimits* limits) { limits->sort_rows = resident_blocks(sor
 void launch_sorted_rows(Workspace& ws, const float* g, int64_t d, int rows, int64_t ld, const RowHead* head, const SortBuffers& buf,
                         uint32_t s_len, uint32_t L, double* delta, int64_t seg_cap, cudaStream_t s) {
     const int tiles = (int)sort_tiles(d);
-    const int blocks = (int)std::min<int64_t>((int64_t)tiles * rows, (int64_t)ws.sm_count * ws.limits.sort_rows);  // all of them run at a time
+    const int blocks = (int)std::min<int64_t>((int64_t)tiles * buf.slots, (int64_t)ws.sm_count * ws.limits.sort_rows);  // all of them run at a time
     launch_kernel_grid(ws, K_SORT_ROWS, sort_rows_kernel, dim3((unsigned)blocks), kSortThreads, kSortSmem, s,
                        reinterpret_cast<const uint32_t*>(g), d, ld, rows, head, buf, tiles, s_len, L, delta, seg_cap);
 }

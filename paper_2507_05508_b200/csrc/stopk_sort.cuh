@@ -17,12 +17,19 @@ constexpr uint32_t kSortFlip = 0x7FFFFFFFu;                  // sort key = flip 
 
 inline int64_t sort_tiles(int64_t d) { return (d + kSortTile - 1) / kSortTile; }
 
+// Rows that are sorted at a time: as many as keep the GPU busy (32M keys), so that all but the first buffer stay small.
+inline int sort_slots(int64_t d, int rows) {
+    const int64_t n = ((int64_t(1) << 25) + d - 1) / d;
+    return n < rows ? (int)n : rows;
+}
+
 struct SortBuffers {
-    uint32_t* a;             // [rows][stride]
-    uint32_t* b;             // [rows][stride]  the sorted row
-    uint32_t* table;         // [rows][256][tiles]
-    uint32_t* totals;        // [rows][256]
+    uint32_t* a;             // [rows][stride]   the sorted row
+    uint32_t* b;             // [slots][stride]
+    uint32_t* table;         // [slots][256][tiles]
+    uint32_t* totals;        // [slots][256]
     int64_t stride;
+    int slots;
 };
 
 int configure_sort_kernels();
