@@ -14,8 +14,8 @@
  *  - Pointers are DEVICE pointers unless marked "host".  The caller owns every buffer; the library
  *    only owns the scratch workspace inside mlmc_ctx.
  *  - All work is enqueued on the caller's stream (a cudaStream_t passed as void*; NULL = default
- *    stream).  Nothing synchronises except mlmc_create, mlmc_destroy and mlmc_get_status (and the
- *    measurement calls of mlmc_instr.h, which are not part of the method).
+ *    stream).  Nothing synchronises except mlmc_create, mlmc_destroy, mlmc_get_status and the first mlmc_compress_stopk of
+ *    a context that needs its scratch memory (and the measurement calls of mlmc_instr.h, which are not part of the method).
  *  - The int return value reports host-side checks made before any launch (arguments, schedule,
  *    probabilities).  Conditions found on the device (message capacity, non-finite input, a bounded
  *    wait that gave up) are written to a sticky status word read by mlmc_get_status; the affected
@@ -24,8 +24,9 @@
  *    when M > 1, ld * sizeof(element) must be a multiple of 16.  d < 2^32.  g is never written.
  *  - Total order for Top-k: |g_i| descending, equal magnitudes by ascending index i.
  *  - One uniform per (seed, step, worker) drives the level draw: three chained SplitMix64 output
- *    rounds, u = (h >> 11) * 2^-53; cdf accumulated in ascending l in fp64, the cdf of the last level
- *    with p > 0 set to 1, l* = min{ l : u < cdf_l }.
+ *    rounds, u = (h >> 11) * 2^-53; cdf accumulated in ascending l in fp64 (adaptive s-Top-k with more than MLMC_MAX_LEVELS
+ *    segments: runs of ceil(L / 1024) segments in ascending order, their sums by a tree), the cdf of the last level with
+ *    p > 0 set to 1, l* = min{ l : u < cdf_l }.
  *  - One mlmc_ctx serves one stream at a time.  Contexts share nothing: calls on different contexts may run
  *    side by side on different streams.
  */
@@ -50,7 +51,7 @@ typedef enum {
     MLMC_ERR_PROB = -3,      /* some p_l <= 0 or sum p != 1 (Lemma 3.2 needs non-zero probabilities) */
     MLMC_ERR_CAPACITY = -4,  /* device: a Top-k message does not fit out->capacity / planes exceed w_max */
     MLMC_ERR_NONFINITE = -5, /* device: NaN or Inf in g */
-    MLMC_ERR_TIMEOUT = -6,   /* reserved (no kernel of this version waits for another thread block) */
+    MLMC_ERR_TIMEOUT = -6,   /* reserved (thread blocks wait for one another only at barriers of clusters and cooperative launches) */
     MLMC_ERR_CUDA = -7,      /* a CUDA runtime call failed */
     MLMC_ERR_NOMEM = -8,     /* workspace allocation failed */
     MLMC_ERR_INTERNAL = -9   /* device: a self-check failed (emitted count differs from k_l - k_{l-1}) */

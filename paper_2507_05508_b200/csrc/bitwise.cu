@@ -19,7 +19,6 @@ struct BitSchedule {
     int L;
     int B;
     int shift[kMaxLevels];      // B - b_l
-    uint32_t mask[kMaxLevels];  // 2^{w_l} - 1
     int width[kMaxLevels];      // w_l
     int bits[kMaxLevels];       // b_l
     // levels of at most 8 bits in runs of at most 8 bits together
@@ -561,14 +560,13 @@ BitSchedule make_schedule(const int32_t* b, int L) {
         sc.bits[l] = b[l];
         sc.width[l] = w;
         sc.shift[l] = sc.B - b[l];
-        sc.mask[l] = (w >= 32) ? 0xFFFFFFFFu : ((1u << w) - 1u);
     }
     for (int l = 0, end; l < L; l = end) {
         for (end = l + 1; end < L && b[end] - (l ? b[l - 1] : 0) <= 8;) ++end;
         for (int i = l; i < end; ++i) {
             sc.run_up[i] = 1u << (24 - sc.B + b[end - 1]);
             sc.in_run[i] = b[end - 1] - b[i];
-            sc.mask4[i] = ((sc.mask[i] << sc.in_run[i]) & 0xFFu) * 0x01010101u;
+            sc.mask4[i] = ((((1u << sc.width[i]) - 1u) << sc.in_run[i]) & 0xFFu) * 0x01010101u;
         }
     }
     return sc;

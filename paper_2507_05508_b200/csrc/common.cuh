@@ -438,14 +438,6 @@ __device__ __forceinline__ void stream_trips(const uint4* __restrict__ src, int6
     cp_async_wait<0>();
 }
 
-// Contiguous range of 16-byte vectors handled by block `bx` of `nb` blocks over a row of d elements.
-__device__ __forceinline__ void block_vector_range(int64_t d, int vec, int bx, int nb, int64_t* v0, int64_t* v1) {
-    const int64_t nvec = (d + vec - 1) / vec;
-    const int64_t per = (nvec + nb - 1) / nb;
-    *v0 = min((int64_t)bx * per, nvec);
-    *v1 = min(*v0 + per, nvec);
-}
-
 // Emit tiles of one row: kEmitTile 32-bit words each (one fp32 or two bf16 elements per word).
 inline int emit_tiles_per_worker(int64_t d, int dtype) {
     const int per_word = (dtype == MLMC_BF16) ? 2 : 1;
