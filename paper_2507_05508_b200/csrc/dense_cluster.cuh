@@ -33,8 +33,11 @@ struct DenseShared {
 
 // Blocks per cluster, 0: the row is too long or the workers too many.  A group per warp if the clusters of all workers fit the
 // GPU at a time (they are placed within a GPC: 16-block clusters leave SMs over), otherwise the largest clusters that do.
-// With more than kDenseGroups groups per block the few warps of the clusters take longer than three kernels on the whole GPU:
-// adaptive bit-wise code, 6 x 400,003 bf16 (25 groups) 20 against 24 us, 8 x 700,000 fp32 (43) 52 against 35.
+// With more than kDenseGroups groups per block the few warps of two workers' clusters take as long as kernels on the whole GPU.
+// us per message, cluster / kernels, 16 blocks, groups per block 20, 28, 36, 48:
+//   bit-wise, fp32, adaptive, 2 workers 14 / 19, 16 / 19, 19 / 19, 21 / 19;  7 workers 15 / 22, 17 / 25, 20 / 28, 23 / 33
+//   RTN, fp32, adaptive, 2 workers 19 / 22, 25 / 23, 28 / 25, 35 / 26;       7 workers 20 / 27, 25 / 32, 28 / 34, 34 / 41
+//   RTN, fp32, given p, 2 workers 10 / 10, 12 / 10, 13 / 11, 16 / 11;        7 workers 10 / 14, 12 / 14, 14 / 16, 16 / 17
 inline int dense_cluster_blocks(const Workspace& ws, int64_t d, int M) {
     const int64_t groups = (d + 1023) / 1024;
     int best = 0;

@@ -523,7 +523,7 @@ sums_candidates_kernel(const float* __restrict__ g, int64_t d, int64_t ld, const
 
     const uint32_t slots0 = (uint32_t)__cvta_generic_to_shared(slots), step = (uint32_t)threads * 4u;
     uint32_t at = slots0;
-    bool over = false;  // the list is full (warp-uniform)
+    bool over = false;  // without energies: the list is full (warp-uniform)
     auto flush = [&]() {  // called by the whole warp
         const uint32_t n = (at - slots0) / step;
         uint32_t upto = n;
@@ -541,7 +541,7 @@ sums_candidates_kernel(const float* __restrict__ g, int64_t d, int64_t ld, const
             uint32_t* to = cand + base + (upto - n);
             for (uint32_t i = 0; i < n; ++i) to[i] = slots[i * threads] & 0x7FFFFFFFu;
         } else {
-            over = true;
+            if (!SUMS) over = true;
             if (lane == 0) cand_overflow[m] = 1;  // too many keys share the boundary bins: the full-sweep passes take over
         }
         at = slots0;
