@@ -327,16 +327,19 @@ class Runner:
             self.B.mlmc_destroy(ctx)
 
 
+SAMPLED_LEAST = 1 << 28  # entries of a call from which adaptive fp32 Top-k of at most 15 levels selects in one sweep
+
+
 def sweeps_charged(w, emit_read_frac=None) -> float:
     """Gradient sweeps charged to the step: what the method needs (a true data dependence separates them: select ->
     emit for Top-k, max -> pack for fixed-p bit-wise, max -> field energies -> pack for adaptive bit-wise), or what
-    the kernels moved where that is less.  Top-k moves one whole histogram sweep, for adaptive fp32 a second whole
-    sweep, and two passes over the listed tiles (emit_read_frac of the row each); the fixed-p candidate sweep,
-    which also skips tiles, is counted as nothing, so the figure is a lower bound of the bytes moved."""
+    the kernels moved where that is less.  Top-k moves one whole sweep, for adaptive fp32 rows too short to be sampled a
+    second one, and two passes over the listed tiles (emit_read_frac of the row each); the fixed-p candidate sweep,
+    which also skips tiles, is counted as nothing: the figure is a lower bound of the bytes moved."""
     if w.kind in ("topk", "stopk"):
         if emit_read_frac is None:
             return 2.0
-        moved = 1.0 + (1.0 if (w.adaptive and w.dtype != "bf16") else 0.0) + 2.0 * emit_read_frac
+        moved = 1.0 + (1.0 if (w.adaptive and w.dtype != "bf16" and w.M * w.d < SAMPLED_LEAST) else 0.0) + 2.0 * emit_read_frac
         return min(2.0, moved)
     if w.kind == "floatbits":
         return 1.0  # App. B's probabilities are fixed: the level is drawn before the data is read, one sweep packs it
@@ -353,7 +356,7 @@ def kernel_alg_bytes(name: str, sweep: float, msg: dict, dense: float, read_frac
     listed = None if read_frac is None else read_frac * sweep
     table = {
         # the digit passes read the row only where a worker's candidates overflowed: no bytes are claimed for them
-        "hist1": sweep, "segment_sweep": sweep, "sums_candidates": sweep if adaptive else None,
+        "hist1": sweep, "bracket_sweep": sweep, "segment_sweep": sweep, "sums_candidates": sweep if adaptive else None,
         "band_count": listed, "emit": None if listed is None else listed + mt,
         "aggregate_topk": mt + dense,
         "absmax": sweep, "bit_stats": sweep, "bit_pack": sweep + mb, "aggregate_bitwise": mb + dense,

@@ -119,12 +119,24 @@ int finish(cudaError_t e) { return e == cudaSuccess ? MLMC_OK : MLMC_ERR_CUDA; }
 // where both boundary bins of a worker's band fall inside, the candidate sweep has nothing left to do.
 void run_selection(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const FinishPlan& plan, bool brackets,
                    cudaStream_t s) {
-    launch_hist1(ws, g, dtype, d, M, ld, brackets, s);
-    launch_resolve1(ws, dtype, M, plan, brackets, s);
+    launch_hist1(ws, g, dtype, d, M, ld, brackets, nullptr, s);
+    launch_resolve1(ws, dtype, M, plan, brackets, false, nullptr, s);
     if (dtype == MLMC_F32) {
-        launch_sums_candidates(ws, g, d, M, ld, plan, brackets, s);
-        launch_digit_passes(ws, g, d, M, ld, plan, s);
+        launch_sums_candidates(ws, g, d, M, ld, plan, brackets, nullptr, s);
+        launch_digit_passes(ws, g, d, M, ld, plan, false, s);
     }
+}
+
+// The same with brackets from a sample of the rows: one sweep.  The three launches in the middle are for workers whose
+// brackets missed, and return at once for the others.
+void run_sampled_selection(Workspace& ws, const void* g, int64_t d, int M, int64_t ld, const int64_t* k, const FinishPlan& plan,
+                           cudaStream_t s) {
+    launch_bracket_sweep(ws, static_cast<const float*>(g), d, M, ld, k, plan, s);
+    launch_resolve1(ws, MLMC_F32, M, plan, false, true, ws.miss, s);
+    launch_hist1(ws, g, MLMC_F32, d, M, ld, false, ws.miss, s);
+    launch_resolve1(ws, MLMC_F32, M, plan, false, false, ws.miss, s);
+    launch_sums_candidates(ws, g, d, M, ld, plan, false, ws.miss, s);
+    launch_digit_passes(ws, g, d, M, ld, plan, true, s);
 }
 
 FinishPlan finish_plan(int64_t d, int L, int nq, bool adaptive, uint64_t seed, uint64_t step, const mlmc_topk_msgs* out) {
@@ -154,8 +166,12 @@ void select_adaptive(Workspace& ws, const void* g, int dtype, int64_t d, int M, 
         launch_cluster_topk(ws, g, dtype, d, M, ld, pl, nullptr, out, s);
         return;
     }
-    launch_begin_adaptive(ws, dtype, d, M, k, L, s);
-    run_selection(ws, g, dtype, d, M, ld, pl, false, s);
+    if (use_brackets(dtype, d, M, L)) {
+        run_sampled_selection(ws, g, d, M, ld, k, pl, s);
+    } else {
+        launch_begin_adaptive(ws, dtype, d, M, k, L, s);
+        run_selection(ws, g, dtype, d, M, ld, pl, false, s);
+    }
     if (out) launch_emit(ws, g, dtype, d, M, ld, *out, s);
 }
 
@@ -183,7 +199,7 @@ void select_drawn(Workspace& ws, const void* g, int dtype, int64_t d, int M, int
 // The kernels' shared-memory limits and cluster attributes belong to the current CUDA context (a device reset starts a new one),
 // so every create sets them.  What the device can place is asked for once per device: the queries take a millisecond.
 bool configure_kernels(int device, KernelLimits* out) {
-    if (configure_select_kernels() != MLMC_OK || configure_emit_kernels() != MLMC_OK || configure_float_kernels() != MLMC_OK ||
+    if (configure_select_kernels() != MLMC_OK || configure_bracket_kernels() != MLMC_OK || configure_emit_kernels() != MLMC_OK || configure_float_kernels() != MLMC_OK ||
         configure_segment_kernels() != MLMC_OK || configure_sort_kernels() != MLMC_OK || configure_rtn_kernels() != MLMC_OK ||
         configure_cluster_kernels() != MLMC_OK || configure_bit_kernels() != MLMC_OK)
         return false;
@@ -199,6 +215,7 @@ bool configure_kernels(int device, KernelLimits* out) {
     }
     KernelLimits l = {};
     emit_limits(&l);
+    bracket_limits(&l);
     float_limits(&l);
     sort_limits(&l);
     rtn_limits(&l);
@@ -247,6 +264,7 @@ int mlmc_create(mlmc_ctx** out, int device, int64_t d_max, int M_max, int L_max)
     ws.cur_sum_ctas = 0;
     // candidate keys: a quarter of the row (boundary bins normally hold a few percent of it); small rows fit whole
     ws.cand_cap = d_max / 4 > (int64_t(1) << 20) ? d_max / 4 : (d_max < (int64_t(1) << 20) ? d_max : (int64_t(1) << 20));
+    ws.cand_cap = (ws.cand_cap + 3) & ~int64_t(3);  // 16-byte rows
     ws.stat_ctas = ws.sm_count * 4;
     const int64_t emit_tiles = (d_max + kEmitTile - 1) / kEmitTile;
     const int64_t agg_tiles = (d_max + kAggTile - 1) / kAggTile;
@@ -289,6 +307,10 @@ int mlmc_create(mlmc_ctx** out, int device, int64_t d_max, int M_max, int L_max)
     const size_t o_brk = pl.take(sizeof(uint4) * M_max);
     const size_t o_bhit = pl.take(sizeof(int) * M_max);
     const size_t o_bstat = pl.take(sizeof(unsigned long long) * 4);
+    const size_t o_runs = pl.take(sizeof(BracketRuns) * M_max);
+    const size_t o_miss = pl.take(sizeof(int) * M_max);
+    // one block of up to 32 warps per SM, or one per worker where there are more workers than SMs
+    const size_t o_partn = pl.take(sizeof(uint32_t) * 32 * std::max(ws.sm_count, M_max));
     ws.seg_scratch = nullptr;
     ws.seg_bytes = 0;
     ws.sig_d = ws.sig_ld = -1;
@@ -336,6 +358,9 @@ int mlmc_create(mlmc_ctx** out, int device, int64_t d_max, int M_max, int L_max)
     ws.S_partial = reinterpret_cast<unsigned long long*>(base + o_S);
     ws.bit_level = reinterpret_cast<int32_t*>(base + o_blevel);
     ws.rtn_partial = reinterpret_cast<double*>(base + o_rtn);
+    ws.runs = reinterpret_cast<BracketRuns*>(base + o_runs);
+    ws.miss = reinterpret_cast<int*>(base + o_miss);
+    ws.part_n = reinterpret_cast<uint32_t*>(base + o_partn);
     ws.prev_bin = reinterpret_cast<uint32_t*>(base + o_pbin);
     ws.bracket = reinterpret_cast<uint4*>(base + o_brk);
     ws.bracket_hit = reinterpret_cast<int*>(base + o_bhit);
@@ -389,7 +414,8 @@ static const char* const kKernelNames[] = {
     "begin", "uniforms", "hist1", "resolve1", "sums_candidates", "cand_pass2", "cand_pass3", "band_header", "copy_probs", "emit",
     "agg_offsets", "aggregate_topk", "absmax", "bit_stats", "bit_pack", "aggregate_bitwise", "tile_list", "band_count",
     "float_pack", "aggregate_floatbits", "rtn_stats", "rtn_emit", "aggregate_dense", "segment_resolve",
-    "segment_sweep", "segment_buckets", "segment_norms", "segment_draw", "cluster_topk", "cluster_bitwise", "cluster_rtn", "sort_rows"};
+    "segment_sweep", "segment_buckets", "segment_norms", "segment_draw", "cluster_topk", "cluster_bitwise", "cluster_rtn", "sort_rows",
+    "sample", "bracket_sweep", "candidate_hist", "missed_hist1", "missed_sums"};
 static_assert(sizeof(kKernelNames) / sizeof(kKernelNames[0]) == K_COUNT, "a name for every kernel id");
 
 int mlmc_kernel_count(void) { return K_COUNT; }
@@ -600,7 +626,7 @@ int mlmc_compress_stopk(mlmc_ctx* ctx, const void* g, int dtype, int64_t d, int 
         if (int rc = reserve_segments(ws)) return rc;
         set_call_size(ws, d, M, dtype == MLMC_BF16 ? 2 : 4);
         launch_begin_adaptive(ws, dtype, d, M, nullptr, 1, s);
-        launch_hist1(ws, g, dtype, d, M, ld, false, s);
+        launch_hist1(ws, g, dtype, d, M, ld, false, nullptr, s);
         launch_segments(ws, g, dtype, d, M, ld, s_len, L, seed, step, s);
         launch_band_header(ws, M, finish_plan(d, 3, 2, false, seed, step, out), s);
         launch_emit(ws, g, dtype, d, M, ld, *out, s);

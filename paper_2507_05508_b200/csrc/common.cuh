@@ -23,6 +23,7 @@ constexpr int kEmitTile = 4096;               // 32-bit words per emit tile (1 f
 constexpr int kEmitTileVecs = kEmitTile / 4;  // 16-byte vectors per tile, for both element types
 constexpr int kEmitGroups = kEmitTile / (kEmitRows * 32);  // batches of kEmitRows * 32 words per tile: 8
 constexpr int kEmitGroupVecs = kEmitTileVecs / kEmitGroups;  // 16-byte vectors per batch: 128
+constexpr int kBatchKeys = kEmitGroupVecs * 4;  // fp32 entries of a batch
 constexpr int kItemTiles = 4;                 // emit tiles per item of the band count: one batch per lane of a warp
 constexpr int kSuperItems = 32;               // items per super-item, super-items per hyper-item: their counts are added up too
 constexpr int kTileBits = 21;                 // of a listed tile: at most 2^20 tiles per worker (d < 2^32)
@@ -60,7 +61,7 @@ enum KernelId {
     K_BEGIN = 0, K_UNIFORMS, K_HIST1, K_RESOLVE1, K_SUMS_CAND, K_CAND2, K_CAND3, K_BAND_HEADER, K_COPY_PROBS, K_EMIT, K_AGG_OFFSETS,
     K_AGG_TOPK, K_ABSMAX, K_BIT_STATS, K_BIT_PACK, K_AGG_BIT, K_TILE_LIST, K_BAND_COUNT, K_FLOAT_PACK, K_AGG_FLOAT,
     K_RTN_STATS, K_RTN_EMIT, K_AGG_DENSE, K_SEG_RESOLVE, K_SEG_SWEEP, K_SEG_BUCKETS, K_SEG_NORMS, K_SEG_DRAW, K_CLUSTER_TOPK,
-    K_BIT_CLUSTER, K_RTN_CLUSTER, K_SORT_ROWS, K_COUNT
+    K_BIT_CLUSTER, K_RTN_CLUSTER, K_SORT_ROWS, K_SAMPLE, K_BRACKET_SWEEP, K_CAND_HIST, K_MISSED_HIST, K_MISSED_SUMS, K_COUNT
 };
 
 // Level probabilities handed to a kernel by value.
@@ -82,11 +83,20 @@ struct DrawnLevels {
 
 constexpr int kTimingPool = 2048;  // event pairs kept between two reads
 
+// Brackets of a worker's thresholds (topk_bracket.cu): runs of leading-digit bins, from the largest keys down.
+struct BracketRuns {
+    int n;
+    int top[kMaxQueries], low[kMaxQueries];  // highest and lowest bin
+    uint8_t code[kMaxQueries + 1];           // level interval of the keys above run i; [n]: below the last one
+};
+constexpr int64_t kBracketLeast = 1 << 21;  // entries of a row: at least twice as many as the largest sample
+
 // What the device can place.
 struct KernelLimits {
     // clusters of 1, 2, .. 16 blocks that run at a time
     int topk_fit[5];             // of the short-row Top-k kernel
     int dense_fit[5];            // of the short-row dense kernels
+    int sample_fit;              // clusters of 16 blocks of the sample kernel
     // blocks per SM
     int band_count[2];           // fp32, bf16
     int aggregate_topk, aggregate_bitwise, aggregate_float;
@@ -154,6 +164,12 @@ struct Workspace {
     int64_t sig_d, sig_ld;       // host: the problem the stored bins belong to
     int sig_M, sig_L, sig_dtype;
     int64_t sig_k[kMaxLevels];
+    // adaptive Top-k with sampled brackets
+    BracketRuns* runs;           // [M]
+    int* miss;                   // [M] 1: a threshold lies outside its bracket, or the candidates did not fit
+    uint32_t* part_n;            // [M][parts] candidates that every warp of the sweep found
+    int sweep_blocks, parts;     // host: blocks and warps of the sweep per worker,
+    uint32_t part_cap;           //       room of each warp
     // s-Top-k with more levels than kMaxLevels
     int64_t big_cap;             // most levels
     void* seg_scratch;           // buffers of the segment norms (stopk_segments.cu), allocated at first use
@@ -511,7 +527,7 @@ inline bool is_sweep(int id) {
     switch (id) {
         case K_HIST1: case K_SUMS_CAND: case K_BAND_COUNT: case K_EMIT: case K_AGG_TOPK: case K_ABSMAX: case K_BIT_STATS:
         case K_BIT_PACK: case K_AGG_BIT: case K_FLOAT_PACK: case K_AGG_FLOAT: case K_RTN_STATS:
-        case K_RTN_EMIT: case K_AGG_DENSE: case K_SEG_SWEEP:
+        case K_RTN_EMIT: case K_AGG_DENSE: case K_SEG_SWEEP: case K_BRACKET_SWEEP:
             return true;
         default:
             return false;
@@ -588,7 +604,7 @@ struct DrawnBand {
 void launch_begin_adaptive(Workspace& ws, int dtype, int64_t d, int M, const int64_t* k, int L, cudaStream_t s);
 void launch_begin_drawn(Workspace& ws, int dtype, int64_t d, int M, const DrawnBand* bands, int L, bool brackets, cudaStream_t s);
 void launch_uniforms(Workspace& ws, int M, uint64_t seed, uint64_t step, cudaStream_t s);
-void launch_hist1(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, bool brackets, cudaStream_t s);
+void launch_hist1(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, bool brackets, const int* only, cudaStream_t s);
 // What the last kernel of a selection does with its thresholds.
 struct FinishPlan {
     int L;              // levels; queries are the L - 1 boundaries (adaptive) or the two of the drawn band
@@ -603,13 +619,19 @@ struct FinishPlan {
     double* out_p_sel;
     int64_t capacity;
 };
-void launch_resolve1(Workspace& ws, int dtype, int M, const FinishPlan& plan, bool brackets, cudaStream_t s);
+void launch_resolve1(Workspace& ws, int dtype, int M, const FinishPlan& plan, bool brackets, bool sampled, int* miss, cudaStream_t s);
 void launch_sums_candidates(Workspace& ws, const void* g, int64_t d, int M, int64_t ld, const FinishPlan& plan, bool brackets,
-                            cudaStream_t s);
-void launch_digit_passes(Workspace& ws, const void* g, int64_t d, int M, int64_t ld, const FinishPlan& plan, cudaStream_t s);
+                            const int* only, cudaStream_t s);
+void launch_digit_passes(Workspace& ws, const void* g, int64_t d, int M, int64_t ld, const FinishPlan& plan, bool sampled, cudaStream_t s);
 void launch_band_header(Workspace& ws, int M, const FinishPlan& plan, cudaStream_t s);
 void launch_copy_probs(Workspace& ws, int M, int L, const double* p_fixed, double* p_out, double* delta_out,
                        cudaStream_t s);
+// topk_bracket.cu: adaptive Top-k of long fp32 rows, one sweep
+int configure_bracket_kernels();
+void bracket_limits(KernelLimits* limits);
+bool use_brackets(int dtype, int64_t d, int M, int L);
+void launch_bracket_sweep(Workspace& ws, const float* g, int64_t d, int M, int64_t ld, const int64_t* k, const FinishPlan& plan,
+                          cudaStream_t s);
 // topk_emit.cu
 int configure_emit_kernels();
 void emit_limits(KernelLimits* limits);

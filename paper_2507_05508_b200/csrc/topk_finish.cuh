@@ -4,7 +4,28 @@
 #include "common.cuh"
 
 namespace mlmc {
+
+// Memory that a selection accumulates into.
+struct ZeroList {
+    static constexpr int kMost = 8;
+    uint32_t* ptr[kMost];
+    uint32_t words[kMost];
+    int n;
+};
+// For nq queries per worker (topk_select.cu).
+ZeroList selection_state(Workspace& ws, int dtype, int64_t d, int M, int nq, bool sums);
+
 namespace {
+
+__device__ __forceinline__ void clear_all(const ZeroList& z) {
+    for (int a = 0; a < z.n; ++a) {
+        uint32_t* p = z.ptr[a];
+        const uint32_t n4 = z.words[a] / 4;
+        for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += gridDim.x * blockDim.x)
+            reinterpret_cast<uint4*>(p)[i] = make_uint4(0u, 0u, 0u, 0u);
+        for (uint32_t i = n4 * 4 + blockIdx.x * blockDim.x + threadIdx.x; i < z.words[a]; i += gridDim.x * blockDim.x) p[i] = 0u;
+    }
+}
 
 __device__ __forceinline__ Query make_query(uint32_t k, int64_t d) {
     Query q = {};

@@ -1,0 +1,98 @@
+"""Adaptive Top-k of long fp32 rows: brackets from a sample of the row."""
+import numpy as np
+import pytest
+import torch
+
+from test_gpu_parity import padded
+
+pytestmark = pytest.mark.gpu
+
+LEAST = 1 << 28       # entries of the smallest call that is sampled; its rows have at least 2^21
+
+
+@pytest.fixture(scope="module")
+def B():
+    from paper_2507_05508_b200 import binding
+    binding.lib()
+    return binding
+
+
+def sampled_entries(d):
+    """Mask of the entries that a sample by clusters of 1, 2, .. 16 blocks reads: sectors of eight, one per stratum."""
+    mask = np.zeros(d, dtype=bool)
+    sectors = d // 8
+    for blocks in (1, 2, 4, 8, 16):
+        strata = 8192 * blocks
+        i = np.arange(strata, dtype=np.uint64)
+        first, end = i * np.uint64(sectors) // np.uint64(strata), (i + np.uint64(1)) * np.uint64(sectors) // np.uint64(strata)
+        h = (i * np.uint64(0x9E3779B1)) & np.uint64(0xFFFFFFFF)
+        at = first + (h * (end - first) >> np.uint64(32))
+        mask[(at[:, None] * np.uint64(8) + np.arange(8, dtype=np.uint64)).astype(np.int64).ravel()] = True
+    return mask
+
+
+def rows(case, M, d, seed=71):
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    g = padded(torch.randn((M, d), generator=gen, device="cuda"), 4)
+    if case == "layers":
+        g *= torch.repeat_interleave(10.0 ** (torch.rand(40, generator=gen, device="cuda") * 4 - 5), -(-d // 40))[:d]
+    elif case == "ties":
+        g.mul_(2.0).round_()
+    elif case == "zeros":
+        g *= torch.rand(d, generator=gen, device="cuda") < 0.03
+    elif case == "unseen":            # the sample sees nothing but zeros: every bracket misses
+        g[:, torch.from_numpy(sampled_entries(d)).cuda()] = 0.0
+    elif case == "constant":
+        g.fill_(0.25)
+    return g
+
+
+@pytest.mark.parametrize("case", ["layers", "normal", "ties", "zeros", "unseen", "constant"])
+@pytest.mark.parametrize("d,M", [((1 << 21) + 1, 128), ((1 << 25) + 515, 8), ((1 << 27) + 3, 2)])
+def test_adaptive_topk_from_a_sample(B, case, d, M):
+    """Probabilities, levels and bands against a sort of every row on the device.  Its fp64 sums over a whole row round by at
+    most d 2^-53 of the sum, 1.5e-8 for the longest row here; running sums of random order stay far below."""
+    g = rows(case, M, d)
+    ctx = B.mlmc_create(0, d, M, 32)
+    try:
+        for k in ([d // 10_000 << l for l in range(13)] + [d], [d * (i + 1) // 10 for i in range(9)] + [d],
+                  [0, 1, 2, d // 3, d // 3 + 1, d, d]):
+            out = B.TopkBuffers(M, max(b - a for a, b in zip([0] + k[:-1], k)))
+            p = torch.zeros((M, len(k)), dtype=torch.float64, device="cuda")
+            delta = torch.zeros_like(p)
+            B.mlmc_level_probs(ctx, g, B.MLMC_TOPK, k, None, p, delta)
+            B.mlmc_compress_topk(ctx, g, k, None, 5, 1, out)
+            assert B.mlmc_get_status(ctx) == B.MLMC_OK
+            u = B.mlmc_read_u(ctx, 5, 1, M)
+            for m in sorted({0, 1, M // 2, M - 1}):
+                order = torch.sort(g[m].abs(), descending=True, stable=True).indices
+                sq = torch.cat([torch.zeros(1, dtype=torch.float64, device="cuda"), g[m].double()[order].square()])
+                norms = torch.stack([sq[a + 1:b + 1].sum() for a, b in zip([0] + k[:-1], k)]).sqrt()
+                assert torch.allclose(delta[m], norms, rtol=1e-9, atol=0.0)
+                want = norms / norms.sum() if norms.sum() > 0 else torch.eye(len(k), dtype=torch.float64, device="cuda")[0]
+                assert torch.allclose(p[m], want, rtol=1e-9, atol=1e-15)
+                level = int(out.level[m])
+                cdf = torch.cumsum(p[m], 0).tolist()
+                assert p[m, level] > 0 and (level == 0 or u[m] >= cdf[level - 1] - 1e-9) and u[m] < cdf[level] + 1e-9
+                band = torch.sort(order[(k[level - 1] if level else 0):k[level]]).values
+                n = int(out.count[m])
+                assert n == band.numel() and torch.equal(out.idx[m, :n].long() & 0xFFFFFFFF, band)
+                value = g[m][band].double() / float(out.p_sel[m])
+                assert torch.allclose(out.val[m, :n].double(), value, rtol=1e-6, atol=0.0)
+    finally:
+        B.mlmc_destroy(ctx)
+
+
+def test_sampled_rows_report_non_finite_entries(B):
+    d = (1 << 27) + 5
+    g = rows("normal", 2, d)
+    g[1, d - 1] = float("nan")
+    k = [d // 100, d // 10, d]
+    out = B.TopkBuffers(2, d)
+    ctx = B.mlmc_create(0, d, 2, 32)
+    try:
+        B.mlmc_compress_topk(ctx, g, k, None, 0, 0, out)
+        assert B.mlmc_get_status(ctx) == B.MLMC_ERR_NONFINITE
+        assert out.level[1] == -1 and out.count[1] == 0 and out.level[0] >= 0
+    finally:
+        B.mlmc_destroy(ctx)
