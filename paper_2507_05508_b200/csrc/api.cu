@@ -514,11 +514,11 @@ int mlmc_level_probs(mlmc_ctx* ctx, const void* g, int dtype, int64_t d, int M, 
             select_adaptive(ws, g, dtype, d, M, ld, sched, L, 0, 0, nullptr, s);
         } else if (kind == MLMC_BITWISE) {
             const DrawPlan plan = bit_draw_plan(ws, b32, L, 0, 0, nullptr);
-            launch_absmax(ws, g, dtype, d, M, ld, plan, nullptr, s);
+            launch_absmax(ws, g, dtype, d, M, ld, plan, nullptr, nullptr, s);
             launch_bit_stats(ws, g, dtype, d, M, ld, b32, L, plan, s);
         } else {
             const DrawPlan plan = rtn_draw_plan(ws, L, 0, 0, nullptr);
-            launch_absmax(ws, g, dtype, d, M, ld, plan, nullptr, s);
+            launch_absmax(ws, g, dtype, d, M, ld, plan, nullptr, nullptr, s);
             launch_rtn_stats(ws, g, dtype, d, M, ld, b32, L, plan, s);
         }
     }
@@ -575,7 +575,7 @@ int mlmc_compress_bitwise(mlmc_ctx* ctx, const void* g, int dtype, int64_t d, in
     set_call_size(ws, d, M, dtype == MLMC_BF16 ? 2 : 4);
     const DrawPlan plan = bit_draw_plan(ws, b32, L, seed, step, out);
     if (launch_bit_cluster(ws, g, dtype, d, M, ld, b32, L, plan, p ? pn : nullptr, *out, s)) return finish(cudaGetLastError());
-    launch_absmax(ws, g, dtype, d, M, ld, plan, p ? pn : nullptr, s);
+    launch_absmax(ws, g, dtype, d, M, ld, plan, p ? pn : nullptr, zero_batches(ws) ? out : nullptr, s);
     if (!p) launch_bit_stats(ws, g, dtype, d, M, ld, b32, L, plan, s);
     launch_bit_pack(ws, g, dtype, d, M, ld, b32, L, *out, s);
     return finish(cudaGetLastError());
@@ -717,7 +717,7 @@ int mlmc_compress_rtn(mlmc_ctx* ctx, const void* g, int dtype, int64_t d, int M,
     set_call_size(ws, d, M, dtype == MLMC_BF16 ? 2 : 4);
     const DrawPlan plan = rtn_draw_plan(ws, L, seed, step, out);
     if (launch_rtn_cluster(ws, g, dtype, d, M, ld, r32, L, plan, p ? pn : nullptr, *out, s)) return finish(cudaGetLastError());
-    launch_absmax(ws, g, dtype, d, M, ld, plan, p ? pn : nullptr, s);  // c = max |g|, and the NaN / Inf check
+    launch_absmax(ws, g, dtype, d, M, ld, plan, p ? pn : nullptr, nullptr, s);  // c = max |g|, and the NaN / Inf check
     if (!p) launch_rtn_stats(ws, g, dtype, d, M, ld, r32, L, plan, s);
     launch_rtn_emit(ws, g, dtype, d, M, ld, r32, L, *out, s);
     return finish(cudaGetLastError());

@@ -75,41 +75,115 @@ __device__ __forceinline__ int zero_code_below(float gmax, int b) {
     return gmax > 0.0f ? __float_as_int(gmax * ldexpf(1.0f - 0x1.0p-20f, -b)) : 0x7FFFFFFF;
 }
 
+// The sign words of a batch (four vectors per lane): from the nibble (bf16: byte) of signs of every vector, in the word's order.
+// Lanes that hold pieces of one word hold pieces of the words of all four vectors; they exchange them so that every lane
+// is left with one word (fp32: every second quartet of lanes holds a copy).
+template <typename T>
+__device__ __forceinline__ void write_signs(const uint4 (&q)[4], uint32_t* __restrict__ out) {
+    const int lane = threadIdx.x & 31;
+    uint32_t x[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        uint32_t s = 0;
+        if constexpr (sizeof(T) == 4) {
+            s = __funnelshift_l(q[j].w, s, 1);
+            s = __funnelshift_l(q[j].z, s, 1);
+            s = __funnelshift_l(q[j].y, s, 1);
+            s = __funnelshift_l(q[j].x, s, 1);
+            x[j] = s << (4 * (lane & 7));
+        } else {
+            auto two = [](uint32_t w) { return ((w >> 15) & 1u) | ((w >> 30) & 2u); };
+            s = two(q[j].x) | two(q[j].y) << 2 | two(q[j].z) << 4 | two(q[j].w) << 6;
+            x[j] = s << (8 * (lane & 3));
+        }
+    }
+    const bool odd = lane & 1, high = lane & 2;
+    uint32_t a = odd ? x[1] : x[0], b = odd ? x[3] : x[2];
+    a |= __shfl_xor_sync(0xFFFFFFFFu, odd ? x[0] : x[1], 1);
+    b |= __shfl_xor_sync(0xFFFFFFFFu, odd ? x[2] : x[3], 1);
+    uint32_t w = high ? b : a;
+    w |= __shfl_xor_sync(0xFFFFFFFFu, high ? a : b, 2);
+    const int j = lane & 3;  // of vector j
+    if constexpr (sizeof(T) == 4) {
+        w |= __shfl_xor_sync(0xFFFFFFFFu, w, 4);
+        if (!(lane & 4)) out[4 * j + (lane >> 3)] = w;
+    } else {
+        out[8 * j + (lane >> 2)] = w;
+    }
+}
+
 // ---- per-worker max |g| as an integer max over magnitude keys; flags NaN / Inf.  With given probabilities (draw != 0)
 // the worker's last block also draws the level and writes the message header.
-template <typename T>
+// KEEP 1: the largest key of every batch (kEmitGroupVecs vectors, a warp's share of a trip) is kept, and the kernels that write
+// the message do not read the batches that round to 0 at the drawn level.  KEEP 2: what they would miss of those, the sign plane
+// of a bit-plane message, is written here too.  8 x 124M fp32 entries: 560, 566 and 620 us; what it saves the message kernels is
+// beside them.  KEEP 0, for calls that L2 holds (8 x 1M entries, bit planes: 32.2 us per step, with 2 33.4).
+template <typename T, int KEEP>
 __global__ void __launch_bounds__(kSweepThreads, 3)
 absmax_kernel(const T* __restrict__ g, int64_t d, int64_t ld, uint32_t* gmax_bits, uint32_t* acc, uint32_t* done,
+              uint32_t* __restrict__ batch_max, int batches_per_worker, uint32_t* __restrict__ planes, int64_t plane_row,
               const __grid_constant__ DrawPlan pl, const __grid_constant__ DrawnLevels drawn, int draw, int* status, int* worker_err) {
     using Tr = ElemTraits<T>;
     __shared__ uint32_t sh_max[kSweepThreads / 32];
     pdl_enter();
-    const int m = blockIdx.y;
+    const int m = blockIdx.y, lane = threadIdx.x & 31;
     const T* row = g + (int64_t)m * ld;
     uint32_t mx = 0;
-    // Chunks of kBatch vectors per thread, all in flight before any is used, dealt round-robin to the blocks of the worker.
-    // (One contiguous range per block ran between 0.75 and 1.0 of the copy rate, depending on the row length.)
-    constexpr int kBatch = 4;
     const int64_t nvec = (d + Tr::kVec - 1) / Tr::kVec, full_end = d / Tr::kVec;  // vectors of the row, and those wholly inside it
-    for (int64_t base = (int64_t)blockIdx.x * kBatch * kSweepThreads; base < nvec; base += (int64_t)gridDim.x * kBatch * kSweepThreads) {
-        const int64_t v = base + threadIdx.x;
-        if (base + kBatch * kSweepThreads > full_end) {  // the row's last chunk
-            for (int64_t u = v; u < nvec; u += kSweepThreads)
-                for_each_in_vector<T>(row, u, d, [&](int64_t, uint32_t bits) { mx = max(mx, Tr::key(bits)); });
-            break;
-        }
-        uint4 q[kBatch];
-#pragma unroll
-        for (int j = 0; j < kBatch; ++j) q[j] = __ldg(reinterpret_cast<const uint4*>(row) + v + j * kSweepThreads);
-#pragma unroll
-        for (int j = 0; j < kBatch; ++j) {
-            if constexpr (Tr::kVec == 4) {
-                mx = max(max(mx, q[j].x & 0x7FFFFFFFu), max(q[j].y & 0x7FFFFFFFu, max(q[j].z & 0x7FFFFFFFu, q[j].w & 0x7FFFFFFFu)));
-            } else {
-                const uint32_t a = __vmaxu2(__vmaxu2(q[j].x & 0x7FFF7FFFu, q[j].y & 0x7FFF7FFFu),
-                                            __vmaxu2(q[j].z & 0x7FFF7FFFu, q[j].w & 0x7FFF7FFFu));
-                mx = max(mx, max(a & 0xFFFFu, a >> 16));
+    if constexpr (KEEP == 0) {
+        // Chunks of kBatch vectors per thread, all in flight before any is used, dealt round-robin to the blocks of the worker.
+        // (One contiguous range per block ran between 0.75 and 1.0 of the copy rate, depending on the row length.)
+        constexpr int kBatch = 4;
+        for (int64_t base = (int64_t)blockIdx.x * kBatch * kSweepThreads; base < nvec; base += (int64_t)gridDim.x * kBatch * kSweepThreads) {
+            const int64_t v = base + threadIdx.x;
+            if (base + kBatch * kSweepThreads > full_end) {  // the row's last chunk
+                for (int64_t u = v; u < nvec; u += kSweepThreads)
+                    for_each_in_vector<T>(row, u, d, [&](int64_t, uint32_t bits) { mx = max(mx, Tr::key(bits)); });
+                break;
             }
+            uint4 q[kBatch];
+#pragma unroll
+            for (int j = 0; j < kBatch; ++j) q[j] = __ldg(reinterpret_cast<const uint4*>(row) + v + j * kSweepThreads);
+#pragma unroll
+            for (int j = 0; j < kBatch; ++j) {
+                if constexpr (Tr::kVec == 4) {
+                    mx = max(max(mx, q[j].x & 0x7FFFFFFFu), max(q[j].y & 0x7FFFFFFFu, max(q[j].z & 0x7FFFFFFFu, q[j].w & 0x7FFFFFFFu)));
+                } else {
+                    const uint32_t a = __vmaxu2(__vmaxu2(q[j].x & 0x7FFF7FFFu, q[j].y & 0x7FFF7FFFu),
+                                                __vmaxu2(q[j].z & 0x7FFF7FFFu, q[j].w & 0x7FFF7FFFu));
+                    mx = max(mx, max(a & 0xFFFFu, a >> 16));
+                }
+            }
+        }
+    } else {
+        // A batch per warp and trip, all four vectors in flight before any is used, dealt round-robin to the blocks of the worker.
+        uint32_t* bmax = batch_max + (int64_t)m * batches_per_worker;
+        const int64_t nbatch = (nvec + kEmitGroupVecs - 1) / kEmitGroupVecs, stride = (int64_t)gridDim.x * (kSweepThreads / 32);
+        for (int64_t b = (int64_t)blockIdx.x * (kSweepThreads / 32) + (threadIdx.x >> 5); b < nbatch; b += stride) {
+            const int64_t v = b * kEmitGroupVecs + lane;
+            uint32_t vm = 0;
+            if ((b + 1) * kEmitGroupVecs > full_end) {  // the row's last batch; its signs are left to the message kernel
+                for (int64_t u = v; u < nvec; u += 32)
+                    for_each_in_vector<T>(row, u, d, [&](int64_t, uint32_t bits) { vm = max(vm, Tr::key(bits)); });
+            } else {
+                uint4 q[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) q[j] = __ldg(reinterpret_cast<const uint4*>(row) + v + j * 32);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if constexpr (Tr::kVec == 4) {
+                        vm = max(max(vm, q[j].x & 0x7FFFFFFFu), max(q[j].y & 0x7FFFFFFFu, max(q[j].z & 0x7FFFFFFFu, q[j].w & 0x7FFFFFFFu)));
+                    } else {
+                        const uint32_t a = __vmaxu2(__vmaxu2(q[j].x & 0x7FFF7FFFu, q[j].y & 0x7FFF7FFFu),
+                                                    __vmaxu2(q[j].z & 0x7FFF7FFFu, q[j].w & 0x7FFF7FFFu));
+                        vm = max(vm, max(a & 0xFFFFu, a >> 16));
+                    }
+                }
+                if (KEEP == 2) write_signs<T>(q, planes + (int64_t)m * plane_row + b * (kEmitGroupVecs * Tr::kVec / 32));
+            }
+            vm = __reduce_max_sync(0xFFFFFFFFu, vm);
+            if (lane == 0) bmax[b] = Tr::kVec == 8 ? vm << 16 : vm;  // as the bits of an fp32 magnitude
+            mx = max(mx, vm);
         }
     }
 #pragma unroll
@@ -312,11 +386,12 @@ bit_stats_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t*
 // word per plane).  The entries come through a ring of two shared-memory slots per warp: the next group's copy is in
 // flight while the current group is coded.  A plane's word is collected by one shift and one funnel shift per entry, from
 // 6 planes on by one bit transpose for all of them.  A group whose largest entry has the code 0 at the drawn level's bits is
-// not coded: its magnitude planes are zero.
+// not coded: its magnitude planes are zero.  The groups of which the sweep before knows that are not even read (8 x 124M fp32
+// entries with layers: 782 -> 424 us).
 // Bound by HBM.  Rows of 32 entries across the lanes with a ballot each took 1.04 ms for 8 x 124M fp32 entries.
 template <typename T>
 __device__ __forceinline__ void pack_group(const uint32_t* slot, const Quantiser& qz, float scale, int zero_below, int w, int64_t word,
-                                           int64_t words, uint32_t* __restrict__ out) {
+                                           int64_t words, uint32_t* __restrict__ out, bool signs = true) {
     const int lane = threadIdx.x & 31;
     const bool live = word < words;
     float x[32];
@@ -341,7 +416,7 @@ __device__ __forceinline__ void pack_group(const uint32_t* slot, const Quantiser
         sign_w = __funnelshift_l(__float_as_uint(x[t]), sign_w, 1);
         mx = fmaxf(mx, fabsf(x[t]));
     }
-    if (live) out[word] = sign_w;
+    if (live && signs) out[word] = sign_w;
     if (!__any_sync(0xFFFFFFFFu, __float_as_int(mx) >= zero_below)) {
         if (live)
             for (int j = 1; j <= w; ++j) out[(int64_t)j * words + word] = 0u;
@@ -365,10 +440,11 @@ __device__ __forceinline__ void pack_group(const uint32_t* slot, const Quantiser
     }
 }
 
-template <typename T>
+template <typename T, bool SKIP>
 __global__ void __launch_bounds__(kBitThreads, 3)
 bit_pack_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* gmax_bits, BitSchedule sc,
-                const int32_t* bit_level, uint32_t* __restrict__ planes, int w_max, int64_t words) {
+                const int32_t* bit_level, const uint32_t* batch_max, int batches_per_worker, uint32_t* __restrict__ planes, int w_max,
+                int64_t words) {
     extern __shared__ __align__(16) uint32_t sh_ring[];  // [warps][2][kGroupSlot]
     pdl_enter();
     const int m = blockIdx.y;
@@ -385,14 +461,54 @@ bit_pack_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* 
     uint32_t* out = planes + (int64_t)m * (1 + w_max) * words;
     uint32_t* ring = sh_ring + warp * 2 * kGroupSlot<T>;
     const int64_t stride = (int64_t)gridDim.x * (blockDim.x / 32);
-    int64_t grp = (int64_t)blockIdx.x * (blockDim.x / 32) + warp;
-    fetch_group<T>(row, d, grp, ngroups, ring);
-    for (int it = 0; grp < ngroups; grp += stride, ++it) {
-        fetch_group<T>(row, d, grp + stride, ngroups, ring + ((it + 1) & 1) * kGroupSlot<T>);
-        cp_async_wait<1>();  // this group has landed (the next one may still be in flight)
-        __syncwarp();
-        pack_group<T>(ring + (it & 1) * kGroupSlot<T>, qz, scale, zero_below, w, grp * 32 + lane, words, out);
-        __syncwarp();  // everyone is done with this slot before the copy after next lands in it
+    if constexpr (!SKIP) {
+        int64_t grp = (int64_t)blockIdx.x * (blockDim.x / 32) + warp;
+        fetch_group<T>(row, d, grp, ngroups, ring);
+        for (int it = 0; grp < ngroups; grp += stride, ++it) {
+            fetch_group<T>(row, d, grp + stride, ngroups, ring + ((it + 1) & 1) * kGroupSlot<T>);
+            cp_async_wait<1>();  // this group has landed (the next one may still be in flight)
+            __syncwarp();
+            pack_group<T>(ring + (it & 1) * kGroupSlot<T>, qz, scale, zero_below, w, grp * 32 + lane, words, out);
+            __syncwarp();  // everyone is done with this slot before the copy after next lands in it
+        }
+    } else {
+        constexpr int kPer = 2 * (int)sizeof(T) / 4;  // batches of a group: 2 or 1
+        const uint32_t* bmax = batch_max + (int64_t)m * batches_per_worker;
+        // A lane looks at the largest key of one of the warp's next 32 groups.
+        for (int64_t base = (int64_t)blockIdx.x * (blockDim.x / 32) + warp; base < ngroups; base += 32 * stride) {
+            const int64_t own = base + lane * stride;
+            bool coded = false;
+            if (own < ngroups) {
+                coded = (own + 1) * 1024 > d;  // the ragged end: its signs are not written yet
+                if (!coded) {
+                    uint32_t mx = bmax[own * kPer];
+                    if (kPer == 2) mx = max(mx, bmax[own * kPer + 1]);
+                    coded = (int)mx >= zero_below;
+                }
+            }
+            uint32_t todo = __ballot_sync(0xFFFFFFFFu, coded), zero = __ballot_sync(0xFFFFFFFFu, own < ngroups && !coded);
+            auto next = [&]() -> int64_t {
+                if (!todo) return ngroups;
+                const int64_t grp = base + (__ffs(todo) - 1) * stride;
+                todo &= todo - 1u;
+                return grp;
+            };
+            int64_t grp = next();
+            fetch_group<T>(row, d, grp, ngroups, ring);
+            for (; zero; zero &= zero - 1u) {  // magnitude planes of zeros, while the first group is on its way
+                uint32_t* to = out + (base + (__ffs(zero) - 1) * stride) * 32 + lane;
+                for (int j = 1; j <= w; ++j) to[(int64_t)j * words] = 0u;
+            }
+            for (int it = 0; grp < ngroups; ++it) {
+                const int64_t after = next();
+                fetch_group<T>(row, d, after, ngroups, ring + ((it + 1) & 1) * kGroupSlot<T>);
+                cp_async_wait<1>();  // this group has landed (the next one may still be in flight)
+                __syncwarp();
+                pack_group<T>(ring + (it & 1) * kGroupSlot<T>, qz, scale, zero_below, w, grp * 32 + lane, words, out, (grp + 1) * 1024 > d);
+                __syncwarp();  // everyone is done with this slot before the copy after next lands in it
+                grp = after;
+            }
+        }
     }
     cp_async_wait<0>();
 }
@@ -588,7 +704,9 @@ int configure_bit_kernels() {
     const bool ok = cudaFuncSetAttribute(aggregate_bitwise_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)kAvgBitSmem + kEmitMaxWorkers * 8) == cudaSuccess &&
                     configure_dense_cluster(bit_cluster_kernel<float>) && configure_dense_cluster(bit_cluster_kernel<bf16_t>) &&
-                    cudaFuncSetAttribute(bit_pack_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                    cudaFuncSetAttribute(bit_pack_kernel<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)bit_pack_smem(4, kBitThreads / 32)) == cudaSuccess &&
+                    cudaFuncSetAttribute(bit_pack_kernel<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)bit_pack_smem(4, kBitThreads / 32)) == cudaSuccess;
     return ok ? MLMC_OK : MLMC_ERR_CUDA;
 }
@@ -617,15 +735,20 @@ DrawPlan bit_draw_plan(Workspace& ws, const int32_t* b, int L, uint64_t seed, ui
 }
 
 void launch_absmax(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const DrawPlan& plan, const double* p,
-                   cudaStream_t s) {
+                   const mlmc_bit_msgs* signs, cudaStream_t s) {
     const DrawnLevels drawn = draw_levels(p, plan.L, plan.seed, plan.step, M);
     const int nb = bit_blocks(ws, d, dtype == MLMC_BF16 ? 8 : 4, M, 8);
+    uint32_t* planes = signs ? signs->planes : nullptr;
+    const int64_t plane_row = signs ? (1 + (int64_t)signs->w_max) * ((d + 31) / 32) : 0;
     auto go = [&](auto kernel, auto* row) {
-        launch_kernel(ws, K_ABSMAX, kernel, dim3(nb, M), kSweepThreads, 0, s, row, d, ld, ws.gmax_bits, ws.acc_word, ws.done,
-                      plan, drawn, p ? 1 : 0, ws.status, ws.worker_err);
+        launch_kernel(ws, K_ABSMAX, kernel, dim3(nb, M), kSweepThreads, 0, s, row, d, ld, ws.gmax_bits, ws.acc_word, ws.done, ws.tile_max,
+                      emit_tiles_per_worker(d, dtype) * kEmitGroups, planes, plane_row, plan, drawn, p ? 1 : 0, ws.status, ws.worker_err);
     };
-    if (dtype == MLMC_BF16) go(absmax_kernel<bf16_t>, static_cast<const bf16_t*>(g));
-    else go(absmax_kernel<float>, static_cast<const float*>(g));
+    const int keep = !zero_batches(ws) ? 0 : signs ? 2 : 1;
+    if (dtype == MLMC_BF16)
+        go(keep == 2 ? absmax_kernel<bf16_t, 2> : keep ? absmax_kernel<bf16_t, 1> : absmax_kernel<bf16_t, 0>, static_cast<const bf16_t*>(g));
+    else
+        go(keep == 2 ? absmax_kernel<float, 2> : keep ? absmax_kernel<float, 1> : absmax_kernel<float, 0>, static_cast<const float*>(g));
 }
 
 template <typename T, typename Acc>
@@ -687,8 +810,9 @@ static void launch_bit_pack_t(Workspace& ws, const T* g, int64_t d, int M, int64
     int64_t nb = ((int64_t)ws.sm_count * 3) / M;  // persistent: three resident blocks per SM, rounded down
     if (nb > by_work) nb = by_work;
     if (nb < 1) nb = 1;
-    launch_kernel(ws, K_BIT_PACK, bit_pack_kernel<T>, dim3((unsigned)nb, M), warps * 32, bit_pack_smem(sizeof(T), warps), s, g, d, ld,
-                  ws.gmax_bits, sc, ws.bit_level, out.planes, out.w_max, words);
+    launch_kernel(ws, K_BIT_PACK, zero_batches(ws) ? bit_pack_kernel<T, true> : bit_pack_kernel<T, false>, dim3((unsigned)nb, M), warps * 32, bit_pack_smem(sizeof(T), warps), s, g, d, ld,
+                  ws.gmax_bits, sc, ws.bit_level, zero_batches(ws), emit_tiles_per_worker(d, sizeof(T) == 2 ? MLMC_BF16 : MLMC_F32) * kEmitGroups,
+                  out.planes, out.w_max, words);
 }
 
 void launch_bit_pack(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* b, int L,

@@ -145,7 +145,8 @@ struct Workspace {
     uint2* tile_list;            // the tiles of all workers that can hold band entries, in any order: {worker << kTileBits | tile, batch mask}
     uint32_t* list_n;            // how many
     int64_t max_tiles;
-    uint32_t* tile_max;          // [M][tiles per worker][kEmitGroups] largest magnitude key of every batch of every emit tile (sweep 1)
+    // [M][tiles per worker][kEmitGroups] largest magnitude key of every batch of every emit tile (first sweep of a message)
+    uint32_t* tile_max;
     uint32_t* group_n;           // [M] how many batches the last emission had to read
     int64_t last_emit_tiles;     // tiles per row of the last emission (host side, for mlmc_read_listed_tiles)
     uint32_t* cand_floor;        // [M] smallest key that can be a candidate of sweep 2 (lower edge of the lowest boundary bin)
@@ -641,9 +642,13 @@ void launch_aggregate_topk(Workspace& ws, const mlmc_topk_msgs& msgs, int M, int
 // bitwise.cu
 int configure_bit_kernels();
 void bit_limits(KernelLimits* limits);
-// Largest magnitude of every worker and the NaN / Inf check; with `p` (given probabilities) also the draw and the header.
+// Largest keys of the batches where the message kernels skip the batches that round to 0: in long sweeps.  Shorter calls lie in L2,
+// and to look first costs more than to read (8 x 1M entries, bit planes: 32.2 us per step, 33.4 with the look).
+inline const uint32_t* zero_batches(const Workspace& ws) { return ws.long_sweeps ? ws.tile_max : nullptr; }
+// Largest magnitude of every worker, in long sweeps of its batches too, and the NaN / Inf check; with `p` (given probabilities) also
+// the draw and the header; with `signs` (a bit-plane message, long sweeps) its sign planes, but for the ragged end of a row.
 void launch_absmax(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const DrawPlan& plan, const double* p,
-                   cudaStream_t s);
+                   const mlmc_bit_msgs* signs, cudaStream_t s);
 DrawPlan bit_draw_plan(Workspace& ws, const int32_t* b, int L, uint64_t seed, uint64_t step, const mlmc_bit_msgs* out);
 // Adaptive: field energies of every level, probabilities, draw and header.
 void launch_bit_stats(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* b, int L,

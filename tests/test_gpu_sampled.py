@@ -1,9 +1,10 @@
-"""Adaptive Top-k of long fp32 rows: brackets from a sample of the row."""
+"""Adaptive Top-k of long fp32 rows: brackets from a sample of the row, and messages that skip batches which round to 0."""
 import numpy as np
 import pytest
 import torch
 
-from test_gpu_parity import padded
+from test_gpu_ext import check_rtn
+from test_gpu_parity import check_bitwise, padded, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -94,5 +95,31 @@ def test_sampled_rows_report_non_finite_entries(B):
         B.mlmc_compress_topk(ctx, g, k, None, 0, 0, out)
         assert B.mlmc_get_status(ctx) == B.MLMC_ERR_NONFINITE
         assert out.level[1] == -1 and out.count[1] == 0 and out.level[0] >= 0
+    finally:
+        B.mlmc_destroy(ctx)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("d", [1_700_000, 1_700_353, 1_700_864 + 1])
+def test_batches_that_round_to_zero_are_not_read(B, ora, dtype, d):
+    """Calls above 100 MB; few entries far above the others, so that most batches round to 0 at the coarse levels and none at the
+    fine ones; random signs, so that a missed sign plane shows."""
+    M = 32 if dtype == "bf16" else 16
+    rng = np.random.default_rng(72)
+    g_np = (rng.standard_normal((M, d)) * 1e-3).astype(np.float32)
+    for m in range(M):
+        g_np[m, rng.integers(0, d, 50)] *= 200.0
+    g_np[0, d // 2], g_np[1, -1], g_np[2, 0] = 1.0, -1.0, 1.0
+    g_np[3] *= 1e-30
+    g = to_dev(g_np)
+    if dtype == "bf16":
+        g = padded(g.to(torch.bfloat16), 8)
+    ctx = B.mlmc_create(0, d, M, 32)
+    try:
+        for step in range(2):         # levels drawn worker by worker
+            check_bitwise(B, ora, ctx, g, [1, 2, 4, 8, 16, 23], [1 / 6] * 6, 1, step)
+            check_rtn(B, ora, ctx, g, [2, 4, 8, 16], [0.2] * 5, 1, step)
+        check_bitwise(B, ora, ctx, g, [1, 2, 4, 8, 16, 23], None, 1, 0)
+        check_rtn(B, ora, ctx, g, [2, 4, 8, 16], None, 1, 0, expect_excluded=2)
     finally:
         B.mlmc_destroy(ctx)
