@@ -202,8 +202,8 @@ sample_kernel(ZeroList z, SampleRanks ranks, Query* queries, const float* __rest
 // the keys of runs go to the warp's own part of the candidate list.  All of this is in a fixed order: the sums, here and over
 // the list, do not change from call to call.  Counts are exact integers, energies fp64 sums.
 //
-// Bound by issue (3.2 instructions per clock and SM, 26 per warp and key) with the integer pipe (59 %) and shared memory (55 %)
-// behind it; the comparisons load the one, the look-ups the other.  8 x 124M entries, 15 levels: 950 us, where the histogram sweep
+// Bound by issue (2.9 instructions per clock and SM, 25 per warp and key) with shared memory (62 %) and the integer pipe (57 %)
+// behind it; the look-ups load the one, the comparisons the other.  8 x 124M entries, 15 levels: 950 us, where the histogram sweep
 // and the sweep for energies and candidates took 605 + 996.  On the way there: three intervals compared wherever a quarter of the
 // keys or less lies above them 973 us, two intervals or look-ups only 961; 21 warps instead of 24 (one scheduler has
 // six and the others five) 1053; the warps of a block in step, so that all look up or all compare, 1044.
