@@ -782,10 +782,13 @@ digit_pass_kernel(const float* __restrict__ g, int64_t d, int64_t ld, uint32_t* 
                     kept += __popc(kept_mask);
                 };
                 uint32_t i = 0;
-                for (; i + 512u <= np; i += 512u) {  // no write reaches keys that have not been read: kept <= i
+                // The keys are kept in place: kept <= i where a trip starts, but its writes reach up to its own last key.  Every lane
+                // has its keys of a trip before the first write.
+                for (; i + 512u <= np; i += 512u) {
                     uint4 q[4];
 #pragma unroll
                     for (int j = 0; j < 4; ++j) q[j] = reinterpret_cast<const uint4*>(cand + i)[j * 32 + lane];
+                    __syncwarp();
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
                         one(q[j].x, true);
@@ -794,7 +797,11 @@ digit_pass_kernel(const float* __restrict__ g, int64_t d, int64_t ld, uint32_t* 
                         one(q[j].w, true);
                     }
                 }
-                for (; i < np; i += 32u) one(i + lane < np ? cand[i + lane] : 0u, i + lane < np);
+                for (; i < np; i += 32u) {
+                    const uint32_t key = i + lane < np ? cand[i + lane] : 0u;
+                    __syncwarp();
+                    one(key, i + lane < np);
+                }
                 __syncwarp();
                 for (uint32_t k = lane; k < kept; k += 32u) take(cand[k], code_of[cand[k] >> 16]);
                 if (lane == 0) parts.count[(int64_t)m * parts.n + p] = kept;

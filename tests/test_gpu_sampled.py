@@ -48,6 +48,33 @@ def rows(case, M, d, seed=71):
     return g
 
 
+def check_adaptive(B, ctx, g, k):
+    """Norms, probabilities, levels and bands of some workers against a stable sort of their rows on the device."""
+    M = g.shape[0]
+    out = B.TopkBuffers(M, max(b - a for a, b in zip([0] + k[:-1], k)))
+    p = torch.zeros((M, len(k)), dtype=torch.float64, device="cuda")
+    delta = torch.zeros_like(p)
+    B.mlmc_level_probs(ctx, g, B.MLMC_TOPK, k, None, p, delta)
+    B.mlmc_compress_topk(ctx, g, k, None, 5, 1, out)
+    assert B.mlmc_get_status(ctx) == B.MLMC_OK
+    u = B.mlmc_read_u(ctx, 5, 1, M)
+    for m in sorted({0, 1, M // 2, M - 1}):
+        order = torch.sort(g[m].abs(), descending=True, stable=True).indices
+        sq = torch.cat([torch.zeros(1, dtype=torch.float64, device="cuda"), g[m].double()[order].square()])
+        norms = torch.stack([sq[a + 1:b + 1].sum() for a, b in zip([0] + k[:-1], k)]).sqrt()
+        assert torch.allclose(delta[m], norms, rtol=1e-9, atol=0.0)
+        want = norms / norms.sum() if norms.sum() > 0 else torch.eye(len(k), dtype=torch.float64, device="cuda")[0]
+        assert torch.allclose(p[m], want, rtol=1e-9, atol=1e-15)
+        level = int(out.level[m])
+        cdf = torch.cumsum(p[m], 0).tolist()
+        assert p[m, level] > 0 and (level == 0 or u[m] >= cdf[level - 1] - 1e-9) and u[m] < cdf[level] + 1e-9
+        band = torch.sort(order[(k[level - 1] if level else 0):k[level]]).values
+        n = int(out.count[m])
+        assert n == band.numel() and torch.equal(out.idx[m, :n].long() & 0xFFFFFFFF, band)
+        value = g[m][band].double() / float(out.p_sel[m])
+        assert torch.allclose(out.val[m, :n].double(), value, rtol=1e-6, atol=0.0)
+
+
 @pytest.mark.parametrize("case", ["layers", "normal", "ties", "zeros", "unseen", "constant"])
 @pytest.mark.parametrize("d,M", [((1 << 21) + 1, 128), ((1 << 25) + 515, 8), ((1 << 27) + 3, 2)])
 def test_adaptive_topk_from_a_sample(B, case, d, M):
@@ -58,28 +85,29 @@ def test_adaptive_topk_from_a_sample(B, case, d, M):
     try:
         for k in ([d // 10_000 << l for l in range(13)] + [d], [d * (i + 1) // 10 for i in range(9)] + [d],
                   [0, 1, 2, d // 3, d // 3 + 1, d, d]):
-            out = B.TopkBuffers(M, max(b - a for a, b in zip([0] + k[:-1], k)))
-            p = torch.zeros((M, len(k)), dtype=torch.float64, device="cuda")
-            delta = torch.zeros_like(p)
-            B.mlmc_level_probs(ctx, g, B.MLMC_TOPK, k, None, p, delta)
-            B.mlmc_compress_topk(ctx, g, k, None, 5, 1, out)
-            assert B.mlmc_get_status(ctx) == B.MLMC_OK
-            u = B.mlmc_read_u(ctx, 5, 1, M)
-            for m in sorted({0, 1, M // 2, M - 1}):
-                order = torch.sort(g[m].abs(), descending=True, stable=True).indices
-                sq = torch.cat([torch.zeros(1, dtype=torch.float64, device="cuda"), g[m].double()[order].square()])
-                norms = torch.stack([sq[a + 1:b + 1].sum() for a, b in zip([0] + k[:-1], k)]).sqrt()
-                assert torch.allclose(delta[m], norms, rtol=1e-9, atol=0.0)
-                want = norms / norms.sum() if norms.sum() > 0 else torch.eye(len(k), dtype=torch.float64, device="cuda")[0]
-                assert torch.allclose(p[m], want, rtol=1e-9, atol=1e-15)
-                level = int(out.level[m])
-                cdf = torch.cumsum(p[m], 0).tolist()
-                assert p[m, level] > 0 and (level == 0 or u[m] >= cdf[level - 1] - 1e-9) and u[m] < cdf[level] + 1e-9
-                band = torch.sort(order[(k[level - 1] if level else 0):k[level]]).values
-                n = int(out.count[m])
-                assert n == band.numel() and torch.equal(out.idx[m, :n].long() & 0xFFFFFFFF, band)
-                value = g[m][band].double() / float(out.p_sel[m])
-                assert torch.allclose(out.val[m, :n].double(), value, rtol=1e-6, atol=0.0)
+            check_adaptive(B, ctx, g, k)
+    finally:
+        B.mlmc_destroy(ctx)
+
+
+@pytest.mark.parametrize("kept", [32, 31, 1])
+def test_candidates_are_kept_in_place(B, kept):
+    """Of every 32 entries of the batches that hold candidates, `kept` share a bin with the threshold and the others lie in the bin
+    above: the pass that keeps the former moves every key by 0 places, by few or by many."""
+    M, d = 8, (1 << 25) + 515
+    gen = torch.Generator(device="cuda").manual_seed(73)
+    g = padded(torch.randn((M, d), generator=gen, device="cuda"), 4)
+    g.mul_(1e-3)
+    for m in range(M):
+        at = torch.arange(d // 50, device="cuda") + m * 12_345
+        key = torch.randint(0, 1 << 16, (len(at),), generator=gen, device="cuda", dtype=torch.int32) + 0x3F000000
+        key += ((at * 7 % 32) >= kept).int() << 16
+        g[m, at] = key.view(torch.float32) * torch.where(at % 3 == 0, -1.0, 1.0)
+    above = d // 50 * (32 - kept) // 32
+    ctx = B.mlmc_create(0, d, M, 32)
+    try:
+        check_adaptive(B, ctx, g, [above + (d // 50 - above) // 3, d])
+        check_adaptive(B, ctx, g, [above // 2, above + (d // 50 - above) // 3, d])
     finally:
         B.mlmc_destroy(ctx)
 
