@@ -89,6 +89,7 @@ struct BracketRuns {
     int top[kMaxQueries], low[kMaxQueries];  // highest and lowest bin
     uint8_t code[kMaxQueries + 1];           // level interval of the keys above run i; [n]: below the last one
 };
+constexpr int kLeftOut = 2;  // Workspace::miss: the sample finds more keys in the brackets than the candidate list has room for
 constexpr int64_t kBracketLeast = 1 << 21;  // entries of a row: at least twice as many as the largest sample
 
 // What the device can place.
@@ -167,7 +168,7 @@ struct Workspace {
     int64_t sig_k[kMaxLevels];
     // adaptive Top-k with sampled brackets
     BracketRuns* runs;           // [M]
-    int* miss;                   // [M] 1: a threshold lies outside its bracket, or the candidates did not fit
+    int* miss;                   // [M] 1: a threshold lies outside its bracket, or the candidates did not fit; kLeftOut
     uint32_t* part_n;            // [M][parts] candidates that every warp of the sweep found
     int sweep_blocks, parts;     // host: blocks and warps of the sweep per worker,
     uint32_t part_cap;           //       room of each warp

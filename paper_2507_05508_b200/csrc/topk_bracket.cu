@@ -6,7 +6,8 @@
 // threshold.  Here a sample says where the thresholds lie, within a bracket of a few bins each, and one read does the
 // rest:
 //   sample         clears what the selection accumulates into; a cluster per worker counts a stratified sample of the
-//                  row and turns every rank into a bracket of bins; brackets that touch form one run;
+//                  row and turns every rank into a bracket of bins; brackets that touch form one run.  A worker whose
+//                  runs hold too many keys (exact zeros, equal magnitudes around a threshold) is left out here;
 //   bracket_sweep  energy and count of the keys between the runs, the keys inside the runs as candidates, the largest
 //                  key of every batch for the emission;
 //   candidate_hist leading-digit counts of the candidates; with the counts between the runs they stand in for the
@@ -33,12 +34,18 @@ constexpr int kBlockSectors = kSampleThreads * kSampleTrips * 4 / kSectorKeys;
 struct SampleRanks {
     uint32_t k[kMaxQueries];
     int nq;
+    uint32_t most;  // sampled keys that the runs may hold
 };
 
 // The half width of a bracket is kSampleSigmas standard deviations of the sample rank of independent keys from one
 // distribution.  Keys that are sampled together may say the same (up to sqrt(8) times the deviation); strata that differ
 // from one another lower it (the ranks then vary within the strata only).
 constexpr double kSampleSigmas = 5.0;
+
+// Share of the candidate list that the runs may fill, by the sample.  The keys are spread over the parts of the list by batches, and one
+// full part sends the worker through the two other sweeps after this one.  8 x 2^25 entries, a threshold among equal magnitudes: at
+// 0.94 of the list 1022 us (two sweeps 1319), at 0.96 1651 (1330), left out 1366 (1363).
+constexpr double kMostRoom = 0.93;
 
 template <int C>
 __global__ void __launch_bounds__(kSampleThreads, 1)
@@ -48,7 +55,9 @@ sample_kernel(ZeroList z, SampleRanks ranks, Query* queries, const float* __rest
     __shared__ uint32_t sh_warp[32], sh_total;
     __shared__ uint32_t sh_at[2][kMaxQueries];
     __shared__ int sh_edge[2][kMaxQueries];
+    __shared__ uint32_t sh_count[2][kMaxQueries];  // sampled keys above the upper edge's bin, those down to the lower edge's
     __shared__ BracketRuns sh_runs;
+    __shared__ uint32_t sh_inside;  // sampled keys in the runs
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = C > 1 ? (int)cluster.block_rank() : 0, m = blockIdx.x / C;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nq = ranks.nq;
@@ -56,7 +65,6 @@ sample_kernel(ZeroList z, SampleRanks ranks, Query* queries, const float* __rest
     pdl_enter();
     clear_all(z);
     if (rank == 0 && threadIdx.x < nq) queries[m * kMaxQueries + threadIdx.x] = make_query(ranks.k[threadIdx.x], d);
-    if (rank == 0 && threadIdx.x == 0) miss[m] = 0;
     __syncthreads();
     constexpr uint32_t kStrata = kBlockSectors * C, n = kStrata * kSectorKeys;  // sampled keys
     if (threadIdx.x < nq) {  // bracket of query j: from the bin of sample rank r_j - half to the bin of sample rank r_j + half
@@ -125,23 +133,23 @@ sample_kernel(ZeroList z, SampleRanks ranks, Query* queries, const float* __rest
         for (int e = 0; e < 2; ++e) {
             const uint32_t at = sh_at[e][j];
             int bin = -1;
+            uint32_t count = 0;
             if (at == 0u) {
                 if (b0 == 0) bin = kBins1 - 1;
             } else if (at > n) {
-                if (b0 == 0) bin = 0;
+                if (b0 == 0) { bin = 0; count = n; }
             } else if (above < at && at <= above + sum) {
                 uint32_t run = above;
 #pragma unroll
                 for (int i = per - 1; i >= 0; --i) {
-                    if (run < at) bin = b0 + i;
+                    if (run < at) { bin = b0 + i; count = e ? run + cnt[i] : run; }
                     run += cnt[i];
                 }
             }
             if (bin >= 0) {
-                if (C > 1) {
-                    for (int q = 0; q < C; ++q) *cluster.map_shared_rank(&sh_edge[e][j], q) = bin;
-                } else {
-                    sh_edge[e][j] = bin;
+                for (int q = 0; q < C; ++q) {
+                    *(C > 1 ? cluster.map_shared_rank(&sh_edge[e][j], q) : &sh_edge[e][j]) = bin;
+                    *(C > 1 ? cluster.map_shared_rank(&sh_count[e][j], q) : &sh_count[e][j]) = count;
                 }
             }
         }
@@ -149,27 +157,38 @@ sample_kernel(ZeroList z, SampleRanks ranks, Query* queries, const float* __rest
     if (C > 1) cluster.sync(); else __syncthreads();
     if (threadIdx.x == 0) {  // runs from the largest keys down; at least one bin lies between two of them
         int R = 0, next = 0, top = 0, low = 0;
+        uint32_t inside = 0, from = 0, to = 0;
         for (int j = 0; j < nq; ++j) {
             if (ranks.k[j] == 0u) next = j + 1;
             if (ranks.k[j] == 0u || (int64_t)ranks.k[j] >= d) continue;
             const int hi = sh_edge[0][j], lo = sh_edge[1][j];
             if (R && hi >= low - 1) {
                 low = min(low, lo);
+                to = max(to, sh_count[1][j]);
             } else {
                 if (R) { sh_runs.top[R - 1] = top; sh_runs.low[R - 1] = low; }
                 sh_runs.code[R] = (uint8_t)j;
+                inside += to - from;
+                from = sh_count[0][j];
+                to = sh_count[1][j];
                 top = hi;
                 low = min(lo, hi);
                 ++R;
             }
             next = j + 1;
         }
+        inside += to - from;
         if (R) { sh_runs.top[R - 1] = top; sh_runs.low[R - 1] = low; }
         sh_runs.code[R] = (uint8_t)next;
         sh_runs.n = R;
-        if (rank == 0) runs[m] = sh_runs;
+        sh_inside = inside;
+        if (rank == 0) {
+            runs[m] = sh_runs;
+            miss[m] = inside > ranks.most ? kLeftOut : 0;
+        }
     }
     __syncthreads();
+    if (sh_inside > ranks.most) return;  // nobody looks at the table
     const int R = sh_runs.n;
     // What the sweep looks up: the interval of a bin, or nq + 1 where it lies in a run.
     constexpr int kWords = kBins1 / 4 / C;
@@ -311,6 +330,7 @@ bracket_sweep_kernel(const float* __restrict__ g, int64_t d, int64_t ld, int L, 
     uint32_t* slots = counts + columns * THREADS + threadIdx.x;                  // [kSlots][THREADS]
     pdl_enter();
     const int m = blockIdx.y;
+    if (miss[m] == kLeftOut) return;  // for all blocks of the worker: none of them gets as far as to mark it
     if (threadIdx.x == 0) sh_runs = runs[m];
     for (int i = threadIdx.x; i < kBins1 / 16; i += THREADS)
         reinterpret_cast<uint4*>(code_of)[i] = reinterpret_cast<const uint4*>(table + (int64_t)m * kBins1)[i];
@@ -552,11 +572,12 @@ bool use_brackets(int dtype, int64_t d, int M, int L) {
 
 void launch_bracket_sweep(Workspace& ws, const float* g, int64_t d, int M, int64_t ld, const int64_t* k, const FinishPlan& plan,
                           cudaStream_t s) {
+    const int C = cluster_of(ws, M);
     SampleRanks r = {};
     r.nq = plan.nq;
     for (int j = 0; j < r.nq; ++j) r.k[j] = (uint32_t)k[j];
+    r.most = (uint32_t)(std::min(kMostRoom * (double)ws.cand_cap / (double)d, 1.0) * (C * kBlockSectors * kSectorKeys));
     const ZeroList z = selection_state(ws, MLMC_F32, d, M, r.nq, true);
-    const int C = cluster_of(ws, M);
     auto sample = [&](auto kernel) {
         launch_kernel_cluster(ws, K_SAMPLE, C, kernel, dim3(M * C), kSampleThreads, kBins1 * sizeof(uint32_t), s, z, r, ws.queries, g, d, ld,
                               ws.runs, ws.table1, ws.miss);

@@ -151,3 +151,33 @@ def test_batches_that_round_to_zero_are_not_read(B, ora, dtype, d):
         check_rtn(B, ora, ctx, g, [2, 4, 8, 16], None, 1, 0, expect_excluded=2)
     finally:
         B.mlmc_destroy(ctx)
+
+
+def kernel_ms(B, ctx, call):
+    """Milliseconds of every kernel in one call."""
+    import ctypes as C
+    call(), call()
+    L, n = B.lib(), B.lib().mlmc_kernel_count()
+    ms, launches = (C.c_double * n)(), (C.c_int64 * n)()
+    L.mlmc_timing_enable(ctx, 1)
+    L.mlmc_timing_read(ctx, ms, launches, B._stream())
+    call()
+    assert L.mlmc_timing_read(ctx, ms, launches, B._stream()) == B.MLMC_OK
+    L.mlmc_timing_enable(ctx, 0)
+    return {L.mlmc_kernel_name(i).decode(): ms[i] for i in range(n) if launches[i]}
+
+
+@pytest.mark.parametrize("case", ["ties", "zeros", "constant"])
+def test_rows_whose_candidates_have_no_room_are_not_swept(B, case):
+    """A threshold among equal magnitudes that are more than the candidate list holds: the sample shows it, and the sweep between
+    the brackets, which takes longer than the histogram sweep that follows, is left out (256 MB a row: 10 us against 190)."""
+    M, d = 8, 1 << 25
+    g = rows(case, M, d)
+    k = [d // 10_000 << l for l in range(14)] + [d]
+    p = torch.zeros((M, len(k)), dtype=torch.float64, device="cuda")
+    ctx = B.mlmc_create(0, d, M, 32)
+    try:
+        ms = kernel_ms(B, ctx, lambda: B.mlmc_level_probs(ctx, g, B.MLMC_TOPK, k, None, p, None))
+        assert ms["bracket_sweep"] < 0.5 * ms["missed_hist1"], ms
+    finally:
+        B.mlmc_destroy(ctx)
