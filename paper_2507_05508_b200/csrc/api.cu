@@ -166,7 +166,7 @@ void select_adaptive(Workspace& ws, const void* g, int dtype, int64_t d, int M, 
         launch_cluster_topk(ws, g, dtype, d, M, ld, pl, nullptr, out, s);
         return;
     }
-    if (use_brackets(dtype, d, M, L)) {
+    if (use_brackets(ws, dtype, d, M, k, L)) {
         run_sampled_selection(ws, g, d, M, ld, k, pl, s);
     } else {
         launch_begin_adaptive(ws, dtype, d, M, k, L, s);

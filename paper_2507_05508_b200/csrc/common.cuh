@@ -631,7 +631,7 @@ void launch_copy_probs(Workspace& ws, int M, int L, const double* p_fixed, doubl
 // topk_bracket.cu: adaptive Top-k of long fp32 rows, one sweep
 int configure_bracket_kernels();
 void bracket_limits(KernelLimits* limits);
-bool use_brackets(int dtype, int64_t d, int M, int L);
+bool use_brackets(const Workspace& ws, int dtype, int64_t d, int M, const int64_t* k, int L);
 void launch_bracket_sweep(Workspace& ws, const float* g, int64_t d, int M, int64_t ld, const int64_t* k, const FinishPlan& plan,
                           cudaStream_t s);
 // topk_emit.cu

@@ -41,6 +41,10 @@ struct SampleRanks {
 // distribution.  Keys that are sampled together may say the same (up to sqrt(8) times the deviation); strata that differ
 // from one another lower it (the ranks then vary within the strata only).
 constexpr double kSampleSigmas = 5.0;
+__host__ __device__ inline double bracket_half(double r, double n) {  // of sample rank r among n sampled keys
+    const double v = r * (1.0 - r / n);
+    return kSampleSigmas * sqrt(v > 0.0 ? v : 0.0) + 1.0;
+}
 
 // Share of the candidate list that the runs may fill, by the sample.  The keys are spread over the parts of the list by batches, and one
 // full part sends the worker through the two other sweeps after this one.  8 x 2^25 entries, a threshold among equal magnitudes: at
@@ -68,7 +72,7 @@ sample_kernel(ZeroList z, SampleRanks ranks, Query* queries, const float* __rest
     __syncthreads();
     constexpr uint32_t kStrata = kBlockSectors * C, n = kStrata * kSectorKeys;  // sampled keys
     if (threadIdx.x < nq) {  // bracket of query j: from the bin of sample rank r_j - half to the bin of sample rank r_j + half
-        const double r = (double)ranks.k[threadIdx.x] / (double)d * n, half = kSampleSigmas * sqrt(r * fmax(1.0 - r / n, 0.0)) + 1.0;
+        const double r = (double)ranks.k[threadIdx.x] / (double)d * n, half = bracket_half(r, n);
         sh_at[0][threadIdx.x] = (uint32_t)fmax(floor(r - half), 0.0);          // 0: up to the largest key
         sh_at[1][threadIdx.x] = (uint32_t)fmin(ceil(r + half), (double)n + 1.0);  // n + 1: down to the smallest
     }
@@ -559,15 +563,37 @@ size_t sweep_smem(int L, int threads) {
 
 int cluster_of(const Workspace& ws, int M) { return M <= ws.limits.sample_fit ? 16 : M * 8 <= ws.sm_count ? 8 : M * 4 <= ws.sm_count ? 4 : M * 2 <= ws.sm_count ? 2 : 1; }
 
+int sweep_blocks_of(const Workspace& ws, int M) { return std::max(1, std::min(ws.sm_count / M, ws.sum_ctas / 2)); }
+
 }  // namespace
 
-// One sweep instead of two gains 0.35 to 0.55 us per million entries; the sample, the candidate histogram and the launches cost
-// 45 us more.  us per step, adaptive p, two sweeps / one: 8 x 8M entries 245 / 249 (ranks that double) and 379 / 387 (five ranks,
-// equal scales), 16 x 4M 245 / 287, 32 x 30M 2242 / 1830 and 4110 / 3819 (ten equal segments: 3196 / 3196).  More levels than the
-// columns of 24 warps have room for were not measured.
+// One sweep instead of two: 45 us more for the sample, the candidate histogram and the launches, and up to 0.55 us less per million
+// entries, the less the more keys lie in the brackets and around them.  That share is taken as the widths of the brackets plus
+// kThresholdShare per threshold in the middle of the row (less towards its ends, where few keys share its bins); what it stands for
+// is fitted to the times below.  us per step, adaptive p, two sweeps / one, entries of one scale and in layers of several:
+//   share 3.7 %    8 x 2^25 five ranks 1155 / 1086, 1038 / 921;  ranks that double 1119 / 1071, 672 / 545
+//   share 6.2 %    32 x 8.4M, ranks that double 1178 / 1187, 789 / 711;  32 x 25M 3174 / 3078, 2050 / 1718
+//   share 9 %      16 x 16.8M ten ranks 1150 / 1166, 950 / 954;  128 x 2^21 five ranks 1251 / 1245, 1379 / 1336
+//   share 11.5 %   32 x 8.4M ten ranks 1188 / 1249, 1020 / 1055;  32 x 25M 3375 / 3385, 2509 / 2491
+//   share 14 %     16 x 16.8M 15 ranks 1144 / 1193, 917 / 971;  64 x 4.3M ten ranks 1229 / 1287, 1053 / 1111
+//   share 29 %     128 x 2^21 15 ranks 1228 / 1432, 1111 / 1317
+// Below 2^28 entries: 8 x 8M 245 / 249 (ranks that double) and 379 / 387 (five ranks), 16 x 4M 245 / 287.
+// The sweep is bound by issue and takes a block per SM: with 75 to 98 workers, of one block each, a third of the SMs or more idle
+// (80 x 3.4M, ranks that double: 1405 / 1513, 1023 / 1024).
+// More levels than the columns of 24 warps have room for were not measured.
 constexpr int64_t kBracketEntries = int64_t(1) << 28;
-bool use_brackets(int dtype, int64_t d, int M, int L) {
-    return dtype == MLMC_F32 && d >= kBracketLeast && d * M >= kBracketEntries && sweep_smem(L, kSweepThreads24) <= (size_t)kSweepSmemMost;
+constexpr double kThresholdShare = 0.008;
+bool use_brackets(const Workspace& ws, int dtype, int64_t d, int M, const int64_t* k, int L) {
+    if (dtype != MLMC_F32 || d < kBracketLeast || d * M < kBracketEntries || sweep_smem(L, kSweepThreads24) > (size_t)kSweepSmemMost)
+        return false;
+    if (3 * sweep_blocks_of(ws, M) * M < 2 * ws.sm_count) return false;
+    const double n = (double)cluster_of(ws, M) * kBlockSectors * kSectorKeys;
+    double share = 0.0;
+    for (int l = 0; l + 1 < L; ++l) {
+        const double q = (double)k[l] / (double)d;
+        if (k[l] > 0 && k[l] < d) share += 2.0 * bracket_half(q * n, n) / n + 2.0 * std::min(q, 1.0 - q) * kThresholdShare;
+    }
+    return share <= 0.12 - 0.02 * (double)kBracketEntries / ((double)d * M);
 }
 
 void launch_bracket_sweep(Workspace& ws, const float* g, int64_t d, int M, int64_t ld, const int64_t* k, const FinishPlan& plan,
@@ -588,7 +614,7 @@ void launch_bracket_sweep(Workspace& ws, const float* g, int64_t d, int M, int64
     else if (C == 2) sample(sample_kernel<2>);
     else sample(sample_kernel<1>);
     constexpr int threads = kSweepThreads24;
-    const int nb = std::max(1, std::min(ws.sm_count / M, ws.sum_ctas / 2)), tpw = emit_tiles_per_worker(d, MLMC_F32);
+    const int nb = sweep_blocks_of(ws, M), tpw = emit_tiles_per_worker(d, MLMC_F32);
     ws.sweep_blocks = nb;
     ws.parts = nb * (threads / 32);
     ws.part_cap = (uint32_t)(ws.cand_cap / ws.parts) & ~3u;  // parts start on 16 bytes

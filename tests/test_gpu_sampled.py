@@ -181,3 +181,32 @@ def test_rows_whose_candidates_have_no_room_are_not_swept(B, case):
         assert ms["bracket_sweep"] < 0.5 * ms["missed_hist1"], ms
     finally:
         B.mlmc_destroy(ctx)
+
+
+def equal(d, n):
+    return [d * (i + 1) // n for i in range(n - 1)] + [d]
+
+
+def doubling(d):
+    return [d // 10_000 << l for l in range(14)] + [d]
+
+
+@pytest.mark.parametrize("d,M,one,two", [
+    (1 << 25, 8, [equal(1 << 25, 10), doubling(1 << 25)], [equal(1 << 25, 15), equal(1 << 25, 16)]),
+    (2_100_001, 128, [equal(2_100_001, 5)], [equal(2_100_001, 10), equal(2_100_001, 15), doubling(2_100_001)]),
+    (3_400_000, 80, [], [equal(3_400_000, 5), doubling(3_400_000)]),
+    ((1 << 25) - 1, 8, [], [[1, (1 << 25) - 1]]),
+])
+def test_calls_that_one_sweep_serves(B, d, M, one, two):
+    """Few workers and levels take one sweep; wide brackets (many workers, and so few samples of each), many levels and sweeps that
+    leave SMs without a block cost more than the second sweep."""
+    g = rows("layers", M, d)
+    ctx = B.mlmc_create(0, d, M, 32)
+    try:
+        for k in one + two:
+            p = torch.zeros((M, len(k)), dtype=torch.float64, device="cuda")
+            names = kernel_ms(B, ctx, lambda: B.mlmc_level_probs(ctx, g, B.MLMC_TOPK, k, None, p, None))
+            assert ("bracket_sweep" in names) == (k in one) and ("sums_candidates" in names) == (k in two), (k, names)
+            check_adaptive(B, ctx, g, k)
+    finally:
+        B.mlmc_destroy(ctx)
