@@ -7,7 +7,7 @@
 // rest:
 //   sample         clears what the selection accumulates into; a cluster per worker counts a stratified sample of the
 //                  row and turns every rank into a bracket of bins; brackets that touch form one run.  A worker whose
-//                  runs hold too many keys (exact zeros, equal magnitudes around a threshold) is left out here;
+//                  runs hold too many keys (exact zeros, equal magnitudes around a threshold) takes the call out of the sweep;
 //   bracket_sweep  energy and count of the keys between the runs, the keys inside the runs as candidates, the largest
 //                  key of every batch for the emission;
 //   candidate_hist leading-digit counts of the candidates; with the counts between the runs they stand in for the
@@ -320,7 +320,7 @@ template <int THREADS>
 __global__ void __launch_bounds__(THREADS, 1)
 bracket_sweep_kernel(const float* __restrict__ g, int64_t d, int64_t ld, int L, const BracketRuns* runs, const uint8_t* table,
                      uint32_t* __restrict__ tile_max, int tiles_per_worker, uint32_t* hist1, double* __restrict__ sum_partial,
-                     int sum_ctas, uint32_t* __restrict__ cand_keys, int64_t cand_cap, uint32_t part_cap, uint32_t* part_n, int* miss,
+                     int sum_ctas, uint32_t* __restrict__ cand_keys, int64_t cand_cap, uint32_t part_cap, uint32_t* part_n, int* miss, int M,
                      int* status, int* worker_err, uint32_t one, double zero) {
     extern __shared__ __align__(16) uint8_t sh_raw[];
     __shared__ BracketRuns sh_runs;
@@ -334,7 +334,14 @@ bracket_sweep_kernel(const float* __restrict__ g, int64_t d, int64_t ld, int L, 
     uint32_t* slots = counts + columns * THREADS + threadIdx.x;                  // [kSlots][THREADS]
     pdl_enter();
     const int m = blockIdx.y;
-    if (miss[m] == kLeftOut) return;  // for all blocks of the worker: none of them gets as far as to mark it
+    // Where one worker is left out all of them are: its two other sweeps take as long as those of all workers (the blocks are dealt
+    // to the workers).  All blocks see the sample's mark of that worker, whoever else has been marked meanwhile.
+    bool left_out = false;
+    for (int i = threadIdx.x; i < M; i += THREADS) left_out |= miss[i] == kLeftOut;
+    if (__syncthreads_or(left_out)) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) miss[m] = kLeftOut;
+        return;
+    }
     if (threadIdx.x == 0) sh_runs = runs[m];
     for (int i = threadIdx.x; i < kBins1 / 16; i += THREADS)
         reinterpret_cast<uint4*>(code_of)[i] = reinterpret_cast<const uint4*>(table + (int64_t)m * kBins1)[i];
@@ -620,7 +627,7 @@ void launch_bracket_sweep(Workspace& ws, const float* g, int64_t d, int M, int64
     ws.part_cap = (uint32_t)(ws.cand_cap / ws.parts) & ~3u;  // parts start on 16 bytes
     launch_kernel(ws, K_BRACKET_SWEEP, bracket_sweep_kernel<threads>, dim3(nb, M), threads, sweep_smem(plan.L, threads), s, g, d, ld, plan.L,
                   ws.runs, ws.table1, ws.tile_max, tpw, ws.hist1, ws.sum_partial, ws.sum_ctas, ws.cand_keys, ws.cand_cap, ws.part_cap,
-                  ws.part_n, ws.miss, ws.status, ws.worker_err, 1u, 0.0);
+                  ws.part_n, ws.miss, M, ws.status, ws.worker_err, 1u, 0.0);
     launch_kernel(ws, K_CAND_HIST, candidate_hist_kernel, dim3(nb, M), kCandHistThreads, kBins1 * sizeof(uint32_t), s, ws.cand_keys,
                   ws.cand_cap, ws.part_cap, ws.part_n, ws.parts, ws.hist1, ws.miss, ws.worker_err);
 }
