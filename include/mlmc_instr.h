@@ -48,6 +48,13 @@ int mlmc_read_listed_tiles(mlmc_ctx* ctx, int M, uint32_t* listed_host, int64_t*
  * Synchronous; a measurement aid. */
 int mlmc_read_bracket_stats(mlmc_ctx* ctx, uint64_t* stats_host, void* stream);
 
+/* Adaptive Top-k of large fp32 calls looks for its thresholds inside brackets from a sample of every row.
+ *   stats_host  host uint64[3], cumulative since mlmc_create: workers whose brackets all held (one sweep) / workers with a
+ *               threshold outside its bracket or more candidates than there was room for (two more sweeps) / workers of calls
+ *               that the sample took out of the sweep, because some worker's brackets hold too many keys (two sweeps).
+ * Synchronous; a measurement aid. */
+int mlmc_read_sample_stats(mlmc_ctx* ctx, uint64_t* stats_host, void* stream);
+
 #ifdef __cplusplus
 }
 #endif

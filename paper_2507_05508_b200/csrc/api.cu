@@ -306,7 +306,7 @@ int mlmc_create(mlmc_ctx** out, int device, int64_t d_max, int M_max, int L_max)
     const size_t o_pbin = pl.take(sizeof(uint32_t) * kMaxLevels * M_max);
     const size_t o_brk = pl.take(sizeof(uint4) * M_max);
     const size_t o_bhit = pl.take(sizeof(int) * M_max);
-    const size_t o_bstat = pl.take(sizeof(unsigned long long) * 4);
+    const size_t o_bstat = pl.take(sizeof(unsigned long long) * 8);
     const size_t o_runs = pl.take(sizeof(BracketRuns) * M_max);
     const size_t o_miss = pl.take(sizeof(int) * M_max);
     // one block of up to 32 warps per SM, or one per worker where there are more workers than SMs
@@ -474,6 +474,15 @@ int mlmc_read_bracket_stats(mlmc_ctx* ctx, uint64_t* stats_host, void* stream) {
     DeviceGuard guard(ctx->ws.device);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (cudaMemcpyAsync(stats_host, ctx->ws.bracket_stats, sizeof(uint64_t) * 3, cudaMemcpyDeviceToHost, s) != cudaSuccess)
+        return MLMC_ERR_CUDA;
+    return finish(cudaStreamSynchronize(s));
+}
+
+int mlmc_read_sample_stats(mlmc_ctx* ctx, uint64_t* stats_host, void* stream) {
+    if (!ctx || !stats_host) return MLMC_ERR_ARG;
+    DeviceGuard guard(ctx->ws.device);
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    if (cudaMemcpyAsync(stats_host, ctx->ws.bracket_stats + 4, sizeof(uint64_t) * 3, cudaMemcpyDeviceToHost, s) != cudaSuccess)
         return MLMC_ERR_CUDA;
     return finish(cudaStreamSynchronize(s));
 }

@@ -162,7 +162,9 @@ struct Workspace {
     uint32_t* prev_bin;          // [M][kMaxLevels] leading-digit bin of threshold j at the last call that resolved it (kKeyNone: none)
     uint4* bracket;              // [M] {lo_a, width_a, lo_b, width_b}: bins collected as candidates by the first sweep
     int* bracket_hit;            // [M] 1: both boundary bins of the drawn band lie in their brackets
-    unsigned long long* bracket_stats;  // [3] workers with both brackets hit / a bracket missed / no bracket yet (cumulative)
+    // [3] workers with both brackets hit / a bracket missed / no bracket yet; from [4] on, sampled brackets: all held / missed / left out
+    // (cumulative)
+    unsigned long long* bracket_stats;
     int64_t sig_d, sig_ld;       // host: the problem the stored bins belong to
     int sig_M, sig_L, sig_dtype;
     int64_t sig_k[kMaxLevels];

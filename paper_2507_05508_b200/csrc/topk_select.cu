@@ -350,8 +350,11 @@ resolve1_kernel(const uint32_t* hist1, Query* queries, uint8_t* table1, uint32_t
             const int bin = sh_bin[threadIdx.x];
             out |= bin < 0 || table1[(int64_t)m * kBins1 + bin] != nq + 1;  // so marked by the sample
         }
-        if (__syncthreads_or(out)) {
-            if (threadIdx.x == 0) miss[m] = 1;
+        const bool left_out = miss[m] == kLeftOut;
+        const bool missed = __syncthreads_or(out);
+        if (threadIdx.x == 0) atomicAdd(&bracket_stats[4 + (!missed ? 0 : left_out ? 2 : 1)], 1ull);
+        if (missed) {
+            if (threadIdx.x == 0 && !left_out) miss[m] = 1;
             uint4* h = reinterpret_cast<uint4*>(const_cast<uint32_t*>(hist1) + (int64_t)m * kBins1);
             for (int i = threadIdx.x; i < kBins1 / 4; i += kResolveThreads) h[i] = make_uint4(0u, 0u, 0u, 0u);
             return;

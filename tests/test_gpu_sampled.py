@@ -8,8 +8,6 @@ from test_gpu_parity import check_bitwise, padded, to_dev
 
 pytestmark = pytest.mark.gpu
 
-LEAST = 1 << 28       # entries of the smallest call that is sampled; its rows have at least 2^21
-
 
 @pytest.fixture(scope="module")
 def B():
@@ -41,8 +39,10 @@ def rows(case, M, d, seed=71):
         g.mul_(2.0).round_()
     elif case == "zeros":
         g *= torch.rand(d, generator=gen, device="cuda") < 0.03
-    elif case == "unseen":            # the sample sees nothing but zeros: every bracket misses
+    elif case == "unseen":            # the sample sees nothing but zeros: more than there is room for
         g[:, torch.from_numpy(sampled_entries(d)).cuda()] = 0.0
+    elif case == "misled":            # the sample sees entries of another scale: every row has a bracket that misses
+        g[:, torch.from_numpy(sampled_entries(d)).cuda()] *= 1000.0
     elif case == "constant":
         g.fill_(0.25)
     return g
@@ -75,17 +75,51 @@ def check_adaptive(B, ctx, g, k):
         assert torch.allclose(out.val[m, :n].double(), value, rtol=1e-6, atol=0.0)
 
 
-@pytest.mark.parametrize("case", ["layers", "normal", "ties", "zeros", "unseen", "constant"])
+HELD, MISSED, LEFT_OUT = range(3)
+
+
+def check_sampled(B, ctx, g, k, want):
+    """check_adaptive, and what became of the workers' brackets: `want` of HELD, MISSED, LEFT_OUT per worker; empty: two sweeps."""
+    before = B.mlmc_read_sample_stats(ctx)
+    check_adaptive(B, ctx, g, k)      # two selections
+    seen = [b - a for a, b in zip(before, B.mlmc_read_sample_stats(ctx))]
+    assert seen == [2 * sum(w == i for w in want) for i in range(3)], (seen, k)
+
+
+@pytest.mark.parametrize("case", ["layers", "normal", "ties", "zeros", "unseen", "misled", "constant"])
 @pytest.mark.parametrize("d,M", [((1 << 21) + 1, 128), ((1 << 25) + 515, 8), ((1 << 27) + 3, 2)])
 def test_adaptive_topk_from_a_sample(B, case, d, M):
     """Probabilities, levels and bands against a sort of every row on the device.  Its fp64 sums over a whole row round by at
     most d 2^-53 of the sum, 1.5e-8 for the longest row here; running sums of random order stay far below."""
     g = rows(case, M, d)
+    want = {"layers": HELD, "normal": HELD, "misled": MISSED}.get(case, LEFT_OUT)
     ctx = B.mlmc_create(0, d, M, 32)
     try:
         for k in ([d // 10_000 << l for l in range(13)] + [d], [d * (i + 1) // 10 for i in range(9)] + [d],
                   [0, 1, 2, d // 3, d // 3 + 1, d, d]):
-            check_adaptive(B, ctx, g, k)
+            if len(k) == 10 and M == 128:
+                check_sampled(B, ctx, g, k, [])         # ten brackets of so small samples are too wide
+            elif case == "ties" and M == 128:
+                check_adaptive(B, ctx, g, k)            # the list has about the room for the equal magnitudes
+            else:
+                check_sampled(B, ctx, g, k, [want] * M)
+    finally:
+        B.mlmc_destroy(ctx)
+
+
+def test_held_and_missed_rows_of_one_call(B):
+    """The workers with a missed bracket take the two sweeps of whole rows, the others do not; a schedule without a threshold."""
+    M, d = 8, (1 << 25) + 515
+    g = rows("normal", M, d)
+    g[5] = rows("misled", 1, d)
+    ctx = B.mlmc_create(0, d, M, 32)
+    try:
+        check_sampled(B, ctx, g, doubling(d), [HELD] * 5 + [MISSED] + [HELD] * 2)
+        g[0] = rows("misled", 1, d)
+        check_sampled(B, ctx, g, equal(d, 5), [MISSED] + [HELD] * 4 + [MISSED] + [HELD] * 2)
+        check_sampled(B, ctx, g, [d], [HELD] * M)
+        g[7] = 0.0
+        check_sampled(B, ctx, g, doubling(d), [LEFT_OUT] * M)
     finally:
         B.mlmc_destroy(ctx)
 
@@ -106,8 +140,8 @@ def test_candidates_are_kept_in_place(B, kept):
     above = d // 50 * (32 - kept) // 32
     ctx = B.mlmc_create(0, d, M, 32)
     try:
-        check_adaptive(B, ctx, g, [above + (d // 50 - above) // 3, d])
-        check_adaptive(B, ctx, g, [above // 2, above + (d // 50 - above) // 3, d])
+        check_sampled(B, ctx, g, [above + (d // 50 - above) // 3, d], [HELD] * M)
+        check_sampled(B, ctx, g, [above // 2, above + (d // 50 - above) // 3, d], [HELD] * M)
     finally:
         B.mlmc_destroy(ctx)
 
@@ -180,7 +214,7 @@ def test_rows_whose_candidates_have_no_room_are_not_swept(B, case, some):
     try:
         ms = kernel_ms(B, ctx, lambda: B.mlmc_level_probs(ctx, g, B.MLMC_TOPK, k, None, p, None))
         assert ms["bracket_sweep"] < 0.5 * ms["missed_hist1"], ms
-        check_adaptive(B, ctx, g, k)
+        check_sampled(B, ctx, g, k, [LEFT_OUT] * M)
     finally:
         B.mlmc_destroy(ctx)
 
@@ -209,6 +243,6 @@ def test_calls_that_one_sweep_serves(B, d, M, one, two):
             p = torch.zeros((M, len(k)), dtype=torch.float64, device="cuda")
             names = kernel_ms(B, ctx, lambda: B.mlmc_level_probs(ctx, g, B.MLMC_TOPK, k, None, p, None))
             assert ("bracket_sweep" in names) == (k in one) and ("sums_candidates" in names) == (k in two), (k, names)
-            check_adaptive(B, ctx, g, k)
+            check_sampled(B, ctx, g, k, [HELD] * M if k in one else [])
     finally:
         B.mlmc_destroy(ctx)
