@@ -127,6 +127,7 @@ def test_floatbits_degenerate_and_errors(B, ora, ctx):
 def check_rtn(B, ora, ctx, g, r, p, seed, step, expect_excluded=1):
     M, d = g.shape
     out = B.RtnBuffers(M, d)
+    out.val.fill_(float("nan"))           # a program hands over the buffers of the step before
     dense = torch.full((d,), float("nan"), dtype=torch.float32, device="cuda")
     B.mlmc_compress_rtn(ctx, g, r, p, seed, step, out)
     B.mlmc_aggregate_rtn(ctx, out, M, d, dense)

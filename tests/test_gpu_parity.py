@@ -17,6 +17,7 @@ pytestmark = pytest.mark.gpu
 
 VAL_RTOL = 1e-6
 AGG_RTOL = 1e-6
+STALE = 0x5A5A5A5A
 MARGIN = 1e-9
 
 
@@ -87,6 +88,7 @@ def check_bitwise(B, ora, ctx, g: torch.Tensor, b, p, seed, step):
     M, d = g.shape
     widths = np.diff(np.concatenate([[0], b]))
     out = B.BitBuffers(M, d, int(widths.max()))
+    out.planes.fill_(STALE)               # a program hands over the buffers of the step before
     dense = torch.full((d,), float("nan"), dtype=torch.float32, device="cuda")
     B.mlmc_compress_bitwise(ctx, g, b, p, seed, step, out)
     B.mlmc_aggregate(ctx, B.MLMC_BITWISE, out, b, M, d, dense)
@@ -106,6 +108,7 @@ def check_bitwise(B, ora, ctx, g: torch.Tensor, b, p, seed, step):
         assert abs(p_sel[m] - o.p_sel) <= 1e-11 * max(o.p_sel, 1e-300) + 1e-15
         w = int(widths[o.level])
         assert np.array_equal(planes[m, :1 + w], o.planes), f"worker {m}: bit planes differ"
+        assert (planes[m, 1 + w:] == STALE).all(), f"worker {m}: planes past the field are written"
         msgs.append(o)
     ref, scale = ora.aggregate_bitwise(msgs, b, d)
     got = dense.cpu().numpy().astype(np.float64)
