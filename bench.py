@@ -327,21 +327,22 @@ class Runner:
             self.B.mlmc_destroy(ctx)
 
 
-SAMPLED_LEAST = 1 << 28  # entries of a call from which adaptive fp32 Top-k of at most 15 levels selects in one sweep
-
-
-def sweeps_charged(w, emit_read_frac=None) -> float:
+def sweeps_charged(w, emit_read_frac=None, sampled=(0, 0, 0)) -> float:
     """Gradient sweeps charged to the step: what the method needs (a true data dependence separates them: select ->
     emit for Top-k, max -> pack for fixed-p bit-wise, max -> field energies -> pack for adaptive bit-wise), or what
-    the kernels moved where that is less.  Top-k moves one whole sweep, for adaptive fp32 rows too short to be sampled a
-    second one, and two passes over the listed tiles (emit_read_frac of the row each); the fixed-p candidate sweep,
-    which also skips tiles, is counted as nothing, and so is the last sweep of the bit-wise and RTN compressors, which
-    skips the batches that round to 0: the figure is a lower bound of the bytes moved."""
+    the kernels moved where that is less.  Top-k moves one whole sweep, for adaptive fp32 rows a second one unless their
+    brackets from a sample held (sampled: workers whose brackets held, missed, were left out, as the library counted them in
+    this run), and two passes over the listed tiles (emit_read_frac of the row each); the fixed-p candidate sweep, which
+    also skips tiles, is counted as nothing, and so is the last sweep of the bit-wise and RTN compressors, which skips the
+    batches that round to 0: the figure is a lower bound of the bytes moved."""
     if w.kind in ("topk", "stopk"):
         if emit_read_frac is None:
             return 2.0
-        moved = 1.0 + (1.0 if (w.adaptive and w.dtype != "bf16" and w.M * w.d < SAMPLED_LEAST) else 0.0) + 2.0 * emit_read_frac
-        return min(2.0, moved)
+        held, missed, left_out = sampled
+        second = 1.0 if w.adaptive and w.dtype != "bf16" else 0.0
+        if held + missed + left_out:
+            second *= (2.0 * missed + left_out) / (held + missed + left_out)
+        return min(2.0, 1.0 + second + 2.0 * emit_read_frac)
     if w.kind == "floatbits":
         return 1.0  # App. B's probabilities are fixed: the level is drawn before the data is read, one sweep packs it
     return 2.0 if w.adaptive else 1.0  # bit-wise and RTN: max -> level statistics -> message (counted without its reads)
@@ -351,13 +352,13 @@ def sweeps_charged(w, emit_read_frac=None) -> float:
 # bytes, share of the row in the listed tiles).  band_count and emit read only the tiles that can hold band entries,
 # so they are charged that share of the row; the candidate sweep of fixed p also skips tiles, by a share that is not
 # read back, so its bytes are unknown (None) there.
-def kernel_alg_bytes(name: str, sweep: float, msg: dict, dense: float, read_frac, adaptive: bool):
+def kernel_alg_bytes(name: str, sweep: float, msg: dict, dense: float, read_frac, adaptive: bool, sampled=(0, 0, 0)):
     mt, mb = msg.get("topk", 0.0), msg.get("bitwise", 0.0)
     mf, md = msg.get("floatbits", 0.0), msg.get("dense", 0.0)
     listed = None if read_frac is None else read_frac * sweep
     table = {
         # the digit passes read the row only where a worker's candidates overflowed: no bytes are claimed for them
-        "hist1": sweep, "bracket_sweep": sweep, "segment_sweep": sweep, "sums_candidates": sweep if adaptive else None,
+        "hist1": sweep, "bracket_sweep": None if sampled[2] else sweep, "segment_sweep": sweep, "sums_candidates": sweep if adaptive else None,
         "band_count": listed, "emit": None if listed is None else listed + mt,
         "aggregate_topk": mt + dense,
         # the message kernels skip the batches that round to 0, by a share that is not read back: only what they write is claimed
@@ -450,6 +451,7 @@ def measure(subs, local: int, rank: int, world: int, steps: int, warmup: int, pe
             listed_n += 1
     r.timing_enable(False)
     emit_read_frac = (listed_acc / listed_n) if listed_n else None
+    sampled = B.mlmc_read_sample_stats(r.topk_ctx()) if r.topk_ctx() else (0, 0, 0)
     msg_by_kind = {kind: v / probe for kind, v in msg_acc.items()}
     msg_bytes = sum(msg_by_kind.values())
 
@@ -459,7 +461,7 @@ def measure(subs, local: int, rank: int, world: int, steps: int, warmup: int, pe
     kernels = {}
     t_all = sum(v[0] for v in per_kernel.values())
     for name, (ms, n) in sorted(per_kernel.items(), key=lambda kv: -kv[1][0]):
-        kb = kernel_alg_bytes(name, sweep_bytes, msg_by_kind, dense_bytes, emit_read_frac, adaptive_topk)
+        kb = kernel_alg_bytes(name, sweep_bytes, msg_by_kind, dense_bytes, emit_read_frac, adaptive_topk, sampled)
         avg_ms = ms / n
         ach = None if not kb else kb / (avg_ms * 1e-3) / 1e9
         kernels[name] = {"ms_per_step": round(ms / probe, 4), "launches_per_step": n / probe,
@@ -467,7 +469,7 @@ def measure(subs, local: int, rank: int, world: int, steps: int, warmup: int, pe
                          "frac": None if ach is None else round(ach / peak, 4)}
     dom_name = next(iter(kernels))
     dom_ms, dom_n = per_kernel[dom_name]
-    dom_bytes = kernel_alg_bytes(dom_name, sweep_bytes, msg_by_kind, dense_bytes, emit_read_frac, adaptive_topk)
+    dom_bytes = kernel_alg_bytes(dom_name, sweep_bytes, msg_by_kind, dense_bytes, emit_read_frac, adaptive_topk, sampled)
     dom_avg_s = dom_ms / dom_n * 1e-3
     achieved = None if not dom_bytes else dom_bytes / dom_avg_s / 1e9
     ratio = ratios.get(f"{dom_name}:{w.dtype}")
@@ -476,7 +478,7 @@ def measure(subs, local: int, rank: int, world: int, steps: int, warmup: int, pe
                 "peak_source": peak_kind,
                 "traffic": None if (ratio is None or not dom_bytes) else ratio * dom_bytes,
                 "alg_bytes_per_launch": dom_bytes, "avg_launch_ms": round(dom_avg_s * 1e3, 4)}
-    b_alg = sum(sweeps_charged(x, emit_read_frac) * sweep_bytes + dense_bytes for x in subs) + 2 * msg_bytes
+    b_alg = sum(sweeps_charged(x, emit_read_frac, sampled) * sweep_bytes + dense_bytes for x in subs) + 2 * msg_bytes
     step_frac = b_alg / (ms_per_step * 1e-3) / 1e9 / peak
 
     # ---- end to end: inputs start in pinned host memory, the dense mean ends in host memory
@@ -544,7 +546,7 @@ def measure(subs, local: int, rank: int, world: int, steps: int, warmup: int, pe
                    "parallelism": "replicas only"},
         "elements_per_s": round(world * len(subs) * w.M * w.d / (ms_per_step * 1e-3), 1),
         "step_roofline": {"alg_bytes_per_step": b_alg,
-                          "sweeps_charged": [round(sweeps_charged(x, emit_read_frac), 3) for x in subs],
+                          "sweeps_charged": [round(sweeps_charged(x, emit_read_frac, sampled), 3) for x in subs],
                           "emit_tiles_read_frac": None if emit_read_frac is None else round(emit_read_frac, 4),
                           "message_bytes_per_step": msg_bytes, "frac_of_peak": round(step_frac, 4),
                           "frac_of_8TBs": round(b_alg / (ms_per_step * 1e-3) / 8e12, 4)},
