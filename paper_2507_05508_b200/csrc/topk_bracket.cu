@@ -13,7 +13,8 @@
 //   candidate_hist leading-digit counts of the candidates; with the counts between the runs they stand in for the
 //                  histogram of the row.
 // The rest is topk_select.cu: resolve1 finds the bin of every threshold (in a run, or the worker is sent through the
-// histogram path: the results never depend on the sample), the digit passes end the selection.
+// histogram path), the digit passes end the selection.  Thresholds and bands never depend on the sample; the energies are the same
+// sums of squares in fp64, added up in an order that follows the runs, so that norms and probabilities agree to rounding.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -236,10 +237,9 @@ constexpr int kFewAbove = 2, kSomeAbove = 1;      // of 32 keys: above the two, 
 constexpr int kSweepThreads24 = 768;              // 24 warps, six per scheduler
 
 // One key against the edges of the lowest runs: x < lo_a: interval R (e0); hi_a <= x < lo_b: R - 1 (e1, c1); with three intervals
-// hi_b <= x < lo_c: R - 2 (e2, c2); otherwise it is set aside.  Written out, since the compiler turns a conditional fp64 addition
-// into an unconditional one and two selections and moves of the sum's halves (25 instructions per key where these are 18): the
-// square is multiplied by 1 or 0, of which only the high word is ever set (m0, m1, m2 are 0 or 1).  Counters as floats and the
-// address by a multiplication, one = 1: the integer pipe has the comparisons to do.
+// hi_b <= x < lo_c: R - 2 (e2, c2); otherwise it is set aside.  No branch and no selection between sums: the square is multiplied by
+// 1 or 0, of which only the high word is ever set (m0, m1, m2 are 0 or 1).  Counters as floats and the address by a multiplication,
+// one = 1: the integer pipe has the comparisons to do.
 __device__ __forceinline__ void window_add_two(uint32_t bits, float lo_a, float hi_a, float lo_b, double& e0, double& e1, double& m0,
                                                double& m1, float& c1, uint32_t& at, uint32_t step, uint32_t one) {
     asm volatile(
