@@ -59,8 +59,8 @@ sample_kernel(ZeroList z, SampleRanks ranks, Query* queries, const float* __rest
     extern __shared__ uint32_t sh_hist[];  // [kBins1]
     __shared__ uint32_t sh_warp[32], sh_total;
     __shared__ uint32_t sh_at[2][kMaxQueries];
-    __shared__ int sh_edge[2][kMaxQueries];
-    __shared__ uint32_t sh_count[2][kMaxQueries];  // sampled keys above the upper edge's bin, those down to the lower edge's
+    // the bracket's edges: {bin, sampled keys above the upper edge's bin, or those down to the lower edge's}
+    __shared__ uint2 sh_edge[2][kMaxQueries];
     __shared__ BracketRuns sh_runs;
     __shared__ uint32_t sh_inside;  // sampled keys in the runs
     cg::cluster_group cluster = cg::this_cluster();
@@ -152,10 +152,8 @@ sample_kernel(ZeroList z, SampleRanks ranks, Query* queries, const float* __rest
                 }
             }
             if (bin >= 0) {
-                for (int q = 0; q < C; ++q) {
-                    *(C > 1 ? cluster.map_shared_rank(&sh_edge[e][j], q) : &sh_edge[e][j]) = bin;
-                    *(C > 1 ? cluster.map_shared_rank(&sh_count[e][j], q) : &sh_count[e][j]) = count;
-                }
+                for (int q = 0; q < C; ++q)
+                    *(C > 1 ? cluster.map_shared_rank(&sh_edge[e][j], q) : &sh_edge[e][j]) = make_uint2((uint32_t)bin, count);
             }
         }
     }
@@ -166,16 +164,17 @@ sample_kernel(ZeroList z, SampleRanks ranks, Query* queries, const float* __rest
         for (int j = 0; j < nq; ++j) {
             if (ranks.k[j] == 0u) next = j + 1;
             if (ranks.k[j] == 0u || (int64_t)ranks.k[j] >= d) continue;
-            const int hi = sh_edge[0][j], lo = sh_edge[1][j];
+            const uint2 upper = sh_edge[0][j], lower = sh_edge[1][j];
+            const int hi = (int)upper.x, lo = (int)lower.x;
             if (R && hi >= low - 1) {
                 low = min(low, lo);
-                to = max(to, sh_count[1][j]);
+                to = max(to, lower.y);
             } else {
                 if (R) { sh_runs.top[R - 1] = top; sh_runs.low[R - 1] = low; }
                 sh_runs.code[R] = (uint8_t)j;
                 inside += to - from;
-                from = sh_count[0][j];
-                to = sh_count[1][j];
+                from = upper.y;
+                to = lower.y;
                 top = hi;
                 low = min(lo, hi);
                 ++R;
@@ -334,14 +333,8 @@ bracket_sweep_kernel(const float* __restrict__ g, int64_t d, int64_t ld, int L, 
     uint32_t* slots = counts + columns * THREADS + threadIdx.x;                  // [kSlots][THREADS]
     pdl_enter();
     const int m = blockIdx.y;
-    // Where one worker is left out all of them are: its two other sweeps take as long as those of all workers (the blocks are dealt
-    // to the workers).  All blocks see the sample's mark of that worker, whoever else has been marked meanwhile.
     bool left_out = false;
     for (int i = threadIdx.x; i < M; i += THREADS) left_out |= miss[i] == kLeftOut;
-    if (__syncthreads_or(left_out)) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) miss[m] = kLeftOut;
-        return;
-    }
     if (threadIdx.x == 0) sh_runs = runs[m];
     for (int i = threadIdx.x; i < kBins1 / 16; i += THREADS)
         reinterpret_cast<uint4*>(code_of)[i] = reinterpret_cast<const uint4*>(table + (int64_t)m * kBins1)[i];
@@ -349,7 +342,12 @@ bracket_sweep_kernel(const float* __restrict__ g, int64_t d, int64_t ld, int L, 
         energy[l * THREADS + threadIdx.x] = 0.0;
         counts[l * THREADS + threadIdx.x] = 0u;
     }
-    __syncthreads();
+    // Where one worker is left out all of them are: its two other sweeps take as long as those of all workers (the blocks are dealt
+    // to the workers).  All blocks see the sample's mark of that worker, whoever else has been marked meanwhile.
+    if (__syncthreads_or(left_out)) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) miss[m] = kLeftOut;
+        return;
+    }
     const int R = sh_runs.n;
     // Edges of the three lowest runs as floats (the order of non-negative floats is that of their bits); a run that is not there
     // lies above every key.
