@@ -278,7 +278,7 @@ int mlmc_create(mlmc_ctx** out, int device, int64_t d_max, int M_max, int L_max)
     const size_t o_hist23 = pl.take(sizeof(uint32_t) * kMaxQueries * kBins23 * 2 * M_max);
     const size_t o_map2 = pl.take((size_t)kMaxQueries * kBins23 * M_max);
     const size_t o_done = pl.take(sizeof(uint32_t) * M_max);
-    const size_t o_acc = pl.take(sizeof(uint32_t) * M_max);
+    const size_t o_acc = pl.take(sizeof(uint32_t) * 2 * M_max);
     const size_t o_queries = pl.take(sizeof(Query) * kMaxQueries * M_max);
     const size_t o_sum = pl.take(sizeof(double) * kMaxLevels * ws.sum_ctas * M_max);
     const size_t o_cpart = pl.take(sizeof(unsigned long long) * kEnergyCells * 2 * M_max);
@@ -297,7 +297,7 @@ int mlmc_create(mlmc_ctx** out, int device, int64_t d_max, int M_max, int L_max)
     const size_t o_groupn = pl.take(sizeof(uint32_t) * M_max);
     const size_t o_cfloor = pl.take(sizeof(uint32_t) * M_max);
     const size_t o_aggoff = pl.take(sizeof(uint32_t) * (agg_tiles + 1) * M_max);
-    const size_t o_gmax = pl.take(sizeof(uint32_t) * M_max);
+    const size_t o_gmax = pl.take(sizeof(uint32_t) * 2 * M_max);
     const size_t o_S = pl.take(sizeof(unsigned long long) * kMaxLevels * ws.stat_ctas * M_max);
     const size_t o_blevel = pl.take(sizeof(int32_t) * M_max);
     ws.big_cap = d_max < (int64_t(1) << 20) ? d_max : (int64_t(1) << 20);

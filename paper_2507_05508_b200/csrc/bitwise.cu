@@ -114,7 +114,9 @@ __device__ __forceinline__ void write_signs(const uint4 (&q)[4], uint32_t* __res
 
 // ---- per-worker max |g| as an integer max over magnitude keys; flags NaN / Inf.  With given probabilities (draw != 0)
 // the worker's last block also draws the level and writes the message header.
-// KEEP 1: the largest key of every batch (kEmitGroupVecs vectors, a warp's share of a trip) is kept, and the kernels that write
+// KEEP 1: the smallest of the batches' largest keys too, behind the workers' largest keys in gmax_bits (a row of one scale has no batch
+// that rounds to 0 at any level, and its message is written without a look at them).
+// KEEP 1 and 2: the largest key of every batch (kEmitGroupVecs vectors, a warp's share of a trip) is kept, and the kernels that write
 // the message do not read the batches that round to 0 at the drawn level.  KEEP 2: what they would miss of those, the sign plane
 // of a bit-plane message, is written here too.  8 x 124M fp32 entries: 560, 566 and 620 us; what it saves the message kernels is
 // beside them.  KEEP 0, for calls that L2 holds (8 x 1M entries, bit planes: 32.2 us per step, with 2 33.4).
@@ -124,11 +126,11 @@ absmax_kernel(const T* __restrict__ g, int64_t d, int64_t ld, uint32_t* gmax_bit
               uint32_t* __restrict__ batch_max, int batches_per_worker, uint32_t* __restrict__ planes, int64_t plane_row,
               const __grid_constant__ DrawPlan pl, const __grid_constant__ DrawnLevels drawn, int draw, int* status, int* worker_err) {
     using Tr = ElemTraits<T>;
-    __shared__ uint32_t sh_max[kSweepThreads / 32];
+    __shared__ uint32_t sh_max[kSweepThreads / 32], sh_min[kSweepThreads / 32];
     pdl_enter();
     const int m = blockIdx.y, lane = threadIdx.x & 31;
     const T* row = g + (int64_t)m * ld;
-    uint32_t mx = 0;
+    uint32_t mx = 0, mn = 0xFFFFFFFFu;
     const int64_t nvec = (d + Tr::kVec - 1) / Tr::kVec, full_end = d / Tr::kVec;  // vectors of the row, and those wholly inside it
     if constexpr (KEEP == 0) {
         // Chunks of kBatch vectors per thread, all in flight before any is used, dealt round-robin to the blocks of the worker.
@@ -184,21 +186,34 @@ absmax_kernel(const T* __restrict__ g, int64_t d, int64_t ld, uint32_t* gmax_bit
             vm = __reduce_max_sync(0xFFFFFFFFu, vm);
             if (lane == 0) bmax[b] = Tr::kVec == 8 ? vm << 16 : vm;  // as the bits of an fp32 magnitude
             mx = max(mx, vm);
+            if (KEEP == 1) mn = min(mn, vm);
         }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
-    if ((threadIdx.x & 31) == 0) sh_max[threadIdx.x >> 5] = mx;
+    if ((threadIdx.x & 31) == 0) {
+        sh_max[threadIdx.x >> 5] = mx;
+        if (KEEP == 1) sh_min[threadIdx.x >> 5] = mn;
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
         for (int w = 1; w < kSweepThreads / 32; ++w) mx = max(mx, sh_max[w]);
         atomicMax(&acc[m], mx);
+        if (KEEP == 1) {
+            for (int w = 1; w < kSweepThreads / 32; ++w) mn = min(mn, sh_min[w]);
+            atomicMax(&acc[gridDim.y + m], ~mn);
+        }
     }
     if (!last_block(&done[m], gridDim.x) || threadIdx.x != 0) return;
     mx = __ldcg(&acc[m]);
     acc[m] = 0u;
     const uint32_t as_f32 = (Tr::kVec == 8) ? (mx << 16) : mx;
     gmax_bits[m] = as_f32;
+    if (KEEP == 1) {
+        mn = ~__ldcg(&acc[gridDim.y + m]);
+        acc[gridDim.y + m] = 0u;
+        gmax_bits[gridDim.y + m] = (Tr::kVec == 8) ? (mn << 16) : mn;
+    }
     if (mx >= Tr::kInfKey) {
         worker_err[m] = MLMC_ERR_NONFINITE;
         set_status(status, MLMC_ERR_NONFINITE);

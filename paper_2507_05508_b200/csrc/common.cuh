@@ -153,8 +153,8 @@ struct Workspace {
     uint32_t* cand_floor;        // [M] smallest key that can be a candidate of sweep 2 (lower edge of the lowest boundary bin)
     uint32_t* agg_offsets;       // [M][agg_tiles_max + 1]
     // bit-wise
-    uint32_t* gmax_bits;         // [M]
-    uint32_t* acc_word;          // [M] running maximum (or error flag) of a sweep; its last block leaves it at zero
+    uint32_t* gmax_bits;         // [2][M] largest key; after the first sweep of a long RTN message the smallest of the batches' largest ones
+    uint32_t* acc_word;          // [2][M] running maxima (or error flag) of a sweep; its last block leaves them at zero
     unsigned long long* S_partial;  // [M][stat_ctas][kMaxLevels]
     int stat_ctas;
     int32_t* bit_level;          // [M] drawn level of a dense message (-1: void), read by the kernel that writes it
@@ -645,8 +645,10 @@ void launch_aggregate_topk(Workspace& ws, const mlmc_topk_msgs& msgs, int M, int
 // bitwise.cu
 int configure_bit_kernels();
 void bit_limits(KernelLimits* limits);
-// Largest keys of the batches where the message kernels skip the batches that round to 0: in long sweeps.  Shorter calls lie in L2,
-// and to look first costs more than to read (8 x 1M entries, bit planes: 32.2 us per step, 33.4 with the look).
+// Largest keys of the batches where the message kernels skip the batches that round to 0: in long sweeps (above 100 MB).  us per step,
+// given p, everything read / with the look, rows in layers: bit planes 106 MB 60 / 56, 400 MB 180 / 147, 4 GB 1484 / 1161; RTN
+// 84 / 78, 271 / 237, 2478 / 2046.  Entries of one scale, where nothing is skipped: bit planes 71 / 70, 205 / 205, 1724 / 1739.
+// Shorter calls lie in L2, and to look first costs more than to read (8 x 1M entries, bit planes: 32.2 us per step, 33.4 with the look).
 inline const uint32_t* zero_batches(const Workspace& ws) { return ws.long_sweeps ? ws.tile_max : nullptr; }
 // Largest magnitude of every worker, in long sweeps of its batches too, and the NaN / Inf check; with `p` (given probabilities) also
 // the draw and the header; with `signs` (a bit-plane message, long sweeps) its sign planes, but for the ragged end of a row.

@@ -257,6 +257,11 @@ struct Residual {
         const double l = first ? 0.0 : (double)rtn_value(v, c, lo);
         return (float)((h - l) * inv_p);
     }
+    // Nothing up to this magnitude leaves anything: fl32(m inv) does not fall as m grows, 1/2 rounds to 0 (ties to even), and the
+    // level before has the coarser grid.
+    __device__ __forceinline__ bool rounds_to_zero(uint32_t magnitude) const {
+        return !(c > 0.0f) || (!top && __fmul_rn(__uint_as_float(magnitude), hi.inv) <= 0.5f);
+    }
     __device__ __forceinline__ void vector(const uint4& q, float* __restrict__ out) const {  // a vector's entries, out 16-byte aligned
         if constexpr (sizeof(T) == 4) {
             reinterpret_cast<float4*>(out)[0] = make_float4((*this)(q.x), (*this)(q.y), (*this)(q.z), (*this)(q.w));
@@ -272,7 +277,12 @@ struct Residual {
 // The dense message of the drawn level: val_i = (C^l - C^{l-1})_i / p_l, rounded to fp32 once.  A warp takes a batch (four 16-byte
 // vectors per lane) at a time.  The batches whose largest key (recorded by the first sweep) rounds to 0 at the drawn level do so
 // at the coarser level before it too: they are written, and not read.  With clipping at the row's largest magnitude that is
-// most of a row wherever its layers differ in scale (8 x 124M fp32 entries: 1290 -> 748 us).  Calls that L2 holds read everything.
+// most of a row wherever its layers differ in scale (8 x 124M fp32 entries: 1290 -> 748 us).  Calls that L2 holds read everything,
+// and so do fp32 rows of which no batch rounds to 0 (the smallest of the largest keys says so): there the looks only cost.  8 x 3.3M
+// entries of one scale 43.6 us with the looks, 37.8 without; 8 x 31M 327, 320; 8 x 124M 1300, 1293.  bf16 rows look always, at
+// the next 32 batches while 32 are written: both ways in one kernel cost them more registers than the looks cost time (8 x 62M of one
+// scale: everything read 687, both ways 700, looks 702; 8 x 25M 277, 279, 277; 8 x 6.6M 74.4, 72.4, 74.7).  fp32 with the looks ahead:
+// 8 x 124M in layers 838, 8 x 31M of one scale 324.
 template <typename T, bool SKIP>
 __global__ void __launch_bounds__(kRtnThreads)
 rtn_emit_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* gmax_bits, RtnSchedule sc,
@@ -288,7 +298,7 @@ rtn_emit_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* 
     const T* row = g + (int64_t)m * ld;
     float* out = val + (int64_t)m * ldv;
     const int64_t nvec = (d + Tr::kVec - 1) / Tr::kVec, full_end = (ldv % 4 == 0) ? d / Tr::kVec : 0;
-    if constexpr (!SKIP) {
+    if (!SKIP || (sizeof(T) == 4 && !residual.rounds_to_zero(gmax_bits[gridDim.y + m]))) {  // no batch is skipped
         // Chunks of kBatch vectors per thread, all in flight before the first is used.
         constexpr int kBatch = 4;
         for (int64_t base = (int64_t)blockIdx.x * kBatch * kRtnThreads; base < nvec; base += (int64_t)gridDim.x * kBatch * kRtnThreads) {
@@ -307,17 +317,17 @@ rtn_emit_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* 
             }
         }
     } else {
-        __shared__ int sh_zero_upto;
         const int lane = threadIdx.x & 31;
-        if (threadIdx.x == 0) sh_zero_upto = !(c > 0.0f) ? 0x7FFFFFFF : level < sc.L - 1 ? rtn_level(c, sc.r[level]).zero_upto : -1;
         const uint32_t* bmax = batch_max + (int64_t)m * batches_per_worker;
         const int64_t nbatch = (nvec + kEmitGroupVecs - 1) / kEmitGroupVecs, stride = (int64_t)gridDim.x * (kRtnThreads / 32);
-        __syncthreads();
-        const int zero_upto = sh_zero_upto;
-        // a lane looks at the largest key of one of the warp's next 32 batches
-        for (int64_t base = (int64_t)blockIdx.x * (kRtnThreads / 32) + (threadIdx.x >> 5); base < nbatch; base += 32 * stride) {
-            const int64_t own = base + lane * stride;
-            const bool zero = own < nbatch && (own + 1) * kEmitGroupVecs <= full_end && (int)bmax[own] <= zero_upto;
+        // a lane looks at the largest key of one of the warp's next 32 batches (bf16: while the 32 before are written)
+        int64_t own = (int64_t)blockIdx.x * (kRtnThreads / 32) + (threadIdx.x >> 5) + lane * stride;
+        uint32_t ahead = sizeof(T) == 2 && own < nbatch ? bmax[own] : 0u;
+        for (; own - lane * stride < nbatch; own += 32 * stride) {
+            const int64_t base = own - lane * stride;
+            const bool inside = own < nbatch && (own + 1) * kEmitGroupVecs <= full_end;
+            const bool zero = inside && residual.rounds_to_zero(sizeof(T) == 2 ? ahead : bmax[own]);
+            if (sizeof(T) == 2) ahead = own + 32 * stride < nbatch ? bmax[own + 32 * stride] : 0u;
             uint32_t todo = __ballot_sync(0xFFFFFFFFu, own < nbatch);
             const uint32_t zeros = __ballot_sync(0xFFFFFFFFu, zero);
             for (; todo; todo &= todo - 1u) {
