@@ -162,7 +162,7 @@ void select_adaptive(Workspace& ws, const void* g, int dtype, int64_t d, int M, 
                      uint64_t seed, uint64_t step, const mlmc_topk_msgs* out, cudaStream_t s) {
     FinishPlan pl = finish_plan(d, L, L - 1, true, seed, step, out);
     for (int l = 0; l < L; ++l) pl.k[l] = (uint32_t)k[l];
-    if (cluster_blocks(ws, dtype, d, M) > 0) {
+    if (cluster_blocks(ws, dtype, d, M, false) > 0) {
         launch_cluster_topk(ws, g, dtype, d, M, ld, pl, nullptr, out, s);
         return;
     }
@@ -175,7 +175,7 @@ void select_adaptive(Workspace& ws, const void* g, int dtype, int64_t d, int M, 
     if (out) launch_emit(ws, g, dtype, d, M, ld, *out, s);
 }
 
-// Longer rows use last call's boundary bins as brackets instead.
+// Longer fp32 rows use last call's boundary bins as brackets instead, where the call keeps them.
 constexpr int64_t kClusterDrawnBytes = 1 << 20;
 
 // Given p: the level of every worker is drawn here (it depends on seed, step and worker only), and the two ranks that
@@ -187,7 +187,7 @@ void select_drawn(Workspace& ws, const void* g, int dtype, int64_t d, int M, int
     DrawnBand bands[kEmitMaxWorkers];
     for (int m = 0; m < M; ++m) bands[m] = draw(counter_uniform(seed, step, (uint64_t)m));
     const FinishPlan pl = finish_plan(d, L, 2, false, seed, step, out);
-    if (d * (dtype == MLMC_BF16 ? 2 : 4) <= kClusterDrawnBytes && cluster_blocks(ws, dtype, d, M) > 0) {
+    if ((!brackets || d * (int64_t)sizeof(float) <= kClusterDrawnBytes) && cluster_blocks(ws, dtype, d, M, true) > 0) {
         launch_cluster_topk(ws, g, dtype, d, M, ld, pl, bands, out, s);
         return;
     }

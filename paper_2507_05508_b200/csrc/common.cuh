@@ -688,7 +688,7 @@ void launch_aggregate_dense(Workspace& ws, const float* val, const int32_t* leve
 // topk_cluster.cu: Top-k messages of short rows in one launch
 int configure_cluster_kernels();
 void cluster_limits(KernelLimits* limits);
-int cluster_blocks(const Workspace& ws, int dtype, int64_t d, int M);
+int cluster_blocks(const Workspace& ws, int dtype, int64_t d, int M, bool given);
 void launch_cluster_topk(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const FinishPlan& plan,
                          const DrawnBand* bands, const mlmc_topk_msgs* out, cudaStream_t s);
 // stopk_segments.cu: s-Top-k with adaptive p and many segments

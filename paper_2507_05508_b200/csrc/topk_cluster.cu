@@ -4,11 +4,15 @@
 //
 // On short rows the kernels of topk_select.cu and topk_emit.cu are chains of launches whose bodies are a few dependent
 // memory round trips each (4 workers of 65,536 entries: 60 us for 10 launches); here the row is read from memory once and
-// the steps are separated by cluster barriers (about a microsecond each).  The steps:
+// the steps are separated by cluster barriers (0.4 to 0.6 us each, with what was written before them).  Bound by the latency of
+// the steps and, in rows of more than a few thousand keys per block, by the issue of the passes over the keys.  The cluster size is
+// a constant of the kernel: loops over the blocks have all their reads in flight, and nothing is divided at run time (4 x 65,536
+// entries, given p: 22.4 us per step with a run-time size, 20.0 so).  The steps:
 //   1. the row is copied to shared memory (16-byte asynchronous copies); histogram of the leading 13 key bits, largest
 //      key per batch, NaN / Inf check;
-//   2. radix select of every query: 13 + 9 + 9 key bits (fp32) or 13 + 2 (bf16).  The bins of the first digit are divided
-//      among the blocks, later digits are counted per boundary bin and a block takes every CL-th query;
+//   2. radix select of every query: 13 + 9 + 9 key bits (fp32) or 13 + 2 (bf16).  The blocks tell one another their counts of
+//      128 ranges of bins; every block then finds the first digit of every query for itself, a warp per query that reads the
+//      bins of one range.  Later digits are counted per boundary bin;
 //   3. adaptive p: energy of the open intervals between the thresholds, mant^2 in 16-bit limbs per (interval, exponent)
 //      cell: exact, whatever the order; then p and the draw, by every block for itself (same data, same result);
 //   4. the band: counts per batch, exchanged between the blocks, then every batch is written at its final position.
@@ -29,23 +33,28 @@ constexpr int kClThreads = 1024;
 constexpr int kClMost = 16;                      // blocks per cluster (8 is the portable limit)
 constexpr int kClDigit1 = 13;
 constexpr int kClBins = 1 << kClDigit1;
+constexpr int kClRange = 64;                     // bins that are first counted together
+constexpr int kClRanges = kClBins / kClRange;
 constexpr int kClHistWords = 8192;               // 16384 16-bit counts, or the energy cells
 constexpr int kClBatches = 91;                   // batches per block at most: as much of the row (182 KB) as shared memory holds
-constexpr int kClEasy = 32;                      // batches per block from which on the cluster grows (64 KB, 16 words per thread)
+constexpr int kClBatchesBf16 = 63;               // given p, bf16: a block's keys fit 16-bit counts
+constexpr int kClSpread = 16;                    // batches per block from which on the cluster grows while all clusters run at a time,
+constexpr int kClEasy = 32;                      // and where they do not
+constexpr int kClTwoWaves = 56;                  // adaptive p, fp32: batches per block with which two waves of clusters are worth it
 constexpr int kClCells = 32 + 256;               // interval + (largest exponent - exponent)
 constexpr int kClCopiesLow = 8;                  // copies of a cell's limbs: 32 where the cells are few enough, else 8
 static_assert(kClCells * 3 * kClCopiesLow <= kClHistWords, "the cells take the place of the histogram");
-static_assert(kClBatches * kBatchWords < 65536 && kClEasy * kBatchWords * 2 < 65536, "16-bit counts, and 16-bit limbs added at most 65535 times");
+static_assert(kClBatches * kBatchWords < 65536 && kClBatchesBf16 * kBatchWords * 2 < 65536, "16-bit counts, and 16-bit limbs added at most 65535 times");
 
 struct ClusterShared {
     Query q[kMaxQueries];
     uint32_t first[kMaxQueries], slots;          // first query of a boundary bin (slot), number of slots
     int bin[kMaxQueries];                        // leading-digit bin of a query; kClBins above, -1 below every bin
-    uint32_t listed, low_bin;                    // keys of the boundary bins; lowest bin with a key
+    uint32_t low_bin;                            // first bin of the row's lowest range with a key
     double E[kMaxLevels];
     EmitParams emit;
     uint32_t top[kClMost];                       // per block: its largest key
-    uint16_t part[kClMost][kClMost];             // [block][range of bins]: the block's keys in the range
+    __align__(16) uint16_t ranges[kClRanges];    // the block's keys in the ranges of leading-digit bins
     uint4 counts[kClMost];                       // per block: {C, A, B, batches}
     uint32_t warp[32];
     uint32_t batch_max[kClBatches];
@@ -57,7 +66,7 @@ constexpr size_t kClSharedMost = 227 * 1024;
 static_assert(kClFixedSmem + kClBatches * kBatchWords * 4 + sizeof(ClusterShared) + 64 <= kClSharedMost &&
               kClFixedSmem + (kClBatches + 1) * kBatchWords * 4 + sizeof(ClusterShared) > kClSharedMost, "the most that fits");
 
-template <typename T>
+template <typename T, int CL, bool ADAPTIVE>  // CL: blocks per cluster
 __global__ void __launch_bounds__(kClThreads, 1)
 cluster_topk_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid_constant__ FinishPlan pl,
                     const __grid_constant__ DrawnList<32> drawn, int batches, int per_block, double* p_all, double* delta_all,
@@ -75,29 +84,35 @@ cluster_topk_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid
     uint32_t* sh_row = reinterpret_cast<uint32_t*>(sh_raw + kClFixedSmem);
     __shared__ ClusterShared sh;
     cg::cluster_group cluster = cg::this_cluster();
-    const int rank = (int)cluster.block_rank(), CL = (int)cluster.num_blocks();
-    const int m = blockIdx.x / CL;
+    const int rank = (int)cluster.block_rank(), m = blockIdx.x / CL;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int nq = pl.nq;
     for (int i = t; i < kClHistWords; i += kClThreads) sh_hist[i] = 0u;
-    if (t == 0) {
-        sh.listed = 0u;
-        sh.low_bin = kClBins;
-    }
-    if (t < nq) sh.q[t] = make_query(pl.adaptive ? pl.k[t] : (t ? drawn.band[m].k_hi : drawn.band[m].k_lo), d);
+    if (t < nq) sh.q[t] = make_query(ADAPTIVE ? pl.k[t] : (t ? drawn.band[m].k_hi : drawn.band[m].k_lo), d);
     cluster.barrier_arrive();
     pdl_enter();
 
-    // ---- 1. the block's batches (512 words each) into shared memory, chunks in the swizzled order of the emission
+    // ---- 1. the block's batches (512 words each) into shared memory, chunks in the swizzled order of the emission; a warp
+    // counts a batch as soon as its own copy of it has landed
     const int b0 = rank * per_block, nb = max(0, min(per_block, batches - b0));
     const T* row = g + (int64_t)m * ld;
-    for (int b = warp; b < nb; b += 32)
-        copy_batch_async<T>(row, d, (b0 + b) / kEmitGroups, (b0 + b) % kEmitGroups, lane, sh_row + b * kBatchWords);
-    cp_async_commit();
-    cp_async_wait<0>();
-    __syncthreads();
+    constexpr int kTrips = (kClBatches + 31) / 32;
+#pragma unroll
+    for (int i = 0; i < kTrips; ++i) {
+        const int b = warp + i * 32;
+        if (b < nb) copy_batch_async<T>(row, d, (b0 + b) / kEmitGroups, (b0 + b) % kEmitGroups, lane, sh_row + b * kBatchWords);
+        cp_async_commit();
+    }
+    __syncthreads();  // the counts are zero
     uint32_t my_top = 0;
-    for (int b = warp; b < nb; b += 32) {
+#pragma unroll
+    for (int i = 0; i < kTrips; ++i) {
+        const int b = warp + i * 32;
+        if (i == 0) cp_async_wait<kTrips - 1>();
+        else if (i + 1 < kTrips) cp_async_wait<1>();
+        else cp_async_wait<0>();
+        __syncwarp();
+        if (b >= nb) continue;
         const uint32_t* w = sh_row + b * kBatchWords;
         const int64_t e0 = (int64_t)(b0 + b) * kBatchWords * EW::S;
         const bool whole = e0 + kBatchWords * EW::S <= d;  // warp-uniform
@@ -108,11 +123,11 @@ cluster_topk_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid
             const uint4 q = *reinterpret_cast<const uint4*>(w + chunk * 4);
             const uint32_t x[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
+            for (int k = 0; k < 4; ++k) {
 #pragma unroll
                 for (int s = 0; s < EW::S; ++s) {
-                    const uint32_t key = EW::key(x[i], s);
-                    if (whole || e0 + (int64_t)(swz(chunk) * 4 + i) * EW::S + s < d) {  // the swizzle is its own inverse
+                    const uint32_t key = EW::key(x[k], s);
+                    if (whole || e0 + (int64_t)(swz(chunk) * 4 + k) * EW::S + s < d) {  // the swizzle is its own inverse
                         const uint32_t bin = key >> kShift1;
                         atomicAdd(&sh_hist[bin >> 1], 1u << ((bin & 1u) * 16u));
                         mx = max(mx, key);
@@ -124,26 +139,32 @@ cluster_topk_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid
         if (lane == 0) sh.batch_max[b] = mx;
         my_top = max(my_top, mx);
     }
+    static_assert(kTrips == 3, "the waits above");
+    __syncwarp();
     if (lane == 0) sh.warp[warp] = my_top;
     __syncthreads();
     my_top = __reduce_max_sync(0xFFFFFFFFu, sh.warp[lane]);
-    cluster.barrier_wait();  // every block of the cluster runs: its shared memory can be written
-    if (t < CL) cluster.map_shared_rank(sh.top, t)[rank] = my_top;
-    const int own = kClBins / CL;  // bins of the first digit that a block resolves, two per word
-    if (warp < CL) {  // warp r: how many of this block's keys lie in the range of block r
-        uint32_t n = 0, low = kClBins;
-        for (int i = lane; i < own / 2; i += 32) {
-            const uint32_t x = sh_hist[warp * (own / 2) + i];
-            n += (x & 0xFFFFu) + (x >> 16);
-            if (x) low = min(low, (uint32_t)(warp * own + 2 * i));
+    {  // the block's keys in every range of kClRange bins
+        constexpr int kPer = kClRanges / 32;
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+            const int range = warp * kPer + i;
+            const uint32_t x = sh_hist[range * (kClRange / 2) + lane];
+            const uint32_t n = __reduce_add_sync(0xFFFFFFFFu, (x & 0xFFFFu) + (x >> 16));
+            if (lane == 0) sh.ranges[range] = (uint16_t)n;
         }
-        n = __reduce_add_sync(0xFFFFFFFFu, n);
-        low = __reduce_min_sync(0xFFFFFFFFu, low);
-        if (lane < CL) cluster.map_shared_rank(&sh.part[0][0], lane)[rank * kClMost + warp] = (uint16_t)n;
-        if (lane == 0 && low < kClBins) atomicMin(&sh.low_bin, low);
     }
+    __syncthreads();
+    cluster.barrier_wait();  // every block of the cluster runs: its shared memory can be written
+    constexpr int kRangeVecs = kClRanges * 2 / 16;
+    uint4* sh_part = reinterpret_cast<uint4*>(sh_hist + kClBins / 2);  // [block][kRangeVecs]: the half of the words that the counts do not use
+    static_assert(kClHistWords - kClBins / 2 >= kClMost * kRangeVecs * 4, "the ranges of all blocks fit behind the counts");
+    if (t < CL * kRangeVecs)
+        cluster.map_shared_rank(sh_part, t / kRangeVecs)[rank * kRangeVecs + t % kRangeVecs] = reinterpret_cast<const uint4*>(sh.ranges)[t % kRangeVecs];
+    if (t < CL) cluster.map_shared_rank(sh.top, t)[rank] = my_top;
     cluster.sync();
     uint32_t top = 0;
+#pragma unroll
     for (int r = 0; r < CL; ++r) top = max(top, sh.top[r]);
     const bool bad = top >= Tr::kInfKey;
     if (rank == 0 && t == 0) {
@@ -154,75 +175,76 @@ cluster_topk_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid
             group_n[m] = 0u;
         }
     }
-    if (bad) {  // the same in every block: no barrier is left waiting
-        cluster.sync();
-        return;
-    }
+    if (bad) return;  // the same in every block; nothing of another block's memory is touched after the barrier above
 
-    // ---- 2. first digit: this block takes the bins [rank, rank + 1) * own
-    if (nq > 0) {
-        // a thread owns `span` consecutive words of the block's range (more than one only in small clusters)
-        constexpr int kMostWords = kClBins / 2 / kClThreads;
-        const int span = max(1, own / 2 / kClThreads), word = (rank * own) / 2 + t * span;
-        uint32_t c[2 * kMostWords] = {}, above = 0, sum = 0;
-        if (t * span < own / 2) {
-            if (span == 1) {
-                uint32_t x[kClMost];
+    if (ADAPTIVE && warp == kClThreads / 32 - 1) {  // without a query
+        uint32_t low = kClRanges;
 #pragma unroll
-                for (int r = 0; r < kClMost; ++r) x[r] = (r < CL) ? cluster.map_shared_rank(sh_hist, r)[word] : 0u;
-#pragma unroll
-                for (int r = 0; r < kClMost; ++r) {
-                    c[0] += x[r] & 0xFFFFu;
-                    c[1] += x[r] >> 16;
-                }
-            } else {
-                for (int r = 0; r < CL; ++r)
-#pragma unroll
-                    for (int i = 0; i < kMostWords; ++i) {
-                        const uint32_t x = i < span ? cluster.map_shared_rank(sh_hist, r)[word + i] : 0u;
-                        c[2 * i] += x & 0xFFFFu;
-                        c[2 * i + 1] += x >> 16;
-                    }
-            }
+        for (int r = 0; r < CL; ++r) {
+            const uint2 x = reinterpret_cast<const uint2*>(sh_part + r * kRangeVecs)[lane];
+            if (x.x | x.y) low = min(low, 4u * lane + (x.x & 0xFFFFu ? 0u : x.x ? 1u : x.y & 0xFFFFu ? 2u : 3u));
         }
+        low = __reduce_min_sync(0xFFFFFFFFu, low);
+        if (lane == 0) sh.low_bin = low * kClRange;
+    }
+    static_assert(kMaxQueries <= kClThreads / 32 && kMaxLevels - 1 < kClThreads / 32, "a warp per query, and one more");
+    // ---- 2. first digit: a warp per query, in every block alike.  The range that holds the rank, then its bins, of which the
+    // counts come from all blocks at a time.  (With the bins divided among the blocks, a scan of them by all threads, and a
+    // barrier for the answers, the step took 2.9 us in 4 blocks and 4.5 in 16, now 0.8 and 2.7.)
+    if (warp < nq && sh.q[warp].trivial == 0u) {
+        const uint32_t k = sh.q[warp].k;
+        uint32_t c[4] = {};  // of ranges kClRanges - 1 - 4 lane, and down
 #pragma unroll
-        for (int i = 0; i < 2 * kMostWords; ++i) sum += c[i];
-        // keys in the ranges above this block's, then in the block's bins above this thread's
-        for (int i = lane; i < CL * kClMost; i += 32) above += (i % kClMost > rank && i % kClMost < CL) ? sh.part[i / kClMost][i % kClMost] : 0u;
-        above = __reduce_add_sync(0xFFFFFFFFu, above);
-        uint32_t suffix = sum;
+        for (int r = 0; r < CL; ++r) {
+            const uint2 x = reinterpret_cast<const uint2*>(sh_part + r * kRangeVecs)[31 - lane];
+            c[0] += x.y >> 16; c[1] += x.y & 0xFFFFu; c[2] += x.x >> 16; c[3] += x.x & 0xFFFFu;
+        }
+        static_assert(kClRanges == 128 && kClRange == 64, "four ranges per lane, two bins per lane");
+        uint32_t upto = c[0] + c[1] + c[2] + c[3], sum = upto;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_down_sync(0xFFFFFFFFu, suffix, o);
-            if (lane + o < 32) suffix += y;
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, upto, o);
+            if (lane >= o) upto += y;
         }
-        __syncthreads();  // sh.warp has been read
-        if (lane == 0) sh.warp[warp] = suffix;
-        __syncthreads();
-        above += suffix - sum + __reduce_add_sync(0xFFFFFFFFu, lane > warp ? sh.warp[lane] : 0u);
-        if (sum) {
-            for (int j = 0; j < nq; ++j) {
-                const uint32_t k = sh.q[j].k;
-                if (above < k && k <= above + sum && sh.q[j].trivial == 0u) {  // this thread's bins hold rank k
-                    uint32_t bin = 0, ab = 0, run = above;
+        int from = __ffs(__ballot_sync(0xFFFFFFFFu, upto >= k)) - 1;  // the first lane that reaches the rank
+        uint32_t run = upto - sum, above = 0, range = 0;
 #pragma unroll
-                    for (int i = 2 * kMostWords - 1; i >= 0; --i) {  // the last bin that is entered holds the rank
-                        if (run < k) {
-                            bin = (uint32_t)(2 * word + i);
-                            ab = run;
-                        }
-                        run += c[i];
-                    }
-                    for (int r = 0; r < CL; ++r) {
-                        Query& q = cluster.map_shared_rank(sh.q, r)[j];
-                        q.prefix = bin << kShift1;
-                        q.rem = k - ab;
-                    }
-                }
+        for (int i = 0; i < 4; ++i) {  // the last range that is entered holds the rank
+            if (run < k) {
+                above = run;
+                range = (uint32_t)(kClRanges - 1 - 4 * lane - i);
             }
+            run += c[i];
         }
-        cluster.sync();
+        above = __shfl_sync(0xFFFFFFFFu, above, from);
+        range = __shfl_sync(0xFFFFFFFFu, range, from);
+        const int word = (int)range * (kClRange / 2) + 31 - lane;
+        uint32_t x[CL], hi = 0, lo = 0;
+#pragma unroll
+        for (int r = 0; r < CL; ++r) x[r] = cluster.map_shared_rank(sh_hist, r)[word];
+#pragma unroll
+        for (int r = 0; r < CL; ++r) {
+            hi += x[r] >> 16;
+            lo += x[r] & 0xFFFFu;
+        }
+        upto = sum = hi + lo;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, upto, o);
+            if (lane >= o) upto += y;
+        }
+        upto += above;
+        from = __ffs(__ballot_sync(0xFFFFFFFFu, upto >= k)) - 1;
+        if (lane == from) {
+            run = upto - sum;
+            const bool second = run + hi < k;
+            sh.q[warp].prefix = (uint32_t)(2 * word + (second ? 0 : 1)) << kShift1;
+            sh.q[warp].rem = k - run - (second ? hi : 0u);
+        }
     }
+    __syncwarp();
+    cluster.barrier_arrive();  // the block has read the others' counts; waited for before its own are cleared
+    __syncthreads();
     // The live queries are contiguous (k = 0 before them, k >= d after them) and their prefixes descend: queries with the
     // same prefix share a histogram slot, numbered by the first of them.  By warp 0, a query per lane.
     auto number_slots = [&](bool first_digit) {
@@ -240,9 +262,8 @@ cluster_topk_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid
         }
     };
     if (warp == 0) number_slots(true);
-    for (int i = t; i < kClHistWords; i += kClThreads) sh_hist[i] = 0u;
     __syncthreads();
-    {
+    if constexpr (ADAPTIVE) {
         // codes of the bins: 64 + slot where a boundary lies in the bin, else the number of boundaries above it
         constexpr int per = kClBins / kClThreads;  // 8 consecutive bins per thread
         const int hi_bin = t * per + per - 1;
@@ -266,6 +287,16 @@ cluster_topk_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid
         }
         reinterpret_cast<uint2*>(sh_tab)[t] = make_uint2(codes[0], codes[1]);
     }
+    cluster.barrier_wait();
+    // Two more digits (bf16: one) are counted per slot.  Few queries in small clusters: every block resolves all of them for
+    // itself, and the third digit has counts of its own, so that nothing is exchanged but the counts.  Otherwise a block
+    // resolves every CL-th query and tells the others, and the third digit takes the place of the second.
+    const uint32_t hist_words = ((max(sh.slots << kBits2, (uint32_t)nq << kShift2) / 2 + 3u) & ~3u);
+    const bool alike = nq * 2 * CL <= 2 * (kClThreads / 32) && 4u * hist_words <= (uint32_t)kClHistWords;
+    uint32_t* const sh_count2 = sh_hist;
+    uint32_t* const sh_count3 = alike ? sh_hist + hist_words : sh_hist;
+    const uint32_t list_from = alike ? 2u * hist_words : hist_words;
+    for (uint32_t i = t; i < list_from; i += kClThreads) sh_hist[i] = 0u;
     __syncthreads();
     const int words4 = nb * kBatchWords / 4;
     // every key of the block's words (place: its element number in shared memory); the padding past the row's end has
@@ -280,134 +311,193 @@ cluster_topk_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid
                 for (int s = 0; s < EW::S; ++s) f(EW::key(x[c], s), (uint32_t)((i * 4 + c) * EW::S + s));
         }
     };
-    // The places of the keys in boundary bins are listed by the first pass over them, behind the counts (two digits of at
-    // most `slots` slots), as far as they fit; otherwise the passes after it look at every key again.
-    const uint32_t hist_words = (sh.slots << kBits2) / 2 > (uint32_t)(nq << kShift2) / 2 ? (sh.slots << kBits2) / 2 : (uint32_t)(nq << kShift2) / 2;
-    uint16_t* sh_list = reinterpret_cast<uint16_t*>(sh_hist + ((hist_words + 3u) & ~3u));
-    const uint32_t list_cap = 2u * (kClHistWords - ((hist_words + 3u) & ~3u));
+    // Slot of a boundary bin, 64 or more (64 less in `slot_of`) for the keys of other bins.  Given p: two bins.
+    uint32_t bin_of[2], slot_of_bin[2];
+    if constexpr (!ADAPTIVE)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const bool live = j < nq && sh.q[j].trivial == 0u;
+            bin_of[j] = live ? sh.q[j].prefix >> kShift1 : 0xFFFFFFFFu;
+            slot_of_bin[j] = live ? sh.q[j].slot2 : 0u;
+        }
+    auto slot_of = [&](uint32_t key, uint32_t& slot) -> bool {
+        if constexpr (ADAPTIVE) {
+            const uint32_t code = sh_tab[key >> kShift1];
+            slot = code - 64u;
+            return code >= 64u;
+        } else {
+            const uint32_t bin = key >> kShift1;
+            slot = bin == bin_of[0] ? slot_of_bin[0] : slot_of_bin[1];
+            return bin == bin_of[0] || bin == bin_of[1];
+        }
+    };
+    // The places of the keys in boundary bins are listed by the first pass over them, behind the counts, every warp its own; a
+    // warp whose list is too short looks at all its keys again.
+    const uint32_t list_cap = 2u * (kClHistWords - list_from) / (kClThreads / 32);
+    uint16_t* const list = reinterpret_cast<uint16_t*>(sh_hist + list_from) + warp * list_cap;
+    uint32_t listed = 0;  // warp-uniform
     auto key_at = [&](uint32_t place) -> uint32_t { return EW::key(sh_row[place / EW::S], place % EW::S); };
     auto for_each_boundary_key = [&](auto&& f) {
-        const uint32_t n = sh.listed;
-        if (n <= list_cap) {
-            for (uint32_t i = t; i < n; i += kClThreads) f(key_at(sh_list[i]));
+        uint32_t slot;
+        if (listed <= list_cap) {
+            for (uint32_t i = lane; i < listed; i += 32) {
+                const uint32_t key = key_at(list[i]);
+                slot_of(key, slot);
+                f(key, slot);
+            }
         } else {
             for_each_key([&](uint32_t key, uint32_t) {
-                if (sh_tab[key >> kShift1] >= 64u) f(key);
+                if (slot_of(key, slot)) f(key, slot);
             });
         }
     };
-    // One more digit of every query: `bits` bits at `shift`, counted per slot.  Warp w of block r takes query r + w CL: a
-    // lane adds up its share of the slot's counts over the blocks, the warp finds the digit and tells every block.
-    auto descend = [&](auto bits_tag, int shift, bool last) {
-        constexpr int bits = decltype(bits_tag)::value;
-        constexpr int words = (1 << bits) / 2 < 32 ? (1 << bits) / 2 : 32;  // lanes with counts
-        constexpr int per = (1 << bits) / 2 / words;                       // words per lane: 8 (9 bits) or 1 (2 bits)
-        cluster.sync();  // every block's counts are complete
-        const int j = rank + warp * CL;
-        if (j < nq && sh.q[j].trivial == 0u) {
-            const int base = (int)(sh.q[j].slot << bits) / 2 + (words - 1 - lane) * per;  // lane 0 owns the largest digits
-            uint32_t c[2 * per] = {}, sum = 0;
-            if (lane < words) {
-                for (int r = 0; r < CL; ++r) {
-                    const uint32_t* src = cluster.map_shared_rank(sh_hist, r) + base;
-                    if constexpr (per == 8) {
-                        const uint4 a = reinterpret_cast<const uint4*>(src)[0], b = reinterpret_cast<const uint4*>(src)[1];
-                        const uint32_t x[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            c[2 * i] += x[i] & 0xFFFFu;
-                            c[2 * i + 1] += x[i] >> 16;
-                        }
-                    } else {
-                        c[0] += src[0] & 0xFFFFu;
-                        c[1] += src[0] >> 16;
-                    }
-                }
-            }
-#pragma unroll
-            for (int i = 0; i < 2 * per; ++i) sum += c[i];
-            uint32_t upto = sum;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, upto, o);
-                if (lane >= o) upto += y;
-            }
-            const uint32_t rem = sh.q[j].rem;
-            uint32_t run = upto - sum, digit = 0, left = 0, n = 0;
-            const bool mine = run < rem && rem <= upto;
-#pragma unroll
-            for (int i = 2 * per - 1; i >= 0; --i) {
-                if (run < rem) {  // the last digit that is entered holds the rank
-                    digit = (uint32_t)((words - 1 - lane) * per * 2 + i);
-                    left = rem - run;
-                    n = c[i];
-                }
-                run += c[i];
-            }
-            const int from = __ffs(__ballot_sync(0xFFFFFFFFu, mine)) - 1;
-            digit = __shfl_sync(0xFFFFFFFFu, digit, from);
-            left = __shfl_sync(0xFFFFFFFFu, left, from);
-            n = __shfl_sync(0xFFFFFFFFu, n, from);
-            const uint32_t prefix = sh.q[j].prefix | (digit << shift), k = sh.q[j].k;
-            __syncwarp();
-            if (lane < CL) {
-                Query& q = cluster.map_shared_rank(sh.q, lane)[j];
-                q.prefix = prefix;
-                q.rem = left;
-                if (last) {
-                    q.T = prefix;
-                    q.r = left;
-                    q.n = n;
-                    q.c = k - left;
-                }
+    // One more digit of the queries, `bits` bits at `shift`.  2 CL warps take a query: a lane has eight of the 512 digits (a
+    // 16-byte vector) in one block, the lanes of one vector add up over the blocks, and the warp whose digits hold the rank tells
+    // this block or, where the blocks divide the queries, all of them.  (A warp per query that reads block after block: 6.7 and
+    // 4.3 us for the two digits of 14 queries in 16 blocks.)  Digits of 2 bits: a warp per query, a block per lane.
+    auto found = [&](int j, uint32_t prefix, uint32_t left, uint32_t n, bool last, bool tell_all) {  // by a whole warp
+        const uint32_t k = sh.q[j].k;
+        if (lane < (tell_all ? CL : 1)) {
+            Query& q = tell_all ? cluster.map_shared_rank(sh.q, lane)[j] : sh.q[j];
+            q.prefix = prefix;
+            q.rem = left;
+            if (last) {
+                q.T = prefix;
+                q.r = left;
+                q.n = n;
+                q.c = k - left;
             }
         }
-        cluster.sync();
     };
-    auto count = [&](uint32_t i) { atomicAdd(&sh_hist[i >> 1], 1u << ((i & 1u) * 16u)); };
+    auto descend = [&](auto bits_tag, int shift, bool last, uint32_t* counts) {
+        constexpr int bits = decltype(bits_tag)::value;
+        cluster.sync();  // every block's counts are complete
+        if constexpr (bits == 2) {
+            if (warp < nq && sh.q[warp].trivial == 0u) {
+                uint2 x = make_uint2(0u, 0u);
+                if (lane < CL) x = reinterpret_cast<const uint2*>(cluster.map_shared_rank(counts, lane))[sh.q[warp].slot];
+                const uint32_t c[4] = {__reduce_add_sync(0xFFFFFFFFu, x.x & 0xFFFFu), __reduce_add_sync(0xFFFFFFFFu, x.x >> 16),
+                                       __reduce_add_sync(0xFFFFFFFFu, x.y & 0xFFFFu), __reduce_add_sync(0xFFFFFFFFu, x.y >> 16)};
+                uint32_t left = sh.q[warp].rem, digit = 3, n = c[3];
+#pragma unroll
+                for (int e = 3; e > 0; --e)
+                    if (digit == (uint32_t)e && left > c[e]) {
+                        left -= c[e];
+                        n = c[e - 1];
+                        digit = (uint32_t)e - 1u;
+                    }
+                __syncwarp();
+                found(warp, sh.q[warp].prefix | (digit << shift), left, n, last, false);
+            }
+            __syncthreads();
+        } else {
+            static_assert(bits == 9, "64 vectors of eight counts");
+            constexpr int warps_each = 2 * CL, at_a_time = (kClThreads / 32) / warps_each;
+            const int part = warp % warps_each;
+            constexpr int vecs = 32 / CL;  // per warp and block
+            const int mine = alike ? nq : (nq - rank + CL - 1) / CL;
+            for (int i0 = 0; i0 < mine; i0 += at_a_time) {
+                const int i = i0 + warp / warps_each, j = alike ? i : rank + i * CL;
+                const bool live = i < mine && sh.q[j].trivial == 0u;
+                uint32_t c[8] = {}, rem = 0;  // digits 8 v + 7 .. 8 v
+                const int v = 63 - (part * vecs + lane % vecs);
+                if (live) {
+                    const uint4 x = reinterpret_cast<const uint4*>(cluster.map_shared_rank(counts, lane / vecs))[sh.q[j].slot * 64u + v];
+                    c[0] = x.w >> 16; c[1] = x.w & 0xFFFFu; c[2] = x.z >> 16; c[3] = x.z & 0xFFFFu;
+                    c[4] = x.y >> 16; c[5] = x.y & 0xFFFFu; c[6] = x.x >> 16; c[7] = x.x & 0xFFFFu;
+                    rem = sh.q[j].rem;
+                }
+#pragma unroll
+                for (int o = vecs; o < 32; o <<= 1)
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) c[e] += __shfl_xor_sync(0xFFFFFFFFu, c[e], o);
+                uint32_t sum = 0;
+#pragma unroll
+                for (int e = 0; e < 8; ++e) sum += c[e];
+                uint32_t upto = sum;  // over the vectors of the warp
+#pragma unroll
+                for (int o = 1; o < vecs; o <<= 1) {
+                    const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, upto, o, vecs);
+                    if (lane % vecs >= o) upto += y;
+                }
+                if (lane == vecs - 1) sh.warp[warp] = upto;
+                __syncthreads();
+                uint32_t run = upto - sum + __reduce_add_sync(0xFFFFFFFFu, lane < part ? sh.warp[warp - part + lane] : 0u);
+                const bool here = live && run < rem && rem <= run + sum;
+                const uint32_t from = __ballot_sync(0xFFFFFFFFu, here);  // a lane of every block, or none
+                if (from) {
+                    uint32_t digit = 0, left = 0, n = 0;
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {  // the last digit that is entered holds the rank
+                        if (run < rem) {
+                            digit = (uint32_t)(8 * v + 7 - e);
+                            left = rem - run;
+                            n = c[e];
+                        }
+                        run += c[e];
+                    }
+                    const int f = __ffs(from) - 1;
+                    digit = __shfl_sync(0xFFFFFFFFu, digit, f);
+                    left = __shfl_sync(0xFFFFFFFFu, left, f);
+                    n = __shfl_sync(0xFFFFFFFFu, n, f);
+                    const uint32_t prefix = sh.q[j].prefix | (digit << shift);
+                    __syncwarp();
+                    found(j, prefix, left, n, last, !alike);
+                }
+                __syncthreads();  // sh.warp has been read
+            }
+            if (!alike) cluster.sync();
+        }
+    };
+    auto count = [&](uint32_t* counts, uint32_t i) { atomicAdd(&counts[i >> 1], 1u << ((i & 1u) * 16u)); };
     if (nq > 0) {
         for_each_key([&](uint32_t key, uint32_t place) {
-            const uint32_t code = sh_tab[key >> kShift1];
-            if (code >= 64u) {
-                count(((code - 64u) << kBits2) | ((key >> kShift2) & ((1u << kBits2) - 1u)));
-                const uint32_t at = atomicAdd(&sh.listed, 1u);
-                if (at < list_cap) sh_list[at] = (uint16_t)place;
+            uint32_t slot;
+            const bool hit = slot_of(key, slot);
+            const uint32_t hits = __ballot_sync(0xFFFFFFFFu, hit);
+            if (hits == 0u) return;
+            if (hit) {
+                count(sh_count2, (slot << kBits2) | ((key >> kShift2) & ((1u << kBits2) - 1u)));
+                const uint32_t at = listed + (uint32_t)__popc(hits & ((1u << lane) - 1u));
+                if (at < list_cap) list[at] = (uint16_t)place;
             }
+            listed += (uint32_t)__popc(hits);
         });
-        descend(std::integral_constant<int, kBits2>(), kShift2, kShift2 == 0);
+        descend(std::integral_constant<int, kBits2>(), kShift2, kShift2 == 0, sh_count2);
         if constexpr (kShift2 > 0) {
             if (warp == 0) number_slots(false);
-            for (uint32_t i = t; i < hist_words; i += kClThreads) sh_hist[i] = 0u;
+            if (!alike)
+                for (uint32_t i = t; i < hist_words; i += kClThreads) sh_hist[i] = 0u;
             __syncthreads();
-            for_each_boundary_key([&](uint32_t key) {
-                const uint32_t s = sh_tab[key >> kShift1] - 64u;
+            for_each_boundary_key([&](uint32_t key, uint32_t s) {
                 for (int j = (int)sh.first[s]; j < nq && sh.q[j].trivial == 0u && sh.q[j].slot2 == s; ++j) {
                     if ((sh.q[j].prefix >> kShift2) == (key >> kShift2)) {
-                        count((sh.q[j].slot << kShift2) | (key & ((1u << kShift2) - 1u)));
+                        count(sh_count3, (sh.q[j].slot << kShift2) | (key & ((1u << kShift2) - 1u)));
                         break;
                     }
                 }
             });
-            descend(std::integral_constant<int, (kShift2 > 0 ? kShift2 : 2)>(), 0, true);
+            descend(std::integral_constant<int, (kShift2 > 0 ? kShift2 : 9)>(), 0, true, sh_count3);
         }
+        cluster.barrier_arrive();  // the block has read the others' counts
     }
 
     // ---- 3. energies of the open intervals
-    if (pl.adaptive) {
+    if constexpr (ADAPTIVE) {
         // A cell is (interval, exponent), numbered interval + (largest exponent - exponent): neither falls as the keys fall.
         auto exponent = [&](uint32_t key) -> int { return (int)((Tr::kVec == 4 ? key : key << 16) >> 23); };
         const int top_e = exponent(top);
-        const int span = nq + 1 + top_e - exponent(min(sh.low_bin, (uint32_t)kClBins - 1u) << kShift1);  // cells of this block
+        const int low_e = exponent(sh.low_bin << kShift1), span = nq + 1 + top_e - low_e;  // cells
         const bool many = span * 3 * 32 > kClHistWords;
         const int copies = many ? kClCopiesLow : 32, copy = lane & (copies - 1);
         // the keys of the boundary bins first, while their list is intact: their cells wait in a register each
         __syncthreads();
-        const uint32_t nlist = sh.listed;
-        const bool by_list = nq > 0 && nlist <= list_cap && nlist <= 8u * kClThreads;
+        const bool by_list = listed <= list_cap && listed <= 8u * 32u;  // warp by warp
         uint32_t held[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) held[i] = (by_list && (uint32_t)(t + i * kClThreads) < nlist) ? sh_list[t + i * kClThreads] : 0xFFFFFFFFu;
+        for (int i = 0; i < 8; ++i) held[i] = (by_list && (uint32_t)(lane + i * 32) < listed) ? list[lane + i * 32] : 0xFFFFFFFFu;
         __syncthreads();
+        if (nq > 0) cluster.barrier_wait();
         for (int i = t; i < kClHistWords; i += kClThreads) sh_hist[i] = 0u;
         __syncthreads();
         auto add = [&](uint32_t interval, uint32_t key) {
@@ -454,12 +544,12 @@ cluster_topk_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid
         }
         cluster.sync();
         double* sh_cell = reinterpret_cast<double*>(sh_hist);  // [kClCells]: sum of mant^2 over the row
-        if (t < 2 * kClCells) {  // thread 2 c + h adds half h of cell c over the blocks
-            unsigned long long x[kClMost], sum = 0;
+        if (t < 2 * kClCells && (t & ~31) < 2 * span) {  // thread 2 c + h adds half h of cell c over the blocks
+            unsigned long long x[CL], sum = 0;
 #pragma unroll
-            for (int r = 0; r < kClMost; ++r) x[r] = (r < CL) ? cluster.map_shared_rank(sh_sum, r)[t] : 0ull;
+            for (int r = 0; r < CL; ++r) x[r] = cluster.map_shared_rank(sh_sum, r)[t];
 #pragma unroll
-            for (int r = 0; r < kClMost; ++r) sum += x[r];
+            for (int r = 0; r < CL; ++r) sum += x[r];
             const unsigned long long hi = __shfl_down_sync(0xFFFFFFFFu, sum, 1);
             const unsigned __int128 tot = ((unsigned __int128)hi << 32) + sum;
             if ((t & 1) == 0) sh_cell[t >> 1] = (double)(unsigned long long)(tot >> 64) * 0x1.0p64 + (double)(unsigned long long)tot;
@@ -471,7 +561,7 @@ cluster_topk_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid
             const uint32_t T_up = l ? sh.q[l - 1].T : kKeyNone, T_dn = l < nq ? sh.q[l].T : 0u;
             const int e_hi = T_up == kKeyNone ? top_e : exponent(T_up), e_lo = T_dn == kKeyNone ? 255 : exponent(T_dn);
             double e = 0.0;
-            for (int x = e_hi - lane; x >= e_lo; x -= 32) {
+            for (int x = e_hi - lane; x >= max(e_lo, low_e); x -= 32) {
                 const double c = sh_cell[l + top_e - x];
                 if (c != 0.0) e += ldexp(c, 2 * ((x ? x : 1) - 150));
             }
@@ -481,9 +571,10 @@ cluster_topk_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid
         }
         __syncthreads();
     }
+    if (!ADAPTIVE && nq > 0) cluster.barrier_wait();
     {
-        const int level = pl.adaptive ? 0 : drawn.band[m].level;
-        const double p_sel = pl.adaptive ? 0.0 : drawn.band[m].p;
+        const int level = ADAPTIVE ? 0 : drawn.band[m].level;
+        const double p_sel = ADAPTIVE ? 0.0 : drawn.band[m].p;
         finish_selection(pl, m, Tr::kVec == 8, sh.q, sh.E, p_all, delta_all, level, p_sel, &sh.emit, status, worker_err);
     }
     if (!pl.want_emit) {
@@ -496,11 +587,9 @@ cluster_topk_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid
     const EmitParams ep = sh.emit;
     const bool on = ep.enabled && ep.expect > 0u;  // the same in every block
     const Band band = {min(ep.Tb, EW::kCap), min(ep.Ta, EW::kCap), ep.ra, ep.rb, (float)ep.inv_p};
-    uint32_t nC = 0, nA = 0, nB = 0, listed = 0;  // of this warp's batches
     for (int b = warp; b < nb; b += 32) {
         uint32_t bC = 0, bA = 0, bB = 0;
         if (on && sh.batch_max[b] >= band.Tb) {
-            ++listed;
             uint32_t cur[kEmitRows];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
@@ -519,22 +608,25 @@ cluster_topk_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid
             sh.batch_a[b] = (uint16_t)bA;
             sh.batch_b[b] = (uint16_t)bB;
         }
-        nC += bC; nA += bA; nB += bB;
-    }
-    // the block's totals, by four warps' worth of shared words
-    __shared__ uint32_t sh_tot[4];
-    if (t < 4) sh_tot[t] = 0u;
-    __syncthreads();
-    if (lane == 0) {
-        if (nC) atomicAdd(&sh_tot[0], nC);
-        if (nA) atomicAdd(&sh_tot[1], nA);
-        if (nB) atomicAdd(&sh_tot[2], nB);
-        if (listed) atomicAdd(&sh_tot[3], listed);
     }
     __syncthreads();
-    if (t < CL) cluster.map_shared_rank(sh.counts, t)[rank] = make_uint4(sh_tot[0], sh_tot[1], sh_tot[2], sh_tot[3]);
+    if (warp == 0) {  // the block's totals, to every block
+        uint32_t nC = 0, nA = 0, nB = 0, listed = 0;
+        for (int b = lane; b < nb; b += 32) {
+            nC += sh.batch_c[b];
+            nA += sh.batch_a[b];
+            nB += sh.batch_b[b];
+            listed += (on && sh.batch_max[b] >= band.Tb) ? 1u : 0u;
+        }
+        nC = __reduce_add_sync(0xFFFFFFFFu, nC);
+        nA = __reduce_add_sync(0xFFFFFFFFu, nA);
+        nB = __reduce_add_sync(0xFFFFFFFFu, nB);
+        listed = __reduce_add_sync(0xFFFFFFFFu, listed);
+        if (lane < CL) cluster.map_shared_rank(sh.counts, lane)[rank] = make_uint4(nC, nA, nB, listed);
+    }
     cluster.sync();  // also: nothing of another block's memory is read after this
     uint4 before = make_uint4(0u, 0u, 0u, 0u), all = before;
+#pragma unroll
     for (int r = 0; r < CL; ++r) {
         const uint4 x = sh.counts[r];
         if (r < rank) { before.x += x.x; before.y += x.y; before.z += x.z; }
@@ -568,43 +660,71 @@ size_t cluster_smem(int per_block) { return kClFixedSmem + (size_t)per_block * k
 
 }  // namespace
 
+// f(cluster size as a constant) for the size 2^i.
+template <typename F>
+static auto with_cluster(int i, F&& f) {
+    switch (i) {
+        case 0: return f(std::integral_constant<int, 1>());
+        case 1: return f(std::integral_constant<int, 2>());
+        case 2: return f(std::integral_constant<int, 4>());
+        case 3: return f(std::integral_constant<int, 8>());
+        default: return f(std::integral_constant<int, 16>());
+    }
+}
+
 int configure_cluster_kernels() {
     auto set = [&](auto kernel) {
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cluster_smem(kClBatches)) != cudaSuccess) return false;
         return cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
     };
-    return set(cluster_topk_kernel<float>) && set(cluster_topk_kernel<bf16_t>) ? MLMC_OK : MLMC_ERR_CUDA;
+    for (int i = 0; i < 5; ++i)
+        if (!with_cluster(i, [&](auto cl) { 
+                return set(cluster_topk_kernel<float, cl(), true>) && set(cluster_topk_kernel<float, cl(), false>) &&
+                       set(cluster_topk_kernel<bf16_t, cl(), true>) && set(cluster_topk_kernel<bf16_t, cl(), false>);
+            }))
+            return MLMC_ERR_CUDA;
+    return MLMC_OK;
 }
 
-void cluster_limits(KernelLimits* limits) { clusters_that_fit(cluster_topk_kernel<float>, kClThreads, cluster_smem(kClBatches), limits->topk_fit); }
+void cluster_limits(KernelLimits* limits) {  // the kernels of all sizes take the same shared memory, and one block per SM
+    clusters_that_fit(cluster_topk_kernel<float, 16, true>, kClThreads, cluster_smem(kClBatches), limits->topk_fit);
+}
 
 // Blocks per cluster for this call, 0: the row is too long, or the workers are too many, for the cluster to be the faster way.
-// The smallest cluster whose blocks have at most kClEasy batches: a barrier and an exchange between more blocks take longer
-// than the work that they share out.  Clusters that do not fit the GPU at a time run one after the other, where the launch
-// chain has the whole GPU: two waves are worth it for fp32 rows whose blocks are not stretched beyond kClEasy batches, three never.
-// bf16 rows (whose chain needs one sweep) only in one wave and not stretched.  us per call, cluster / chain, layered rows:
-//   fp32, adaptive     131k x 12 33 / 77, x 16 (two waves) 61 / 77, x 32 (three) 93 / 90; 262k x 8 (two) 75 / 75, x 16 (three)
-//                      112 / 83; 700k x 4 58 / 78, x 8 (two, stretched) 105 / 89, x 32 258 / 134
-//   fp32, given p      262k x 4 24 / 54, x 8 (two) 46 / 55, x 16 (three) 68 / 60
-//   bf16, adaptive     262k x 12 50 / 56, x 16 (two) 68 / 58; 500k x 4 46 / 51; 700k x 4 (stretched) 59 / 53, x 32 236 / 85
-//   bf16, given p      500k x 4 22 / 36, x 8 (two) 40 / 36, x 32 99 / 55
-int cluster_blocks(const Workspace& ws, int dtype, int64_t d, int M) {
+// kClSpread batches per block while the clusters of all workers run at a time, else kClEasy (4 x 65,536 entries, given p: 18.9 us per
+// step on 8 blocks, 20.0 on 4, where M clusters of 16 would not fit 131k x 8 takes 63 us on 16 and 36 on 8); longer rows are
+// stretched over 16 blocks.  Clusters that do not fit the GPU at a time run one after the other, where the launch chain has the
+// whole GPU: how far that pays depends on what the chain has to do.  us per step, cluster / chain, layered rows:
+//   fp32, adaptive  700k x 3 53 / 76, 400k x 6 46 / 79; two waves 262k x 8 63 / 78, 400k x 12 82 / 90, 700k x 8 100 / 89; three
+//                   262k x 16 95 / 90, 131k x 32 93 / 100
+//   fp32, given p   700k x 3 34 / 56, 700k x 6 39 / 60; two waves 262k x 8 43 / 56, 500k x 8 52 / 60, 700k x 12 67 / 69; three
+//                   262k x 16 67 / 64
+//   bf16, adaptive  500k x 4 47 / 53, 700k x 4 61 / 55, 1M x 3 70 / 54; two waves 500k x 8 75 / 58
+//   bf16, given p   500k x 4 23 / 33, 1M x 3 30 / 36; two waves 500k x 8 38 / 39, 1M x 8 53 / 45
+int cluster_blocks(const Workspace& ws, int dtype, int64_t d, int M, bool given) {
     const int64_t batches = (int64_t)emit_tiles_per_worker(d, dtype) * kEmitGroups;
     if (M > 32) return 0;
     int i = 0;
-    while (i < 4 && ws.limits.topk_fit[i + 1] > 0 && batches > (int64_t)kClEasy << i) ++i;
+    while (i < 4 && ws.limits.topk_fit[i + 1] > 0 && batches > (int64_t)(M <= ws.limits.topk_fit[i + 1] ? kClSpread : kClEasy) << i) ++i;
     const int fit = ws.limits.topk_fit[i];
     if (fit == 0) return 0;
     const int64_t per = (batches + (1 << i) - 1) >> i;
     const int waves = (M + fit - 1) / fit;
-    const int64_t most = dtype == MLMC_BF16 ? (waves == 1 ? kClEasy : 0) : waves == 1 ? kClBatches : waves == 2 ? kClEasy : 0;
+    int64_t most = 0;
+    if (dtype == MLMC_BF16) {
+        if (given) most = waves == 1 ? kClBatchesBf16 : waves == 2 ? kClEasy : 0;
+        else most = waves == 1 ? kClEasy : 0;
+    } else {
+        if (given) most = waves <= 2 ? kClBatches : 0;
+        else most = waves == 1 ? kClBatches : waves == 2 ? kClTwoWaves : 0;
+    }
     return per <= most ? 1 << i : 0;
 }
 
 void launch_cluster_topk(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const FinishPlan& plan,
                          const DrawnBand* bands, const mlmc_topk_msgs* out, cudaStream_t s) {
     const int tiles = emit_tiles_per_worker(d, dtype);
-    const int batches = tiles * kEmitGroups, cl = cluster_blocks(ws, dtype, d, M), per = (batches + cl - 1) / cl;
+    const int batches = tiles * kEmitGroups, cl = cluster_blocks(ws, dtype, d, M, bands != nullptr), per = (batches + cl - 1) / cl;
     if (out) ws.last_emit_tiles = tiles;
     DrawnList<32> drawn = {};
     if (bands)
@@ -614,8 +734,12 @@ void launch_cluster_topk(Workspace& ws, const void* g, int dtype, int64_t d, int
                               batches, per, ws.p_all, ws.delta_all, out ? out->idx : nullptr, out ? out->val : nullptr, ws.group_n,
                               ws.status, ws.worker_err);
     };
-    if (dtype == MLMC_BF16) go(cluster_topk_kernel<bf16_t>, static_cast<const bf16_t*>(g));
-    else go(cluster_topk_kernel<float>, static_cast<const float*>(g));
+    int log2 = 0;
+    while (1 << log2 < cl) ++log2;
+    with_cluster(log2, [&](auto size) {
+        if (dtype == MLMC_BF16) go(bands ? cluster_topk_kernel<bf16_t, size(), false> : cluster_topk_kernel<bf16_t, size(), true>, static_cast<const bf16_t*>(g));
+        else go(bands ? cluster_topk_kernel<float, size(), false> : cluster_topk_kernel<float, size(), true>, static_cast<const float*>(g));
+    });
 }
 
 }  // namespace mlmc

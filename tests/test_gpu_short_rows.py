@@ -1,7 +1,10 @@
-"""The average of short Top-k messages in one launch."""
+"""Short Top-k rows: the cluster kernel at every cluster size, and the average in one launch."""
 import numpy as np
 import pytest
 import torch
+
+from test_gpu_dispatch import doubling, geometric, layered
+from test_gpu_parity import check_topk, padded
 
 pytestmark = pytest.mark.gpu
 
@@ -18,6 +21,38 @@ def ctx(B):
     c = B.mlmc_create(0, 2_500_000, 32, 32)
     yield c
     B.mlmc_destroy(c)
+
+
+def rows(kind, d, M, dtype):
+    rng = np.random.default_rng(d)
+    if kind == "layers":
+        return layered(d, M, dtype)
+    if kind == "one_bin":      # every key is a boundary key: the lists of the warps are too short
+        x = 1.0 + 0.02 * rng.random((M, d))
+    elif kind == "ties":
+        x = rng.choice(np.array([0.5, -0.5, 0.25, 3.0, 0.1]), (M, d))
+    else:                      # zeros, and entries over the whole exponent range
+        x = rng.standard_normal((M, d)) * 10.0 ** rng.uniform(-30, 10, (M, d)) * (rng.random((M, d)) < 0.3)
+    return padded(torch.from_numpy(x.astype(np.float32)).cuda().to(torch.bfloat16 if dtype == "bf16" else torch.float32), 8)
+
+
+# rows of a block, of clusters of two to sixteen, and one entry more; few queries (every block resolves them all) and 31
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("kind", ["layers", "one_bin", "ties", "zeros"])
+@pytest.mark.parametrize("d", [7, 513, 8_192, 8_193, 16_385, 30_001, 65_537, 300_001])
+def test_cluster_sizes(B, ora, ctx, dtype, kind, d):
+    g = rows(kind, d, 2, dtype)
+    few, many = [max(1, d // 9), d], sorted({d * (i + 1) // 32 for i in range(31)} - {0}) + [d]
+    for k in (few, [0] + few, many, [0, 0] + many[2:-1] + [d]):
+        check_topk(B, ora, ctx, g, k, None, 5, 1, expect_excluded=1)
+        check_topk(B, ora, ctx, g, k, geometric(len(k)), 5, 2, expect_excluded=1)
+
+
+# the longest bf16 rows of a cluster with given p, in one wave and in two
+@pytest.mark.parametrize("d,M", [(1_032_192, 2), (1_032_193, 2), (524_288, 12), (524_289, 12)])
+def test_bf16_rows_given_p(B, ora, ctx, d, M):
+    k = doubling(d, d // 500)
+    check_topk(B, ora, ctx, layered(d, M, "bf16"), k, geometric(len(k)), 3, 1, expect_excluded=1)
 
 
 # edges of the tiles; empty, void and dense messages; lanes per search edge from 32 to 4
