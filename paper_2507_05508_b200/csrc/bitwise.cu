@@ -32,21 +32,26 @@ struct BitSchedule {
 // The divisor is fixed, so the quotient comes from its correctly rounded reciprocal by two correction steps (Markstein,
 // "Computation of elementary functions on the IBM RISC System/6000 processor", 1990: with the reciprocal correctly rounded
 // and a quotient within one ulp, one step of remainder and correction rounds like the division).  The truncation is the
-// addition of 2^23 with rounding toward zero.  Seven fp32 operations; the fp64 product and conversions used before took
-// two slots of the conversion unit.  The remainders must not underflow and the reciprocal must be normal: where gmax lies
+// addition of 2^23 with rounding toward zero.  (The fp64 product and conversions used before took two slots of the conversion
+// unit.)  The remainders must not underflow and the reciprocal must be normal: where gmax lies
 // outside [2^-60, 2^100], numerator and divisor are moved by a power of two.  (That is exact, except for numerators whose
 // quotient lies far below 2^-23: their code is 0 either way.)
+// The operations are done on pairs of entries (packed fp32 instructions round like the single ones): they are what binds the kernels,
+// by issue.  Only |g| = gmax has the quotient 1, so that the limit is taken where a group's largest entry says so.
 struct Quantiser {
     float gmax, inv, move;
+    int top;  // bits of the largest magnitude
     __device__ __forceinline__ explicit Quantiser(float g) {
+        top = __float_as_int(g);
         gmax = g > 0.0f ? g : 1.0f;
         move = gmax < 0x1.0p-60f ? 0x1.0p100f : gmax > 0x1.0p100f ? 0x1.0p-64f : 1.0f;
         gmax *= move;
         inv = __frcp_rn(gmax);
     }
-    // The codes of N entries at b bits (scale 2^b, b <= 23): in the low 23 bits, the bits of 2^23 above.
+    // The codes of N entries at b bits (scale 2^b, b <= 23): in the low 23 bits, the bits of 2^23 above.  limit: gmax may be among them.
     template <int N>
-    __device__ __forceinline__ void codes(const float (&v)[N], float scale, uint32_t (&q)[N]) const {
+    __device__ __forceinline__ void codes(const float (&v)[N], float scale, bool limit, uint32_t (&q)[N]) const {
+        static_assert(N % 2 == 0, "pairs");
         if (move != 1.0f) {
             float x[N];
 #pragma unroll
@@ -55,17 +60,24 @@ struct Quantiser {
         } else {
             quotients(v, scale, q);
         }
+        if (limit) {  // e = 1 has no b-bit fraction: the largest e below it has the code 2^b - 1
+            const uint32_t most = __float_as_uint(8388608.0f + scale) - 1u;
+#pragma unroll
+            for (int i = 0; i < N; ++i) q[i] = min(q[i], most);
+        }
     }
     template <int N>
     __device__ __forceinline__ void quotients(const float (&v)[N], float scale, uint32_t (&q)[N]) const {
+        const uint64_t inv2 = pair(inv, inv), minus2 = pair(-gmax, -gmax), scale2 = pair(scale, scale), one2 = pair(8388608.0f, 8388608.0f);
 #pragma unroll
-        for (int i = 0; i < N; ++i) {
-            const float x = fabsf(v[i]);
-            float e = __fmul_rn(x, inv);
-            e = __fmaf_rn(__fmaf_rn(-e, gmax, x), inv, e);
-            e = __fmaf_rn(__fmaf_rn(-e, gmax, x), inv, e);
-            // e = 1 has no b-bit fraction: the largest e below it has the code 2^b - 1
-            q[i] = __float_as_uint(__fmaf_rz(fminf(e, 0x1.fffffep-1f), scale, 8388608.0f));
+        for (int i = 0; i < N; i += 2) {
+            const uint64_t x = pair(fabsf(v[i]), fabsf(v[i + 1]));
+            uint64_t e = mul_pair(x, inv2);
+            e = fma_pair(fma_pair(e, minus2, x), inv2, e);
+            e = fma_pair(fma_pair(e, minus2, x), inv2, e);
+            e = fma_pair_toward_zero(e, scale2, one2);
+            q[i] = (uint32_t)e;
+            q[i + 1] = (uint32_t)(e >> 32);
         }
     }
 };
@@ -234,7 +246,8 @@ absmax_kernel(const T* __restrict__ g, int64_t d, int64_t ld, uint32_t* gmax_bit
 // four entries per instruction: levels that share a byte (1, 1, 2 and 4 bits, say) are packed into words of four entries
 // once, then a level is a mask and a byte product.  Shifts are multiplications where they can be: the shifter and the logic
 // share a pipe of half the rate, which bound the kernel.  8 x 124M fp32 entries, six
-// levels: 1.0 ms with every entry taken through every level and the fp64 quotient, 0.82 field by field, now 0.73 (bf16 codes of 36M x 16: 0.55 -> 0.37).
+// levels: 1.0 ms with every entry taken through every level and the fp64 quotient, 0.82 field by field, 0.70 with single quotients, now
+// 0.66 (0.62 is the first sweep of the same row; bf16 codes of 36M x 16: 0.55 -> 0.37).
 constexpr int kBitHeld = 8;
 
 template <typename T, int LMAX, typename Acc>
@@ -248,7 +261,7 @@ __device__ __forceinline__ void take_fields(const float (&v)[kBitHeld], const Qu
     if constexpr (sizeof(Acc) == 4) {
         uint32_t q[kBitHeld], w[kBitHeld / 4];
         uint32_t run = 0u;
-        qz.codes(v, scale, q);
+        qz.codes(v, scale, mx == qz.top, q);
 #pragma unroll
         for (int l = 0; l < LMAX; ++l) {
             if (l >= sc.L) break;
@@ -268,7 +281,7 @@ __device__ __forceinline__ void take_fields(const float (&v)[kBitHeld], const Qu
         }
     } else {
         uint32_t q[kBitHeld], prev[kBitHeld];
-        qz.codes(v, scale, q);
+        qz.codes(v, scale, mx == qz.top, q);
 #pragma unroll
         for (int e = 0; e < kBitHeld; ++e) {
             q[e] -= 0x4B000000u;
@@ -438,7 +451,7 @@ __device__ __forceinline__ void pack_group(const uint32_t* slot, const Quantiser
         return;
     }
     uint32_t q[32];
-    qz.codes(x, scale, q);  // the bits above a field leave with the shifts, or are planes that are not written
+    qz.codes(x, scale, __any_sync(0xFFFFFFFFu, __float_as_int(mx) == qz.top), q);  // the bits above a field leave with the shifts, or are planes that are not written
     if (w < 6) {
         for (int j = 1; j <= w; ++j) {
             const int up = 31 - (w - j);
@@ -529,7 +542,7 @@ bit_pack_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* 
 }
 
 // ---- short rows: all of the above in one launch (dense_cluster.cuh).  Fields of at most 8 bits, at most kDenseLevels levels.
-// 6 x 400,003 bf16 entries, six levels, adaptive: 22 us for the three kernels above, 15 for this one.
+// 6 x 400,003 bf16 entries, six levels, adaptive: 22 us for the three kernels above, 15 for this one, now 13.5.
 constexpr int kBitDenseWarps = 32;
 
 template <typename T>

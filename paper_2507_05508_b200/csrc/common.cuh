@@ -218,6 +218,35 @@ __device__ __forceinline__ void shared_push_if_negative(int flag, uint32_t& at, 
                  : "+r"(at) : "r"(flag), "r"(x), "r"(step) : "memory");
 }
 
+// Two fp32 numbers in a 64-bit register: packed instructions take one issue slot for both (and the time of two), and round each like
+// the single instruction.  The compiler (nvcc 12.9) merges a packed product into an addition that follows it, .rn or not: where
+// both have to round, the addition is written as a multiply-add with a 1 that the compiler does not know.
+__device__ __forceinline__ uint64_t pair(float lo, float hi) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ uint64_t mul_pair(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t add_pair(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t fma_pair(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t fma_pair_toward_zero(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rz.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
 // mant^2 of an fp32 entry (the implicit bit included, below the normal range none): the entry is mant 2^(max(e,1) - 150).
 __device__ __forceinline__ uint64_t mantissa_squared(uint32_t bits) {
     const uint32_t mant = min(bits & 0x7FFFFFFFu, (bits & 0x7FFFFFu) | 0x800000u);  // the key itself where it lies below 2^23

@@ -83,7 +83,8 @@ __device__ __forceinline__ uint32_t dense_load(cg::cluster_group& cluster, const
     if (threadIdx.x < CL) cluster.map_shared_rank(sh.top, threadIdx.x)[cluster.block_rank()] = mx;
     cluster.sync();
     mx = 0;
-    for (int r = 0; r < CL; ++r) mx = max(mx, sh.top[r]);
+#pragma unroll
+    for (int r = 0; r < kDenseMost; ++r) mx = max(mx, r < CL ? sh.top[r] : 0u);
     return mx;
 }
 
@@ -92,11 +93,20 @@ __device__ __forceinline__ uint32_t dense_load(cg::cluster_group& cluster, const
 template <typename A, int WARPS, typename S>
 __device__ __forceinline__ S dense_sums(cg::cluster_group& cluster, const A (&acc)[kDenseLevels], DenseShared<WARPS, S>& sh) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, CL = (int)cluster.num_blocks();
-    if constexpr (sizeof(A) == 4) {
+    if constexpr (sizeof(A) == 4) {  // a level per lane, then a level per warp
+        uint32_t mine = 0;
 #pragma unroll
         for (int l = 0; l < kDenseLevels; ++l) {
             const uint32_t x = __reduce_add_sync(0xFFFFFFFFu, acc[l]);
-            if (lane == 0) sh.warp_sum[l][warp] = (S)x;
+            mine = lane == l ? x : mine;
+        }
+        if (lane < kDenseLevels) sh.warp_sum[lane][warp] = (S)mine;
+        __syncthreads();
+        static_assert(WARPS <= 32 && (sizeof(A) != 4 || WARPS >= kDenseLevels), "the warps' sums of a level fit a warp");
+        if (warp < kDenseLevels) {
+            const uint32_t x = lane < WARPS ? (uint32_t)sh.warp_sum[warp][lane] : 0u;
+            const S s = (S)__reduce_add_sync(0xFFFFFFFFu, x & 0xFFFFu) + (S)__reduce_add_sync(0xFFFFFFFFu, x >> 16) * (S)65536;
+            if (lane < CL) cluster.map_shared_rank(&sh.sum[0][0], lane)[cluster.block_rank() * kDenseLevels + warp] = s;
         }
     } else {
         // half of the levels go to the partner lane in each of the first three steps: lane l ends with level l / 4
@@ -116,18 +126,19 @@ __device__ __forceinline__ S dense_sums(cg::cluster_group& cluster, const A (&ac
         z += __shfl_xor_sync(0xFFFFFFFFu, z, 2);
         z += __shfl_xor_sync(0xFFFFFFFFu, z, 1);
         if ((lane & 3) == 0) sh.warp_sum[lane >> 2][warp] = z;
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < kDenseLevels * CL; i += WARPS * 32) {
-        S s = 0;
+        __syncthreads();
+        for (int i = threadIdx.x; i < kDenseLevels * CL; i += WARPS * 32) {
+            S s = 0;
 #pragma unroll
-        for (int w = 0; w < WARPS; ++w) s += sh.warp_sum[i % kDenseLevels][w];
-        cluster.map_shared_rank(&sh.sum[0][0], i / kDenseLevels)[cluster.block_rank() * kDenseLevels + i % kDenseLevels] = s;
+            for (int w = 0; w < WARPS; ++w) s += sh.warp_sum[i % kDenseLevels][w];
+            cluster.map_shared_rank(&sh.sum[0][0], i / kDenseLevels)[cluster.block_rank() * kDenseLevels + i % kDenseLevels] = s;
+        }
     }
     cluster.sync();
     S total = 0;
     if (threadIdx.x < kDenseLevels)
-        for (int r = 0; r < CL; ++r) total += sh.sum[r][threadIdx.x];
+#pragma unroll
+        for (int r = 0; r < kDenseMost; ++r) total += r < CL ? sh.sum[r][threadIdx.x] : S(0);
     return total;
 }
 
