@@ -75,9 +75,10 @@ __device__ RtnLevel rtn_level(float c, int r) {
 // warp's entries rounds to 0 contribute nothing and are skipped: the clipping value is the row's largest magnitude, and
 // in a gradient with per-layer scales most entries are small beside it.  The first level that is left has C^{l-1} = 0, so
 // its residual is its value.  The differences and sums are fp64 (a difference of two fp32 values is exact); what bounds the
-// kernel where nothing is skipped is the conversion of one fp32 value to fp64 per entry and level (16 per clock and SM).
+// kernel where nothing is skipped is issue: a value per entry and level is found, widened to fp64, subtracted, squared and added.
 // 8 x 124M fp32 entries, L = 5: 2.29 ms with every entry taken through every level; 1.02 with one trip in flight and one and
-// a half waves of blocks, now 0.87.
+// a half waves of blocks, 0.85 with every value through the conversion unit, 0.79 with single instructions for the grid values, now 0.74
+// (0.57 is the first sweep of the same row).
 constexpr int kRtnHeld = 8;
 
 template <typename T>
@@ -97,12 +98,27 @@ __device__ __forceinline__ void rtn_expand(const uint4* q, float (&v)[kRtnHeld])
     }
 }
 
-// One trip of a warp: kRtnHeld entries per lane.
+// The conversion unit takes 16 numbers per clock and SM, a quarter of what the fp64 unit adds up.  So every second number (x >= 0; one
+// of four or three of four are within 1 %) goes another way: its bits moved to the places of a double are x 2^-896, zero and the numbers below the normal range included, and
+// the product with 2^896 is exact.
+__device__ __forceinline__ double widen(float x, bool by_product) {
+    if (!by_product) return (double)x;
+    const uint32_t b = __float_as_uint(x);
+    return __hiloint2double((int)(b >> 3), (int)(b << 29)) * 0x1p896;
+}
+
+// One trip of a warp: kRtnHeld entries per lane.  Magnitudes: C^l(-v) = -C^l(v).  The grid values of two entries are found together, by
+// packed instructions.  one = 1, an argument: the compiler merges a packed product and the addition after it into one rounding, also
+// where both say that they round, and the rounding of t = fl32(v inv) decides ties.  So the addition is a multiply-add of t with one.
 template <int LMAX>
-__device__ __forceinline__ void take_levels(const float (&v)[kRtnHeld], float c, const RtnLevel* levels, int L, double (&acc)[LMAX]) {
+__device__ __forceinline__ void take_levels(const float (&signed_v)[kRtnHeld], float c, const RtnLevel* levels, int L, float one, double (&acc)[LMAX]) {
+    float v[kRtnHeld];
     int mx = 0;
 #pragma unroll
-    for (int e = 0; e < kRtnHeld; ++e) mx = max(mx, __float_as_int(v[e]) & 0x7FFFFFFF);
+    for (int e = 0; e < kRtnHeld; ++e) {
+        v[e] = fabsf(signed_v[e]);
+        mx = max(mx, __float_as_int(v[e]));
+    }
     mx = __reduce_max_sync(0xFFFFFFFFu, mx);
     double prev[kRtnHeld];  // C^{l-1}
     bool first = true;      // C^{l-1} = 0 for every entry of the warp (warp-uniform)
@@ -117,7 +133,7 @@ __device__ __forceinline__ void take_levels(const float (&v)[kRtnHeld], float c,
             double odd = 0.0;  // two chains of additions
 #pragma unroll
             for (int e = 0; e < kRtnHeld; ++e) {
-                const double res = (double)v[e] - prev[e];
+                const double res = widen(v[e], e & 1) - prev[e];
                 if (e & 1) odd = fma(res, res, odd);
                 else acc[l] = fma(res, res, acc[l]);
             }
@@ -127,20 +143,24 @@ __device__ __forceinline__ void take_levels(const float (&v)[kRtnHeld], float c,
         const RtnLevel lv = levels[l];
         if (mx <= lv.zero_upto) continue;  // the grids get finer: once a level is not skipped, none after it is
         float x[kRtnHeld];
+        const uint64_t inv2 = pair(lv.inv, lv.inv), delta2 = pair(lv.delta, lv.delta), up2 = pair(12582912.0f, 12582912.0f),
+                       down2 = pair(-12582912.0f, -12582912.0f), one2 = pair(one, one);
 #pragma unroll
-        for (int e = 0; e < kRtnHeld; ++e) {
-            const float k = __fadd_rn(__fadd_rn(__fmul_rn(v[e], lv.inv), 12582912.0f), -12582912.0f);
-            x[e] = __fmul_rn(k, lv.delta);
+        for (int e = 0; e < kRtnHeld; e += 2) {
+            const uint64_t k = add_pair(fma_pair(mul_pair(pair(v[e], v[e + 1]), inv2), one2, up2), down2);
+            const uint64_t y = mul_pair(k, delta2);
+            x[e] = __uint_as_float((uint32_t)y);
+            x[e + 1] = __uint_as_float((uint32_t)(y >> 32));
         }
         if (mx > lv.free_upto) {
 #pragma unroll
-            for (int e = 0; e < kRtnHeld; ++e) x[e] = fminf(fmaxf(x[e], -c), c);
+            for (int e = 0; e < kRtnHeld; ++e) x[e] = fminf(x[e], c);
         }
         double odd = 0.0;
         if (first) {
 #pragma unroll
             for (int e = 0; e < kRtnHeld; ++e) {
-                prev[e] = (double)x[e];
+                prev[e] = widen(x[e], e & 1);
                 if (e & 1) odd = fma(prev[e], prev[e], odd);
                 else acc[l] = fma(prev[e], prev[e], acc[l]);
             }
@@ -148,7 +168,7 @@ __device__ __forceinline__ void take_levels(const float (&v)[kRtnHeld], float c,
         } else {
 #pragma unroll
             for (int e = 0; e < kRtnHeld; ++e) {
-                const double cur = (double)x[e], res = cur - prev[e];
+                const double cur = widen(x[e], e & 1), res = cur - prev[e];
                 if (e & 1) odd = fma(res, res, odd);
                 else acc[l] = fma(res, res, acc[l]);
                 prev[e] = cur;
@@ -173,7 +193,7 @@ __device__ __forceinline__ void take_entry(float v, float c, const RtnLevel* lev
 template <typename T, int LMAX>
 __global__ void __launch_bounds__(kRtnThreads, LMAX <= 6 ? 4 : 3)
 rtn_stats_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* gmax_bits, const __grid_constant__ RtnSchedule sc, double* partial,
-                 int rtn_ctas, uint32_t* done, const __grid_constant__ DrawPlan pl, int* status, int* worker_err) {
+                 int rtn_ctas, uint32_t* done, const __grid_constant__ DrawPlan pl, int* status, int* worker_err, float one) {
     using Tr = ElemTraits<T>;
     extern __shared__ __align__(16) uint4 sh_vectors[];  // [4][vectors per trip][kRtnThreads]
     __shared__ double sh_red[LMAX][kRtnThreads / 32];
@@ -197,7 +217,7 @@ rtn_stats_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t*
         stream_trips<kVecs, kRtnThreads>(reinterpret_cast<const uint4*>(row), blockIdx.x, gridDim.x, trips, sh_vectors, [&](const uint4 (&q)[kVecs]) {
             float v[kRtnHeld];
             rtn_expand<T>(q, v);
-            take_levels<LMAX>(v, c, sh_lv, sc.L, acc);
+            take_levels<LMAX>(v, c, sh_lv, sc.L, one, acc);
         });
         if (blockIdx.x == gridDim.x - 1) {  // the rest of the row, fewer than kTrip + 1 vectors, one by one
             for (int64_t i = trips * kTrip * Tr::kVec + threadIdx.x; i < d; i += kRtnThreads) {
@@ -363,7 +383,7 @@ template <typename T>
 __global__ void __launch_bounds__(kRtnDenseWarps * 32, 1)
 rtn_cluster_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid_constant__ RtnSchedule sc,
                    const __grid_constant__ DrawPlan pl, const __grid_constant__ DrawnLevels drawn, int adaptive, int per_block,
-                   float* __restrict__ val, int64_t ldv, int* status, int* worker_err) {
+                   float* __restrict__ val, int64_t ldv, int* status, int* worker_err, float one) {
     using Tr = ElemTraits<T>;
     extern __shared__ __align__(16) uint32_t sh_slots[];
     __shared__ DenseShared<kRtnDenseWarps, double> sh;
@@ -408,7 +428,7 @@ rtn_cluster_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid_
                     for (int j = 0; j < kVecs; ++j) q[j] = x[j * 32];
                     float v[kRtnHeld];
                     rtn_expand<T>(q, v);
-                    take_levels<kRtnDenseLevels>(v, c, sh_lv, sc.L, acc);
+                    take_levels<kRtnDenseLevels>(v, c, sh_lv, sc.L, one, acc);
                 } else {  // entries past the row's end are not entries
                     for (int e = (u & 3) * 256 + lane; e < (u & 3) * 256 + 256 && e0 + e < d; e += 32)
                         take_entry<kRtnDenseLevels>(Tr::value(entry(u >> 2, e)), c, sh_lv, sc.L, acc);
@@ -524,7 +544,7 @@ void launch_rtn_stats_t(Workspace& ws, const T* g, int64_t d, int M, int64_t ld,
     // four: 866 for 8 x 124M entries)
     const int nb = std::min(rtn_blocks(ws, d, ElemTraits<T>::kVec, M, 4 * resident), ws.rtn_ctas);
     launch_kernel(ws, K_RTN_STATS, rtn_stats_kernel<T, LMAX>, dim3(nb, M), kRtnThreads, smem, s, g, d, ld, ws.gmax_bits, sc,
-                  ws.rtn_partial, ws.rtn_ctas, ws.done, plan, ws.status, ws.worker_err);
+                  ws.rtn_partial, ws.rtn_ctas, ws.done, plan, ws.status, ws.worker_err, 1.0f);
 }
 }  // namespace
 
@@ -549,7 +569,7 @@ bool launch_rtn_cluster(Workspace& ws, const void* g, int dtype, int64_t d, int 
     const int per = (int)(((d + 1023) / 1024 + cl - 1) / cl);
     auto go = [&](auto kernel, auto* row, size_t elem) {
         launch_kernel_cluster(ws, K_RTN_CLUSTER, cl, kernel, dim3(M * cl), kRtnDenseWarps * 32, per * 1024 * elem, s, row, d, ld, sc, plan,
-                              drawn, p ? 0 : 1, per, out.val, out.ldv, ws.status, ws.worker_err);
+                              drawn, p ? 0 : 1, per, out.val, out.ldv, ws.status, ws.worker_err, 1.0f);
     };
     if (dtype == MLMC_BF16) go(rtn_cluster_kernel<bf16_t>, static_cast<const bf16_t*>(g), 2);
     else go(rtn_cluster_kernel<float>, static_cast<const float*>(g), 4);

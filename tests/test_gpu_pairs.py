@@ -1,0 +1,47 @@
+"""Level statistics on pairs of entries: zeros, numbers below the normal range and the largest magnitude in either place."""
+import numpy as np
+import pytest
+import torch
+
+from test_gpu_ext import check_rtn
+from test_gpu_parity import check_bitwise, padded
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    from paper_2507_05508_b200 import binding
+    binding.lib()
+    return binding
+
+
+@pytest.fixture(scope="module")
+def ctx(B):
+    c = B.mlmc_create(0, 700_000, 3, 32)
+    yield c
+    B.mlmc_destroy(c)
+
+
+def rows(kind, d, dtype):
+    rng = np.random.default_rng(d)
+    x = rng.standard_normal((2, d))
+    if kind == "tiny":           # most entries below the normal range or zero, the others small beside the largest
+        x *= 10.0 ** rng.uniform(-44, -36, (2, d)) * (rng.random((2, d)) < 0.7)
+        x[:, ::97] = 1e-33 * rng.standard_normal(x[:, ::97].shape)
+    elif kind == "largest":      # half of the entries have the largest magnitude
+        x = np.where(rng.random((2, d)) < 0.5, np.sign(x) * 0.75, x * 0.1)
+    elif kind == "large":
+        x *= 1e35
+    return padded(torch.from_numpy(x.astype(np.float32)).cuda().to(torch.bfloat16 if dtype == "bf16" else torch.float32), 8)
+
+
+# short rows in one launch and long ones in three
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("kind", ["tiny", "largest", "large"])
+@pytest.mark.parametrize("d", [20_003, 600_001])
+def test_statistics(B, ora, ctx, dtype, kind, d):
+    g = rows(kind, d, dtype)
+    check_rtn(B, ora, ctx, g, [2, 4, 8, 16], None, 3, 1)
+    check_bitwise(B, ora, ctx, g, [1, 2, 4, 8, 16, 23], None, 3, 1)
+    check_bitwise(B, ora, ctx, g, [2, 14, 23], None, 3, 2)
