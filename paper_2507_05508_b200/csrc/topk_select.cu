@@ -86,7 +86,7 @@ __global__ void uniforms_kernel(double* u_dev, int M, uint64_t seed, uint64_t st
 // A warp takes one batch of the emit tiles at a time (kEmitGroupVecs consecutive 16-byte vectors, four per lane, all in
 // flight before the first is used) and stores the batch's largest key: the emission reads only the batches whose
 // largest key reaches the lower threshold of the drawn band.
-// BR (fp32, fixed p): the keys whose leading digit lies in one of the worker's two brackets (the bins around last
+// BR (fixed p): the keys whose leading digit lies in one of the worker's two brackets (the bins around last
 // call's boundary bins) are collected as candidates in the same sweep.  A batch whose largest key lies below both
 // brackets is not tested (in a gradient with per-layer scales that is most batches).  Every warp stages its keys in a
 // private shared-memory buffer and moves the buffer to the candidate list when it fills up (one global counter update
@@ -102,14 +102,14 @@ __device__ __forceinline__ uint32_t nth_key(const uint4& lo, const uint4& hi, in
     return ((at & 1) ? yw : xz) & 0x7FFFFFFFu;
 }
 
-template <typename T, bool BR>
+template <bool BR>
 __global__ void __launch_bounds__(kHistThreads, 1)
-hist1_kernel(const T* __restrict__ g, int64_t d, int64_t ld, uint32_t* __restrict__ hist1,
+hist1_kernel(const float* __restrict__ g, int64_t d, int64_t ld, uint32_t* __restrict__ hist1,
              uint32_t* __restrict__ tile_max, int tiles_per_worker, int* status, int* worker_err,
              const uint4* bracket, uint32_t* __restrict__ cand_keys, int64_t cand_cap,
              uint32_t* cand_count, int* cand_overflow, const int* only) {
     extern __shared__ uint32_t sh_hist[];
-    using Tr = ElemTraits<T>;
+    using Tr = ElemTraits<float>;
     for (int b = threadIdx.x; b < kBins1; b += blockDim.x) sh_hist[b] = 0;
     pdl_enter();
     const int m = blockIdx.y;
@@ -149,20 +149,14 @@ hist1_kernel(const T* __restrict__ g, int64_t d, int64_t ld, uint32_t* __restric
         }
     };
     __syncthreads();
-    const T* row = g + (int64_t)m * ld;
+    const float* row = g + (int64_t)m * ld;
     uint32_t* tmax = tile_max + (int64_t)m * tiles_per_worker * kEmitGroups;
     const int64_t nvec = (d + Tr::kVec - 1) / Tr::kVec;
     const int64_t full_end = d / Tr::kVec;  // vectors that lie wholly inside the row
     bool bad = false;
     auto count_key = [&](uint32_t bits) { atomicAdd(&sh_hist[Tr::key(bits) >> Tr::kShift1], 1u); };  // Inf / NaN: see the maxima
     auto vector_max = [&](const uint4& q) -> uint32_t {  // largest key of one vector
-        if constexpr (Tr::kVec == 4) {
-            return max(max(q.x & 0x7FFFFFFFu, q.y & 0x7FFFFFFFu), max(q.z & 0x7FFFFFFFu, q.w & 0x7FFFFFFFu));
-        } else {
-            const uint32_t a = __vmaxu2(__vmaxu2(q.x & 0x7FFF7FFFu, q.y & 0x7FFF7FFFu),
-                                        __vmaxu2(q.z & 0x7FFF7FFFu, q.w & 0x7FFF7FFFu));
-            return max(a & 0xFFFFu, a >> 16);
-        }
+        return max(max(q.x & 0x7FFFFFFFu, q.y & 0x7FFFFFFFu), max(q.z & 0x7FFFFFFFu, q.w & 0x7FFFFFFFu));
     };
     constexpr int kBatch = kEmitGroupVecs / 32;
     static_assert(kBatch == 4, "a warp takes a batch in one trip of four vectors per lane");
@@ -179,12 +173,7 @@ hist1_kernel(const T* __restrict__ g, int64_t d, int64_t ld, uint32_t* __restric
             uint32_t vm = 0;
 #pragma unroll
             for (int j = 0; j < kBatch; ++j) {
-                if constexpr (Tr::kVec == 4) {
-                    count_key(q[j].x); count_key(q[j].y); count_key(q[j].z); count_key(q[j].w);
-                } else {
-                    count_key(q[j].x & 0xFFFFu); count_key(q[j].x >> 16); count_key(q[j].y & 0xFFFFu); count_key(q[j].y >> 16);
-                    count_key(q[j].z & 0xFFFFu); count_key(q[j].z >> 16); count_key(q[j].w & 0xFFFFu); count_key(q[j].w >> 16);
-                }
+                count_key(q[j].x); count_key(q[j].y); count_key(q[j].z); count_key(q[j].w);
                 vm = max(vm, vector_max(q[j]));
             }
             wm = __reduce_max_sync(0xFFFFFFFFu, vm);
@@ -214,7 +203,7 @@ hist1_kernel(const T* __restrict__ g, int64_t d, int64_t ld, uint32_t* __restric
         } else {  // the row's end, vector by vector; batches past it have the largest key 0
             uint32_t vm = 0;
             for (int64_t u = v; u < min(nvec, (int64_t)(b + 1) * kEmitGroupVecs); u += 32) {
-                for_each_in_vector<T>(row, u, d, [&](int64_t, uint32_t bits) {
+                for_each_in_vector<float>(row, u, d, [&](int64_t, uint32_t bits) {
                     count_key(bits);
                     vm = max(vm, Tr::key(bits));
                     if (BR && in_bracket(bits)) {
@@ -242,6 +231,169 @@ hist1_kernel(const T* __restrict__ g, int64_t d, int64_t ld, uint32_t* __restric
     for (int b = threadIdx.x; b < kBins1; b += blockDim.x) {
         const uint32_t c = sh_hist[b];
         if (c) atomicAdd(&out[b], c);
+    }
+}
+
+// The same sweep for bf16 rows.  With one count per bin 32 keys meet 3.5 deep in a bank (deeper in a layer whose keys share few bins),
+// and the shared-memory atomics bound the sweep: 92 % of the L1 wavefronts.  Here a bin has 16 counts, one for every second lane, so
+// that at most two lanes of a warp meet in a bank.  They have room for kColumnBins bins, 20 octaves from below the octave of the
+// largest key that a sample of the row holds.  Beside the window, down to 32 octaves below its top, a bin has one count; what lies
+// outside of that is counted in memory, key by key, and zeros in a register.  A block whose sample lies below the window by more
+// than one key of kColumnMisses keeps one count per bin for all, and so do short rows, where the sample takes longer than it saves
+// (8 x 1M keys: 63.3 us per step, 65.7 with columns).
+// 32 x 25.6M keys: 406 us, now 337 (floor 250); 8 x 40M, given p: 260 us per step, now 235; 8 x 12M 167 either way.  On the way: all
+// 32 keys of a warp by the general way whenever one lies outside the window (each lane its own way 355 us); every key by the general
+// way 386; windows of 22 and 24 octaves leave too little L1 for the loads in flight (362 us, and 334 without the bins beside).
+constexpr int kColumnBins = 20 * 128;
+constexpr int kColumns = 16;
+constexpr int kFarBelow = 12 * 128, kFarAbove = 8 * 128;
+constexpr int kFarBins = kFarBelow + kColumnBins + kFarAbove;  // numbered through the window
+constexpr int kColumnSmem = (kColumnBins * kColumns + kFarBins) * (int)sizeof(uint32_t);
+constexpr uint32_t kColumnMisses = 64;
+constexpr int64_t kColumnBatches = 8;  // per warp, from which on a row is long enough
+static_assert(kColumnSmem >= kBins1 * (int)sizeof(uint32_t), "either kind of counts");
+
+__global__ void __launch_bounds__(kHistThreads, 1)
+hist1_bf16_kernel(const bf16_t* __restrict__ g, int64_t d, int64_t ld, uint32_t* __restrict__ hist1, uint32_t* __restrict__ tile_max,
+                  int tiles_per_worker, int sample, int* status, int* worker_err) {
+    extern __shared__ uint32_t sh_hist[];
+    __shared__ uint32_t sh_warp[kHistThreads / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int i = threadIdx.x; i < kColumnSmem / 16; i += kHistThreads) reinterpret_cast<uint4*>(sh_hist)[i] = make_uint4(0u, 0u, 0u, 0u);
+    pdl_enter();
+    const int m = blockIdx.y;
+    const bf16_t* row = g + (int64_t)m * ld;
+    const int64_t nvec = (d + 7) / 8, full_end = d / 8;  // vectors of the row, and those wholly inside it
+    auto vector_max = [](const uint4& q) -> uint32_t {
+        const uint32_t a = __vmaxu2(__vmaxu2(q.x & 0x7FFF7FFFu, q.y & 0x7FFF7FFFu), __vmaxu2(q.z & 0x7FFF7FFFu, q.w & 0x7FFF7FFFu));
+        return max(a & 0xFFFFu, a >> 16);
+    };
+    uint32_t lowest = 0;  // first bin of the window
+    bool columns = false;
+    if (sample) {
+        const int64_t stride = full_end / kHistThreads;
+        const uint4 q = __ldg(reinterpret_cast<const uint4*>(row) + threadIdx.x * stride + (blockIdx.x * 37 + threadIdx.x * 11) % stride);
+        uint32_t top = __reduce_max_sync(0xFFFFFFFFu, vector_max(q));
+        if (lane == 0) sh_warp[warp] = top;
+        __syncthreads();
+        top = __reduce_max_sync(0xFFFFFFFFu, sh_warp[lane]);
+        const uint32_t end = top & ~127u;  // the largest keys are few
+        lowest = end > (uint32_t)kColumnBins ? end - kColumnBins : 0u;
+        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+        uint32_t out = 0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const uint32_t key = (w[i / 2] >> (16 * (i & 1))) & 0x7FFFu;
+            out += key < lowest ? 1u : 0u;
+        }
+        out = __reduce_add_sync(0xFFFFFFFFu, out);
+        __syncthreads();
+        if (lane == 0) sh_warp[warp] = out;
+        __syncthreads();
+        out = __reduce_add_sync(0xFFFFFFFFu, sh_warp[lane]);
+        columns = out * kColumnMisses <= 8u * kHistThreads;  // block-uniform
+    } else {
+        __syncthreads();
+    }
+    uint32_t* out = hist1 + (int64_t)m * kBins1;
+    uint32_t* tmax = tile_max + (int64_t)m * tiles_per_worker * kEmitGroups;
+    const uint32_t column0 = (uint32_t)__cvta_generic_to_shared(sh_hist) + (lane & (kColumns - 1)) * 4u - lowest * (kColumns * 4u);
+    uint32_t* const sh_far = sh_hist + kColumnBins * kColumns;
+    const uint32_t far0 = (uint32_t)__cvta_generic_to_shared(sh_far) + (kFarBelow - (int)lowest) * 4;
+    uint32_t zeros = 0;
+    auto count_column = [&](uint32_t key) { asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(column0 + key * (kColumns * 4u)) : "memory"); };
+    auto count_key = [&](uint32_t bits) {
+        const uint32_t key = bits & 0x7FFFu;  // Inf / NaN: see the maxima
+        if (!columns) atomicAdd(&sh_hist[key], 1u);
+        else if (key - lowest < (uint32_t)kColumnBins) count_column(key);
+        else if (key == 0u) ++zeros;
+        else if (key - lowest + (uint32_t)kFarBelow < (uint32_t)kFarBins) atomicAdd(&sh_far[key - lowest + kFarBelow], 1u);
+        else atomicAdd(&out[key], 1u);
+    };
+    constexpr int kBatch = kEmitGroupVecs / 32;
+    const int nbatch = tiles_per_worker * kEmitGroups;
+    bool bad = false;
+    for (int b = blockIdx.x * (kHistThreads / 32) + warp; b < nbatch; b += gridDim.x * (kHistThreads / 32)) {
+        const int64_t v = (int64_t)b * kEmitGroupVecs + lane;
+        uint32_t vm = 0;
+        if ((int64_t)(b + 1) * kEmitGroupVecs <= full_end) {  // warp-uniform
+            uint4 q[kBatch];
+#pragma unroll
+            for (int j = 0; j < kBatch; ++j) q[j] = __ldg(reinterpret_cast<const uint4*>(row) + v + j * 32);
+            if (columns) {
+#pragma unroll
+                for (int j = 0; j < kBatch; ++j) {
+                    const uint32_t w[4] = {q[j].x & 0x7FFF7FFFu, q[j].y & 0x7FFF7FFFu, q[j].z & 0x7FFF7FFFu, q[j].w & 0x7FFF7FFFu};
+                    const uint32_t hi = __vmaxu2(__vmaxu2(w[0], w[1]), __vmaxu2(w[2], w[3])), lo = __vminu2(__vminu2(w[0], w[1]), __vminu2(w[2], w[3]));
+                    const uint32_t most = max(hi & 0xFFFFu, hi >> 16), least = min(lo & 0xFFFFu, lo >> 16);
+                    vm = max(vm, most);
+                    if (__all_sync(0xFFFFFFFFu, least >= lowest && most - lowest < (uint32_t)kColumnBins)) {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            count_column(w[i] & 0xFFFFu);
+                            count_column(w[i] >> 16);
+                        }
+                    } else if (least - lowest + (uint32_t)kFarBelow < (uint32_t)kFarBins && most - lowest + (uint32_t)kFarBelow < (uint32_t)kFarBins) {
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            const uint32_t key = i & 1 ? w[i / 2] >> 16 : w[i / 2] & 0xFFFFu;
+                            const uint32_t at = key - lowest < (uint32_t)kColumnBins ? column0 + key * (kColumns * 4u) : far0 + key * 4u;
+                            asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(at) : "memory");
+                        }
+                    } else {
+#pragma unroll 1
+                        for (int i = 0; i < 8; ++i) {
+                            const uint32_t x = i & 4 ? (i & 2 ? w[3] : w[2]) : (i & 2 ? w[1] : w[0]);
+                            count_key(i & 1 ? x >> 16 : x & 0xFFFFu);
+                        }
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < kBatch; ++j) {
+                    const uint32_t w[4] = {q[j].x, q[j].y, q[j].z, q[j].w};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        atomicAdd(&sh_hist[w[i] & 0x7FFFu], 1u);
+                        atomicAdd(&sh_hist[(w[i] >> 16) & 0x7FFFu], 1u);
+                    }
+                    vm = max(vm, vector_max(q[j]));
+                }
+            }
+        } else {  // the row's end, vector by vector; batches past it have the largest key 0
+            for (int64_t u = v; u < min(nvec, (int64_t)(b + 1) * kEmitGroupVecs); u += 32)
+                for_each_in_vector<bf16_t>(row, u, d, [&](int64_t, uint32_t bits) {
+                    count_key(bits);
+                    vm = max(vm, bits & 0x7FFFu);
+                });
+        }
+        vm = __reduce_max_sync(0xFFFFFFFFu, vm);
+        bad |= vm >= ElemTraits<bf16_t>::kInfKey;  // a non-finite entry shows in the largest key of its batch
+        if (lane == 0) tmax[b] = vm;
+    }
+    if (bad && lane == 0) {
+        worker_err[m] = MLMC_ERR_NONFINITE;
+        set_status(status, MLMC_ERR_NONFINITE);
+    }
+    __syncthreads();
+    if (columns) {
+        zeros = __reduce_add_sync(0xFFFFFFFFu, zeros);
+        if (lane == 0 && zeros) atomicAdd(&out[0], zeros);
+        for (int b = threadIdx.x; b < kColumnBins; b += kHistThreads) {
+            uint32_t c = 0;
+#pragma unroll
+            for (int i = 0; i < kColumns; ++i) c += sh_hist[b * kColumns + ((i + lane) & (kColumns - 1))];
+            if (c) atomicAdd(&out[lowest + b], c);
+        }
+        for (int b = threadIdx.x; b < kFarBins; b += kHistThreads) {
+            const uint32_t c = sh_far[b];
+            if (c) atomicAdd(&out[(int)lowest - kFarBelow + b], c);
+        }
+    } else {
+        for (int b = threadIdx.x; b < kBins1; b += kHistThreads) {
+            const uint32_t c = sh_hist[b];
+            if (c) atomicAdd(&out[b], c);
+        }
     }
 }
 
@@ -1115,17 +1267,20 @@ void launch_hist1(Workspace& ws, const void* g, int dtype, int64_t d, int M, int
     // whole blocks per worker leave more than 5 % of the SMs idle (32 workers: 456 against 401 us for 26M bf16 keys each).
     const int waves = ws.sm_count / M * M * 20 < ws.sm_count * 19 ? 2 : 1;
     const int nb = blocks_per_worker(ws, d, dtype == MLMC_BF16 ? 8 : 4, kHistThreads, M, waves);
-    auto go = [&](auto kernel, auto* row) {
+    auto go = [&](auto kernel) {
+        const float* row = static_cast<const float*>(g);
         launch_kernel(ws, only ? K_MISSED_HIST : K_HIST1, kernel, dim3(nb, M), kHistThreads, smem, s, row, d, ld, ws.hist1, ws.tile_max, tpw,
                       ws.status, ws.worker_err, ws.bracket, ws.cand_keys, ws.cand_cap, ws.cand_count, ws.cand_overflow, only);
     };
     if (dtype == MLMC_BF16) {
-        go(hist1_kernel<bf16_t, false>, static_cast<const bf16_t*>(g));
+        const int64_t batches = ((int64_t)tpw * kEmitGroups + nb * (kHistThreads / 32) - 1) / (nb * (kHistThreads / 32));  // per warp
+        launch_kernel(ws, K_HIST1, hist1_bf16_kernel, dim3(nb, M), kHistThreads, kColumnSmem, s, static_cast<const bf16_t*>(g), d, ld, ws.hist1,
+                      ws.tile_max, tpw, batches >= kColumnBatches ? 1 : 0, ws.status, ws.worker_err);
     } else if (brackets) {
         smem += (kHistThreads / 32) * (kWarpStage + 1) * sizeof(uint32_t);
-        go(hist1_kernel<float, true>, static_cast<const float*>(g));
+        go(hist1_kernel<true>);
     } else {
-        go(hist1_kernel<float, false>, static_cast<const float*>(g));
+        go(hist1_kernel<false>);
     }
 }
 
@@ -1192,8 +1347,8 @@ int configure_select_kernels() {
     auto set = [](auto kernel, int bytes) {
         return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess;
     };
-    const bool ok = set(resolve1_kernel, kResolveSmem) && set(hist1_kernel<float, false>, hist) && set(hist1_kernel<float, true>, hist + stage) &&
-                    set(hist1_kernel<bf16_t, false>, hist) && set(sums_candidates_kernel<true>, kS2SmemMost) &&
+    const bool ok = set(resolve1_kernel, kResolveSmem) && set(hist1_kernel<false>, hist) && set(hist1_kernel<true>, hist + stage) &&
+                    set(hist1_bf16_kernel, kColumnSmem) && set(sums_candidates_kernel<true>, kS2SmemMost) &&
                     set(sums_candidates_kernel<false>, (int)s2_smem(0, false, kS2Threads)) && set(digit_pass_kernel<2, true>, columns) &&
                     set(digit_pass_kernel<2, false>, digits) && set(digit_pass_kernel<3, true>, digits) &&
                     set(digit_pass_kernel<3, false>, digits);

@@ -1,0 +1,59 @@
+"""Long bf16 rows: the histogram with several counts per bin, and what lies outside its window."""
+import pytest
+import torch
+
+from test_gpu_parity import padded
+from test_gpu_sampled import check_adaptive
+
+pytestmark = pytest.mark.gpu
+
+M, D = 100, 262_147  # one block per worker, eight batches per warp and a ragged end
+
+
+@pytest.fixture(scope="module")
+def B():
+    from paper_2507_05508_b200 import binding
+    binding.lib()
+    return binding
+
+
+def sampled(d):
+    """Mask of the keys that the first block of a row samples: a vector of eight per stratum."""
+    stride = (d // 8) // 1024
+    t = torch.arange(1024)
+    at = t * stride + (t * 11) % stride
+    mask = torch.zeros(d, dtype=torch.bool)
+    mask[(at[:, None] * 8 + torch.arange(8)).flatten()] = True
+    return mask.cuda()
+
+
+@pytest.mark.parametrize("case", ["layers", "zeros", "few_zeros", "wide", "tiny", "sample_above", "sample_below", "constant"])
+@pytest.mark.parametrize("d", [D, 700_001])
+def test_thresholds_and_norms(B, case, d):
+    gen = torch.Generator(device="cuda").manual_seed(d)
+    g = torch.randn((M, d), generator=gen, device="cuda")
+    if case == "layers":
+        g *= torch.repeat_interleave(10.0 ** (torch.rand(40, generator=gen, device="cuda") * 4 - 5), -(-d // 40))[:d]
+    elif case in ("zeros", "few_zeros"):
+        g *= torch.rand((M, d), generator=gen, device="cuda") < (0.05 if case == "zeros" else 0.995)
+    elif case == "wide":              # over 60 octaves
+        g *= 2.0 ** (torch.rand((M, d), generator=gen, device="cuda") * 60 - 40)
+    elif case == "tiny":              # the window starts at the smallest numbers
+        g *= 2.0 ** -120
+    elif case == "sample_above":      # the window lies above everything else, by 16, 26 and 50 octaves
+        g[:, sampled(d)] = 8.0
+        for i, octaves in enumerate((16, 26, 50)):
+            g[i::3, ~sampled(d)] *= 2.0 ** -octaves
+    elif case == "sample_below":      # and below, by 4, 10 and 50
+        g[:, sampled(d)] = 1.0
+        for i, octaves in enumerate((4, 10, 50)):
+            g[i::3, ~sampled(d)] *= 2.0 ** octaves
+    else:
+        g.fill_(0.25)
+    g = padded(g.to(torch.bfloat16), 8)
+    ctx = B.mlmc_create(0, d, M, 32)
+    try:
+        check_adaptive(B, ctx, g, [d // 500 << l for l in range(8)] + [d])
+        check_adaptive(B, ctx, g, [0, 1, d // 3, d // 3 + 1, d - 1, d])
+    finally:
+        B.mlmc_destroy(ctx)
