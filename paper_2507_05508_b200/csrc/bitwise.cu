@@ -411,15 +411,17 @@ bit_stats_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t*
 }
 
 // ---- pack: a warp turns 1024 consecutive entries into 32 words of each plane, a lane owning 32 consecutive entries (one
-// word per plane).  The entries come through a ring of two shared-memory slots per warp: the next group's copy is in
-// flight while the current group is coded.  A plane's word is collected by one shift and one funnel shift per entry, from
+// word per plane).  The entries come through a slot of shared memory per warp: the next group's copy starts when the current
+// group's entries are in registers, and is in flight while they are coded.  A plane's word is collected by one shift and one funnel shift per entry, from
 // 6 planes on by one bit transpose for all of them.  A group whose largest entry has the code 0 at the drawn level's bits is
 // not coded: its magnitude planes are zero.  The groups of which the sweep before knows that are not even read (8 x 124M fp32
-// entries with layers: 782 -> 424 us).
+// entries with layers: 782 -> 424 us).  Those calls have four blocks per SM, since one warp's groups are not another's: 482 us with three
+// blocks of two slots per warp, now 439.  Calls that read everything are as fast with three (8 x 3M 53.6 us per step, 55.5 with four).
 // Bound by HBM.  Rows of 32 entries across the lanes with a ballot each took 1.04 ms for 8 x 124M fp32 entries.
-template <typename T>
+// after_read: called when the lane has its entries of the group in registers.
+template <typename T, typename F>
 __device__ __forceinline__ void pack_group(const uint32_t* slot, const Quantiser& qz, float scale, int zero_below, int w, int64_t word,
-                                           int64_t words, uint32_t* __restrict__ out, bool signs = true) {
+                                           int64_t words, uint32_t* __restrict__ out, bool signs, F&& after_read) {
     const int lane = threadIdx.x & 31;
     const bool live = word < words;
     float x[32];
@@ -437,6 +439,7 @@ __device__ __forceinline__ void pack_group(const uint32_t* slot, const Quantiser
             }
         }
     }
+    after_read();
     uint32_t sign_w = 0;
     float mx = 0.0f;
 #pragma unroll
@@ -469,11 +472,11 @@ __device__ __forceinline__ void pack_group(const uint32_t* slot, const Quantiser
 }
 
 template <typename T, bool SKIP>
-__global__ void __launch_bounds__(kBitThreads, 3)
+__global__ void __launch_bounds__(kBitThreads, SKIP ? 4 : 3)
 bit_pack_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* gmax_bits, BitSchedule sc,
                 const int32_t* bit_level, const uint32_t* batch_max, int batches_per_worker, uint32_t* __restrict__ planes, int w_max,
                 int64_t words) {
-    extern __shared__ __align__(16) uint32_t sh_ring[];  // [warps][2][kGroupSlot]
+    extern __shared__ __align__(16) uint32_t sh_ring[];  // [warps][kGroupSlot]
     pdl_enter();
     const int m = blockIdx.y;
     const int level = bit_level[m];
@@ -487,17 +490,18 @@ bit_pack_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* 
     const float scale = (float)(1u << bits);
     const T* row = g + (int64_t)m * ld;
     uint32_t* out = planes + (int64_t)m * (1 + w_max) * words;
-    uint32_t* ring = sh_ring + warp * 2 * kGroupSlot<T>;
+    uint32_t* ring = sh_ring + warp * kGroupSlot<T>;
     const int64_t stride = (int64_t)gridDim.x * (blockDim.x / 32);
     if constexpr (!SKIP) {
         int64_t grp = (int64_t)blockIdx.x * (blockDim.x / 32) + warp;
         fetch_group<T>(row, d, grp, ngroups, ring);
-        for (int it = 0; grp < ngroups; grp += stride, ++it) {
-            fetch_group<T>(row, d, grp + stride, ngroups, ring + ((it + 1) & 1) * kGroupSlot<T>);
-            cp_async_wait<1>();  // this group has landed (the next one may still be in flight)
+        for (; grp < ngroups; grp += stride) {
+            cp_async_wait<0>();
             __syncwarp();
-            pack_group<T>(ring + (it & 1) * kGroupSlot<T>, qz, scale, zero_below, w, grp * 32 + lane, words, out);
-            __syncwarp();  // everyone is done with this slot before the copy after next lands in it
+            pack_group<T>(ring, qz, scale, zero_below, w, grp * 32 + lane, words, out, true, [&]() {
+                __syncwarp();  // the slot has been read by every lane
+                fetch_group<T>(row, d, grp + stride, ngroups, ring);
+            });
         }
     } else {
         constexpr int kPer = 2 * (int)sizeof(T) / 4;  // batches of a group: 2 or 1
@@ -527,13 +531,14 @@ bit_pack_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* 
                 uint32_t* to = out + (base + (__ffs(zero) - 1) * stride) * 32 + lane;
                 for (int j = 1; j <= w; ++j) to[(int64_t)j * words] = 0u;
             }
-            for (int it = 0; grp < ngroups; ++it) {
+            while (grp < ngroups) {
                 const int64_t after = next();
-                fetch_group<T>(row, d, after, ngroups, ring + ((it + 1) & 1) * kGroupSlot<T>);
-                cp_async_wait<1>();  // this group has landed (the next one may still be in flight)
+                cp_async_wait<0>();
                 __syncwarp();
-                pack_group<T>(ring + (it & 1) * kGroupSlot<T>, qz, scale, zero_below, w, grp * 32 + lane, words, out, (grp + 1) * 1024 > d);
-                __syncwarp();  // everyone is done with this slot before the copy after next lands in it
+                pack_group<T>(ring, qz, scale, zero_below, w, grp * 32 + lane, words, out, (grp + 1) * 1024 > d, [&]() {
+                    __syncwarp();  // the slot has been read by every lane
+                    fetch_group<T>(row, d, after, ngroups, ring);
+                });
                 grp = after;
             }
         }
@@ -608,7 +613,7 @@ bit_cluster_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid_
     const int zero_below = zero_code_below(gmax, sc.bits[level]);
     uint32_t* out = planes + (int64_t)m * (1 + w_max) * words;
     for (int i = warp; i < n; i += kBitDenseWarps)
-        pack_group<T>(sh_slots + i * kGroupSlot<T>, qz, scale, zero_below, sc.width[level], (g0 + i) * 32 + lane, words, out);
+        pack_group<T>(sh_slots + i * kGroupSlot<T>, qz, scale, zero_below, sc.width[level], (g0 + i) * 32 + lane, words, out, true, []() {});
 }
 
 // ---- server average of bit-plane messages.  8 x 124M entries, six levels: 372 us with one worker in flight, now 250.
@@ -724,7 +729,7 @@ int bit_blocks(const Workspace& ws, int64_t d, int vec, int M, int waves) {
     return (int)(nb < 1 ? 1 : nb);
 }
 
-size_t bit_pack_smem(size_t elem, int warps) { return (size_t)warps * 2 * 1024 * elem; }
+size_t bit_pack_smem(size_t elem, int warps) { return (size_t)warps * 1024 * elem; }
 
 }  // namespace
 
@@ -835,7 +840,7 @@ static void launch_bit_pack_t(Workspace& ws, const T* g, int64_t d, int M, int64
     const int64_t ngroups = (words + 31) / 32;
     const int warps = (int)std::min<int64_t>(ngroups, kBitThreads / 32);  // of short rows as many blocks as possible fit an SM
     const int64_t by_work = (ngroups + warps - 1) / warps;
-    int64_t nb = ((int64_t)ws.sm_count * 3) / M;  // persistent: three resident blocks per SM, rounded down
+    int64_t nb = ((int64_t)ws.sm_count * (zero_batches(ws) ? 4 : 3)) / M;  // persistent: one wave, rounded down
     if (nb > by_work) nb = by_work;
     if (nb < 1) nb = 1;
     launch_kernel(ws, K_BIT_PACK, zero_batches(ws) ? bit_pack_kernel<T, true> : bit_pack_kernel<T, false>, dim3((unsigned)nb, M), warps * 32, bit_pack_smem(sizeof(T), warps), s, g, d, ld,

@@ -14,6 +14,8 @@ namespace mlmc {
 namespace {
 
 constexpr int kFloatThreads = 256;
+template <typename T>
+constexpr int kFloatBlocks = sizeof(T) == 4 ? 4 : 3;  // of the message kernel, per SM
 
 struct MantissaSchedule {
     int L;
@@ -62,20 +64,21 @@ __device__ __forceinline__ uint32_t plane_word(const uint32_t* x, int bit) {
 // A warp turns 1024 consecutive entries into 32 words of the sign plane and of each mantissa plane and into 1024 exponent
 // bytes.  A lane owns 32 consecutive entries, so every word is collected in the lane's own registers (2 instructions
 // per entry and plane; from 6 planes on one bit transpose for all of them is cheaper).  The entries come through a
-// ring of two shared-memory slots per warp filled by 16-byte asynchronous copies; the 16-byte chunks of a lane are
-// XOR-ed with its number so that the lanes' reads fall into different banks.
+// slot of shared memory per warp filled by 16-byte asynchronous copies: the next group's copy starts when this group's words are in
+// registers.  The 16-byte chunks of a lane are XOR-ed with its number so that the lanes' reads fall into different banks.
 // The draw does not depend on the data (it is the host's); the worker's last block writes the header.
-// Bound by HBM (reads 4 or 2 bytes, writes 1 byte and 1 + w bits per entry).  Ballots over rows of 32 entries took 1.14 ms
+// Bound by HBM (reads 4 or 2 bytes, writes 1 byte and 1 + w bits per entry).  8 x 1M fp32 entries: 29.4 us per step with two slots and
+// three blocks per SM, now 27.5 with one and four (8 x 124M: the same); bf16 rows are 1 % slower with four blocks.  Ballots over rows of 32 entries took 1.14 ms
 // for 8 x 124M fp32 entries (0.72 of the copy rate).
 template <typename T>
-__global__ void __launch_bounds__(kFloatThreads, 3)
+__global__ void __launch_bounds__(kFloatThreads, kFloatBlocks<T>)
 float_pack_kernel(const T* __restrict__ g, int64_t d, int64_t ld, MantissaSchedule sc, const __grid_constant__ DrawnLevels drawn,
                   uint8_t* __restrict__ expo, uint32_t* __restrict__ planes, int w_max, int64_t words,
                   int32_t* out_level, double* out_p_sel, uint32_t* acc, uint32_t* done, int* status) {
     constexpr int kChunks = kGroupChunks<T>;
     constexpr int kSlot = kGroupSlot<T>;
     constexpr int kMantBits = sizeof(T) == 4 ? 23 : 7;
-    extern __shared__ __align__(16) uint32_t sh_ring[];  // [warps][2][kSlot]
+    extern __shared__ __align__(16) uint32_t sh_ring[];  // [warps][kSlot]
     const int m = blockIdx.y;
     const int level = drawn.level[m];
     pdl_enter();
@@ -92,7 +95,7 @@ float_pack_kernel(const T* __restrict__ g, int64_t d, int64_t ld, MantissaSchedu
     const T* row = g + (int64_t)m * ld;
     uint32_t* out = planes + (int64_t)m * (1 + w_max) * words;
     uint8_t* ex = expo + (int64_t)m * words * 32;
-    uint32_t* ring = sh_ring + warp * 2 * kSlot;
+    uint32_t* ring = sh_ring + warp * kSlot;
     const int64_t ngroups = (words + 31) / 32;
     const int64_t stride = (int64_t)gridDim.x * (blockDim.x / 32);
     auto fetch = [&](int64_t grp, uint32_t* slot) { fetch_group<T>(row, d, grp, ngroups, slot); };
@@ -100,18 +103,17 @@ float_pack_kernel(const T* __restrict__ g, int64_t d, int64_t ld, MantissaSchedu
     uint32_t top = 0;  // largest exponent field seen, at the top of the word
     int64_t grp = (int64_t)blockIdx.x * (blockDim.x / 32) + warp;
     fetch(grp, ring);
-    for (int it = 0; grp < ngroups; grp += stride, ++it) {
-        fetch(grp + stride, ring + ((it + 1) & 1) * kSlot);
-        cp_async_wait<1>();
+    for (; grp < ngroups; grp += stride) {
+        cp_async_wait<0>();
         __syncwarp();
-        const uint32_t* slot = ring + (it & 1) * kSlot;
         uint32_t x[32];
 #pragma unroll
         for (int c = 0; c < kChunks; ++c) {
-            const uint4 q = *reinterpret_cast<const uint4*>(slot + group_place<T>(lane, c));
+            const uint4 q = *reinterpret_cast<const uint4*>(ring + group_place<T>(lane, c));
             x[4 * c] = q.x; x[4 * c + 1] = q.y; x[4 * c + 2] = q.z; x[4 * c + 3] = q.w;
         }
-        __syncwarp();  // the slot has been read by every lane: the copy after next may land in it
+        __syncwarp();  // the slot has been read by every lane: the next copy may land in it
+        fetch(grp + stride, ring);
         const int64_t word = grp * 32 + lane;
         const bool live = word < words;
         uint32_t e[8];  // the lane's exponent bytes
@@ -278,7 +280,7 @@ aggregate_float_kernel(const uint8_t* __restrict__ expo, const uint32_t* __restr
     }
 }
 
-size_t float_pack_smem(size_t elem, int warps) { return (size_t)warps * 2 * 1024 * elem; }
+size_t float_pack_smem(size_t elem, int warps) { return (size_t)warps * 1024 * elem; }
 
 }  // namespace
 
@@ -300,7 +302,7 @@ void launch_compress_floatbits(Workspace& ws, const void* g, int dtype, int64_t 
     const int64_t ngroups = (words + 31) / 32;
     const int warps = (int)std::min<int64_t>(ngroups, kFloatThreads / 32);  // of short rows as many blocks as possible fit an SM
     const int64_t by_work = (ngroups + warps - 1) / warps;
-    int64_t nb = ((int64_t)ws.sm_count * 3) / M;  // persistent: three resident blocks per SM, rounded down
+    int64_t nb = ((int64_t)ws.sm_count * (dtype == MLMC_BF16 ? kFloatBlocks<bf16_t> : kFloatBlocks<float>)) / M;  // persistent: one wave, rounded down
     if (nb > by_work) nb = by_work;
     if (nb < 1) nb = 1;
     const DrawnLevels drawn = draw_levels(p, L, seed, step, M);
