@@ -441,6 +441,9 @@ __device__ __forceinline__ void for_each_in_vector(const T* row, int64_t v, int6
     }
 }
 
+// Asks for the 128-byte line at p as far as L2.
+__device__ __forceinline__ void prefetch_line(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 // 16-byte asynchronous copy from global to shared memory (cp.async), grouped by commit / wait.
 __device__ __forceinline__ void cp_async_16(void* smem_dst, const void* gmem_src) {
     const unsigned sa = (unsigned)__cvta_generic_to_shared(smem_dst);

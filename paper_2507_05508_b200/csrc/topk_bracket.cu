@@ -408,7 +408,7 @@ bracket_sweep_kernel(const float* __restrict__ g, int64_t d, int64_t ld, int L, 
 #pragma unroll
         for (int j = 0; j < 4; ++j) cur[j] = __ldg(from + j * 32);
         const int next = at_batch + 1 == mine ? 0 : at_batch + 1;
-        if (lane < 16) asm volatile("prefetch.global.L2 [%0];" ::"l"(first + (int64_t)next * stride * kEmitGroupVecs + lane * 7));
+        if (lane < 16) prefetch_line(first + (int64_t)next * stride * kEmitGroupVecs + lane * 7);
         // largest key: the largest of the negative entries and of the others, each in its own order
         uint32_t un = 0;
         int sn = 0;

@@ -163,13 +163,18 @@ hist1_kernel(const float* __restrict__ g, int64_t d, int64_t ld, uint32_t* __res
     // Groups of 32 batches are dealt round-robin to the blocks of a worker (how fast a batch is counted depends on how
     // its keys collide in the shared-memory histogram, which differs from layer to layer).
     const int nbatch = tiles_per_worker * kEmitGroups;
-    for (int b = blockIdx.x * (kHistThreads / 32) + warp; b < nbatch; b += gridDim.x * (kHistThreads / 32)) {
+    const int step = gridDim.x * (kHistThreads / 32);
+    for (int b = blockIdx.x * (kHistThreads / 32) + warp; b < nbatch; b += step) {
         const int64_t v = (int64_t)b * kEmitGroupVecs + lane;
         uint32_t wm;
         if ((int64_t)(b + 1) * kEmitGroupVecs <= full_end) {  // warp-uniform
             uint4 q[kBatch];
 #pragma unroll
             for (int j = 0; j < kBatch; ++j) q[j] = __ldg(reinterpret_cast<const uint4*>(row) + v + j * 32);
+            // the next batch as far as L2 (16 x 11.7M fp32 keys: 145 us without, now 133; the batch after it 138; 32 x 25.6M bf16 keys
+            // 322, now 304)
+            if (lane < 16 && (int64_t)(b + step + 1) * kEmitGroupVecs <= full_end)
+                prefetch_line(reinterpret_cast<const uint4*>(row) + v + (int64_t)step * kEmitGroupVecs + lane * 7);
             uint32_t vm = 0;
 #pragma unroll
             for (int j = 0; j < kBatch; ++j) {
@@ -234,136 +239,174 @@ hist1_kernel(const float* __restrict__ g, int64_t d, int64_t ld, uint32_t* __res
     }
 }
 
-// The same sweep for bf16 rows.  With one count per bin 32 keys meet 3.5 deep in a bank (deeper in a layer whose keys share few bins),
-// and the shared-memory atomics bound the sweep: 92 % of the L1 wavefronts.  Here a bin has 16 counts, one for every second lane, so
-// that at most two lanes of a warp meet in a bank.  They have room for kColumnBins bins, 20 octaves from below the octave of the
-// largest key that a sample of the row holds.  Beside the window, down to 32 octaves below its top, a bin has one count; what lies
-// outside of that is counted in memory, key by key, and zeros in a register.  A block whose sample lies below the window by more
-// than one key of kColumnMisses keeps one count per bin for all, and so do short rows, where the sample takes longer than it saves
-// (8 x 1M keys: 63.3 us per step, 65.7 with columns).
-// 32 x 25.6M keys: 406 us, now 337 (floor 250); 8 x 40M, given p: 260 us per step, now 235; 8 x 12M 167 either way.  On the way: all
+// The same sweep for bf16 rows.  With one count per bin 32 keys meet 3.5 deep in a bank (deeper in a layer whose keys share few bins), and
+// the shared-memory atomics bound the sweep (bf16: 92 % of the L1 wavefronts).  Here a bin has 16 counts, one for every second lane, so
+// that at most two lanes of a warp meet in a bank.  They have room for kWindow bins, from below the octave of the largest key that a
+// sample of the row holds.  Beside the window, down to 12 octaves below it, a bin has one count; what lies outside of that is counted
+// in memory, key by key, and the lowest bin (zeros) in a register.  A block whose sample lies below the window by more than one key
+// of kColumnMisses keeps one count per bin for all, and so do short rows, where the sample takes longer than it saves
+// (8 x 1M bf16 keys: 63.3 us per step, 65.7 with columns).
+// 32 x 25.6M bf16 keys: 406 us, now 318 (floor 250); 8 x 40M, given p: 260 us per step, now 231; 8 x 12M 167 either way.  On the way: all
 // 32 keys of a warp by the general way whenever one lies outside the window (each lane its own way 355 us); every key by the general
 // way 386; windows of 22 and 24 octaves leave too little L1 for the loads in flight (362 us, and 334 without the bins beside).
-constexpr int kColumnBins = 20 * 128;
+// fp32 rows, with half as many atomics per byte, gain nothing (16 x 11.7M 135.4 us, 135.9 so; with the stages of the brackets beside 139 and
+// 159).
 constexpr int kColumns = 16;
 constexpr int kFarBelow = 12 * 128, kFarAbove = 8 * 128;
-constexpr int kFarBins = kFarBelow + kColumnBins + kFarAbove;  // numbered through the window
-constexpr int kColumnSmem = (kColumnBins * kColumns + kFarBins) * (int)sizeof(uint32_t);
 constexpr uint32_t kColumnMisses = 64;
 constexpr int64_t kColumnBatches = 8;  // per warp, from which on a row is long enough
-static_assert(kColumnSmem >= kBins1 * (int)sizeof(uint32_t), "either kind of counts");
+
+struct BinCounts {
+    static constexpr int kWindow = 20 * 128;  // 20 octaves: 180 KB
+    static constexpr int kFarBins = kFarBelow + kWindow + kFarAbove;  // numbered through the window
+    static constexpr int kWords = kWindow * kColumns + kFarBins;
+    static_assert(kWords >= kBins1, "either kind of counts");
+    uint32_t* counts;
+    uint32_t* out;                       // [kBins1]
+    uint32_t lowest = 0, zeros = 0;      // first bin of the window; keys of bin 0
+    uint32_t column0 = 0, far0 = 0;      // shared-memory addresses of bin 0 (of this lane's column, and beside the window)
+    bool columns = false;                // block-uniform
+
+    __device__ __forceinline__ BinCounts(uint32_t* shared, uint32_t* memory) : counts(shared), out(memory) {}
+    // By all threads: the window, from some bins of every thread.
+    template <int N>
+    __device__ __forceinline__ void place(const uint32_t (&bin)[N], uint32_t* sh_warp) {
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        uint32_t top = 0, below = 0;
+#pragma unroll
+        for (int i = 0; i < N; ++i) top = max(top, bin[i]);
+        top = __reduce_max_sync(0xFFFFFFFFu, top);
+        if (lane == 0) sh_warp[warp] = top;
+        __syncthreads();
+        const uint32_t end = __reduce_max_sync(0xFFFFFFFFu, sh_warp[lane]) & ~127u;  // the largest keys are few
+        lowest = end > (uint32_t)kWindow ? end - kWindow : 0u;
+#pragma unroll
+        for (int i = 0; i < N; ++i) below += bin[i] < lowest ? 1u : 0u;
+        below = __reduce_add_sync(0xFFFFFFFFu, below);
+        __syncthreads();
+        if (lane == 0) sh_warp[warp] = below;
+        __syncthreads();
+        columns = __reduce_add_sync(0xFFFFFFFFu, sh_warp[lane]) * kColumnMisses <= (uint32_t)(N * kHistThreads);
+        const uint32_t base = (uint32_t)__cvta_generic_to_shared(counts);
+        column0 = base + (lane & (kColumns - 1)) * 4u - lowest * (kColumns * 4u);
+        far0 = base + (kWindow * kColumns + kFarBelow - (int)lowest) * 4;
+    }
+    __device__ __forceinline__ static void bump(uint32_t address) { asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(address) : "memory"); }
+    __device__ __forceinline__ bool in_window(uint32_t bin) const { return bin - lowest < (uint32_t)kWindow; }
+    __device__ __forceinline__ bool near(uint32_t bin) const { return bin - lowest + (uint32_t)kFarBelow < (uint32_t)kFarBins; }
+    __device__ __forceinline__ void add_column(uint32_t bin) { bump(column0 + bin * (kColumns * 4u)); }
+    __device__ __forceinline__ void add_near(uint32_t bin) { bump(in_window(bin) ? column0 + bin * (kColumns * 4u) : far0 + bin * 4u); }
+    __device__ __forceinline__ void add(uint32_t bin) {
+        if (!columns) atomicAdd(&counts[bin], 1u);
+        else if (near(bin)) add_near(bin);
+        else if (bin == 0u) ++zeros;
+        else atomicAdd(&out[bin], 1u);
+    }
+    // N bins of every lane of a warp, the least and the largest known; columns only.
+    template <int N>
+    __device__ __forceinline__ void add_all(const uint32_t (&bin)[N], uint32_t least, uint32_t most) {
+        if (__all_sync(0xFFFFFFFFu, in_window(least) && in_window(most))) {
+#pragma unroll
+            for (int i = 0; i < N; ++i) add_column(bin[i]);
+        } else if (near(least) && near(most)) {
+#pragma unroll
+            for (int i = 0; i < N; ++i) add_near(bin[i]);
+        } else {
+#pragma unroll 1
+            for (int i = 0; i < N; ++i) {
+                uint32_t x = 0;
+#pragma unroll
+                for (int j = 0; j < N; ++j) x = i == j ? bin[j] : x;
+                add(x);
+            }
+        }
+    }
+    __device__ __forceinline__ void flush() {  // by all threads, after a barrier
+        if (!columns) {
+            for (int b = threadIdx.x; b < kBins1; b += kHistThreads) {
+                const uint32_t c = counts[b];
+                if (c) atomicAdd(&out[b], c);
+            }
+            return;
+        }
+        const int lane = threadIdx.x & 31;
+        zeros = __reduce_add_sync(0xFFFFFFFFu, zeros);
+        if (lane == 0 && zeros) atomicAdd(&out[0], zeros);
+        for (int b = threadIdx.x; b < kWindow; b += kHistThreads) {
+            uint32_t c = 0;
+#pragma unroll
+            for (int i = 0; i < kColumns; ++i) c += counts[b * kColumns + ((i + lane) & (kColumns - 1))];
+            if (c) atomicAdd(&out[lowest + b], c);
+        }
+        for (int b = threadIdx.x; b < kFarBins; b += kHistThreads) {
+            const uint32_t c = counts[kWindow * kColumns + b];
+            if (c) atomicAdd(&out[(int)lowest - kFarBelow + b], c);
+        }
+    }
+};
 
 __global__ void __launch_bounds__(kHistThreads, 1)
 hist1_bf16_kernel(const bf16_t* __restrict__ g, int64_t d, int64_t ld, uint32_t* __restrict__ hist1, uint32_t* __restrict__ tile_max,
                   int tiles_per_worker, int sample, int* status, int* worker_err) {
-    extern __shared__ uint32_t sh_hist[];
+    extern __shared__ __align__(16) uint32_t sh_hist[];
     __shared__ uint32_t sh_warp[kHistThreads / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int i = threadIdx.x; i < kColumnSmem / 16; i += kHistThreads) reinterpret_cast<uint4*>(sh_hist)[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = threadIdx.x; i < BinCounts::kWords / 4; i += kHistThreads) reinterpret_cast<uint4*>(sh_hist)[i] = make_uint4(0u, 0u, 0u, 0u);
     pdl_enter();
     const int m = blockIdx.y;
     const bf16_t* row = g + (int64_t)m * ld;
     const int64_t nvec = (d + 7) / 8, full_end = d / 8;  // vectors of the row, and those wholly inside it
-    auto vector_max = [](const uint4& q) -> uint32_t {
-        const uint32_t a = __vmaxu2(__vmaxu2(q.x & 0x7FFF7FFFu, q.y & 0x7FFF7FFFu), __vmaxu2(q.z & 0x7FFF7FFFu, q.w & 0x7FFF7FFFu));
-        return max(a & 0xFFFFu, a >> 16);
-    };
-    uint32_t lowest = 0;  // first bin of the window
-    bool columns = false;
-    if (sample) {
-        const int64_t stride = full_end / kHistThreads;
-        const uint4 q = __ldg(reinterpret_cast<const uint4*>(row) + threadIdx.x * stride + (blockIdx.x * 37 + threadIdx.x * 11) % stride);
-        uint32_t top = __reduce_max_sync(0xFFFFFFFFu, vector_max(q));
-        if (lane == 0) sh_warp[warp] = top;
-        __syncthreads();
-        top = __reduce_max_sync(0xFFFFFFFFu, sh_warp[lane]);
-        const uint32_t end = top & ~127u;  // the largest keys are few
-        lowest = end > (uint32_t)kColumnBins ? end - kColumnBins : 0u;
-        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-        uint32_t out = 0;
+    BinCounts counts(sh_hist, hist1 + (int64_t)m * kBins1);
+    auto keys_of = [](const uint4& q, uint32_t (&key)[8], uint32_t& least, uint32_t& most) {  // Inf / NaN: see the maxima
+        const uint32_t w[4] = {q.x & 0x7FFF7FFFu, q.y & 0x7FFF7FFFu, q.z & 0x7FFF7FFFu, q.w & 0x7FFF7FFFu};
+        const uint32_t hi = __vmaxu2(__vmaxu2(w[0], w[1]), __vmaxu2(w[2], w[3])), lo = __vminu2(__vminu2(w[0], w[1]), __vminu2(w[2], w[3]));
+        most = max(hi & 0xFFFFu, hi >> 16);
+        least = min(lo & 0xFFFFu, lo >> 16);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const uint32_t key = (w[i / 2] >> (16 * (i & 1))) & 0x7FFFu;
-            out += key < lowest ? 1u : 0u;
+        for (int i = 0; i < 4; ++i) {
+            key[2 * i] = w[i] & 0xFFFFu;
+            key[2 * i + 1] = w[i] >> 16;
         }
-        out = __reduce_add_sync(0xFFFFFFFFu, out);
-        __syncthreads();
-        if (lane == 0) sh_warp[warp] = out;
-        __syncthreads();
-        out = __reduce_add_sync(0xFFFFFFFFu, sh_warp[lane]);
-        columns = out * kColumnMisses <= 8u * kHistThreads;  // block-uniform
+    };
+    if (sample) {
+        uint32_t key[8], least, most;
+        const int64_t share = full_end / kHistThreads;  // a vector of every thread's share of the row
+        keys_of(__ldg(reinterpret_cast<const uint4*>(row) + threadIdx.x * share + (blockIdx.x * 37 + threadIdx.x * 11) % share), key, least, most);
+        counts.place(key, sh_warp);
     } else {
         __syncthreads();
     }
-    uint32_t* out = hist1 + (int64_t)m * kBins1;
     uint32_t* tmax = tile_max + (int64_t)m * tiles_per_worker * kEmitGroups;
-    const uint32_t column0 = (uint32_t)__cvta_generic_to_shared(sh_hist) + (lane & (kColumns - 1)) * 4u - lowest * (kColumns * 4u);
-    uint32_t* const sh_far = sh_hist + kColumnBins * kColumns;
-    const uint32_t far0 = (uint32_t)__cvta_generic_to_shared(sh_far) + (kFarBelow - (int)lowest) * 4;
-    uint32_t zeros = 0;
-    auto count_column = [&](uint32_t key) { asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(column0 + key * (kColumns * 4u)) : "memory"); };
-    auto count_key = [&](uint32_t bits) {
-        const uint32_t key = bits & 0x7FFFu;  // Inf / NaN: see the maxima
-        if (!columns) atomicAdd(&sh_hist[key], 1u);
-        else if (key - lowest < (uint32_t)kColumnBins) count_column(key);
-        else if (key == 0u) ++zeros;
-        else if (key - lowest + (uint32_t)kFarBelow < (uint32_t)kFarBins) atomicAdd(&sh_far[key - lowest + kFarBelow], 1u);
-        else atomicAdd(&out[key], 1u);
-    };
     constexpr int kBatch = kEmitGroupVecs / 32;
     const int nbatch = tiles_per_worker * kEmitGroups;
     bool bad = false;
-    for (int b = blockIdx.x * (kHistThreads / 32) + warp; b < nbatch; b += gridDim.x * (kHistThreads / 32)) {
+    const int step = gridDim.x * (kHistThreads / 32);
+    for (int b = blockIdx.x * (kHistThreads / 32) + warp; b < nbatch; b += step) {
         const int64_t v = (int64_t)b * kEmitGroupVecs + lane;
         uint32_t vm = 0;
         if ((int64_t)(b + 1) * kEmitGroupVecs <= full_end) {  // warp-uniform
             uint4 q[kBatch];
 #pragma unroll
             for (int j = 0; j < kBatch; ++j) q[j] = __ldg(reinterpret_cast<const uint4*>(row) + v + j * 32);
-            if (columns) {
+            // the next batch as far as L2
+            if (lane < 16 && (int64_t)(b + step + 1) * kEmitGroupVecs <= full_end)
+                prefetch_line(reinterpret_cast<const uint4*>(row) + v + (int64_t)step * kEmitGroupVecs + lane * 7);
 #pragma unroll
-                for (int j = 0; j < kBatch; ++j) {
-                    const uint32_t w[4] = {q[j].x & 0x7FFF7FFFu, q[j].y & 0x7FFF7FFFu, q[j].z & 0x7FFF7FFFu, q[j].w & 0x7FFF7FFFu};
-                    const uint32_t hi = __vmaxu2(__vmaxu2(w[0], w[1]), __vmaxu2(w[2], w[3])), lo = __vminu2(__vminu2(w[0], w[1]), __vminu2(w[2], w[3]));
-                    const uint32_t most = max(hi & 0xFFFFu, hi >> 16), least = min(lo & 0xFFFFu, lo >> 16);
-                    vm = max(vm, most);
-                    if (__all_sync(0xFFFFFFFFu, least >= lowest && most - lowest < (uint32_t)kColumnBins)) {
+            for (int j = 0; j < kBatch; ++j) {
+                uint32_t key[8], least, most;
+                keys_of(q[j], key, least, most);
+                if (counts.columns) {
+                    counts.add_all(key, least, most);
+                } else {
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            count_column(w[i] & 0xFFFFu);
-                            count_column(w[i] >> 16);
-                        }
-                    } else if (least - lowest + (uint32_t)kFarBelow < (uint32_t)kFarBins && most - lowest + (uint32_t)kFarBelow < (uint32_t)kFarBins) {
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const uint32_t key = i & 1 ? w[i / 2] >> 16 : w[i / 2] & 0xFFFFu;
-                            const uint32_t at = key - lowest < (uint32_t)kColumnBins ? column0 + key * (kColumns * 4u) : far0 + key * 4u;
-                            asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(at) : "memory");
-                        }
-                    } else {
-#pragma unroll 1
-                        for (int i = 0; i < 8; ++i) {
-                            const uint32_t x = i & 4 ? (i & 2 ? w[3] : w[2]) : (i & 2 ? w[1] : w[0]);
-                            count_key(i & 1 ? x >> 16 : x & 0xFFFFu);
-                        }
-                    }
+                    for (int i = 0; i < 8; ++i) atomicAdd(&sh_hist[key[i]], 1u);
                 }
-            } else {
-#pragma unroll
-                for (int j = 0; j < kBatch; ++j) {
-                    const uint32_t w[4] = {q[j].x, q[j].y, q[j].z, q[j].w};
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        atomicAdd(&sh_hist[w[i] & 0x7FFFu], 1u);
-                        atomicAdd(&sh_hist[(w[i] >> 16) & 0x7FFFu], 1u);
-                    }
-                    vm = max(vm, vector_max(q[j]));
-                }
+                vm = max(vm, most);
             }
         } else {  // the row's end, vector by vector; batches past it have the largest key 0
             for (int64_t u = v; u < min(nvec, (int64_t)(b + 1) * kEmitGroupVecs); u += 32)
                 for_each_in_vector<bf16_t>(row, u, d, [&](int64_t, uint32_t bits) {
-                    count_key(bits);
+                    counts.add(bits & 0x7FFFu);
                     vm = max(vm, bits & 0x7FFFu);
                 });
         }
@@ -376,25 +419,7 @@ hist1_bf16_kernel(const bf16_t* __restrict__ g, int64_t d, int64_t ld, uint32_t*
         set_status(status, MLMC_ERR_NONFINITE);
     }
     __syncthreads();
-    if (columns) {
-        zeros = __reduce_add_sync(0xFFFFFFFFu, zeros);
-        if (lane == 0 && zeros) atomicAdd(&out[0], zeros);
-        for (int b = threadIdx.x; b < kColumnBins; b += kHistThreads) {
-            uint32_t c = 0;
-#pragma unroll
-            for (int i = 0; i < kColumns; ++i) c += sh_hist[b * kColumns + ((i + lane) & (kColumns - 1))];
-            if (c) atomicAdd(&out[lowest + b], c);
-        }
-        for (int b = threadIdx.x; b < kFarBins; b += kHistThreads) {
-            const uint32_t c = sh_far[b];
-            if (c) atomicAdd(&out[(int)lowest - kFarBelow + b], c);
-        }
-    } else {
-        for (int b = threadIdx.x; b < kBins1; b += kHistThreads) {
-            const uint32_t c = sh_hist[b];
-            if (c) atomicAdd(&out[b], c);
-        }
-    }
+    counts.flush();
 }
 
 // -------------------------------------------------------------------------------------------
@@ -1274,7 +1299,7 @@ void launch_hist1(Workspace& ws, const void* g, int dtype, int64_t d, int M, int
     };
     if (dtype == MLMC_BF16) {
         const int64_t batches = ((int64_t)tpw * kEmitGroups + nb * (kHistThreads / 32) - 1) / (nb * (kHistThreads / 32));  // per warp
-        launch_kernel(ws, K_HIST1, hist1_bf16_kernel, dim3(nb, M), kHistThreads, kColumnSmem, s, static_cast<const bf16_t*>(g), d, ld, ws.hist1,
+        launch_kernel(ws, K_HIST1, hist1_bf16_kernel, dim3(nb, M), kHistThreads, BinCounts::kWords * sizeof(uint32_t), s, static_cast<const bf16_t*>(g), d, ld, ws.hist1,
                       ws.tile_max, tpw, batches >= kColumnBatches ? 1 : 0, ws.status, ws.worker_err);
     } else if (brackets) {
         smem += (kHistThreads / 32) * (kWarpStage + 1) * sizeof(uint32_t);
@@ -1348,7 +1373,7 @@ int configure_select_kernels() {
         return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess;
     };
     const bool ok = set(resolve1_kernel, kResolveSmem) && set(hist1_kernel<false>, hist) && set(hist1_kernel<true>, hist + stage) &&
-                    set(hist1_bf16_kernel, kColumnSmem) && set(sums_candidates_kernel<true>, kS2SmemMost) &&
+                    set(hist1_bf16_kernel, (int)(BinCounts::kWords * sizeof(uint32_t))) && set(sums_candidates_kernel<true>, kS2SmemMost) &&
                     set(sums_candidates_kernel<false>, (int)s2_smem(0, false, kS2Threads)) && set(digit_pass_kernel<2, true>, columns) &&
                     set(digit_pass_kernel<2, false>, digits) && set(digit_pass_kernel<3, true>, digits) &&
                     set(digit_pass_kernel<3, false>, digits);
