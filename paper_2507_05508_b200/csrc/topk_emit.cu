@@ -30,11 +30,15 @@ namespace mlmc {
 namespace {
 
 constexpr int kBandThreads = 256;               // 8 warps per block, one tile per warp at a time
-constexpr int kWriteSlots = 3;                  // shared-memory batches per warp of the write pass,
-constexpr int kWriteBlocks = 3;                 // and blocks per SM
+// Shared-memory batches per warp of the write pass, and blocks per SM.  fp32: 8 x 124M 150 us with three and three, 140 with two and
+// four (141 with two and five).  bf16: 32 x 25.6M 185 and 177, but 8 x 3M 95 us per step and 98.7.
+template <typename T>
+constexpr int kWriteSlots = EmitWord<T>::S == 1 ? 2 : 3;
+template <typename T>
+constexpr int kWriteBlocks = EmitWord<T>::S == 1 ? 4 : 3;
 // words of shared memory per warp of the write pass: the batches and the offsets of one batch's entries
 template <typename T>
-constexpr int kWriteWords = kWriteSlots * kEmitRows * 32 + kEmitRows * 32 * EmitWord<T>::S / 2;
+constexpr int kWriteWords = kWriteSlots<T> * kEmitRows * 32 + kEmitRows * 32 * EmitWord<T>::S / 2;
 
 // Where a tile's counts are added up: {C, A, B, batches} per item, super-item and hyper-item of every worker.
 struct CountLevels {
@@ -137,15 +141,15 @@ band_count_kernel(const T* __restrict__ g, int64_t d, int64_t ld, int tiles_per_
 
 // Pass 2: every listed tile is read again and its band entries are written at their final positions.
 template <typename T>
-__global__ void __launch_bounds__(kBandThreads, kWriteBlocks)
+__global__ void __launch_bounds__(kBandThreads, kWriteBlocks<T>)
 band_write_kernel(const T* __restrict__ g, int64_t d, int64_t ld, int tiles_per_worker, int M, const EmitParams* emit,
                   const uint4* tiles, CountLevels lv, const uint2* list, const uint32_t* list_n,
                   uint32_t* __restrict__ idx_out, float* __restrict__ val_out, int64_t capacity, uint32_t* group_n,
                   int* status) {
     using EW = EmitWord<T>;
     constexpr int S = EW::S;
-    // every warp stages its batches in a ring of three shared-memory slots: two copies are in flight while a
-    // batch is ranked, and the words of a batch can be addressed by a run-time index
+    // every warp stages its batches in a ring of shared-memory slots: the next copies are in flight while a batch is ranked, and the
+    // words of a batch can be addressed by a run-time index
     extern __shared__ __align__(16) uint32_t sh_dyn[];  // [warps][kWriteWords]
     pdl_enter();
     const int lane = threadIdx.x & 31;
@@ -170,7 +174,7 @@ band_write_kernel(const T* __restrict__ g, int64_t d, int64_t ld, int tiles_per_
     }
     const uint32_t total = *list_n;
     uint32_t* ring = sh_dyn + (threadIdx.x >> 5) * kWriteWords<T>;
-    uint16_t* stage = reinterpret_cast<uint16_t*>(ring + kWriteSlots * kBatchWords);
+    uint16_t* stage = reinterpret_cast<uint16_t*>(ring + kWriteSlots<T> * kBatchWords);
     uint2 next = gw < (int)total ? list[gw] : make_uint2(0u, 0u);
     for (uint32_t f = gw; f < total; f += warps) {
         const uint2 entry = next;
@@ -213,16 +217,20 @@ band_write_kernel(const T* __restrict__ g, int64_t d, int64_t ld, int tiles_per_
         for (int it = 0; todo; ++it) {
             const int b = __ffs(todo) - 1;
             todo &= todo - 1u;
-            __syncwarp();  // the batch before this one has been read by every lane: its slot takes the copy two ahead
-            if (ahead) {
-                copy_batch_async<T>(row, d, tile, __ffs(ahead) - 1, lane, ring + ((it + 2) % kWriteSlots) * kBatchWords);
-                ahead &= ahead - 1u;
-            }
-            cp_async_commit();  // one group per step, empty at the end of the tile
-            cp_async_wait<2>();  // this batch has landed
+            auto copy_two_ahead = [&]() {  // into a slot whose batch has been read by every lane
+                __syncwarp();
+                if (ahead) {
+                    copy_batch_async<T>(row, d, tile, __ffs(ahead) - 1, lane, ring + ((it + 2) % kWriteSlots<T>) * kBatchWords);
+                    ahead &= ahead - 1u;
+                }
+                cp_async_commit();  // one group per step, empty at the end of the tile
+            };
+            if (kWriteSlots<T> == 3) copy_two_ahead();
+            cp_async_wait<kWriteSlots<T> == 3 ? 2 : 1>();  // this batch has landed
             __syncwarp();
             const uint32_t e0 = (uint32_t)((tile * kEmitTile + (int64_t)b * kBatchWords) * S);
-            emit_batch<T>(ring + (it % kWriteSlots) * kBatchWords, stage, band, tile_ties, e0, run, idx_w, val_w, capacity);
+            emit_batch<T>(ring + (it % kWriteSlots<T>) * kBatchWords, stage, band, tile_ties, e0, run, idx_w, val_w, capacity);
+            if (kWriteSlots<T> == 2) copy_two_ahead();
         }
     }
     cp_async_wait<0>();
@@ -517,7 +525,7 @@ void launch_emit_t(Workspace& ws, const T* g, int dtype, int64_t d, int M, int64
     auto blocks = [&](int per_sm) { return (unsigned)std::min<int64_t>(by_work, (int64_t)ws.sm_count * per_sm * 2); };
     launch_kernel(ws, K_BAND_COUNT, band_count_kernel<T>, dim3(blocks(resident)), kBandThreads, (size_t)M * sizeof(uint2), s, g, d,
                   ld, tpw, M, ws.emit, ws.tile_desc, lv, ws.tile_list, ws.list_n);
-    launch_kernel(ws, K_EMIT, band_write_kernel<T>, dim3(blocks(kWriteBlocks)), kBandThreads, smem_w, s, g, d, ld, tpw, M, ws.emit,
+    launch_kernel(ws, K_EMIT, band_write_kernel<T>, dim3(blocks(kWriteBlocks<T>)), kBandThreads, smem_w, s, g, d, ld, tpw, M, ws.emit,
                   ws.tile_desc, lv, ws.tile_list, ws.list_n, out.idx, out.val, out.capacity, ws.group_n, ws.status);
 }
 
