@@ -441,6 +441,30 @@ __device__ __forceinline__ void for_each_in_vector(const T* row, int64_t v, int6
     }
 }
 
+// A warp's 1024 histogram bins in coalesced vectors: lane l has the vectors i * 32 + l of the 256.
+__device__ __forceinline__ void load_bins(const uint32_t* bins, uint4 (&x)[8]) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) x[i] = reinterpret_cast<const uint4*>(bins)[i * 32 + (threadIdx.x & 31)];
+}
+// Hands every lane the 32 bins from 32 * mine through shared memory (rows: 256 vectors per warp; vector j of bin group t at j ^ t, so that
+// neither side meets in a bank).  Read directly, every load touches 32 lines (16 x 11.7M entries, given p: 254 us per step, 251 so).
+__device__ __forceinline__ void hand_over_bins(const uint4 (&x)[8], uint4* rows, int mine, uint32_t (&cnt)[32]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int owner = i * 4 + (lane >> 3);
+        rows[owner * 8 + ((lane ^ owner) & 7)] = x[i];
+    }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const uint4 y = rows[mine * 8 + ((i ^ mine) & 7)];
+        cnt[4 * i] = y.x; cnt[4 * i + 1] = y.y; cnt[4 * i + 2] = y.z; cnt[4 * i + 3] = y.w;
+    }
+}
+
+constexpr size_t kBinRowsSmem = (size_t)kBins1 * sizeof(uint32_t);  // rows of 32 warps
+
 // Asks for the 128-byte line at p as far as L2.
 __device__ __forceinline__ void prefetch_line(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 

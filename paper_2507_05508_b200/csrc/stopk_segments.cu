@@ -117,17 +117,18 @@ segment_resolve_kernel(uint32_t* hist1, int m0, uint32_t sort_all, uint32_t sort
     __shared__ uint32_t sh_warp[32], sh_most[32];
     pdl_enter();
     const int row = blockIdx.x, m = m0 + row;
+    const int group = kSegThreads - 1 - (int)threadIdx.x, warp = threadIdx.x >> 5;
+    uint4 vectors[8];
+    load_bins(hist1 + (int64_t)m * kBins1 + (31 - warp) * 1024, vectors);
     if (worker_err[m]) {
         if (threadIdx.x == 0) sc.head[row].sorted = 0u;
         return;
     }
-    const int group = kSegThreads - 1 - (int)threadIdx.x;
     uint4* src = reinterpret_cast<uint4*>(hist1 + (int64_t)m * kBins1 + group * 32);
     uint32_t cnt[32];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const uint4 x = src[i];
-        cnt[4 * i] = x.x; cnt[4 * i + 1] = x.y; cnt[4 * i + 2] = x.z; cnt[4 * i + 3] = x.w;
+    {
+        extern __shared__ __align__(16) uint4 sh_vectors[];  // [32 warps][256]
+        hand_over_bins(vectors, sh_vectors + warp * 256, group & 31, cnt);
     }
     uint32_t sum = 0, total;
 #pragma unroll
@@ -838,7 +839,9 @@ int rows_within(size_t bytes, int most, int64_t d, int64_t L) {
 int configure_segment_kernels() {
     const bool ok =
         cudaFuncSetAttribute(segment_sweep_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSegSweepSmem) == cudaSuccess &&
-        cudaFuncSetAttribute(segment_sweep_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSegSweepSmem) == cudaSuccess;
+        cudaFuncSetAttribute(segment_sweep_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSegSweepSmem) == cudaSuccess &&
+        cudaFuncSetAttribute(segment_resolve_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBinRowsSmem) == cudaSuccess &&
+        cudaFuncSetAttribute(segment_resolve_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBinRowsSmem) == cudaSuccess;
     return ok ? MLMC_OK : MLMC_ERR_CUDA;
 }
 
@@ -870,7 +873,7 @@ void launch_segments(Workspace& ws, const void* g, int dtype, int64_t d, int M, 
     for (int m0 = 0; m0 < M; m0 += together) {
         const int rows = std::min(together, M - m0);
         auto resolve = [&](auto kernel) {
-            launch_kernel(ws, K_SEG_RESOLVE, kernel, dim3(rows), kSegThreads, 0, s, ws.hist1, m0, sort_from(du, rows),
+            launch_kernel(ws, K_SEG_RESOLVE, kernel, dim3(rows), kSegThreads, kBinRowsSmem, s, ws.hist1, m0, sort_from(du, rows),
                           std::max(kFewEqual, du / 32), sl, nl, sc, ws.worker_err);
         };
         auto norms = [&](auto norm, auto draw) {

@@ -236,23 +236,50 @@ band_write_kernel(const T* __restrict__ g, int64_t d, int64_t ld, int tiles_per_
     cp_async_wait<0>();
 }
 
-// offsets[m][t] = first message entry of worker m whose index is >= t * kAggTile  (t = 0..ntiles)
-__global__ void agg_offsets_kernel(const uint32_t* idx, const int64_t* count, const int32_t* level, int64_t capacity, int M,
-                                   int ntiles, uint32_t* offsets) {
-    pdl_enter();
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)M * (ntiles + 1)) return;
-    const int m = (int)(i / (ntiles + 1)), t = (int)(i % (ntiles + 1));
-    const int64_t n = (level[m] < 0) ? 0 : count[m];
-    const uint32_t* a = idx + (int64_t)m * capacity;
-    const uint64_t target = (uint64_t)t * kAggTile;
-    int64_t lo = 0, hi = n;
-    while (lo < hi) {
-        const int64_t mid = (lo + hi) >> 1;
-        if ((uint64_t)a[mid] < target) lo = mid + 1; else hi = mid;
+// First of the n entries of an index-sorted list that is not below `target`, by 2^lanes_log2 neighbouring lanes (of a warp that is here
+// with all its lanes): of the entries that are left, every lane looks at the first of its share.  One lane: halves.
+__device__ __forceinline__ uint32_t first_not_below(const uint32_t* __restrict__ a, uint32_t n, uint64_t target, int lanes_log2) {
+    const int lane = threadIdx.x & 31, part = lane & ((1 << lanes_log2) - 1);
+    uint32_t lo = 0, hi = n;
+    if (lanes_log2 == 0) {
+        while (lo < hi) {
+            const uint32_t mid = lo + ((hi - lo) >> 1);
+            if ((uint64_t)__ldg(&a[mid]) < target) lo = mid + 1u; else hi = mid;
+        }
+        return lo;
     }
-    offsets[i] = (uint32_t)lo;
+    while (__any_sync(0xFFFFFFFFu, lo < hi)) {
+        const uint32_t left = hi - lo;  // wraps where the search has ended: that lane looks at nothing
+        auto place = [&](uint32_t l) { return lo + (uint32_t)(((uint64_t)left * l) >> lanes_log2); };
+        const bool below = lo < hi && (uint64_t)__ldg(&a[place((uint32_t)part)]) < target;
+        const uint32_t votes = __ballot_sync(0xFFFFFFFFu, below) >> (lane - part);
+        const uint32_t c = (uint32_t)__popc(lanes_log2 == 5 ? votes : votes & ((1u << (1 << lanes_log2)) - 1u));
+        if (lo < hi) {
+            const uint32_t from = c ? place(c - 1u) + 1u : lo, to = c == 0u ? lo : c >> lanes_log2 ? hi : place(c);
+            lo = from;
+            hi = to;
+        }
+    }
+    return lo;
 }
+
+// offsets[m][t] = first message entry of worker m whose index is >= t * kAggTile  (t = 0..ntiles), by 2^lanes_log2 lanes each: four
+// take half as many loads one after the other (8 x 3M 12.6 us, now 10.5), one where so many searches are bound by their loads
+// (8 x 124M 18 us, with two lanes 26).
+constexpr int64_t kFewOffsets = 1 << 17;
+inline int offset_lanes(int64_t n_off) { return n_off <= kFewOffsets ? 2 : 0; }
+__global__ void __launch_bounds__(256)
+agg_offsets_kernel(const uint32_t* idx, const int64_t* count, const int32_t* level, int64_t capacity, int M, int ntiles, int lanes_log2,
+                   uint32_t* offsets) {
+    pdl_enter();
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> lanes_log2;
+    const bool there = i < (int64_t)M * (ntiles + 1);
+    const int m = there ? (int)(i / (ntiles + 1)) : 0, t = there ? (int)(i % (ntiles + 1)) : 0;
+    const uint32_t n = there && level[m] >= 0 ? (uint32_t)count[m] : 0u;
+    const uint32_t at = first_not_below(idx + (int64_t)m * capacity, n, (uint64_t)t * kAggTile, lanes_log2);
+    if (there && (threadIdx.x & ((1 << lanes_log2) - 1)) == 0) offsets[i] = at;
+}
+inline unsigned offset_blocks(int64_t n_off) { return (unsigned)(((n_off << offset_lanes(n_off)) + 255) / 256); }
 
 // M is at most kEmitMaxWorkers: the offsets of all workers for one tile are fetched together.
 __global__ void __launch_bounds__(256)
@@ -414,25 +441,12 @@ aggregate_topk_direct_kernel(const uint32_t* __restrict__ idx, const float* __re
     pdl_enter();
     const int lane = threadIdx.x & 31;
     const int64_t base = (int64_t)blockIdx.x * TILE;
-    {   // An edge is the first entry that is not below its coordinate.  Of the `hi - lo` entries that are left, every lane looks at
-        // the first of its share.
+    {   // an edge is the first entry that is not below its coordinate
         const int edge = threadIdx.x >> lanes_log2, m = edge >> 1, part = threadIdx.x & ((1 << lanes_log2) - 1);
         const uint64_t target = (uint64_t)base + (edge & 1 ? TILE : 0);
-        const uint32_t* a = idx + (int64_t)m * capacity;
-        uint32_t lo = 0, hi = m < M && level[m] >= 0 ? (uint32_t)count[m] : 0u;
-        while (__any_sync(0xFFFFFFFFu, lo < hi)) {
-            const uint32_t n = hi - lo;  // wraps where the search has ended: that lane looks at nothing
-            auto place = [&](uint32_t l) { return lo + (uint32_t)(((uint64_t)n * l) >> lanes_log2); };
-            const bool below = lo < hi && (uint64_t)__ldg(&a[place((uint32_t)part)]) < target;
-            const uint32_t votes = __ballot_sync(0xFFFFFFFFu, below) >> (lane - part);
-            const uint32_t c = (uint32_t)__popc(lanes_log2 == 5 ? votes : votes & ((1u << (1 << lanes_log2)) - 1u));
-            if (lo < hi) {
-                const uint32_t from = c ? place(c - 1u) + 1u : lo, to = c == 0u ? lo : c >> lanes_log2 ? hi : place(c);
-                lo = from;
-                hi = to;
-            }
-        }
-        if (part == 0 && m < M) sh_edge[edge] = lo;
+        const uint32_t n = m < M && level[m] >= 0 ? (uint32_t)count[m] : 0u;
+        const uint32_t at = first_not_below(idx + (int64_t)(m < M ? m : 0) * capacity, n, target, lanes_log2);
+        if (part == 0 && m < M) sh_edge[edge] = at;
     }
     for (int i = threadIdx.x; i < TILE / 4; i += kDirectThreads) reinterpret_cast<float4*>(acc)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     __syncthreads();
@@ -551,8 +565,8 @@ void launch_aggregate_topk(Workspace& ws, const mlmc_topk_msgs& msgs, int M, int
         return;
     }
     const int64_t n_off = (int64_t)M * (ntiles + 1);
-    launch_kernel(ws, K_AGG_OFFSETS, agg_offsets_kernel, dim3((unsigned)((n_off + 255) / 256)), 256, 0, s, msgs.idx, msgs.count,
-                  msgs.level, msgs.capacity, M, ntiles, ws.agg_offsets);
+    launch_kernel(ws, K_AGG_OFFSETS, agg_offsets_kernel, dim3(offset_blocks(n_off)), 256, 0, s, msgs.idx, msgs.count,
+                  msgs.level, msgs.capacity, M, ntiles, offset_lanes(n_off), ws.agg_offsets);
     const int grid = std::min(ntiles, ws.sm_count * ws.limits.aggregate_topk);
     launch_kernel(ws, K_AGG_TOPK, aggregate_topk_warps_kernel, dim3(grid), kAggWarps * 32, 0, s, msgs.idx, msgs.val,
                   msgs.capacity, M, d, ntiles, ws.agg_offsets, out);
@@ -610,8 +624,8 @@ extern "C" int mlmc_aggregate_topk_noalloc(const mlmc_topk_msgs* msgs, int M, in
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     // every entry in [0, n_off) is rewritten by this kernel, so nothing is left over from an earlier call
-    agg_offsets_kernel<<<(unsigned)((n_off + 255) / 256), 256, 0, s>>>(msgs->idx, msgs->count, msgs->level,
-                                                                       msgs->capacity, M, (int)ntiles, offsets);
+    agg_offsets_kernel<<<offset_blocks(n_off), 256, 0, s>>>(msgs->idx, msgs->count, msgs->level,
+                                                                       msgs->capacity, M, (int)ntiles, offset_lanes(n_off), offsets);
     int64_t grid = (int64_t)g_static_sm_count[dev] * 8;
     if (grid > ntiles) grid = ntiles;
     aggregate_topk_kernel<<<(unsigned)grid, 256, 2 * M * sizeof(uint32_t), s>>>(msgs->idx, msgs->val, msgs->capacity, M, d,

@@ -24,7 +24,6 @@ namespace {
 
 constexpr int kHistThreads = 1024;
 constexpr int kResolveThreads = 1024;
-constexpr int kResolveSmem = kBins1 * (int)sizeof(uint32_t);
 constexpr int kDigitThreads = 512;
 
 // -------------------------------------------------------------------------------------------
@@ -422,11 +421,22 @@ hist1_bf16_kernel(const bf16_t* __restrict__ g, int64_t d, int64_t ld, uint32_t*
     counts.flush();
 }
 
+// Slots of queries that share what they look for, by a warp, a query per lane.  The live queries are contiguous and equal values are
+// neighbours: the slots ascend from 0, and first[slot] is the first query of each.
+__device__ __forceinline__ uint32_t shared_slot(bool live, uint32_t value, uint32_t* first) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t before = __shfl_up_sync(0xFFFFFFFFu, value, 1), lives = __ballot_sync(0xFFFFFFFFu, live);
+    const bool is_first = live && (lane == 0 || !((lives >> (lane - 1)) & 1u) || before != value);
+    const uint32_t slot = (uint32_t)__popc(__ballot_sync(0xFFFFFFFFu, is_first) & ((2u << lane) - 1u)) - 1u;
+    if (first && is_first) first[slot] = (uint32_t)lane;
+    return slot;
+}
+
 // -------------------------------------------------------------------------------------------
 // after sweep 1: every live query descends into its bin
 // -------------------------------------------------------------------------------------------
-// One block per worker; thread t owns the 32 bins from 32 t.  One scan over the 1024 sums, then the thread whose bins
-// hold a query's rank walks them.  bf16: the digit is the whole key, so the query is resolved, and the energies of the
+// One block per worker; thread t owns the 32 bins from 32 t.  One scan over the 1024 sums, then a warp per query goes through the bins of
+// the thread that holds its rank.  bf16: the digit is the whole key, so the query is resolved, and the energies of the
 // intervals follow from the counts.  fp32: the kernel writes the bin table of the second sweep: a bin that holds no
 // threshold maps to its open interval  #{ j : bin_j > b }  (code < 64); a bin that holds one maps to 64 + its slot.
 __global__ void __launch_bounds__(kResolveThreads, 1)
@@ -438,44 +448,41 @@ resolve1_kernel(const uint32_t* hist1, Query* queries, uint8_t* table1, uint32_t
     __shared__ Query sh_q[kMaxQueries];
     __shared__ int sh_bin[kMaxQueries];
     __shared__ uint32_t sh_slot[kMaxQueries];
+    __shared__ uint2 sh_owner[kMaxQueries];      // thread whose bins hold the rank, keys above those
     __shared__ double sh_E[kMaxLevels];
     __shared__ double sh_part[kMaxLevels][kResolveThreads / 32];  // bf16, adaptive
     pdl_enter();
     const int m = blockIdx.x, nq = pl.nq;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // What is needed from memory is asked for at a time: the kernel is a chain of latencies.
+    constexpr int per = kBins1 / kResolveThreads;
+    static_assert(per == 32 && kResolveThreads == 1024, "32 bins per thread, 32 warps");
+    uint4 vectors[per / 4];
+    load_bins(hist1 + (int64_t)m * kBins1 + warp * 1024, vectors);
+    uint4 br = make_uint4(0u, 0u, 0u, 0u);
+    int drawn_level = 0, full = 0;
+    if (threadIdx.x == 32 && bracket) {
+        br = bracket[m];
+        drawn_level = emit[m].level;
+        full = cand_overflow[m];
+    }
+    Query query = {};
+    if (threadIdx.x < nq) query = queries[m * kMaxQueries + threadIdx.x];
+    const int missed_before = miss ? miss[m] : 0;
     if (worker_err[m]) {
         if (is_bf16 && threadIdx.x == 0) fail_worker(pl, m, &emit[m]);
         return;
     }
-    if (miss && !sampled && !miss[m]) return;  // resolved from the sampled brackets
-    constexpr int per = kBins1 / kResolveThreads;
-    static_assert(per == 32 && kResolveThreads == 1024, "32 bins per thread, 32 warps");
-    // A thread's bins are 128 consecutive bytes: the warp reads its 4 KB in coalesced vectors and hands them over through shared
-    // memory (vector j of thread t at j ^ t, so that neither side meets in a bank).  Read directly, every load touches 32 lines
-    // (16 x 11.7M entries, given p: 254 us per step, now 251; 1000 segments 247, now 243).
+    if (miss && !sampled && !missed_before) return;  // resolved from the sampled brackets
     uint32_t cnt[per];
     {
         extern __shared__ __align__(16) uint4 sh_vectors[];  // [32 warps][256]
-        const uint4* src = reinterpret_cast<const uint4*>(hist1 + (int64_t)m * kBins1) + warp * 256;
-        uint4* rows = sh_vectors + warp * 256;
-        uint4 x[per / 4];
-#pragma unroll
-        for (int i = 0; i < per / 4; ++i) x[i] = src[i * 32 + lane];
-#pragma unroll
-        for (int i = 0; i < per / 4; ++i) {
-            const int owner = i * 4 + (lane >> 3);
-            rows[owner * 8 + ((lane ^ owner) & 7)] = x[i];
-        }
-        __syncwarp();
-#pragma unroll
-        for (int i = 0; i < per / 4; ++i) {
-            const uint4 y = rows[lane * 8 + ((i ^ lane) & 7)];
-            cnt[4 * i] = y.x; cnt[4 * i + 1] = y.y; cnt[4 * i + 2] = y.z; cnt[4 * i + 3] = y.w;
-        }
+        hand_over_bins(vectors, sh_vectors + warp * 256, lane, cnt);
     }
     if (threadIdx.x < nq) {
-        sh_q[threadIdx.x] = queries[m * kMaxQueries + threadIdx.x];
+        sh_q[threadIdx.x] = query;
         sh_bin[threadIdx.x] = -1;
+        sh_owner[threadIdx.x] = make_uint2(0xFFFFFFFFu, 0u);
     }
     uint32_t sum = 0;
 #pragma unroll
@@ -496,24 +503,28 @@ resolve1_kernel(const uint32_t* hist1, Query* queries, uint8_t* table1, uint32_t
     const int b0 = threadIdx.x * per;
     for (int j = 0; j < nq; ++j) {
         const uint32_t k = sh_q[j].k;
-        if (sh_q[j].trivial == 0u && above < k && k <= above + sum) {  // the thread that owns rank k
-            uint32_t run = above;
-            int bin = 0;
-            uint32_t ab = 0, c = 0;
+        if (sh_q[j].trivial == 0u && above < k && k <= above + sum) sh_owner[j] = make_uint2(threadIdx.x, above);  // whose bins hold rank k
+    }
+    __syncthreads();
+    // A warp per query goes through the owner's 32 bins, which are still in shared memory.  (The owner alone, one query after the other where
+    // a thread or a warp has several: 3 us more with 14 queries.)
+    if (warp < nq && sh_q[warp].trivial == 0u && sh_owner[warp].x < (uint32_t)kResolveThreads) {
+        extern __shared__ __align__(16) uint4 sh_vectors[];
+        const uint32_t k = sh_q[warp].k, owner = sh_owner[warp].x, group = owner & 31u, i = 31u - lane;  // lane 0: the largest bin
+        const uint32_t c = reinterpret_cast<const uint32_t*>(sh_vectors + (owner & ~31u) * 8u + group * 8u + (((i >> 2) ^ group) & 7u))[i & 3u];
+        uint32_t upto = c;
 #pragma unroll
-            for (int i = per - 1; i >= 0; --i) {  // the largest bin b with #{digit >= b} >= k
-                if (run < k) {
-                    bin = b0 + i;
-                    ab = run;
-                    c = cnt[i];
-                }
-                run += cnt[i];
-            }
-            sh_bin[j] = bin;
-            sh_q[j].c = ab;
-            sh_q[j].n = c;
-            sh_q[j].r = k - ab;
-            if (is_bf16) sh_q[j].T = (uint32_t)bin;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, upto, o);
+            if (lane >= o) upto += y;
+        }
+        const uint32_t ab = sh_owner[warp].y + upto - c;
+        if (ab < k && k <= ab + c) {  // the largest bin b with #{digit >= b} >= k
+            sh_bin[warp] = (int)(owner * per + i);
+            sh_q[warp].c = ab;
+            sh_q[warp].n = c;
+            sh_q[warp].r = k - ab;
+            if (is_bf16) sh_q[warp].T = owner * per + i;
         }
     }
     if (threadIdx.x < nq && sh_q[threadIdx.x].trivial)  // "nothing inside" sits above every bin, "everything inside" below
@@ -522,12 +533,12 @@ resolve1_kernel(const uint32_t* hist1, Query* queries, uint8_t* table1, uint32_t
     if (sampled) {
         // The histogram holds the keys of the sampled brackets only, and between them the number of keys there: a threshold
         // that does not lie in a bracket, or a full candidate list, sends the worker through the sweeps of the whole row.
-        bool out = miss[m] != 0;
+        bool out = missed_before != 0;
         if (threadIdx.x < nq && sh_q[threadIdx.x].trivial == 0u) {
             const int bin = sh_bin[threadIdx.x];
             out |= bin < 0 || table1[(int64_t)m * kBins1 + bin] != nq + 1;  // so marked by the sample
         }
-        const bool left_out = miss[m] == kLeftOut;
+        const bool left_out = missed_before == kLeftOut;
         const bool missed = __syncthreads_or(out);
         if (threadIdx.x == 0) atomicAdd(&bracket_stats[4 + (!missed ? 0 : left_out ? 2 : 1)], 1ull);
         if (missed) {
@@ -571,23 +582,20 @@ resolve1_kernel(const uint32_t* hist1, Query* queries, uint8_t* table1, uint32_t
         return;
     }
     // slots of the second digit pass: live queries in the same bin share one (bins descend with j)
-    if (threadIdx.x < nq) {
-        const int j = threadIdx.x;
-        uint32_t slot = 0;
-        int prev = -2;
-        for (int i = 0; i <= j; ++i) {
-            if (sh_q[i].trivial) continue;
-            if (prev != -2 && sh_bin[i] != prev) ++slot;
-            prev = sh_bin[i];
+    if (warp == 0) {
+        const int j = lane;
+        const bool live = j < nq && sh_q[j].trivial == 0u;
+        const uint32_t slot = shared_slot(live, live ? (uint32_t)sh_bin[j] : 0u, nullptr);
+        if (j < nq) {
+            sh_slot[j] = live ? slot : kNoSlot;
+            Query q = sh_q[j];
+            if (live) {
+                q.prefix = (uint32_t)sh_bin[j] << 16;
+                q.rem = q.r;
+                q.slot = q.slot2 = slot;
+            }
+            queries[m * kMaxQueries + j] = q;
         }
-        sh_slot[j] = sh_q[j].trivial ? kNoSlot : slot;
-        Query q = sh_q[j];
-        if (!q.trivial) {
-            q.prefix = (uint32_t)sh_bin[j] << 16;
-            q.rem = q.r;
-            q.slot = q.slot2 = slot;
-        }
-        queries[m * kMaxQueries + j] = q;
     }
     if (threadIdx.x == 32) {
         // the smallest key that can be a candidate: the lower edge of the lowest boundary bin (no live query: none)
@@ -601,9 +609,8 @@ resolve1_kernel(const uint32_t* hist1, Query* queries, uint8_t* table1, uint32_t
         if (bracket) {
             // Did the first sweep already collect the keys of both boundary bins of the drawn band?  If not, its
             // candidates are dropped and the candidate sweep runs.  Either way the bins are remembered.
-            const uint4 br = bracket[m];
-            const int lv = emit[m].level;
-            hit = cand_overflow[m] == 0;
+            const int lv = drawn_level;
+            hit = full == 0;
             for (int j = 0; j < nq; ++j) {
                 if (sh_q[j].trivial) continue;
                 const uint32_t bin = (uint32_t)sh_bin[j];
@@ -873,15 +880,19 @@ digit_pass_kernel(const float* __restrict__ g, int64_t d, int64_t ld, uint32_t* 
     pdl_enter();
     const int m = blockIdx.y, nq = pl.nq;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (worker_err[m]) {
+    // asked for at a time, and the queries before the last block needs them
+    const uint32_t listed = cand_count[m];
+    const int full = cand_overflow[m], missed = SUMS && parts.miss ? parts.miss[m] : 1, bad = worker_err[m];
+    if (threadIdx.x < nq) sh_q[threadIdx.x] = queries[m * kMaxQueries + threadIdx.x];
+    if (bad) {
         if (PASS == 3 && blockIdx.x == 0 && threadIdx.x == 0) fail_worker(pl, m, &emit[m]);
         return;
     }
     uint32_t* sh_hist = sh_digit;
     uint32_t* sh_cell = sh_digit + nq * kBins23;
-    const bool in_parts = SUMS && parts.miss && !parts.miss[m];
-    const bool over = !in_parts && cand_overflow[m] != 0;
-    const uint32_t n = over || in_parts ? 0u : cand_count[m];
+    const bool in_parts = SUMS && !missed;
+    const bool over = !in_parts && full != 0;
+    const uint32_t n = over || in_parts ? 0u : listed;
     uint32_t* out = hist_out + (int64_t)m * kMaxQueries * kBins23;
     // pass 2, parts: energy of the keys of a run's bins without a threshold, a column per interval and thread; the order of
     // the keys in the parts is fixed, so the sums are too
@@ -1068,8 +1079,6 @@ digit_pass_kernel(const float* __restrict__ g, int64_t d, int64_t ld, uint32_t* 
 
     // one warp per query walks its 256-bin histogram from the top digit down
     __shared__ uint32_t sh_digit_of[kMaxQueries];
-    if (threadIdx.x < nq) sh_q[threadIdx.x] = queries[m * kMaxQueries + threadIdx.x];
-    __syncthreads();
     for (int j = warp; j < nq; j += kDigitThreads / 32) {
         if (sh_q[j].trivial) continue;
         const uint32_t* h = out + sh_q[j].slot * kBins23;
@@ -1110,15 +1119,12 @@ digit_pass_kernel(const float* __restrict__ g, int64_t d, int64_t ld, uint32_t* 
     __syncthreads();
     if (PASS == 2) {
         // slots of pass 3: live queries with the same prefix share one (prefixes descend with j)
-        if (threadIdx.x < nq && !sh_q[threadIdx.x].trivial) {
-            const int j = threadIdx.x;
-            uint32_t slot = 0, prev = 0xFFFFFFFFu;
-            for (int i = 0; i <= j; ++i) {
-                if (sh_q[i].trivial) continue;
-                if (prev != 0xFFFFFFFFu && sh_q[i].prefix != prev) ++slot;
-                prev = sh_q[i].prefix;
-            }
-            sh_q[j].slot = slot;
+        __shared__ uint32_t sh_first[kMaxQueries];  // first query of a boundary bin
+        if (warp == 0) {
+            const bool live = lane < nq && sh_q[lane].trivial == 0u;
+            const uint32_t slot = shared_slot(live, live ? sh_q[lane].prefix : 0u, nullptr);
+            if (live) sh_q[lane].slot = slot;
+            shared_slot(live, live ? sh_q[lane].slot2 : 0u, sh_first);
         }
         __syncthreads();
         if (threadIdx.x < nq) queries[m * kMaxQueries + threadIdx.x] = sh_q[threadIdx.x];
@@ -1131,8 +1137,8 @@ digit_pass_kernel(const float* __restrict__ g, int64_t d, int64_t ld, uint32_t* 
             uint8_t* mp = map2 + (int64_t)m * kMaxQueries * kBins23;
             for (int i = threadIdx.x; i < nslot * kBins23; i += kDigitThreads) {
                 const uint32_t s = (uint32_t)i / kBins23, x = (uint32_t)i % kBins23;
-                int j = first;
-                while (j < last && (sh_q[j].slot2 < s || (sh_q[j].slot2 == s && sh_digit_of[j] > x))) ++j;
+                int j = (int)sh_first[s];
+                while (j < last && sh_q[j].slot2 == s && sh_digit_of[j] > x) ++j;
                 const bool here = j < last && sh_q[j].slot2 == s && sh_digit_of[j] == x;
                 mp[i] = here ? (uint8_t)sh_q[j].slot : (SUMS ? (uint8_t)(64u + (uint32_t)j + s) : (uint8_t)0xFFu);
             }
@@ -1310,7 +1316,7 @@ void launch_hist1(Workspace& ws, const void* g, int dtype, int64_t d, int M, int
 }
 
 void launch_resolve1(Workspace& ws, int dtype, int M, const FinishPlan& plan, bool brackets, bool sampled, int* miss, cudaStream_t s) {
-    launch_kernel(ws, K_RESOLVE1, resolve1_kernel, dim3(M), kResolveThreads, kResolveSmem, s, ws.hist1, ws.queries, ws.table1,
+    launch_kernel(ws, K_RESOLVE1, resolve1_kernel, dim3(M), kResolveThreads, kBinRowsSmem, s, ws.hist1, ws.queries, ws.table1,
                   ws.cand_floor, plan, dtype == MLMC_BF16 ? 1 : 0, ws.status, ws.worker_err, ws.emit,
                   brackets ? ws.bracket : nullptr, ws.bracket_hit, ws.prev_bin, ws.bracket_stats, ws.cand_count,
                   ws.cand_overflow, ws.p_all, ws.delta_all, sampled ? 1 : 0, miss);
@@ -1372,7 +1378,7 @@ int configure_select_kernels() {
     auto set = [](auto kernel, int bytes) {
         return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess;
     };
-    const bool ok = set(resolve1_kernel, kResolveSmem) && set(hist1_kernel<false>, hist) && set(hist1_kernel<true>, hist + stage) &&
+    const bool ok = set(resolve1_kernel, (int)kBinRowsSmem) && set(hist1_kernel<false>, hist) && set(hist1_kernel<true>, hist + stage) &&
                     set(hist1_bf16_kernel, (int)(BinCounts::kWords * sizeof(uint32_t))) && set(sums_candidates_kernel<true>, kS2SmemMost) &&
                     set(sums_candidates_kernel<false>, (int)s2_smem(0, false, kS2Threads)) && set(digit_pass_kernel<2, true>, columns) &&
                     set(digit_pass_kernel<2, false>, digits) && set(digit_pass_kernel<3, true>, digits) &&
