@@ -4,6 +4,7 @@ import pytest
 import torch
 
 from test_gpu_dispatch import doubling, geometric, layered
+from test_gpu_ext import check_stopk
 from test_gpu_parity import check_topk, padded
 
 pytestmark = pytest.mark.gpu
@@ -53,6 +54,15 @@ def test_cluster_sizes(B, ora, ctx, dtype, kind, d):
 def test_bf16_rows_given_p(B, ora, ctx, d, M):
     k = doubling(d, d // 500)
     check_topk(B, ora, ctx, layered(d, M, "bf16"), k, geometric(len(k)), 3, 1, expect_excluded=1)
+
+
+# more segments than levels, given p: the longest fp32 rows of a cluster, which keep no brackets
+@pytest.mark.parametrize("d", [262_145, 745_472, 745_473])
+def test_segments_given_p(B, ora, ctx, d):
+    s = d // 100
+    L = -(-d // s)
+    check_stopk(B, ora, ctx, layered(d, 3), s, geometric(L), 3, 1)
+    check_stopk(B, ora, ctx, rows("ties", d, 2, "f32"), s, [1.0 / L] * L, 3, 2)
 
 
 # edges of the tiles; empty, void and dense messages; lanes per search edge from 32 to 4
