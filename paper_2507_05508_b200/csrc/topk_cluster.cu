@@ -693,7 +693,8 @@ void cluster_limits(KernelLimits* limits) {  // the kernels of all sizes take th
 // Blocks per cluster for this call, 0: the row is too long, or the workers are too many, for the cluster to be the faster way.
 // kClSpread batches per block while the clusters of all workers run at a time, else kClEasy (4 x 65,536 entries, given p: 18.9 us per
 // step on 8 blocks, 20.0 on 4, where M clusters of 16 would not fit 131k x 8 takes 63 us on 16 and 36 on 8); longer rows are
-// stretched over 16 blocks.  Clusters that do not fit the GPU at a time run one after the other, where the launch chain has the
+// stretched over 16 blocks.  fp32 rows with given p have two digits of two queries to tell all of 16 blocks, which takes longer than it
+// spares: up to 8 blocks while kClEasy batches suffice (3 x 131,072 22.2 us on 16, 18.9 on 8; adaptive p 29.2 and 30.2, bf16 17.9 and 19.7).  Clusters that do not fit the GPU at a time run one after the other, where the launch chain has the
 // whole GPU: how far that pays depends on what the chain has to do.  us per step, cluster / chain, layered rows:
 //   fp32, adaptive  700k x 3 53 / 76, 400k x 6 46 / 79; two waves 262k x 8 63 / 78, 400k x 12 82 / 90, 700k x 8 100 / 89; three
 //                   262k x 16 95 / 90, 131k x 32 93 / 100
@@ -705,7 +706,10 @@ int cluster_blocks(const Workspace& ws, int dtype, int64_t d, int M, bool given)
     const int64_t batches = (int64_t)emit_tiles_per_worker(d, dtype) * kEmitGroups;
     if (M > 32) return 0;
     int i = 0;
-    while (i < 4 && ws.limits.topk_fit[i + 1] > 0 && batches > (int64_t)(M <= ws.limits.topk_fit[i + 1] ? kClSpread : kClEasy) << i) ++i;
+    const int spread_to = given && dtype == MLMC_F32 ? 3 : 4;
+    while (i < 4 && ws.limits.topk_fit[i + 1] > 0 &&
+           batches > (int64_t)(M <= ws.limits.topk_fit[i + 1] && i < spread_to ? kClSpread : kClEasy) << i)
+        ++i;
     const int fit = ws.limits.topk_fit[i];
     if (fit == 0) return 0;
     const int64_t per = (batches + (1 << i) - 1) >> i;
