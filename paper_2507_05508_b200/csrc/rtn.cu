@@ -60,7 +60,8 @@ __device__ RtnLevel rtn_level(float c, int r) {
     v.delta = gq.delta;
     // t = fl32(m inv) does not fall as m grows, and t <= 1/2 rounds to 0 (ties to even)
     v.zero_upto = v.free_upto = -1;
-    if (!(gq.inv <= 3.0e38f)) return v;  // c below the normal range: 1 / delta overflows, and 0 inv is not a number
+    // c below the normal range: 1 / delta overflows, and 0 inv is not a number; one bit, c at the end of the range: delta overflows
+    if (!(gq.inv <= 3.0e38f && gq.delta <= 3.0e38f)) return v;
     uint32_t z = min(__float_as_uint(0.5f / gq.inv), 0x7F7FFFFFu);
     while (z > 0u && __fmul_rn(__uint_as_float(z), gq.inv) > 0.5f) --z;
     while (z < 0x7F7FFFFFu && __fmul_rn(__uint_as_float(z + 1u), gq.inv) <= 0.5f) ++z;
@@ -68,6 +69,11 @@ __device__ RtnLevel rtn_level(float c, int r) {
     const float f = c - gq.delta;  // |k delta| <= |v| + delta / 2 (1 + 2^-20)
     if (f > 0.0f) v.free_upto = __float_as_int(f);
     return v;
+}
+
+// C^l(-v) = -C^l(v) for every entry of the row and every level?  The first level has the largest delta, the last one the largest 1 / delta.
+__device__ __forceinline__ bool odd_levels(const RtnLevel* levels, int L) {
+    return L < 2 || (levels[0].zero_upto >= 0 && levels[L - 2].zero_upto >= 0);
 }
 
 // Residual energies of every level: partial[m][block][l] = sum over the block's entries of (C^l - C^{l-1})^2.
@@ -107,9 +113,11 @@ __device__ __forceinline__ double widen(float x, bool by_product) {
     return __hiloint2double((int)(b >> 3), (int)(b << 29)) * 0x1p896;
 }
 
-// One trip of a warp: kRtnHeld entries per lane.  Magnitudes: C^l(-v) = -C^l(v).  The grid values of two entries are found together, by
-// packed instructions.  one = 1, an argument: the compiler merges a packed product and the addition after it into one rounding, also
-// where both say that they round, and the rounding of t = fl32(v inv) decides ties.  So the addition is a multiply-add of t with one.
+// One trip of a warp: kRtnHeld entries per lane.  Magnitudes: C^l(-v) = -C^l(v), except in rows with a level whose 1 / delta or delta
+// overflows: the product 0 Inf is not a number and comes out of the clipping as -c (with delta = 0 that of every entry).  Those rows
+// go entry by entry.  The grid values of two entries are found together, by packed instructions.  one = 1, an argument: the compiler
+// merges a packed product and the addition after it into one rounding, also where both say that they round, and the rounding of
+// t = fl32(v inv) decides ties.  So the addition is a multiply-add of t with one.
 template <int LMAX>
 __device__ __forceinline__ void take_levels(const float (&signed_v)[kRtnHeld], float c, const RtnLevel* levels, int L, float one, double (&acc)[LMAX]) {
     float v[kRtnHeld];
@@ -213,14 +221,17 @@ rtn_stats_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t*
         constexpr int kVecs = kRtnHeld / Tr::kVec;  // 16-byte vectors per lane and trip
         constexpr int kTrip = kRtnThreads * kVecs;
         const int64_t full_end = d / Tr::kVec;
-        const int64_t trips = full_end / kTrip;
+        const bool odd = odd_levels(sh_lv, sc.L);
+        const int64_t trips = odd ? full_end / kTrip : 0;
         stream_trips<kVecs, kRtnThreads>(reinterpret_cast<const uint4*>(row), blockIdx.x, gridDim.x, trips, sh_vectors, [&](const uint4 (&q)[kVecs]) {
             float v[kRtnHeld];
             rtn_expand<T>(q, v);
             take_levels<LMAX>(v, c, sh_lv, sc.L, one, acc);
         });
-        if (blockIdx.x == gridDim.x - 1) {  // the rest of the row, fewer than kTrip + 1 vectors, one by one
-            for (int64_t i = trips * kTrip * Tr::kVec + threadIdx.x; i < d; i += kRtnThreads) {
+        // the rest of the row, one by one: fewer than kTrip + 1 vectors for the last block, or everything for all blocks
+        if (!odd || blockIdx.x == gridDim.x - 1) {
+            const int64_t step = odd ? kRtnThreads : (int64_t)gridDim.x * kRtnThreads;
+            for (int64_t i = trips * kTrip * Tr::kVec + (odd ? 0 : (int64_t)blockIdx.x * kRtnThreads) + threadIdx.x; i < d; i += step) {
                 float v;
                 if constexpr (Tr::kVec == 4) v = reinterpret_cast<const float*>(row)[i];
                 else v = __uint_as_float((uint32_t)reinterpret_cast<const uint16_t*>(row)[i] << 16);
@@ -263,12 +274,13 @@ template <typename T>
 struct Residual {
     double inv_p;
     float c;
-    bool top, first;
+    bool top, first, flat;  // flat: a small entry leaves nothing (not so where delta overflows and 0 delta is not a number)
     RtnGrid hi, lo;
     __device__ __forceinline__ Residual(float c_, const RtnSchedule& sc, int level, double p)
         : inv_p(p > 0.0 ? 1.0 / p : 0.0), c(c_), top(level == sc.L - 1), first(level == 0) {
         hi = rtn_grid(c > 0.0f ? c : 1.0f, top ? 1 : sc.r[level]);
         lo = rtn_grid(c > 0.0f ? c : 1.0f, first ? 1 : sc.r[level - 1]);
+        flat = !top && (first ? hi : lo).delta <= 3.0e38f;
     }
     __device__ __forceinline__ float operator()(uint32_t bits) const {
         const float v = ElemTraits<T>::value(bits);
@@ -280,7 +292,7 @@ struct Residual {
     // Nothing up to this magnitude leaves anything: fl32(m inv) does not fall as m grows, 1/2 rounds to 0 (ties to even), and the
     // level before has the coarser grid.
     __device__ __forceinline__ bool rounds_to_zero(uint32_t magnitude) const {
-        return !(c > 0.0f) || (!top && __fmul_rn(__uint_as_float(magnitude), hi.inv) <= 0.5f);
+        return !(c > 0.0f) || (flat && __fmul_rn(__uint_as_float(magnitude), hi.inv) <= 0.5f);
     }
     __device__ __forceinline__ void vector(const uint4& q, float* __restrict__ out) const {  // a vector's entries, out 16-byte aligned
         if constexpr (sizeof(T) == 4) {
@@ -418,10 +430,11 @@ rtn_cluster_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid_
         for (int l = 0; l < kRtnDenseLevels; ++l) acc[l] = 0.0;
         if (c > 0.0f) {
             constexpr int kVecs = kRtnHeld / Tr::kVec;  // a warp takes a quarter of a group
+            const bool odd = odd_levels(sh_lv, sc.L);
 #pragma unroll 1
             for (int u = warp; u < 4 * n; u += kRtnDenseWarps) {
                 const int64_t e0 = (g0 + (u >> 2)) * 1024;
-                if (e0 + 1024 <= d) {
+                if (odd && e0 + 1024 <= d) {
                     const uint4* x = reinterpret_cast<const uint4*>(sh_slots + (u >> 2) * kGroupSlot<T>) + (u & 3) * kVecs * 32 + lane;
                     uint4 q[kVecs];
 #pragma unroll
@@ -429,7 +442,7 @@ rtn_cluster_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid_
                     float v[kRtnHeld];
                     rtn_expand<T>(q, v);
                     take_levels<kRtnDenseLevels>(v, c, sh_lv, sc.L, one, acc);
-                } else {  // entries past the row's end are not entries
+                } else {  // one by one; entries past the row's end are not entries
                     for (int e = (u & 3) * 256 + lane; e < (u & 3) * 256 + 256 && e0 + e < d; e += 32)
                         take_entry<kRtnDenseLevels>(Tr::value(entry(u >> 2, e)), c, sh_lv, sc.L, acc);
                 }

@@ -45,3 +45,27 @@ def test_statistics(B, ora, ctx, dtype, kind, d):
     check_rtn(B, ora, ctx, g, [2, 4, 8, 16], None, 3, 1)
     check_bitwise(B, ora, ctx, g, [1, 2, 4, 8, 16, 23], None, 3, 1)
     check_bitwise(B, ora, ctx, g, [2, 14, 23], None, 3, 2)
+
+
+# Largest magnitudes for which a grid step or its reciprocal leaves the fp32 range: an entry and its negative then differ in the clipping.
+@pytest.mark.parametrize("widths", [[2, 4, 8, 16], [1, 2, 9], [16], [1]])
+@pytest.mark.parametrize("largest", [1e-41, 1e-44, 1e-36, 2e38, 3.3e38])
+@pytest.mark.parametrize("d", [5_003, 20_003, 600_001])
+def test_grids_out_of_range(B, ora, ctx, d, largest, widths):
+    rng = np.random.default_rng(d)
+    x = np.clip(rng.standard_normal((2, d)), -3, 3) / 3 * largest * (rng.random((2, d)) < 0.9)
+    x[0, 5], x[1, 6] = largest, -largest
+    g = padded(torch.from_numpy(x.astype(np.float32)).cuda(), 8)
+    L = len(widths) + 1
+    p = torch.zeros((2, L), dtype=torch.float64, device="cuda")
+    delta = torch.zeros((2, L), dtype=torch.float64, device="cuda")
+    B.mlmc_level_probs(ctx, g, B.MLMC_RTN, widths, None, p, delta)
+    assert B.mlmc_get_status(ctx) == 0
+    for m in range(2):
+        o = ora.rtn(x[m].astype(np.float32), widths, None)
+        # either side adds d squares in fp64, in an order of its own: d roundings of 2^-53 each at most, halved by the root
+        assert np.allclose(delta[m].cpu().numpy(), o.delta, rtol=d * 2.0 ** -53 + 1e-14, atol=0)
+        assert np.allclose(p[m].cpu().numpy(), o.p, rtol=2 * (d * 2.0 ** -53 + 1e-14), atol=1e-300)
+    if largest < 1.0:  # otherwise the messages' values, divided by their probability, leave the range
+        check_rtn(B, ora, ctx, g, widths, None, 3, 1)
+        check_rtn(B, ora, ctx, g, widths, [1.0 / L] * L, 3, 2)
