@@ -69,3 +69,21 @@ def test_grids_out_of_range(B, ora, ctx, d, largest, widths):
     if largest < 1.0:  # otherwise the messages' values, divided by their probability, leave the range
         check_rtn(B, ora, ctx, g, widths, None, 3, 1)
         check_rtn(B, ora, ctx, g, widths, [1.0 / L] * L, 3, 2)
+
+
+# A call of more than 100 MB, whose message looks at the batches: no entry rounds to 0 where delta overflows.
+def test_grid_out_of_range_in_a_long_message(B, ora):
+    d = 26_300_003
+    x = np.random.default_rng(0).uniform(-1.0, 1.0, (1, d)).astype(np.float32)
+    x[0, :d // 2] *= 1e-3
+    x *= np.float32(3e38)
+    out = B.RtnBuffers(1, d)
+    c = B.mlmc_create(0, d, 1, 32)
+    try:
+        B.mlmc_compress_rtn(c, padded(torch.from_numpy(x).cuda(), 8), [1, 2], [0.999, 0.0005, 0.0005], 3, 1, out)
+        assert B.mlmc_get_status(c) == 0
+        o = ora.rtn(x[0], [1, 2], [0.999, 0.0005, 0.0005], seed=3, step=1, worker=0)
+        assert o.level == 0 and int(out.level[0]) == 0
+        assert np.array_equal(out.val[0, :d].cpu().numpy(), o.val)  # +-c, divided by p in fp64 and rounded once
+    finally:
+        B.mlmc_destroy(c)
