@@ -236,6 +236,11 @@ band_write_kernel(const T* __restrict__ g, int64_t d, int64_t ld, int tiles_per_
     cp_async_wait<0>();
 }
 
+// Entries of worker m's message; a voided one, or a count below 0, has none.
+__device__ __forceinline__ uint32_t message_entries(const int64_t* count, const int32_t* level, int m) {
+    return level[m] < 0 ? 0u : (uint32_t)max(count[m], (int64_t)0);
+}
+
 // First of the n entries of an index-sorted list that is not below `target`, by 2^lanes_log2 neighbouring lanes (of a warp that is here
 // with all its lanes): of the entries that are left, every lane looks at the first of its share.  One lane: halves.
 __device__ __forceinline__ uint32_t first_not_below(const uint32_t* __restrict__ a, uint32_t n, uint64_t target, int lanes_log2) {
@@ -275,7 +280,7 @@ agg_offsets_kernel(const uint32_t* idx, const int64_t* count, const int32_t* lev
     const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> lanes_log2;
     const bool there = i < (int64_t)M * (ntiles + 1);
     const int m = there ? (int)(i / (ntiles + 1)) : 0, t = there ? (int)(i % (ntiles + 1)) : 0;
-    const uint32_t n = there && level[m] >= 0 ? (uint32_t)count[m] : 0u;
+    const uint32_t n = there ? message_entries(count, level, m) : 0u;
     const uint32_t at = first_not_below(idx + (int64_t)m * capacity, n, (uint64_t)t * kAggTile, lanes_log2);
     if (there && (threadIdx.x & ((1 << lanes_log2) - 1)) == 0) offsets[i] = at;
 }
@@ -444,7 +449,7 @@ aggregate_topk_direct_kernel(const uint32_t* __restrict__ idx, const float* __re
     {   // an edge is the first entry that is not below its coordinate
         const int edge = threadIdx.x >> lanes_log2, m = edge >> 1, part = threadIdx.x & ((1 << lanes_log2) - 1);
         const uint64_t target = (uint64_t)base + (edge & 1 ? TILE : 0);
-        const uint32_t n = m < M && level[m] >= 0 ? (uint32_t)count[m] : 0u;
+        const uint32_t n = m < M ? message_entries(count, level, m) : 0u;
         const uint32_t at = first_not_below(idx + (int64_t)(m < M ? m : 0) * capacity, n, target, lanes_log2);
         if (part == 0 && m < M) sh_edge[edge] = at;
     }

@@ -86,3 +86,29 @@ def test_average_in_one_launch(B, ctx, d, M):
     B.mlmc_aggregate(ctx, B.MLMC_TOPK, out, None, M, d, dense)
     # the additions are those of the loop above, in the same order; the product with 1 / M rounds once
     assert np.array_equal(dense.cpu().numpy(), ref * np.float32(1.0 / M))
+
+
+# in one launch, in two, and in two without a context; some lanes per search and one
+@pytest.mark.parametrize("d", [5_000, 2_424_833, 70_000_001])
+def test_counts_below_zero_are_empty_messages(B, d):
+    M = 9
+    rng = np.random.default_rng(d)
+    out = B.TopkBuffers(M, 1000)
+    ref = np.zeros(d, dtype=np.float32)
+    for m in range(M):
+        idx = np.sort(rng.choice(d, 1000, replace=False)).astype(np.int32)
+        val = rng.standard_normal(1000).astype(np.float32)
+        out.idx[m], out.val[m] = torch.from_numpy(idx).cuda(), torch.from_numpy(val).cuda()
+        out.count[m], out.level[m] = (-1, -(1 << 40), 1000)[m % 3], 0
+        if m % 3 == 2:
+            ref[idx] += val
+    ref *= np.float32(1.0 / M)
+    c = B.mlmc_create(0, d, M, 32)
+    try:
+        for average in (lambda to: B.mlmc_aggregate(c, B.MLMC_TOPK, out, None, M, d, to),
+                        lambda to: B.mlmc_aggregate_topk_noalloc(out, M, d, to)):
+            dense = torch.full((d,), float("nan"), device="cuda")
+            average(dense)
+            assert np.array_equal(dense.cpu().numpy(), ref)  # the same additions in the same order
+    finally:
+        B.mlmc_destroy(c)
