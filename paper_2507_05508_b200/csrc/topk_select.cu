@@ -867,8 +867,12 @@ struct CandParts {
     int n_sum;               // energy sums per interval that the sweep left
 };
 
+// The grid has kDigitBlocks blocks per SM, and the compiler may use the registers of as many: left to itself it takes 32 for the third
+// digit with energies and spills (16 x 11.7M fp32 keys, 31 levels: 56 us, 46 with 40 registers, 42 so; the step 923, now 884).
+constexpr int kDigitBlocks = 2;
+
 template <int PASS, bool SUMS>
-__global__ void __launch_bounds__(kDigitThreads)
+__global__ void __launch_bounds__(kDigitThreads, kDigitBlocks)
 digit_pass_kernel(const float* __restrict__ g, int64_t d, int64_t ld, uint32_t* cand_keys, int64_t cand_cap,
                   const uint32_t* cand_count, const int* cand_overflow, const uint8_t* table1, uint8_t* map2,
                   uint32_t* hist_out, uint32_t* done, Query* queries, FinishPlan pl, unsigned long long* cand_S,
@@ -1339,7 +1343,7 @@ void launch_sums_candidates(Workspace& ws, const void* g, int64_t d, int M, int6
 void launch_digit_passes(Workspace& ws, const void* g, int64_t d, int M, int64_t ld, const FinishPlan& plan, bool sampled, cudaStream_t s) {
     const bool sums = plan.adaptive != 0;
     const CandParts parts = {sampled ? ws.miss : nullptr, ws.part_n, ws.parts, ws.part_cap, ws.sweep_blocks};
-    int nb = (ws.sm_count * 2) / M;
+    int nb = (ws.sm_count * kDigitBlocks) / M;
     const int64_t by_work = (d + kDigitThreads * 4 - 1) / (kDigitThreads * 4);
     if (nb > by_work) nb = (int)by_work;
     if (nb < 1) nb = 1;
