@@ -27,7 +27,7 @@ def sampled(d):
     return mask.cuda()
 
 
-@pytest.mark.parametrize("case", ["layers", "zeros", "few_zeros", "wide", "tiny", "sample_above", "sample_below", "constant"])
+@pytest.mark.parametrize("case", ["layers", "zeros", "few_zeros", "wide", "tiny", "sample_above", "sample_below", "constant", "uniform", "signs"])
 @pytest.mark.parametrize("d", [D, 700_001])
 def test_thresholds_and_norms(B, case, d):
     gen = torch.Generator(device="cuda").manual_seed(d)
@@ -48,6 +48,10 @@ def test_thresholds_and_norms(B, case, d):
         g[:, sampled(d)] = 1.0
         for i, octaves in enumerate((4, 10, 50)):
             g[i::3, ~sampled(d)] *= 2.0 ** octaves
+    elif case == "uniform":           # half of the keys lie in the octave of the largest
+        g.uniform_(-1.0, 1.0, generator=gen)
+    elif case == "signs":
+        g.sign_()
     else:
         g.fill_(0.25)
     g = padded(g.to(torch.bfloat16), 8)
