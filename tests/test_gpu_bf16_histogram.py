@@ -7,8 +7,6 @@ from test_gpu_sampled import check_adaptive
 
 pytestmark = pytest.mark.gpu
 
-M, D = 100, 262_147  # one block per worker, eight batches per warp and a ragged end
-
 
 @pytest.fixture(scope="module")
 def B():
@@ -17,19 +15,39 @@ def B():
     return binding
 
 
-def sampled(d):
-    """Mask of the keys that the first block of a row samples: a vector of eight per stratum."""
-    stride = (d // 8) // 1024
+WARPS, TILE, BATCH = 32, 8192, 1024  # warps of a block; entries of a tile and of a batch
+FROM = 8                             # batches per warp from which on a row is sampled
+
+
+def blocks(d, M):
+    """Blocks per row: those of launch_hist1."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    waves = 2 if sms // M * M * 20 < sms * 19 else 1
+    return max(1, min(-(-d // (8 * 4096)), sms * waves // M))
+
+
+def batches_per_warp(d, M):
+    return -(-(-(-d // TILE) * TILE // BATCH) // (blocks(d, M) * WARPS))
+
+
+def sampled(d, M):
+    """Mask of the keys that the blocks of a row sample: a vector of eight per thread, from its share of the row."""
+    share = (d // 8) // 1024
     t = torch.arange(1024)
-    at = t * stride + (t * 11) % stride
     mask = torch.zeros(d, dtype=torch.bool)
-    mask[(at[:, None] * 8 + torch.arange(8)).flatten()] = True
+    for block in range(blocks(d, M)):
+        at = t * share + (block * 37 + t * 11) % share
+        mask[(at[:, None] * 8 + torch.arange(8)).flatten()] = True
     return mask.cuda()
 
 
+# one block per row: the longest row that is too short to be sampled, one entry more, a ragged end; two blocks per row
 @pytest.mark.parametrize("case", ["layers", "zeros", "few_zeros", "wide", "tiny", "sample_above", "sample_below", "constant", "uniform", "signs"])
-@pytest.mark.parametrize("d", [D, 700_001])
-def test_thresholds_and_norms(B, case, d):
+@pytest.mark.parametrize("d,per_sm,n,columns", [(28 * TILE, 1.0, 1, False), (28 * TILE + 1, 1.0, 1, True), (262_147, 1.0, 1, True),
+                                                (700_001, 0.68, 2, True)])
+def test_thresholds_and_norms(B, case, d, per_sm, n, columns):
+    M = int(torch.cuda.get_device_properties(0).multi_processor_count * per_sm)
+    assert blocks(d, M) == n and (batches_per_warp(d, M) >= FROM) == columns
     gen = torch.Generator(device="cuda").manual_seed(d)
     g = torch.randn((M, d), generator=gen, device="cuda")
     if case == "layers":
@@ -41,13 +59,13 @@ def test_thresholds_and_norms(B, case, d):
     elif case == "tiny":              # the window starts at the smallest numbers
         g *= 2.0 ** -120
     elif case == "sample_above":      # the window lies above everything else, by 16, 26 and 50 octaves
-        g[:, sampled(d)] = 8.0
+        g[:, sampled(d, M)] = 8.0
         for i, octaves in enumerate((16, 26, 50)):
-            g[i::3, ~sampled(d)] *= 2.0 ** -octaves
+            g[i::3, ~sampled(d, M)] *= 2.0 ** -octaves
     elif case == "sample_below":      # and below, by 4, 10 and 50
-        g[:, sampled(d)] = 1.0
+        g[:, sampled(d, M)] = 1.0
         for i, octaves in enumerate((4, 10, 50)):
-            g[i::3, ~sampled(d)] *= 2.0 ** octaves
+            g[i::3, ~sampled(d, M)] *= 2.0 ** octaves
     elif case == "uniform":           # half of the keys lie in the octave of the largest
         g.uniform_(-1.0, 1.0, generator=gen)
     elif case == "signs":
