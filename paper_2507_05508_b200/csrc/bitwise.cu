@@ -411,12 +411,12 @@ bit_stats_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t*
 }
 
 // ---- pack: a warp turns 1024 consecutive entries into 32 words of each plane, a lane owning 32 consecutive entries (one
-// word per plane).  The entries come through a slot of shared memory per warp: the next group's copy starts when the current
-// group's entries are in registers, and is in flight while they are coded.  A plane's word is collected by one shift and one funnel shift per entry, from
-// 6 planes on by one bit transpose for all of them.  A group whose largest entry has the code 0 at the drawn level's bits is
-// not coded: its magnitude planes are zero.  The groups of which the sweep before knows that are not even read (8 x 124M fp32
-// entries with layers: 782 -> 424 us).  Those calls have four blocks per SM, since one warp's groups are not another's: 482 us with three
-// blocks of two slots per warp, now 439.  Calls that read everything are as fast with three (8 x 3M 53.6 us per step, 55.5 with four).
+// word per plane).  The entries come through one or two slots of shared memory per warp: a slot takes its next group's copy when the
+// group before it is in registers, and the copy is in flight while that is coded.  A plane's word is collected by one shift and one
+// funnel shift per entry, from 6 planes on by one bit transpose for all of them.  A group whose largest entry has the code 0 at the drawn
+// level's bits is not coded: its magnitude planes are zero.  The groups of which the sweep before knows that are not even read (8 x 124M
+// fp32 entries with layers: 782 -> 424 us).  Calls that read everything have three blocks per SM and one slot per warp (8 x 3M 53.6 us
+// per step, 55.5 with four blocks); for the others see launch_bit_pack_t.
 // Bound by HBM.  Rows of 32 entries across the lanes with a ballot each took 1.04 ms for 8 x 124M fp32 entries.
 // after_read: called when the lane has its entries of the group in registers.
 template <typename T, typename F>
@@ -471,12 +471,15 @@ __device__ __forceinline__ void pack_group(const uint32_t* slot, const Quantiser
     }
 }
 
-template <typename T, bool SKIP>
-__global__ void __launch_bounds__(kBitThreads, SKIP ? 4 : 3)
+template <typename T, bool SKIP, int BLOCKS>
+constexpr int kPackSlots = SKIP && (BLOCKS == 3 || sizeof(T) == 2) ? 2 : 1;  // groups in flight per warp; four blocks of fp32 have room for one
+
+template <typename T, bool SKIP, int BLOCKS>  // BLOCKS: per SM
+__global__ void __launch_bounds__(kBitThreads, BLOCKS)
 bit_pack_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* gmax_bits, BitSchedule sc,
                 const int32_t* bit_level, const uint32_t* batch_max, int batches_per_worker, uint32_t* __restrict__ planes, int w_max,
                 int64_t words) {
-    extern __shared__ __align__(16) uint32_t sh_ring[];  // [warps][kGroupSlot]
+    extern __shared__ __align__(16) uint32_t sh_ring[];  // [warps][SLOTS][kGroupSlot]
     pdl_enter();
     const int m = blockIdx.y;
     const int level = bit_level[m];
@@ -490,7 +493,8 @@ bit_pack_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* 
     const float scale = (float)(1u << bits);
     const T* row = g + (int64_t)m * ld;
     uint32_t* out = planes + (int64_t)m * (1 + w_max) * words;
-    uint32_t* ring = sh_ring + warp * kGroupSlot<T>;
+    constexpr int SLOTS = kPackSlots<T, SKIP, BLOCKS>;
+    uint32_t* ring = sh_ring + warp * SLOTS * kGroupSlot<T>;
     const int64_t stride = (int64_t)gridDim.x * (blockDim.x / 32);
     if constexpr (!SKIP) {
         int64_t grp = (int64_t)blockIdx.x * (blockDim.x / 32) + warp;
@@ -525,21 +529,26 @@ bit_pack_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const uint32_t* 
                 todo &= todo - 1u;
                 return grp;
             };
-            int64_t grp = next();
-            fetch_group<T>(row, d, grp, ngroups, ring);
+            int64_t grp[SLOTS];
+#pragma unroll
+            for (int i = 0; i < SLOTS; ++i) {
+                grp[i] = next();
+                fetch_group<T>(row, d, grp[i], ngroups, ring + i * kGroupSlot<T>);
+            }
             for (; zero; zero &= zero - 1u) {  // magnitude planes of zeros, while the first group is on its way
                 uint32_t* to = out + (base + (__ffs(zero) - 1) * stride) * 32 + lane;
                 for (int j = 1; j <= w; ++j) to[(int64_t)j * words] = 0u;
             }
-            while (grp < ngroups) {
+            for (int at = 0; grp[0] < ngroups; at = SLOTS == 1 ? 0 : at ^ kGroupSlot<T>) {
                 const int64_t after = next();
-                cp_async_wait<0>();
+                cp_async_wait<SLOTS - 1>();
                 __syncwarp();
-                pack_group<T>(ring, qz, scale, zero_below, w, grp * 32 + lane, words, out, (grp + 1) * 1024 > d, [&]() {
+                pack_group<T>(ring + at, qz, scale, zero_below, w, grp[0] * 32 + lane, words, out, (grp[0] + 1) * 1024 > d, [&]() {
                     __syncwarp();  // the slot has been read by every lane
-                    fetch_group<T>(row, d, after, ngroups, ring);
+                    fetch_group<T>(row, d, after, ngroups, ring + at);
                 });
-                grp = after;
+                if (SLOTS == 2) grp[0] = grp[SLOTS - 1];
+                grp[SLOTS - 1] = after;
             }
         }
     }
@@ -729,7 +738,7 @@ int bit_blocks(const Workspace& ws, int64_t d, int vec, int M, int waves) {
     return (int)(nb < 1 ? 1 : nb);
 }
 
-size_t bit_pack_smem(size_t elem, int warps) { return (size_t)warps * 1024 * elem; }
+size_t bit_pack_smem(size_t elem, int warps, int slots) { return (size_t)warps * slots * 1024 * elem; }
 
 }  // namespace
 
@@ -737,10 +746,8 @@ int configure_bit_kernels() {
     const bool ok = cudaFuncSetAttribute(aggregate_bitwise_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)kAvgBitSmem + kEmitMaxWorkers * 8) == cudaSuccess &&
                     configure_dense_cluster(bit_cluster_kernel<float>) && configure_dense_cluster(bit_cluster_kernel<bf16_t>) &&
-                    cudaFuncSetAttribute(bit_pack_kernel<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)bit_pack_smem(4, kBitThreads / 32)) == cudaSuccess &&
-                    cudaFuncSetAttribute(bit_pack_kernel<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)bit_pack_smem(4, kBitThreads / 32)) == cudaSuccess;
+                    cudaFuncSetAttribute(bit_pack_kernel<float, true, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)bit_pack_smem(4, kBitThreads / 32, kPackSlots<float, true, 3>)) == cudaSuccess;
     return ok ? MLMC_OK : MLMC_ERR_CUDA;
 }
 
@@ -840,12 +847,30 @@ static void launch_bit_pack_t(Workspace& ws, const T* g, int64_t d, int M, int64
     const int64_t ngroups = (words + 31) / 32;
     const int warps = (int)std::min<int64_t>(ngroups, kBitThreads / 32);  // of short rows as many blocks as possible fit an SM
     const int64_t by_work = (ngroups + warps - 1) / warps;
-    int64_t nb = ((int64_t)ws.sm_count * (zero_batches(ws) ? 4 : 3)) / M;  // persistent: one wave, rounded down
-    if (nb > by_work) nb = by_work;
-    if (nb < 1) nb = 1;
-    launch_kernel(ws, K_BIT_PACK, zero_batches(ws) ? bit_pack_kernel<T, true> : bit_pack_kernel<T, false>, dim3((unsigned)nb, M), warps * 32, bit_pack_smem(sizeof(T), warps), s, g, d, ld,
-                  ws.gmax_bits, sc, ws.bit_level, zero_batches(ws), emit_tiles_per_worker(d, sizeof(T) == 2 ? MLMC_BF16 : MLMC_F32) * kEmitGroups,
-                  out.planes, out.w_max, words);
+    auto blocks = [&](int per_sm) {  // persistent: one wave, rounded down
+        return std::max<int64_t>(1, std::min(by_work, (int64_t)ws.sm_count * per_sm / M));
+    };
+    auto go = [&](auto kernel, int per_sm, int slots) {
+        launch_kernel(ws, K_BIT_PACK, kernel, dim3((unsigned)blocks(per_sm), M), warps * 32, bit_pack_smem(sizeof(T), warps, slots), s, g, d, ld,
+                      ws.gmax_bits, sc, ws.bit_level, zero_batches(ws), emit_tiles_per_worker(d, sizeof(T) == 2 ? MLMC_BF16 : MLMC_F32) * kEmitGroups,
+                      out.planes, out.w_max, words);
+    };
+    if (!zero_batches(ws)) {
+        go(bit_pack_kernel<T, false, 3>, 3, kPackSlots<T, false, 3>);
+        return;
+    }
+    // The groups that are left to read lie where the layers are large: some warps have far more of them than others.  Where a warp has
+    // few groups the call lasts as long as the longest such chain, and three blocks per SM with registers to spare and two copies in
+    // flight are the faster way; with many, four blocks (64 registers: the bf16 kernel spills some, and is the faster one all the same).
+    // us per step, adaptive p, three / four: fp32 8 x 3.3M 92 / 100, 8 x 6.6M 154 / 154, 8 x 12.5M 266 / 267, 8 x 20M 392 / 390,
+    // 8 x 62M 1041 / 1023; bf16 8 x 7M 131 / 136, 8 x 11M 198 / 199, 8 x 15M 254 / 254, 8 x 18M 303 / 297, 32 x 25.6M 1491 / 1445.
+    // Earlier where whole blocks per worker leave more than 5 % of three blocks per SM idle (given p): fp32 32 x 2M 126 / 123,
+    // bf16 32 x 2.1M 103 / 102, 32 x 1.7M 74.5 / 75.9.
+    constexpr int64_t kManyGroups = 24, kManyGroupsIdle = 12;
+    const int64_t per_warp = (ngroups + blocks(4) * warps - 1) / (blocks(4) * warps);
+    const bool idle = ws.sm_count * 3 / M * M * 20 < ws.sm_count * 3 * 19;
+    if (per_warp > (idle ? kManyGroupsIdle : kManyGroups)) go(bit_pack_kernel<T, true, 4>, 4, kPackSlots<T, true, 4>);
+    else go(bit_pack_kernel<T, true, 3>, 3, kPackSlots<T, true, 3>);
 }
 
 void launch_bit_pack(Workspace& ws, const void* g, int dtype, int64_t d, int M, int64_t ld, const int32_t* b, int L,

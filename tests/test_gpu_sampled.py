@@ -188,6 +188,22 @@ def test_batches_that_round_to_zero_are_not_read(B, ora, dtype, d):
         B.mlmc_destroy(ctx)
 
 
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("d", [12 * 144 * 1024, 12 * 144 * 1024 + 1])
+def test_groups_per_warp(B, ora, dtype, d):
+    """The last row of 32 workers whose message has three blocks per SM (148 SMs: twelve groups for each of 144 warps), and the first with
+    four: layers, so that some groups are read and some are not."""
+    M = 32
+    gen = torch.Generator(device="cuda").manual_seed(d)
+    scale = torch.repeat_interleave(10.0 ** (torch.rand(40, generator=gen, device="cuda") * 4 - 5), -(-d // 40))[:d]
+    g = padded((torch.randn((M, d), generator=gen, device="cuda") * scale).to(torch.bfloat16 if dtype == "bf16" else torch.float32), 8)
+    ctx = B.mlmc_create(0, d, M, 32)
+    try:
+        check_bitwise(B, ora, ctx, g, [1, 2, 4, 8, 16, 23], [1 / 6] * 6, 1, 0)
+    finally:
+        B.mlmc_destroy(ctx)
+
+
 def kernel_ms(B, ctx, call):
     """Milliseconds of every kernel in one call."""
     import ctypes as C
