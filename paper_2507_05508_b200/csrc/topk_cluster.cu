@@ -40,6 +40,7 @@ constexpr int kClBatches = 91;                   // batches per block at most: a
 constexpr int kClBatchesBf16 = 63;               // given p, bf16: a block's keys fit 16-bit counts
 constexpr int kClSpread = 16;                    // batches per block from which on the cluster grows while all clusters run at a time,
 constexpr int kClEasy = 32;                      // and where they do not
+constexpr int kClFew = 64;                       // given p, fp32: from which on 16 blocks take the place of 8, if they run at a time
 constexpr int kClTwoWaves = 56;                  // adaptive p, fp32: batches per block with which two waves of clusters are worth it
 constexpr int kClCells = 32 + 256;               // interval + (largest exponent - exponent)
 constexpr int kClCopiesLow = 8;                  // copies of a cell's limbs: 32 where the cells are few enough, else 8
@@ -691,26 +692,31 @@ void cluster_limits(KernelLimits* limits) {  // the kernels of all sizes take th
 }
 
 // Blocks per cluster for this call, 0: the row is too long, or the workers are too many, for the cluster to be the faster way.
-// kClSpread batches per block while the clusters of all workers run at a time, else kClEasy (4 x 65,536 entries, given p: 18.9 us per
-// step on 8 blocks, 20.0 on 4, where M clusters of 16 would not fit 131k x 8 takes 63 us on 16 and 36 on 8); longer rows are
-// stretched over 16 blocks.  fp32 rows with given p have two digits of two queries to tell all of 16 blocks, which takes longer than it
-// spares: up to 8 blocks while kClEasy batches suffice (3 x 131,072 22.2 us on 16, 18.9 on 8; adaptive p 29.2 and 30.2, bf16 17.9 and 19.7).  Clusters that do not fit the GPU at a time run one after the other, where the launch chain has the
-// whole GPU: how far that pays depends on what the chain has to do.  us per step, cluster / chain, layered rows:
+// kClSpread batches per block while the clusters of all workers run at a time, else kClEasy (4 x 65,536 entries, given p: 17.3 us per
+// step on 8 blocks, 20.0 on 4; where M clusters of 16 would not fit, 131k x 8 takes 63 us on 16 and 36 on 8); longer rows are stretched over
+// 16 blocks.  fp32 rows with given p have two digits of two queries to tell all of 16 blocks, which takes longer than it spares, and few
+// clusters of 16 run at a time: 8 blocks up to kClFew batches in each, and as many as a block holds where the clusters of 16 would take turns
+// (16 blocks / 8: 131k x 3 22.3 / 19.8, 262k x 3 24.4 / 22.8, 280k x 6 29.3 / 28.8, 310k x 2 26.2 / 26.7, 372k x 4 29.9 / 31.8; 131k x 8 40.7 / 22.7,
+// 262k x 9 45 / 26.7, 372k x 12 57.9 / 37.7).  Clusters that do not fit the GPU at a time run one after the other, where the launch chain has
+// the whole GPU: how far that pays depends on what the chain has to do.  us per step, cluster / chain, layered rows:
 //   fp32, adaptive  700k x 3 53 / 76, 400k x 6 46 / 79; two waves 262k x 8 63 / 78, 400k x 12 82 / 90, 700k x 8 100 / 89; three
 //                   262k x 16 95 / 90, 131k x 32 93 / 100
-//   fp32, given p   700k x 3 34 / 56, 700k x 6 39 / 60; two waves 262k x 8 43 / 56, 500k x 8 52 / 60, 700k x 12 67 / 69; three
-//                   262k x 16 67 / 64
+//   fp32, given p   700k x 3 34 / 56, 700k x 6 39 / 60; two waves 262k x 16 45 / 61, 262k x 28 54 / 78, 372k x 28 69 / 91, 500k x 8 52 / 60,
+//                   700k x 12 67 / 69
 //   bf16, adaptive  500k x 4 47 / 53, 700k x 4 61 / 55, 1M x 3 70 / 54; two waves 500k x 8 75 / 58
 //   bf16, given p   500k x 4 23 / 33, 1M x 3 30 / 36; two waves 500k x 8 38 / 39, 1M x 8 53 / 45
 int cluster_blocks(const Workspace& ws, int dtype, int64_t d, int M, bool given) {
     const int64_t batches = (int64_t)emit_tiles_per_worker(d, dtype) * kEmitGroups;
     if (M > 32) return 0;
+    const int* fits = ws.limits.topk_fit;
+    auto enough = [&](int i) {  // batches per block up to which 2^i blocks are not made 2^(i + 1)
+        const bool at_a_time = M <= fits[i + 1];
+        if (i == 3 && given && dtype == MLMC_F32) return at_a_time ? kClFew : kClBatches;
+        return at_a_time ? kClSpread : kClEasy;
+    };
     int i = 0;
-    const int spread_to = given && dtype == MLMC_F32 ? 3 : 4;
-    while (i < 4 && ws.limits.topk_fit[i + 1] > 0 &&
-           batches > (int64_t)(M <= ws.limits.topk_fit[i + 1] && i < spread_to ? kClSpread : kClEasy) << i)
-        ++i;
-    const int fit = ws.limits.topk_fit[i];
+    while (i < 4 && fits[i + 1] > 0 && batches > (int64_t)enough(i) << i) ++i;
+    const int fit = fits[i];
     if (fit == 0) return 0;
     const int64_t per = (batches + (1 << i) - 1) >> i;
     const int waves = (M + fit - 1) / fit;

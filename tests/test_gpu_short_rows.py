@@ -65,6 +65,17 @@ def test_segments_given_p(B, ora, ctx, d):
     check_stopk(B, ora, ctx, rows("ties", d, 2, "f32"), s, [1.0 / L] * L, 3, 2)
 
 
+# fp32, given p: the longest rows on 8 blocks where clusters of 16 run at a time and where they take turns, and one entry more
+@pytest.mark.parametrize("d,M", [(262_144, 2), (262_145, 2), (262_144, 20), (372_736, 9), (372_737, 9), (372_736, 24)])
+def test_rows_on_eight_blocks(B, ora, ctx, d, M):
+    s = d // 40
+    L = -(-d // s)
+    check_stopk(B, ora, ctx, layered(d, M), s, geometric(L), 3, 1)
+    if d <= 262_144:
+        k = doubling(d, d // 500)
+        check_topk(B, ora, ctx, layered(d, M), k, geometric(len(k)), 3, 1, expect_excluded=1)
+
+
 # edges of the tiles; empty, void and dense messages; lanes per search edge from 32 to 4
 @pytest.mark.parametrize("d", [1, 1_023, 1_025, 4_097, 200_001, 1_212_417])
 @pytest.mark.parametrize("M", [1, 3, 9, 32])
