@@ -454,7 +454,8 @@ __device__ __forceinline__ void pack_group(const uint32_t* slot, const Quantiser
         return;
     }
     uint32_t q[32];
-    qz.codes(x, scale, __any_sync(0xFFFFFFFFu, __float_as_int(mx) == qz.top), q);  // the bits above a field leave with the shifts, or are planes that are not written
+    // the bits above a field leave with the shifts, or are planes that are not written
+    qz.codes(x, scale, __any_sync(0xFFFFFFFFu, __float_as_int(mx) == qz.top), q);
     if (w < 6) {
         for (int j = 1; j <= w; ++j) {
             const int up = 31 - (w - j);

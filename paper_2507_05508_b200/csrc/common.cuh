@@ -447,7 +447,7 @@ __device__ __forceinline__ void load_bins(const uint32_t* bins, uint4 (&x)[8]) {
     for (int i = 0; i < 8; ++i) x[i] = reinterpret_cast<const uint4*>(bins)[i * 32 + (threadIdx.x & 31)];
 }
 // Hands every lane the 32 bins from 32 * mine through shared memory (rows: 256 vectors per warp; vector j of bin group t at j ^ t, so that
-// neither side meets in a bank).  Read directly, every load touches 32 lines (16 x 11.7M entries, given p: 254 us per step, 251 so).
+// neither side meets in a bank).  Read directly, every load touches 32 lines (segment_resolve of 16 rows 23.6 us, 20.9 so).
 __device__ __forceinline__ void hand_over_bins(const uint4 (&x)[8], uint4* rows, int mine, uint32_t (&cnt)[32]) {
     const int lane = threadIdx.x & 31;
 #pragma unroll

@@ -105,8 +105,8 @@ __device__ __forceinline__ void rtn_expand(const uint4* q, float (&v)[kRtnHeld])
 }
 
 // The conversion unit takes 16 numbers per clock and SM, a quarter of what the fp64 unit adds up.  So every second number (x >= 0; one
-// of four or three of four are within 1 %) goes another way: its bits moved to the places of a double are x 2^-896, zero and the numbers below the normal range included, and
-// the product with 2^896 is exact.
+// of four or three of four are within 1 %) goes another way: its bits moved to the places of a double are x 2^-896, zero and the numbers
+// below the normal range included, and the product with 2^896 is exact.
 __device__ __forceinline__ double widen(float x, bool by_product) {
     if (!by_product) return (double)x;
     const uint32_t b = __float_as_uint(x);

@@ -7,7 +7,7 @@
 // the steps are separated by cluster barriers (0.4 to 0.6 us each, with what was written before them).  Bound by the latency of
 // the steps and, in rows of more than a few thousand keys per block, by the issue of the passes over the keys.  The cluster size is
 // a constant of the kernel: loops over the blocks have all their reads in flight, and nothing is divided at run time (4 x 65,536
-// entries, given p: 22.4 us per step with a run-time size, 20.0 so).  The steps:
+// entries, given p, on 4 blocks: 22.4 us per step with a run-time size, 20.0 so).  The steps:
 //   1. the row is copied to shared memory (16-byte asynchronous copies); histogram of the leading 13 key bits, largest
 //      key per batch, NaN / Inf check;
 //   2. radix select of every query: 13 + 9 + 9 key bits (fp32) or 13 + 2 (bf16).  The blocks tell one another their counts of
@@ -161,7 +161,8 @@ cluster_topk_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid
     uint4* sh_part = reinterpret_cast<uint4*>(sh_hist + kClBins / 2);  // [block][kRangeVecs]: the half of the words that the counts do not use
     static_assert(kClHistWords - kClBins / 2 >= kClMost * kRangeVecs * 4, "the ranges of all blocks fit behind the counts");
     if (t < CL * kRangeVecs)
-        cluster.map_shared_rank(sh_part, t / kRangeVecs)[rank * kRangeVecs + t % kRangeVecs] = reinterpret_cast<const uint4*>(sh.ranges)[t % kRangeVecs];
+        cluster.map_shared_rank(sh_part, t / kRangeVecs)[rank * kRangeVecs + t % kRangeVecs] =
+            reinterpret_cast<const uint4*>(sh.ranges)[t % kRangeVecs];
     if (t < CL) cluster.map_shared_rank(sh.top, t)[rank] = my_top;
     cluster.sync();
     uint32_t top = 0;
@@ -293,7 +294,7 @@ cluster_topk_kernel(const T* __restrict__ g, int64_t d, int64_t ld, const __grid
     // itself, and the third digit has counts of its own, so that nothing is exchanged but the counts.  Otherwise a block
     // resolves every CL-th query and tells the others, and the third digit takes the place of the second.
     const uint32_t hist_words = ((max(sh.slots << kBits2, (uint32_t)nq << kShift2) / 2 + 3u) & ~3u);
-    const bool alike = nq * 2 * CL <= 2 * (kClThreads / 32) && 4u * hist_words <= (uint32_t)kClHistWords;
+    const bool alike = nq * CL <= kClThreads / 32 && 4u * hist_words <= (uint32_t)kClHistWords;
     uint32_t* const sh_count2 = sh_hist;
     uint32_t* const sh_count3 = alike ? sh_hist + hist_words : sh_hist;
     const uint32_t list_from = alike ? 2u * hist_words : hist_words;
@@ -679,7 +680,7 @@ int configure_cluster_kernels() {
         return cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
     };
     for (int i = 0; i < 5; ++i)
-        if (!with_cluster(i, [&](auto cl) { 
+        if (!with_cluster(i, [&](auto cl) {
                 return set(cluster_topk_kernel<float, cl(), true>) && set(cluster_topk_kernel<float, cl(), false>) &&
                        set(cluster_topk_kernel<bf16_t, cl(), true>) && set(cluster_topk_kernel<bf16_t, cl(), false>);
             }))
@@ -687,15 +688,18 @@ int configure_cluster_kernels() {
     return MLMC_OK;
 }
 
-void cluster_limits(KernelLimits* limits) {  // the kernels of all sizes take the same shared memory, and one block per SM
+// Asked of one kernel for all: they have the same threads and shared memory, 64 registers at most (1024 threads take all of an SM's), and
+// with the shared memory of the longest rows one block per SM.
+void cluster_limits(KernelLimits* limits) {
+    static_assert(kClThreads == 1024 && 2 * (kClFixedSmem + kClBatches * kBatchWords * 4) > kClSharedMost, "one block per SM");
     clusters_that_fit(cluster_topk_kernel<float, 16, true>, kClThreads, cluster_smem(kClBatches), limits->topk_fit);
 }
 
 // Blocks per cluster for this call, 0: the row is too long, or the workers are too many, for the cluster to be the faster way.
-// kClSpread batches per block while the clusters of all workers run at a time, else kClEasy (4 x 65,536 entries, given p: 17.3 us per
-// step on 8 blocks, 20.0 on 4; where M clusters of 16 would not fit, 131k x 8 takes 63 us on 16 and 36 on 8); longer rows are stretched over
-// 16 blocks.  fp32 rows with given p have two digits of two queries to tell all of 16 blocks, which takes longer than it spares, and few
-// clusters of 16 run at a time: 8 blocks up to kClFew batches in each, and as many as a block holds where the clusters of 16 would take turns
+// kClSpread batches per block while the clusters of all workers run at a time, else kClEasy (4 x 65,536 entries: 18.9 us per step on 8
+// blocks, 19.7 on 4, adaptive p 26.4 and 30.3; where M clusters of 16 would not fit, 131k x 8 adaptive takes 63 us on 16 and 36 on 8); longer
+// rows are stretched over 16 blocks.  fp32 rows with given p have two digits of two queries to tell all of 16 blocks, which takes longer
+// than it spares, and few clusters of 16 run at a time: 8 blocks up to kClFew batches in each, and as many as a block holds where the clusters of 16 would take turns
 // (16 blocks / 8: 131k x 3 22.3 / 19.8, 262k x 3 24.4 / 22.8, 280k x 6 29.3 / 28.8, 310k x 2 26.2 / 26.7, 372k x 4 29.9 / 31.8; 131k x 8 40.7 / 22.7,
 // 262k x 9 45 / 26.7, 372k x 12 57.9 / 37.7).  Clusters that do not fit the GPU at a time run one after the other, where the launch chain has
 // the whole GPU: how far that pays depends on what the chain has to do.  us per step, cluster / chain, layered rows:
@@ -747,8 +751,11 @@ void launch_cluster_topk(Workspace& ws, const void* g, int dtype, int64_t d, int
     int log2 = 0;
     while (1 << log2 < cl) ++log2;
     with_cluster(log2, [&](auto size) {
-        if (dtype == MLMC_BF16) go(bands ? cluster_topk_kernel<bf16_t, size(), false> : cluster_topk_kernel<bf16_t, size(), true>, static_cast<const bf16_t*>(g));
-        else go(bands ? cluster_topk_kernel<float, size(), false> : cluster_topk_kernel<float, size(), true>, static_cast<const float*>(g));
+        constexpr int CL = size();
+        if (dtype == MLMC_BF16)
+            go(bands ? cluster_topk_kernel<bf16_t, CL, false> : cluster_topk_kernel<bf16_t, CL, true>, static_cast<const bf16_t*>(g));
+        else
+            go(bands ? cluster_topk_kernel<float, CL, false> : cluster_topk_kernel<float, CL, true>, static_cast<const float*>(g));
     });
 }
 

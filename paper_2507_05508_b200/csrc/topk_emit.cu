@@ -30,8 +30,10 @@ namespace mlmc {
 namespace {
 
 constexpr int kBandThreads = 256;               // 8 warps per block, one tile per warp at a time
-// Shared-memory batches per warp of the write pass, and blocks per SM.  fp32: 8 x 124M 150 us with three and three, 140 with two and
-// four (141 with two and five).  bf16: 32 x 25.6M 185 and 177, but 8 x 3M 95 us per step and 98.7.
+// Shared-memory batches per warp of the write pass, and blocks per SM.  fp32, three and three / two and four: 16 x 11.7M in layers, level
+// 0, 10, 50 and 99 of 100 (a few batches listed to all) 42.5 / 40.7, 56 / 53, 120 / 106, 147 / 132 us; 8 x 124M, 20 levels, level 0, 10,
+// 19: 309 / 281, 789 / 737, 843 / 791; 8 x 3M the same (17 to 28).  bf16 has as many entries in half of the batches: 32 x 25.6M 176 / 179,
+// 442 / 444, 457 / 457, 8 x 40M 90 / 90, 187 / 186, 199 / 198, and the steps of 8 x 3M become 5 to 8 % longer (75 / 81).
 template <typename T>
 constexpr int kWriteSlots = EmitWord<T>::S == 1 ? 2 : 3;
 template <typename T>

@@ -170,8 +170,7 @@ hist1_kernel(const float* __restrict__ g, int64_t d, int64_t ld, uint32_t* __res
             uint4 q[kBatch];
 #pragma unroll
             for (int j = 0; j < kBatch; ++j) q[j] = __ldg(reinterpret_cast<const uint4*>(row) + v + j * 32);
-            // the next batch as far as L2 (16 x 11.7M fp32 keys: 145 us without, now 133; the batch after it 138; 32 x 25.6M bf16 keys
-            // 322, now 304)
+            // the next batch as far as L2 (16 x 11.7M keys, with brackets: 145 us without, now 133; the batch after it 138)
             if (lane < 16 && (int64_t)(b + step + 1) * kEmitGroupVecs <= full_end)
                 prefetch_line(reinterpret_cast<const uint4*>(row) + v + (int64_t)step * kEmitGroupVecs + lane * 7);
             uint32_t vm = 0;
@@ -246,10 +245,10 @@ hist1_kernel(const float* __restrict__ g, int64_t d, int64_t ld, uint32_t* __res
 // deviation 355, 347, 334).  Beside the window, down to 12 octaves below it, a bin has one count; what lies outside of that is counted
 // in memory, key by key, and the lowest bin (zeros) in a register.  A block whose sample lies below the window by more than one key
 // of kColumnMisses keeps one count per bin for all, and so do short rows, where the sample takes longer than it saves
-// (8 x 1M bf16 keys: 63.3 us per step, 65.7 with columns).
-// 32 x 25.6M bf16 keys: 406 us, now 318 (floor 250); 8 x 40M, given p: 260 us per step, now 231; 8 x 12M 167 either way.  On the way: all
-// 32 keys of a warp by the general way whenever one lies outside the window (each lane its own way 355 us); every key by the general
-// way 386; windows of 22 and 24 octaves leave too little L1 for the loads in flight (362 us, and 334 without the bins beside).
+// (us per step without / with columns: 8 x 1M keys 60.9 / 62.7, 32 x 1.2M 113 / 118, 8 x 2M 75.7 / 74.9, 8 x 3M 95.5 / 93.4, from 8 x 4M on with).
+// 32 x 25.6M keys in layers: 401 us with one count per bin, now 311 (floor 250); 8 x 40M 164, 129; 8 x 12M 59, 53.  On the way to it, where it
+// took 337: all 32 keys of a warp by the general way whenever one lies outside the window (each lane its own way 355 us); every key by the
+// general way 386; windows of 22 and 24 octaves leave too little L1 for the loads in flight (362 us, and 334 without the bins beside).
 // fp32 rows, with half as many atomics per byte, gain nothing (16 x 11.7M 135.4 us, 135.9 so; with the stages of the brackets beside 139 and
 // 159).
 constexpr int kColumns = 16;
@@ -295,7 +294,8 @@ struct BinCounts {
         found = __reduce_add_sync(0xFFFFFFFFu, sh_warp[lane]);
         columns = (found >> 16) * kColumnMisses <= (uint32_t)(N * kHistThreads);
         // (an octave less below, then: its keys are counted beside the window)
-        if ((found & 0xFFFFu) * kColumnMisses > (uint32_t)(N * kHistThreads)) lowest = octave + 128u > (uint32_t)kWindow ? octave + 128u - kWindow : 0u;
+        if ((found & 0xFFFFu) * kColumnMisses > (uint32_t)(N * kHistThreads))
+            lowest = octave + 128u > (uint32_t)kWindow ? octave + 128u - kWindow : 0u;
         const uint32_t base = (uint32_t)__cvta_generic_to_shared(counts);
         column0 = base + (lane & (kColumns - 1)) * 4u - lowest * (kColumns * 4u);
         far0 = base + (kWindow * kColumns + kFarBelow - (int)lowest) * 4;
@@ -398,7 +398,7 @@ hist1_bf16_kernel(const bf16_t* __restrict__ g, int64_t d, int64_t ld, uint32_t*
             uint4 q[kBatch];
 #pragma unroll
             for (int j = 0; j < kBatch; ++j) q[j] = __ldg(reinterpret_cast<const uint4*>(row) + v + j * 32);
-            // the next batch as far as L2
+            // the next batch as far as L2 (32 x 25.6M keys: 5 % of the kernel)
             if (lane < 16 && (int64_t)(b + step + 1) * kEmitGroupVecs <= full_end)
                 prefetch_line(reinterpret_cast<const uint4*>(row) + v + (int64_t)step * kEmitGroupVecs + lane * 7);
 #pragma unroll
